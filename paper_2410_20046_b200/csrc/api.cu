@@ -225,9 +225,9 @@ const char *dqrm_kernel_name(int kernel_id)
 {
     static const char *names[DQ_K_COUNT] = {
         "begin", "refresh_kernel", "fwd_kernel", "memset", "prepare_kernel", "sort_scan_kernel",
-        "sort_scatter_kernel", "seg_count_kernel", "seg_emit_kernel", "seg_reduce_kernel", "seg_fixup_kernel",
+        "sort_scatter_kernel", "seg_count_kernel", "seg_emit_kernel", "seg_sum_kernel",
         "absmax_kernel", "row_stream_kernel<quant>", "row_stream_kernel<update>", "row_stream_kernel<fused>",
-        "copy", "seg_fixup_big_kernel", "cluster_sort_kernel", "dp_pack_kernel", "dp_sum_update_kernel", "pack_kernel", "packed_fwd_kernel", "fwd_codes_kernel", "decode_payload_kernel"};
+        "copy", "cluster_sort_kernel", "dp_pack_kernel", "dp_sum_update_kernel", "pack_kernel", "packed_fwd_kernel", "fwd_codes_kernel", "decode_payload_kernel"};
     return (kernel_id >= 0 && kernel_id < DQ_K_COUNT) ? names[kernel_id] : "?";
 }
 
@@ -273,7 +273,7 @@ int dqrm_emb_bwd(dqrm_ctx *ctx, const float *grad_out, const int32_t *indices, c
     if (L > 0 && (!indices || !unique_rows || !grad_rows)) return DQRM_ERR_INVALID_ARG;
     if (!ws_ok(workspace, workspace_bytes, dq_bwd_ws_bytes(ctx, L, (int64_t)ctx->T * B))) return DQRM_ERR_WORKSPACE;
     return dq_launch_bwd(ctx, grad_out, indices, offsets, unique_rows, uniq_off, grad_rows, B, L, workspace,
-                         workspace_bytes, as_stream(stream), nullptr);
+                         workspace_bytes, as_stream(stream));
 }
 
 int dqrm_grad_quant_int8(dqrm_ctx *ctx, const float *grad_rows, const int32_t *uniq_off, int8_t *codes,
@@ -314,9 +314,7 @@ int dqrm_train_step(dqrm_ctx *ctx, float *tables, const int32_t *indices, const 
         DQRM_CUDA_TRY(ctx, cudaEventRecord(ctx->ev_fork, st));
         DQRM_CUDA_TRY(ctx, cudaStreamWaitEvent(ctx->side, ctx->ev_fork, 0));
     }
-    int rc = dq_launch_bwd_sort(ctx, indices, offsets, unique_rows, uniq_off, B, L, workspace, workspace_bytes, ss, nullptr, true);
-    if (rc == DQRM_OK)
-        rc = dq_launch_bwd_reduce(ctx, grad_out, unique_rows, uniq_off, grad_rows, B, L, workspace, workspace_bytes, ss);
+    int rc = dq_launch_bwd(ctx, grad_out, indices, offsets, unique_rows, uniq_off, grad_rows, B, L, workspace, workspace_bytes, ss);
     int rc2 = dq_launch_fwd(ctx, tables, indices, offsets, scales, bits, out, nullptr, B, L, st);
     if (overlap) {   // join even after an error so that the caller's stream stays ordered behind the side stream
         cudaEventRecord(ctx->ev_join, ctx->side);
@@ -371,7 +369,8 @@ int dqrm_sort_batch(dqrm_ctx *ctx, const int32_t *indices, const int32_t *offset
     if (!ws_ok(workspace, workspace_bytes, dq_bwd_ws_bytes(ctx, L, (int64_t)ctx->T * B))) return DQRM_ERR_WORKSPACE;
     cudaStream_t st = as_stream(stream);
     if (ctx->prof_on) dq_mark(ctx, st, DQ_K_BEGIN);
-    const int rc = dq_launch_bwd_sort(ctx, indices, offsets, unique_rows, uniq_off, B, L, workspace, workspace_bytes, st, nullptr, true);
+    bool by_table = false;
+    const int rc = dq_launch_bwd_sort(ctx, indices, offsets, unique_rows, uniq_off, B, L, workspace, workspace_bytes, st, true, &by_table);
     {
         std::lock_guard<std::mutex> lock(ctx->sorted_mu);
         dqrm_ctx::SortedBatch &sb = ctx->sorted[workspace];
@@ -386,6 +385,7 @@ int dqrm_sort_batch(dqrm_ctx *ctx, const int32_t *indices, const int32_t *offset
         sb.capture_id = id;
         sb.L = L;
         sb.B = B;
+        sb.by_table = by_table;
         sb.fresh = true;
     }
     return rc;
@@ -403,7 +403,7 @@ int dqrm_train_step_sorted(dqrm_ctx *ctx, float *tables, const int32_t *indices,
     if (L > 0 && (!indices || !unique_rows || !grad_rows || !codes)) return DQRM_ERR_INVALID_ARG;
     if (!ws_ok(workspace, workspace_bytes, dq_bwd_ws_bytes(ctx, L, (int64_t)ctx->T * B))) return DQRM_ERR_WORKSPACE;
     cudaEvent_t sort_done = nullptr;
-    bool sort_captured = false;
+    bool sort_captured = false, by_table = false;
     unsigned long long sort_capture_id = 0;
     {   // the workspace must hold this batch, sorted by dqrm_sort_batch and not consumed yet: the summation
         // trusts the segment lists in it and zeroes nothing itself
@@ -414,6 +414,7 @@ int dqrm_train_step_sorted(dqrm_ctx *ctx, float *tables, const int32_t *indices,
         it->second.fresh = false;
         sort_done = it->second.done;
         sort_captured = it->second.captured;
+        by_table = it->second.by_table;
         sort_capture_id = it->second.capture_id;
     }
     cudaStream_t st = as_stream(stream);
@@ -435,7 +436,8 @@ int dqrm_train_step_sorted(dqrm_ctx *ctx, float *tables, const int32_t *indices,
         if (captured == sort_captured && (!captured || id == sort_capture_id))
             DQRM_CUDA_TRY(ctx, cudaStreamWaitEvent(ss, sort_done, 0));
     }
-    int rc = dq_launch_bwd_reduce(ctx, grad_out, unique_rows, uniq_off, grad_rows, B, L, workspace, workspace_bytes, ss);
+    int rc = dq_launch_bwd_sum(ctx, grad_out, unique_rows, uniq_off, grad_rows, B, L, by_table, workspace,
+                               workspace_bytes, ss);
     // The forward goes to the context's lowest-priority stream: its many blocks then do not keep the next batch's
     // sort, which a pipelined loop runs on a stream of its own, from getting SMs (with the forward on the caller's
     // high-priority stream the sort's clusters started only when the forward had handed out its last block;
@@ -589,7 +591,8 @@ int dqrm_train_step_host(dqrm_ctx *ctx, float *tables, const int32_t *h_indices,
     DQRM_CUDA_TRY(ctx, cudaStreamWaitEvent(ctx->side, ctx->ev_fork, 0));
     char *step_ws = ws + y.step_ws;
     const size_t step_ws_bytes = workspace_bytes - y.step_ws;
-    int rc = dq_launch_bwd_sort(ctx, d_idx, d_off, d_ur, d_uo, B, L, step_ws, step_ws_bytes, ctx->side, nullptr, true);
+    bool by_table = false;
+    int rc = dq_launch_bwd_sort(ctx, d_idx, d_off, d_ur, d_uo, B, L, step_ws, step_ws_bytes, ctx->side, true, &by_table);
     if (rc == DQRM_OK) rc = dq_launch_fwd(ctx, tables, d_idx, d_off, scales, bits, d_out, nullptr, B, L, st);
     // join every stream even after an error, so that the caller's stream stays ordered behind them
     cudaEventRecord(ctx->ev_h_fwd, st);
@@ -598,7 +601,7 @@ int dqrm_train_step_host(dqrm_ctx *ctx, float *tables, const int32_t *h_indices,
     cudaEventRecord(ctx->ev_h_out, ctx->copy_out);
     // the gradient summation follows the sort on the second stream as soon as the upstream gradient has arrived
     cudaStreamWaitEvent(ctx->side, ctx->ev_h_go, 0);
-    if (rc == DQRM_OK) rc = dq_launch_bwd_reduce(ctx, d_go, d_ur, d_uo, d_gr, B, L, step_ws, step_ws_bytes, ctx->side);
+    if (rc == DQRM_OK) rc = dq_launch_bwd_sum(ctx, d_go, d_ur, d_uo, d_gr, B, L, by_table, step_ws, step_ws_bytes, ctx->side);
     cudaEventRecord(ctx->ev_join, ctx->side);
     cudaStreamWaitEvent(st, ctx->ev_join, 0);
     if (rc == DQRM_OK)

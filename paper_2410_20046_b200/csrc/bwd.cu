@@ -10,15 +10,13 @@
 //                scatter: stable least-significant-digit scatter of (key, payload);
 //                         counts the next pass's tile histogram on the way
 //   seg_count / seg_emit  head flags of the sorted keys -> unique_rows, uniq_off,
-//                         segment starts, first segment of every 32-entry chunk
-//   seg_reduce   one lane group per 32-entry chunk of the sorted order: gathers the
-//                upstream gradient rows (128-bit loads), sums runs in FP64; runs that are
-//                whole segments are rounded and written, runs cut by a chunk boundary
-//                leave an FP64 partial
-//   seg_fixup    one warp per cut segment: adds its partials in a fixed order
+//                         segment starts, first segment of every tile of the sum
+//   seg_sum      every warp walks a range of the sorted order: gathers the upstream gradient rows,
+//                sums runs in FP64, rounds and writes them; of a run that spans ranges every
+//                range leaves an FP64 partial and the last to arrive adds them
 // The sort is stable and every sum has a fixed shape, so results are reproducible bit
 // for bit.  The per-table abs-max of the summed gradient (needed by the INT8 gradient
-// quantiser) is folded into the last two kernels.
+// quantiser) is folded into the last kernel.
 #include "common.cuh"
 #include "seg_reduce.cuh"
 #include "cluster_sort.cuh"
@@ -31,15 +29,15 @@ constexpr int ST_TILE = ST_THREADS * ST_ITEMS;   // 2048 entries per tile
 constexpr int ST_WARPS = ST_THREADS / 32;
 constexpr int NB_MAX = 512;                      // bins per pass (<= 9 bit digits)
 constexpr int HIST_CHUNK = 64;                   // tiles per chunk of the radix sort's offset computation
-constexpr int SEG_CHUNK = segred::CHUNK;         // sorted entries per reduce work item
 
 struct Layout {
     int passes, digit_bits, nb;
-    int ck;                                    // sorted entries per lane group of the reduce: 32, or 16
-    int64_t num_tiles, num_chunks;             // num_chunks = ceil(L / ck)
-    // zeroed at call start: [0, zero_small)
-    size_t absmax, counters, tile_heads, zero_small, digit_base, chunk_sum, tilehist;
-    size_t keys_a, vals_a, pairs_a, pairs_b, seg_start, chunk_first, long_list, partials, table_cnt, tb;
+    int64_t num_tiles;
+    int sum_shift;                             // the summing kernel: log2 of its tile of sorted entries, tiles,
+    int64_t sum_tiles, sum_ranges;             // ranges of range_tiles tiles (at most sum_ranges)
+    int range_tiles;
+    size_t absmax, tile_heads, digit_base, chunk_sum, tilehist;
+    size_t keys_a, vals_a, pairs_a, pairs_b, seg_start, chunk_first, tile_done, partials, table_cnt, tb;
     size_t total;
 };
 
@@ -52,22 +50,18 @@ Layout make_layout(const dqrm_ctx *ctx, int64_t L)
     y.nb = 1 << y.digit_bits;
     int64_t Lc = L < 1 ? 1 : L;
     y.num_tiles = (Lc + ST_TILE - 1) / ST_TILE;
-    // A chunk is walked in order by one lane group.  A batch whose 32-entry chunks would not even give every SM
-    // one block of the reduce takes 16-entry chunks: twice the groups, each half as long (measured: 19 -> 14 us
-    // at batch 128, but 24 -> 29 us at 208 blocks, where the extra pieces cost more than the shorter walks save).
-    y.ck = SEG_CHUNK;
-    {
-        const int D = ctx->D;
-        const int rl = D <= 4 ? 4 : D <= 8 ? 8 : D <= 16 ? 4 : D <= 64 ? 16 : 32;      // lanes per row of the reduce
-        if (rl <= 16 && (Lc / SEG_CHUNK) / (256 / rl) < (int64_t)ctx->num_sms) y.ck = SEG_CHUNK / 2;
-    }
-    y.num_chunks = (Lc + y.ck - 1) / y.ck;
+    // the sum: every warp that the GPU holds at once walks one range of tiles
+    const int lpr = segred::lanes_per_row(ctx->D), I = segred::tile_entries(lpr);
+    y.sum_shift = dq_log2c(I);
+    y.sum_tiles = (Lc + I - 1) >> y.sum_shift;
+    int64_t warps = (int64_t)ctx->num_sms * segred::blocks_per_sm(lpr) / segred::column_blocks(ctx->D) * segred::WARPS;
+    if (warps < 1) warps = 1;
+    y.sum_ranges = y.sum_tiles < warps ? y.sum_tiles : warps;
+    y.range_tiles = (int)((y.sum_tiles + warps - 1) / warps);
     size_t o = 0;
     auto take = [&](size_t bytes) { size_t at = o; o = align_up(o + bytes, 256); return at; };
     y.absmax = take(sizeof(u32) * ctx->T);
-    y.counters = take(sizeof(u32) * 8);
     y.tile_heads = take(sizeof(u32) * y.num_tiles);
-    y.zero_small = o;
     y.digit_base = take(sizeof(u32) * NB_MAX);
     y.chunk_sum = take(sizeof(u32) * y.nb * ((y.num_tiles + HIST_CHUNK - 1) / HIST_CHUNK));
     y.tilehist = take(sizeof(u32) * y.nb * y.num_tiles);
@@ -78,15 +72,12 @@ Layout make_layout(const dqrm_ctx *ctx, int64_t L)
     y.seg_start = take(sizeof(u32) * (Lc + ctx->T + 1));     // (lists by table: one slot more per table)
     y.table_cnt = take(sizeof(u32) * ctx->T);
     y.tb = take(sizeof(u32) * (ctx->T + 1));
-    y.chunk_first = take(sizeof(u32) * y.num_chunks);
-    y.long_list = take(sizeof(uint4) * y.num_chunks);
-    y.partials = take(sizeof(double) * y.num_chunks * 2 * ctx->D);
+    y.chunk_first = take(sizeof(u32) * y.sum_tiles);
+    y.tile_done = take(sizeof(u32) * y.sum_tiles);
+    y.partials = take(sizeof(double) * y.sum_ranges * 2 * ctx->D);
     y.total = o;
     return y;
 }
-
-// counters[]: see segred::CNT_*
-using segred::CNT_U;
 
 // ---------------------------------------------------------------------------------
 // one thread per bag: (arena-row key, gradient-row payload) of every lookup of the bag, as one 8-byte pair:
@@ -305,7 +296,8 @@ __global__ void __launch_bounds__(ST_THREADS)
 seg_emit_kernel(const u32 *__restrict__ keys, int64_t L, const u32 *__restrict__ tile_heads,
                 const int64_t *__restrict__ row_off, int T,
                 u32 *__restrict__ seg_start, u32 *__restrict__ chunk_first,
-                int32_t *__restrict__ unique_rows, int32_t *__restrict__ uniq_off, u32 *__restrict__ counters, int ck)
+                int32_t *__restrict__ unique_rows, int32_t *__restrict__ uniq_off, u32 *__restrict__ tile_done,
+                u32 *__restrict__ absmax, int ck_shift)
 {
     extern __shared__ unsigned char smem_raw[];
     int64_t *s_off = reinterpret_cast<int64_t *>(smem_raw);   // [T+1]
@@ -313,9 +305,11 @@ seg_emit_kernel(const u32 *__restrict__ keys, int64_t L, const u32 *__restrict__
     __shared__ u32 s_prefix;
     // this thread's keys first: they depend on nothing, so they fly beside the loads of the prefix below
     const int64_t i0 = (int64_t)blockIdx.x * ST_TILE + (int64_t)threadIdx.x * ST_ITEMS;
-    const int ck_shift = 31 - __clz(ck);
+    const int ck = 1 << ck_shift;
     u32 k[ST_ITEMS], prev0; int n;
     load_tile_keys(keys, L, i0, k, prev0, n);
+    if (blockIdx.x == 0)
+        for (int t = threadIdx.x; t < T; t += ST_THREADS) absmax[t] = 0u;
     for (int t = threadIdx.x; t <= T; t += ST_THREADS) s_off[t] = row_off[t];
     // heads in all earlier tiles
     u32 p = 0;
@@ -382,12 +376,14 @@ seg_emit_kernel(const u32 *__restrict__ keys, int64_t L, const u32 *__restrict__
                 t_prev = t;
             }
             const u32 u_of_i = heads_before - 1;
-            if ((i & (int64_t)(ck - 1)) == 0) chunk_first[i >> ck_shift] = u_of_i;     // ck is 16 or 32
+            if ((i & (int64_t)(ck - 1)) == 0) {
+                chunk_first[i >> ck_shift] = u_of_i;
+                tile_done[i >> ck_shift] = 0u;
+            }
             if (i == L - 1) {
                 const u32 U = u_of_i + 1;
                 seg_start[U] = (u32)L;
                 for (int tt = t_prev + 1; tt <= T; ++tt) uniq_off[tt] = (int32_t)U;
-                counters[CNT_U] = U;
             }
         }
         prev = k[e];
@@ -395,62 +391,17 @@ seg_emit_kernel(const u32 *__restrict__ keys, int64_t L, const u32 *__restrict__
 }
 
 // ---------------------------------------------------------------------------------
-// RL/RV/RC: lanes per row, floats per lane vector and vectors per lane of the reduce kernel;
-// LPR/CH: the same for the fix-up kernels (always 128-bit vectors)
-template <int RL, int RV, int RC, int LPR, int CH>
-int launch_reduce(dqrm_ctx *ctx, const Layout &y, char *ws, const u32 *keys, const u32 *vals, int32_t *unique_rows,
-                  int32_t *uniq_off, const float *grad_out, float *grad_rows, int64_t L, int64_t G, cudaStream_t st)
+template <int LPR, int VEC>
+int launch_sum(dqrm_ctx *ctx, const segred::Args &a, cudaStream_t st)
 {
     using namespace segred;
-    const int64_t cap = (int64_t)ctx->num_sms * 8;
-    const int64_t gpb = 256 / RL;                            // one lane group per chunk
-    int64_t blocks = (y.num_chunks + gpb - 1) / gpb;
-    int grid = (int)(blocks < 1 ? 1 : (blocks > cap ? cap : blocks));
-    u32 *counters = reinterpret_cast<u32 *>(ws + y.counters);
-    u32 *absmax = reinterpret_cast<u32 *>(ws + y.absmax);
-    const u32 *seg_start = reinterpret_cast<const u32 *>(ws + y.seg_start);
-    double *partials = reinterpret_cast<double *>(ws + y.partials);
-    uint4 *long_list = reinterpret_cast<uint4 *>(ws + y.long_list);
-    const size_t red_smem = (size_t)(ctx->T + 1) * 3 * sizeof(u32) + (size_t)gpb * 2 * y.ck * sizeof(u32);
-    ByTable bt;
-    bt.table_cnt = reinterpret_cast<const u32 *>(ws + y.table_cnt);
-    bt.tb = reinterpret_cast<const u32 *>(ws + y.tb);
-    bt.row_off = ctx->d_row_off;
-    bt.unique_rows = unique_rows;
-    bt.uniq_off = uniq_off;
-    const u32 *chunk_first = reinterpret_cast<const u32 *>(ws + y.chunk_first);
-#define DQ_LAUNCH_REDUCE(EXACT, CK)                                                                                  \
-    seg_reduce_kernel<RL, RV, RC, EXACT, CK><<<grid, 256, red_smem, st>>>(                                          \
-        keys, vals, seg_start, chunk_first, uniq_off, grad_out, grad_rows, partials, long_list, counters, absmax,    \
-        ctx->T, ctx->D, L, G, y.num_chunks, ctx->d_status, bt)
-    const bool exact = ctx->D == RL * RV * RC;
-    if constexpr (RL <= 16) {
-        if (y.ck == SEG_CHUNK / 2) {
-            if (exact) DQ_LAUNCH_REDUCE(true, SEG_CHUNK / 2); else DQ_LAUNCH_REDUCE(false, SEG_CHUNK / 2);
-        } else {
-            if (exact) DQ_LAUNCH_REDUCE(true, SEG_CHUNK); else DQ_LAUNCH_REDUCE(false, SEG_CHUNK);
-        }
-    } else {
-        if (exact) DQ_LAUNCH_REDUCE(true, SEG_CHUNK); else DQ_LAUNCH_REDUCE(false, SEG_CHUNK);
-    }
-#undef DQ_LAUNCH_REDUCE
+    const size_t smem = smem_bytes(ctx->T);
+    const int64_t ranges = (a.num_tiles + a.range_tiles - 1) / a.range_tiles;
+    const dim3 grid((unsigned)((ranges + WARPS - 1) / WARPS), (unsigned)column_blocks(ctx->D));
+    if (ctx->D == LPR * VEC) seg_sum_kernel<LPR, VEC, true><<<grid, THREADS, smem, st>>>(a);
+    else seg_sum_kernel<LPR, VEC, false><<<grid, THREADS, smem, st>>>(a);
     DQRM_CUDA_TRY(ctx, cudaGetLastError());
-    dq_mark(ctx, st, DQ_K_SEG_REDUCE);
-    int64_t fblocks = (y.num_chunks + 7) / 8;                // at most one cut segment per chunk, a warp each
-    int fgrid = (int)(fblocks < (int64_t)ctx->num_sms * 4 ? (fblocks < 1 ? 1 : fblocks) : (int64_t)ctx->num_sms * 4);
-    const size_t fix_smem = (size_t)(256 / LPR) * ctx->D * sizeof(double);
-    if (fix_smem > 48 * 1024) {
-        bool &raised = ctx->smem_raised[dq_smem_slot_fixup(LPR, CH)];
-        if (!raised) {
-            DQRM_CUDA_TRY(ctx, cudaFuncSetAttribute(seg_fixup_kernel<LPR, CH>,
-                                                    cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fix_smem));
-            raised = true;
-        }
-    }
-    seg_fixup_kernel<LPR, CH><<<fgrid, 256, fix_smem, st>>>(partials, long_list, counters, grad_rows, absmax, ctx->D,
-                                                            y.num_chunks);
-    DQRM_CUDA_TRY(ctx, cudaGetLastError());
-    dq_mark(ctx, st, DQ_K_SEG_FIXUP);
+    dq_mark(ctx, st, DQ_K_SEG_SUM);
     return DQRM_OK;
 }
 
@@ -507,19 +458,18 @@ size_t dq_bwd_ws_bytes(const dqrm_ctx *ctx, int64_t L, int64_t G)
 // segment starts).  It needs no upstream gradient, so a training step runs it beside the forward.
 int dq_launch_bwd_sort(dqrm_ctx *ctx, const int32_t *indices, const int32_t *offsets,
                        int32_t *unique_rows, int32_t *uniq_off, int B, int64_t L,
-                       void *ws_, size_t ws_bytes, cudaStream_t st, const u32 **absmax_bits_out, bool lists_by_table)
+                       void *ws_, size_t ws_bytes, cudaStream_t st, bool lists_by_table, bool *by_table)
 {
     const Layout y = make_layout(ctx, L);
     if (ws_bytes < y.total) return DQRM_ERR_WORKSPACE;
     char *ws = reinterpret_cast<char *>(ws_);
     const int64_t G = (int64_t)ctx->T * B;
-    if (absmax_bits_out) *absmax_bits_out = reinterpret_cast<const u32 *>(ws + y.absmax);
+    if (by_table) *by_table = false;
     const bool fits_cluster = (L + ctx->T - 1) / ctx->T <= (int64_t)csort::CLUSTER * 12288;   // (a table beyond its
     // blocks' shared memory still sorts, through global staging, but slowly)
     const bool try_cluster = ctx->sort_path != 1 && fits_cluster;
-    DQRM_CUDA_TRY(ctx, cudaMemsetAsync(ws, 0, y.zero_small, st));
-    dq_mark(ctx, st, DQ_K_MEMSET);
     if (L == 0) {
+        DQRM_CUDA_TRY(ctx, cudaMemsetAsync(ws + y.absmax, 0, sizeof(u32) * ctx->T, st));
         DQRM_CUDA_TRY(ctx, cudaMemsetAsync(uniq_off, 0, sizeof(int32_t) * (ctx->T + 1), st));
         return DQRM_OK;
     }
@@ -532,6 +482,10 @@ int dq_launch_bwd_sort(dqrm_ctx *ctx, const int32_t *indices, const int32_t *off
     bool sorted = false;
     // (tables far beyond the shared-memory slices sort faster with the global radix sort)
     if (try_cluster) {
+        if (!lists_by_table) {
+            DQRM_CUDA_TRY(ctx, cudaMemsetAsync(ws + y.tile_heads, 0, sizeof(u32) * y.num_tiles, st));
+            dq_mark(ctx, st, DQ_K_MEMSET);
+        }
         // one cluster of eight blocks per table (sixteen when so few tables would leave most SMs idle); falls
         // through to the narrower cluster, then to the global radix sort, if a launch is refused
         csort::Args ca;
@@ -549,9 +503,10 @@ int dq_launch_bwd_sort(dqrm_ctx *ctx, const int32_t *indices, const int32_t *off
         ca.chunk_first = reinterpret_cast<u32 *>(ws + y.chunk_first);
         ca.table_cnt = reinterpret_cast<u32 *>(ws + y.table_cnt);
         ca.tb = reinterpret_cast<u32 *>(ws + y.tb);
-        ca.counters = reinterpret_cast<u32 *>(ws + y.counters);
-        ca.ck_shift = y.ck == SEG_CHUNK ? 5 : 4;
-        ca.fmt_slot = segred::CNT_FMT; ca.fmt_by_table = segred::LISTS_BY_TABLE; ca.fmt_broken = segred::LISTS_BROKEN;
+        ca.tile_done = reinterpret_cast<u32 *>(ws + y.tile_done);
+        ca.absmax = reinterpret_cast<u32 *>(ws + y.absmax);
+        ca.ck_shift = y.sum_shift;
+        ca.cnt_broken = segred::CNT_BROKEN;
         const int64_t per_table = (L + ctx->T - 1) / ctx->T;
         const bool wide = ctx->T * csort::CLUSTER_WIDE * 2 <= ctx->num_sms && per_table >= csort::CLUSTER_WIDE * 1024;
         cudaError_t e = cudaErrorUnknown;
@@ -599,7 +554,10 @@ int dq_launch_bwd_sort(dqrm_ctx *ctx, const int32_t *indices, const int32_t *off
     }
         skeys = keys[0];
     }
-    if (sorted && lists_by_table) return DQRM_OK;      // the lists are there; unique_rows and uniq_off come with the sums
+    if (sorted && lists_by_table) {                    // the lists are there; unique_rows and uniq_off come with the sums
+        if (by_table) *by_table = true;
+        return DQRM_OK;
+    }
     if (!sorted) {        // (a cluster sort that did not number the segments itself has counted the segment heads of every tile)
         seg_count_kernel<<<(unsigned)y.num_tiles, ST_THREADS, 0, st>>>(skeys, L, reinterpret_cast<u32 *>(ws + y.tile_heads));
         DQRM_CUDA_TRY(ctx, cudaGetLastError());
@@ -608,43 +566,54 @@ int dq_launch_bwd_sort(dqrm_ctx *ctx, const int32_t *indices, const int32_t *off
     seg_emit_kernel<<<(unsigned)y.num_tiles, ST_THREADS, (size_t)(ctx->T + 1) * sizeof(int64_t), st>>>(
         skeys, L, reinterpret_cast<const u32 *>(ws + y.tile_heads), ctx->d_row_off, ctx->T,
         reinterpret_cast<u32 *>(ws + y.seg_start), reinterpret_cast<u32 *>(ws + y.chunk_first), unique_rows, uniq_off,
-        reinterpret_cast<u32 *>(ws + y.counters), y.ck);
+        reinterpret_cast<u32 *>(ws + y.tile_done), reinterpret_cast<u32 *>(ws + y.absmax), y.sum_shift);
     DQRM_CUDA_TRY(ctx, cudaGetLastError());
     dq_mark(ctx, st, DQ_K_SEG_EMIT);
     return DQRM_OK;
 }
 
 // second half: segmented sum of the upstream gradient over the sorted lookups
-int dq_launch_bwd_reduce(dqrm_ctx *ctx, const float *grad_out, int32_t *unique_rows, int32_t *uniq_off, float *grad_rows,
-                         int B, int64_t L, void *ws_, size_t ws_bytes, cudaStream_t st)
+int dq_launch_bwd_sum(dqrm_ctx *ctx, const float *grad_out, int32_t *unique_rows, int32_t *uniq_off, float *grad_rows,
+                      int B, int64_t L, bool by_table, void *ws_, size_t ws_bytes, cudaStream_t st)
 {
     const Layout y = make_layout(ctx, L);
     if (ws_bytes < y.total) return DQRM_ERR_WORKSPACE;
     if (L == 0) return DQRM_OK;
     char *ws = reinterpret_cast<char *>(ws_);
-    const int64_t G = (int64_t)ctx->T * B;
+    segred::Args a = {};
     // both sort paths leave the sorted pairs in the first key / payload buffers
-    const u32 *skeys = reinterpret_cast<const u32 *>(ws + y.keys_a), *svals = reinterpret_cast<const u32 *>(ws + y.vals_a);
-    const int D = ctx->D, d4 = D / 4;
-#define DQ_RED(RL, RV, RC, LPR, CH) \
-    return launch_reduce<RL, RV, RC, LPR, CH>(ctx, y, ws, skeys, svals, unique_rows, uniq_off, grad_out, grad_rows, L, G, st)
-    if (D <= 4) DQ_RED(4, 1, 1, 1, 1);
-    if (D <= 8) DQ_RED(8, 1, 1, 2, 1);
-    if (D <= 16) DQ_RED(4, 4, 1, 4, 1);
-    if (D <= 32) DQ_RED(16, 2, 1, 8, 1);
-    if (D <= 64) DQ_RED(16, 4, 1, 16, 1);
-    if (d4 <= 32) DQ_RED(32, 4, 1, 32, 1);
-    if (d4 <= 64) DQ_RED(32, 4, 2, 32, 2);
-    if (d4 <= 128) DQ_RED(32, 4, 4, 32, 4);
-    DQ_RED(32, 4, 8, 32, 8);
-#undef DQ_RED
+    a.keys = reinterpret_cast<const u32 *>(ws + y.keys_a);
+    a.vals = reinterpret_cast<const u32 *>(ws + y.vals_a);
+    a.seg_start = reinterpret_cast<const u32 *>(ws + y.seg_start);
+    a.chunk_first = reinterpret_cast<const u32 *>(ws + y.chunk_first);
+    a.range_done = reinterpret_cast<u32 *>(ws + y.tile_done);
+    a.by_table = by_table ? 1 : 0;
+    a.table_cnt = reinterpret_cast<const u32 *>(ws + y.table_cnt);
+    a.tb = reinterpret_cast<const u32 *>(ws + y.tb);
+    a.row_off = ctx->d_row_off;
+    a.unique_rows = unique_rows; a.uniq_off = uniq_off;
+    a.grad_out = grad_out; a.grad_rows = grad_rows;
+    a.partials = reinterpret_cast<double *>(ws + y.partials);
+    a.absmax = reinterpret_cast<u32 *>(ws + y.absmax);
+    a.T = ctx->T; a.D = ctx->D;
+    a.L = L; a.G = (int64_t)ctx->T * B; a.num_tiles = y.sum_tiles;
+    a.range_tiles = y.range_tiles;
+    a.status = ctx->d_status;
+    const int D = ctx->D;
+    if (D <= 4) return launch_sum<4, 1>(ctx, a, st);
+    if (D <= 8) return launch_sum<4, 2>(ctx, a, st);
+    if (D <= 16) return launch_sum<4, 4>(ctx, a, st);
+    if (D <= 32) return launch_sum<8, 4>(ctx, a, st);
+    if (D <= 64) return launch_sum<32, 2>(ctx, a, st);
+    return launch_sum<32, 4>(ctx, a, st);
 }
 
 int dq_launch_bwd(dqrm_ctx *ctx, const float *grad_out, const int32_t *indices, const int32_t *offsets,
                   int32_t *unique_rows, int32_t *uniq_off, float *grad_rows, int B, int64_t L,
-                  void *ws, size_t ws_bytes, cudaStream_t st, const u32 **absmax_bits_out)
+                  void *ws, size_t ws_bytes, cudaStream_t st)
 {
-    int rc = dq_launch_bwd_sort(ctx, indices, offsets, unique_rows, uniq_off, B, L, ws, ws_bytes, st, absmax_bits_out, true);
+    bool by_table = false;
+    int rc = dq_launch_bwd_sort(ctx, indices, offsets, unique_rows, uniq_off, B, L, ws, ws_bytes, st, true, &by_table);
     if (rc != DQRM_OK) return rc;
-    return dq_launch_bwd_reduce(ctx, grad_out, unique_rows, uniq_off, grad_rows, B, L, ws, ws_bytes, st);
+    return dq_launch_bwd_sum(ctx, grad_out, unique_rows, uniq_off, grad_rows, B, L, by_table, ws, ws_bytes, st);
 }

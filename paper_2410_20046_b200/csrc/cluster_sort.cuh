@@ -48,10 +48,13 @@ struct Args {
     //   seg_start[tb0 + t + u] = sorted position where the table's segment u begins, [.. + count] = the table's end
     //   chunk_first[c]         = the table's segment that holds sorted entry c << ck_shift (for c inside the table)
     //   table_cnt[t], tb[t]    = segments and first sorted position of table t (tb[T] = L)
-    // and counters[fmt_slot] says so; the kernel that sums the segments adds the tables' bases
+    //                            (cnt_broken instead when boundary offsets are unusable)
+    // and zeroes what the kernel behind it counts in (tile_done[c], absmax[t]); that kernel, which sums the segments,
+    // adds the tables' bases
     int lists_by_table;
-    u32 *seg_start, *chunk_first, *table_cnt, *tb, *counters;
-    int ck_shift, fmt_slot, fmt_by_table, fmt_broken;
+    u32 *seg_start, *chunk_first, *table_cnt, *tb, *tile_done, *absmax;
+    int ck_shift;
+    u32 cnt_broken;
 };
 
 __device__ __forceinline__ u32 *remote(cg::cluster_group &cluster, u32 *p, unsigned rank)
@@ -88,10 +91,11 @@ cluster_sort_kernel(const Args a)
     const u32 lt = (1u << lane) - 1u;
 
     int64_t tb0 = __ldg(a.offsets + (int64_t)t * a.B), tb1 = __ldg(a.offsets + (int64_t)(t + 1) * a.B);
-    if (tb0 < 0 || tb1 < tb0 || tb1 > a.L) {
+    if (tb0 < 0 || tb1 < tb0 || tb1 > a.L ||
+        (a.lists_by_table && ((t == 0 && tb0 != 0) || (t == a.T - 1 && tb1 != a.L)))) {
         if (threadIdx.x == 0 && c == 0) {
             dq_report(a.status, DQRM_ERR_INDEX_RANGE);
-            if (a.lists_by_table) atomicMax(&a.counters[a.fmt_slot], (u32)a.fmt_broken);   // nothing downstream runs
+            if (a.lists_by_table) a.table_cnt[t] = a.cnt_broken;       // nothing downstream runs
         }
         return;                                    // uniform over the cluster
     }
@@ -99,7 +103,7 @@ cluster_sort_kernel(const Args a)
     if (a.lists_by_table && c == 0 && threadIdx.x == 0) {
         a.tb[t] = (u32)tb0;
         if (t == a.T - 1) a.tb[a.T] = (u32)tb1;
-        if (t == 0) atomicMax(&a.counters[a.fmt_slot], (u32)a.fmt_by_table);
+        a.absmax[t] = 0u;
         if (n == 0) a.table_cnt[t] = 0u;
     }
     if (n == 0) return;
@@ -359,7 +363,10 @@ cluster_sort_kernel(const Args a)
                 if (i < w1) {
                     const u32 upto = before_me + __popc(m & (lt | (1u << lane)));     // segment starts in [0, i]
                     if (head) segs[upto - 1] = (u32)j;
-                    if (((u32)j & ck_mask) == 0u) a.chunk_first[j >> a.ck_shift] = upto - 1;
+                    if (((u32)j & ck_mask) == 0u) {
+                        a.chunk_first[j >> a.ck_shift] = upto - 1;
+                        a.tile_done[j >> a.ck_shift] = 0u;
+                    }
                 }
                 before_me += __popc(m);
             }

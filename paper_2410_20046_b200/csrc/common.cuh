@@ -44,6 +44,7 @@ struct dqrm_ctx {
         int64_t L = 0;
         int B = 0;
         cudaEvent_t done = nullptr;
+        bool by_table = false;          // how the sort left its lists (dq_launch_bwd_sort)
         bool captured = false;
         unsigned long long capture_id = 0;
     };
@@ -63,8 +64,8 @@ struct dqrm_ctx {
 
 enum {
     DQ_K_BEGIN = 0, DQ_K_REFRESH, DQ_K_FWD, DQ_K_MEMSET, DQ_K_PREPARE, DQ_K_SORT_SCAN, DQ_K_SORT_SCATTER,
-    DQ_K_SEG_COUNT, DQ_K_SEG_EMIT, DQ_K_SEG_REDUCE, DQ_K_SEG_FIXUP, DQ_K_ABSMAX, DQ_K_QUANT, DQ_K_UPDATE,
-    DQ_K_QUANT_UPDATE, DQ_K_COPY, DQ_K_SEG_FIXUP_BIG, DQ_K_CLUSTER_SORT, DQ_K_DP_PACK, DQ_K_DP_SUM_UPDATE, DQ_K_PACK, DQ_K_PACKED_FWD, DQ_K_FWD_CODES, DQ_K_DECODE_PAYLOAD, DQ_K_COUNT
+    DQ_K_SEG_COUNT, DQ_K_SEG_EMIT, DQ_K_SEG_SUM, DQ_K_ABSMAX, DQ_K_QUANT, DQ_K_UPDATE,
+    DQ_K_QUANT_UPDATE, DQ_K_COPY, DQ_K_CLUSTER_SORT, DQ_K_DP_PACK, DQ_K_DP_SUM_UPDATE, DQ_K_PACK, DQ_K_PACKED_FWD, DQ_K_FWD_CODES, DQ_K_DECODE_PAYLOAD, DQ_K_COUNT
 };
 constexpr int DQ_PROF_MAX = 4096;
 
@@ -94,7 +95,6 @@ static inline size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; 
 // slots of dqrm_ctx::smem_raised
 constexpr int DQ_SMEM_SLOT_CSORT = 24;
 constexpr int dq_log2c(int x) { return x <= 1 ? 0 : 1 + dq_log2c(x / 2); }
-constexpr int dq_smem_slot_fixup(int lpr, int ch) { return dq_log2c(lpr) * 4 + dq_log2c(ch); }
 
 // ---------------------------------------------------------------------------------
 // quantiser arithmetic: each operation is one IEEE round-to-nearest FP32 operation
@@ -181,16 +181,6 @@ __device__ __forceinline__ void dq_fq4(const float4 &v, const QuantScale &q, flo
 }
 
 
-// 16-byte asynchronous copy global -> shared (data never passes through registers)
-__device__ __forceinline__ void dq_cp_async16(void *smem_dst, const void *gmem_src)
-{
-    unsigned d = (unsigned)__cvta_generic_to_shared(smem_dst);
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 16;\n" ::"r"(d), "l"(gmem_src) : "memory");
-}
-__device__ __forceinline__ void dq_cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
-template <int N>
-__device__ __forceinline__ void dq_cp_async_wait() { asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory"); }
-
 // asks L2 for the 128-byte line that holds p (no register, no scoreboard entry: the later load finds it there)
 __device__ __forceinline__ void dq_prefetch_l2(const void *p) { asm volatile("prefetch.global.L2 [%0];\n" ::"l"(p)); }
 
@@ -202,7 +192,19 @@ __device__ __forceinline__ uint64_t dq_policy_evict_last()
     asm volatile("createpolicy.fractional.L2::evict_last.b64 %0, 1.0;\n" : "=l"(pol));
     return pol;
 }
-__device__ __forceinline__ float4 dq_ld_nc_keep(const float4 *p, uint64_t pol)
+__device__ __forceinline__ uint64_t dq_policy_evict_first()
+{
+    uint64_t pol;
+    asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;\n" : "=l"(pol));
+    return pol;
+}
+__device__ __forceinline__ uint64_t dq_policy_evict_normal()
+{
+    uint64_t pol;
+    asm volatile("createpolicy.fractional.L2::evict_normal.b64 %0, 1.0;\n" : "=l"(pol));
+    return pol;
+}
+__device__ __forceinline__ float4 dq_ld_nc(const float4 *p, uint64_t pol)
 {
     float4 v;
     asm volatile("ld.global.nc.L2::cache_hint.v4.f32 {%0, %1, %2, %3}, [%4], %5;\n"
@@ -268,21 +270,20 @@ int dq_launch_fwd(dqrm_ctx *ctx, const float *tables, const int32_t *indices, co
 
 size_t dq_bwd_ws_bytes(const dqrm_ctx *ctx, int64_t L, int64_t G);
 // per-table |grad| maxima (float bit patterns) inside a workspace that dq_launch_bwd_sort and
-// dq_launch_bwd_reduce have filled
+// dq_launch_bwd_sum have filled
 const u32 *dq_bwd_absmax_bits(const dqrm_ctx *ctx, int64_t L, const void *ws);
-// absmax_bits_out: device pointer (inside ws) to per-table |grad| maxima as float bit patterns
 int dq_launch_bwd(dqrm_ctx *ctx, const float *grad_out, const int32_t *indices, const int32_t *offsets,
                   int32_t *unique_rows, int32_t *uniq_off, float *grad_rows, int B, int64_t L,
-                  void *ws, size_t ws_bytes, cudaStream_t st, const u32 **absmax_bits_out);
+                  void *ws, size_t ws_bytes, cudaStream_t st);
 
-// lists_by_table: dq_launch_bwd_reduce follows on the same workspace; the cluster sort then numbers each table's
-// segments itself, no separate kernel numbers them over the batch, and unique_rows / uniq_off are written by
-// dq_launch_bwd_reduce.  Without it they are complete when the sort is.
+// lists_by_table: dq_launch_bwd_sum follows on the same workspace; the cluster sort then numbers each table's
+// segments itself (*by_table says whether it did), no separate kernel numbers them over the batch, and unique_rows /
+// uniq_off are written by dq_launch_bwd_sum.  Without it they are complete when the sort is.
 int dq_launch_bwd_sort(dqrm_ctx *ctx, const int32_t *indices, const int32_t *offsets, int32_t *unique_rows,
                        int32_t *uniq_off, int B, int64_t L, void *ws, size_t ws_bytes, cudaStream_t st,
-                       const u32 **absmax_bits_out, bool lists_by_table = false);
-int dq_launch_bwd_reduce(dqrm_ctx *ctx, const float *grad_out, int32_t *unique_rows, int32_t *uniq_off,
-                         float *grad_rows, int B, int64_t L, void *ws, size_t ws_bytes, cudaStream_t st);
+                       bool lists_by_table, bool *by_table);
+int dq_launch_bwd_sum(dqrm_ctx *ctx, const float *grad_out, int32_t *unique_rows, int32_t *uniq_off, float *grad_rows,
+                      int B, int64_t L, bool by_table, void *ws, size_t ws_bytes, cudaStream_t st);
 
 size_t dq_quant_ws_bytes(const dqrm_ctx *ctx);
 int dq_launch_grad_absmax(dqrm_ctx *ctx, const float *grad_rows, const int32_t *uniq_off, float *absmax,

@@ -153,7 +153,7 @@ fwd_onehot_kernel(const FwdArgs a)
                 for (int b = 0; b < NB; ++b) {
                     const int bag = k0 + b * RPW + grp;
                     if (bag < 32 && ((one >> bag) & 1u) && (EXACT || c4 < d4))
-                        v[b] = dq_ld_nc_keep(tbl_lane + (int64_t)ib[b] * d4 + c * LPR, keep);   // the update reads the row again
+                        v[b] = dq_ld_nc(tbl_lane + (int64_t)ib[b] * d4 + c * LPR, keep);   // the update reads the row again
                 }
 #pragma unroll
                 for (int b = 0; b < NB; ++b) {

@@ -1,602 +1,480 @@
-// Segmented reduction of the upstream gradient over the sorted lookups (second half of
-// the backward; paper Section 4.3 / Appendix B.1: duplicates of a row are coalesced).
+// Segmented sum of the upstream gradient over the sorted lookups (second half of the backward; paper
+// Section 4.3 / Appendix B.1: duplicates of a row are coalesced).
 //
-// Input: keys[L] (arena rows, ascending), vals[L] (row of grad_out for each lookup, in
-// stable order), chunk_first[c] = index of the segment that holds sorted entry 32*c,
-// seg_start[] = sorted position where every segment begins; the segments are numbered over
-// the whole batch or per table (see LISTS_* below), and in the second case this kernel also
-// writes unique_rows and uniq_off.  Work is dealt in chunks of 32 sorted entries, one lane group per chunk,
-// but a segment is summed by the group in whose chunk it BEGINS, tail in the next chunk
-// included; the group sees where that tail ends from the next chunk's keys, which it loads
-// with its own.  All sums are FP64 and have a shape fixed by the entry positions, so results
-// are reproducible.  Only a segment whose tail is not over within the next chunk (a hot row)
-// is summed in pieces: every chunk it covers leaves an FP64 partial and the segment is
-// finished by one of the fix-up kernels (a warp for up to 32 pieces, a block beyond that).
-// The per-table abs-max of the rounded sums is collected on the way.
+// Input: keys[L] (arena rows, ascending), vals[L] (row of grad_out for each lookup, in stable order),
+// chunk_first[c] = index of the segment that holds sorted entry c*I, seg_start[] = sorted position where
+// every segment begins; the segments are numbered over the whole batch, or per table (Args::by_table), and
+// in the second case this kernel also writes unique_rows and uniq_off.
+//
+// A warp walks a contiguous range of the sorted order by itself (no block barrier inside the walk), a tile of I
+// entries at a time.  The sum is bound by the latency of the chain index -> payload -> row: indices are fetched a
+// tile ahead, the rows of the next tile are asked into L2 as soon as its payloads are there (without that the kernel
+// took 89 instead of 71 us on 852 K rows of 256 bytes, 541 instead of 318 us on 8.5 M), and the next batch of rows is
+// requested before the present one is summed.  A row takes LPR lanes with VEC features each.  Rows of 36 features and
+// more take the whole warp: every branch on a run's end is then uniform and a run that goes on is simply carried in
+// registers.  Narrower rows are taken by 32/LPR lane groups at once, C consecutive entries each; a segmented scan over
+// the groups (shuffles) joins the runs that cross them.  Only a run cut by the edge of a warp's range leaves a partial
+// in global memory; the warp that brings a run's last partial adds all of them, in order (nobody waits).  All sums are
+// FP64 and have a shape fixed by the entry positions and the launch, so results are reproducible.  The per-table
+// abs-max of the rounded sums is collected on the way.
+//
+// Measured on B200 (cold L2, alone) against the kernel before it, which walked 32-entry chunks per lane group and left
+// a partial per chunk for a second launch: 426 K rows of 64 bytes 26.7 + 10.6 -> 25.4 us, 852 K rows of 256 bytes
+// 69.9 + 12.9 -> 70.9 us, 8.5 M lookups of 256-byte rows 330 + 63 -> 318 us.
 #pragma once
-#include <type_traits>
 #include "common.cuh"
 
 namespace segred {
 
-constexpr int CHUNK = 32;            // sorted entries per lane group of the reduce (16 for a small batch of narrow rows)
-constexpr int PREFETCH_ROW_BYTES = 512;   // rows up to this size are prefetched into L2 by the reduce's head phase
-constexpr int BIG_PIECES = 32;       // cut segments with more pieces go to the block-wide fix-up
-enum { CNT_LONG = 0, CNT_U = 1, CNT_BIG = 2, CNT_FMT = 3 };
-// counters[CNT_FMT]: how the segment lists that the sort left are laid out.
-//   LISTS_GLOBAL    seg_start[u], chunk_first[c] and uniq_off[] number the segments over the whole batch (seg_emit)
-//   LISTS_BY_TABLE  the cluster sort numbered each table's segments from 0: table t's starts sit at
-//                   seg_start[tb[t] + t + .] (tb[t] = first sorted position of the table, one slot more than it
-//                   has segments: the last holds the table's end), chunk_first[c] counts within the table that
-//                   holds entry c*CK, table_cnt[t] says how many segments the table has; unique_rows and
-//                   uniq_off are then written by the reduce, which adds the tables' bases
-//   LISTS_BROKEN    a table's boundary offsets were unusable (reported): nothing is summed, no row is updated
-enum { LISTS_GLOBAL = 0, LISTS_BY_TABLE = 1, LISTS_BROKEN = 2 };
-struct ByTable {
-    const u32 *table_cnt;       // [T]
-    const u32 *tb;              // [T+1]
-    const int64_t *row_off;     // [T+1]
-    int32_t *unique_rows;       // [U] out
-    int32_t *uniq_off;          // [T+1] out
+constexpr int THREADS = 256;
+constexpr int WARPS = THREADS / 32;
+constexpr u32 CNT_BROKEN = 0xFFFFFFFFu;      // table_cnt[t]: the table's boundary offsets were unusable (reported)
+
+// lanes per row and features per lane for feature size D (D > 128: 128 features per block of the grid's y)
+__host__ __device__ constexpr int lanes_per_row(int D) { return D <= 16 ? 4 : D <= 32 ? 8 : 32; }
+__host__ __device__ constexpr int floats_per_lane(int D) { return D <= 4 ? 1 : D <= 8 ? 2 : D <= 32 ? 4 : D <= 64 ? 2 : 4; }
+__host__ __device__ constexpr int column_blocks(int D) { return (D + 127) / 128; }
+// rows of a lane group in flight, entries of a tile, resident blocks.  Lane groups: eight rows and two blocks (with
+// three the kernel spills and takes 31 us instead of 25 at 426 K rows of 64 bytes); whole warps: 4 KB in flight (two
+// batches in turn) and three blocks (four blocks: 78 instead of 71 us at 852 K rows of 256 bytes)
+__host__ __device__ constexpr int batch_entries(int lpr, int vec) { return lpr == 32 ? 16 / vec : 8; }
+__host__ __device__ constexpr int tile_entries(int lpr) { return lpr == 4 ? 64 : 32; }
+__host__ __device__ constexpr int blocks_per_sm(int lpr) { return lpr == 32 ? 3 : 2; }
+
+struct Args {
+    const u32 *keys, *vals, *seg_start, *chunk_first;
+    u32 *range_done;            // [ranges] zero: partials that have arrived for the run that begins in a range
+    // by_table: the cluster sort numbered each table's segments from 0: table t's starts sit at
+    // seg_start[tb[t] + t + .] (tb[t] = first sorted position of the table, one slot more than it has segments: the
+    // last holds the table's end), chunk_first[c] counts within the table that holds entry c*I, table_cnt[t] says
+    // how many segments the table has (CNT_BROKEN: nothing is summed, no row is updated); unique_rows and uniq_off
+    // are then written here, with the tables' bases added
+    int by_table;
+    const u32 *table_cnt, *tb;
+    const int64_t *row_off;
+    int32_t *unique_rows, *uniq_off;
+    const float *grad_out;
+    float *grad_rows;
+    double *partials;           // [ranges][2][D]: run that enters the range, run that leaves it
+    u32 *absmax;                // [T] zero
+    int T, D;
+    int64_t L, G, num_tiles;
+    int range_tiles;            // tiles per warp
+    int *status;
 };
 
-template <int LPR>
-__device__ __forceinline__ u32 group_mask()
+inline size_t smem_bytes(int T) { return (size_t)(T + 1) * 3 * sizeof(u32); }
+
+// largest t in [lo, T) with list[t] <= x (list ascends; of tables that share a start, the last)
+__device__ __forceinline__ int last_not_above(const u32 *list, int lo, int T, u32 x)
 {
-    if constexpr (LPR >= 32) {
-        return 0xffffffffu;
-    } else {
-        const int lane = threadIdx.x & 31;
-        return ((1u << LPR) - 1u) << (lane / LPR * LPR);
+    int hi = T;
+    while (hi - lo > 1) {
+        const int mid = (lo + hi) >> 1;
+        if (list[mid] <= x) lo = mid; else hi = mid;
     }
+    return lo;
 }
 
-template <int LPR>
-__device__ __forceinline__ float group_max(float m)
-{
-    const u32 gm = group_mask<LPR>();
-#pragma unroll
-    for (int o = LPR / 2; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(gm, m, o));
-    return m;
-}
-
-// running abs-max of one table at a time (segment numbers only ascend along a lane group's work)
-struct AbsmaxTracker {
-    int t = -1;
-    u32 u_end = 0;          // first segment past table t
-    float m = 0.f;
-};
-
-template <int LPR>
-__device__ __forceinline__ void absmax_push(AbsmaxTracker &tr, u32 *absmax)
-{
-    float m = group_max<LPR>(tr.m);      // called group-uniformly
-    if ((threadIdx.x % LPR) == 0 && tr.t >= 0 && m > 0.f) atomicMax(&absmax[tr.t], __float_as_uint(m));
-    tr.m = 0.f;
-}
-
-// s_uoff[t] = first segment (unique row) of table t, s_uoff[T] = number of segments
-template <int LPR>
-__device__ __forceinline__ void absmax_note(AbsmaxTracker &tr, u32 u, float m, const u32 *s_uoff, int T, u32 *absmax)
-{
-    if (u >= tr.u_end) {
-        absmax_push<LPR>(tr, absmax);
-        int lo = 0, hi = T;              // invariant: s_uoff[lo] <= u < s_uoff[hi]
-        while (hi - lo > 1) {
-            const int mid = (lo + hi) >> 1;
-            if (s_uoff[mid] <= u) lo = mid; else hi = mid;
-        }
-        tr.t = lo;
-        tr.u_end = s_uoff[lo + 1];
-    }
-    tr.m = fmaxf(tr.m, m);
-}
-
-template <int CH>
-__device__ __forceinline__ float round_store(const double (&acc)[CH][4], float *dst_row, int lane, int lpr, int d4)
-{
-    float m = 0.f;
-#pragma unroll
-    for (int ch = 0; ch < CH; ++ch) {
-        int c4 = ch * lpr + lane;
-        if (c4 < d4) {
-            float4 r = make_float4((float)acc[ch][0], (float)acc[ch][1], (float)acc[ch][2], (float)acc[ch][3]);
-            *reinterpret_cast<float4 *>(dst_row + 4 * c4) = r;
-            m = fmaxf(fmaxf(m, fmaxf(fabsf(r.x), fabsf(r.y))), fmaxf(fabsf(r.z), fabsf(r.w)));
-        }
-    }
-    return m;
-}
-
-// VEC consecutive floats (1, 2 or 4) as one load
+// VEC consecutive floats (1, 2 or 4)
 template <int VEC> struct Vec;
 template <> struct Vec<1> { typedef float type; };
 template <> struct Vec<2> { typedef float2 type; };
 template <> struct Vec<4> { typedef float4 type; };
 
-template <int VEC>
-__device__ __forceinline__ void vec_add(double (&acc)[VEC], const typename Vec<VEC>::type &v)
+__device__ __forceinline__ float ld_row(const float *p, uint64_t pol)
 {
-    if constexpr (VEC == 1) { acc[0] += (double)v; }
-    else if constexpr (VEC == 2) { acc[0] += (double)v.x; acc[1] += (double)v.y; }
-    else { acc[0] += (double)v.x; acc[1] += (double)v.y; acc[2] += (double)v.z; acc[3] += (double)v.w; }
+    float v;
+    asm volatile("ld.global.nc.L2::cache_hint.f32 %0, [%1], %2;\n" : "=f"(v) : "l"(p), "l"(pol));
+    return v;
+}
+__device__ __forceinline__ float2 ld_row(const float2 *p, uint64_t pol)
+{
+    float2 v;
+    asm volatile("ld.global.nc.L2::cache_hint.v2.f32 {%0, %1}, [%2], %3;\n" : "=f"(v.x), "=f"(v.y) : "l"(p), "l"(pol));
+    return v;
+}
+__device__ __forceinline__ float4 ld_row(const float4 *p, uint64_t pol) { return dq_ld_nc(p, pol); }
+__device__ __forceinline__ void st_row(float *p, float v, uint64_t pol)
+{
+    asm volatile("st.global.L2::cache_hint.f32 [%0], %1, %2;\n" ::"l"(p), "f"(v), "l"(pol) : "memory");
+}
+__device__ __forceinline__ void st_row(float2 *p, const float2 &v, uint64_t pol)
+{
+    asm volatile("st.global.L2::cache_hint.v2.f32 [%0], {%1, %2}, %3;\n" ::"l"(p), "f"(v.x), "f"(v.y), "l"(pol) : "memory");
+}
+__device__ __forceinline__ void st_row(float4 *p, const float4 &v, uint64_t pol) { dq_st_keep(p, v, pol); }
+
+__device__ __forceinline__ void add(double (&acc)[1], float v) { acc[0] += (double)v; }
+__device__ __forceinline__ void add(double (&acc)[2], const float2 &v) { acc[0] += (double)v.x; acc[1] += (double)v.y; }
+__device__ __forceinline__ void add(double (&acc)[4], const float4 &v)
+{
+    acc[0] += (double)v.x; acc[1] += (double)v.y; acc[2] += (double)v.z; acc[3] += (double)v.w;
+}
+// rounds a finished sum
+__device__ __forceinline__ float rounded(const double (&a)[1], float &mx) { const float r = (float)a[0]; mx = fabsf(r); return r; }
+__device__ __forceinline__ float2 rounded(const double (&a)[2], float &mx)
+{
+    const float2 r = make_float2((float)a[0], (float)a[1]);
+    mx = fmaxf(fabsf(r.x), fabsf(r.y));
+    return r;
+}
+__device__ __forceinline__ float4 rounded(const double (&a)[4], float &mx)
+{
+    const float4 r = make_float4((float)a[0], (float)a[1], (float)a[2], (float)a[3]);
+    mx = fmaxf(fmaxf(fabsf(r.x), fabsf(r.y)), fmaxf(fabsf(r.z), fabsf(r.w)));
+    return r;
 }
 
-// One lane group (LPR lanes) owns one chunk of 32 sorted entries and walks in order the segments that
-// BEGIN in it, NB upstream-gradient rows in flight at a time: a segment's tail in the next chunk is
-// read by the same group, and a leading run that began in the chunk before is skipped, so the common
-// segment that straddles a chunk boundary needs no partial sum.  Lane `lane` holds, for ch < CH, the
-// VEC consecutive features starting at (ch*LPR + lane)*VEC.  Per chunk, one lane per entry compares
-// neighbouring keys once (this chunk's and the next one's); the resulting bit masks of segment heads
-// and the payloads (parked in shared memory) are all the walk needs, so an entry costs one shared
-// load, one address, one 128-bit load, a bit test and the FP64 adds.
-// (256-byte rows want four resident blocks per SM: that caps the kernel at 64 registers.  64-byte rows are capped
-// at three blocks' worth, 78 registers with a few spills: alone the kernel loses a microsecond, beside the sort of
-// the next batch the step gains three, because the two then fit on an SM together)
-template <int LPR, int VEC, int CH, bool EXACT, int CK = 32, bool OWN = (LPR >= 8)>
-__global__ void __launch_bounds__(256, (LPR == 16 && VEC == 4 && CH == 1) ? 4 : (LPR == 4 && VEC == 4) ? 3 : 1)
-seg_reduce_kernel(const u32 *__restrict__ keys, const u32 *__restrict__ vals,
-                  const u32 *__restrict__ seg_start, const u32 *__restrict__ chunk_first,
-                  const int32_t *__restrict__ uniq_off,
-                  const float *__restrict__ grad_out, float *__restrict__ grad_rows,
-                  double *__restrict__ partials, uint4 *__restrict__ long_list, u32 *__restrict__ counters,
-                  u32 *__restrict__ absmax, int T, int D_any,
-                  int64_t L, int64_t G, int64_t num_chunks, int *__restrict__ status, const ByTable bt)
+// abs-max of a row where the tile holds rows of several tables (rare in large batches: kept out of the unrolled code).
+// Called by all lanes of a group together.
+template <int LPR>
+__device__ __noinline__ void note_max(u32 *absmax, const u32 *s_uoff, int t_first, int T, u32 u, float x)
 {
-    // EXACT: the feature size fills the lanes exactly, so it is a compile-time constant and the
-    // per-vector range checks fall away
-    const int D = EXACT ? LPR * VEC * CH : D_any;
-    extern __shared__ unsigned char smem_raw[];
-    u32 *s_uoff = reinterpret_cast<u32 *>(smem_raw);                                     // [T+1]
-    u32 *s_tb = s_uoff + (T + 1);                                                        // [T+1] (lists by table)
-    u32 *s_row = s_tb + (T + 1);                                                         // [T+1] (lists by table)
-    u32 *s_vals = s_row + (T + 1) + (size_t)(threadIdx.x / LPR) * (2 * CK);           // this group's [2*CK]
-    // (the first T+1 threads fetch what either layout of the lists needs before the layout is known, so that the
-    // kernel starts with one round trip to memory, not two)
-    u32 r_tb = 0u, r_cnt = 0u, r_uo = 0u, r_row = 0u;
-    if ((int)threadIdx.x <= T) {
-        r_tb = bt.tb[threadIdx.x];
-        r_uo = (u32)uniq_off[threadIdx.x];
-        r_row = (u32)bt.row_off[threadIdx.x];      // (arena rows are 32-bit keys throughout)
-    }
-    if ((int)threadIdx.x < T) r_cnt = bt.table_cnt[threadIdx.x];
-    const u32 fmt = counters[CNT_FMT];
-    if (fmt == LISTS_BROKEN) {                    // (block-uniform)
-        if (blockIdx.x == 0) {
-            for (int t = threadIdx.x; t <= T; t += blockDim.x) bt.uniq_off[t] = 0;
-            if (threadIdx.x == 0) counters[CNT_U] = 0u;
+    const unsigned lane_w = threadIdx.x & 31;
+    const unsigned mask = LPR == 32 ? 0xffffffffu : (((1u << (LPR & 31)) - 1u) << (lane_w / LPR * LPR));
+    const u32 m = __reduce_max_sync(mask, __float_as_uint(x));
+    if (lane_w % LPR == 0 && m) atomicMax(absmax + last_not_above(s_uoff, t_first, T, u), m);
+}
+
+// blockIdx.x * WARPS + warp: range of tiles; blockIdx.y: block of 128 features (one unless D > 128)
+template <int LPR, int VEC, bool EXACT>
+__global__ void __launch_bounds__(THREADS, blocks_per_sm(LPR))
+seg_sum_kernel(const Args a)
+{
+    constexpr int C = batch_entries(LPR, VEC);    // rows of a lane group in flight
+    constexpr int GP = 32 / LPR;                  // lane groups of the warp
+    constexpr int I = tile_entries(LPR);
+    constexpr int W = I / 32;                     // index words per lane, words of head bits
+    constexpr int NB = I / (GP * C);              // batches per tile (one when the warp has several groups)
+    static_assert(GP == 1 ? NB % 2 == 0 : NB == 1, "");
+    typedef typename Vec<VEC>::type vec_t;
+    extern __shared__ u32 s_uoff[];                                                      // [T+1]
+    u32 *s_tb = s_uoff + (a.T + 1);                                                      // [T+1] (by table)
+    u32 *s_row = s_tb + (a.T + 1);                                                       // [T+1] (by table)
+    __shared__ u32 s_broken;
+
+    const int T = a.T, D = EXACT ? LPR * VEC : a.D, dv = D / VEC;
+    const int wl = threadIdx.x & 31, lane = wl % LPR, grp = wl / LPR;
+    const int cv = (EXACT ? 0 : blockIdx.y * LPR) + lane;      // this lane's vector of the row
+    const bool on = EXACT || cv < dv;
+    const bool first_col = EXACT || blockIdx.y == 0;
+    const u32 range = blockIdx.x * WARPS + (threadIdx.x >> 5);
+    const u32 tile0 = min((u32)a.num_tiles, range * (u32)a.range_tiles);
+    const u32 tile1 = min((u32)a.num_tiles, tile0 + (u32)a.range_tiles);
+
+    // ---- indices of a tile, one entry per lane and word.  An entry starts a segment when its key differs from the key
+    // before it; entries past the end count as heads, so that the last run closes like any other
+    u32 kn[W], vn[W], kp[W];
+    auto fetch = [&](u32 tile) {
+#pragma unroll
+        for (int w = 0; w < W; ++w) {
+            const int64_t i = (int64_t)tile * I + w * 32 + wl;
+            kn[w] = vn[w] = kp[w] = 0u;
+            if (i < a.L) {
+                kn[w] = __ldg(a.keys + i);
+                vn[w] = __ldg(a.vals + i);
+                kp[w] = i > 0 ? __ldg(a.keys + i - 1) : ~kn[w];
+            }
         }
-        return;
-    }
-    const bool by_table = fmt == LISTS_BY_TABLE;
-    if (by_table) {
-        // the tables' first segments: a running sum over their segment counts (T is small against the batch; one
-        // warp adds them up 32 at a time)
-        if (threadIdx.x < 32) {
+    };
+    u32 kc[W], vc[W], hw[W];                      // the present tile's keys, payloads and head bits
+    auto take = [&](u32 tile) {
+#pragma unroll
+        for (int w = 0; w < W; ++w) {
+            const bool past = (int64_t)tile * I + w * 32 + wl >= a.L;
+            hw[w] = __ballot_sync(0xffffffffu, past || kn[w] != kp[w]);
+            kc[w] = kn[w];
+            vc[w] = vn[w];
+            if ((int64_t)vc[w] >= a.G) { dq_report(a.status, DQRM_ERR_INDEX_RANGE); vc[w] = 0u; }
+        }
+    };
+    fetch(tile0);
+    u32 u_base = tile0 < tile1 ? a.chunk_first[tile0] : 0u;
+    if (a.by_table) {
+        if (threadIdx.x < 32) {                   // the tables' first segments: a running sum over their counts
             u32 run = 0;
+            bool broken = false;
             for (int t0 = 0; t0 < T; t0 += 32) {
-                const int t = t0 + (int)threadIdx.x;
-                const u32 cnt = t0 == 0 ? r_cnt : (t < T ? bt.table_cnt[t] : 0u);
+                const int t = t0 + wl;
+                const u32 cnt = t < T ? a.table_cnt[t] : 0u;
+                broken |= cnt == CNT_BROKEN;
                 u32 incl = cnt;
 #pragma unroll
                 for (int o = 1; o < 32; o <<= 1) {
                     const u32 v = __shfl_up_sync(0xffffffffu, incl, o);
-                    if ((int)threadIdx.x >= o) incl += v;
+                    if (wl >= o) incl += v;
                 }
                 if (t < T) s_uoff[t] = run + incl - cnt;
                 run += __shfl_sync(0xffffffffu, incl, 31);
             }
-            if (threadIdx.x == 0) s_uoff[T] = run;
+            broken = __any_sync(0xffffffffu, broken);
+            if (wl == 0) { s_uoff[T] = run; s_broken = broken; }
         }
-        for (int t = threadIdx.x; t <= T; t += blockDim.x) {
-            s_tb[t] = t == (int)threadIdx.x ? r_tb : bt.tb[t];
-            s_row[t] = t == (int)threadIdx.x ? r_row : (u32)bt.row_off[t];
-        }
-        __syncthreads();
-        if (blockIdx.x == 0) {
-            for (int t = threadIdx.x; t <= T; t += blockDim.x) bt.uniq_off[t] = (int32_t)s_uoff[t];
-            if (threadIdx.x == 0) counters[CNT_U] = s_uoff[T];
-        }
+        for (int t = threadIdx.x; t <= T; t += THREADS) { s_tb[t] = a.tb[t]; s_row[t] = (u32)a.row_off[t]; }
     } else {
-        for (int t = threadIdx.x; t <= T; t += blockDim.x) s_uoff[t] = t == (int)threadIdx.x ? r_uo : (u32)uniq_off[t];
-        __syncthreads();
+        for (int t = threadIdx.x; t <= T; t += THREADS) s_uoff[t] = (u32)a.uniq_off[t];
+        if (threadIdx.x == 0) s_broken = 0u;
     }
+    __syncthreads();
+    if (a.by_table && blockIdx.x == 0 && first_col)
+        for (int t = threadIdx.x; t <= T; t += THREADS) a.uniq_off[t] = s_broken ? 0 : (int32_t)s_uoff[t];
+    if (s_broken || tile0 >= tile1) return;       // (warp-uniform; no block barrier below)
 
-    typedef typename Vec<VEC>::type vec_t;
-    constexpr int NB = (VEC == 4 && LPR > 4) ? 4 : 8;   // rows in flight per lane
-    constexpr int EPL = CK / LPR;              // chunk entries one lane looks at
-    const int dv = D / VEC;                       // vectors per row
-    const int lane = threadIdx.x % LPR;
-    const u32 gmask = group_mask<LPR>();
-    const int gbase = (threadIdx.x & 31) / LPR * LPR;
-    const vec_t *g_lane = reinterpret_cast<const vec_t *>(grad_out) + lane;
-    const int64_t group = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / LPR;
-    const int64_t n_groups = (int64_t)gridDim.x * blockDim.x / LPR;
-    AbsmaxTracker tr;
-    bool bad = false;
+    // a one-index batch reads every upstream-gradient row once, a pooled one as often as the bag has indices
     const uint64_t keep = dq_policy_evict_last();
+    const uint64_t pol = a.L <= a.G ? dq_policy_evict_first() : dq_policy_evict_normal();
+    const vec_t *go = reinterpret_cast<const vec_t *>(a.grad_out) + (on ? cv : 0);
+    vec_t v[2][C];                                // two batches in turn when the warp takes one row at a time
+    // the rows of batch b of the present tile, all at once (row 0 for entries past the end, and a vector of the row for
+    // lanes past its end: nothing is done with either)
+    auto request = [&](int b, vec_t (&r)[C]) {
+        const int e0 = b * (GP * C) + grp * C;
+#pragma unroll
+        for (int k = 0; k < C; ++k) {
+            const int e = e0 + k;
+            u32 row = __shfl_sync(0xffffffffu, vc[0], e & 31);
+            if (W == 2) { const u32 r1 = __shfl_sync(0xffffffffu, vc[W - 1], e & 31); if (e >= 32) row = r1; }
+            r[k] = ld_row(go + (int64_t)row * dv, pol);       // (no condition: a branch per row would expose every shuffle)
+        }
+    };
+    // asks L2 for the rows of the tile whose indices have just arrived: a row per lane and word
+    auto prefetch = [&]() {
+        const int c0 = EXACT ? 0 : blockIdx.y * LPR * VEC;
+        const int bytes = (EXACT ? D : min(D - c0, LPR * VEC)) * (int)sizeof(float);
+#pragma unroll
+        for (int w = 0; w < W; ++w) {
+            const char *row = reinterpret_cast<const char *>(a.grad_out + (int64_t)((int64_t)vn[w] < a.G ? vn[w] : 0u) * D + c0);
+#pragma unroll
+            for (int b = 0; b < LPR * VEC * 4; b += 128)
+                if (EXACT || b < bytes) dq_prefetch_l2(row + b);
+            if (!EXACT) dq_prefetch_l2(row + bytes - 4);      // (rows that do not begin on a line's start)
+        }
+    };
+    take(tile0);
+    request(0, v[0]);
+    fetch(tile0 + 1);
 
-    for (int64_t c = group; c < num_chunks; c += n_groups) {
-        const int64_t i0 = c * CK;
-        const int n = (int)(min(i0 + (int64_t)CK, L) - i0);
-        const int n_next = (int)max((int64_t)0, min((int64_t)CK, L - i0 - CK));
-        // Heads: entry e starts a segment when its key differs from the key before it; the same for the
-        // chunk behind, whose first head tells where this chunk's last segment ends.  All loads are issued
-        // before the first vote so that they are in flight together.
-        u32 kc[EPL], kp[EPL], vv[EPL], kn[OWN ? EPL : 1], knp[OWN ? EPL : 1], vn[OWN ? EPL : 1];
+    const bool head0 = hw[0] & 1u;
+    int t_first = a.by_table ? last_not_above(s_tb, 0, T, tile0 * I) : last_not_above(s_uoff, 0, T, u_base);
+    if (a.by_table) u_base += s_uoff[t_first];
+    const u32 u_lead = u_base;                    // the run that enters the range, if one does
+    u_base -= head0;                              // segment of entry e of the tile = u_base + heads in [0, e]
+    bool open_lead = !head0;                      // no segment has begun in the range yet
+    bool one_table = false;                       // everything that the present tile closes belongs to table t_first
+    int t_max = t_first;
+    float m = 0.f;                                // abs-max of the rows of table t_max that this thread has rounded
+    auto push_max = [&]() {
+        const u32 mb = __reduce_max_sync(0xffffffffu, __float_as_uint(m));
+        if (wl == 0 && mb) atomicMax(a.absmax + t_max, mb);
+        m = 0.f;
+    };
+    // rounds a finished sum and writes it; leaves a piece of a cut run (called by all lanes of a group)
+    auto store_row = [&](u32 u, const double (&acc)[VEC]) {
+        float x = 0.f;
+        if (on) st_row(reinterpret_cast<vec_t *>(a.grad_rows + (int64_t)u * D) + cv, rounded(acc, x), keep);  // quantise+update reads it next
+        if (one_table) m = fmaxf(m, x);
+        else note_max<LPR>(a.absmax, s_uoff, t_first, T, u, x);
+    };
+    auto store_piece = [&](int slot, const double (&acc)[VEC]) {
+        if (on) {
+            double *p = a.partials + ((size_t)range * 2 + slot) * D + cv * VEC;
 #pragma unroll
-        for (int j = 0; j < EPL; ++j) {
-            const int e = j * LPR + lane;
-            const int64_t i = i0 + e;
-            kc[j] = kp[j] = vv[j] = 0u;
-            if (e < n) {
-                vv[j] = vals[i];
-                kc[j] = keys[i];
-                kp[j] = i > 0 ? keys[i - 1] : ~kc[j];
-            }
-            if (OWN) {
-                kn[j] = knp[j] = vn[j] = 0u;
-                if (e < n_next) {
-                    vn[j] = vals[i + CK];
-                    kn[j] = keys[i + CK];
-                    knp[j] = keys[i + CK - 1];
+            for (int q = 0; q < VEC; ++q) p[q] = acc[q];
+        }
+    };
+    double acc[VEC];                              // GP == 1: the open run; else: what the tiles before left of it
+#pragma unroll
+    for (int q = 0; q < VEC; ++q) acc[q] = 0.0;
+
+    for (u32 tile = tile0; tile < tile1; ++tile) {
+        const int n = (int)min((int64_t)I, a.L - (int64_t)tile * I);
+        u32 n_heads = __popc(hw[0]) - (n < I ? I - n : 0);
+        if (W == 2) n_heads += __popc(hw[W - 1]);
+        // the table of the run that is open when the tile begins (of the first entry's when none is)
+        const bool fresh = tile == tile0 && head0;
+        while (t_first < T - 1 && u_base + fresh >= s_uoff[t_first + 1]) ++t_first;
+        one_table = u_base + n_heads < s_uoff[t_first + 1];
+        if (one_table && t_first != t_max) { push_max(); t_max = t_first; }
+        if (a.by_table && first_col) {
+            u32 before = 0;
+#pragma unroll
+            for (int w = 0; w < W; ++w) {         // every entry that starts a segment names the segment's row
+                if (w * 32 + wl < n && ((hw[w] >> wl) & 1u)) {
+                    const u32 u = u_base + before + __popc(hw[w] & (0xffffffffu >> (31 - wl)));
+                    const int t = one_table ? t_first : last_not_above(s_uoff, t_first, T, u);
+                    a.unique_rows[u] = (int32_t)(kc[w] - s_row[t]);
                 }
+                before += __popc(hw[w]);
             }
         }
-        // OWN: did the run that enters this chunk begin in the chunk before?  (the keys ascend: it did unless the
-        // key 33 entries back is still the same).  Otherwise: the key behind the chunk tells whether its last run ends
-        u32 k_x = 0u;
-        if (OWN) { if (i0 > CK) k_x = keys[i0 - CK - 1]; }
-        else if (i0 + n < L) k_x = keys[i0 + n];
-        u32 u_first = chunk_first[c];
-        int t_first = 0;                          // lists by table: the table that holds the chunk's first entry
-        if (by_table) {
-            int lo = 0, hi = T;                   // largest t with s_tb[t] <= i0 (empty tables share a start: the last)
-            while (hi - lo > 1) {
-                const int mid = (lo + hi) >> 1;
-                if ((int64_t)s_tb[mid] <= i0) lo = mid; else hi = mid;
-            }
-            t_first = lo;
-            u_first += s_uoff[lo];
-        }
-        __syncwarp(gmask);                        // the previous chunk's payloads are no longer read
-        u32 heads = 0, heads_n = 0;
+        if (tile + 1 < tile1) prefetch();
+        if constexpr (GP == 1) {
+            u32 u = u_base;
+            const u32 heads = n < I ? hw[0] & ((1u << n) - 1u) : hw[0];
 #pragma unroll
-        for (int j = 0; j < EPL; ++j) {
-            const int e = j * LPR + lane;
-            if (e < n) {
-                u32 v = vv[j];
-                if ((int64_t)v >= G) { bad = true; v = 0u; }
-                s_vals[e] = v;
-                // the walk reaches this entry's upstream-gradient row up to 32 dependent steps from now: have L2
-                // fetch it meanwhile, so that all of a chunk's rows are in flight at once without holding registers
-                if (PREFETCH_ROW_BYTES >= D * (int)sizeof(float)) {
-                    const char *row = reinterpret_cast<const char *>(grad_out) + (int64_t)v * D * sizeof(float);
-#pragma unroll
-                    for (int b = 0; b < PREFETCH_ROW_BYTES; b += 128)
-                        if (b < D * (int)sizeof(float)) dq_prefetch_l2(row + b);
+            for (int b = 0; b < NB; ++b) {
+                if (b + 1 < NB) {
+                    request(b + 1, v[(b + 1) & 1]);
+                } else if (tile + 1 < tile1) {
+                    take(tile + 1);
+                    request(0, v[0]);
+                    fetch(tile + 2);
                 }
-            }
-            const u32 lm = LPR >= 32 ? 0xffffffffu : ((1u << LPR) - 1u);
-            if (OWN) {
-                if (e < n_next) {
-                    u32 v = vn[j];
-                    if ((int64_t)v >= G) { bad = true; v = 0u; }
-                    s_vals[CK + e] = v;
-                }
-                const bool head_n = (e < n_next) && (kn[j] != knp[j]);
-                heads_n |= ((__ballot_sync(gmask, head_n) >> gbase) & lm) << (j * LPR);
-            }
-            const bool head = (e < n) && (kc[j] != kp[j]);
-            heads |= ((__ballot_sync(gmask, head) >> gbase) & lm) << (j * LPR);
-        }
-        if (by_table) {
-            // every entry that starts a segment names the segment's row: segment of entry e = u_first + heads in (0, e]
-            u32 base = s_row[t_first];
-            const bool one_table = (int64_t)s_tb[min(t_first + 1, T)] >= i0 + n;     // (group-uniform)
+                const u32 bits = (heads >> (b * C)) & ((1u << C) - 1u);
+                if (bits == 0u && n >= (b + 1) * C) {         // inside a run
 #pragma unroll
-            for (int j = 0; j < EPL; ++j) {
-                const int e = j * LPR + lane;
-                if (e < n && kc[j] != kp[j]) {
-                    if (!one_table) {             // the chunk straddles tables: this key's own table
-                        int lo = t_first, hi = T;
-                        while (hi - lo > 1) {
-                            const int mid = (lo + hi) >> 1;
-                            if (s_row[mid] <= kc[j]) lo = mid; else hi = mid;
+                    for (int k = 0; k < C; ++k) add(acc, v[b & 1][k]);
+                } else {
+#pragma unroll
+                    for (int k = 0; k < C; ++k) {
+                        if ((bits >> k) & 1u) {               // (warp-uniform)
+                            if (open_lead) { store_piece(0, acc); open_lead = false; }
+                            else if (!(fresh && b * C + k == 0)) store_row(u, acc);
+                            ++u;
+#pragma unroll
+                            for (int q = 0; q < VEC; ++q) acc[q] = 0.0;
                         }
-                        base = s_row[lo];
+                        if (b * C + k < n) add(acc, v[b & 1][k]);
                     }
-                    const u32 ue = u_first + __popc(heads & ~1u & (0xffffffffu >> (31 - e)));
-                    bt.unique_rows[ue] = (int32_t)(kc[j] - base);
                 }
             }
-        }
-        if (n_next < CK) heads_n |= 1u << n_next;   // the end of the array closes a run like a head
-        const u32 k_0 = __shfl_sync(gmask, kc[0], gbase);
-        // the chunk's last key sits in lane (n-1) % LPR, register (n-1) / LPR
-        u32 k_last = 0u;
-#pragma unroll
-        for (int j = 0; j < EPL; ++j)
-            if ((n - 1) / LPR == j) k_last = kc[j];
-        k_last = __shfl_sync(gmask, k_last, gbase + (n - 1) % LPR);
-        __syncwarp(gmask);
-
-        // ---- which entries this group sums: [ea, eb) relative to i0, eb up to 2*CK.
-        // A segment is summed where it BEGINS, together with its tail in the next chunk; a leading run that
-        // began in the chunk before and ends here was summed there.  Only a segment whose tail is not over
-        // within the next chunk is summed in pieces (FP64 partials, folded by the fix-up kernel).
-        // (Without OWN - rows so narrow that the extra keys and payloads would cost more registers than the
-        // fix-up saves - a group sums exactly its chunk and every run cut by a chunk boundary is a piece.)
-        const bool any_head = heads != 0u;
-        const int f = any_head ? __ffs(heads) - 1 : n;                 // first head (n: none)
-        bool lead_piece, trail_long;
-        int ea, eb;
-        if (OWN) {
-            const bool closes_here = any_head || n < CK;
-            const bool began_prev = (i0 <= CK) || (k_x != k_0);
-            lead_piece = f > 0 && !(closes_here && began_prev);
-            ea = lead_piece ? 0 : f;
-            trail_long = any_head && heads_n == 0u;
-            eb = n + ((any_head && heads_n != 0u) ? __ffs(heads_n) - 1 : 0);    // (an extension only when n == CK)
+            u_base = u;
         } else {
-            lead_piece = f > 0;
-            ea = 0;
-            trail_long = !((i0 + n == L) || (k_x != k_last));
-            eb = n;
-        }
-        if (eb <= ea) continue;                   // group-uniform
-        heads &= ~1u;                             // the walk starts a run at its first entry either way
-        u32 u = u_first + ((ea > 0) ? 1u : 0u);   // segment of entry ea (ea > 0: it is the chunk's first head)
-        int run_start = ea;
-        double acc[CH][VEC];
+            const u32 word = W == 2 && grp * C >= 32 ? hw[W - 1] : hw[0];
+            const int es = grp * C, sh = es & 31;
+            u32 hb = (word >> sh) & ((1u << C) - 1u);
+            const int nv = min(max(n - es, 0), C);
+            if (nv < C) hb &= (1u << nv) - 1u;
+            const u32 before = __popc(word & ((1u << sh) - 1u)) + (W == 2 && es >= 32 ? __popc(hw[0]) : 0);
+            u32 u = u_base + before;              // the run that is open when the group begins
+            const u32 u_in = u;
+            bool seen = false;
+            double in[VEC], sum[VEC];             // what the group adds to that run; the present run
 #pragma unroll
-        for (int ch = 0; ch < CH; ++ch)
+            for (int q = 0; q < VEC; ++q) in[q] = sum[q] = 0.0;
 #pragma unroll
-            for (int q = 0; q < VEC; ++q) acc[ch][q] = 0.0;
-
-        // closes run [rs, re) (chunk-relative) of segment u
-        auto flush = [&](int rs, int re) {
-            const bool begins = !(lead_piece && rs == 0);
-            const bool ends = !(trail_long && re == eb);
-            if (begins && ends) {
-                float m = 0.f;
+            for (int k = 0; k < C; ++k) {
+                if (k < nv) {
+                    if ((hb >> k) & 1u) {
+                        if (seen) store_row(u, sum);
+                        else {
 #pragma unroll
-                for (int ch = 0; ch < CH; ++ch) {
-                    const int cv = ch * LPR + lane;
-                    if (EXACT || cv < dv) {
-                        float *dst = grad_rows + (int64_t)u * D + cv * VEC;
-                        if constexpr (VEC == 1) { float r = (float)acc[ch][0]; *dst = r; m = fmaxf(m, fabsf(r)); }
-                        else if constexpr (VEC == 2) {
-                            float2 r = make_float2((float)acc[ch][0], (float)acc[ch][1]);
-                            *reinterpret_cast<float2 *>(dst) = r;
-                            m = fmaxf(m, fmaxf(fabsf(r.x), fabsf(r.y)));
-                        } else {
-                            float4 r = make_float4((float)acc[ch][0], (float)acc[ch][1], (float)acc[ch][2], (float)acc[ch][3]);
-                            dq_st_keep(reinterpret_cast<float4 *>(dst), r, keep);   // quantise+update reads it next
-                            m = fmaxf(fmaxf(m, fmaxf(fabsf(r.x), fabsf(r.y))), fmaxf(fabsf(r.z), fabsf(r.w)));
+                            for (int q = 0; q < VEC; ++q) in[q] = sum[q];
                         }
-                    }
-                }
-                absmax_note<LPR>(tr, u, m, s_uoff, T, absmax);
-            } else {
-                double *pdst = partials + ((size_t)c * 2 + (begins ? 1 : 0)) * D;
+                        seen = true;
+                        ++u;
 #pragma unroll
-                for (int ch = 0; ch < CH; ++ch) {
-                    const int cv = ch * LPR + lane;
-                    if (EXACT || cv < dv) {
-#pragma unroll
-                        for (int q = 0; q < VEC; ++q) pdst[cv * VEC + q] = acc[ch][q];
+                        for (int q = 0; q < VEC; ++q) sum[q] = 0.0;
                     }
-                }
-                if (begins && lane == 0) {
-                    // the segment begins here: leave all the fix-up needs to know about it in one record
-                    int lo = 0, hi = T;              // its table: largest t with s_uoff[t] <= u
-                    while (hi - lo > 1) {
-                        const int mid = (lo + hi) >> 1;
-                        if (s_uoff[mid] <= u) lo = mid; else hi = mid;
-                    }
-                    // (lists by table: the table's starts sit at seg_start[tb[t] + t + .], the slot behind its last
-                    // segment holds its end)
-                    const int64_t at = by_table ? (int64_t)s_tb[lo] + lo + (u - s_uoff[lo]) : (int64_t)u;
-                    const u32 sa = seg_start[at], sb = seg_start[at + 1];
-                    const u32 npieces = (sb - 1) / CK - sa / CK + 1;
-                    const uint4 rec = make_uint4(u, sa / CK, npieces, (u32)lo);
-                    // (the list has a slot per chunk and every chunk begins at most one such segment; the bound only
-                    // matters for a workspace that is summed twice without a sort in between, which must not write
-                    // outside the list)
-                    if (npieces > BIG_PIECES) {
-                        const u32 k = atomicAdd(&counters[CNT_BIG], 1u);
-                        if ((int64_t)k < num_chunks) long_list[num_chunks - 1 - k] = rec;
-                    } else {
-                        const u32 k = atomicAdd(&counters[CNT_LONG], 1u);
-                        if ((int64_t)k < num_chunks) long_list[k] = rec;
-                    }
+                    add(sum, v[0][k]);
                 }
             }
-        };
-
-        // whole batches of NB entries need no per-entry range checks
-        auto walk = [&](int e0, auto full_tag) {
-            constexpr bool FULL = decltype(full_tag)::value;
-            vec_t r[NB][CH];
-#pragma unroll
-            for (int k = 0; k < NB; ++k) {
-                if (FULL || e0 + k < eb) {
-                    const vec_t *src = g_lane + (int64_t)s_vals[e0 + k] * dv;
-#pragma unroll
-                    for (int ch = 0; ch < CH; ++ch)
-                        if (EXACT || ch * LPR + lane < dv) r[k][ch] = __ldcs(src + ch * LPR);   // every row is read once
-                }
+            __syncwarp();
+            u_base += n_heads;
+            const bool enters_lead = open_lead;
+            open_lead = open_lead && n_heads == 0u;
+            if (tile + 1 < tile1) {
+                take(tile + 1);
+                request(0, v[0]);
+                fetch(tile + 2);
             }
+            // segmented scan over the groups: sum becomes the open run behind the group, counted from the last head
+            bool any = seen;
 #pragma unroll
-            for (int k = 0; k < NB; ++k) {
-                const int e = e0 + k;
-                if (FULL || e < eb) {
-                    if (e > ea && e < CK && ((heads >> e) & 1u)) {
-                        flush(run_start, e);
-                        u += 1;
-                        run_start = e;
+            for (int o = 1; o < GP; o <<= 1) {
+                const bool any_o = __shfl_up_sync(0xffffffffu, any, o * LPR);
 #pragma unroll
-                        for (int ch = 0; ch < CH; ++ch)
-#pragma unroll
-                            for (int q = 0; q < VEC; ++q) acc[ch][q] = 0.0;
-                    }
-#pragma unroll
-                    for (int ch = 0; ch < CH; ++ch)
-                        if (EXACT || ch * LPR + lane < dv) vec_add<VEC>(acc[ch], r[k][ch]);
+                for (int q = 0; q < VEC; ++q) {
+                    const double x = __shfl_up_sync(0xffffffffu, sum[q], o * LPR);
+                    if (grp >= o && !any) sum[q] = x + sum[q];
                 }
+                if (grp >= o) any |= any_o;
             }
-        };
-        int e0 = ea;
-        for (; e0 + NB <= eb; e0 += NB) walk(e0, std::true_type{});
-        if (e0 < eb) walk(e0, std::false_type{});
-        flush(run_start, eb);
-    }
-    absmax_push<LPR>(tr, absmax);      // group-uniform: all lanes of a group walk the same chunks
-    if (bad) dq_report(status, DQRM_ERR_INDEX_RANGE);
-}
-
-// pieces of a listed segment: the chunk in which it begins holds the first (slot 1), later chunks slot 0
-__device__ __forceinline__ const double *piece_ptr(const double *partials, int64_t c0, int64_t p, int D)
-{
-    return partials + ((size_t)(c0 + p) * 2 + (p == 0 ? 1 : 0)) * D;
-}
-
-template <int CH, int UN>
-__device__ __forceinline__ void add_pieces(double (&acc)[CH][4], const double *partials, int64_t c0,
-                                           int64_t p_begin, int64_t p_end, int64_t stride, int D, int lane,
-                                           int lpr, int d4)
-{
-    for (int64_t p = p_begin; p < p_end; p += stride * UN) {
-        double2 x[UN][CH], y[UN][CH];
+            const bool any_in = __shfl_up_sync(0xffffffffu, any, LPR) && grp > 0;
+            const bool any_all = __shfl_sync(0xffffffffu, any, 31);
 #pragma unroll
-        for (int k = 0; k < UN; ++k) {
-            const int64_t pk = p + k * stride;
-            if (pk < p_end) {
-                const double *src = piece_ptr(partials, c0, pk, D);
-#pragma unroll
-                for (int ch = 0; ch < CH; ++ch) {
-                    int c4 = ch * lpr + lane;
-                    if (c4 < d4) {
-                        x[k][ch] = __ldcg(reinterpret_cast<const double2 *>(src + 4 * c4));
-                        y[k][ch] = __ldcg(reinterpret_cast<const double2 *>(src + 4 * c4 + 2));
-                    }
-                }
+            for (int q = 0; q < VEC; ++q) {
+                const double x = __shfl_up_sync(0xffffffffu, sum[q], LPR);
+                if (grp > 0) in[q] = (any_in ? x : acc[q] + x) + in[q];
+                else in[q] = acc[q] + in[q];
+                const double last = __shfl_sync(0xffffffffu, sum[q], (GP - 1) * LPR + lane);
+                acc[q] = any_all ? last : acc[q] + last;
             }
-        }
-#pragma unroll
-        for (int k = 0; k < UN; ++k) {
-            if (p + k * stride < p_end) {
-#pragma unroll
-                for (int ch = 0; ch < CH; ++ch) {
-                    int c4 = ch * lpr + lane;
-                    if (c4 < d4) {
-                        acc[ch][0] += x[k][ch].x; acc[ch][1] += x[k][ch].y;
-                        acc[ch][2] += y[k][ch].x; acc[ch][3] += y[k][ch].y;
-                    }
-                }
+            if (seen) {
+                if (enters_lead && before == 0u) store_piece(0, in);
+                else if (!(fresh && before == 0u)) store_row(u_in, in);
             }
+            __syncwarp();
         }
     }
-}
-
-// A record of the list: x = segment (unique row), y = chunk in which it begins, z = number of pieces, w = table.
-
-// one warp per listed segment of at most BIG_PIECES pieces
-template <int LPR, int CH>
-__device__ __forceinline__ void
-fixup_small(const double *__restrict__ partials, const uint4 *__restrict__ long_list, u32 count,
-            float *__restrict__ grad_rows, u32 *__restrict__ absmax, int D)
-{
-    constexpr int SG = 32 / LPR;
-    const int d4 = D >> 2;
-    const int wl = threadIdx.x & 31;
-    const int sub = wl / LPR, lane = wl % LPR;
-    const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int64_t n_warps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    for (int64_t s = warp; s < count; s += n_warps) {
-        const uint4 rec = __ldcg(long_list + s);
-        double acc[CH][4];
-#pragma unroll
-        for (int ch = 0; ch < CH; ++ch) acc[ch][0] = acc[ch][1] = acc[ch][2] = acc[ch][3] = 0.0;
-        add_pieces<CH, 4>(acc, partials, rec.y, sub, rec.z, SG, D, lane, LPR, d4);
-#pragma unroll
-        for (int o = LPR; o < 32; o <<= 1)
-#pragma unroll
-            for (int ch = 0; ch < CH; ++ch)
-#pragma unroll
-                for (int q = 0; q < 4; ++q) acc[ch][q] += __shfl_xor_sync(0xffffffffu, acc[ch][q], o);
-        float m = 0.f;
-        if (sub == 0) m = round_store<CH>(acc, grad_rows + (int64_t)rec.x * D, lane, LPR, d4);
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-        if (wl == 0 && m > 0.f) atomicMax(&absmax[rec.w], __float_as_uint(m));
+    // ---- the run that is open at the end of the range
+    const int64_t i1 = min((int64_t)tile1 * I, a.L);
+    const bool ends = i1 == a.L || __ldg(a.keys + i1) != __ldg(a.keys + i1 - 1);
+    const bool cut_lead = !head0, cut_trail = !open_lead && !ends;
+    if (grp == 0) {
+        if (open_lead || cut_trail) store_piece(open_lead ? 0 : 1, acc);
+        else store_row(u_base, acc);
     }
-}
+    __syncwarp();
+    push_max();
 
-// one block per listed segment of more than BIG_PIECES pieces (the hottest rows)
-template <int LPR, int CH>
-__device__ __forceinline__ void
-fixup_big(const double *__restrict__ partials, const uint4 *__restrict__ long_list, u32 count,
-          float *__restrict__ grad_rows, u32 *__restrict__ absmax, int D, int64_t num_chunks,
-          double *s_part /*[256/LPR][D]*/)
-{
-    constexpr int NSG = 256 / LPR;
-    const int d4 = D >> 2;
-    const int sub = threadIdx.x / LPR, lane = threadIdx.x % LPR;
-    for (u32 s = blockIdx.x; s < count; s += gridDim.x) {
-        const uint4 rec = __ldcg(long_list + (num_chunks - 1 - s));
-        double acc[CH][4];
+    // ---- the warp that brings a cut run's last piece adds the pieces
+    if (!(cut_lead || cut_trail)) return;
+    u32 last = 0, first_range = 0;
+    if (wl == 0 ? cut_lead : (wl == 1 && cut_trail)) {
+        const u32 u = wl == 0 ? u_lead : u_base;
+        const int t = last_not_above(s_uoff, 0, T, u);
+        const int64_t at = a.by_table ? (int64_t)s_tb[t] + t + (u - s_uoff[t]) : (int64_t)u;
+        const u32 R = (u32)a.range_tiles * I;
+        const u32 sa = __ldg(a.seg_start + at), sb = __ldg(a.seg_start + at + 1);
+        first_range = sa / R;
+        const u32 pieces = (sb - 1) / R - first_range + 1;
+        __threadfence();
+        last = atomicAdd(a.range_done + first_range, 1u) == pieces * gridDim.y - 1u ? pieces : 0u;
+        __threadfence();
+    }
+    __syncwarp();
+#pragma unroll 1
+    for (int q = 0; q < 2; ++q) {
+        const int np = (int)__shfl_sync(0xffffffffu, last, q);
+        if (np == 0) continue;
+        const u32 u = q ? u_base : u_lead;
+        const double *pieces = a.partials + (size_t)__shfl_sync(0xffffffffu, first_range, q) * 2 * D;
+        for (int col = 0; col < dv; col += LPR) { // all features: the blocks of the other columns are done too
+            const int cc = col + lane;
+            const bool in = EXACT || cc < dv;
+            double sum[VEC];
 #pragma unroll
-        for (int ch = 0; ch < CH; ++ch) acc[ch][0] = acc[ch][1] = acc[ch][2] = acc[ch][3] = 0.0;
-        add_pieces<CH, (CH == 1 ? 8 : 4)>(acc, partials, rec.y, sub, rec.z, NSG, D, lane, LPR, d4);
-        __syncthreads();
+            for (int x = 0; x < VEC; ++x) sum[x] = 0.0;
+            // (a small batch's hottest row has a piece per tile: eight of them in flight, or its chain is what the
+            // kernel waits for)
+            for (int p0 = grp; in && p0 < np; p0 += 8 * GP) {
+                double x[8][VEC];
 #pragma unroll
-        for (int ch = 0; ch < CH; ++ch) {
-            int c4 = ch * LPR + lane;
-            if (c4 < d4) {
-                double *dst = s_part + (size_t)sub * D + 4 * c4;
-                dst[0] = acc[ch][0]; dst[1] = acc[ch][1]; dst[2] = acc[ch][2]; dst[3] = acc[ch][3];
-            }
-        }
-        __syncthreads();
-        if (sub == 0) {
-            // lane group 0 adds the NSG sub-sums in order
-            float m = 0.f;
+                for (int j = 0; j < 8; ++j) {
+                    const int p = p0 + j * GP;
 #pragma unroll
-            for (int ch = 0; ch < CH; ++ch) {
-                int c4 = ch * LPR + lane;
-                if (c4 < d4) {
-                    double t0 = 0, t1 = 0, t2 = 0, t3 = 0;
-                    for (int g = 0; g < NSG; ++g) {
-                        const double *src = s_part + (size_t)g * D + 4 * c4;
-                        t0 += src[0]; t1 += src[1]; t2 += src[2]; t3 += src[3];
-                    }
-                    float4 r = make_float4((float)t0, (float)t1, (float)t2, (float)t3);
-                    *reinterpret_cast<float4 *>(grad_rows + (int64_t)rec.x * D + 4 * c4) = r;
-                    m = fmaxf(fmaxf(m, fmaxf(fabsf(r.x), fabsf(r.y))), fmaxf(fabsf(r.z), fabsf(r.w)));
+                    for (int q2 = 0; q2 < VEC; ++q2)
+                        x[j][q2] = p < np ? __ldcg(pieces + ((size_t)p * 2 + (p == 0 ? 1 : 0)) * D + cc * VEC + q2) : 0.0;
                 }
+#pragma unroll
+                for (int j = 0; j < 8; ++j)
+#pragma unroll
+                    for (int q2 = 0; q2 < VEC; ++q2) sum[q2] += x[j][q2];
             }
-            m = group_max<LPR>(m);
-            if (lane == 0 && m > 0.f) atomicMax(&absmax[rec.w], __float_as_uint(m));
+#pragma unroll
+            for (int o = LPR; o < 32; o <<= 1)
+#pragma unroll
+                for (int x = 0; x < VEC; ++x) sum[x] += __shfl_xor_sync(0xffffffffu, sum[x], o);
+            if (grp == 0) {
+                float x = 0.f;
+                if (in) st_row(reinterpret_cast<vec_t *>(a.grad_rows + (int64_t)u * D) + cc, rounded(sum, x), keep);
+                note_max<LPR>(a.absmax, s_uoff, 0, T, u, x);
+            }
+            __syncwarp();
         }
     }
-}
-
-// both fix-ups in one launch: every block first takes its share of the hottest rows, then its
-// warps take the other listed segments
-template <int LPR, int CH>
-__global__ void __launch_bounds__(256)
-seg_fixup_kernel(const double *__restrict__ partials, const uint4 *__restrict__ long_list,
-                 const u32 *__restrict__ counters, float *__restrict__ grad_rows, u32 *__restrict__ absmax,
-                 int D, int64_t num_chunks)
-{
-    extern __shared__ unsigned char smem_raw[];
-    double *s_part = reinterpret_cast<double *>(smem_raw);                         // [256/LPR][D]
-    const u32 n_big = (u32)min((int64_t)__ldcg(counters + CNT_BIG), num_chunks);
-    const u32 n_small = (u32)min((int64_t)__ldcg(counters + CNT_LONG), num_chunks);
-    fixup_big<LPR, CH>(partials, long_list, n_big, grad_rows, absmax, D, num_chunks, s_part);
-    fixup_small<LPR, CH>(partials, long_list, n_small, grad_rows, absmax, D);
 }
 
 }  // namespace segred

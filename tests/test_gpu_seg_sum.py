@@ -1,0 +1,47 @@
+"""GPU parity of the segmented sum at the sizes where its split can go wrong: tables whose runs end on, before and
+behind the edges of tiles and of the warps' ranges, a run that covers many ranges, one lookup, every row width class."""
+import numpy as np
+import pytest
+
+from dqrm_inputs import workloads as W
+from gpu_util import Case, bit_equal
+
+pytestmark = pytest.mark.gpu
+
+# lengths of the runs of equal rows, table by table (rows 0, 1, 2, ...)
+SPLITS = {
+    "one": [[1], [1]],
+    "tile_edges": [[31, 1, 1, 31, 32, 33, 63, 1, 64, 65, 31], [32], [64], [1, 63, 128, 7]],
+    "all_unique": [[1] * 700, [1] * 70, [2] * 99],
+    "one_run_over_ranges": [[3, 240_000, 5], [1]],
+    "long_and_short": [[1, 20_000] * 6 + [1] * 3_000, [150_000]],
+}
+
+
+@pytest.mark.parametrize("sort_path", [0, 1])
+@pytest.mark.parametrize("D", [4, 8, 12, 16, 20, 32, 36, 64, 128, 200])
+@pytest.mark.parametrize("split", list(SPLITS))
+def test_runs_at_the_edges(oracle, split, D, sort_path):
+    if split in ("one_run_over_ranges", "long_and_short") and D not in (4, 16, 20, 64, 200):
+        pytest.skip("the large splits take one size of each kind")
+    runs = SPLITS[split]
+    counts = [sum(r) for r in runs]
+    B = max(counts)                     # bags of one index; tables with fewer lookups end in empty bags
+    wl = W.Workload("runs", tuple(max(4, len(r)) for r in runs), D=D, B=B, alpha=None)
+    rng = np.random.default_rng(len(split) + D)
+    idx = np.concatenate([rng.permutation(np.repeat(np.arange(len(r)), r)) for r in runs]).astype(np.int32)
+    lens = np.zeros((wl.T, B), dtype=np.int64)
+    for t, n in enumerate(counts):
+        lens[t, :n] = 1
+    off = np.concatenate([[0], np.cumsum(lens.reshape(-1))]).astype(np.int32)
+    go = rng.standard_normal((B, wl.T, D)).astype(np.float32)
+    c = Case(wl, max_lookups=len(idx))
+    c.ctx.set_sort_path(sort_path)
+    ur, uo, gr = c.gpu_bwd(idx, off, go)
+    o_ur, o_uo, o_gr = oracle.emb_bwd(go, wl.T, D, B, idx, off)
+    assert bit_equal(uo, o_uo) and bit_equal(ur, o_ur)
+    # n terms of magnitude below 6 in FP64, in two orders: the sums differ by at most 2 n^2 * 6 * 2^-53 and each is
+    # rounded once, to within 2^-24 of itself
+    n = max(max(r) for r in runs)
+    np.testing.assert_allclose(gr, o_gr, rtol=2.0 ** -23, atol=12.0 * n * n * 2.0 ** -53)
+    c.ctx.close()
