@@ -65,8 +65,8 @@ int dqrm_create(dqrm_ctx **out, int T, int D, const int64_t *h_row_off)
     ctx->T = T;
     ctx->D = D;
     ctx->total_rows = h_row_off[T];
-    ctx->key_bits = 1;
-    while (((int64_t)1 << ctx->key_bits) < ctx->total_rows) ctx->key_bits++;
+    for (int t = 0; t < T; ++t)
+        while (((int64_t)1 << ctx->row_bits) < h_row_off[t + 1] - h_row_off[t]) ctx->row_bits++;
     ctx->h_row_off = new (std::nothrow) int64_t[T + 1];
     if (!ctx->h_row_off) { delete ctx; return DQRM_ERR_INVALID_ARG; }
     memcpy(ctx->h_row_off, h_row_off, sizeof(int64_t) * (T + 1));
@@ -224,8 +224,8 @@ int dqrm_profile_end(dqrm_ctx *ctx, void *stream, float *h_ms_per_kernel, int32_
 const char *dqrm_kernel_name(int kernel_id)
 {
     static const char *names[DQ_K_COUNT] = {
-        "begin", "refresh_kernel", "fwd_kernel", "memset", "prepare_kernel", "sort_scan_kernel",
-        "sort_scatter_kernel", "seg_count_kernel", "seg_emit_kernel", "seg_sum_kernel",
+        "begin", "refresh_kernel", "fwd_kernel", "memset", "rs_setup_kernel", "rs_hist_kernel", "rs_scan_kernel",
+        "rs_scatter_kernel", "seg_count_kernel", "seg_emit_kernel", "seg_sum_kernel",
         "absmax_kernel", "row_stream_kernel<quant>", "row_stream_kernel<update>", "row_stream_kernel<fused>",
         "copy", "cluster_sort_kernel", "dp_pack_kernel", "dp_sum_update_kernel", "pack_kernel", "packed_fwd_kernel", "fwd_codes_kernel", "decode_payload_kernel"};
     return (kernel_id >= 0 && kernel_id < DQ_K_COUNT) ? names[kernel_id] : "?";

@@ -4,11 +4,8 @@
 // straight-through quantiser hand every lookup its bag's upstream gradient unchanged.
 //
 // Pipeline (all on one stream, no inter-block waits anywhere):
-//   prepare      one thread per bag: arena-row key + gradient-row payload per lookup,
-//                digit histograms of every radix pass, first pass's per-tile histogram
-//   per pass     scan   : per-digit exclusive scan of the tile histograms (+ digit base)
-//                scatter: stable least-significant-digit scatter of (key, payload);
-//                         counts the next pass's tile histogram on the way
+//   sort         one cluster of blocks per table (cluster_sort.cuh), or a radix sort of all
+//                tables at once (radix_sort.cuh); the cluster sort can also number the segments
 //   seg_count / seg_emit  head flags of the sorted keys -> unique_rows, uniq_off,
 //                         segment starts, first segment of every tile of the sum
 //   seg_sum      every warp walks a range of the sorted order: gathers the upstream gradient rows,
@@ -20,6 +17,7 @@
 #include "common.cuh"
 #include "seg_reduce.cuh"
 #include "cluster_sort.cuh"
+#include "radix_sort.cuh"
 
 namespace {
 
@@ -27,16 +25,14 @@ constexpr int ST_THREADS = 256;
 constexpr int ST_ITEMS = 8;
 constexpr int ST_TILE = ST_THREADS * ST_ITEMS;   // 2048 entries per tile
 constexpr int ST_WARPS = ST_THREADS / 32;
-constexpr int NB_MAX = 512;                      // bins per pass (<= 9 bit digits)
-constexpr int HIST_CHUNK = 64;                   // tiles per chunk of the radix sort's offset computation
 
 struct Layout {
-    int passes, digit_bits, nb;
-    int64_t num_tiles;
+    int passes, digit_bits;                    // radix sort: digits of the row number within a table
+    int64_t radix_tiles, num_tiles;
     int sum_shift;                             // the summing kernel: log2 of its tile of sorted entries, tiles,
     int64_t sum_tiles, sum_ranges;             // ranges of range_tiles tiles (at most sum_ranges)
     int range_tiles;
-    size_t absmax, tile_heads, digit_base, chunk_sum, tilehist;
+    size_t absmax, tile_heads, tile0, tile_table, totals, tilehist;
     size_t keys_a, vals_a, pairs_a, pairs_b, seg_start, chunk_first, tile_done, partials, table_cnt, tb;
     size_t total;
 };
@@ -44,12 +40,11 @@ struct Layout {
 Layout make_layout(const dqrm_ctx *ctx, int64_t L)
 {
     Layout y;
-    y.passes = (ctx->key_bits + 8) / 9;
-    if (y.passes < 1) y.passes = 1;
-    y.digit_bits = (ctx->key_bits + y.passes - 1) / y.passes;
-    y.nb = 1 << y.digit_bits;
+    y.passes = (ctx->row_bits + rsort::MAX_DIGIT_BITS - 1) / rsort::MAX_DIGIT_BITS;
+    y.digit_bits = (ctx->row_bits + y.passes - 1) / y.passes;
     int64_t Lc = L < 1 ? 1 : L;
     y.num_tiles = (Lc + ST_TILE - 1) / ST_TILE;
+    y.radix_tiles = rsort::max_tiles(ctx->T, Lc);
     // the sum: every warp that the GPU holds at once walks one range of tiles
     const int lpr = segred::lanes_per_row(ctx->D), I = segred::tile_entries(lpr);
     y.sum_shift = dq_log2c(I);
@@ -62,9 +57,10 @@ Layout make_layout(const dqrm_ctx *ctx, int64_t L)
     auto take = [&](size_t bytes) { size_t at = o; o = align_up(o + bytes, 256); return at; };
     y.absmax = take(sizeof(u32) * ctx->T);
     y.tile_heads = take(sizeof(u32) * y.num_tiles);
-    y.digit_base = take(sizeof(u32) * NB_MAX);
-    y.chunk_sum = take(sizeof(u32) * y.nb * ((y.num_tiles + HIST_CHUNK - 1) / HIST_CHUNK));
-    y.tilehist = take(sizeof(u32) * y.nb * y.num_tiles);
+    y.tile0 = take(sizeof(u32) * (ctx->T + 1));
+    y.tile_table = take(sizeof(u32) * y.radix_tiles);
+    y.totals = take((sizeof(u32) * ctx->T) << y.digit_bits);
+    y.tilehist = take((sizeof(u32) * y.radix_tiles) << y.digit_bits);
     y.keys_a = take(sizeof(u32) * Lc);
     y.vals_a = take(sizeof(u32) * Lc);
     y.pairs_a = take(sizeof(uint2) * Lc);
@@ -77,184 +73,6 @@ Layout make_layout(const dqrm_ctx *ctx, int64_t L)
     y.partials = take(sizeof(double) * y.sum_ranges * 2 * ctx->D);
     y.total = o;
     return y;
-}
-
-// ---------------------------------------------------------------------------------
-// one thread per bag: (arena-row key, gradient-row payload) of every lookup of the bag, as one 8-byte pair:
-// the passes move pairs, so that a digit's short run in a tile still leaves as whole 32-byte sectors
-__global__ void __launch_bounds__(256)
-prepare_kernel(const int32_t *__restrict__ indices, const int32_t *__restrict__ offsets,
-               const int64_t *__restrict__ row_off, int T, int B, int64_t G, int64_t L,
-               uint2 *__restrict__ pairs, int payload_position, int *__restrict__ status)
-{
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
-        if (__ldg(offsets) != 0 || (int64_t)__ldg(offsets + G) != L) dq_report(status, DQRM_ERR_INDEX_RANGE);
-    }
-    for (int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; g < G; g += (int64_t)gridDim.x * blockDim.x) {
-        int32_t a = __ldg(offsets + g), e = __ldg(offsets + g + 1);
-        if (a < 0 || e < a || (int64_t)e > L) { dq_report(status, DQRM_ERR_INDEX_RANGE); continue; }
-        const int t = (int)(g / B);
-        const u32 payload = (u32)((g - (int64_t)t * B) * T + t);      // row of grad_out [B][T][D]
-        const int64_t r0 = __ldg(row_off + t);
-        const int64_t nrows = __ldg(row_off + t + 1) - r0;
-        for (int32_t j = a; j < e; ++j) {
-            int32_t idx = __ldg(indices + j);
-            if (idx < 0 || idx >= nrows) {
-                dq_report(status, DQRM_ERR_INDEX_RANGE);
-                idx = idx < 0 ? 0 : (int32_t)(nrows - 1);
-            }
-            pairs[j] = make_uint2((u32)(r0 + idx), payload_position ? (u32)j : payload);
-        }
-    }
-}
-
-// Per pass, three small kernels turn the digit counts of every tile of 2048 entries into the scatter's
-// offsets without a single global atomic: tilehist[tile][digit] counts; a thread per digit then walks the
-// 64 tiles of a chunk and leaves the running count in their place and the chunk's total in
-// chunk_sum[chunk][digit]; one block does the same over the chunks and scans the digits' totals.  The
-// scatter adds the three: digit base + chunks before + tiles before within the chunk.
-__global__ void __launch_bounds__(ST_THREADS)
-sort_hist_kernel(const uint2 *__restrict__ pairs, int64_t L, int shift, int nb, u32 *__restrict__ tilehist)
-{
-    __shared__ u32 cnt[NB_MAX];
-    for (int i = threadIdx.x; i < nb; i += ST_THREADS) cnt[i] = 0u;
-    __syncthreads();
-    const u32 mask = (u32)nb - 1u;
-    const int64_t base = (int64_t)blockIdx.x * ST_TILE + threadIdx.x;
-    u32 key[ST_ITEMS];
-#pragma unroll
-    for (int k = 0; k < ST_ITEMS; ++k) {
-        const int64_t i = base + (int64_t)k * ST_THREADS;
-        key[k] = i < L ? pairs[i].x : 0u;
-    }
-#pragma unroll
-    for (int k = 0; k < ST_ITEMS; ++k)
-        if (base + (int64_t)k * ST_THREADS < L) atomicAdd(&cnt[(key[k] >> shift) & mask], 1u);
-    __syncthreads();
-    for (int i = threadIdx.x; i < nb; i += ST_THREADS) tilehist[(size_t)blockIdx.x * nb + i] = cnt[i];
-}
-
-// block = chunk of HIST_CHUNK tiles, thread = digit
-__global__ void __launch_bounds__(NB_MAX)
-sort_chunk_kernel(u32 *__restrict__ tilehist, int64_t num_tiles, int nb, u32 *__restrict__ chunk_sum)
-{
-    const int d = threadIdx.x;
-    if (d >= nb) return;
-    const int64_t t0 = (int64_t)blockIdx.x * HIST_CHUNK;
-    const int n = (int)min((int64_t)HIST_CHUNK, num_tiles - t0);
-    u32 run = 0;
-    for (int b = 0; b < n; b += 8) {
-        u32 c[8];
-#pragma unroll
-        for (int k = 0; k < 8; ++k) c[k] = b + k < n ? tilehist[(size_t)(t0 + b + k) * nb + d] : 0u;
-#pragma unroll
-        for (int k = 0; k < 8; ++k)
-            if (b + k < n) { tilehist[(size_t)(t0 + b + k) * nb + d] = run; run += c[k]; }
-    }
-    chunk_sum[(size_t)blockIdx.x * nb + d] = run;
-}
-
-// one block, thread = digit: running counts over the chunks, then an exclusive scan of the digits' totals
-__global__ void __launch_bounds__(NB_MAX)
-sort_base_kernel(u32 *__restrict__ chunk_sum, int64_t num_chunks, int nb, u32 *__restrict__ digit_base)
-{
-    __shared__ u32 wsum[NB_MAX / 32];
-    const int d = threadIdx.x, lane = d & 31, warp = d >> 5;
-    u32 run = 0;
-    if (d < nb) {
-        for (int64_t c = 0; c < num_chunks; c += 8) {
-            u32 v[8];
-#pragma unroll
-            for (int k = 0; k < 8; ++k) v[k] = c + k < num_chunks ? chunk_sum[(size_t)(c + k) * nb + d] : 0u;
-#pragma unroll
-            for (int k = 0; k < 8; ++k)
-                if (c + k < num_chunks) { chunk_sum[(size_t)(c + k) * nb + d] = run; run += v[k]; }
-        }
-    }
-    u32 incl = run;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const u32 v = __shfl_up_sync(0xffffffffu, incl, o);
-        if (lane >= o) incl += v;
-    }
-    if (lane == 31) wsum[warp] = incl;
-    __syncthreads();
-    u32 woff = 0;
-    for (int w = 0; w < warp; ++w) woff += wsum[w];
-    if (d < nb) digit_base[d] = woff + incl - run;
-}
-
-// stable scatter of one tile by one digit
-// LAST: the final pass leaves keys and payloads in arrays of their own, as the kernels behind the sort read them
-template <bool LAST>
-__global__ void __launch_bounds__(ST_THREADS)
-sort_scatter_kernel(const uint2 *__restrict__ pairs_in, uint2 *__restrict__ pairs_out,
-                    u32 *__restrict__ keys_out, u32 *__restrict__ vals_out,
-                    const u32 *__restrict__ tilehist, const u32 *__restrict__ chunk_sum,
-                    const u32 *__restrict__ digit_base, int64_t L, int shift, int nb, int *__restrict__ status)
-{
-    __shared__ u32 cnt[ST_WARPS][NB_MAX];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int64_t tile = blockIdx.x;
-    const u32 mask = (u32)nb - 1u;
-    for (int i = threadIdx.x; i < ST_WARPS * NB_MAX; i += ST_THREADS) (&cnt[0][0])[i] = 0u;
-    __syncthreads();
-
-    u32 key[ST_ITEMS], val[ST_ITEMS], rank[ST_ITEMS];
-    const int64_t base = tile * ST_TILE + (int64_t)warp * (32 * ST_ITEMS) + lane;
-#pragma unroll
-    for (int k = 0; k < ST_ITEMS; ++k) {
-        int64_t i = base + k * 32;
-        bool valid = i < L;
-        const uint2 pr = valid ? pairs_in[i] : make_uint2(0u, 0u);
-        key[k] = pr.x;
-        val[k] = pr.y;
-    }
-    const u32 lt = (1u << lane) - 1u;
-#pragma unroll
-    for (int k = 0; k < ST_ITEMS; ++k) {
-        bool valid = (base + k * 32) < L;
-        u32 digit = valid ? ((key[k] >> shift) & mask) : (u32)nb;      // nb = "no item"
-        u32 peers = __match_any_sync(0xffffffffu, digit);
-        int leader = __ffs(peers) - 1;
-        u32 pre = 0;
-        if (lane == leader && valid) {
-            pre = cnt[warp][digit];
-            cnt[warp][digit] = pre + __popc(peers);
-        }
-        pre = __shfl_sync(0xffffffffu, pre, leader);
-        rank[k] = pre + __popc(peers & lt);
-        __syncwarp();
-    }
-    __syncthreads();
-    // per digit: running offset over warps, starting at this tile's global offset
-    for (int b = threadIdx.x; b < nb; b += ST_THREADS) {
-        u32 run = digit_base[b] + chunk_sum[(size_t)(tile / HIST_CHUNK) * nb + b] + tilehist[(size_t)tile * nb + b];
-#pragma unroll
-        for (int w = 0; w < ST_WARPS; ++w) {
-            u32 c = cnt[w][b];
-            cnt[w][b] = run;
-            run += c;
-        }
-    }
-    __syncthreads();
-#pragma unroll
-    for (int k = 0; k < ST_ITEMS; ++k) {
-        if ((base + k * 32) < L) {
-            u32 digit = (key[k] >> shift) & mask;
-            u32 pos = cnt[warp][digit] + rank[k];
-            if ((int64_t)pos < L) {
-                if (LAST) {
-                    keys_out[pos] = key[k];
-                    vals_out[pos] = val[k];
-                } else {
-                    pairs_out[pos] = make_uint2(key[k], val[k]);
-                }
-            } else {
-                dq_report(status, DQRM_ERR_INDEX_RANGE);   // only reachable with inconsistent offsets
-            }
-        }
-    }
 }
 
 // ---------------------------------------------------------------------------------
@@ -350,43 +168,48 @@ seg_emit_kernel(const u32 *__restrict__ keys, int64_t L, const u32 *__restrict__
     for (int w = 0; w < warp; ++w) woff += wsum[w];
     u32 heads_before = tile_prefix + woff + incl - c;   // heads strictly before entry i0
 
-    // tables of the keys: found once for the key before this thread's entries, then only advanced
+    // only the entries that start a segment are looked at (the walk over all eight with a test each took 35 us for
+    // 8.5 M entries).  Tables of the keys: found once for the key before this thread's entries, then only advanced
     // (keys ascend), so a head costs a comparison instead of two searches
+    u32 heads = 0;
+    {
+        u32 prev = prev0;
+#pragma unroll
+        for (int e = 0; e < ST_ITEMS; ++e) {
+            if (e < n && (i0 + e == 0 || k[e] != prev)) heads |= 1u << e;
+            prev = k[e];
+        }
+    }
+    if (n <= 0) return;
     int t_prev = -1, t = 0;
-    if (n > 0) {
+    if (heads || i0 + n == L) {
         if (i0 > 0) t_prev = dq_table_of(s_off, T, (int64_t)prev0);
         t = t_prev < 0 ? 0 : t_prev;
     }
-    u32 prev = prev0;
+    for (u32 h = heads, u = heads_before; h; h &= h - 1u, ++u) {
+        const int e = __ffs(h) - 1;
+        const int64_t i = i0 + e;
+        seg_start[u] = (u32)i;
+        u32 ke = k[0];
 #pragma unroll
-    for (int e = 0; e < ST_ITEMS; ++e) {
-        if (e < n) {
-            const int64_t i = i0 + e;
-            const bool head = (i == 0 || k[e] != prev);
-            if (head) {
-                const u32 u = heads_before;
-                heads_before += 1;
-                seg_start[u] = (u32)i;
-                // a sort that refused a table leaves that table's keys undefined: keep them inside the arena and
-                // the walk inside the offset list, whatever they hold
-                const int64_t key = min((int64_t)k[e], s_off[T] - 1);
-                while (t < T - 1 && key >= s_off[t + 1]) ++t;
-                unique_rows[u] = (int32_t)max((int64_t)0, key - s_off[t]);
-                for (int tt = t_prev + 1; tt <= t; ++tt) uniq_off[tt] = (int32_t)u;
-                t_prev = t;
-            }
-            const u32 u_of_i = heads_before - 1;
-            if ((i & (int64_t)(ck - 1)) == 0) {
-                chunk_first[i >> ck_shift] = u_of_i;
-                tile_done[i >> ck_shift] = 0u;
-            }
-            if (i == L - 1) {
-                const u32 U = u_of_i + 1;
-                seg_start[U] = (u32)L;
-                for (int tt = t_prev + 1; tt <= T; ++tt) uniq_off[tt] = (int32_t)U;
-            }
-        }
-        prev = k[e];
+        for (int x = 1; x < ST_ITEMS; ++x) if (e == x) ke = k[x];
+        // a sort that refused a table leaves that table's keys undefined: keep them inside the arena and
+        // the walk inside the offset list, whatever they hold
+        const int64_t key = min((int64_t)ke, s_off[T] - 1);
+        while (t < T - 1 && key >= s_off[t + 1]) ++t;
+        unique_rows[u] = (int32_t)max((int64_t)0, key - s_off[t]);
+        for (int tt = t_prev + 1; tt <= t; ++tt) uniq_off[tt] = (int32_t)u;
+        t_prev = t;
+    }
+    // the chunks that begin among this thread's entries (a chunk is a power of two, at least eight entries)
+    if ((i0 & (int64_t)(ck - 1)) == 0) {
+        chunk_first[i0 >> ck_shift] = heads_before + (heads & 1u) - 1u;
+        tile_done[i0 >> ck_shift] = 0u;
+    }
+    if (i0 + n == L) {
+        const u32 U = heads_before + __popc(heads);
+        seg_start[U] = (u32)L;
+        for (int tt = t_prev + 1; tt <= T; ++tt) uniq_off[tt] = (int32_t)U;
     }
 }
 
@@ -402,6 +225,50 @@ int launch_sum(dqrm_ctx *ctx, const segred::Args &a, cudaStream_t st)
     else seg_sum_kernel<LPR, VEC, false><<<grid, THREADS, smem, st>>>(a);
     DQRM_CUDA_TRY(ctx, cudaGetLastError());
     dq_mark(ctx, st, DQ_K_SEG_SUM);
+    return DQRM_OK;
+}
+
+template <bool FIRST, bool LAST>
+int launch_radix_pass(dqrm_ctx *ctx, const rsort::Args &a, const uint2 *in, uint2 *out, u32 *keys, u32 *vals, int shift,
+                      cudaStream_t st)
+{
+    const unsigned tiles = (unsigned)rsort::max_tiles(a.T, a.L);
+    const int nb = 1 << a.dbits;
+    rsort::rs_hist_kernel<FIRST><<<tiles, rsort::THREADS, 0, st>>>(a, in, shift);
+    DQRM_CUDA_TRY(ctx, cudaGetLastError());
+    dq_mark(ctx, st, DQ_K_SORT_HIST);
+    rsort::rs_scan_kernel<<<dim3((unsigned)((nb + rsort::SCAN_DIGITS - 1) / rsort::SCAN_DIGITS), (unsigned)a.T),
+                            rsort::SCAN_DIGITS * rsort::SCAN_GROUPS, 0, st>>>(a);
+    DQRM_CUDA_TRY(ctx, cudaGetLastError());
+    dq_mark(ctx, st, DQ_K_SORT_SCAN);
+    bool &raised = ctx->smem_raised[(FIRST ? 1 : 0) + (LAST ? 2 : 0)];
+    if (!raised)
+        DQRM_CUDA_TRY(ctx, cudaFuncSetAttribute(rsort::rs_scatter_kernel<FIRST, LAST>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                (int)rsort::scatter_smem(1 << rsort::MAX_DIGIT_BITS)));
+    raised = true;
+    rsort::rs_scatter_kernel<FIRST, LAST><<<tiles, rsort::THREADS, rsort::scatter_smem(nb), st>>>(a, in, out, keys, vals, shift);
+    DQRM_CUDA_TRY(ctx, cudaGetLastError());
+    dq_mark(ctx, st, DQ_K_SORT_SCATTER);
+    return DQRM_OK;
+}
+
+int launch_radix_sort(dqrm_ctx *ctx, const rsort::Args &a, int passes, uint2 *const (&pairs)[2], u32 *keys, u32 *vals,
+                      cudaStream_t st)
+{
+    rsort::rs_setup_kernel<<<1, 1024, rsort::setup_smem(a.T), st>>>(a);
+    DQRM_CUDA_TRY(ctx, cudaGetLastError());
+    dq_mark(ctx, st, DQ_K_SORT_SETUP);
+    for (int p = 0; p < passes; ++p) {
+        const uint2 *in = pairs[(p + 1) & 1];          // (the first pass reads the indices)
+        uint2 *out = pairs[p & 1];
+        const int shift = p * a.dbits;
+        int rc;
+        if (p == 0) rc = passes == 1 ? launch_radix_pass<true, true>(ctx, a, in, out, keys, vals, shift, st)
+                                     : launch_radix_pass<true, false>(ctx, a, in, out, keys, vals, shift, st);
+        else rc = p + 1 == passes ? launch_radix_pass<false, true>(ctx, a, in, out, keys, vals, shift, st)
+                                  : launch_radix_pass<false, false>(ctx, a, in, out, keys, vals, shift, st);
+        if (rc != DQRM_OK) return rc;
+    }
     return DQRM_OK;
 }
 
@@ -476,8 +343,6 @@ int dq_launch_bwd_sort(dqrm_ctx *ctx, const int32_t *indices, const int32_t *off
     u32 *keys[1] = {reinterpret_cast<u32 *>(ws + y.keys_a)};
     u32 *vals[1] = {reinterpret_cast<u32 *>(ws + y.vals_a)};
     uint2 *pairs[2] = {reinterpret_cast<uint2 *>(ws + y.pairs_a), reinterpret_cast<uint2 *>(ws + y.pairs_b)};
-    u32 *tilehist = reinterpret_cast<u32 *>(ws + y.tilehist), *chunk_sum = reinterpret_cast<u32 *>(ws + y.chunk_sum);
-    u32 *digit_base = reinterpret_cast<u32 *>(ws + y.digit_base);
     const u32 *skeys = nullptr;      // sorted keys; the sorted payloads sit beside them in vals[0]
     bool sorted = false;
     // (tables far beyond the shared-memory slices sort faster with the global radix sort)
@@ -521,37 +386,19 @@ int dq_launch_bwd_sort(dqrm_ctx *ctx, const int32_t *indices, const int32_t *off
         }
     }
     if (!sorted) {
-    {
-        int64_t blocks = (G + 255) / 256;
-        int64_t cap = (int64_t)ctx->num_sms * 8;
-        int grid = (int)(blocks > cap ? cap : blocks);
-        prepare_kernel<<<grid, 256, 0, st>>>(indices, offsets, ctx->d_row_off, ctx->T, B, G, L, pairs[0],
-                                             ctx->payload_position, ctx->d_status);
-        DQRM_CUDA_TRY(ctx, cudaGetLastError());
-        dq_mark(ctx, st, DQ_K_PREPARE);
-    }
-    const int64_t hist_chunks = (y.num_tiles + HIST_CHUNK - 1) / HIST_CHUNK;
-    for (int p = 0; p < y.passes; ++p) {
-        const uint2 *pin = pairs[p & 1];
-        const int shift = p * y.digit_bits;
-        sort_hist_kernel<<<(unsigned)y.num_tiles, ST_THREADS, 0, st>>>(pin, L, shift, y.nb, tilehist);
-        DQRM_CUDA_TRY(ctx, cudaGetLastError());
-        dq_mark(ctx, st, DQ_K_SORT_SCAN);
-        sort_chunk_kernel<<<(unsigned)hist_chunks, NB_MAX, 0, st>>>(tilehist, y.num_tiles, y.nb, chunk_sum);
-        DQRM_CUDA_TRY(ctx, cudaGetLastError());
-        dq_mark(ctx, st, DQ_K_SORT_SCAN);
-        sort_base_kernel<<<1, NB_MAX, 0, st>>>(chunk_sum, hist_chunks, y.nb, digit_base);
-        DQRM_CUDA_TRY(ctx, cudaGetLastError());
-        dq_mark(ctx, st, DQ_K_SORT_SCAN);
-        if (p + 1 < y.passes)
-            sort_scatter_kernel<false><<<(unsigned)y.num_tiles, ST_THREADS, 0, st>>>(
-                pin, pairs[(p + 1) & 1], nullptr, nullptr, tilehist, chunk_sum, digit_base, L, shift, y.nb, ctx->d_status);
-        else
-            sort_scatter_kernel<true><<<(unsigned)y.num_tiles, ST_THREADS, 0, st>>>(
-                pin, nullptr, keys[0], vals[0], tilehist, chunk_sum, digit_base, L, shift, y.nb, ctx->d_status);
-        DQRM_CUDA_TRY(ctx, cudaGetLastError());
-        dq_mark(ctx, st, DQ_K_SORT_SCATTER);
-    }
+        rsort::Args ra;
+        ra.indices = indices; ra.offsets = offsets; ra.row_off = ctx->d_row_off;
+        ra.T = ctx->T; ra.B = B; ra.L = L; ra.G = G;
+        ra.tb = reinterpret_cast<u32 *>(ws + y.tb);
+        ra.tile0 = reinterpret_cast<u32 *>(ws + y.tile0);
+        ra.tile_table = reinterpret_cast<u32 *>(ws + y.tile_table);
+        ra.tilehist = reinterpret_cast<u32 *>(ws + y.tilehist);
+        ra.totals = reinterpret_cast<u32 *>(ws + y.totals);
+        ra.dbits = y.digit_bits;
+        ra.payload_position = ctx->payload_position;
+        ra.status = ctx->d_status;
+        const int rc = launch_radix_sort(ctx, ra, y.passes, pairs, keys[0], vals[0], st);
+        if (rc != DQRM_OK) return rc;
         skeys = keys[0];
     }
     if (sorted && lists_by_table) {                    // the lists are there; unique_rows and uniq_off come with the sums

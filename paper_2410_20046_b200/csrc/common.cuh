@@ -21,7 +21,7 @@ struct dqrm_ctx {
     int last_cuda_error = 0;
     int device = 0;
     int num_sms = 0;
-    int key_bits = 1;               // bits of an arena row number
+    int row_bits = 1;               // bits of a row number within its table, largest table
     int sort_path = 0;              // 0: per-table cluster sort, 1: global radix sort
     cudaStream_t side = nullptr;    // second stream: a training step sorts the indices and sums the gradient beside its forward
     cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
@@ -63,7 +63,7 @@ struct dqrm_ctx {
 };
 
 enum {
-    DQ_K_BEGIN = 0, DQ_K_REFRESH, DQ_K_FWD, DQ_K_MEMSET, DQ_K_PREPARE, DQ_K_SORT_SCAN, DQ_K_SORT_SCATTER,
+    DQ_K_BEGIN = 0, DQ_K_REFRESH, DQ_K_FWD, DQ_K_MEMSET, DQ_K_SORT_SETUP, DQ_K_SORT_HIST, DQ_K_SORT_SCAN, DQ_K_SORT_SCATTER,
     DQ_K_SEG_COUNT, DQ_K_SEG_EMIT, DQ_K_SEG_SUM, DQ_K_ABSMAX, DQ_K_QUANT, DQ_K_UPDATE,
     DQ_K_QUANT_UPDATE, DQ_K_COPY, DQ_K_CLUSTER_SORT, DQ_K_DP_PACK, DQ_K_DP_SUM_UPDATE, DQ_K_PACK, DQ_K_PACKED_FWD, DQ_K_FWD_CODES, DQ_K_DECODE_PAYLOAD, DQ_K_COUNT
 };
