@@ -119,9 +119,9 @@ __device__ __forceinline__ float dq_dequant(int q, float s) { return __fmul_rn((
 // The same codes without the IEEE-division sequence, for a scale shared by many elements,
 // four elements at a time.
 //
-//   QuantScale holds s and r = RN(1/s).  q0 = RN(x * r) equals x/s up to a relative error
-//   below 2^-22 (one rounding of r, one of the product), and RN(x/s) is within 2^-24 of
-//   x/s.  Only half-integers of magnitude below 2^(b-1) decide a b-bit code (beyond them the
+//   QuantScale holds s and r = RN(1/s).  q0 = x * r (not rounded: it only ever sits inside a fused
+//   multiply-add) equals x/s up to a relative error below 2^-23 (the rounding of r), and RN(x/s) is
+//   within 2^-24 of x/s.  Only half-integers of magnitude below 2^(b-1) decide a b-bit code (beyond them the
 //   clamp gives the same code either way), and there |q0 - RN(x/s)| < 2^(b-23).  So if q0 is
 //   farther than TOL = 2^(b-21) from every half-integer, rounding q0 gives the same code as
 //   rounding RN(x/s).  Vectors with an element inside that window (about one in 10^4 for
@@ -162,12 +162,15 @@ __device__ __forceinline__ void dq_fq4(const float4 &v, const QuantScale &q, flo
     bool done = false;
     if (q.fast) {
         const float2 r2 = make_float2(q.r, q.r), m2 = make_float2(MAGIC, MAGIC), nm2 = make_float2(-MAGIC, -MAGIC);
-        const float2 neg1 = make_float2(-1.f, -1.f);
-        const float2 qa = __fmul2_rn(make_float2(v.x, v.y), r2), qb = __fmul2_rn(make_float2(v.z, v.w), r2);
-        const float2 ra = __fadd2_rn(__fadd2_rn(qa, m2), nm2), rb = __fadd2_rn(__fadd2_rn(qb, m2), nm2);
-        const float2 da = __ffma2_rn(ra, neg1, qa), db = __ffma2_rn(rb, neg1, qb);     // q0 - rint(q0)
+        const float2 va = make_float2(v.x, v.y), vb = make_float2(v.z, v.w), neg1 = make_float2(-1.f, -1.f);
+        const float2 ra = __fadd2_rn(__ffma2_rn(va, r2, m2), nm2), rb = __fadd2_rn(__ffma2_rn(vb, r2, m2), nm2);    // rint(x * r)
+        const float2 da = __ffma2_rn(va, r2, __fmul2_rn(ra, neg1)), db = __ffma2_rn(vb, r2, __fmul2_rn(rb, neg1)); // x * r - rint(x * r)
         const float m = fmaxf(fmaxf(fabsf(da.x), fabsf(da.y)), fmaxf(fabsf(db.x), fabsf(db.y)));
-        if (m < q.tie_lim) {
+        const float c = fmaxf(fmaxf(fabsf(ra.x), fabsf(ra.y)), fmaxf(fabsf(rb.x), fabsf(rb.y)));
+        if (m < q.tie_lim && c <= q.hi) {              // (with a fresh scale every code lies inside: nothing to clamp)
+            codes = make_float4(ra.x, ra.y, rb.x, rb.y);
+            done = true;
+        } else if (m < q.tie_lim) {
             codes = make_float4(fminf(fmaxf(ra.x, q.lo), q.hi), fminf(fmaxf(ra.y, q.lo), q.hi),
                                 fminf(fmaxf(rb.x, q.lo), q.hi), fminf(fmaxf(rb.y, q.lo), q.hi));
             done = true;

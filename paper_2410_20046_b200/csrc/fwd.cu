@@ -17,6 +17,7 @@
 //   * fwd_bags_kernel (any other batch): a lane group walks one bag at a time, NB of its
 //     rows per batch, and sums them in bag order in FP64, rounded once, so the result
 //     does not depend on the launch shape.
+#include <type_traits>
 #include "common.cuh"
 
 namespace {
@@ -180,17 +181,22 @@ fwd_onehot_kernel(const FwdArgs a)
     if (bad) dq_report(a.status, DQRM_ERR_INDEX_RANGE);
 }
 
-template <int LPR, int CH, bool EXACT>
+// A lane group walks one bag at a time.  The bag's indices are loaded LPR at a time, one per lane, and checked once;
+// the rows are then fetched NB at a time, their numbers handed round by shuffle, and summed in bag order.  Measured on
+// B200 the kernel is bound by instruction issue (rows of hot tables come from the caches), which is why nothing is done
+// per row by every lane that one lane can do, and why whole batches of NB rows carry no range checks.
+template <int LPR, int CH, bool EXACT, bool CODES>
 __global__ void __launch_bounds__(FW_THREADS)
 fwd_bags_kernel(const FwdArgs a)
 {
-    constexpr int NB = NBOf<LPR, CH>::v;
+    constexpr int NB = NBOf<LPR, CH>::v < LPR ? NBOf<LPR, CH>::v : LPR;
     constexpr int GPB = FW_THREADS / LPR;
     const int D = EXACT ? 4 * LPR * CH : a.D;
     const int d4 = D >> 2;
     const int t = blockIdx.y;
     const int lane = threadIdx.x % LPR;
     const int grp = threadIdx.x / LPR;
+    const unsigned gmask = LPR == 32 ? 0xffffffffu : (((1u << (LPR & 31)) - 1u) << ((threadIdx.x & 31) / LPR * LPR));
     const TableCtx tc = table_ctx(a, t, D);
     bool bad = false;
 
@@ -200,31 +206,39 @@ fwd_bags_kernel(const FwdArgs a)
         double acc[CH][4];
 #pragma unroll
         for (int c = 0; c < CH; ++c) acc[c][0] = acc[c][1] = acc[c][2] = acc[c][3] = 0.0;
-        for (int32_t j0 = lo; j0 < hi; j0 += NB) {
-            int32_t idx[NB];
+        int32_t mine = lo + lane < hi ? __ldg(a.indices + lo + lane) : 0;
+        for (int32_t j0 = lo; j0 < hi; j0 += LPR) {
+            const int32_t row = clamp_index(mine, tc.nrows, bad);      // (lanes past the bag's end hold row 0)
+            if (j0 + LPR + lane < hi) mine = __ldg(a.indices + j0 + LPR + lane); else mine = 0;
+            const int cnt = min(LPR, hi - j0);
+            auto rows = [&](int b0, auto full_tag) {
+                constexpr bool FULL = decltype(full_tag)::value;
 #pragma unroll
-            for (int b = 0; b < NB; ++b) idx[b] = (j0 + b < hi) ? clamp_index(__ldg(a.indices + j0 + b), tc.nrows, bad) : 0;
+                for (int c = 0; c < CH; ++c) {
+                    const int c4 = c * LPR + lane;
+                    float4 v[NB];
 #pragma unroll
-            for (int c = 0; c < CH; ++c) {
-                const int c4 = c * LPR + lane;
-                float4 v[NB];
+                    for (int b = 0; b < NB; ++b) {
+                        const int32_t r = __shfl_sync(gmask, row, b0 + b, LPR);
+                        v[b] = __ldg(reinterpret_cast<const float4 *>(tc.tbl + (int64_t)r * D) + (EXACT || c4 < d4 ? c4 : 0));
+                    }
 #pragma unroll
-                for (int b = 0; b < NB; ++b)
-                    if (j0 + b < hi && (EXACT || c4 < d4))
-                        v[b] = __ldg(reinterpret_cast<const float4 *>(tc.tbl + (int64_t)idx[b] * D) + c4);
-#pragma unroll
-                for (int b = 0; b < NB; ++b) {
-                    if (j0 + b < hi && (EXACT || c4 < d4)) {
-                        float4 cd, f;
-                        dq_fq4(v[b], tc.qs, cd, f);
-                        acc[c][0] += (double)f.x;
-                        acc[c][1] += (double)f.y;
-                        acc[c][2] += (double)f.z;
-                        acc[c][3] += (double)f.w;
-                        if (a.codes_out) store_codes(a.codes_out, j0 + b, D, c4, cd);
+                    for (int b = 0; b < NB; ++b) {
+                        if (FULL || b0 + b < cnt) {
+                            float4 cd, f;
+                            dq_fq4(v[b], tc.qs, cd, f);
+                            acc[c][0] += (double)f.x;
+                            acc[c][1] += (double)f.y;
+                            acc[c][2] += (double)f.z;
+                            acc[c][3] += (double)f.w;
+                            if (CODES && (EXACT || c4 < d4)) store_codes(a.codes_out, j0 + b0 + b, D, c4, cd);
+                        }
                     }
                 }
-            }
+            };
+            int b0 = 0;
+            for (; b0 + NB <= cnt; b0 += NB) rows(b0, std::true_type{});
+            if (b0 < cnt) rows(b0, std::false_type{});
         }
         float4 *o = reinterpret_cast<float4 *>(a.out + ((int64_t)i * a.T + t) * D);
 #pragma unroll
@@ -250,7 +264,8 @@ int launch2(dqrm_ctx *ctx, const FwdArgs &a, cudaStream_t st)
     if (bx < 1) bx = 1;
     dim3 grid((unsigned)bx, (unsigned)ctx->T);
     if (onehot) fwd_onehot_kernel<LPR, CH, EXACT><<<grid, FW_THREADS, 0, st>>>(a);
-    else fwd_bags_kernel<LPR, CH, EXACT><<<grid, FW_THREADS, 0, st>>>(a);
+    else if (a.codes_out) fwd_bags_kernel<LPR, CH, EXACT, true><<<grid, FW_THREADS, 0, st>>>(a);
+    else fwd_bags_kernel<LPR, CH, EXACT, false><<<grid, FW_THREADS, 0, st>>>(a);
     DQRM_CUDA_TRY(ctx, cudaGetLastError());
     dq_mark(ctx, st, DQ_K_FWD);
     return DQRM_OK;
