@@ -119,20 +119,22 @@ __device__ __forceinline__ float dq_dequant(int q, float s) { return __fmul_rn((
 // The same codes without the IEEE-division sequence, for a scale shared by many elements,
 // four elements at a time.
 //
-//   QuantScale holds s and r = RN(1/s).  q0 = x * r (not rounded: it only ever sits inside a fused
-//   multiply-add) equals x/s up to a relative error below 2^-23 (the rounding of r), and RN(x/s) is
-//   within 2^-24 of x/s.  Only half-integers of magnitude below 2^(b-1) decide a b-bit code (beyond them the
-//   clamp gives the same code either way), and there |q0 - RN(x/s)| < 2^(b-23).  So if q0 is
-//   farther than TOL = 2^(b-21) from every half-integer, rounding q0 gives the same code as
-//   rounding RN(x/s).  Vectors with an element inside that window (about one in 10^4 for
-//   4-bit codes) are redone with the IEEE division.  Rounding to an integer is done by
-//   adding and subtracting 1.5*2^23 (round-to-nearest-even, no conversion instruction);
-//   the result is the code as a float, which is also what the dequantiser multiplies.
-//   The multiplies and adds use the packed two-float instructions of sm_100.
+//   QuantScale holds s and k = 1/(s n), n = 2^b - 1 the width of the code range.  One saturating
+//   multiply-add maps x to z = (x/s - lo)/n in [0, 1]: the saturation is the clamp (and gives a NaN
+//   the code lo, as the clamp of the plain definition does).  z n, rounded to an integer, is code - lo.
+//   Away from the clamp z n is within 2^(b-22) of RN(x/s) - lo: two roundings of k at magnitude below
+//   2^(b-1), one of z and one of lo/n at magnitude 1, one of the quotient.  So if z n is farther than
+//   TOL = 2^(b-21) from every half-integer, rounding it gives the code that rounding RN(x/s) gives; a
+//   saturated z is an integer already.  Where an element lies inside that window (about one vector in
+//   10^4 for 4-bit codes) it is redone with the IEEE division.  Rounding to an integer is done by
+//   adding and subtracting 1.5*2^23 (round-to-nearest-even, no conversion instruction); with
+//   m = lo - code the dequantised value is one multiply-add, m (-s) + lo s, whose addend is exact
+//   (lo is a power of two) and whose one rounding is that of code * s.
+//   The multiply-adds use the packed two-float instructions of sm_100.
 //   Bit widths above 10 and scales outside [2^-100, 2^100] always take the IEEE path.
 // ---------------------------------------------------------------------------------
 struct QuantScale {
-    float s, r, lo, hi, tie_lim;
+    float s, k, off, n, lo, hi, tie_lim;
     bool fast;
 };
 
@@ -140,9 +142,11 @@ __device__ __forceinline__ QuantScale dq_make_scale(float s, int bits)
 {
     QuantScale q;
     q.s = s;
-    q.r = __frcp_rn(s);
     q.lo = -(float)(1 << (bits - 1));
     q.hi = (float)((1 << (bits - 1)) - 1);
+    q.n = q.hi - q.lo;
+    q.k = __frcp_rn(__fmul_rn(s, q.n));
+    q.off = __fdiv_rn(-q.lo, q.n);
     q.tie_lim = 0.5f - (float)(1 << (bits - 1)) * 9.5367431640625e-07f;     // 0.5 - 2^(b-21)
     q.fast = (bits <= 10) && (s >= 7.8886090522101181e-31f) && (s <= 1.2676506002282294e+30f);
     return q;
@@ -155,34 +159,52 @@ __device__ __forceinline__ float dq_codef_ieee(float x, const QuantScale &q)
     return __fadd_rn(fminf(fmaxf(rintf(__fdiv_rn(x, q.s)), q.lo), q.hi), 0.0f);
 }
 
+// Two elements: m = lo - code (an integer held as a float), and the larger distance of z n from an integer
+__device__ __forceinline__ float2 dq_codes2(const float2 &v, const QuantScale &q, float &dist)
+{
+    const float MAGIC = 12582912.0f;                   // 1.5 * 2^23
+    const float2 z = make_float2(__saturatef(__fmaf_rn(v.x, q.k, q.off)), __saturatef(__fmaf_rn(v.y, q.k, q.off)));
+    const float2 m = __fadd2_rn(__ffma2_rn(z, make_float2(-q.n, -q.n), make_float2(MAGIC, MAGIC)), make_float2(-MAGIC, -MAGIC));
+    const float2 d = __ffma2_rn(z, make_float2(q.n, q.n), m);
+    dist = fmaxf(dist, fmaxf(fabsf(d.x), fabsf(d.y)));
+    return m;
+}
+
 // codes (as floats, integer values in [lo, hi]) and dequantised values of four elements
 __device__ __forceinline__ void dq_fq4(const float4 &v, const QuantScale &q, float4 &codes, float4 &deq)
 {
-    const float MAGIC = 12582912.0f;                   // 1.5 * 2^23
-    bool done = false;
-    if (q.fast) {
-        const float2 r2 = make_float2(q.r, q.r), m2 = make_float2(MAGIC, MAGIC), nm2 = make_float2(-MAGIC, -MAGIC);
-        const float2 va = make_float2(v.x, v.y), vb = make_float2(v.z, v.w), neg1 = make_float2(-1.f, -1.f);
-        const float2 ra = __fadd2_rn(__ffma2_rn(va, r2, m2), nm2), rb = __fadd2_rn(__ffma2_rn(vb, r2, m2), nm2);    // rint(x * r)
-        const float2 da = __ffma2_rn(va, r2, __fmul2_rn(ra, neg1)), db = __ffma2_rn(vb, r2, __fmul2_rn(rb, neg1)); // x * r - rint(x * r)
-        const float m = fmaxf(fmaxf(fabsf(da.x), fabsf(da.y)), fmaxf(fabsf(db.x), fabsf(db.y)));
-        const float c = fmaxf(fmaxf(fabsf(ra.x), fabsf(ra.y)), fmaxf(fabsf(rb.x), fabsf(rb.y)));
-        if (m < q.tie_lim && c <= q.hi) {              // (with a fresh scale every code lies inside: nothing to clamp)
-            codes = make_float4(ra.x, ra.y, rb.x, rb.y);
-            done = true;
-        } else if (m < q.tie_lim) {
-            codes = make_float4(fminf(fmaxf(ra.x, q.lo), q.hi), fminf(fmaxf(ra.y, q.lo), q.hi),
-                                fminf(fmaxf(rb.x, q.lo), q.hi), fminf(fmaxf(rb.y, q.lo), q.hi));
-            done = true;
-        }
-    }
-    if (!done)
+    float dist = q.fast ? 0.f : 1.f;
+    const float2 ma = dq_codes2(make_float2(v.x, v.y), q, dist), mb = dq_codes2(make_float2(v.z, v.w), q, dist);
+    if (dist < q.tie_lim) {
+        const float2 neg1 = make_float2(-1.f, -1.f), lo2 = make_float2(q.lo, q.lo);
+        const float2 ns2 = make_float2(-q.s, -q.s), los2 = make_float2(q.lo * q.s, q.lo * q.s);
+        const float2 ca = __ffma2_rn(ma, neg1, lo2), cb = __ffma2_rn(mb, neg1, lo2);
+        const float2 ea = __ffma2_rn(ma, ns2, los2), eb = __ffma2_rn(mb, ns2, los2);
+        codes = make_float4(ca.x, ca.y, cb.x, cb.y);
+        deq = make_float4(ea.x, ea.y, eb.x, eb.y);
+    } else {
         codes = make_float4(dq_codef_ieee(v.x, q), dq_codef_ieee(v.y, q), dq_codef_ieee(v.z, q), dq_codef_ieee(v.w, q));
-    const float2 s2 = make_float2(q.s, q.s);
-    const float2 ea = __fmul2_rn(make_float2(codes.x, codes.y), s2), eb = __fmul2_rn(make_float2(codes.z, codes.w), s2);
-    deq = make_float4(ea.x, ea.y, eb.x, eb.y);
+        deq = make_float4(__fmul_rn(codes.x, q.s), __fmul_rn(codes.y, q.s), __fmul_rn(codes.z, q.s), __fmul_rn(codes.w, q.s));
+    }
 }
 
+// Dequantised values of N elements of one table (N even) with one check for all of them
+template <int N>
+__device__ __forceinline__ void dq_fq_many(const float (&x)[N], const QuantScale &q, float (&deq)[N])
+{
+    const float2 ns2 = make_float2(-q.s, -q.s), los2 = make_float2(q.lo * q.s, q.lo * q.s);
+    float dist = q.fast ? 0.f : 1.f;
+#pragma unroll
+    for (int k = 0; k < N; k += 2) {
+        const float2 e = __ffma2_rn(dq_codes2(make_float2(x[k], x[k + 1]), q, dist), ns2, los2);
+        deq[k] = e.x;
+        deq[k + 1] = e.y;
+    }
+    if (!(dist < q.tie_lim)) {
+#pragma unroll
+        for (int k = 0; k < N; ++k) deq[k] = __fmul_rn(dq_codef_ieee(x[k], q), q.s);
+    }
+}
 
 // asks L2 for the 128-byte line that holds p (no register, no scoreboard entry: the later load finds it there)
 __device__ __forceinline__ void dq_prefetch_l2(const void *p) { asm volatile("prefetch.global.L2 [%0];\n" ::"l"(p)); }

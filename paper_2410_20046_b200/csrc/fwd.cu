@@ -140,6 +140,31 @@ fwd_onehot_kernel(const FwdArgs a)
         float4 *out_lane = reinterpret_cast<float4 *>(a.out) + ((int64_t)i0 * a.T + t) * d4 + lane;
 
         // ---- rows, RPW per step, NB steps in flight
+        if (one == 0xffffffffu) {                  // (nearly always: no checks)
+#pragma unroll 1
+            for (int k0 = 0; k0 < 32; k0 += RPW * NB) {
+                int32_t ib[NB];
+#pragma unroll
+                for (int b = 0; b < NB; ++b) ib[b] = __shfl_sync(0xffffffffu, idx, (k0 + b * RPW + grp) & 31);
+#pragma unroll
+                for (int c = 0; c < CH; ++c) {
+                    const bool on = EXACT || c * LPR + lane < d4;
+                    float4 v[NB];
+#pragma unroll
+                    for (int b = 0; b < NB; ++b)           // the update reads the row again
+                        v[b] = dq_ld_nc(tbl_lane + (int64_t)ib[b] * d4 + (on ? c * LPR : -lane), keep);
+#pragma unroll
+                    for (int b = 0; b < NB; ++b) {
+                        const int bag = k0 + b * RPW + grp;
+                        float4 cd, f;
+                        dq_fq4(v[b], tc.qs, cd, f);
+                        if (on && (RPW * NB <= 32 || bag < 32))
+                            __stcs(out_lane + (int64_t)bag * TD4 + c * LPR, f);     // written once, read by nobody here
+                    }
+                }
+            }
+            continue;
+        }
 #pragma unroll 1
         for (int k0 = 0; k0 < 32; k0 += RPW * NB) {
             if ((one >> k0) == 0u) break;
@@ -181,18 +206,36 @@ fwd_onehot_kernel(const FwdArgs a)
     if (bad) dq_report(a.status, DQRM_ERR_INDEX_RANGE);
 }
 
+// VEC consecutive floats (2 or 4)
+template <int VEC> struct Vec;
+template <> struct Vec<2> { typedef float2 type; };
+template <> struct Vec<4> { typedef float4 type; };
+__device__ __forceinline__ void unpack(const float2 &v, float *x) { x[0] = v.x; x[1] = v.y; }
+__device__ __forceinline__ void unpack(const float4 &v, float *x) { x[0] = v.x; x[1] = v.y; x[2] = v.z; x[3] = v.w; }
+__device__ __forceinline__ void store_sum(float2 *o, const double (&a)[2]) { *o = make_float2((float)a[0], (float)a[1]); }
+__device__ __forceinline__ void store_sum(float4 *o, const double (&a)[4])
+{
+    *o = make_float4((float)a[0], (float)a[1], (float)a[2], (float)a[3]);
+}
+
 // A lane group walks one bag at a time.  The bag's indices are loaded LPR at a time, one per lane, and checked once;
 // the rows are then fetched NB at a time, their numbers handed round by shuffle, and summed in bag order.  Measured on
 // B200 the kernel is bound by instruction issue (rows of hot tables come from the caches), which is why nothing is done
-// per row by every lane that one lane can do, and why whole batches of NB rows carry no range checks.
-template <int LPR, int CH, bool EXACT, bool CODES>
+// per row by every lane that one lane can do, why the quantiser checks NB rows at once, and why rows of 36 to 64
+// features in long bags take a whole warp with two features a lane: lane groups that walk bags of different lengths
+// side by side wait for each other (8.5 M lookups of 256-byte rows, cold: 646 us with the indices loaded by every
+// lane, 460 by lane groups, 354 by warps; four rows at a time: eight take 386, sixteen 497, the last batch of a bag
+// being padded).  In bags of a few indices the offsets' and the indices' latency counts, and twice as many bags in
+// flight are worth more (64 K lookups, three a bag, 36 features: 28 against 34 us).
+template <int LPR, int VEC, int CH, bool EXACT, bool CODES>
 __global__ void __launch_bounds__(FW_THREADS)
 fwd_bags_kernel(const FwdArgs a)
 {
-    constexpr int NB = NBOf<LPR, CH>::v < LPR ? NBOf<LPR, CH>::v : LPR;
+    typedef typename Vec<VEC>::type vec_t;
+    constexpr int NB = CH >= 2 ? 1 : LPR < 4 ? LPR : 4;
     constexpr int GPB = FW_THREADS / LPR;
-    const int D = EXACT ? 4 * LPR * CH : a.D;
-    const int d4 = D >> 2;
+    const int D = EXACT ? VEC * LPR * CH : a.D;
+    const int dv = D / VEC;
     const int t = blockIdx.y;
     const int lane = threadIdx.x % LPR;
     const int grp = threadIdx.x / LPR;
@@ -203,52 +246,76 @@ fwd_bags_kernel(const FwdArgs a)
     for (int i = blockIdx.x * GPB + grp; i < a.B; i += gridDim.x * GPB) {
         int32_t lo = __ldg(a.offsets + tc.g0 + i), hi = __ldg(a.offsets + tc.g0 + i + 1);
         if (lo < 0 || hi < lo || (int64_t)hi > a.L) { bad = true; hi = lo = 0; }
-        double acc[CH][4];
+        double acc[CH][VEC];
 #pragma unroll
-        for (int c = 0; c < CH; ++c) acc[c][0] = acc[c][1] = acc[c][2] = acc[c][3] = 0.0;
+        for (int c = 0; c < CH; ++c)
+#pragma unroll
+            for (int q = 0; q < VEC; ++q) acc[c][q] = 0.0;
         int32_t mine = lo + lane < hi ? __ldg(a.indices + lo + lane) : 0;
         for (int32_t j0 = lo; j0 < hi; j0 += LPR) {
             const int32_t row = clamp_index(mine, tc.nrows, bad);      // (lanes past the bag's end hold row 0)
-            if (j0 + LPR + lane < hi) mine = __ldg(a.indices + j0 + LPR + lane); else mine = 0;
+            mine = j0 + LPR + lane < hi ? __ldg(a.indices + j0 + LPR + lane) : 0;
             const int cnt = min(LPR, hi - j0);
             auto rows = [&](int b0, auto full_tag) {
                 constexpr bool FULL = decltype(full_tag)::value;
 #pragma unroll
                 for (int c = 0; c < CH; ++c) {
-                    const int c4 = c * LPR + lane;
-                    float4 v[NB];
+                    const int cv = c * LPR + lane;
+                    vec_t v[NB];
 #pragma unroll
                     for (int b = 0; b < NB; ++b) {
                         const int32_t r = __shfl_sync(gmask, row, b0 + b, LPR);
-                        v[b] = __ldg(reinterpret_cast<const float4 *>(tc.tbl + (int64_t)r * D) + (EXACT || c4 < d4 ? c4 : 0));
+                        v[b] = __ldg(reinterpret_cast<const vec_t *>(tc.tbl + (int64_t)r * D) + (EXACT || cv < dv ? cv : 0));
+                    }
+                    float x[NB * VEC], f[NB * VEC];
+#pragma unroll
+                    for (int b = 0; b < NB; ++b) unpack(v[b], x + b * VEC);
+                    if constexpr (CODES) {
+#pragma unroll
+                        for (int b = 0; b < NB; ++b) {
+                            float4 cd, fq;
+                            dq_fq4(make_float4(x[b * VEC], x[b * VEC + 1], x[b * VEC + 2], x[b * VEC + 3]), tc.qs, cd, fq);
+                            f[b * VEC] = fq.x; f[b * VEC + 1] = fq.y; f[b * VEC + 2] = fq.z; f[b * VEC + 3] = fq.w;
+                            if ((FULL || b0 + b < cnt) && (EXACT || cv < dv)) store_codes(a.codes_out, j0 + b0 + b, D, cv, cd);
+                        }
+                    } else {
+                        dq_fq_many<NB * VEC>(x, tc.qs, f);
                     }
 #pragma unroll
-                    for (int b = 0; b < NB; ++b) {
-                        if (FULL || b0 + b < cnt) {
-                            float4 cd, f;
-                            dq_fq4(v[b], tc.qs, cd, f);
-                            acc[c][0] += (double)f.x;
-                            acc[c][1] += (double)f.y;
-                            acc[c][2] += (double)f.z;
-                            acc[c][3] += (double)f.w;
-                            if (CODES && (EXACT || c4 < d4)) store_codes(a.codes_out, j0 + b0 + b, D, c4, cd);
-                        }
-                    }
+                    for (int b = 0; b < NB; ++b)
+                        if (FULL || b0 + b < cnt)
+#pragma unroll
+                            for (int q = 0; q < VEC; ++q) acc[c][q] += (double)f[b * VEC + q];
                 }
             };
             int b0 = 0;
             for (; b0 + NB <= cnt; b0 += NB) rows(b0, std::true_type{});
             if (b0 < cnt) rows(b0, std::false_type{});
         }
-        float4 *o = reinterpret_cast<float4 *>(a.out + ((int64_t)i * a.T + t) * D);
+        vec_t *o = reinterpret_cast<vec_t *>(a.out + ((int64_t)i * a.T + t) * D);
 #pragma unroll
         for (int c = 0; c < CH; ++c) {
-            const int c4 = c * LPR + lane;
-            if (EXACT || c4 < d4)
-                o[c4] = make_float4((float)acc[c][0], (float)acc[c][1], (float)acc[c][2], (float)acc[c][3]);
+            const int cv = c * LPR + lane;
+            if (EXACT || cv < dv) store_sum(o + cv, acc[c]);
         }
     }
     if (bad) dq_report(a.status, DQRM_ERR_INDEX_RANGE);
+}
+
+// rows of 36 to 64 features: a warp per bag from eight indices a bag on
+inline bool warp_per_bag(const FwdArgs &a, int lpr) { return lpr == 16 && !a.codes_out && a.L >= 8 * (int64_t)a.T * a.B; }
+
+template <int LPR, int CH, bool EXACT>
+void launch_bags(const FwdArgs &a, dim3 grid, cudaStream_t st)
+{
+    if constexpr (LPR == 16) {
+        if (warp_per_bag(a, LPR)) {
+            fwd_bags_kernel<32, 2, CH, EXACT, false><<<grid, FW_THREADS, 0, st>>>(a);
+            return;
+        }
+    }
+    if (a.codes_out) fwd_bags_kernel<LPR, 4, CH, EXACT, true><<<grid, FW_THREADS, 0, st>>>(a);
+    else fwd_bags_kernel<LPR, 4, CH, EXACT, false><<<grid, FW_THREADS, 0, st>>>(a);
 }
 
 template <int LPR, int CH, bool EXACT>
@@ -257,15 +324,14 @@ int launch2(dqrm_ctx *ctx, const FwdArgs &a, cudaStream_t st)
     constexpr int GPB = FW_THREADS / LPR;
     // the one-index kernel does not emit codes; a caller that asks for them gets the general kernel
     const bool onehot = a.L == (int64_t)a.T * a.B && a.codes_out == nullptr;
-    const int per_block = onehot ? FW_THREADS : GPB;
+    const int per_block = onehot ? FW_THREADS : warp_per_bag(a, LPR) ? GPB / 2 : GPB;
     int bx = (a.B + per_block - 1) / per_block;
     const int cap = (ctx->num_sms * 32 + ctx->T - 1) / ctx->T;     // a few waves over all tables
     if (bx > cap) bx = cap;
     if (bx < 1) bx = 1;
     dim3 grid((unsigned)bx, (unsigned)ctx->T);
     if (onehot) fwd_onehot_kernel<LPR, CH, EXACT><<<grid, FW_THREADS, 0, st>>>(a);
-    else if (a.codes_out) fwd_bags_kernel<LPR, CH, EXACT, true><<<grid, FW_THREADS, 0, st>>>(a);
-    else fwd_bags_kernel<LPR, CH, EXACT, false><<<grid, FW_THREADS, 0, st>>>(a);
+    else launch_bags<LPR, CH, EXACT>(a, grid, st);
     DQRM_CUDA_TRY(ctx, cudaGetLastError());
     dq_mark(ctx, st, DQ_K_FWD);
     return DQRM_OK;
