@@ -15,6 +15,8 @@ namespace {
 
 constexpr int PK_THREADS = 256;
 constexpr int PK_CHUNK4 = 4096;          // 128-bit vectors per chunk
+constexpr int PK_UNROLL = 8;             // vectors of a thread in flight (one at a time: 427 us for 2.16 GB at 4 bits, eight: 405,
+                                         // sixteen: 437; block and chunk sizes make no difference)
 
 template <int BITS>
 __device__ __forceinline__ u32 pack4(const float4 &codes)
@@ -48,6 +50,22 @@ pack_kernel(const float4 *__restrict__ arena4, const int64_t *__restrict__ row_o
         const int t0 = dq_table_of(v4_off, T, c0);
         const bool one_table = c1 <= v4_off[t0 + 1];
         QuantScale qs = dq_make_scale(__ldg(scales + t0), BITS);
+        if (one_table && c1 - c0 == PK_CHUNK4) {
+            // a thread's vectors of PK_UNROLL rounds are all in flight before the first is quantised
+#pragma unroll 1
+            for (int r = 0; r < PK_CHUNK4; r += PK_THREADS * PK_UNROLL) {
+                float4 v[PK_UNROLL];
+#pragma unroll
+                for (int k = 0; k < PK_UNROLL; ++k) v[k] = __ldcs(arena4 + c0 + r + k * PK_THREADS + threadIdx.x);
+#pragma unroll
+                for (int k = 0; k < PK_UNROLL; ++k) {
+                    float4 cd, dq;
+                    dq_fq4(v[k], qs, cd, dq);
+                    store_packed<BITS>(packed, c0 + r + k * PK_THREADS + threadIdx.x, pack4<BITS>(cd));
+                }
+            }
+            continue;
+        }
         for (int64_t i = c0 + threadIdx.x; i < c1; i += PK_THREADS) {
             if (!one_table) qs = dq_make_scale(__ldg(scales + dq_table_of(v4_off, T, i)), BITS);
             float4 cd, dq;
@@ -58,8 +76,10 @@ pack_kernel(const float4 *__restrict__ arena4, const int64_t *__restrict__ row_o
 }
 
 // ---- packed lookups -------------------------------------------------------------------
-// A lane owns EPL consecutive elements of a row (8 when the feature size allows, else 4): one
-// load of EPL*BITS/8 bytes, EPL/4 128-bit stores.
+// A lane owns EPL consecutive elements of a row: one load of EPL*BITS/8 bytes, EPL/4 128-bit stores.  Four where a
+// warp covers a one-index row that way (D <= 128): a store instruction then fills whole sectors, while with eight
+// elements every store writes 16 bytes of each 32 (852 K rows of 64 features at 4 bits: 56 us with eight, 44 with four).
+// A pooled bag is stored once for many loads and takes eight.
 template <int BITS, int EPL>
 struct Unit {
     static constexpr int BYTES = BITS * EPL / 8;
@@ -220,6 +240,32 @@ packed_fwd_onehot_kernel(const PfArgs a)
         const unsigned one = __ballot_sync(0xffffffffu, single);
         unsigned rare = __ballot_sync(0xffffffffu, (i < a.B) && !single);
         float4 *out_lane = reinterpret_cast<float4 *>(a.out) + ((int64_t)i0 * a.T + t) * (a.D >> 2) + lane * (EPL / 4);
+        if (one == 0xffffffffu) {                      // (nearly always: no checks)
+#pragma unroll 1
+            for (int k0 = 0; k0 < 32; k0 += RPW * NB) {
+                int32_t ib[NB];
+#pragma unroll
+                for (int b = 0; b < NB; ++b) ib[b] = __shfl_sync(0xffffffffu, idx, (k0 + b * RPW + grp) & 31);
+#pragma unroll
+                for (int c = 0; c < CH; ++c) {
+                    const bool on = c * LPR + lane < units;
+                    const int u = on ? c * LPR + lane : 0;
+                    Unit<BITS, EPL> v[NB];
+#pragma unroll
+                    for (int b = 0; b < NB; ++b) v[b].load(a.packed, (r0 + ib[b]) * units + u);
+#pragma unroll
+                    for (int b = 0; b < NB; ++b) {
+                        const int bag = k0 + b * RPW + grp;
+                        if (on && (RPW * NB <= 32 || bag < 32)) {
+                            float4 *o = out_lane + (int64_t)bag * TD4 + c * LPR * (EPL / 4);
+                            __stcs(o, scale4(v[b].template quad<0>(), s));         // written once, read by nobody here
+                            if constexpr (EPL == 8) __stcs(o + 1, scale4(v[b].template quad<1>(), s));
+                        }
+                    }
+                }
+            }
+            continue;
+        }
 #pragma unroll 1
         for (int k0 = 0; k0 < 32; k0 += RPW * NB) {
             if ((one >> k0) == 0u) break;
@@ -309,7 +355,8 @@ int dispatch_pfwd2(dqrm_ctx *ctx, const PfArgs &a, cudaStream_t st)
 template <int BITS>
 int dispatch_pfwd(dqrm_ctx *ctx, const PfArgs &a, cudaStream_t st)
 {
-    if (a.D % 8 == 0) return dispatch_pfwd2<BITS, 8>(ctx, a, st);
+    const bool onehot = a.L == (int64_t)a.T * a.B;
+    if (a.D % 8 == 0 && (a.D > 128 || !onehot)) return dispatch_pfwd2<BITS, 8>(ctx, a, st);
     return dispatch_pfwd2<BITS, 4>(ctx, a, st);
 }
 
