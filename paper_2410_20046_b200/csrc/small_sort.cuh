@@ -1,0 +1,288 @@
+// Per-table stable sort of a small batch's lookups by row: one block per table, a bitonic network over
+// (row, position) held in registers.  At a few hundred to a few thousand lookups a table the radix sort of
+// cluster_sort.cuh is all fixed cost (digit tables, cluster barriers, three passes for large tables): 128 lookups a table take
+// 3.5 us here and 12.3 there.  The network needs log2(n) (log2(n) + 1) / 2 steps whatever the row count; most of them
+// stay inside a warp, and unrolled they cost about 0.15 us each (with the steps in a loop, 1.5 times that).
+//
+// Every thread holds EPT consecutive entries: steps across less than EPT entries are register moves, across less than
+// 32 * EPT shuffles, wider ones go through shared memory (two buffers in turn, one barrier a step).  Row and position
+// make every key distinct, so the order is that of a stable sort.  A table with more lookups than the block holds
+// (an uneven batch) is sorted by the block in global memory instead, with 8-bit digits: slow, but it need not be fast.
+// The lists that it leaves are those of the cluster sort's lists_by_table.
+#pragma once
+#include "cluster_sort.cuh"
+
+namespace ssort {
+
+typedef unsigned long long u64;
+
+constexpr int MAX_THREADS = 1024;
+
+inline size_t smem_bytes(int threads, int ept)
+{
+    const size_t net = (size_t)threads * ept * 2 * sizeof(u64);
+    const size_t digits = (size_t)(threads / 32) * csort::BINS * sizeof(u32);
+    return net > digits ? net : digits;
+}
+
+__host__ __device__ constexpr int log2c(int x) { return x <= 1 ? 0 : 1 + log2c(x / 2); }
+
+__device__ __forceinline__ u64 shfl_xor64(u64 v, int mask)
+{
+    return __shfl_xor_sync(0xffffffffu, v, mask);
+}
+
+// (row within the table, payload) of the lookup at position p of table t
+__device__ __forceinline__ uint2 lookup(const csort::Args &a, int t, int64_t tb0, int64_t n, int64_t nrows, int64_t p, bool &bad)
+{
+    const int32_t *off_t = a.offsets + (int64_t)t * a.B;
+    int32_t idx = __ldg(a.indices + tb0 + p);
+    bool single = false;
+    if (n == a.B) {
+        const int64_t o0 = __ldg(off_t + p), o1 = __ldg(off_t + p + 1);
+        single = o0 == tb0 + p && o1 == tb0 + p + 1;
+        bad |= o0 > o1;
+    }
+    bad |= (idx < 0) | (idx >= nrows);
+    idx = (int32_t)min((int64_t)max(idx, 0), nrows - 1);
+    int64_t bag = p;
+    if (!single) {                                 // largest bag b with offsets[t*B + b] <= tb0 + p
+        int lo = 0, hi = a.B;
+        while (hi - lo > 1) {
+            const int mid = (lo + hi) >> 1;
+            if ((int64_t)__ldg(off_t + mid) <= tb0 + p) lo = mid; else hi = mid;
+        }
+        bag = lo;
+    }
+    return make_uint2((u32)idx, a.payload_position ? (u32)(tb0 + p) : (u32)(bag * a.T + t));
+}
+
+// The block's table in global memory, 8 bits a pass; returns the buffer that holds the result
+template <int THREADS>
+__device__ __noinline__ const uint2 *sort_in_memory(const csort::Args &a, int t, int64_t tb0, int64_t n, int64_t nrows, u32 *s_cnt)
+{
+    constexpr int WARPS = THREADS / 32, BINS = csort::BINS;
+    __shared__ u32 s_scan[BINS / 32];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    bool bad = false;
+    for (int64_t p = threadIdx.x; p < n; p += THREADS) a.gp[0][tb0 + p] = lookup(a, t, tb0, n, nrows, p, bad);
+    if (bad) dq_report(a.status, DQRM_ERR_INDEX_RANGE);
+    __syncthreads();
+    const int64_t part = ((n + WARPS - 1) / WARPS + 31) / 32 * 32;
+    const int64_t w0 = min(n, (int64_t)warp * part), w1 = min(n, w0 + part);
+    int s = 0;
+    for (int shift = 0; ((int64_t)1 << shift) < nrows; shift += 8) {
+        const uint2 *src = a.gp[s] + tb0;
+        uint2 *dst = a.gp[s ^ 1] + tb0;
+        for (int i = threadIdx.x; i < WARPS * BINS; i += THREADS) s_cnt[i] = 0u;
+        __syncthreads();
+        for (int64_t i = w0 + lane; i < w1; i += 32) atomicAdd(&s_cnt[warp * BINS + ((src[i].x >> shift) & 255u)], 1u);
+        __syncthreads();
+        u32 tot = 0, incl = 0;
+        if (threadIdx.x < BINS) {
+            for (int w = 0; w < WARPS; ++w) tot += s_cnt[w * BINS + threadIdx.x];
+            incl = tot;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const u32 v = __shfl_up_sync(0xffffffffu, incl, o);
+                if (lane >= o) incl += v;
+            }
+            if (lane == 31) s_scan[warp] = incl;
+        }
+        __syncthreads();
+        if (threadIdx.x < BINS) {
+            u32 run = incl - tot;
+            for (int w = 0; w < warp; ++w) run += s_scan[w];
+            for (int w = 0; w < WARPS; ++w) {
+                const u32 c = s_cnt[w * BINS + threadIdx.x];
+                s_cnt[w * BINS + threadIdx.x] = run;
+                run += c;
+            }
+        }
+        __syncthreads();
+        for (int64_t i0 = w0; i0 < w1; i0 += 32) {
+            const bool valid = i0 + lane < w1;
+            const uint2 pr = valid ? src[i0 + lane] : make_uint2(0u, 0u);
+            const u32 d = (pr.x >> shift) & 255u;
+            const u32 peers = csort::same_digit_lanes(d, valid);
+            const int leader = __ffs(peers) - 1;
+            u32 base = 0;
+            if (valid && lane == leader) { base = s_cnt[warp * BINS + d]; s_cnt[warp * BINS + d] = base + __popc(peers); }
+            base = __shfl_sync(0xffffffffu, base, leader & 31);
+            __syncwarp();
+            if (valid) dst[base + __popc(peers & ((1u << lane) - 1u))] = pr;
+        }
+        __syncthreads();
+        s ^= 1;
+    }
+    return a.gp[s] + tb0;
+}
+
+template <int THREADS, int EPT>
+__global__ void __launch_bounds__(THREADS)
+small_sort_kernel(const csort::Args a)
+{
+    constexpr int WARPS = THREADS / 32, N = THREADS * EPT;
+    extern __shared__ u64 s_net[];                 // [2][N]
+    __shared__ u32 s_warp[WARPS];
+    __shared__ u32 s_total;
+    const int t = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int64_t tb0 = __ldg(a.offsets + (int64_t)t * a.B), tb1 = __ldg(a.offsets + (int64_t)(t + 1) * a.B);
+    if (tb0 < 0 || tb1 < tb0 || tb1 > a.L || (t == 0 && tb0 != 0) || (t == a.T - 1 && tb1 != a.L)) {
+        if (tid == 0) {
+            dq_report(a.status, DQRM_ERR_INDEX_RANGE);
+            a.table_cnt[t] = a.cnt_broken;         // nothing downstream runs
+        }
+        return;
+    }
+    const int64_t n = tb1 - tb0, r0 = __ldg(a.row_off + t), nrows = __ldg(a.row_off + t + 1) - r0;
+    if (tid == 0) {
+        a.tb[t] = (u32)tb0;
+        if (t == a.T - 1) a.tb[a.T] = (u32)tb1;
+        a.absmax[t] = 0u;
+        if (n == 0) a.table_cnt[t] = 0u;
+    }
+    bool bad = false;
+    if (n != a.B)                                  // (otherwise every lookup looks at its own bag's offsets)
+        for (int i = tid; i < a.B; i += THREADS) bad |= __ldg(a.offsets + (int64_t)t * a.B + i) > __ldg(a.offsets + (int64_t)t * a.B + i + 1);
+    if (bad) dq_report(a.status, DQRM_ERR_INDEX_RANGE);
+    if (n == 0) return;
+    const uint2 *mem = nullptr;                    // the sorted pairs of a table that does not fit the block
+    u64 e[EPT];                                    // row << 32 | position, later row << 32 | payload
+    if (n > N) {
+        mem = sort_in_memory<THREADS>(a, t, tb0, n, nrows, reinterpret_cast<u32 *>(s_net));
+    } else {
+        u32 pay[EPT];
+#pragma unroll
+        for (int k = 0; k < EPT; ++k) {            // (loads coalesced: thread tid takes entries tid, tid + THREADS, ...)
+            const int p = k * THREADS + tid;
+            e[k] = ~0ull;
+            pay[k] = 0u;
+            if (p < n) {
+                const uint2 pr = lookup(a, t, tb0, n, nrows, p, bad);
+                e[k] = (u64)pr.x << 32 | (u32)p;
+                pay[k] = pr.y;
+            }
+        }
+        if (bad) dq_report(a.status, DQRM_ERR_INDEX_RANGE);
+        int top = 1;                               // entries that the network covers: a power of two from 32 * EPT on
+        while ((1 << top) < n) ++top;
+        u64 *buf = s_net;
+        if (EPT > 1) {                             // to EPT consecutive entries per thread
+#pragma unroll
+            for (int k = 0; k < EPT; ++k) buf[k * THREADS + tid] = e[k];
+            __syncthreads();
+#pragma unroll
+            for (int k = 0; k < EPT; ++k) e[k] = buf[tid * EPT + k];
+            buf = s_net + N;
+        }
+        const int i0 = tid * EPT;                  // first entry of this thread
+        constexpr int TOP = log2c(N);
+#pragma unroll
+        for (int p = 1; p <= TOP; ++p) {
+            if (p > top) break;                    // (block-uniform)
+#pragma unroll
+            for (int s = p - 1; s >= 0; --s) {
+                const int stride = 1 << s;
+                if (stride >= 32 * EPT) {
+#pragma unroll
+                    for (int k = 0; k < EPT; ++k) buf[i0 + k] = e[k];
+                    __syncthreads();
+                    const bool up = ((i0 >> p) & 1) == 0, low = (i0 & stride) == 0;
+#pragma unroll
+                    for (int k = 0; k < EPT; ++k) {
+                        const u64 o = buf[(i0 + k) ^ stride];
+                        e[k] = (up == low) == (e[k] < o) ? e[k] : o;
+                    }
+                    buf = buf == s_net ? s_net + N : s_net;
+                } else if (stride >= EPT) {
+                    const bool up = ((i0 >> p) & 1) == 0, low = (i0 & stride) == 0;
+#pragma unroll
+                    for (int k = 0; k < EPT; ++k) {
+                        const u64 o = shfl_xor64(e[k], stride / EPT);
+                        e[k] = (up == low) == (e[k] < o) ? e[k] : o;
+                    }
+                } else {
+#pragma unroll
+                    for (int k = 0; k < EPT; ++k) {
+                        if ((k & stride) == 0) {
+                            const bool up = (((i0 + k) >> p) & 1) == 0;
+                            const u64 x = e[k], y = e[(k + stride) % EPT];
+                            const bool swap = up ? y < x : x < y;
+                            e[k] = swap ? y : x;
+                            e[(k + stride) % EPT] = swap ? x : y;
+                        }
+                    }
+                }
+            }
+        }
+        // the payloads come back by position
+        __syncthreads();
+        u32 *s_pay = reinterpret_cast<u32 *>(s_net);
+#pragma unroll
+        for (int k = 0; k < EPT; ++k) s_pay[k * THREADS + tid] = pay[k];
+        __syncthreads();
+#pragma unroll
+        for (int k = 0; k < EPT; ++k)
+            if (i0 + k < n) e[k] = (e[k] & 0xffffffff00000000ull) | s_pay[(u32)e[k]];
+        __syncthreads();
+        u64 *s_out = s_net;
+#pragma unroll
+        for (int k = 0; k < EPT; ++k) s_out[i0 + k] = e[k];
+        __syncthreads();
+    }
+    // ---- sorted keys and payloads, and where the segments stand: THREADS consecutive entries at a time
+    u32 *segs = a.seg_start + tb0 + t;
+    const u32 ck_mask = (1u << a.ck_shift) - 1u;
+    u32 base = 0;                                  // segments that begin before these entries
+    for (int64_t c0 = 0; c0 < n; c0 += THREADS) {
+        const int64_t i = c0 + tid, j = tb0 + i;
+        bool head = false;
+        if (i < n) {
+            u32 row, pay, prev;
+            if (mem) {
+                row = mem[i].x;
+                pay = mem[i].y;
+                prev = i > 0 ? mem[i - 1].x : ~row;
+            } else {
+                row = (u32)(s_net[i] >> 32);
+                pay = (u32)s_net[i];
+                prev = i > 0 ? (u32)(s_net[i - 1] >> 32) : ~row;
+            }
+            a.keys_out[j] = (u32)(r0 + row);
+            a.vals_out[j] = pay;
+            head = row != prev;
+        }
+        const u32 m = __ballot_sync(0xffffffffu, head);
+        if (lane == 0) s_warp[warp] = __popc(m);
+        __syncthreads();
+        if (warp == 0) {
+            const u32 v = lane < WARPS ? s_warp[lane] : 0u;
+            u32 incl = v;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const u32 x = __shfl_up_sync(0xffffffffu, incl, o);
+                if (lane >= o) incl += x;
+            }
+            if (lane < WARPS) s_warp[lane] = incl - v;
+            if (lane == 31) s_total = incl;
+        }
+        __syncthreads();
+        if (i < n) {
+            const u32 upto = base + s_warp[warp] + __popc(m & (0xffffffffu >> (31 - lane)));      // segment starts in [0, i]
+            if (head) segs[upto - 1] = (u32)j;
+            if (((u32)j & ck_mask) == 0u) {
+                a.chunk_first[j >> a.ck_shift] = upto - 1;
+                a.tile_done[j >> a.ck_shift] = 0u;
+            }
+        }
+        base += s_total;
+        __syncthreads();
+    }
+    if (tid == 0) {
+        a.table_cnt[t] = base;
+        segs[base] = (u32)tb1;                     // the slot behind the last segment holds the table's end
+    }
+}
+
+}  // namespace ssort

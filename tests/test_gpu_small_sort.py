@@ -1,0 +1,37 @@
+"""GPU parity of the block sort of small batches at its edges: around each block size, uneven tables that do not fit
+the block, one lookup, one row, many tables."""
+import numpy as np
+import pytest
+
+from dqrm_inputs import workloads as W
+from gpu_util import Case, bit_equal
+
+pytestmark = pytest.mark.gpu
+
+# lookups per table
+COUNTS = {
+    "around_256": [255, 256, 257, 1], "around_512": [512, 511, 513, 0], "around_1024": [1024, 1023, 1025, 1024],
+    "one_table_holds_all": [0, 3, 4000, 0], "single": [1], "many_tables": [2048, 2047, 31, 32, 33] * 16,
+}
+
+
+@pytest.mark.parametrize("rows", [1, 7, 300, 70_000])
+@pytest.mark.parametrize("name", list(COUNTS))
+def test_block_sort(oracle, name, rows):
+    counts = COUNTS[name]
+    B, D = max(1, max(counts)), 8
+    wl = W.Workload("small", tuple(max(1, rows + t) for t in range(len(counts))), D=D, B=B, alpha=None)
+    rng = np.random.default_rng(rows + B)
+    idx = np.concatenate([rng.integers(0, wl.rows[t], n) for t, n in enumerate(counts)]).astype(np.int32)
+    lens = np.zeros((wl.T, B), dtype=np.int64)
+    for t, n in enumerate(counts):                  # some bags empty, some with several indices
+        np.add.at(lens[t], rng.integers(0, B, n) if t % 2 else np.arange(n), 1)
+    off = np.concatenate([[0], np.cumsum(lens.reshape(-1))]).astype(np.int32)
+    go = rng.standard_normal((B, wl.T, D)).astype(np.float32)
+    c = Case(wl, max_lookups=len(idx))
+    ur, uo, gr = c.gpu_bwd(idx, off, go)
+    o_ur, o_uo, o_gr = oracle.emb_bwd(go, wl.T, D, B, idx, off)
+    assert bit_equal(uo, o_uo) and bit_equal(ur, o_ur)
+    # at most 4000 terms of magnitude below 6 in FP64 in two orders, each sum rounded once
+    np.testing.assert_allclose(gr, o_gr, rtol=2.0 ** -23, atol=12.0 * 4000 ** 2 * 2.0 ** -53)
+    c.ctx.close()
