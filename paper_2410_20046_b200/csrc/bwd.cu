@@ -14,6 +14,7 @@
 // The sort is stable and every sum has a fixed shape, so results are reproducible bit
 // for bit.  The per-table abs-max of the summed gradient (needed by the INT8 gradient
 // quantiser) is folded into the last kernel.
+#include <algorithm>
 #include "common.cuh"
 #include "seg_reduce.cuh"
 #include "cluster_sort.cuh"
@@ -30,11 +31,14 @@ constexpr int ST_WARPS = ST_THREADS / 32;
 struct Layout {
     int passes, digit_bits;                    // radix sort: digits of the row number within a table
     int64_t radix_tiles, num_tiles;
-    int sum_shift;                             // the summing kernel: log2 of its tile of sorted entries, tiles,
-    int64_t sum_tiles, sum_ranges;             // ranges of range_tiles tiles (at most sum_ranges)
+    // the summing kernel: log2 of the entries between two of chunk_first, small tiles, tiles, at most sum_ranges ranges of
+    // range_tiles tiles
+    int sum_shift;
+    bool sum_small;
+    int64_t sum_tiles, sum_ranges;
     int range_tiles;
     size_t absmax, tile_heads, tile0, tile_table, totals, tilehist;
-    size_t keys_a, vals_a, pairs_a, pairs_b, seg_start, chunk_first, tile_done, partials, table_cnt, tb;
+    size_t keys_a, vals_a, pairs_a, pairs_b, seg_start, chunk_first, tile_done, partials, group_partials, table_cnt, tb;
     size_t total;
 };
 
@@ -47,11 +51,13 @@ Layout make_layout(const dqrm_ctx *ctx, int64_t L)
     y.num_tiles = (Lc + ST_TILE - 1) / ST_TILE;
     y.radix_tiles = rsort::max_tiles(ctx->T, Lc);
     // the sum: every warp that the GPU holds at once walks one range of tiles
-    const int lpr = segred::lanes_per_row(ctx->D), I = segred::tile_entries(lpr);
-    y.sum_shift = dq_log2c(I);
-    y.sum_tiles = (Lc + I - 1) >> y.sum_shift;
+    const int lpr = segred::lanes_per_row(ctx->D);
     int64_t warps = (int64_t)ctx->num_sms * segred::blocks_per_sm(lpr) / segred::column_blocks(ctx->D) * segred::WARPS;
     if (warps < 1) warps = 1;
+    y.sum_small = Lc < 32 * warps;
+    const int I = segred::tile_entries(lpr, y.sum_small);
+    y.sum_shift = segred::chunk_shift(lpr, y.sum_small);
+    y.sum_tiles = (Lc + I - 1) / I;
     y.sum_ranges = y.sum_tiles < warps ? y.sum_tiles : warps;
     y.range_tiles = (int)((y.sum_tiles + warps - 1) / warps);
     size_t o = 0;
@@ -69,9 +75,10 @@ Layout make_layout(const dqrm_ctx *ctx, int64_t L)
     y.seg_start = take(sizeof(u32) * (Lc + ctx->T + 1));     // (lists by table: one slot more per table)
     y.table_cnt = take(sizeof(u32) * ctx->T);
     y.tb = take(sizeof(u32) * (ctx->T + 1));
-    y.chunk_first = take(sizeof(u32) * y.sum_tiles);
-    y.tile_done = take(sizeof(u32) * y.sum_tiles);
-    y.partials = take(sizeof(double) * y.sum_ranges * 2 * ctx->D);
+    y.chunk_first = take(sizeof(u32) * (Lc / 8 + 1));      // (the most that any L up to this one may need)
+    y.tile_done = take(sizeof(uint2) * (Lc / 8 + 1));
+    y.partials = take(sizeof(double) * std::min(Lc / 8 + 1, warps) * 2 * ctx->D);
+    y.group_partials = take(sizeof(double) * (std::min(Lc / 8 + 1, warps) / segred::FOLD_GROUP + 1) * 2 * ctx->D);
     y.total = o;
     return y;
 }
@@ -115,7 +122,7 @@ __global__ void __launch_bounds__(ST_THREADS)
 seg_emit_kernel(const u32 *__restrict__ keys, int64_t L, const u32 *__restrict__ tile_heads,
                 const int64_t *__restrict__ row_off, int T,
                 u32 *__restrict__ seg_start, u32 *__restrict__ chunk_first,
-                int32_t *__restrict__ unique_rows, int32_t *__restrict__ uniq_off, u32 *__restrict__ tile_done,
+                int32_t *__restrict__ unique_rows, int32_t *__restrict__ uniq_off, uint2 *__restrict__ tile_done,
                 u32 *__restrict__ absmax, int ck_shift)
 {
     extern __shared__ unsigned char smem_raw[];
@@ -205,7 +212,7 @@ seg_emit_kernel(const u32 *__restrict__ keys, int64_t L, const u32 *__restrict__
     // the chunks that begin among this thread's entries (a chunk is a power of two, at least eight entries)
     if ((i0 & (int64_t)(ck - 1)) == 0) {
         chunk_first[i0 >> ck_shift] = heads_before + (heads & 1u) - 1u;
-        tile_done[i0 >> ck_shift] = 0u;
+        tile_done[i0 >> ck_shift] = make_uint2(0u, 0u);
     }
     if (i0 + n == L) {
         const u32 U = heads_before + __popc(heads);
@@ -216,14 +223,20 @@ seg_emit_kernel(const u32 *__restrict__ keys, int64_t L, const u32 *__restrict__
 
 // ---------------------------------------------------------------------------------
 template <int LPR, int VEC>
-int launch_sum(dqrm_ctx *ctx, const segred::Args &a, cudaStream_t st)
+int launch_sum(dqrm_ctx *ctx, const segred::Args &a, bool small, cudaStream_t st)
 {
     using namespace segred;
     const size_t smem = smem_bytes(ctx->T);
     const int64_t ranges = (a.num_tiles + a.range_tiles - 1) / a.range_tiles;
     const dim3 grid((unsigned)((ranges + WARPS - 1) / WARPS), (unsigned)column_blocks(ctx->D));
-    if (ctx->D == LPR * VEC) seg_sum_kernel<LPR, VEC, true><<<grid, THREADS, smem, st>>>(a);
-    else seg_sum_kernel<LPR, VEC, false><<<grid, THREADS, smem, st>>>(a);
+    const bool exact = ctx->D == LPR * VEC;
+    if (LPR == 32 && small) {
+        if (exact) seg_sum_kernel<LPR, VEC, true, LPR == 32><<<grid, THREADS, smem, st>>>(a);
+        else seg_sum_kernel<LPR, VEC, false, LPR == 32><<<grid, THREADS, smem, st>>>(a);
+    } else {
+        if (exact) seg_sum_kernel<LPR, VEC, true, false><<<grid, THREADS, smem, st>>>(a);
+        else seg_sum_kernel<LPR, VEC, false, false><<<grid, THREADS, smem, st>>>(a);
+    }
     DQRM_CUDA_TRY(ctx, cudaGetLastError());
     dq_mark(ctx, st, DQ_K_SEG_SUM);
     return DQRM_OK;
@@ -394,7 +407,7 @@ int dq_launch_bwd_sort(dqrm_ctx *ctx, const int32_t *indices, const int32_t *off
         ca.chunk_first = reinterpret_cast<u32 *>(ws + y.chunk_first);
         ca.table_cnt = reinterpret_cast<u32 *>(ws + y.table_cnt);
         ca.tb = reinterpret_cast<u32 *>(ws + y.tb);
-        ca.tile_done = reinterpret_cast<u32 *>(ws + y.tile_done);
+        ca.tile_done = reinterpret_cast<uint2 *>(ws + y.tile_done);
         ca.absmax = reinterpret_cast<u32 *>(ws + y.absmax);
         ca.ck_shift = y.sum_shift;
         ca.cnt_broken = segred::CNT_BROKEN;
@@ -445,7 +458,7 @@ int dq_launch_bwd_sort(dqrm_ctx *ctx, const int32_t *indices, const int32_t *off
     seg_emit_kernel<<<(unsigned)y.num_tiles, ST_THREADS, (size_t)(ctx->T + 1) * sizeof(int64_t), st>>>(
         skeys, L, reinterpret_cast<const u32 *>(ws + y.tile_heads), ctx->d_row_off, ctx->T,
         reinterpret_cast<u32 *>(ws + y.seg_start), reinterpret_cast<u32 *>(ws + y.chunk_first), unique_rows, uniq_off,
-        reinterpret_cast<u32 *>(ws + y.tile_done), reinterpret_cast<u32 *>(ws + y.absmax), y.sum_shift);
+        reinterpret_cast<uint2 *>(ws + y.tile_done), reinterpret_cast<u32 *>(ws + y.absmax), y.sum_shift);
     DQRM_CUDA_TRY(ctx, cudaGetLastError());
     dq_mark(ctx, st, DQ_K_SEG_EMIT);
     return DQRM_OK;
@@ -465,7 +478,7 @@ int dq_launch_bwd_sum(dqrm_ctx *ctx, const float *grad_out, int32_t *unique_rows
     a.vals = reinterpret_cast<const u32 *>(ws + y.vals_a);
     a.seg_start = reinterpret_cast<const u32 *>(ws + y.seg_start);
     a.chunk_first = reinterpret_cast<const u32 *>(ws + y.chunk_first);
-    a.range_done = reinterpret_cast<u32 *>(ws + y.tile_done);
+    a.range_done = reinterpret_cast<uint2 *>(ws + y.tile_done);
     a.by_table = by_table ? 1 : 0;
     a.table_cnt = reinterpret_cast<const u32 *>(ws + y.table_cnt);
     a.tb = reinterpret_cast<const u32 *>(ws + y.tb);
@@ -473,18 +486,19 @@ int dq_launch_bwd_sum(dqrm_ctx *ctx, const float *grad_out, int32_t *unique_rows
     a.unique_rows = unique_rows; a.uniq_off = uniq_off;
     a.grad_out = grad_out; a.grad_rows = grad_rows;
     a.partials = reinterpret_cast<double *>(ws + y.partials);
+    a.group_partials = reinterpret_cast<double *>(ws + y.group_partials);
     a.absmax = reinterpret_cast<u32 *>(ws + y.absmax);
     a.T = ctx->T; a.D = ctx->D;
     a.L = L; a.G = (int64_t)ctx->T * B; a.num_tiles = y.sum_tiles;
     a.range_tiles = y.range_tiles;
     a.status = ctx->d_status;
     const int D = ctx->D;
-    if (D <= 4) return launch_sum<4, 1>(ctx, a, st);
-    if (D <= 8) return launch_sum<4, 2>(ctx, a, st);
-    if (D <= 16) return launch_sum<4, 4>(ctx, a, st);
-    if (D <= 32) return launch_sum<8, 4>(ctx, a, st);
-    if (D <= 64) return launch_sum<32, 2>(ctx, a, st);
-    return launch_sum<32, 4>(ctx, a, st);
+    if (D <= 4) return launch_sum<4, 1>(ctx, a, y.sum_small, st);
+    if (D <= 8) return launch_sum<4, 2>(ctx, a, y.sum_small, st);
+    if (D <= 16) return launch_sum<4, 4>(ctx, a, y.sum_small, st);
+    if (D <= 32) return launch_sum<8, 4>(ctx, a, y.sum_small, st);
+    if (D <= 64) return launch_sum<32, 2>(ctx, a, y.sum_small, st);
+    return launch_sum<32, 4>(ctx, a, y.sum_small, st);
 }
 
 int dq_launch_bwd(dqrm_ctx *ctx, const float *grad_out, const int32_t *indices, const int32_t *offsets,

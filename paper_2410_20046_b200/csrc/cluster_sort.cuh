@@ -52,7 +52,8 @@ struct Args {
     // and zeroes what the kernel behind it counts in (tile_done[c], absmax[t]); that kernel, which sums the segments,
     // adds the tables' bases
     int lists_by_table;
-    u32 *seg_start, *chunk_first, *table_cnt, *tb, *tile_done, *absmax;
+    u32 *seg_start, *chunk_first, *table_cnt, *tb, *absmax;
+    uint2 *tile_done;
     int ck_shift;
     u32 cnt_broken;
 };
@@ -365,7 +366,7 @@ cluster_sort_kernel(const Args a)
                     if (head) segs[upto - 1] = (u32)j;
                     if (((u32)j & ck_mask) == 0u) {
                         a.chunk_first[j >> a.ck_shift] = upto - 1;
-                        a.tile_done[j >> a.ck_shift] = 0u;
+                        a.tile_done[j >> a.ck_shift] = make_uint2(0u, 0u);
                     }
                 }
                 before_me += __popc(m);

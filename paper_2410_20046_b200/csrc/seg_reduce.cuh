@@ -2,7 +2,7 @@
 // Section 4.3 / Appendix B.1: duplicates of a row are coalesced).
 //
 // Input: keys[L] (arena rows, ascending), vals[L] (row of grad_out for each lookup, in stable order),
-// chunk_first[c] = index of the segment that holds sorted entry c*I, seg_start[] = sorted position where
+// chunk_first[c] = index of the segment that holds sorted entry c << chunk_shift, seg_start[] = sorted position where
 // every segment begins; the segments are numbered over the whole batch, or per table (Args::by_table), and
 // in the second case this kernel also writes unique_rows and uniq_off.
 //
@@ -14,7 +14,9 @@
 // more take the whole warp: every branch on a run's end is then uniform and a run that goes on is simply carried in
 // registers.  Narrower rows are taken by 32/LPR lane groups at once, C consecutive entries each; a segmented scan over
 // the groups (shuffles) joins the runs that cross them.  Only a run cut by the edge of a warp's range leaves a partial
-// in global memory; the warp that brings a run's last partial adds all of them, in order (nobody waits).  All sums are
+// in global memory; the warp that brings a run's last partial adds all of them, in order (nobody waits; the pieces of a
+// long run are first added by groups of 32 ranges, or one warp's chain over hundreds of them is what the kernel waits
+// for).  All sums are
 // FP64 and have a shape fixed by the entry positions and the launch, so results are reproducible.  The per-table
 // abs-max of the rounded sums is collected on the way.
 //
@@ -28,6 +30,7 @@ namespace segred {
 
 constexpr int THREADS = 256;
 constexpr int WARPS = THREADS / 32;
+constexpr u32 FOLD_GROUP = 32;               // ranges whose pieces of one run are added before the groups' sums are
 constexpr u32 CNT_BROKEN = 0xFFFFFFFFu;      // table_cnt[t]: the table's boundary offsets were unusable (reported)
 
 // lanes per row and features per lane for feature size D (D > 128: 128 features per block of the grid's y)
@@ -37,16 +40,22 @@ __host__ __device__ constexpr int column_blocks(int D) { return (D + 127) / 128;
 // rows of a lane group in flight, entries of a tile, resident blocks.  Lane groups: eight rows and two blocks (with
 // three the kernel spills and takes 31 us instead of 25 at 426 K rows of 64 bytes); whole warps: 4 KB in flight (two
 // batches in turn) and three blocks (four blocks: 78 instead of 71 us at 852 K rows of 256 bytes)
-__host__ __device__ constexpr int batch_entries(int lpr, int vec) { return lpr == 32 ? 16 / vec : 8; }
-__host__ __device__ constexpr int tile_entries(int lpr) { return lpr == 4 ? 64 : 32; }
+__host__ __device__ constexpr int batch_entries(int lpr, int vec, bool small) { return lpr == 32 ? (small ? 4 : 16 / vec) : 8; }
+// A warp that has one tile takes its batches of rows one after the other, 4 to 8 us for 32 rows, so a batch of wide
+// rows that would not even give every resident warp a tile of 32 entries is cut into tiles of 8
+__host__ __device__ constexpr int tile_entries(int lpr, bool small) { return lpr == 4 ? 64 : lpr == 32 && small ? 8 : 32; }
+__host__ __device__ constexpr int chunk_shift(int lpr, bool small) { return lpr == 32 && small ? 3 : 5; }    // of chunk_first
 __host__ __device__ constexpr int blocks_per_sm(int lpr) { return lpr == 32 ? 3 : 2; }
 
 struct Args {
     const u32 *keys, *vals, *seg_start, *chunk_first;
-    u32 *range_done;            // [ranges] zero: partials that have arrived for the run that begins in a range
+    // zero: .x [range] partials that have arrived for the run that begins in a range, .y [group][2] for a run of many
+    // pieces, those of its pieces that lie in a group of 32 ranges (the run that comes into the group, the one that begins
+    // in it)
+    uint2 *range_done;
     // by_table: the cluster sort numbered each table's segments from 0: table t's starts sit at
     // seg_start[tb[t] + t + .] (tb[t] = first sorted position of the table, one slot more than it has segments: the
-    // last holds the table's end), chunk_first[c] counts within the table that holds entry c*I, table_cnt[t] says
+    // last holds the table's end), chunk_first[c] counts within the table that holds entry c << chunk_shift, table_cnt[t] says
     // how many segments the table has (CNT_BROKEN: nothing is summed, no row is updated); unique_rows and uniq_off
     // are then written here, with the tables' bases added
     int by_table;
@@ -56,6 +65,7 @@ struct Args {
     const float *grad_out;
     float *grad_rows;
     double *partials;           // [ranges][2][D]: run that enters the range, run that leaves it
+    double *group_partials;     // [ranges / 32 + 1][2][D]: the same for groups of 32 ranges
     u32 *absmax;                // [T] zero
     int T, D;
     int64_t L, G, num_tiles;
@@ -138,14 +148,14 @@ __device__ __noinline__ void note_max(u32 *absmax, const u32 *s_uoff, int t_firs
 }
 
 // blockIdx.x * WARPS + warp: range of tiles; blockIdx.y: block of 128 features (one unless D > 128)
-template <int LPR, int VEC, bool EXACT>
+template <int LPR, int VEC, bool EXACT, bool SMALL>
 __global__ void __launch_bounds__(THREADS, blocks_per_sm(LPR))
 seg_sum_kernel(const Args a)
 {
-    constexpr int C = batch_entries(LPR, VEC);    // rows of a lane group in flight
+    constexpr int C = batch_entries(LPR, VEC, SMALL);    // rows of a lane group in flight
     constexpr int GP = 32 / LPR;                  // lane groups of the warp
-    constexpr int I = tile_entries(LPR);
-    constexpr int W = I / 32;                     // index words per lane, words of head bits
+    constexpr int I = tile_entries(LPR, SMALL);
+    constexpr int W = (I + 31) / 32;              // index words per lane, words of head bits
     constexpr int NB = I / (GP * C);              // batches per tile (one when the warp has several groups)
     static_assert(GP == 1 ? NB % 2 == 0 : NB == 1, "");
     typedef typename Vec<VEC>::type vec_t;
@@ -164,14 +174,14 @@ seg_sum_kernel(const Args a)
     const u32 tile1 = min((u32)a.num_tiles, tile0 + (u32)a.range_tiles);
 
     // ---- indices of a tile, one entry per lane and word.  An entry starts a segment when its key differs from the key
-    // before it; entries past the end count as heads, so that the last run closes like any other
+    // before it
     u32 kn[W], vn[W], kp[W];
     auto fetch = [&](u32 tile) {
 #pragma unroll
         for (int w = 0; w < W; ++w) {
             const int64_t i = (int64_t)tile * I + w * 32 + wl;
             kn[w] = vn[w] = kp[w] = 0u;
-            if (i < a.L) {
+            if (i < a.L && (I % 32 == 0 || wl < I)) {
                 kn[w] = __ldg(a.keys + i);
                 vn[w] = __ldg(a.vals + i);
                 kp[w] = i > 0 ? __ldg(a.keys + i - 1) : ~kn[w];
@@ -179,18 +189,17 @@ seg_sum_kernel(const Args a)
         }
     };
     u32 kc[W], vc[W], hw[W];                      // the present tile's keys, payloads and head bits
-    auto take = [&](u32 tile) {
+    auto take = [&]() {
 #pragma unroll
         for (int w = 0; w < W; ++w) {
-            const bool past = (int64_t)tile * I + w * 32 + wl >= a.L;
-            hw[w] = __ballot_sync(0xffffffffu, past || kn[w] != kp[w]);
+            hw[w] = __ballot_sync(0xffffffffu, kn[w] != kp[w]);       // (equal past the end)
             kc[w] = kn[w];
             vc[w] = vn[w];
             if ((int64_t)vc[w] >= a.G) { dq_report(a.status, DQRM_ERR_INDEX_RANGE); vc[w] = 0u; }
         }
     };
     fetch(tile0);
-    u32 u_base = tile0 < tile1 ? a.chunk_first[tile0] : 0u;
+    u32 u_base = tile0 < tile1 ? a.chunk_first[(int64_t)tile0 * I >> chunk_shift(LPR, SMALL)] : 0u;
     if (a.by_table) {
         if (threadIdx.x < 32) {                   // the tables' first segments: a running sum over their counts
             u32 run = 0;
@@ -244,6 +253,7 @@ seg_sum_kernel(const Args a)
         const int bytes = (EXACT ? D : min(D - c0, LPR * VEC)) * (int)sizeof(float);
 #pragma unroll
         for (int w = 0; w < W; ++w) {
+            if (I % 32 != 0 && wl >= I) break;
             const char *row = reinterpret_cast<const char *>(a.grad_out + (int64_t)((int64_t)vn[w] < a.G ? vn[w] : 0u) * D + c0);
 #pragma unroll
             for (int b = 0; b < LPR * VEC * 4; b += 128)
@@ -251,7 +261,7 @@ seg_sum_kernel(const Args a)
             if (!EXACT) dq_prefetch_l2(row + bytes - 4);      // (rows that do not begin on a line's start)
         }
     };
-    take(tile0);
+    take();
     request(0, v[0]);
     fetch(tile0 + 1);
 
@@ -289,7 +299,7 @@ seg_sum_kernel(const Args a)
 
     for (u32 tile = tile0; tile < tile1; ++tile) {
         const int n = (int)min((int64_t)I, a.L - (int64_t)tile * I);
-        u32 n_heads = __popc(hw[0]) - (n < I ? I - n : 0);
+        u32 n_heads = __popc(hw[0]);
         if (W == 2) n_heads += __popc(hw[W - 1]);
         // the table of the run that is open when the tile begins (of the first entry's when none is)
         const bool fresh = tile == tile0 && head0;
@@ -311,13 +321,13 @@ seg_sum_kernel(const Args a)
         if (tile + 1 < tile1) prefetch();
         if constexpr (GP == 1) {
             u32 u = u_base;
-            const u32 heads = n < I ? hw[0] & ((1u << n) - 1u) : hw[0];
+            const u32 heads = hw[0];
 #pragma unroll
             for (int b = 0; b < NB; ++b) {
                 if (b + 1 < NB) {
                     request(b + 1, v[(b + 1) & 1]);
                 } else if (tile + 1 < tile1) {
-                    take(tile + 1);
+                    take();
                     request(0, v[0]);
                     fetch(tile + 2);
                 }
@@ -343,9 +353,8 @@ seg_sum_kernel(const Args a)
         } else {
             const u32 word = W == 2 && grp * C >= 32 ? hw[W - 1] : hw[0];
             const int es = grp * C, sh = es & 31;
-            u32 hb = (word >> sh) & ((1u << C) - 1u);
+            const u32 hb = (word >> sh) & ((1u << C) - 1u);
             const int nv = min(max(n - es, 0), C);
-            if (nv < C) hb &= (1u << nv) - 1u;
             const u32 before = __popc(word & ((1u << sh) - 1u)) + (W == 2 && es >= 32 ? __popc(hw[0]) : 0);
             u32 u = u_base + before;              // the run that is open when the group begins
             const u32 u_in = u;
@@ -375,7 +384,7 @@ seg_sum_kernel(const Args a)
             const bool enters_lead = open_lead;
             open_lead = open_lead && n_heads == 0u;
             if (tile + 1 < tile1) {
-                take(tile + 1);
+                take();
                 request(0, v[0]);
                 fetch(tile + 2);
             }
@@ -421,7 +430,8 @@ seg_sum_kernel(const Args a)
 
     // ---- the warp that brings a cut run's last piece adds the pieces
     if (!(cut_lead || cut_trail)) return;
-    u32 last = 0, first_range = 0;
+    const u32 group = range / FOLD_GROUP;
+    u32 last = 0, first_range = 0, groups = 0;    // pieces to add here; the run's first range; its groups, when it has many pieces
     if (wl == 0 ? cut_lead : (wl == 1 && cut_trail)) {
         const u32 u = wl == 0 ? u_lead : u_base;
         const int t = last_not_above(s_uoff, 0, T, u);
@@ -429,50 +439,81 @@ seg_sum_kernel(const Args a)
         const u32 R = (u32)a.range_tiles * I;
         const u32 sa = __ldg(a.seg_start + at), sb = __ldg(a.seg_start + at + 1);
         first_range = sa / R;
-        const u32 pieces = (sb - 1) / R - first_range + 1;
+        const u32 last_range = (sb - 1) / R, g0 = first_range / FOLD_GROUP;
+        u32 pieces = last_range - first_range + 1;
+        u32 *arrived = &a.range_done[first_range].x;
+        if (pieces > FOLD_GROUP) {
+            groups = last_range / FOLD_GROUP - g0 + 1;
+            pieces = min(last_range, group * FOLD_GROUP + FOLD_GROUP - 1) - max(first_range, group * FOLD_GROUP) + 1;
+            arrived = &a.range_done[2 * group + (group == g0 ? 1 : 0)].y;
+        }
         __threadfence();
-        last = atomicAdd(a.range_done + first_range, 1u) == pieces * gridDim.y - 1u ? pieces : 0u;
+        last = atomicAdd(arrived, 1u) == pieces * gridDim.y - 1u ? pieces : 0u;
         __threadfence();
     }
     __syncwarp();
+    // adds np partials of D features each (`at(p)` = where piece p lies), this lane's features of columns cc
+    auto fold = [&](int np, int cc, double (&sum)[VEC], auto at) {
+#pragma unroll
+        for (int x = 0; x < VEC; ++x) sum[x] = 0.0;
+        for (int p0 = grp; (EXACT || cc < dv) && p0 < np; p0 += 8 * GP) {
+            double x[8][VEC];
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+                const int p = p0 + j * GP;
+                const double *src = at(min(p, np - 1)) + cc * VEC;
+#pragma unroll
+                for (int q = 0; q < VEC; ++q) x[j][q] = p < np ? __ldcg(src + q) : 0.0;
+            }
+#pragma unroll
+            for (int j = 0; j < 8; ++j)
+#pragma unroll
+                for (int q = 0; q < VEC; ++q) sum[q] += x[j][q];
+        }
+#pragma unroll
+        for (int o = LPR; o < 32; o <<= 1)
+#pragma unroll
+            for (int x = 0; x < VEC; ++x) sum[x] += __shfl_xor_sync(0xffffffffu, sum[x], o);
+    };
+    auto store_total = [&](u32 u, int cc, const double (&sum)[VEC]) {
+        if (grp == 0) {
+            float x = 0.f;
+            if (EXACT || cc < dv) st_row(reinterpret_cast<vec_t *>(a.grad_rows + (int64_t)u * D) + cc, rounded(sum, x), keep);
+            note_max<LPR>(a.absmax, s_uoff, 0, T, u, x);
+        }
+        __syncwarp();
+    };
 #pragma unroll 1
-    for (int q = 0; q < 2; ++q) {
+    for (int q = 0; q < 2; ++q) {                 // (columns: all of them, the blocks of the others are done too)
         const int np = (int)__shfl_sync(0xffffffffu, last, q);
         if (np == 0) continue;
-        const u32 u = q ? u_base : u_lead;
-        const double *pieces = a.partials + (size_t)__shfl_sync(0xffffffffu, first_range, q) * 2 * D;
-        for (int col = 0; col < dv; col += LPR) { // all features: the blocks of the other columns are done too
-            const int cc = col + lane;
-            const bool in = EXACT || cc < dv;
+        const u32 u = q ? u_base : u_lead, f = __shfl_sync(0xffffffffu, first_range, q);
+        const u32 ng = __shfl_sync(0xffffffffu, groups, q), g0 = f / FOLD_GROUP;
+        const u32 p_first = ng ? max(f, group * FOLD_GROUP) : f;
+        for (int cc = lane; cc - lane < dv; cc += LPR) {
             double sum[VEC];
+            fold(np, cc, sum, [&](int p) { return a.partials + ((size_t)(p_first + p) * 2 + (p_first + p == f ? 1 : 0)) * D; });
+            if (ng == 0) {
+                store_total(u, cc, sum);
+            } else if (grp == 0 && (EXACT || cc < dv)) {
 #pragma unroll
-            for (int x = 0; x < VEC; ++x) sum[x] = 0.0;
-            // (a small batch's hottest row has a piece per tile: eight of them in flight, or its chain is what the
-            // kernel waits for)
-            for (int p0 = grp; in && p0 < np; p0 += 8 * GP) {
-                double x[8][VEC];
-#pragma unroll
-                for (int j = 0; j < 8; ++j) {
-                    const int p = p0 + j * GP;
-#pragma unroll
-                    for (int q2 = 0; q2 < VEC; ++q2)
-                        x[j][q2] = p < np ? __ldcg(pieces + ((size_t)p * 2 + (p == 0 ? 1 : 0)) * D + cc * VEC + q2) : 0.0;
-                }
-#pragma unroll
-                for (int j = 0; j < 8; ++j)
-#pragma unroll
-                    for (int q2 = 0; q2 < VEC; ++q2) sum[q2] += x[j][q2];
+                for (int x = 0; x < VEC; ++x) a.group_partials[((size_t)group * 2 + (group == g0 ? 1 : 0)) * D + cc * VEC + x] = sum[x];
             }
-#pragma unroll
-            for (int o = LPR; o < 32; o <<= 1)
-#pragma unroll
-                for (int x = 0; x < VEC; ++x) sum[x] += __shfl_xor_sync(0xffffffffu, sum[x], o);
-            if (grp == 0) {
-                float x = 0.f;
-                if (in) st_row(reinterpret_cast<vec_t *>(a.grad_rows + (int64_t)u * D) + cc, rounded(sum, x), keep);
-                note_max<LPR>(a.absmax, s_uoff, 0, T, u, x);
-            }
+        }
+        if (ng) {
             __syncwarp();
+            bool final = false;
+            if (wl == 0) {
+                __threadfence();
+                final = atomicAdd(&a.range_done[f].x, 1u) == ng - 1u;
+                __threadfence();
+            }
+            if (!__shfl_sync(0xffffffffu, final, 0)) continue;
+            for (int cc = lane; cc - lane < dv; cc += LPR) {
+                double sum[VEC];
+                fold((int)ng, cc, sum, [&](int p) { return a.group_partials + ((size_t)(g0 + p) * 2 + (p == 0 ? 1 : 0)) * D; });
+                store_total(u, cc, sum);
+            }
         }
     }
 }

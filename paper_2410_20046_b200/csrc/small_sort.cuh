@@ -273,7 +273,7 @@ small_sort_kernel(const csort::Args a)
             if (head) segs[upto - 1] = (u32)j;
             if (((u32)j & ck_mask) == 0u) {
                 a.chunk_first[j >> a.ck_shift] = upto - 1;
-                a.tile_done[j >> a.ck_shift] = 0u;
+                a.tile_done[j >> a.ck_shift] = make_uint2(0u, 0u);
             }
         }
         base += s_total;
