@@ -1,4 +1,5 @@
-"""ctypes binding of ``libdqrm_b200.so``: argument marshalling only."""
+"""Binding of ``libdqrm_b200.so``: argument marshalling only.  The calls that a training or serving loop makes go
+through the native module ``_dqrm_native`` (csrc/binding.cpp), the others through ctypes."""
 from __future__ import annotations
 
 import ctypes
@@ -68,7 +69,13 @@ SIGNATURES = {
     "dqrm_kernel_count": (_i, []),
 }
 
+# functions that the native module calls, in the order in which it wants their addresses
+NATIVE = ("dqrm_scale_refresh", "dqrm_emb_fwd", "dqrm_emb_bwd", "dqrm_grad_quant_int8", "dqrm_row_update",
+          "dqrm_train_step", "dqrm_sort_batch", "dqrm_train_step_sorted", "dqrm_train_step_host", "dqrm_pack_tables",
+          "dqrm_packed_fwd")
+
 _lib = None
+_native = None
 
 
 class DqrmError(RuntimeError):
@@ -97,6 +104,23 @@ def load_library(path: Optional[str] = None):
     if path is None:
         _lib = lib
     return lib
+
+
+def load_native():
+    """The native module, bound to the loaded library.  Raises if it has not been built: there is no fallback."""
+    global _native
+    if _native is None:
+        import torch  # noqa: F401  (its libraries must be loaded before the module's)
+
+        lib = load_library()
+        try:
+            from . import _dqrm_native as native
+        except ImportError as e:
+            raise ImportError(f"the native binding is missing ({e}): build it with "
+                              "`python -m paper_2410_20046_b200.build`") from e
+        native.bind(*[ctypes.cast(getattr(lib, name), _vp).value for name in NATIVE])
+        _native = native
+    return _native
 
 
 def _ptr(t, dtype=None, device="cuda"):
@@ -131,6 +155,8 @@ class Context:
         import torch
 
         self.lib = load_library()
+        self._n = load_native()
+        self._hv = 0
         self.T = len(row_off) - 1
         self.D = int(D)
         arr = (_i64 * (self.T + 1))(*[int(x) for x in row_off])
@@ -138,6 +164,7 @@ class Context:
         rc = self.lib.dqrm_create(ctypes.byref(h), self.T, self.D, arr)
         self._h = h if rc == OK else None
         self._check("dqrm_create", rc)
+        self._hv = h.value
         self.max_lookups = int(max_lookups)
         self.max_bags = int(max_bags)
         self.workspace_bytes = int(self.lib.dqrm_workspace_bytes(self._h, self.max_lookups, self.max_bags))
@@ -167,6 +194,7 @@ class Context:
         if getattr(self, "_h", None):
             self.lib.dqrm_destroy(self._h)
             self._h = None
+            self._hv = 0
 
     def __del__(self):
         try:
@@ -226,18 +254,14 @@ class Context:
         return int(self.lib.dqrm_packed_bytes(self._h, int(bits)))
 
     def pack_tables(self, tables, scales, bits, packed, stream=None):
-        import torch
-
-        self._check("dqrm_pack_tables", self.lib.dqrm_pack_tables(
-            self._h, _ptr(tables, torch.float32), _ptr(scales, torch.float32), int(bits), _ptr(packed, torch.uint8),
-            _stream(stream)))
+        rc = self._n.pack_tables(self._hv, tables, scales, bits, packed, stream)
+        if rc:
+            self._check("dqrm_pack_tables", rc)
 
     def packed_fwd(self, packed, indices, offsets, scales, bits, out, *, B, L, stream=None):
-        import torch
-
-        self._check("dqrm_packed_fwd", self.lib.dqrm_packed_fwd(
-            self._h, _ptr(packed, torch.uint8), _ptr(indices, torch.int32), _ptr(offsets, torch.int32),
-            _ptr(scales, torch.float32), int(bits), _ptr(out, torch.float32), int(B), int(L), _stream(stream)))
+        rc = self._n.packed_fwd(self._hv, packed, indices, offsets, scales, bits, out, B, L, stream)
+        if rc:
+            self._check("dqrm_packed_fwd", rc)
 
     # ---- table-sharded forward payload ----
     def emb_fwd_codes(self, tables, indices, offsets, scales, bits, payload, *, B, L, stream=None):
@@ -276,52 +300,38 @@ class Context:
 
     # ---- the calls of include/dqrm.h ----
     def scale_refresh(self, tables, bits, scales, minmax=None, stream=None):
-        import torch
-
-        self._check("dqrm_scale_refresh", self.lib.dqrm_scale_refresh(
-            self._h, _ptr(tables, torch.float32), _ptr(bits, torch.int32), _ptr(scales, torch.float32),
-            _ptr(minmax, torch.float32), self._scratch_ptr, self.scratch_bytes, _stream(stream)))
+        rc = self._n.scale_refresh(self._hv, tables, bits, scales, minmax, self._scratch_ptr, self.scratch_bytes, stream)
+        if rc:
+            self._check("dqrm_scale_refresh", rc)
 
     def emb_fwd(self, tables, indices, offsets, scales, bits, out, codes_out=None, *, B, L, stream=None):
-        import torch
-
-        self._check("dqrm_emb_fwd", self.lib.dqrm_emb_fwd(
-            self._h, _ptr(tables, torch.float32), _ptr(indices, torch.int32), _ptr(offsets, torch.int32),
-            _ptr(scales, torch.float32), _ptr(bits, torch.int32), _ptr(out, torch.float32),
-            _ptr(codes_out, torch.int8), int(B), int(L), _stream(stream)))
+        rc = self._n.emb_fwd(self._hv, tables, indices, offsets, scales, bits, out, codes_out, B, L, stream)
+        if rc:
+            self._check("dqrm_emb_fwd", rc)
 
     def emb_bwd(self, grad_out, indices, offsets, unique_rows, uniq_off, grad_rows, *, B, L, stream=None):
-        import torch
-
-        self._check("dqrm_emb_bwd", self.lib.dqrm_emb_bwd(
-            self._h, _ptr(grad_out, torch.float32), _ptr(indices, torch.int32), _ptr(offsets, torch.int32),
-            _ptr(unique_rows, torch.int32), _ptr(uniq_off, torch.int32), _ptr(grad_rows, torch.float32),
-            int(B), int(L), self._ws_ptr, self.workspace_bytes, _stream(stream)))
+        rc = self._n.emb_bwd(self._hv, grad_out, indices, offsets, unique_rows, uniq_off, grad_rows, B, L, self._ws_ptr,
+                             self.workspace_bytes, stream)
+        if rc:
+            self._check("dqrm_emb_bwd", rc)
 
     def grad_quant_int8(self, grad_rows, uniq_off, codes, grad_scales, stream=None):
-        import torch
-
-        self._check("dqrm_grad_quant_int8", self.lib.dqrm_grad_quant_int8(
-            self._h, _ptr(grad_rows, torch.float32), _ptr(uniq_off, torch.int32), _ptr(codes, torch.int8),
-            _ptr(grad_scales, torch.float32), self._scratch_ptr, self.scratch_bytes, _stream(stream)))
+        rc = self._n.grad_quant_int8(self._hv, grad_rows, uniq_off, codes, grad_scales, self._scratch_ptr,
+                                     self.scratch_bytes, stream)
+        if rc:
+            self._check("dqrm_grad_quant_int8", rc)
 
     def row_update(self, tables, unique_rows, uniq_off, codes, grad_scales, lr, stream=None):
-        import torch
-
-        self._check("dqrm_row_update", self.lib.dqrm_row_update(
-            self._h, _ptr(tables, torch.float32), _ptr(unique_rows, torch.int32), _ptr(uniq_off, torch.int32),
-            _ptr(codes, torch.int8), _ptr(grad_scales, torch.float32), float(lr), _stream(stream)))
+        rc = self._n.row_update(self._hv, tables, unique_rows, uniq_off, codes, grad_scales, lr, stream)
+        if rc:
+            self._check("dqrm_row_update", rc)
 
     def train_step(self, tables, indices, offsets, grad_out, scales, bits, out, unique_rows, uniq_off,
                    grad_rows, codes, grad_scales, lr, *, B, L, stream=None):
-        import torch
-
-        self._check("dqrm_train_step", self.lib.dqrm_train_step(
-            self._h, _ptr(tables, torch.float32), _ptr(indices, torch.int32), _ptr(offsets, torch.int32),
-            _ptr(grad_out, torch.float32), _ptr(scales, torch.float32), _ptr(bits, torch.int32),
-            _ptr(out, torch.float32), _ptr(unique_rows, torch.int32), _ptr(uniq_off, torch.int32),
-            _ptr(grad_rows, torch.float32), _ptr(codes, torch.int8), _ptr(grad_scales, torch.float32),
-            float(lr), int(B), int(L), self._ws_ptr, self.workspace_bytes, _stream(stream)))
+        rc = self._n.train_step(self._hv, tables, indices, offsets, grad_out, scales, bits, out, unique_rows, uniq_off,
+                                grad_rows, codes, grad_scales, lr, B, L, self._ws_ptr, self.workspace_bytes, stream)
+        if rc:
+            self._check("dqrm_train_step", rc)
 
     # ---- the step in two calls; `ws` picks a workspace (number 0 exists, the others are made on first use) ----
     def _workspace(self, ws: int) -> int:
@@ -336,22 +346,18 @@ class Context:
         return more[ws][1]
 
     def sort_batch(self, indices, offsets, unique_rows, uniq_off, *, B, L, ws=0, stream=None):
-        import torch
-
-        self._check("dqrm_sort_batch", self.lib.dqrm_sort_batch(
-            self._h, _ptr(indices, torch.int32), _ptr(offsets, torch.int32), _ptr(unique_rows, torch.int32),
-            _ptr(uniq_off, torch.int32), int(B), int(L), self._workspace(ws), self.workspace_bytes, _stream(stream)))
+        rc = self._n.sort_batch(self._hv, indices, offsets, unique_rows, uniq_off, B, L, self._workspace(ws),
+                                self.workspace_bytes, stream)
+        if rc:
+            self._check("dqrm_sort_batch", rc)
 
     def train_step_sorted(self, tables, indices, offsets, grad_out, scales, bits, out, unique_rows, uniq_off,
                           grad_rows, codes, grad_scales, lr, *, B, L, ws=0, stream=None):
-        import torch
-
-        self._check("dqrm_train_step_sorted", self.lib.dqrm_train_step_sorted(
-            self._h, _ptr(tables, torch.float32), _ptr(indices, torch.int32), _ptr(offsets, torch.int32),
-            _ptr(grad_out, torch.float32), _ptr(scales, torch.float32), _ptr(bits, torch.int32),
-            _ptr(out, torch.float32), _ptr(unique_rows, torch.int32), _ptr(uniq_off, torch.int32),
-            _ptr(grad_rows, torch.float32), _ptr(codes, torch.int8), _ptr(grad_scales, torch.float32),
-            float(lr), int(B), int(L), self._workspace(ws), self.workspace_bytes, _stream(stream)))
+        rc = self._n.train_step_sorted(self._hv, tables, indices, offsets, grad_out, scales, bits, out, unique_rows,
+                                       uniq_off, grad_rows, codes, grad_scales, lr, B, L, self._workspace(ws),
+                                       self.workspace_bytes, stream)
+        if rc:
+            self._check("dqrm_train_step_sorted", rc)
 
     def stream_wait_forward(self, stream):
         self._check("dqrm_stream_wait_forward", self.lib.dqrm_stream_wait_forward(self._h, _stream(stream)))
@@ -372,14 +378,11 @@ class Context:
 
     def train_step_host(self, tables, h_indices, h_offsets, h_grad_out, scales, bits, h_out, lr, *, B, L,
                         stream=None):
-        import torch
-
         assert self.host_workspace is not None, "create the Context with host_step=True"
-        self._check("dqrm_train_step_host", self.lib.dqrm_train_step_host(
-            self._h, _ptr(tables, torch.float32), _ptr(h_indices, torch.int32, "cpu"),
-            _ptr(h_offsets, torch.int32, "cpu"), _ptr(h_grad_out, torch.float32, "cpu"),
-            _ptr(scales, torch.float32), _ptr(bits, torch.int32), _ptr(h_out, torch.float32, "cpu"),
-            float(lr), int(B), int(L), self._hws_ptr, self.host_workspace_bytes, _stream(stream)))
+        rc = self._n.train_step_host(self._hv, tables, h_indices, h_offsets, h_grad_out, scales, bits, h_out, lr, B, L,
+                                     self._hws_ptr, self.host_workspace_bytes, stream)
+        if rc:
+            self._check("dqrm_train_step_host", rc)
 
 
 def grad_quant_int8_static(T, D, grad_rows, uniq_off, codes, grad_scales, stream=None) -> int:

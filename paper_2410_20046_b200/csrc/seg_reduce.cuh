@@ -42,7 +42,7 @@ __host__ __device__ constexpr int column_blocks(int D) { return (D + 127) / 128;
 // batches in turn) and three blocks (four blocks: 78 instead of 71 us at 852 K rows of 256 bytes)
 __host__ __device__ constexpr int batch_entries(int lpr, int vec, bool small) { return lpr == 32 ? (small ? 4 : 16 / vec) : 8; }
 // A warp that has one tile takes its batches of rows one after the other, 4 to 8 us for 32 rows, so a batch of wide
-// rows that would not even give every resident warp a tile of 32 entries is cut into tiles of 8
+// rows that would give every resident warp less than three tiles of 32 entries is cut into tiles of 8
 __host__ __device__ constexpr int tile_entries(int lpr, bool small) { return lpr == 4 ? 64 : lpr == 32 && small ? 8 : 32; }
 __host__ __device__ constexpr int chunk_shift(int lpr, bool small) { return lpr == 32 && small ? 3 : 5; }    // of chunk_first
 __host__ __device__ constexpr int blocks_per_sm(int lpr) { return lpr == 32 ? 3 : 2; }
