@@ -98,6 +98,7 @@ __device__ __forceinline__ void load_tile_keys(const u32 *__restrict__ keys, int
 __global__ void __launch_bounds__(ST_THREADS)
 seg_count_kernel(const u32 *__restrict__ keys, int64_t L, u32 *__restrict__ tile_heads)
 {
+    dq_wait_before();
     __shared__ u32 wsum[ST_WARPS];
     const int64_t i0 = (int64_t)blockIdx.x * ST_TILE + (int64_t)threadIdx.x * ST_ITEMS;
     u32 k[ST_ITEMS], prev; int n;
@@ -126,6 +127,7 @@ seg_emit_kernel(const u32 *__restrict__ keys, int64_t L, const u32 *__restrict__
                 int32_t *__restrict__ unique_rows, int32_t *__restrict__ uniq_off, uint2 *__restrict__ tile_done,
                 u32 *__restrict__ absmax, int ck_shift)
 {
+    dq_wait_before();
     extern __shared__ unsigned char smem_raw[];
     int64_t *s_off = reinterpret_cast<int64_t *>(smem_raw);   // [T+1]
     __shared__ u32 wsum[ST_WARPS];
@@ -231,14 +233,13 @@ int launch_sum(dqrm_ctx *ctx, const segred::Args &a, bool small, cudaStream_t st
     const int64_t ranges = (a.num_tiles + a.range_tiles - 1) / a.range_tiles;
     const dim3 grid((unsigned)((ranges + WARPS - 1) / WARPS), (unsigned)column_blocks(ctx->D));
     const bool exact = ctx->D == LPR * VEC;
+#define DQ_SUM(EXACT, SMALL) DQRM_CUDA_TRY(ctx, (dq_launch(seg_sum_kernel<LPR, VEC, EXACT, SMALL>, grid, dim3(THREADS), smem, st, a)))
     if (LPR == 32 && small) {
-        if (exact) seg_sum_kernel<LPR, VEC, true, LPR == 32><<<grid, THREADS, smem, st>>>(a);
-        else seg_sum_kernel<LPR, VEC, false, LPR == 32><<<grid, THREADS, smem, st>>>(a);
+        if (exact) DQ_SUM(true, LPR == 32); else DQ_SUM(false, LPR == 32);
     } else {
-        if (exact) seg_sum_kernel<LPR, VEC, true, false><<<grid, THREADS, smem, st>>>(a);
-        else seg_sum_kernel<LPR, VEC, false, false><<<grid, THREADS, smem, st>>>(a);
+        if (exact) DQ_SUM(true, false); else DQ_SUM(false, false);
     }
-    DQRM_CUDA_TRY(ctx, cudaGetLastError());
+#undef DQ_SUM
     dq_mark(ctx, st, DQ_K_SEG_SUM);
     return DQRM_OK;
 }
@@ -249,20 +250,18 @@ int launch_radix_pass(dqrm_ctx *ctx, const rsort::Args &a, const uint2 *in, uint
 {
     const unsigned tiles = (unsigned)rsort::max_tiles(a.T, a.L);
     const int nb = 1 << a.dbits;
-    rsort::rs_hist_kernel<FIRST><<<tiles, rsort::THREADS, 0, st>>>(a, in, shift);
-    DQRM_CUDA_TRY(ctx, cudaGetLastError());
+    DQRM_CUDA_TRY(ctx, dq_launch(rsort::rs_hist_kernel<FIRST>, dim3(tiles), dim3(rsort::THREADS), 0, st, a, in, shift));
     dq_mark(ctx, st, DQ_K_SORT_HIST);
-    rsort::rs_scan_kernel<<<dim3((unsigned)((nb + rsort::SCAN_DIGITS - 1) / rsort::SCAN_DIGITS), (unsigned)a.T),
-                            rsort::SCAN_DIGITS * rsort::SCAN_GROUPS, 0, st>>>(a);
-    DQRM_CUDA_TRY(ctx, cudaGetLastError());
+    DQRM_CUDA_TRY(ctx, dq_launch(rsort::rs_scan_kernel, dim3((unsigned)((nb + rsort::SCAN_DIGITS - 1) / rsort::SCAN_DIGITS), (unsigned)a.T),
+                                 dim3(rsort::SCAN_DIGITS * rsort::SCAN_GROUPS), 0, st, a));
     dq_mark(ctx, st, DQ_K_SORT_SCAN);
     bool &raised = ctx->smem_raised[(FIRST ? 1 : 0) + (LAST ? 2 : 0)];
     if (!raised)
         DQRM_CUDA_TRY(ctx, cudaFuncSetAttribute(rsort::rs_scatter_kernel<FIRST, LAST>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                 (int)rsort::scatter_smem(1 << rsort::MAX_DIGIT_BITS)));
     raised = true;
-    rsort::rs_scatter_kernel<FIRST, LAST><<<tiles, rsort::THREADS, rsort::scatter_smem(nb), st>>>(a, in, out, keys, vals, shift);
-    DQRM_CUDA_TRY(ctx, cudaGetLastError());
+    DQRM_CUDA_TRY(ctx, (dq_launch(rsort::rs_scatter_kernel<FIRST, LAST>, dim3(tiles), dim3(rsort::THREADS), rsort::scatter_smem(nb),
+                                  st, a, in, out, keys, vals, shift)));
     dq_mark(ctx, st, DQ_K_SORT_SCATTER);
     return DQRM_OK;
 }
@@ -270,8 +269,7 @@ int launch_radix_pass(dqrm_ctx *ctx, const rsort::Args &a, const uint2 *in, uint
 int launch_radix_sort(dqrm_ctx *ctx, const rsort::Args &a, int passes, uint2 *const (&pairs)[2], u32 *keys, u32 *vals,
                       cudaStream_t st)
 {
-    rsort::rs_setup_kernel<<<1, 1024, rsort::setup_smem(a.T), st>>>(a);
-    DQRM_CUDA_TRY(ctx, cudaGetLastError());
+    DQRM_CUDA_TRY(ctx, dq_launch(rsort::rs_setup_kernel, dim3(1), dim3(1024), rsort::setup_smem(a.T), st, a));
     dq_mark(ctx, st, DQ_K_SORT_SETUP);
     for (int p = 0; p < passes; ++p) {
         const uint2 *in = pairs[(p + 1) & 1];          // (the first pass reads the indices)
@@ -306,10 +304,12 @@ cudaError_t launch_cluster_sort(dqrm_ctx *ctx, csort::Args ca, int64_t per_table
         cfg.blockDim = dim3(csort::THREADS);
         cfg.dynamicSmemBytes = csort::smem_bytes(ca.cap);
         cfg.stream = st;
-        cudaLaunchAttribute attr[1];
+        cudaLaunchAttribute attr[2];
         attr[0].id = cudaLaunchAttributeClusterDimension;
         attr[0].val.clusterDim.x = CL; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
-        cfg.attrs = attr; cfg.numAttrs = 1;
+        attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr[1].val.programmaticStreamSerializationAllowed = 1;
+        cfg.attrs = attr; cfg.numAttrs = 2;
         e = cudaLaunchKernelEx(&cfg, csort::cluster_sort_kernel<CL>, ca);
     }
     if (e != cudaSuccess) (void)cudaGetLastError();
@@ -325,8 +325,7 @@ cudaError_t launch_small_sort2(dqrm_ctx *ctx, const csort::Args &ca, cudaStream_
 {
     const size_t smem = ssort::smem_bytes(THREADS, EPT);
     static_assert(THREADS >= csort::BINS && (size_t)THREADS * EPT * 2 * sizeof(ssort::u64) <= 48 * 1024, "");
-    ssort::small_sort_kernel<THREADS, EPT><<<(unsigned)ctx->T, THREADS, smem, st>>>(ca);
-    return cudaGetLastError();
+    return dq_launch(ssort::small_sort_kernel<THREADS, EPT>, dim3((unsigned)ctx->T), dim3(THREADS), smem, st, ca);
 }
 
 bool launch_small_sort(dqrm_ctx *ctx, const csort::Args &ca, int64_t per_table, bool even, cudaStream_t st, cudaError_t &e)
@@ -452,15 +451,14 @@ int dq_launch_bwd_sort(dqrm_ctx *ctx, const int32_t *indices, const int32_t *off
         return DQRM_OK;
     }
     if (!sorted) {        // (a cluster sort that did not number the segments itself has counted the segment heads of every tile)
-        seg_count_kernel<<<(unsigned)y.num_tiles, ST_THREADS, 0, st>>>(skeys, L, reinterpret_cast<u32 *>(ws + y.tile_heads));
-        DQRM_CUDA_TRY(ctx, cudaGetLastError());
+        DQRM_CUDA_TRY(ctx, dq_launch(seg_count_kernel, dim3((unsigned)y.num_tiles), dim3(ST_THREADS), 0, st, skeys, L,
+                                     reinterpret_cast<u32 *>(ws + y.tile_heads)));
         dq_mark(ctx, st, DQ_K_SEG_COUNT);
     }
-    seg_emit_kernel<<<(unsigned)y.num_tiles, ST_THREADS, (size_t)(ctx->T + 1) * sizeof(int64_t), st>>>(
-        skeys, L, reinterpret_cast<const u32 *>(ws + y.tile_heads), ctx->d_row_off, ctx->T,
+    DQRM_CUDA_TRY(ctx, dq_launch(seg_emit_kernel, dim3((unsigned)y.num_tiles), dim3(ST_THREADS),
+        (size_t)(ctx->T + 1) * sizeof(int64_t), st, skeys, L, reinterpret_cast<const u32 *>(ws + y.tile_heads), ctx->d_row_off, ctx->T,
         reinterpret_cast<u32 *>(ws + y.seg_start), reinterpret_cast<u32 *>(ws + y.chunk_first), unique_rows, uniq_off,
-        reinterpret_cast<uint2 *>(ws + y.tile_done), reinterpret_cast<u32 *>(ws + y.absmax), y.sum_shift);
-    DQRM_CUDA_TRY(ctx, cudaGetLastError());
+        reinterpret_cast<uint2 *>(ws + y.tile_done), reinterpret_cast<u32 *>(ws + y.absmax), y.sum_shift));
     dq_mark(ctx, st, DQ_K_SEG_EMIT);
     return DQRM_OK;
 }

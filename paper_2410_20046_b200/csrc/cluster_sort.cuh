@@ -77,6 +77,7 @@ template <int CL>
 __global__ void __launch_bounds__(THREADS)
 cluster_sort_kernel(const Args a)
 {
+    dq_wait_before();
     extern __shared__ uint2 s_dyn[];               // pair buffers [2][cap]: (row within table, payload)
     __shared__ u32 s_cnt[WARPS][BINS];
     __shared__ u32 s_hist[BINS];

@@ -64,7 +64,7 @@ struct dqrm_ctx {
 
 enum {
     DQ_K_BEGIN = 0, DQ_K_REFRESH, DQ_K_FWD, DQ_K_MEMSET, DQ_K_SORT_SETUP, DQ_K_SORT_HIST, DQ_K_SORT_SCAN, DQ_K_SORT_SCATTER,
-    DQ_K_SEG_COUNT, DQ_K_SEG_EMIT, DQ_K_SEG_SUM, DQ_K_ABSMAX, DQ_K_QUANT, DQ_K_UPDATE,
+    DQ_K_SEG_COUNT, DQ_K_SEG_EMIT, DQ_K_SEG_SUM, DQ_K_ZERO, DQ_K_ABSMAX, DQ_K_QUANT, DQ_K_UPDATE,
     DQ_K_QUANT_UPDATE, DQ_K_COPY, DQ_K_SMALL_SORT, DQ_K_CLUSTER_SORT, DQ_K_DP_PACK, DQ_K_DP_SUM_UPDATE, DQ_K_PACK, DQ_K_PACKED_FWD, DQ_K_FWD_CODES, DQ_K_DECODE_PAYLOAD, DQ_K_COUNT
 };
 constexpr int DQ_PROF_MAX = 4096;
@@ -89,6 +89,31 @@ static inline void dq_mark(dqrm_ctx *ctx, cudaStream_t st, int kernel_id)
             return DQRM_ERR_CUDA;                                  \
         }                                                          \
     } while (0)
+
+// Kernel launch with programmatic stream serialisation: the grid may be set up while the kernel before it on the stream
+// is still finishing, and waits for it (all of it, memory included) in dq_wait_before, which every kernel launched this
+// way calls before it touches memory.  The kernel before does not announce its end early: with that the waiting blocks
+// take room from it (measured, calls of 53 K lookups: 61.4 us plain, 48.5 this way, 53.3 with an early announcement; of
+// 3328 lookups 40.2, 29.7 and 30.5).
+template <typename... P, typename... A>
+static inline cudaError_t dq_launch(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A... args)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, P(args)...);
+}
+__device__ __forceinline__ void dq_wait_before()
+{
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+}
 
 static inline size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 

@@ -107,6 +107,7 @@ template <int LPR, int CH, bool EXACT>
 __global__ void __launch_bounds__(FW_THREADS, 5)
 fwd_onehot_kernel(const FwdArgs a)
 {
+    dq_wait_before();
     constexpr int NB = NBOf<LPR, CH>::v;      // row steps in flight
     constexpr int RPW = 32 / LPR;             // rows one warp instruction covers
     constexpr int WPB = FW_THREADS / 32;
@@ -231,6 +232,7 @@ template <int LPR, int VEC, int CH, bool EXACT, bool CODES>
 __global__ void __launch_bounds__(FW_THREADS)
 fwd_bags_kernel(const FwdArgs a)
 {
+    dq_wait_before();
     typedef typename Vec<VEC>::type vec_t;
     constexpr int NB = CH >= 2 ? 1 : LPR < 4 ? LPR : 4;
     constexpr int GPB = FW_THREADS / LPR;
@@ -306,16 +308,13 @@ fwd_bags_kernel(const FwdArgs a)
 inline bool warp_per_bag(const FwdArgs &a, int lpr) { return lpr == 16 && !a.codes_out && a.L >= 8 * (int64_t)a.T * a.B; }
 
 template <int LPR, int CH, bool EXACT>
-void launch_bags(const FwdArgs &a, dim3 grid, cudaStream_t st)
+cudaError_t launch_bags(const FwdArgs &a, dim3 grid, cudaStream_t st)
 {
     if constexpr (LPR == 16) {
-        if (warp_per_bag(a, LPR)) {
-            fwd_bags_kernel<32, 2, CH, EXACT, false><<<grid, FW_THREADS, 0, st>>>(a);
-            return;
-        }
+        if (warp_per_bag(a, LPR)) return dq_launch(fwd_bags_kernel<32, 2, CH, EXACT, false>, grid, dim3(FW_THREADS), 0, st, a);
     }
-    if (a.codes_out) fwd_bags_kernel<LPR, 4, CH, EXACT, true><<<grid, FW_THREADS, 0, st>>>(a);
-    else fwd_bags_kernel<LPR, 4, CH, EXACT, false><<<grid, FW_THREADS, 0, st>>>(a);
+    if (a.codes_out) return dq_launch(fwd_bags_kernel<LPR, 4, CH, EXACT, true>, grid, dim3(FW_THREADS), 0, st, a);
+    return dq_launch(fwd_bags_kernel<LPR, 4, CH, EXACT, false>, grid, dim3(FW_THREADS), 0, st, a);
 }
 
 template <int LPR, int CH, bool EXACT>
@@ -330,9 +329,8 @@ int launch2(dqrm_ctx *ctx, const FwdArgs &a, cudaStream_t st)
     if (bx > cap) bx = cap;
     if (bx < 1) bx = 1;
     dim3 grid((unsigned)bx, (unsigned)ctx->T);
-    if (onehot) fwd_onehot_kernel<LPR, CH, EXACT><<<grid, FW_THREADS, 0, st>>>(a);
-    else launch_bags<LPR, CH, EXACT>(a, grid, st);
-    DQRM_CUDA_TRY(ctx, cudaGetLastError());
+    DQRM_CUDA_TRY(ctx, (onehot ? dq_launch(fwd_onehot_kernel<LPR, CH, EXACT>, grid, dim3(FW_THREADS), 0, st, a)
+                               : launch_bags<LPR, CH, EXACT>(a, grid, st)));
     dq_mark(ctx, st, DQ_K_FWD);
     return DQRM_OK;
 }

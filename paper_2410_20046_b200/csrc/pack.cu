@@ -39,6 +39,7 @@ __global__ void __launch_bounds__(PK_THREADS)
 pack_kernel(const float4 *__restrict__ arena4, const int64_t *__restrict__ row_off, int T, int D, int64_t n4,
             const float *__restrict__ scales, uint8_t *__restrict__ packed)
 {
+    dq_wait_before();
     extern __shared__ unsigned char smem_raw[];
     int64_t *v4_off = reinterpret_cast<int64_t *>(smem_raw);       // table starts in 128-bit vectors
     const int d4 = D >> 2;
@@ -187,6 +188,7 @@ template <int BITS, int EPL, int LPR, int CH>
 __global__ void __launch_bounds__(PK_THREADS)
 packed_fwd_kernel(const PfArgs a)
 {
+    dq_wait_before();
     constexpr int GPB = PK_THREADS / LPR;
     const int units = a.D / EPL;
     const int t = blockIdx.y;
@@ -210,6 +212,7 @@ template <int BITS, int EPL, int LPR, int CH>
 __global__ void __launch_bounds__(PK_THREADS)
 packed_fwd_onehot_kernel(const PfArgs a)
 {
+    dq_wait_before();
     constexpr int NB = CH >= 2 ? 1 : 4;
     constexpr int RPW = 32 / LPR;
     constexpr int WPB = PK_THREADS / 32;
@@ -310,9 +313,8 @@ int launch_pack(dqrm_ctx *ctx, const float *tables, const float *scales, uint8_t
 {
     const int64_t n4 = ctx->total_rows * (ctx->D / 4);
     const size_t smem = (size_t)(ctx->T + 1) * sizeof(int64_t);
-    pack_kernel<BITS><<<ctx->num_sms * 8, PK_THREADS, smem, st>>>(reinterpret_cast<const float4 *>(tables), ctx->d_row_off,
-                                                                  ctx->T, ctx->D, n4, scales, packed);
-    DQRM_CUDA_TRY(ctx, cudaGetLastError());
+    DQRM_CUDA_TRY(ctx, dq_launch(pack_kernel<BITS>, dim3(ctx->num_sms * 8), dim3(PK_THREADS), smem, st,
+                                 reinterpret_cast<const float4 *>(tables), ctx->d_row_off, ctx->T, ctx->D, n4, scales, packed));
     dq_mark(ctx, st, DQ_K_PACK);
     return DQRM_OK;
 }
@@ -328,9 +330,8 @@ int launch_pfwd(dqrm_ctx *ctx, const PfArgs &a, cudaStream_t st)
     if (bx > cap) bx = cap;
     if (bx < 1) bx = 1;
     dim3 grid((unsigned)bx, (unsigned)ctx->T);
-    if (onehot) packed_fwd_onehot_kernel<BITS, EPL, LPR, CH><<<grid, PK_THREADS, 0, st>>>(a);
-    else packed_fwd_kernel<BITS, EPL, LPR, CH><<<grid, PK_THREADS, 0, st>>>(a);
-    DQRM_CUDA_TRY(ctx, cudaGetLastError());
+    DQRM_CUDA_TRY(ctx, (onehot ? dq_launch(packed_fwd_onehot_kernel<BITS, EPL, LPR, CH>, grid, dim3(PK_THREADS), 0, st, a)
+                               : dq_launch(packed_fwd_kernel<BITS, EPL, LPR, CH>, grid, dim3(PK_THREADS), 0, st, a)));
     dq_mark(ctx, st, DQ_K_PACKED_FWD);
     return DQRM_OK;
 }

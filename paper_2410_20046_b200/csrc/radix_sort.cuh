@@ -44,6 +44,7 @@ inline size_t scatter_smem(int nb) { return (size_t)TILE * sizeof(uint2) + (size
 __global__ void __launch_bounds__(1024)
 rs_setup_kernel(const Args a)
 {
+    dq_wait_before();
     extern __shared__ u32 s_tb[];                      // [T+1]
     u32 *s_t0 = s_tb + (a.T + 1);                      // [T+1]
     const int lane = threadIdx.x & 31;
@@ -120,6 +121,7 @@ template <bool FIRST>
 __global__ void __launch_bounds__(THREADS)
 rs_hist_kernel(const Args a, const uint2 *__restrict__ pairs, int shift)
 {
+    dq_wait_before();
     __shared__ u32 cnt[1 << MAX_DIGIT_BITS];
     Tile x;
     if (!tile_of(a, x)) return;
@@ -153,6 +155,7 @@ rs_hist_kernel(const Args a, const uint2 *__restrict__ pairs, int shift)
 __global__ void __launch_bounds__(SCAN_DIGITS * SCAN_GROUPS)
 rs_scan_kernel(const Args a)
 {
+    dq_wait_before();
     __shared__ u32 part[SCAN_GROUPS][SCAN_DIGITS];
     const int nb = 1 << a.dbits;
     const int dl = threadIdx.x % SCAN_DIGITS, g = threadIdx.x / SCAN_DIGITS, d = blockIdx.x * SCAN_DIGITS + dl;
@@ -212,6 +215,7 @@ __global__ void __launch_bounds__(THREADS, 3)
 rs_scatter_kernel(const Args a, const uint2 *__restrict__ pairs_in, uint2 *__restrict__ pairs_out,
                   u32 *__restrict__ keys_out, u32 *__restrict__ vals_out, int shift)
 {
+    dq_wait_before();
     extern __shared__ uint2 s_pair[];                  // [TILE]
     const int nb = 1 << a.dbits;
     u32 *s_delta = reinterpret_cast<u32 *>(s_pair + TILE);                               // [nb]

@@ -44,6 +44,7 @@ refresh_kernel(const V *__restrict__ arena4, const int64_t *__restrict__ row_off
                float *__restrict__ minmax, u32 *__restrict__ partials /*[grid][T][2]*/,
                u32 *__restrict__ done)
 {
+    dq_wait_before();
     extern __shared__ unsigned char smem_raw[];
     int64_t *v4_off = reinterpret_cast<int64_t *>(smem_raw);             // [T+1] table starts in float4 units
     u32 *s_min = reinterpret_cast<u32 *>(v4_off + (T + 1));              // [T]
@@ -154,16 +155,14 @@ int dq_launch_refresh(dqrm_ctx *ctx, const float *tables, const int32_t *bits, f
     size_t smem = (size_t)(ctx->T + 1) * sizeof(int64_t) + (size_t)ctx->T * 2 * sizeof(u32);
     if (ctx->row_summary) {
         // every row's (min, max) is kept current by the update kernels: 8 bytes per row are read, not 4*D
-        refresh_kernel<float2><<<grid, RF_THREADS, smem, st>>>(ctx->row_summary, ctx->d_row_off, ctx->T, 1,
-                                                               ctx->total_rows, bits, scales, minmax,
-                                                               reinterpret_cast<u32 *>(ws), ctx->d_done);
+        DQRM_CUDA_TRY(ctx, dq_launch(refresh_kernel<float2>, dim3(grid), dim3(RF_THREADS), smem, st, ctx->row_summary, ctx->d_row_off,
+                                     ctx->T, 1, ctx->total_rows, bits, scales, minmax, reinterpret_cast<u32 *>(ws), ctx->d_done));
     } else {
         const int64_t n4 = ctx->total_rows * (ctx->D / 4);
-        refresh_kernel<float4><<<grid, RF_THREADS, smem, st>>>(reinterpret_cast<const float4 *>(tables), ctx->d_row_off,
-                                                               ctx->T, ctx->D / 4, n4, bits, scales, minmax,
-                                                               reinterpret_cast<u32 *>(ws), ctx->d_done);
+        DQRM_CUDA_TRY(ctx, dq_launch(refresh_kernel<float4>, dim3(grid), dim3(RF_THREADS), smem, st,
+                                     reinterpret_cast<const float4 *>(tables), ctx->d_row_off, ctx->T, ctx->D / 4, n4, bits,
+                                     scales, minmax, reinterpret_cast<u32 *>(ws), ctx->d_done));
     }
-    DQRM_CUDA_TRY(ctx, cudaGetLastError());
     dq_mark(ctx, st, DQ_K_REFRESH);
     return DQRM_OK;
 }

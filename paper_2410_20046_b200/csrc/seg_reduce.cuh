@@ -152,6 +152,7 @@ template <int LPR, int VEC, bool EXACT, bool SMALL>
 __global__ void __launch_bounds__(THREADS, blocks_per_sm(LPR))
 seg_sum_kernel(const Args a)
 {
+    dq_wait_before();
     constexpr int C = batch_entries(LPR, VEC, SMALL);    // rows of a lane group in flight
     constexpr int GP = 32 / LPR;                  // lane groups of the warp
     constexpr int I = tile_entries(LPR, SMALL);

@@ -122,6 +122,7 @@ template <int THREADS, int EPT>
 __global__ void __launch_bounds__(THREADS)
 small_sort_kernel(const csort::Args a)
 {
+    dq_wait_before();
     constexpr int WARPS = THREADS / 32, N = THREADS * EPT;
     extern __shared__ u64 s_net[];                 // [2][N]
     __shared__ u32 s_warp[WARPS];
