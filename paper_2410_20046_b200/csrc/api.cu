@@ -308,7 +308,10 @@ int dqrm_train_step(dqrm_ctx *ctx, float *tables, const int32_t *indices, const 
     // tables nor the forward's output, so it runs on the context's second stream while the forward runs on
     // the caller's (per-launch profiling keeps one stream, because its events time consecutive launches).
     // The quantise-and-update kernel writes the rows the forward reads, so it waits for both.
-    const bool overlap = ctx->overlap && !ctx->prof_on && L > 0;
+    // Below 16 MB of gathered rows the fork and the join cost more than the overlap gives, and the step is one chain of
+    // launches on the caller's stream (measured on B200, two streams / one: 512 lookups of 64-byte rows 20.5 / 18.5 us,
+    // 53 K of 64 bytes 34.8 / 32.6, 213 K of 64 bytes 46.6 / 43.9, 64 K of 512 bytes 87.4 / 89.8).
+    const bool overlap = ctx->overlap && !ctx->prof_on && L * ctx->D * (int64_t)sizeof(float) >= ((int64_t)16 << 20);
     cudaStream_t ss = overlap ? ctx->side : st;
     if (overlap) {
         DQRM_CUDA_TRY(ctx, cudaEventRecord(ctx->ev_fork, st));
