@@ -46,6 +46,20 @@ HostStepLayout host_layout(const dqrm_ctx *ctx, int64_t L, int64_t G)
     return y;
 }
 
+// The staging buffers of one call are filled while the call before it still runs, so their places must not move with the
+// number of lookups: they are laid out for the most lookups that `workspace_bytes` has room for (at least L where the
+// workspace is large enough for the call).
+int64_t host_lookups_for(const dqrm_ctx *ctx, size_t workspace_bytes, int64_t L, int64_t G)
+{
+    int64_t lo = L, hi = (int64_t)(workspace_bytes / sizeof(int32_t));      // the indices alone bound it
+    if (hi > ((int64_t)1 << 31) - 1) hi = ((int64_t)1 << 31) - 1;
+    while (lo < hi) {
+        const int64_t mid = lo + (hi - lo + 1) / 2;
+        if (host_layout(ctx, mid, G).total <= workspace_bytes) lo = mid; else hi = mid - 1;
+    }
+    return lo;
+}
+
 }  // namespace
 
 extern "C" {
@@ -547,8 +561,13 @@ int dqrm_train_step_host(dqrm_ctx *ctx, float *tables, const int32_t *h_indices,
         return DQRM_ERR_INVALID_ARG;
     if (L > 0 && !h_indices) return DQRM_ERR_INVALID_ARG;
     const int64_t G = (int64_t)ctx->T * B;
-    const HostStepLayout y = host_layout(ctx, L, G);
-    if (!ws_ok(workspace, workspace_bytes, y.total)) return DQRM_ERR_WORKSPACE;
+    if (!ws_ok(workspace, workspace_bytes, host_layout(ctx, L, G).total)) return DQRM_ERR_WORKSPACE;
+    // the places follow from (workspace, its size, bags): worked out again only when one of them is another
+    const dqrm_ctx::HostPlace place{workspace, workspace_bytes, G};
+    const bool moved = !(place == ctx->h_place);
+    if (moved) ctx->h_lookups = host_lookups_for(ctx, workspace_bytes, L, G);
+    ctx->h_place = place;
+    const HostStepLayout y = host_layout(ctx, ctx->h_lookups, G);
     char *ws = reinterpret_cast<char *>(workspace);
     cudaStream_t st = as_stream(stream);
     const bool plain = !ctx->overlap || ctx->prof_on || L == 0;        // everything in order on the caller's stream
@@ -564,6 +583,7 @@ int dqrm_train_step_host(dqrm_ctx *ctx, float *tables, const int32_t *h_indices,
     float *d_gs = reinterpret_cast<float *>(ws + y.grad_scales);
     const size_t go_bytes = sizeof(float) * G * ctx->D;
     if (plain) {
+        ctx->h_place = {nullptr, 0, 0};     // the next call's copies come behind this one, which records no event of its own
         if (L > 0) DQRM_CUDA_TRY(ctx, cudaMemcpyAsync(d_idx, h_indices, sizeof(int32_t) * L, cudaMemcpyHostToDevice, st));
         DQRM_CUDA_TRY(ctx, cudaMemcpyAsync(d_off, h_offsets, sizeof(int32_t) * (G + 1), cudaMemcpyHostToDevice, st));
         DQRM_CUDA_TRY(ctx, cudaMemcpyAsync(d_go, h_grad_out, go_bytes, cudaMemcpyHostToDevice, st));
@@ -579,8 +599,10 @@ int dqrm_train_step_host(dqrm_ctx *ctx, float *tables, const int32_t *h_indices,
     // sort and the forward.  The inputs of this call land in the staging set that the call before the last one used,
     // as soon as that call is over: they do not wait for the previous call, whose kernels and output copy they
     // overlap.  The caller's stream waits for everything before the call's work on it is complete.
-    if (ctx->h_set_used[set]) DQRM_CUDA_TRY(ctx, cudaStreamWaitEvent(ctx->copy_in, ctx->ev_h_free[set], 0));
-    else {      // first use of this set: only what the caller's stream already holds comes first
+    if (ctx->h_set_used[set] && !moved) DQRM_CUDA_TRY(ctx, cudaStreamWaitEvent(ctx->copy_in, ctx->ev_h_free[set], 0));
+    else {      // first use of this set in this place: what the caller's stream already holds and the calls before it come first
+        for (int k = 0; k < 2; ++k)
+            if (ctx->h_set_used[k]) DQRM_CUDA_TRY(ctx, cudaStreamWaitEvent(ctx->copy_in, ctx->ev_h_free[k], 0));
         DQRM_CUDA_TRY(ctx, cudaEventRecord(ctx->ev_h_start, st));
         DQRM_CUDA_TRY(ctx, cudaStreamWaitEvent(ctx->copy_in, ctx->ev_h_start, 0));
     }

@@ -35,6 +35,13 @@ struct dqrm_ctx {
     cudaEvent_t ev_h_free[2] = {nullptr, nullptr}, ev_h_idx = nullptr;
     bool h_set_used[2] = {false, false};
     unsigned host_calls = 0;
+    struct HostPlace {              // what the places of the staging buffers follow from
+        const void *ws;
+        size_t bytes;
+        int64_t G;
+        bool operator==(const HostPlace &o) const { return ws == o.ws && bytes == o.bytes && G == o.G; }
+    } h_place = {nullptr, 0, 0};
+    int64_t h_lookups = 0;          // lookups that they have room for there
     float2 *row_summary = nullptr;  // [total_rows] (min, max) of every row, caller's memory; null: not kept
     // what the context knows, on the host, about each workspace dqrm_sort_batch has written: whether it holds a
     // sorted batch that no step has taken yet, of which size, and the event recorded behind that sort (with the
