@@ -163,6 +163,13 @@ int dqrm_grad_quant_int8(dqrm_ctx *ctx, const float *grad_rows, const int32_t *u
                          int8_t *codes, float *grad_scales,
                          void *workspace, size_t workspace_bytes, void *stream);
 
+/* The same for a caller that knows on the host how many values (U*D) there can be, for
+ * instance the size of its buffers: few values are quantised in one launch instead of three.
+ * max_values only chooses the kernel; the result does not depend on it. */
+int dqrm_grad_quant_int8_bounded(dqrm_ctx *ctx, const float *grad_rows, const int32_t *uniq_off,
+                                 int8_t *codes, float *grad_scales, int64_t max_values,
+                                 void *workspace, size_t workspace_bytes, void *stream);
+
 /* Touched-row SGD update (Appendix B.1, Section 3.1): for every unique row u of table t,
  *   g = (float)codes[u][d] * grad_scales[t];  step = lr * g;  W[row][d] = W[row][d] - step
  * (three separately rounded FP32 operations).  Rows not listed are not read or written.

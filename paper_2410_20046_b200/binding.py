@@ -37,6 +37,7 @@ SIGNATURES = {
     "dqrm_emb_fwd": (_i, [_vp, _vp, _vp, _vp, _vp, _vp, _vp, _vp, _i, _i64, _vp]),
     "dqrm_emb_bwd": (_i, [_vp, _vp, _vp, _vp, _vp, _vp, _vp, _i, _i64, _vp, _sz, _vp]),
     "dqrm_grad_quant_int8": (_i, [_vp, _vp, _vp, _vp, _vp, _vp, _sz, _vp]),
+    "dqrm_grad_quant_int8_bounded": (_i, [_vp, _vp, _vp, _vp, _vp, _i64, _vp, _sz, _vp]),
     "dqrm_row_update": (_i, [_vp, _vp, _vp, _vp, _vp, _vp, _f, _vp]),
     "dqrm_sort_batch": (_i, [_vp, _vp, _vp, _vp, _vp, _i, _i64, _vp, _sz, _vp]),
     "dqrm_train_step_sorted": (_i, [_vp, _vp, _vp, _vp, _vp, _vp, _vp, _vp, _vp, _vp, _vp, _vp, _vp, _f, _i, _i64,
@@ -70,8 +71,8 @@ SIGNATURES = {
 }
 
 # functions that the native module calls, in the order in which it wants their addresses
-NATIVE = ("dqrm_scale_refresh", "dqrm_emb_fwd", "dqrm_emb_bwd", "dqrm_grad_quant_int8", "dqrm_row_update",
-          "dqrm_train_step", "dqrm_sort_batch", "dqrm_train_step_sorted", "dqrm_train_step_host", "dqrm_pack_tables",
+NATIVE = ("dqrm_scale_refresh", "dqrm_emb_fwd", "dqrm_emb_bwd", "dqrm_grad_quant_int8_bounded",
+          "dqrm_row_update", "dqrm_train_step", "dqrm_sort_batch", "dqrm_train_step_sorted", "dqrm_train_step_host", "dqrm_pack_tables",
           "dqrm_packed_fwd")
 
 _lib = None

@@ -290,13 +290,20 @@ int dqrm_emb_bwd(dqrm_ctx *ctx, const float *grad_out, const int32_t *indices, c
                          workspace_bytes, as_stream(stream));
 }
 
+int dqrm_grad_quant_int8_bounded(dqrm_ctx *ctx, const float *grad_rows, const int32_t *uniq_off, int8_t *codes,
+                         float *grad_scales, int64_t max_values, void *workspace, size_t workspace_bytes, void *stream)
+{
+    if (!ctx || !grad_rows || !uniq_off || !codes || !grad_scales || max_values < 0) return DQRM_ERR_INVALID_ARG;
+    if (!ws_ok(workspace, workspace_bytes, dq_quant_ws_bytes(ctx))) return DQRM_ERR_WORKSPACE;
+    return dq_launch_grad_quant(ctx, grad_rows, uniq_off, codes, grad_scales, max_values, workspace, workspace_bytes,
+                                as_stream(stream));
+}
+
 int dqrm_grad_quant_int8(dqrm_ctx *ctx, const float *grad_rows, const int32_t *uniq_off, int8_t *codes,
                          float *grad_scales, void *workspace, size_t workspace_bytes, void *stream)
 {
-    if (!ctx || !grad_rows || !uniq_off || !codes || !grad_scales) return DQRM_ERR_INVALID_ARG;
-    if (!ws_ok(workspace, workspace_bytes, dq_quant_ws_bytes(ctx))) return DQRM_ERR_WORKSPACE;
-    return dq_launch_grad_quant(ctx, grad_rows, uniq_off, codes, grad_scales, workspace, workspace_bytes,
-                                as_stream(stream));
+    return dqrm_grad_quant_int8_bounded(ctx, grad_rows, uniq_off, codes, grad_scales, INT64_MAX, workspace, workspace_bytes,
+                                        stream);
 }
 
 int dqrm_row_update(dqrm_ctx *ctx, float *tables, const int32_t *unique_rows, const int32_t *uniq_off,

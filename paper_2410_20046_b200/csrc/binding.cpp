@@ -5,6 +5,7 @@
 #define PY_SSIZE_T_CLEAN
 #include <Python.h>
 #include <c10/cuda/CUDAStream.h>
+#include <algorithm>
 #include <torch/csrc/autograd/python_variable.h>
 #include "dqrm.h"
 
@@ -15,7 +16,7 @@ struct Abi {
     decltype(&dqrm_scale_refresh) scale_refresh;
     decltype(&dqrm_emb_fwd) emb_fwd;
     decltype(&dqrm_emb_bwd) emb_bwd;
-    decltype(&dqrm_grad_quant_int8) grad_quant_int8;
+    decltype(&dqrm_grad_quant_int8_bounded) grad_quant_int8;
     decltype(&dqrm_row_update) row_update;
     decltype(&dqrm_train_step) train_step;
     decltype(&dqrm_sort_batch) sort_batch;
@@ -41,6 +42,7 @@ struct Reader {
     PyObject *const *args;
     Py_ssize_t n, at = 0;
     bool ok;
+    int64_t numel = 0;                                  // of the tensor read last
 
     Reader(PyObject *const *a, Py_ssize_t count, Py_ssize_t want) : args(a), n(count), ok(count == want)
     {
@@ -65,6 +67,7 @@ struct Reader {
             return nullptr;
         }
         if (t.is_cuda() != device) { fail(device ? "expected a CUDA tensor" : "expected a host tensor"); return nullptr; }
+        numel = t.numel();
         return t.data_ptr();
     }
     float *f32() { return static_cast<float *>(pointer(at::kFloat)); }
@@ -148,9 +151,9 @@ DQ_CALL(emb_bwd, 12,
     DQ_RETURN(abi.emb_bwd(ctx, go, idx, off, ur, uo, gr, B, L, ws, bytes, st));)
 
 DQ_CALL(grad_quant_int8, 8,
-    float *gr = r.f32(); int32_t *uo = r.i32(); int8_t *codes = r.i8(); float *gs = r.f32(); void *ws = r.address();
-    size_t bytes = (size_t)r.integer(); void *st = r.stream();
-    DQ_RETURN(abi.grad_quant_int8(ctx, gr, uo, codes, gs, ws, bytes, st));)
+    float *gr = r.f32(); int64_t room = r.numel; int32_t *uo = r.i32(); int8_t *codes = r.i8(); room = std::min(room, r.numel);
+    float *gs = r.f32(); void *ws = r.address(); size_t bytes = (size_t)r.integer(); void *st = r.stream();
+    DQ_RETURN(abi.grad_quant_int8(ctx, gr, uo, codes, gs, room, ws, bytes, st));)
 
 DQ_CALL(row_update, 8,
     float *tables = r.f32(); int32_t *ur = r.i32(); int32_t *uo = r.i32(); int8_t *codes = r.i8(); float *gs = r.f32();

@@ -360,7 +360,7 @@ int dq_launch_dp_merge_update(dqrm_ctx *ctx, float *tables, int W, int64_t rank_
                               int64_t n_entries, int64_t max_table_entries, int32_t *union_rows, int32_t *union_off,
                               int32_t *sums_out, void *ws, size_t ws_bytes, cudaStream_t st);
 int dq_launch_grad_quant(dqrm_ctx *ctx, const float *grad_rows, const int32_t *uniq_off, int8_t *codes,
-                         float *grad_scales, void *ws, size_t ws_bytes, cudaStream_t st);
+                         float *grad_scales, int64_t max_values, void *ws, size_t ws_bytes, cudaStream_t st);
 int dq_launch_row_update(dqrm_ctx *ctx, float *tables, const int32_t *unique_rows, const int32_t *uniq_off,
                          const int8_t *codes, const float *grad_scales, float lr, cudaStream_t st);
 int dq_launch_row_summary(dqrm_ctx *ctx, const float *tables, float2 *summary, cudaStream_t st);

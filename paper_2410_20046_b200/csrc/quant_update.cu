@@ -8,6 +8,7 @@
 // A group of LPR lanes owns a contiguous range of unique rows and keeps a few of them in flight;
 // rows are distinct, so the read-modify-write of the master rows needs no atomics.  All
 // streams are 128-bit per lane.
+#include <cooperative_groups.h>
 #include <mutex>
 #include "common.cuh"
 #include "row_stream.cuh"
@@ -79,6 +80,104 @@ int launch_absmax(dqrm_ctx *ctx, const float *grad_rows, const int32_t *uniq_off
     return DQRM_OK;
 }
 
+// Quantiser in one launch: a cluster of up to eight blocks takes a table, finds its abs-max (over shared memory of the
+// cluster) and quantises what it still holds in registers; what does not fit in them is read again.  Three launches that
+// clear the maxima, find them and quantise are bound by the launches' own latency until the values fill the memory system.
+// Measured on B200 (us, graph replay; one launch / three), 26 tables: 8 K values a table 3.2 / 6.5, 64 K 4.4 / 9.4,
+// 128 K 5.9 / 13.8, 512 K 19 / 33; one table: 8 K 2.7 / 5.2, 128 K 4.1 / 5.8, 256 K 8.0 / 6.0 (eight blocks are too few
+// for what they do not hold).  So it takes batches that the clusters hold, and up to four times that where the
+// clusters of all tables fill the chip.  256 threads a block while that holds a table, 512 then: 40 tables of 64 K values
+// take 5.2 us with 256 and 8.4 with 512 (a second wave).
+constexpr int QC_VEC = 8;             // vectors of four that a thread holds
+constexpr int QC_CLUSTER = 8;
+
+template <int QC_THREADS>
+__global__ void __launch_bounds__(QC_THREADS, 1024 / QC_THREADS)
+quant_table_kernel(const float4 *__restrict__ grad_rows, const int32_t *__restrict__ uniq_off, int d4,
+                   char4 *__restrict__ codes, float *__restrict__ grad_scales)
+{
+    namespace cg = cooperative_groups;
+    cg::cluster_group cluster = cg::this_cluster();
+    __shared__ float s_warp[QC_THREADS / 32], s_block[QC_CLUSTER];
+    const int rank = (int)cluster.block_rank(), blocks = (int)cluster.num_blocks(), t = (int)blockIdx.x / blocks;
+    auto started = cluster.barrier_arrive();           // (shared memory of a block that has not begun is out of reach)
+    dq_wait_before();
+    const int64_t first = __ldg(uniq_off + t), rows = max((int64_t)__ldg(uniq_off + t + 1) - first, (int64_t)0);
+    const int64_t n = rows * d4, stride = (int64_t)blocks * QC_THREADS;
+    const float4 *g = grad_rows + first * d4;
+    char4 *c = codes + first * d4;
+    const int64_t i0 = (int64_t)rank * QC_THREADS + threadIdx.x;
+    float4 x[QC_VEC];
+    float m = 0.f;
+#pragma unroll
+    for (int k = 0; k < QC_VEC; ++k) {
+        x[k] = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (i0 + k * stride < n) x[k] = __ldg(g + i0 + k * stride);
+    }
+#pragma unroll
+    for (int k = 0; k < QC_VEC; ++k)
+        m = fmaxf(m, fmaxf(fmaxf(fabsf(x[k].x), fabsf(x[k].y)), fmaxf(fabsf(x[k].z), fabsf(x[k].w))));
+    for (int64_t i = i0 + QC_VEC * stride; i < n; i += stride) {
+        const float4 y = __ldg(g + i);
+        m = fmaxf(m, fmaxf(fmaxf(fabsf(y.x), fabsf(y.y)), fmaxf(fabsf(y.z), fabsf(y.w))));
+    }
+    const u32 wm = __reduce_max_sync(0xffffffffu, __float_as_uint(m));      // (non-negative floats order as their bits)
+    if (threadIdx.x % 32 == 0) s_warp[threadIdx.x / 32] = __uint_as_float(wm);
+    __syncthreads();
+    cluster.barrier_wait(std::move(started));
+    if (threadIdx.x < (unsigned)blocks) {
+        float b = 0.f;
+#pragma unroll
+        for (int w = 0; w < QC_THREADS / 32; ++w) b = fmaxf(b, s_warp[w]);
+        cluster.map_shared_rank(s_block, threadIdx.x)[rank] = b;
+    }
+    cluster.sync();
+    m = 0.f;
+    for (int b = 0; b < blocks; ++b) m = fmaxf(m, s_block[b]);
+    const float s = dq_scale_from_absmax(m, 8);
+    if (rank == 0 && threadIdx.x == 0) grad_scales[t] = s;
+    const QuantScale qs = dq_make_scale(s, 8);
+    auto put = [&](int64_t i, const float4 &v) {
+        float4 q, unused;
+        dq_fq4(v, qs, q, unused);
+        __stcs(c + i, make_char4((signed char)(int)q.x, (signed char)(int)q.y, (signed char)(int)q.z, (signed char)(int)q.w));
+    };
+#pragma unroll
+    for (int k = 0; k < QC_VEC; ++k)
+        if (i0 + k * stride < n) put(i0 + k * stride, x[k]);
+    for (int64_t i = i0 + QC_VEC * stride; i < n; i += stride) put(i, __ldg(g + i));
+}
+
+// whether a batch of up to max_vectors goes through the kernel above
+inline bool quant_by_table(const dqrm_ctx *ctx, int64_t max_vectors)
+{
+    const int64_t held = (int64_t)ctx->T * QC_CLUSTER * 512 * QC_VEC;
+    return max_vectors <= ((int64_t)ctx->T * QC_CLUSTER >= ctx->num_sms ? 4 * held : held);
+}
+
+template <int QC_THREADS>
+int launch_quant_table(dqrm_ctx *ctx, const float *grad_rows, const int32_t *uniq_off, int8_t *codes, float *grad_scales,
+                       int64_t per_table, cudaStream_t st)
+{
+    unsigned blocks = 1;
+    while (blocks < (unsigned)QC_CLUSTER && per_table > (int64_t)blocks * QC_THREADS * 2) blocks *= 2;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)ctx->T * blocks);
+    cfg.blockDim = dim3(QC_THREADS);
+    cfg.stream = st;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = blocks; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 2;
+    DQRM_CUDA_TRY(ctx, cudaLaunchKernelEx(&cfg, quant_table_kernel<QC_THREADS>, reinterpret_cast<const float4 *>(grad_rows), uniq_off,
+                                          ctx->D / 4, reinterpret_cast<char4 *>(codes), grad_scales));
+    dq_mark(ctx, st, DQ_K_QUANT);
+    return DQRM_OK;
+}
+
 template <int MODE, int LPR, int CH, bool EXACT, bool TRACK = false>
 __global__ void __launch_bounds__(QU_THREADS)
 row_stream_kernel(float *__restrict__ tables, const int64_t *__restrict__ row_off,
@@ -143,9 +242,15 @@ int dispatch(dqrm_ctx *ctx, float *tables, const int32_t *unique_rows, const int
 size_t dq_quant_ws_bytes(const dqrm_ctx *ctx) { return align_up(sizeof(u32) * ctx->T, 256); }
 
 int dq_launch_grad_quant(dqrm_ctx *ctx, const float *grad_rows, const int32_t *uniq_off, int8_t *codes,
-                         float *grad_scales, void *ws, size_t ws_bytes, cudaStream_t st)
+                         float *grad_scales, int64_t max_values, void *ws, size_t ws_bytes, cudaStream_t st)
 {
     if (ws_bytes < dq_quant_ws_bytes(ctx)) return DQRM_ERR_WORKSPACE;
+    if (quant_by_table(ctx, max_values / 4)) {
+        const int64_t per_table = (max_values / 4 + ctx->T - 1) / ctx->T;
+        if (per_table <= (int64_t)QC_CLUSTER * 256 * QC_VEC)
+            return launch_quant_table<256>(ctx, grad_rows, uniq_off, codes, grad_scales, per_table, st);
+        return launch_quant_table<512>(ctx, grad_rows, uniq_off, codes, grad_scales, per_table, st);
+    }
     u32 *absmax = reinterpret_cast<u32 *>(ws);
     const int rc = launch_absmax(ctx, grad_rows, uniq_off, absmax, st);
     if (rc != DQRM_OK) return rc;
