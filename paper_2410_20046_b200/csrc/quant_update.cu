@@ -84,10 +84,10 @@ int launch_absmax(dqrm_ctx *ctx, const float *grad_rows, const int32_t *uniq_off
 // cluster) and quantises what it still holds in registers; what does not fit in them is read again.  Three launches that
 // clear the maxima, find them and quantise are bound by the launches' own latency until the values fill the memory system.
 // Measured on B200 (us, graph replay; one launch / three), 26 tables: 8 K values a table 3.2 / 6.5, 64 K 4.4 / 9.4,
-// 128 K 5.9 / 13.8, 512 K 19 / 33; one table: 8 K 2.7 / 5.2, 128 K 4.1 / 5.8, 256 K 8.0 / 6.0 (eight blocks are too few
-// for what they do not hold).  So it takes batches that the clusters hold, and up to four times that where the
-// clusters of all tables fill the chip.  256 threads a block while that holds a table, 512 then: 40 tables of 64 K values
-// take 5.2 us with 256 and 8.4 with 512 (a second wave).
+// 128 K 5.9 / 13.8, 512 K 19 / 33; one table: 8 K 2.7 / 5.2, 128 K 4.1 / 5.8, 256 K 5.6 / 5.9, 320 K 6.6 / 5.9 (eight
+// blocks are too few for what they do not hold); seven tables of 512 K 10.2 / 13.2.  256 threads a block while that
+// holds a table (40 tables of 64 K values take 5.2 us with 256 and 8.4 with 512: a second wave), 512 then, and 1024
+// where the tables are few and do not fill the chip with 512 (seven of 256 K: 5.8 us, 8.0 with 512).
 constexpr int QC_VEC = 8;             // vectors of four that a thread holds
 constexpr int QC_CLUSTER = 8;
 
@@ -151,8 +151,8 @@ quant_table_kernel(const float4 *__restrict__ grad_rows, const int32_t *__restri
 // whether a batch of up to max_vectors goes through the kernel above
 inline bool quant_by_table(const dqrm_ctx *ctx, int64_t max_vectors)
 {
-    const int64_t held = (int64_t)ctx->T * QC_CLUSTER * 512 * QC_VEC;
-    return max_vectors <= ((int64_t)ctx->T * QC_CLUSTER >= ctx->num_sms ? 4 * held : held);
+    const int64_t held = (int64_t)ctx->T * QC_CLUSTER * 1024 * QC_VEC;
+    return max_vectors <= (ctx->T >= 6 ? 2 * held : held);
 }
 
 template <int QC_THREADS>
@@ -249,6 +249,8 @@ int dq_launch_grad_quant(dqrm_ctx *ctx, const float *grad_rows, const int32_t *u
         const int64_t per_table = (max_values / 4 + ctx->T - 1) / ctx->T;
         if (per_table <= (int64_t)QC_CLUSTER * 256 * QC_VEC)
             return launch_quant_table<256>(ctx, grad_rows, uniq_off, codes, grad_scales, per_table, st);
+        if (per_table > (int64_t)QC_CLUSTER * 512 * QC_VEC && ctx->T * QC_CLUSTER < ctx->num_sms)
+            return launch_quant_table<1024>(ctx, grad_rows, uniq_off, codes, grad_scales, per_table, st);
         return launch_quant_table<512>(ctx, grad_rows, uniq_off, codes, grad_scales, per_table, st);
     }
     u32 *absmax = reinterpret_cast<u32 *>(ws);

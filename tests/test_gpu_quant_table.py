@@ -18,7 +18,8 @@ SHAPES = {
     (64, "one table holds nearly all"): ([0, 9000, 1, 0, 0, 0, 3, 0], None),
     (1020, "wide rows"): ([5, 0, 70], None),
     (16, "larger than the registers"): ([9000] * 10 + [0, 200] * 5, None),
-    (16, "large buffers"): ([128, 0, 700], 140_000),
+    (64, "blocks of 1024"): ([4096, 2050, 0, 1], None),
+    (16, "large buffers"): ([128, 0, 700], 300_000),
 }
 
 
