@@ -241,7 +241,7 @@ const char *dqrm_kernel_name(int kernel_id)
         "begin", "refresh_kernel", "fwd_kernel", "memset", "rs_setup_kernel", "rs_hist_kernel", "rs_scan_kernel",
         "rs_scatter_kernel", "seg_count_kernel", "seg_emit_kernel", "seg_sum_kernel",
         "zero_kernel", "absmax_kernel", "row_stream_kernel<quant>", "row_stream_kernel<update>", "row_stream_kernel<fused>",
-        "copy", "small_sort_kernel", "cluster_sort_kernel", "dp_pack_kernel", "dp_sum_update_kernel", "pack_kernel", "packed_fwd_kernel", "fwd_codes_kernel", "decode_payload_kernel"};
+        "copy", "small_sort_kernel", "small_step_kernel", "cluster_sort_kernel", "dp_pack_kernel", "dp_sum_update_kernel", "pack_kernel", "packed_fwd_kernel", "fwd_codes_kernel", "decode_payload_kernel"};
     return (kernel_id >= 0 && kernel_id < DQ_K_COUNT) ? names[kernel_id] : "?";
 }
 
@@ -325,6 +325,12 @@ int dqrm_train_step(dqrm_ctx *ctx, float *tables, const int32_t *indices, const 
     if (!ws_ok(workspace, workspace_bytes, dq_bwd_ws_bytes(ctx, L, (int64_t)ctx->T * B))) return DQRM_ERR_WORKSPACE;
     cudaStream_t st = as_stream(stream);
     if (ctx->prof_on) dq_mark(ctx, st, DQ_K_BEGIN);
+    if (dq_small_step_takes(ctx, B, L)) {
+        const int rc = dq_launch_fwd(ctx, tables, indices, offsets, scales, bits, out, nullptr, B, L, st, true);
+        if (rc != DQRM_OK) return rc;
+        return dq_launch_small_step(ctx, tables, indices, offsets, grad_out, unique_rows, uniq_off, grad_rows, codes,
+                                    grad_scales, lr, B, L, workspace, workspace_bytes, st);
+    }
     // The backward up to the summed gradient needs the indices and the upstream gradient but neither the
     // tables nor the forward's output, so it runs on the context's second stream while the forward runs on
     // the caller's (per-launch profiling keeps one stream, because its events time consecutive launches).

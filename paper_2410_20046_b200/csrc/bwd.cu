@@ -20,6 +20,7 @@
 #include "cluster_sort.cuh"
 #include "radix_sort.cuh"
 #include "small_sort.cuh"
+#include "small_step.cuh"
 
 namespace {
 
@@ -498,6 +499,44 @@ int dq_launch_bwd_sum(dqrm_ctx *ctx, const float *grad_out, int32_t *unique_rows
     if (D <= 32) return launch_sum<8, 4>(ctx, a, y.sum_small, st);
     if (D <= 64) return launch_sum<32, 2>(ctx, a, y.sum_small, st);
     return launch_sum<32, 4>(ctx, a, y.sum_small, st);
+}
+
+// The one-launch step takes tables of up to 512 lookups and 16 K gathered values, up to 4096 lookups in all (what a block
+// counts in front of its own).  Measured on B200 (graph replay, us a step with the forward, this way / in four launches):
+// 4 tables of 128 lookups of 16 features 9.3 / 15.7, 512 of 16 14.2 / 18.5, 1024 of 16 22.3 / 21.0, 256 of 64 15.9 / 17.8,
+// 512 of 64 24.8 / 22.0, 128 of 128 14.7 / 18.1, 256 of 128 22.8 / 20.0; 26 tables of 128 of 16 13.9 / 16.1, of 64
+// 15.8 / 20.9, of 128 19.8 / 20.7.  (With a row summary attached, or the sort chosen by the caller, the launches stay apart.)
+bool dq_small_step_takes(const dqrm_ctx *ctx, int B, int64_t L)
+{
+    const int64_t per_table = (L + ctx->T - 1) / ctx->T, want = L == (int64_t)ctx->T * B ? per_table : per_table + per_table / 4;
+    return L > 0 && L <= sstep::MAX_LOOKUPS && want <= sstep::THREADS && want * ctx->D <= 16384 && ctx->D <= 128 &&
+           ctx->T <= ctx->num_sms && ctx->sort_path != 1 && !ctx->row_summary && !ctx->payload_position;
+}
+
+int dq_launch_small_step(dqrm_ctx *ctx, float *tables, const int32_t *indices, const int32_t *offsets, const float *grad_out,
+                         int32_t *unique_rows, int32_t *uniq_off, float *grad_rows, int8_t *codes, float *grad_scales, float lr,
+                         int B, int64_t L, void *ws_, size_t ws_bytes, cudaStream_t st)
+{
+    const Layout y = make_layout(ctx, L);
+    if (ws_bytes < y.total) return DQRM_ERR_WORKSPACE;
+    char *ws = reinterpret_cast<char *>(ws_);
+    sstep::Args x = {};
+    x.s.indices = indices; x.s.offsets = offsets; x.s.row_off = ctx->d_row_off;
+    x.s.T = ctx->T; x.s.B = B; x.s.L = L;
+    x.s.gp[0] = reinterpret_cast<uint2 *>(ws + y.pairs_a); x.s.gp[1] = reinterpret_cast<uint2 *>(ws + y.pairs_b);
+    x.s.status = ctx->d_status;
+    x.grad_out = grad_out; x.tables = tables; x.grad_rows = grad_rows;
+    x.unique_rows = unique_rows; x.uniq_off = uniq_off; x.codes = codes; x.grad_scales = grad_scales;
+    x.lr = lr; x.D = ctx->D;
+    while ((4 << x.lpr_log) < ctx->D) ++x.lpr_log;
+    const size_t smem = sstep::smem_bytes(ctx->T);
+    bool &raised = ctx->smem_raised[DQ_SMEM_SLOT_STEP];
+    if (!raised)
+        DQRM_CUDA_TRY(ctx, cudaFuncSetAttribute(sstep::small_step_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    raised = true;
+    DQRM_CUDA_TRY(ctx, dq_launch(sstep::small_step_kernel, dim3((unsigned)ctx->T), dim3(sstep::THREADS), smem, st, x));
+    dq_mark(ctx, st, DQ_K_SMALL_STEP);
+    return DQRM_OK;
 }
 
 int dq_launch_bwd(dqrm_ctx *ctx, const float *grad_out, const int32_t *indices, const int32_t *offsets,

@@ -72,7 +72,7 @@ struct dqrm_ctx {
 enum {
     DQ_K_BEGIN = 0, DQ_K_REFRESH, DQ_K_FWD, DQ_K_MEMSET, DQ_K_SORT_SETUP, DQ_K_SORT_HIST, DQ_K_SORT_SCAN, DQ_K_SORT_SCATTER,
     DQ_K_SEG_COUNT, DQ_K_SEG_EMIT, DQ_K_SEG_SUM, DQ_K_ZERO, DQ_K_ABSMAX, DQ_K_QUANT, DQ_K_UPDATE,
-    DQ_K_QUANT_UPDATE, DQ_K_COPY, DQ_K_SMALL_SORT, DQ_K_CLUSTER_SORT, DQ_K_DP_PACK, DQ_K_DP_SUM_UPDATE, DQ_K_PACK, DQ_K_PACKED_FWD, DQ_K_FWD_CODES, DQ_K_DECODE_PAYLOAD, DQ_K_COUNT
+    DQ_K_QUANT_UPDATE, DQ_K_COPY, DQ_K_SMALL_SORT, DQ_K_SMALL_STEP, DQ_K_CLUSTER_SORT, DQ_K_DP_PACK, DQ_K_DP_SUM_UPDATE, DQ_K_PACK, DQ_K_PACKED_FWD, DQ_K_FWD_CODES, DQ_K_DECODE_PAYLOAD, DQ_K_COUNT
 };
 constexpr int DQ_PROF_MAX = 4096;
 
@@ -122,10 +122,16 @@ __device__ __forceinline__ void dq_wait_before()
     asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
+// the kernel launched behind this one may begin once all blocks have come here; its dq_wait_before still waits for their end
+__device__ __forceinline__ void dq_let_next()
+{
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
 static inline size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
 // slots of dqrm_ctx::smem_raised
-constexpr int DQ_SMEM_SLOT_CSORT = 24;
+constexpr int DQ_SMEM_SLOT_STEP = 4, DQ_SMEM_SLOT_CSORT = 24;
 constexpr int dq_log2c(int x) { return x <= 1 ? 0 : 1 + dq_log2c(x / 2); }
 
 // ---------------------------------------------------------------------------------
@@ -323,7 +329,13 @@ int dq_launch_refresh(dqrm_ctx *ctx, const float *tables, const int32_t *bits, f
 
 int dq_launch_fwd(dqrm_ctx *ctx, const float *tables, const int32_t *indices, const int32_t *offsets,
                   const float *scales, const int32_t *bits, float *out, int8_t *codes_out,
-                  int B, int64_t L, cudaStream_t st);
+                  int B, int64_t L, cudaStream_t st, bool let_next = false);
+
+// the step's backward, quantiser and update in one launch, for small batches
+bool dq_small_step_takes(const dqrm_ctx *ctx, int B, int64_t L);
+int dq_launch_small_step(dqrm_ctx *ctx, float *tables, const int32_t *indices, const int32_t *offsets, const float *grad_out,
+                         int32_t *unique_rows, int32_t *uniq_off, float *grad_rows, int8_t *codes, float *grad_scales, float lr,
+                         int B, int64_t L, void *ws, size_t ws_bytes, cudaStream_t st);
 
 size_t dq_bwd_ws_bytes(const dqrm_ctx *ctx, int64_t L, int64_t G);
 // per-table |grad| maxima (float bit patterns) inside a workspace that dq_launch_bwd_sort and

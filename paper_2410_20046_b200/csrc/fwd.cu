@@ -41,6 +41,7 @@ struct FwdArgs {
     int T, D, B;
     int64_t L;
     int *status;
+    int let_next;                // the kernel behind this one may begin (it waits itself where it has to)
 };
 
 __device__ __forceinline__ void store_codes(int8_t *codes_out, int64_t j, int D, int c4, const float4 &c)
@@ -108,6 +109,7 @@ __global__ void __launch_bounds__(FW_THREADS, 5)
 fwd_onehot_kernel(const FwdArgs a)
 {
     dq_wait_before();
+    if (a.let_next) dq_let_next();
     constexpr int NB = NBOf<LPR, CH>::v;      // row steps in flight
     constexpr int RPW = 32 / LPR;             // rows one warp instruction covers
     constexpr int WPB = FW_THREADS / 32;
@@ -233,6 +235,7 @@ __global__ void __launch_bounds__(FW_THREADS)
 fwd_bags_kernel(const FwdArgs a)
 {
     dq_wait_before();
+    if (a.let_next) dq_let_next();
     typedef typename Vec<VEC>::type vec_t;
     constexpr int NB = CH >= 2 ? 1 : LPR < 4 ? LPR : 4;
     constexpr int GPB = FW_THREADS / LPR;
@@ -346,10 +349,10 @@ int launch(dqrm_ctx *ctx, const FwdArgs &a, cudaStream_t st)
 
 int dq_launch_fwd(dqrm_ctx *ctx, const float *tables, const int32_t *indices, const int32_t *offsets,
                   const float *scales, const int32_t *bits, float *out, int8_t *codes_out,
-                  int B, int64_t L, cudaStream_t st)
+                  int B, int64_t L, cudaStream_t st, bool let_next)
 {
     FwdArgs a{tables, ctx->d_row_off, indices, offsets, scales, bits, out, codes_out, ctx->T, ctx->D, B, L,
-              ctx->d_status};
+              ctx->d_status, let_next ? 1 : 0};
     const int d4 = ctx->D / 4;
     if (d4 <= 1) return launch<1, 1>(ctx, a, st);
     if (d4 <= 2) return launch<2, 1>(ctx, a, st);

@@ -118,6 +118,93 @@ __device__ __noinline__ const uint2 *sort_in_memory(const csort::Args &a, int t,
     return a.gp[s] + tb0;
 }
 
+// The block's table (n <= THREADS * EPT lookups) into s_net[0 .. n): row << 32 | payload; s_net has 2 * THREADS * EPT places
+template <int THREADS, int EPT>
+__device__ __forceinline__ void sort_in_block(const csort::Args &a, int t, int64_t tb0, int64_t n, int64_t nrows, u64 *s_net, bool &bad)
+{
+    constexpr int N = THREADS * EPT;
+    const int tid = threadIdx.x;
+    u64 e[EPT];                                    // row << 32 | position, later row << 32 | payload
+    u32 pay[EPT];
+#pragma unroll
+    for (int k = 0; k < EPT; ++k) {            // (loads coalesced: thread tid takes entries tid, tid + THREADS, ...)
+        const int p = k * THREADS + tid;
+        e[k] = ~0ull;
+        pay[k] = 0u;
+        if (p < n) {
+            const uint2 pr = lookup(a, t, tb0, n, nrows, p, bad);
+            e[k] = (u64)pr.x << 32 | (u32)p;
+            pay[k] = pr.y;
+        }
+    }
+    int top = 1;                               // entries that the network covers: a power of two from 32 * EPT on
+    while ((1 << top) < n) ++top;
+    const bool live = (tid & ~31) * EPT < (1 << top);       // (warps of places beyond only keep the barriers)
+    u64 *buf = s_net;
+    if (EPT > 1) {                             // to EPT consecutive entries per thread
+#pragma unroll
+        for (int k = 0; k < EPT; ++k) buf[k * THREADS + tid] = e[k];
+        __syncthreads();
+#pragma unroll
+        for (int k = 0; k < EPT; ++k) e[k] = buf[tid * EPT + k];
+        buf = s_net + N;
+    }
+    const int i0 = tid * EPT;                  // first entry of this thread
+    constexpr int TOP = log2c(N);
+#pragma unroll
+    for (int p = 1; p <= TOP; ++p) {
+        if (p > top) break;                    // (block-uniform)
+#pragma unroll
+        for (int s = p - 1; s >= 0; --s) {
+            const int stride = 1 << s;
+            if (stride >= 32 * EPT) {
+#pragma unroll
+                for (int k = 0; k < EPT; ++k) buf[i0 + k] = e[k];
+                __syncthreads();
+                const bool up = ((i0 >> p) & 1) == 0, low = (i0 & stride) == 0;
+#pragma unroll
+                for (int k = 0; k < EPT; ++k) {
+                    const u64 o = buf[(i0 + k) ^ stride];
+                    e[k] = (up == low) == (e[k] < o) ? e[k] : o;
+                }
+                buf = buf == s_net ? s_net + N : s_net;
+            } else if (stride >= EPT) {
+                const bool up = ((i0 >> p) & 1) == 0, low = (i0 & stride) == 0;
+#pragma unroll
+                for (int k = 0; live && k < EPT; ++k) {
+                    const u64 o = shfl_xor64(e[k], stride / EPT);
+                    e[k] = (up == low) == (e[k] < o) ? e[k] : o;
+                }
+            } else {
+#pragma unroll
+                for (int k = 0; k < EPT; ++k) {
+                    if ((k & stride) == 0) {
+                        const bool up = (((i0 + k) >> p) & 1) == 0;
+                        const u64 x = e[k], y = e[(k + stride) % EPT];
+                        const bool swap = up ? y < x : x < y;
+                        e[k] = swap ? y : x;
+                        e[(k + stride) % EPT] = swap ? x : y;
+                    }
+                }
+            }
+        }
+    }
+    // the payloads come back by position
+    __syncthreads();
+    u32 *s_pay = reinterpret_cast<u32 *>(s_net);
+#pragma unroll
+    for (int k = 0; k < EPT; ++k) s_pay[k * THREADS + tid] = pay[k];
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < EPT; ++k)
+        if (i0 + k < n) e[k] = (e[k] & 0xffffffff00000000ull) | s_pay[(u32)e[k]];
+    __syncthreads();
+    u64 *s_out = s_net;
+#pragma unroll
+    for (int k = 0; k < EPT; ++k) s_out[i0 + k] = e[k];
+    __syncthreads();
+}
+
 template <int THREADS, int EPT>
 __global__ void __launch_bounds__(THREADS)
 small_sort_kernel(const csort::Args a)
@@ -149,88 +236,11 @@ small_sort_kernel(const csort::Args a)
     if (bad) dq_report(a.status, DQRM_ERR_INDEX_RANGE);
     if (n == 0) return;
     const uint2 *mem = nullptr;                    // the sorted pairs of a table that does not fit the block
-    u64 e[EPT];                                    // row << 32 | position, later row << 32 | payload
     if (n > N) {
         mem = sort_in_memory<THREADS>(a, t, tb0, n, nrows, reinterpret_cast<u32 *>(s_net));
     } else {
-        u32 pay[EPT];
-#pragma unroll
-        for (int k = 0; k < EPT; ++k) {            // (loads coalesced: thread tid takes entries tid, tid + THREADS, ...)
-            const int p = k * THREADS + tid;
-            e[k] = ~0ull;
-            pay[k] = 0u;
-            if (p < n) {
-                const uint2 pr = lookup(a, t, tb0, n, nrows, p, bad);
-                e[k] = (u64)pr.x << 32 | (u32)p;
-                pay[k] = pr.y;
-            }
-        }
+        sort_in_block<THREADS, EPT>(a, t, tb0, n, nrows, s_net, bad);
         if (bad) dq_report(a.status, DQRM_ERR_INDEX_RANGE);
-        int top = 1;                               // entries that the network covers: a power of two from 32 * EPT on
-        while ((1 << top) < n) ++top;
-        u64 *buf = s_net;
-        if (EPT > 1) {                             // to EPT consecutive entries per thread
-#pragma unroll
-            for (int k = 0; k < EPT; ++k) buf[k * THREADS + tid] = e[k];
-            __syncthreads();
-#pragma unroll
-            for (int k = 0; k < EPT; ++k) e[k] = buf[tid * EPT + k];
-            buf = s_net + N;
-        }
-        const int i0 = tid * EPT;                  // first entry of this thread
-        constexpr int TOP = log2c(N);
-#pragma unroll
-        for (int p = 1; p <= TOP; ++p) {
-            if (p > top) break;                    // (block-uniform)
-#pragma unroll
-            for (int s = p - 1; s >= 0; --s) {
-                const int stride = 1 << s;
-                if (stride >= 32 * EPT) {
-#pragma unroll
-                    for (int k = 0; k < EPT; ++k) buf[i0 + k] = e[k];
-                    __syncthreads();
-                    const bool up = ((i0 >> p) & 1) == 0, low = (i0 & stride) == 0;
-#pragma unroll
-                    for (int k = 0; k < EPT; ++k) {
-                        const u64 o = buf[(i0 + k) ^ stride];
-                        e[k] = (up == low) == (e[k] < o) ? e[k] : o;
-                    }
-                    buf = buf == s_net ? s_net + N : s_net;
-                } else if (stride >= EPT) {
-                    const bool up = ((i0 >> p) & 1) == 0, low = (i0 & stride) == 0;
-#pragma unroll
-                    for (int k = 0; k < EPT; ++k) {
-                        const u64 o = shfl_xor64(e[k], stride / EPT);
-                        e[k] = (up == low) == (e[k] < o) ? e[k] : o;
-                    }
-                } else {
-#pragma unroll
-                    for (int k = 0; k < EPT; ++k) {
-                        if ((k & stride) == 0) {
-                            const bool up = (((i0 + k) >> p) & 1) == 0;
-                            const u64 x = e[k], y = e[(k + stride) % EPT];
-                            const bool swap = up ? y < x : x < y;
-                            e[k] = swap ? y : x;
-                            e[(k + stride) % EPT] = swap ? x : y;
-                        }
-                    }
-                }
-            }
-        }
-        // the payloads come back by position
-        __syncthreads();
-        u32 *s_pay = reinterpret_cast<u32 *>(s_net);
-#pragma unroll
-        for (int k = 0; k < EPT; ++k) s_pay[k * THREADS + tid] = pay[k];
-        __syncthreads();
-#pragma unroll
-        for (int k = 0; k < EPT; ++k)
-            if (i0 + k < n) e[k] = (e[k] & 0xffffffff00000000ull) | s_pay[(u32)e[k]];
-        __syncthreads();
-        u64 *s_out = s_net;
-#pragma unroll
-        for (int k = 0; k < EPT; ++k) s_out[i0 + k] = e[k];
-        __syncthreads();
     }
     // ---- sorted keys and payloads, and where the segments stand: THREADS consecutive entries at a time
     u32 *segs = a.seg_start + tb0 + t;

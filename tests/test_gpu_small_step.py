@@ -1,0 +1,76 @@
+"""GPU parity of the small batch's step in one launch behind the forward, at its edges: tables of no, one and many
+lookups, runs that cross many lane groups' shares, an uneven batch whose table does not fit the block, feature sizes
+whose last lanes are idle, and the batch on either side of the largest that it takes."""
+import numpy as np
+import pytest
+
+from dqrm_inputs import workloads as W
+from gpu_util import Case, bit_equal
+
+pytestmark = pytest.mark.gpu
+
+# feature size: lookups per table
+SHAPES = {
+    "single": (16, [1]), "empty_tables": (4, [0, 3, 0, 0, 40, 0]), "tiny": (16, [128, 128, 128, 128]), "idle_lanes": (20, [33, 257, 64]),
+    "block": (16, [512, 511, 513, 512]), "beyond_it": (16, [513, 513, 513, 513]), "all": (32, [512] * 8), "and_one": (4, [512] * 7 + [513]),
+    "one_table_holds_all": (8, [0, 2, 3200, 0, 0, 0, 1, 0]), "wide": (128, [127, 128]), "narrow": (4, [300] * 13),
+    "many_tables": (8, [1, 0, 40, 33] * 30),
+}
+
+
+@pytest.mark.parametrize("rows", [1, 9, 50_000])
+@pytest.mark.parametrize("name", list(SHAPES))
+def test_small_step(oracle, name, rows):
+    import torch
+
+    D, counts = SHAPES[name]
+    T, B = len(counts), max(1, max(counts))
+    wl = W.Workload("step", tuple(rows + t for t in range(T)), D=D, B=B, alpha=None)
+    rng = np.random.default_rng(rows + B + D)
+    idx = np.concatenate([rng.integers(0, wl.rows[t], n) for t, n in enumerate(counts)]).astype(np.int32)
+    lens = np.zeros((T, B), dtype=np.int64)
+    for t, n in enumerate(counts):
+        np.add.at(lens[t], rng.integers(0, B, n) if t % 2 else np.arange(n), 1)
+    off = np.concatenate([[0], np.cumsum(lens.reshape(-1))]).astype(np.int32)
+    # gradients are multiples of 2^-8 below 4, so sums of a few thousand are exact in FP32 and every output has one value
+    go = (rng.integers(-1024, 1025, (B, T, D)) / 256).astype(np.float32)
+    L = len(idx)
+    c = Case(wl, max_lookups=L)
+    o_tables = W.tables_np(wl)
+    o_scales, _ = oracle.scale_refresh(o_tables, c.row_off, D, c.bits_np)
+    d_tables = c.dev(o_tables)
+    r = oracle.train_step(o_tables, c.row_off, D, B, idx, off, go, o_scales, c.bits_np, wl.lr)
+    out, uo, gs = c.empty((B, T, D), torch.float32), c.empty(T + 1, torch.int32), c.empty(T, torch.float32)
+    ur, gr, codes = c.empty(L, torch.int32), c.empty((L, D), torch.float32), c.empty((L, D), torch.int8)
+    c.ctx.train_step(d_tables, c.dev(idx), c.dev(off), c.dev(go), c.dev(o_scales), c.bits, out, ur, uo, gr, codes, gs,
+                     wl.lr, B=B, L=L)
+    c.ctx.raise_on_device_error()
+    U = int(r["uniq_off"][-1])
+    np.testing.assert_allclose(out.cpu().numpy(), r["out"], rtol=1e-5, atol=1e-6)      # (the forward's own tolerance)
+    assert bit_equal(uo.cpu().numpy(), r["uniq_off"]) and bit_equal(ur.cpu().numpy()[:U], r["unique_rows"])
+    assert bit_equal(gr.cpu().numpy()[:U], r["grad_rows"]) and bit_equal(gs.cpu().numpy(), r["grad_scales"])
+    assert bit_equal(codes.cpu().numpy()[:U], r["codes"]) and bit_equal(d_tables.cpu().numpy(), o_tables)
+    c.ctx.close()
+
+
+@pytest.mark.parametrize("boundary", [(0, 1), (2, 500), (2, -3), (4, 80)])
+def test_unusable_boundaries_touch_no_row(boundary):
+    import torch
+    import paper_2410_20046_b200 as dq
+
+    T, B, D = 4, 32, 16
+    wl = W.Workload("step", (40,) * T, D=D, B=B, alpha=None)
+    c = Case(wl)
+    tables = W.tables_np(wl)
+    d_tables = c.dev(tables)
+    off = np.arange(T * B + 1, dtype=np.int32)
+    off[boundary[0] * B] = boundary[1]
+    out, uo, gs = c.empty((B, T, D), torch.float32), c.empty(T + 1, torch.int32), c.empty(T, torch.float32)
+    ur, gr = c.empty(T * B, torch.int32), c.empty((T * B, D), torch.float32)
+    c.ctx.train_step(d_tables, c.dev(np.zeros(T * B, np.int32)), c.dev(off), c.dev(np.ones((B, T, D), np.float32)),
+                     c.dev(np.full(T, 0.1, np.float32)), c.bits, out, ur, uo, gr, c.empty((T * B, D), torch.int8), gs, wl.lr,
+                     B=B, L=T * B)
+    with pytest.raises(dq.DqrmError):
+        c.ctx.raise_on_device_error()
+    assert bit_equal(d_tables.cpu().numpy(), tables)
+    c.ctx.close()
