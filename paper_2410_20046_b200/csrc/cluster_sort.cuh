@@ -71,10 +71,12 @@ __device__ __forceinline__ u32 same_digit_lanes(u32 d, bool valid)
     return valid ? peers : 0u;
 }
 
-// (no minimum of resident blocks is asked for: with one, the compiler spends registers that the kernels running
-// beside the sort then lack - measured, the training step beside it went from 61 to 72 us)
+// (two blocks resident for clusters of eight, so that the clusters of all tables run at once: without the bound the
+// kernel takes 95 registers and 26 tables of 16 K lookups 40 us instead of 32, with three 37.  Clusters of sixteen are
+// launched for a few tables only and have their SMs to themselves: 36.6 us without the bound, 42.2 with it, for one table
+// of 64 K lookups)
 template <int CL>
-__global__ void __launch_bounds__(THREADS)
+__global__ void __launch_bounds__(THREADS, CL > 8 ? 1 : 2)
 cluster_sort_kernel(const Args a)
 {
     dq_wait_before();
@@ -143,27 +145,33 @@ cluster_sort_kernel(const Args a)
         (__ldg(a.offsets) != 0 || (int64_t)__ldg(a.offsets + (int64_t)a.T * a.B) != a.L))
         dq_report(a.status, DQRM_ERR_INDEX_RANGE);
     bool bad = false;
-    for (int i = threadIdx.x; i < my_n; i += THREADS) {
-        const int64_t p = (int64_t)c * npc + i;    // position within the table's lookups
-        int32_t idx = __ldg(a.indices + tb0 + p);
-        bool single = false;
-        if (n == a.B) {
-            const int64_t o0 = __ldg(off_t + p), o1 = __ldg(off_t + p + 1);
-            single = o0 == tb0 + p && o1 == tb0 + p + 1;
-            if (o0 > o1) dq_report(a.status, DQRM_ERR_INDEX_RANGE);
+    for (int i0 = threadIdx.x; i0 < my_n; i0 += 4 * THREADS) {
+        int32_t idx[4], o0[4], o1[4];              // (four lookups in flight: one at a time, 34 us instead of 32 for 26 tables of 16 K)
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const int64_t p = (int64_t)c * npc + min(i0 + k * THREADS, my_n - 1);      // position within the table's lookups
+            idx[k] = __ldg(a.indices + tb0 + p);
+            o0[k] = n == a.B ? __ldg(off_t + p) : 1;
+            o1[k] = n == a.B ? __ldg(off_t + p + 1) : 1;
         }
-        bad |= (idx < 0) | (idx >= nrows);
-        idx = (int32_t)min((int64_t)max(idx, 0), nrows - 1);
-        int64_t bag = p;
-        if (!single) {                             // largest bag b with offsets[t*B + b] <= tb0 + p
-            int lo = 0, hi = a.B;
-            while (hi - lo > 1) {
-                int mid = (lo + hi) >> 1;
-                if ((int64_t)__ldg(off_t + mid) <= tb0 + p) lo = mid; else hi = mid;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const int i = i0 + k * THREADS;
+            if (i >= my_n) break;
+            const int64_t p = (int64_t)c * npc + i;
+            const bool single = o0[k] == tb0 + p && o1[k] == tb0 + p + 1;
+            bad |= (o0[k] > o1[k]) | (idx[k] < 0) | (idx[k] >= nrows);
+            int64_t bag = p;
+            if (!single || n != a.B) {             // largest bag b with offsets[t*B + b] <= tb0 + p
+                int lo = 0, hi = a.B;
+                while (hi - lo > 1) {
+                    const int mid = (lo + hi) >> 1;
+                    if ((int64_t)__ldg(off_t + mid) <= tb0 + p) lo = mid; else hi = mid;
+                }
+                bag = lo;
             }
-            bag = lo;
+            pb0[i] = make_uint2((u32)min((int64_t)max(idx[k], 0), nrows - 1), a.payload_position ? (u32)(tb0 + p) : (u32)(bag * a.T + t));
         }
-        pb0[i] = make_uint2((u32)idx, a.payload_position ? (u32)(tb0 + p) : (u32)(bag * a.T + t));
     }
     if (bad) dq_report(a.status, DQRM_ERR_INDEX_RANGE);
 
