@@ -92,6 +92,13 @@ __device__ __forceinline__ void load_tile_keys(const u32 *__restrict__ keys, int
 {
     n = (int)max((int64_t)0, min((int64_t)ST_ITEMS, L - i0));
     prev = (i0 > 0 && i0 <= L) ? keys[i0 - 1] : 0xFFFFFFFFu;
+    static_assert(ST_ITEMS == 8, "");
+    if (n == ST_ITEMS) {                // (eight loads of a word by every thread: 16 us for 8.5 M keys)
+        const uint4 x = __ldg(reinterpret_cast<const uint4 *>(keys + i0)), y = __ldg(reinterpret_cast<const uint4 *>(keys + i0) + 1);
+        k[0] = x.x; k[1] = x.y; k[2] = x.z; k[3] = x.w;
+        k[4] = y.x; k[5] = y.y; k[6] = y.z; k[7] = y.w;
+        return;
+    }
 #pragma unroll
     for (int e = 0; e < ST_ITEMS; ++e) k[e] = (e < n) ? keys[i0 + e] : 0u;
 }

@@ -382,7 +382,9 @@ cluster_sort_kernel(const Args a)
             }
         }
     }
-    cluster.sync();      // nobody leaves while its shared memory may still be read or written
+    // nobody leaves while its shared memory may still be read or written (with the lists, the last remote access came before
+    // the barrier behind the totals)
+    if (!a.lists_by_table) cluster.sync();
 }
 
 inline size_t smem_bytes(int cap) { return (size_t)2 * cap * sizeof(uint2); }

@@ -23,8 +23,10 @@ __device__ __forceinline__ int table_of_row(const int32_t *uoff, int T, int64_t 
     return lo;
 }
 
-// rows in flight per lane group: fewer when a lane already holds several vectors of every row
-template <int CH> struct RowsInFlight { static constexpr int v = CH >= 4 ? 1 : (CH == 2 ? 2 : 4); };
+// rows in flight per lane group: fewer when a lane already holds several vectors of every row, and where fewer groups
+// share a warp the registers are better spent on more warps (160 K rows of 64 features: two rows 29.7 us, three 31.7,
+// four 32.0; 108 K rows of 16 features: two 13.3, four 12.3)
+template <int LPR, int CH> struct RowsInFlight { static constexpr int v = CH >= 4 ? 1 : (CH == 2 || LPR >= 16 ? 2 : 4); };
 
 // EXACT: the feature size is 4*LPR*CH, a compile-time constant, and the per-vector range checks fall away
 inline size_t smem_bytes(int T) { return (size_t)(T + 1) * sizeof(int32_t) + (size_t)T * sizeof(float); }
@@ -39,7 +41,7 @@ row_stream_body(unsigned char *smem_raw, float *__restrict__ tables, const int64
                 int8_t *__restrict__ codes, float *__restrict__ grad_scales, float lr, int T, int D_any,
                 int *__restrict__ status, float2 *__restrict__ row_summary = nullptr)
 {
-    constexpr int NB = RowsInFlight<CH>::v;
+    constexpr int NB = RowsInFlight<LPR, CH>::v;
     const int D = EXACT ? 4 * LPR * CH : D_any;
     int32_t *s_uoff = reinterpret_cast<int32_t *>(smem_raw);      // [T+1]
     float *s_scale = reinterpret_cast<float *>(s_uoff + (T + 1)); // [T] gradient scale of every table
@@ -65,6 +67,11 @@ row_stream_body(unsigned char *smem_raw, float *__restrict__ tables, const int64
     bool bad = false;
     float s = 1.f;
     QuantScale qs = dq_make_scale(1.f, 8);
+    int32_t next[NB];                   // row numbers of the batch to come
+    if (MODE != MODE_QUANT) {
+#pragma unroll
+        for (int b = 0; b < NB; ++b) next[b] = u_begin + b < u_end ? __ldg(unique_rows + u_begin + b) : 0;
+    }
     for (int64_t u = u_begin; u < u_end;) {
         if (u >= cur_end) {
             cur_t = table_of_row(s_uoff, T, u);
@@ -84,7 +91,7 @@ row_stream_body(unsigned char *smem_raw, float *__restrict__ tables, const int64
             if (b < nb && MODE != MODE_QUANT) {
                 // a row number outside its table is reported and kept inside the arena, never followed
                 // (no branch: the rows' index loads stay in flight together)
-                const int64_t row = __ldg(unique_rows + u + b);
+                const int64_t row = next[b];
                 bad |= (row < 0) | (row >= nrows);
                 wrow[b] = reinterpret_cast<float4 *>(tables + (r0 + min(max(row, (int64_t)0), nrows - 1)) * D);
             }
@@ -102,6 +109,11 @@ row_stream_body(unsigned char *smem_raw, float *__restrict__ tables, const int64
                     }
                 }
             }
+        }
+        if (MODE != MODE_QUANT) {
+            // the next batch's row numbers arrive under cover of this one (asking its master rows into L2 as well gave nothing)
+#pragma unroll
+            for (int b = 0; b < NB; ++b) next[b] = u + nb + b < u_end ? __ldg(unique_rows + u + nb + b) : 0;
         }
 #pragma unroll
         for (int b = 0; b < NB; ++b) {
