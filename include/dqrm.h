@@ -249,7 +249,9 @@ size_t dqrm_host_step_workspace_bytes(const dqrm_ctx *ctx, int64_t max_lookups, 
  * directions).  The workspace holds two sets of staging buffers that consecutive calls use in
  * turn, so the inputs of a call are copied while the call before it is still computing and
  * sending its output; a caller that issues calls back to back therefore keeps both directions
- * of the host link busy.  With dqrm_set_overlap(ctx, 0) everything stays on `stream`.
+ * of the host link busy.  (The staging buffers' places follow from the workspace, its size and
+ * T*B; where one of these is another than in the call before, or that call had no lookups, the
+ * copies wait for the work on `stream`.)  With dqrm_set_overlap(ctx, 0) everything stays on `stream`.
  * tables, scales and bits stay on the device.  The sparse gradient (unique rows, codes,
  * scales) stays in the workspace.  h_grad_out and h_out must stay valid and untouched
  * until the call's work on `stream` is complete. */
@@ -346,10 +348,11 @@ int dqrm_decode_payload(dqrm_ctx *ctx, const uint8_t *payload, const float *scal
 
 /* ---- choice of the backward's sort (no counterpart in the paper) --------------------
  * dqrm_emb_bwd and dqrm_train_step order the batch's lookups by row before they sum
- * duplicates.  path 0 (default): one thread-block cluster per table (eight blocks, sixteen
- * when the batch has very few tables) sorts that table's lookups in distributed shared
- * memory; a batch with more lookups per table than such a cluster holds takes path 1 by
- * itself.  path 1: one global least-significant-digit radix sort over all tables.  Both give
+ * duplicates.  path 0 (default): per table, one block with a sorting network (up to about a
+ * thousand lookups a table), or one thread-block cluster (eight blocks, sixteen when the batch
+ * has very few tables) in distributed shared memory; a batch with more lookups per table than
+ * such a cluster holds takes path 1 by itself.  path 1: a least-significant-digit radix sort in
+ * global memory, per table, all tables in the same launches.  All give
  * identical outputs; the choice only affects speed. */
 int dqrm_set_sort_path(dqrm_ctx *ctx, int path);
 
@@ -357,9 +360,12 @@ int dqrm_set_sort_path(dqrm_ctx *ctx, int path);
  * sort, gradient summation: neither needs the tables or the forward's output) on a second
  * stream owned by the context (created by dqrm_create), beside the forward on the caller's
  * stream, and join the two before the touched rows are updated; the caller's stream sees one
- * ordered step.  dqrm_train_step_sorted also moves its forward to a third, lowest-priority
- * stream of the context (forked from and joined to the caller's stream), so that the forward's
- * many blocks do not keep a sort of the next batch, running elsewhere, off the SMs.
+ * ordered step.  dqrm_train_step does so from 16 MB of gathered rows on; smaller batches, for
+ * which fork and join cost more than the overlap gives, stay on the caller's stream (the
+ * smallest as one launch behind the forward).  dqrm_train_step_sorted also moves its forward to
+ * a third, lowest-priority stream of the context (forked from and joined to the caller's
+ * stream), so that the forward's many blocks do not keep a sort of the next batch, running
+ * elsewhere, off the SMs.
  * on = 0 keeps every launch on the caller's stream.  Default: 1. */
 int dqrm_set_overlap(dqrm_ctx *ctx, int on);
 
