@@ -68,7 +68,7 @@ zero_kernel(u32 *__restrict__ p, int n)
 }
 
 // per-table maxima of |grad_rows|: cleared by a kernel and not by a memset, behind which the next kernel could not be
-// set up early (four calls of a small batch: 29.9 us with the memset, 26.7 with the kernel)
+// set up early (four calls of a small batch, before one launch took these: 29.9 us with the memset, 26.7 with the kernel)
 int launch_absmax(dqrm_ctx *ctx, const float *grad_rows, const int32_t *uniq_off, u32 *absmax, cudaStream_t st)
 {
     const size_t smem = (size_t)(ctx->T + 1) * sizeof(int32_t) + (size_t)ctx->T * sizeof(u32);
@@ -178,8 +178,10 @@ int launch_quant_table(dqrm_ctx *ctx, const float *grad_rows, const int32_t *uni
     return DQRM_OK;
 }
 
+// (with the rows' (min, max) stored the compiler would take registers that cost a resident block: 190 K rows of 64 features
+// 38.9 us with four blocks, 48.7 without the bound; 108 K rows of 16 features 15.7 with three)
 template <int MODE, int LPR, int CH, bool EXACT, bool TRACK = false>
-__global__ void __launch_bounds__(QU_THREADS)
+__global__ void __launch_bounds__(QU_THREADS, TRACK && CH == 1 ? (LPR >= 16 ? 4 : 3) : 1)
 row_stream_kernel(float *__restrict__ tables, const int64_t *__restrict__ row_off,
                   const int32_t *__restrict__ unique_rows, const int32_t *__restrict__ uniq_off,
                   const float *__restrict__ grad_rows, const u32 *__restrict__ absmax,

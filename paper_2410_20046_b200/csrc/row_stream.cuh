@@ -67,8 +67,8 @@ row_stream_body(unsigned char *smem_raw, float *__restrict__ tables, const int64
     bool bad = false;
     float s = 1.f;
     QuantScale qs = dq_make_scale(1.f, 8);
-    int32_t next[NB];                   // row numbers of the batch to come
-    if (MODE != MODE_QUANT) {
+    int32_t next[NB];                   // row numbers of the batch to come (not beside the (min, max): registers)
+    if (MODE != MODE_QUANT && !TRACK) {
 #pragma unroll
         for (int b = 0; b < NB; ++b) next[b] = u_begin + b < u_end ? __ldg(unique_rows + u_begin + b) : 0;
     }
@@ -91,7 +91,7 @@ row_stream_body(unsigned char *smem_raw, float *__restrict__ tables, const int64
             if (b < nb && MODE != MODE_QUANT) {
                 // a row number outside its table is reported and kept inside the arena, never followed
                 // (no branch: the rows' index loads stay in flight together)
-                const int64_t row = next[b];
+                const int64_t row = TRACK ? __ldg(unique_rows + u + b) : next[b];
                 bad |= (row < 0) | (row >= nrows);
                 wrow[b] = reinterpret_cast<float4 *>(tables + (r0 + min(max(row, (int64_t)0), nrows - 1)) * D);
             }
@@ -110,7 +110,7 @@ row_stream_body(unsigned char *smem_raw, float *__restrict__ tables, const int64
                 }
             }
         }
-        if (MODE != MODE_QUANT) {
+        if (MODE != MODE_QUANT && !TRACK) {
             // the next batch's row numbers arrive under cover of this one (asking its master rows into L2 as well gave nothing)
 #pragma unroll
             for (int b = 0; b < NB; ++b) next[b] = u + nb + b < u_end ? __ldg(unique_rows + u + nb + b) : 0;
