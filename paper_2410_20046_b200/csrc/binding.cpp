@@ -6,6 +6,7 @@
 #include <Python.h>
 #include <c10/cuda/CUDAStream.h>
 #include <algorithm>
+#include <torch/csrc/Exceptions.h>
 #include <torch/csrc/autograd/python_variable.h>
 #include "dqrm.h"
 
@@ -94,7 +95,9 @@ struct Reader {
     float number()
     {
         if (!ok) return 0.f;
-        const double v = PyFloat_AsDouble(args[at++]);
+        PyObject *o = PyNumber_Float(args[at++]);      // (float(...) of whatever the caller passed)
+        const double v = o ? PyFloat_AsDouble(o) : -1.0;
+        Py_XDECREF(o);
         if (v == -1.0 && PyErr_Occurred()) ok = false;
         return (float)v;
     }
@@ -118,20 +121,31 @@ struct Reader {
     }
 };
 
+// The interpreter's lock is given back for the call, and taken again whichever way the call is left
+struct WithoutGil {
+    PyThreadState *state = PyEval_SaveThread();
+    ~WithoutGil() { PyEval_RestoreThread(state); }
+};
+
 // (arguments are read in the order of the braces, which is the order of the C ABI)
+// torch's own calls may throw (a tensor without storage under tracing or vmap, no CUDA device for the current stream):
+// nothing may leave through the interpreter's C frames, so exceptions become Python errors here
 #define DQ_CALL(NAME, COUNT, ...)                                                   \
     PyObject *py_##NAME(PyObject *, PyObject *const *args, Py_ssize_t n)            \
     {                                                                               \
+        HANDLE_TH_ERRORS                                                            \
         Reader r(args, n, COUNT);                                                   \
         dqrm_ctx *ctx = static_cast<dqrm_ctx *>(r.address());                       \
         __VA_ARGS__                                                                 \
+        END_HANDLE_TH_ERRORS                                                        \
     }
 #define DQ_RETURN(CALL)                                                             \
     if (!r.ok) return nullptr;                                                      \
     int status;                                                                     \
-    Py_BEGIN_ALLOW_THREADS                                                          \
-    status = CALL;                                                                  \
-    Py_END_ALLOW_THREADS                                                            \
+    {                                                                               \
+        WithoutGil released;                                                        \
+        status = CALL;                                                              \
+    }                                                                               \
     return PyLong_FromLong(status)
 
 DQ_CALL(scale_refresh, 8,
