@@ -36,13 +36,6 @@ class Stream:
 CASES = {
     # a tensor inside vmap has no data pointer
     "vmap": "raises(lambda: torch.vmap(lambda x: (host_step(x, stream=Stream()), x)[1])(torch.zeros(3, 4)))",
-    # nor has one that only stands for a tensor while a program is traced
-    "fake": """
-from torch._subclasses.fake_tensor import FakeTensorMode
-with FakeTensorMode():
-    x = torch.zeros(4)
-raises(lambda: host_step(x, stream=Stream()))
-""",
     # a sparse tensor has no strides to ask about
     "sparse": "raises(lambda: host_step(torch.eye(3).to_sparse(), stream=Stream()), (RuntimeError, AssertionError))",
     # the current stream where there is no device
