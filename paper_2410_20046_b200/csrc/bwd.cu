@@ -538,8 +538,11 @@ int dq_launch_small_step(dqrm_ctx *ctx, float *tables, const int32_t *indices, c
     while ((4 << x.lpr_log) < ctx->D) ++x.lpr_log;
     const size_t smem = sstep::smem_bytes(ctx->T);
     bool &raised = ctx->smem_raised[DQ_SMEM_SLOT_STEP];
+    // (the limit belongs to the function on the device, not to this context: every context sets the same, that of the most
+    // tables that dq_small_step_takes lets through, or one with few tables would lower it for one with many)
     if (!raised)
-        DQRM_CUDA_TRY(ctx, cudaFuncSetAttribute(sstep::small_step_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        DQRM_CUDA_TRY(ctx, cudaFuncSetAttribute(sstep::small_step_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                (int)sstep::smem_bytes(ctx->num_sms)));
     raised = true;
     DQRM_CUDA_TRY(ctx, dq_launch(sstep::small_step_kernel, dim3((unsigned)ctx->T), dim3(sstep::THREADS), smem, st, x));
     dq_mark(ctx, st, DQ_K_SMALL_STEP);

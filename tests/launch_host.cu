@@ -1,0 +1,63 @@
+// The launch code of the backward over a stand-in for the CUDA runtime: launches are counted, refused and checked against
+// the functions' shared-memory limits on the host, and nothing runs on a device.  One scenario per run, named by argv[1];
+// 0 when what it asserts holds.
+#include "../paper_2410_20046_b200/csrc/bwd.cu"
+#include <cstdio>
+#include <cstring>
+#include "launch_host.h"
+
+namespace {
+
+#define WANT(X)                                                                                          \
+    do {                                                                                                 \
+        if (!(X)) { std::printf("line %d: not so: %s\n", __LINE__, #X); return 1; }                      \
+    } while (0)
+
+char workspace[16 << 20];
+int32_t dummy[4];
+
+struct Ctx {
+    dqrm_ctx c;
+    Ctx(int T, int D)
+    {
+        c.T = T;
+        c.D = D;
+        c.num_sms = 148;
+        c.row_bits = 10;
+        c.total_rows = (int64_t)1000 * T;
+    }
+    int sort(int B, int64_t L, bool *by_table)
+    {
+        return dq_launch_bwd_sort(&c, dummy, dummy, dummy, dummy, B, L, workspace, sizeof(workspace), nullptr, true, by_table);
+    }
+    int small_step(int B, int64_t L)
+    {
+        return dq_launch_small_step(&c, nullptr, dummy, dummy, nullptr, dummy, dummy, nullptr, nullptr, nullptr, 0.1f, B, L,
+                                    workspace, sizeof(workspace), nullptr);
+    }
+};
+
+// contexts of many and of few tables take small steps in turn
+int contexts_in_turn()
+{
+    Ctx many(26, 16), few(4, 16), most(148, 16);
+    for (int k = 0; k < 2; ++k) {
+        WANT(many.small_step(8, 26 * 8) == DQRM_OK);
+        WANT(few.small_step(128, 4 * 128) == DQRM_OK);
+    }
+    for (int k = 0; k < 2; ++k) {
+        WANT(most.small_step(8, 148 * 8) == DQRM_OK);
+        WANT(few.small_step(128, 4 * 128) == DQRM_OK);
+    }
+    return 0;
+}
+
+}  // namespace
+
+int main(int argc, char **argv)
+{
+    const char *name = argc > 1 ? argv[1] : "";
+    if (!strcmp(name, "contexts_in_turn")) return contexts_in_turn();
+    std::printf("no scenario %s\n", name);
+    return 2;
+}

@@ -74,3 +74,35 @@ def test_unusable_boundaries_touch_no_row(boundary):
         c.ctx.raise_on_device_error()
     assert bit_equal(d_tables.cpu().numpy(), tables)
     c.ctx.close()
+
+
+def test_contexts_of_many_and_of_few_tables_take_turns(oracle):
+    """Two live contexts on one device: the kernel's shared-memory limit is the device's, not a context's."""
+    import torch
+
+    B, D = 16, 16
+    cases = []
+    for T in (100, 3):
+        wl = W.Workload("turns", (40,) * T, D=D, B=B, alpha=None)
+        c = Case(wl)
+        o_tables = W.tables_np(wl)
+        o_scales, _ = oracle.scale_refresh(o_tables, c.row_off, D, c.bits_np)
+        cases.append((c, o_tables, o_scales, c.dev(o_tables)))
+    for turn in range(3):
+        for c, o_tables, o_scales, d_tables in cases:
+            wl, L = c.wl, c.wl.T * B
+            rng = np.random.default_rng(turn + wl.T)
+            idx = rng.integers(0, 40, L).astype(np.int32)
+            off = np.arange(L + 1, dtype=np.int32)
+            go = (rng.integers(-1024, 1025, (B, wl.T, D)) / 256).astype(np.float32)
+            r = oracle.train_step(o_tables, c.row_off, D, B, idx, off, go, o_scales, c.bits_np, wl.lr)
+            out, uo, gs = c.empty((B, wl.T, D), torch.float32), c.empty(wl.T + 1, torch.int32), c.empty(wl.T, torch.float32)
+            ur, gr, codes = c.empty(L, torch.int32), c.empty((L, D), torch.float32), c.empty((L, D), torch.int8)
+            c.ctx.train_step(d_tables, c.dev(idx), c.dev(off), c.dev(go), c.dev(o_scales), c.bits, out, ur, uo, gr, codes,
+                             gs, wl.lr, B=B, L=L)
+            c.ctx.raise_on_device_error()
+            U = int(r["uniq_off"][-1])
+            assert bit_equal(uo.cpu().numpy(), r["uniq_off"]) and bit_equal(codes.cpu().numpy()[:U], r["codes"])
+            assert bit_equal(d_tables.cpu().numpy(), o_tables)
+    for c, *_ in cases:
+        c.ctx.close()
