@@ -421,10 +421,14 @@ int dq_launch_bwd_sort(dqrm_ctx *ctx, const int32_t *indices, const int32_t *off
         ca.cnt_broken = segred::CNT_BROKEN;
         const int64_t per_table = (L + ctx->T - 1) / ctx->T;
         cudaError_t e = cudaErrorUnknown;
-        if (lists_by_table && launch_small_sort(ctx, ca, per_table, L == G, st, e) && e == cudaSuccess) {
-            dq_mark(ctx, st, DQ_K_SMALL_SORT);
-            if (by_table) *by_table = true;
-            return DQRM_OK;
+        if (lists_by_table && launch_small_sort(ctx, ca, per_table, L == G, st, e)) {
+            if (e == cudaSuccess) {
+                dq_mark(ctx, st, DQ_K_SMALL_SORT);
+                if (by_table) *by_table = true;
+                return DQRM_OK;
+            }
+            ctx->last_cuda_error = (int)e;         // (taken off the runtime, so that nobody finds it behind the sort that follows)
+            (void)cudaGetLastError();
         }
         const bool wide = ctx->T * csort::CLUSTER_WIDE * 2 <= ctx->num_sms && per_table >= csort::CLUSTER_WIDE * 1024;
         if (wide) e = launch_cluster_sort<csort::CLUSTER_WIDE>(ctx, ca, per_table, st);

@@ -52,12 +52,30 @@ int contexts_in_turn()
     return 0;
 }
 
+// each sort that is refused leaves the next one to run, and no error for whoever asks next
+int refused_sorts()
+{
+    for (const int refused : {0, 1, 2}) {          // block sort, cluster sort, radix sort
+        fake::launches = 0;
+        fake::refuse.clear();
+        for (int k = 0; k < refused; ++k) fake::refuse.insert(k);
+        Ctx x(4, 16);
+        bool by_table = false;
+        WANT(x.sort(128, 4 * 128, &by_table) == DQRM_OK);
+        WANT(by_table == (refused < 2));
+        WANT(x.c.last_cuda_error == (refused ? (int)cudaErrorInvalidValue : 0));
+        WANT(cudaGetLastError() == cudaSuccess);
+    }
+    return 0;
+}
+
 }  // namespace
 
 int main(int argc, char **argv)
 {
     const char *name = argc > 1 ? argv[1] : "";
     if (!strcmp(name, "contexts_in_turn")) return contexts_in_turn();
+    if (!strcmp(name, "refused_sorts")) return refused_sorts();
     std::printf("no scenario %s\n", name);
     return 2;
 }

@@ -7,7 +7,7 @@ import subprocess
 import pytest
 
 HERE = os.path.dirname(os.path.abspath(__file__))
-SCENARIOS = ["contexts_in_turn"]
+SCENARIOS = ["contexts_in_turn", "refused_sorts"]
 
 
 @pytest.fixture(scope="module")
