@@ -99,7 +99,10 @@ cluster_sort_kernel(const Args a)
         (a.lists_by_table && ((t == 0 && tb0 != 0) || (t == a.T - 1 && tb1 != a.L)))) {
         if (threadIdx.x == 0 && c == 0) {
             dq_report(a.status, DQRM_ERR_INDEX_RANGE);
-            if (a.lists_by_table) a.table_cnt[t] = a.cnt_broken;       // nothing downstream runs
+            if (a.lists_by_table) {                // nothing is summed; the quantiser behind finds an empty gradient
+                a.table_cnt[t] = a.cnt_broken;
+                a.absmax[t] = 0u;
+            }
         }
         return;                                    // uniform over the cluster
     }

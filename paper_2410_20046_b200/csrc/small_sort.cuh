@@ -219,7 +219,8 @@ small_sort_kernel(const csort::Args a)
     if (tb0 < 0 || tb1 < tb0 || tb1 > a.L || (t == 0 && tb0 != 0) || (t == a.T - 1 && tb1 != a.L)) {
         if (tid == 0) {
             dq_report(a.status, DQRM_ERR_INDEX_RANGE);
-            a.table_cnt[t] = a.cnt_broken;         // nothing downstream runs
+            a.table_cnt[t] = a.cnt_broken;         // nothing is summed; the quantiser behind finds an empty gradient
+            a.absmax[t] = 0u;
         }
         return;
     }

@@ -381,3 +381,37 @@ def test_bad_arguments_are_refused_on_the_host():
     assert lib.dqrm_emb_bwd(*args, None, c.ctx.workspace_bytes, st) == dq.ERR_WORKSPACE
     torch.cuda.synchronize()
     c.ctx.close()
+
+
+@pytest.mark.parametrize("calls", ["one", "two"])
+@pytest.mark.parametrize("B", [300, 1500])                   # the block sort, the cluster sort
+def test_gradient_scales_of_a_batch_with_unusable_boundaries(oracle, B, calls):
+    """Nothing of such a batch is summed: every table's gradient scale is that of an empty gradient, whatever the
+    workspace held before."""
+    import torch
+    import paper_2410_20046_b200 as dq
+
+    T, D = 3, 64
+    wl = W.Workload("broken", (50, 7, 300), D=D, B=B, alpha=None)
+    c = Case(wl)
+    tables = W.tables_np(wl)
+    d_tables, L = c.dev(tables), T * B
+    c.ctx.workspace.fill_(0x7f)                              # (3.4e38 where the maxima stand)
+    off = np.arange(L + 1, dtype=np.int32)
+    off[B] = L + 3                                           # where table 1 begins
+    idx, d_off, go = c.dev(np.zeros(L, np.int32)), c.dev(off), c.dev(np.ones((B, T, D), np.float32))
+    out, uo, gs = c.empty((B, T, D), torch.float32), c.empty(T + 1, torch.int32), c.empty(T, torch.float32)
+    ur, gr, codes = c.empty(L, torch.int32), c.empty((L, D), torch.float32), c.empty((L, D), torch.int8)
+    scales = c.dev(np.full(T, 0.1, np.float32))
+    rest = (scales, c.bits, out, ur, uo, gr, codes, gs, wl.lr)
+    if calls == "one":
+        c.ctx.train_step(d_tables, idx, d_off, go, *rest, B=B, L=L)
+    else:
+        c.ctx.sort_batch(idx, d_off, ur, uo, B=B, L=L)
+        c.ctx.train_step_sorted(d_tables, idx, d_off, go, *rest, B=B, L=L)
+    with pytest.raises(dq.DqrmError):
+        c.ctx.raise_on_device_error()
+    assert not uo.cpu().numpy().any()
+    assert (gs.cpu().numpy() == oracle.scale_from_absmax(0.0, 8)).all()
+    assert bit_equal(d_tables.cpu().numpy(), tables)
+    c.ctx.close()
