@@ -17,6 +17,7 @@
 //   * fwd_bags_kernel (any other batch): a lane group walks one bag at a time, NB of its
 //     rows per batch, and sums them in bag order in FP64, rounded once, so the result
 //     does not depend on the launch shape.
+//   * fwd_long_bags_kernel: the same for long bags of rows of 36 to 64 features, a warp a bag.
 #include <type_traits>
 #include "common.cuh"
 
@@ -209,115 +210,147 @@ fwd_onehot_kernel(const FwdArgs a)
     if (bad) dq_report(a.status, DQRM_ERR_INDEX_RANGE);
 }
 
-// VEC consecutive floats (2 or 4)
-template <int VEC> struct Vec;
-template <> struct Vec<2> { typedef float2 type; };
-template <> struct Vec<4> { typedef float4 type; };
-__device__ __forceinline__ void unpack(const float2 &v, float *x) { x[0] = v.x; x[1] = v.y; }
-__device__ __forceinline__ void unpack(const float4 &v, float *x) { x[0] = v.x; x[1] = v.y; x[2] = v.z; x[3] = v.w; }
-__device__ __forceinline__ void store_sum(float2 *o, const double (&a)[2]) { *o = make_float2((float)a[0], (float)a[1]); }
-__device__ __forceinline__ void store_sum(float4 *o, const double (&a)[4])
-{
-    *o = make_float4((float)a[0], (float)a[1], (float)a[2], (float)a[3]);
-}
+// Resident blocks asked for.  The gather wants warps more than registers: left to itself the compiler takes 76 and up, and
+// 426 K rows of 256 bytes, two a bag, take 70 us with three blocks and 54 with four; 65 K rows of 1 KB 33 with four and 28
+// with five; of 2 KB, which then spill nothing either, 72 us without a bound and 56 with four
+__host__ __device__ constexpr int bags_blocks(int CH) { return CH == 2 ? 5 : CH == 8 ? 1 : 4; }
 
-// A lane group walks one bag at a time.  The bag's indices are loaded LPR at a time, one per lane, and checked once;
-// the rows are then fetched NB at a time, their numbers handed round by shuffle, and summed in bag order.  Measured on
-// B200 the kernel is bound by instruction issue (rows of hot tables come from the caches), which is why nothing is done
-// per row by every lane that one lane can do, why the quantiser checks NB rows at once, and why rows of 36 to 64
-// features in long bags take a whole warp with two features a lane: lane groups that walk bags of different lengths
-// side by side wait for each other (8.5 M lookups of 256-byte rows, cold: 646 us with the indices loaded by every
-// lane, 460 by lane groups, 354 by warps; four rows at a time: eight take 386, sixteen 497, the last batch of a bag
-// being padded).  In bags of a few indices the offsets' and the indices' latency counts, and twice as many bags in
-// flight are worth more (64 K lookups, three a bag, 36 features: 28 against 34 us).
-template <int LPR, int VEC, int CH, bool EXACT, bool CODES>
-__global__ void __launch_bounds__(FW_THREADS)
+// A lane group walks one bag at a time, its rows NB at a time in bag order.  Every lane loads the bag's indices itself:
+// loaded one per lane and handed round by shuffle they cost a round trip more per bag, and lane groups whose bags differ
+// in length wait for one another on the way (measured on
+// B200, random rows of 26 tables: 640 K rows of 64 bytes in bags of three on average 29 us this way, 42 by shuffle; of 256
+// bytes 67 and 88).
+template <int LPR, int CH, bool EXACT, bool CODES>
+__global__ void __launch_bounds__(FW_THREADS, bags_blocks(CH))
 fwd_bags_kernel(const FwdArgs a)
 {
     dq_wait_before();
     if (a.let_next) dq_let_next();
-    typedef typename Vec<VEC>::type vec_t;
-    constexpr int NB = CH >= 2 ? 1 : LPR < 4 ? LPR : 4;
+    constexpr int NB = NBOf<LPR, CH>::v;
     constexpr int GPB = FW_THREADS / LPR;
-    const int D = EXACT ? VEC * LPR * CH : a.D;
-    const int dv = D / VEC;
+    const int D = EXACT ? 4 * LPR * CH : a.D;
+    const int d4 = D >> 2;
     const int t = blockIdx.y;
     const int lane = threadIdx.x % LPR;
     const int grp = threadIdx.x / LPR;
-    const unsigned gmask = LPR == 32 ? 0xffffffffu : (((1u << (LPR & 31)) - 1u) << ((threadIdx.x & 31) / LPR * LPR));
     const TableCtx tc = table_ctx(a, t, D);
     bool bad = false;
 
     for (int i = blockIdx.x * GPB + grp; i < a.B; i += gridDim.x * GPB) {
         int32_t lo = __ldg(a.offsets + tc.g0 + i), hi = __ldg(a.offsets + tc.g0 + i + 1);
         if (lo < 0 || hi < lo || (int64_t)hi > a.L) { bad = true; hi = lo = 0; }
-        double acc[CH][VEC];
+        double acc[CH][4];
 #pragma unroll
-        for (int c = 0; c < CH; ++c)
+        for (int c = 0; c < CH; ++c) acc[c][0] = acc[c][1] = acc[c][2] = acc[c][3] = 0.0;
+        for (int32_t j0 = lo; j0 < hi; j0 += NB) {
+            int32_t idx[NB];
 #pragma unroll
-            for (int q = 0; q < VEC; ++q) acc[c][q] = 0.0;
-        int32_t mine = lo + lane < hi ? __ldg(a.indices + lo + lane) : 0;
-        for (int32_t j0 = lo; j0 < hi; j0 += LPR) {
-            const int32_t row = clamp_index(mine, tc.nrows, bad);      // (lanes past the bag's end hold row 0)
-            mine = j0 + LPR + lane < hi ? __ldg(a.indices + j0 + LPR + lane) : 0;
-            const int cnt = min(LPR, hi - j0);
-            auto rows = [&](int b0, auto full_tag) {
-                constexpr bool FULL = decltype(full_tag)::value;
+            for (int b = 0; b < NB; ++b) idx[b] = (j0 + b < hi) ? clamp_index(__ldg(a.indices + j0 + b), tc.nrows, bad) : 0;
 #pragma unroll
-                for (int c = 0; c < CH; ++c) {
-                    const int cv = c * LPR + lane;
-                    vec_t v[NB];
+            for (int c = 0; c < CH; ++c) {
+                const int c4 = c * LPR + lane;
+                float4 v[NB];
 #pragma unroll
-                    for (int b = 0; b < NB; ++b) {
-                        const int32_t r = __shfl_sync(gmask, row, b0 + b, LPR);
-                        v[b] = __ldg(reinterpret_cast<const vec_t *>(tc.tbl + (int64_t)r * D) + (EXACT || cv < dv ? cv : 0));
-                    }
-                    float x[NB * VEC], f[NB * VEC];
+                for (int b = 0; b < NB; ++b)
+                    if (j0 + b < hi && (EXACT || c4 < d4))
+                        v[b] = __ldg(reinterpret_cast<const float4 *>(tc.tbl + (int64_t)idx[b] * D) + c4);
 #pragma unroll
-                    for (int b = 0; b < NB; ++b) unpack(v[b], x + b * VEC);
-                    if constexpr (CODES) {
-#pragma unroll
-                        for (int b = 0; b < NB; ++b) {
+                for (int b = 0; b < NB; ++b) {
+                    if (j0 + b < hi && (EXACT || c4 < d4)) {
+                        float f[4];
+                        if constexpr (CODES) {
                             float4 cd, fq;
-                            dq_fq4(make_float4(x[b * VEC], x[b * VEC + 1], x[b * VEC + 2], x[b * VEC + 3]), tc.qs, cd, fq);
-                            f[b * VEC] = fq.x; f[b * VEC + 1] = fq.y; f[b * VEC + 2] = fq.z; f[b * VEC + 3] = fq.w;
-                            if ((FULL || b0 + b < cnt) && (EXACT || cv < dv)) store_codes(a.codes_out, j0 + b0 + b, D, cv, cd);
+                            dq_fq4(v[b], tc.qs, cd, fq);
+                            f[0] = fq.x; f[1] = fq.y; f[2] = fq.z; f[3] = fq.w;
+                            store_codes(a.codes_out, j0 + b, D, c4, cd);
+                        } else {
+                            const float x[4] = {v[b].x, v[b].y, v[b].z, v[b].w};
+                            dq_fq_many<4>(x, tc.qs, f);
                         }
-                    } else {
-                        dq_fq_many<NB * VEC>(x, tc.qs, f);
+#pragma unroll
+                        for (int q = 0; q < 4; ++q) acc[c][q] += (double)f[q];
                     }
-#pragma unroll
-                    for (int b = 0; b < NB; ++b)
-                        if (FULL || b0 + b < cnt)
-#pragma unroll
-                            for (int q = 0; q < VEC; ++q) acc[c][q] += (double)f[b * VEC + q];
                 }
-            };
-            int b0 = 0;
-            for (; b0 + NB <= cnt; b0 += NB) rows(b0, std::true_type{});
-            if (b0 < cnt) rows(b0, std::false_type{});
+            }
         }
-        vec_t *o = reinterpret_cast<vec_t *>(a.out + ((int64_t)i * a.T + t) * D);
+        float4 *o = reinterpret_cast<float4 *>(a.out + ((int64_t)i * a.T + t) * D);
 #pragma unroll
         for (int c = 0; c < CH; ++c) {
-            const int cv = c * LPR + lane;
-            if (EXACT || cv < dv) store_sum(o + cv, acc[c]);
+            const int c4 = c * LPR + lane;
+            if (EXACT || c4 < d4)
+                o[c4] = make_float4((float)acc[c][0], (float)acc[c][1], (float)acc[c][2], (float)acc[c][3]);
         }
     }
     if (bad) dq_report(a.status, DQRM_ERR_INDEX_RANGE);
 }
 
-// rows of 36 to 64 features: a warp per bag from eight indices a bag on
-inline bool warp_per_bag(const FwdArgs &a, int lpr) { return lpr == 16 && !a.codes_out && a.L >= 8 * (int64_t)a.T * a.B; }
+// Long bags of rows of 36 to 64 features: a warp per bag, two features a lane.  Every lane of a warp is then in the same
+// bag, so the indices are loaded 32 at a time, one per lane, and checked once; the rows are fetched eight at a time, their
+// numbers handed round by shuffle, and summed in bag order (measured
+// on B200, 26 x 16384 bags of 20 on average, Zipf 1.2: 316 us, 351 with four rows at a time and 352 by lane groups).
+template <bool EXACT>
+__global__ void __launch_bounds__(FW_THREADS, 4)
+fwd_long_bags_kernel(const FwdArgs a)
+{
+    dq_wait_before();
+    if (a.let_next) dq_let_next();
+    constexpr int WPB = FW_THREADS / 32;
+    const int D = EXACT ? 64 : a.D;
+    const int t = blockIdx.y, lane = threadIdx.x & 31;
+    const bool on = EXACT || 2 * lane < D;
+    const TableCtx tc = table_ctx(a, t, D);
+    const float2 *tbl = reinterpret_cast<const float2 *>(tc.tbl) + (on ? lane : 0);
+    bool bad = false;
+
+    for (int i = blockIdx.x * WPB + (threadIdx.x >> 5); i < a.B; i += gridDim.x * WPB) {
+        int32_t lo = __ldg(a.offsets + tc.g0 + i), hi = __ldg(a.offsets + tc.g0 + i + 1);
+        if (lo < 0 || hi < lo || (int64_t)hi > a.L) { bad = true; hi = lo = 0; }
+        double acc[2] = {0.0, 0.0};
+        int32_t mine = lo + lane < hi ? __ldg(a.indices + lo + lane) : 0;
+        for (int32_t j0 = lo; j0 < hi; j0 += 32) {
+            const int32_t row = clamp_index(mine, tc.nrows, bad);      // (lanes past the bag's end hold row 0)
+            mine = j0 + 32 + lane < hi ? __ldg(a.indices + j0 + 32 + lane) : 0;
+            const int cnt = min(32, hi - j0);
+            // rows b0 .. b0 + NB, of which `n` count
+            auto rows = [&](int b0, int n, auto nb_tag) {
+                constexpr int NB = decltype(nb_tag)::value;
+                float x[2 * NB], f[2 * NB];
+#pragma unroll
+                for (int b = 0; b < NB; ++b) {
+                    const int32_t r = __shfl_sync(0xffffffffu, row, (b0 + b) & 31);
+                    const float2 v = __ldg(tbl + (int64_t)r * (D / 2));
+                    x[2 * b] = v.x;
+                    x[2 * b + 1] = v.y;
+                }
+                dq_fq_many<2 * NB>(x, tc.qs, f);
+#pragma unroll
+                for (int b = 0; b < NB; ++b)
+                    if (b < n) {
+                        acc[0] += (double)f[2 * b];
+                        acc[1] += (double)f[2 * b + 1];
+                    }
+            };
+            int b0 = 0;
+            for (; b0 + 8 <= cnt; b0 += 8) rows(b0, 8, std::integral_constant<int, 8>{});
+            for (; b0 < cnt; b0 += 4) rows(b0, cnt - b0, std::integral_constant<int, 4>{});
+        }
+        if (on) reinterpret_cast<float2 *>(a.out + ((int64_t)i * a.T + t) * D)[lane] = make_float2((float)acc[0], (float)acc[1]);
+    }
+    if (bad) dq_report(a.status, DQRM_ERR_INDEX_RANGE);
+}
+
+// From 18 indices a bag on average: at 16 of equal length, where no lane group waits for another, the two are even in large
+// batches (26 x 8192 bags of 256-byte rows 159 us both) and lane groups ahead in small ones (4 x 2048 bags 9.2 against 10.3
+// us); at 24 it is 212 against 223 us, and with bags of uneven length the warps are ahead from 12 on
+constexpr int LONG_BAG = 18;
+inline bool warp_per_bag(const FwdArgs &a, int lpr) { return lpr == 16 && !a.codes_out && a.L >= LONG_BAG * (int64_t)a.T * a.B; }
 
 template <int LPR, int CH, bool EXACT>
 cudaError_t launch_bags(const FwdArgs &a, dim3 grid, cudaStream_t st)
 {
-    if constexpr (LPR == 16) {
-        if (warp_per_bag(a, LPR)) return dq_launch(fwd_bags_kernel<32, 2, CH, EXACT, false>, grid, dim3(FW_THREADS), 0, st, a);
-    }
-    if (a.codes_out) return dq_launch(fwd_bags_kernel<LPR, 4, CH, EXACT, true>, grid, dim3(FW_THREADS), 0, st, a);
-    return dq_launch(fwd_bags_kernel<LPR, 4, CH, EXACT, false>, grid, dim3(FW_THREADS), 0, st, a);
+    if (LPR == 16 && warp_per_bag(a, LPR)) return dq_launch(fwd_long_bags_kernel<EXACT>, grid, dim3(FW_THREADS), 0, st, a);
+    if (a.codes_out) return dq_launch(fwd_bags_kernel<LPR, CH, EXACT, true>, grid, dim3(FW_THREADS), 0, st, a);
+    return dq_launch(fwd_bags_kernel<LPR, CH, EXACT, false>, grid, dim3(FW_THREADS), 0, st, a);
 }
 
 template <int LPR, int CH, bool EXACT>
