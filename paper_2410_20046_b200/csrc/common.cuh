@@ -244,6 +244,29 @@ __device__ __forceinline__ void dq_fq_many(const float (&x)[N], const QuantScale
     }
 }
 
+// Dequantised values of four elements, and their codes as the bytes of a word (a code added to 1.5*2^23 stands in the low
+// bits of the sum: no conversion instruction)
+__device__ __forceinline__ u32 dq_fq4_bytes(const float (&x)[4], const QuantScale &q, float (&deq)[4])
+{
+    const float2 ns2 = make_float2(-q.s, -q.s), los2 = make_float2(q.lo * q.s, q.lo * q.s);
+    float dist = q.fast ? 0.f : 1.f;
+    const float2 ma = dq_codes2(make_float2(x[0], x[1]), q, dist), mb = dq_codes2(make_float2(x[2], x[3]), q, dist);
+    const float2 ea = __ffma2_rn(ma, ns2, los2), eb = __ffma2_rn(mb, ns2, los2);
+    deq[0] = ea.x; deq[1] = ea.y; deq[2] = eb.x; deq[3] = eb.y;
+    float c[4] = {__fsub_rn(q.lo, ma.x), __fsub_rn(q.lo, ma.y), __fsub_rn(q.lo, mb.x), __fsub_rn(q.lo, mb.y)};
+    if (!(dist < q.tie_lim)) {
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            c[k] = dq_codef_ieee(x[k], q);
+            deq[k] = __fmul_rn(c[k], q.s);
+        }
+    }
+    u32 w = 0;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) w |= (__float_as_uint(__fadd_rn(c[k], 12582912.0f)) & 0xffu) << (8 * k);
+    return w;
+}
+
 // asks L2 for the 128-byte line that holds p (no register, no scoreboard entry: the later load finds it there)
 __device__ __forceinline__ void dq_prefetch_l2(const void *p) { asm volatile("prefetch.global.L2 [%0];\n" ::"l"(p)); }
 

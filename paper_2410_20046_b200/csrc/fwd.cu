@@ -257,16 +257,12 @@ fwd_bags_kernel(const FwdArgs a)
 #pragma unroll
                 for (int b = 0; b < NB; ++b) {
                     if (j0 + b < hi && (EXACT || c4 < d4)) {
+                        const float x[4] = {v[b].x, v[b].y, v[b].z, v[b].w};
                         float f[4];
-                        if constexpr (CODES) {
-                            float4 cd, fq;
-                            dq_fq4(v[b], tc.qs, cd, fq);
-                            f[0] = fq.x; f[1] = fq.y; f[2] = fq.z; f[3] = fq.w;
-                            store_codes(a.codes_out, j0 + b, D, c4, cd);
-                        } else {
-                            const float x[4] = {v[b].x, v[b].y, v[b].z, v[b].w};
+                        if constexpr (CODES)
+                            *reinterpret_cast<u32 *>(a.codes_out + (int64_t)(j0 + b) * D + 4 * c4) = dq_fq4_bytes(x, tc.qs, f);
+                        else
                             dq_fq_many<4>(x, tc.qs, f);
-                        }
 #pragma unroll
                         for (int q = 0; q < 4; ++q) acc[c][q] += (double)f[q];
                     }
