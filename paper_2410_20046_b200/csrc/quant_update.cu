@@ -8,6 +8,7 @@
 // A group of LPR lanes owns a contiguous range of unique rows and keeps a few of them in flight;
 // rows are distinct, so the read-modify-write of the master rows needs no atomics.  All
 // streams are 128-bit per lane.
+#include <algorithm>
 #include <cooperative_groups.h>
 #include <mutex>
 #include "common.cuh"
@@ -88,13 +89,66 @@ int launch_absmax(dqrm_ctx *ctx, const float *grad_rows, const int32_t *uniq_off
 // blocks are too few for what they do not hold); seven tables of 512 K 10.2 / 13.2.  256 threads a block while that
 // holds a table (40 tables of 64 K values take 5.2 us with 256 and 8.4 with 512: a second wave), 512 then, and 1024
 // where the tables are few and do not fill the chip with 512 (seven of 256 K: 5.8 us, 8.0 with 512).
+//
+// How the values spread over the tables is not known before the launch, and one table may hold nearly all of them.  A
+// table beyond `limit` vectors, twice what its cluster holds, is therefore left by its cluster to all: its abs-max is found
+// by every block that is there (one partial a block), and a second launch, made only when max_values allows such a table,
+// quantises it with the whole chip.  Measured on B200 (us; this way / its cluster alone / three launches), 26 tables of which
+// one has 61 K rows of 64 values and the others 1024: 18.5 / 103 / 18.6; 2048 rows of 64 in every table 7.4 / 6.0 / 18.3, the
+// second launch having nothing to do; all rows, 4096 of 64, in one of 26 tables 12.3 / 14.8 / 10.4.
 constexpr int QC_VEC = 8;             // vectors of four that a thread holds
 constexpr int QC_CLUSTER = 8;
+constexpr int QH_THREADS = 512;
+
+struct Heavy {
+    int64_t limit;                    // vectors of a table that its cluster takes itself
+    u32 *partial;                     // [T][blocks] abs-max that a block found in a table beyond it; null: there can be none
+    int blocks;                       // blocks that look for it
+};
+
+__device__ __forceinline__ int64_t table_vectors(const int32_t *uniq_off, int t, int d4)
+{
+    return max((int64_t)__ldg(uniq_off + t + 1) - __ldg(uniq_off + t), (int64_t)0) * d4;
+}
+
+// whether a table is beyond the limit (the same answer in every thread of the block)
+__device__ __forceinline__ bool any_heavy(const int32_t *uniq_off, int T, int d4, int64_t limit)
+{
+    bool any = false;
+    for (int t = threadIdx.x; t < T; t += blockDim.x) any |= table_vectors(uniq_off, t, d4) > limit;
+    return __syncthreads_or(any);
+}
+
+__device__ __forceinline__ float abs_max4(const float4 &v)
+{
+    return fmaxf(fmaxf(fabsf(v.x), fabsf(v.y)), fmaxf(fabsf(v.z), fabsf(v.w)));
+}
+
+// abs-max over the block, in thread 0 (non-negative floats order as their bits)
+template <int THREADS>
+__device__ __forceinline__ float block_max(float m, float *s_warp)
+{
+    const u32 wm = __reduce_max_sync(0xffffffffu, __float_as_uint(m));
+    __syncthreads();                                   // (s_warp may still be read)
+    if (threadIdx.x % 32 == 0) s_warp[threadIdx.x / 32] = __uint_as_float(wm);
+    __syncthreads();
+    float b = 0.f;
+    if (threadIdx.x == 0)
+        for (int w = 0; w < THREADS / 32; ++w) b = fmaxf(b, s_warp[w]);
+    return b;
+}
+
+__device__ __forceinline__ void put_codes(char4 *c, const float4 &v, const QuantScale &qs)
+{
+    float4 q, unused;
+    dq_fq4(v, qs, q, unused);
+    __stcs(c, make_char4((signed char)(int)q.x, (signed char)(int)q.y, (signed char)(int)q.z, (signed char)(int)q.w));
+}
 
 template <int QC_THREADS>
 __global__ void __launch_bounds__(QC_THREADS, 1024 / QC_THREADS)
-quant_table_kernel(const float4 *__restrict__ grad_rows, const int32_t *__restrict__ uniq_off, int d4,
-                   char4 *__restrict__ codes, float *__restrict__ grad_scales)
+quant_table_kernel(const float4 *__restrict__ grad_rows, const int32_t *__restrict__ uniq_off, int T, int d4,
+                   char4 *__restrict__ codes, float *__restrict__ grad_scales, const Heavy heavy)
 {
     namespace cg = cooperative_groups;
     cg::cluster_group cluster = cg::this_cluster();
@@ -102,67 +156,132 @@ quant_table_kernel(const float4 *__restrict__ grad_rows, const int32_t *__restri
     const int rank = (int)cluster.block_rank(), blocks = (int)cluster.num_blocks(), t = (int)blockIdx.x / blocks;
     auto started = cluster.barrier_arrive();           // (shared memory of a block that has not begun is out of reach)
     dq_wait_before();
-    const int64_t first = __ldg(uniq_off + t), rows = max((int64_t)__ldg(uniq_off + t + 1) - first, (int64_t)0);
-    const int64_t n = rows * d4, stride = (int64_t)blocks * QC_THREADS;
-    const float4 *g = grad_rows + first * d4;
-    char4 *c = codes + first * d4;
-    const int64_t i0 = (int64_t)rank * QC_THREADS + threadIdx.x;
-    float4 x[QC_VEC];
-    float m = 0.f;
+    const int64_t n = t < T ? table_vectors(uniq_off, t, d4) : 0;
+    if (t < T && n <= heavy.limit) {                   // (the same in the whole cluster)
+        const int64_t first = __ldg(uniq_off + t), stride = (int64_t)blocks * QC_THREADS;
+        const float4 *g = grad_rows + first * d4;
+        char4 *c = codes + first * d4;
+        const int64_t i0 = (int64_t)rank * QC_THREADS + threadIdx.x;
+        float4 x[QC_VEC];
+        float m = 0.f;
 #pragma unroll
-    for (int k = 0; k < QC_VEC; ++k) {
-        x[k] = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (i0 + k * stride < n) x[k] = __ldg(g + i0 + k * stride);
+        for (int k = 0; k < QC_VEC; ++k) {
+            x[k] = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (i0 + k * stride < n) x[k] = __ldg(g + i0 + k * stride);
+        }
+#pragma unroll
+        for (int k = 0; k < QC_VEC; ++k) m = fmaxf(m, abs_max4(x[k]));
+        for (int64_t i = i0 + QC_VEC * stride; i < n; i += stride) m = fmaxf(m, abs_max4(__ldg(g + i)));
+        const u32 wm = __reduce_max_sync(0xffffffffu, __float_as_uint(m));
+        if (threadIdx.x % 32 == 0) s_warp[threadIdx.x / 32] = __uint_as_float(wm);
+        __syncthreads();
+        cluster.barrier_wait(std::move(started));
+        if (threadIdx.x < (unsigned)blocks) {
+            float b = 0.f;
+#pragma unroll
+            for (int w = 0; w < QC_THREADS / 32; ++w) b = fmaxf(b, s_warp[w]);
+            cluster.map_shared_rank(s_block, threadIdx.x)[rank] = b;
+        }
+        cluster.sync();
+        m = 0.f;
+        for (int b = 0; b < blocks; ++b) m = fmaxf(m, s_block[b]);
+        const float s = dq_scale_from_absmax(m, 8);
+        if (rank == 0 && threadIdx.x == 0) grad_scales[t] = s;
+        const QuantScale qs = dq_make_scale(s, 8);
+#pragma unroll
+        for (int k = 0; k < QC_VEC; ++k)
+            if (i0 + k * stride < n) put_codes(c + i0 + k * stride, x[k], qs);
+        for (int64_t i = i0 + QC_VEC * stride; i < n; i += stride) put_codes(c + i, __ldg(g + i), qs);
+    } else {
+        cluster.barrier_wait(std::move(started));
     }
+    if (heavy.partial == nullptr || (int)blockIdx.x >= heavy.blocks || !any_heavy(uniq_off, T, d4, heavy.limit)) return;
+    for (int h = 0; h < T; ++h) {
+        const int64_t nh = table_vectors(uniq_off, h, d4), stride = (int64_t)heavy.blocks * QC_THREADS;
+        if (nh <= heavy.limit) continue;
+        const float4 *g = grad_rows + (int64_t)__ldg(uniq_off + h) * d4;
+        float m = 0.f;
+        for (int64_t i = (int64_t)blockIdx.x * QC_THREADS + threadIdx.x; i < nh; i += 4 * stride) {
+            float4 x[4];
 #pragma unroll
-    for (int k = 0; k < QC_VEC; ++k)
-        m = fmaxf(m, fmaxf(fmaxf(fabsf(x[k].x), fabsf(x[k].y)), fmaxf(fabsf(x[k].z), fabsf(x[k].w))));
-    for (int64_t i = i0 + QC_VEC * stride; i < n; i += stride) {
-        const float4 y = __ldg(g + i);
-        m = fmaxf(m, fmaxf(fmaxf(fabsf(y.x), fabsf(y.y)), fmaxf(fabsf(y.z), fabsf(y.w))));
+            for (int k = 0; k < 4; ++k) x[k] = __ldg(g + min(i + k * stride, nh - 1));
+#pragma unroll
+            for (int k = 0; k < 4; ++k) m = fmaxf(m, abs_max4(x[k]));
+        }
+        m = block_max<QC_THREADS>(m, s_warp);
+        if (threadIdx.x == 0) heavy.partial[(size_t)h * heavy.blocks + blockIdx.x] = __float_as_uint(m);
     }
-    const u32 wm = __reduce_max_sync(0xffffffffu, __float_as_uint(m));      // (non-negative floats order as their bits)
-    if (threadIdx.x % 32 == 0) s_warp[threadIdx.x / 32] = __uint_as_float(wm);
-    __syncthreads();
-    cluster.barrier_wait(std::move(started));
-    if (threadIdx.x < (unsigned)blocks) {
-        float b = 0.f;
-#pragma unroll
-        for (int w = 0; w < QC_THREADS / 32; ++w) b = fmaxf(b, s_warp[w]);
-        cluster.map_shared_rank(s_block, threadIdx.x)[rank] = b;
-    }
-    cluster.sync();
-    m = 0.f;
-    for (int b = 0; b < blocks; ++b) m = fmaxf(m, s_block[b]);
-    const float s = dq_scale_from_absmax(m, 8);
-    if (rank == 0 && threadIdx.x == 0) grad_scales[t] = s;
-    const QuantScale qs = dq_make_scale(s, 8);
-    auto put = [&](int64_t i, const float4 &v) {
-        float4 q, unused;
-        dq_fq4(v, qs, q, unused);
-        __stcs(c + i, make_char4((signed char)(int)q.x, (signed char)(int)q.y, (signed char)(int)q.z, (signed char)(int)q.w));
-    };
-#pragma unroll
-    for (int k = 0; k < QC_VEC; ++k)
-        if (i0 + k * stride < n) put(i0 + k * stride, x[k]);
-    for (int64_t i = i0 + QC_VEC * stride; i < n; i += stride) put(i, __ldg(g + i));
 }
 
-// whether a batch of up to max_vectors goes through the kernel above
+// the tables that the kernel above has left, by the whole grid
+__global__ void __launch_bounds__(QH_THREADS)
+quant_heavy_kernel(const float4 *__restrict__ grad_rows, const int32_t *__restrict__ uniq_off, int T, int d4,
+                   char4 *__restrict__ codes, float *__restrict__ grad_scales, const Heavy heavy)
+{
+    dq_wait_before();
+    __shared__ u32 s_max;
+    if (!any_heavy(uniq_off, T, d4, heavy.limit)) return;
+    for (int h = 0; h < T; ++h) {
+        const int64_t nh = table_vectors(uniq_off, h, d4), stride = (int64_t)gridDim.x * QH_THREADS;
+        if (nh <= heavy.limit) continue;
+        __syncthreads();                               // (the maximum of the table before has been read)
+        if (threadIdx.x == 0) s_max = 0u;
+        __syncthreads();
+        u32 m = 0u;
+        for (int b = threadIdx.x; b < heavy.blocks; b += QH_THREADS) m = max(m, heavy.partial[(size_t)h * heavy.blocks + b]);
+        m = __reduce_max_sync(0xffffffffu, m);
+        if (threadIdx.x % 32 == 0 && m) atomicMax(&s_max, m);
+        __syncthreads();
+        const float s = dq_scale_from_absmax(__uint_as_float(s_max), 8);
+        if (blockIdx.x == 0 && threadIdx.x == 0) grad_scales[h] = s;
+        const QuantScale qs = dq_make_scale(s, 8);
+        const int64_t first = (int64_t)__ldg(uniq_off + h) * d4;
+        for (int64_t i = (int64_t)blockIdx.x * QH_THREADS + threadIdx.x; i < nh; i += 4 * stride) {
+            float4 x[4];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) x[k] = __ldg(grad_rows + first + min(i + k * stride, nh - 1));
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+                if (i + k * stride < nh) put_codes(codes + first + i + k * stride, x[k], qs);
+        }
+    }
+}
+
+constexpr int64_t cluster_holds(int threads) { return (int64_t)QC_CLUSTER * threads * QC_VEC; }
+
+// whether a batch of up to max_vectors goes through the kernels above.  With few tables up to what the cluster of one holds:
+// beyond it three launches are faster for that one (three tables, one of 128 K vectors: 11.8 us here)
 inline bool quant_by_table(const dqrm_ctx *ctx, int64_t max_vectors)
 {
-    const int64_t held = (int64_t)ctx->T * QC_CLUSTER * 1024 * QC_VEC;
-    return max_vectors <= (ctx->T >= 6 ? 2 * held : held);
+    return max_vectors <= (ctx->T >= 6 ? 2 * ctx->T * cluster_holds(1024) : cluster_holds(1024));
 }
 
 template <int QC_THREADS>
 int launch_quant_table(dqrm_ctx *ctx, const float *grad_rows, const int32_t *uniq_off, int8_t *codes, float *grad_scales,
-                       int64_t per_table, cudaStream_t st)
+                       int64_t max_vectors, u32 *ws, size_t ws_bytes, cudaStream_t st, bool &taken)
 {
+    const int64_t per_table = (max_vectors + ctx->T - 1) / ctx->T;
     unsigned blocks = 1;
     while (blocks < (unsigned)QC_CLUSTER && per_table > (int64_t)blocks * QC_THREADS * 2) blocks *= 2;
+    // more blocks where no table can then be beyond them: a second launch costs more than they do
+    const int64_t held = (int64_t)QC_THREADS * QC_VEC;
+    if (max_vectors <= 2 * QC_CLUSTER * held)
+        while (max_vectors > 2 * blocks * held) blocks *= 2;
+    Heavy heavy = {2 * blocks * held, nullptr, 0};
+    unsigned clusters = (unsigned)ctx->T;
+    if (max_vectors > heavy.limit) {
+        heavy.blocks = 4 * ctx->num_sms;
+        clusters = std::max(clusters, ((unsigned)ctx->num_sms + blocks - 1) / blocks);
+        heavy.blocks = std::min(heavy.blocks, (int)(clusters * blocks));
+        taken = ws_bytes >= sizeof(u32) * ctx->T * heavy.blocks;
+        if (!taken) return DQRM_OK;
+        heavy.partial = ws;
+    } else {
+        heavy.limit = INT64_MAX;       // (the bound may be wrong; the result must not be)
+        taken = true;
+    }
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)ctx->T * blocks);
+    cfg.gridDim = dim3(clusters * blocks);
     cfg.blockDim = dim3(QC_THREADS);
     cfg.stream = st;
     cudaLaunchAttribute attr[2];
@@ -172,9 +291,14 @@ int launch_quant_table(dqrm_ctx *ctx, const float *grad_rows, const int32_t *uni
     attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 2;
-    DQRM_CUDA_TRY(ctx, cudaLaunchKernelEx(&cfg, quant_table_kernel<QC_THREADS>, reinterpret_cast<const float4 *>(grad_rows), uniq_off,
-                                          ctx->D / 4, reinterpret_cast<char4 *>(codes), grad_scales));
-    dq_mark(ctx, st, DQ_K_QUANT);
+    const float4 *g = reinterpret_cast<const float4 *>(grad_rows);
+    char4 *c = reinterpret_cast<char4 *>(codes);
+    DQRM_CUDA_TRY(ctx, cudaLaunchKernelEx(&cfg, quant_table_kernel<QC_THREADS>, g, uniq_off, ctx->T, ctx->D / 4, c, grad_scales, heavy));
+    dq_mark(ctx, st, DQ_K_QUANT_TABLE);
+    if (heavy.partial == nullptr) return DQRM_OK;
+    DQRM_CUDA_TRY(ctx, dq_launch(quant_heavy_kernel, dim3(ctx->num_sms), dim3(QH_THREADS), 0, st, g, uniq_off, ctx->T, ctx->D / 4, c,
+                                 grad_scales, heavy));
+    dq_mark(ctx, st, DQ_K_QUANT_HEAVY);
     return DQRM_OK;
 }
 
@@ -248,12 +372,20 @@ int dq_launch_grad_quant(dqrm_ctx *ctx, const float *grad_rows, const int32_t *u
 {
     if (ws_bytes < dq_quant_ws_bytes(ctx)) return DQRM_ERR_WORKSPACE;
     if (quant_by_table(ctx, max_values / 4)) {
-        const int64_t per_table = (max_values / 4 + ctx->T - 1) / ctx->T;
-        if (per_table <= (int64_t)QC_CLUSTER * 256 * QC_VEC)
-            return launch_quant_table<256>(ctx, grad_rows, uniq_off, codes, grad_scales, per_table, st);
-        if (per_table > (int64_t)QC_CLUSTER * 512 * QC_VEC && ctx->T * QC_CLUSTER < ctx->num_sms)
-            return launch_quant_table<1024>(ctx, grad_rows, uniq_off, codes, grad_scales, per_table, st);
-        return launch_quant_table<512>(ctx, grad_rows, uniq_off, codes, grad_scales, per_table, st);
+        const int64_t most = max_values / 4, per_table = (most + ctx->T - 1) / ctx->T;
+        // threads a block: as many as the tables' mean needs; more where one table may then hold everything without being
+        // beyond its cluster, and the clusters still run at once (53 K vectors over 26 tables: 4.1 us with 512
+        // threads, 4.8 with 256 and the second launch)
+        int threads = per_table <= cluster_holds(256) ? 256
+                      : per_table > cluster_holds(512) && ctx->T * QC_CLUSTER < ctx->num_sms ? 1024 : 512;
+        for (int more = threads; more <= 1024 && ctx->T * QC_CLUSTER * more <= ctx->num_sms * 1024; more *= 2)
+            if (most <= 2 * cluster_holds(more)) { threads = more; break; }
+        u32 *w = reinterpret_cast<u32 *>(ws);
+        bool taken = false;            // (not with a workspace that has no room for the partial maxima)
+        const int rc = threads == 256    ? launch_quant_table<256>(ctx, grad_rows, uniq_off, codes, grad_scales, most, w, ws_bytes, st, taken)
+                       : threads == 512 ? launch_quant_table<512>(ctx, grad_rows, uniq_off, codes, grad_scales, most, w, ws_bytes, st, taken)
+                                        : launch_quant_table<1024>(ctx, grad_rows, uniq_off, codes, grad_scales, most, w, ws_bytes, st, taken);
+        if (rc != DQRM_OK || taken) return rc;
     }
     u32 *absmax = reinterpret_cast<u32 *>(ws);
     const int rc = launch_absmax(ctx, grad_rows, uniq_off, absmax, st);

@@ -20,6 +20,10 @@ SHAPES = {
     (16, "larger than the registers"): ([9000] * 10 + [0, 200] * 5, None),
     (64, "blocks of 1024"): ([4096, 2050, 0, 1], None),
     (16, "large buffers"): ([128, 0, 700], 300_000),
+    # tables beyond what their cluster takes, which all blocks share
+    (64, "one of many shared"): ([0, 30_000, 1, 0, 3] + [40] * 21, None), (36, "two shared"): ([20_000, 7, 0, 20_000] + [9] * 22, None),
+    (16, "few tables, one shared"): ([40_000, 1, 0], None), (64, "just not shared"): ([0, 2048, 0, 0, 0, 0, 0, 0], None),
+    (64, "just shared"): ([0, 2049, 0, 0, 0, 0, 0, 0], None), (20, "last one shared"): ([1] * 150 + [9_000], None),
 }
 
 
@@ -43,4 +47,26 @@ def test_quant_table(oracle, shape):
     codes = d_codes.cpu().numpy()
     assert bit_equal(gs.cpu().numpy(), o_gs) and bit_equal(codes[:len(gr)], o_codes)
     assert (codes[len(gr):] == 99).all()
+    c.ctx.close()
+
+
+@pytest.mark.parametrize("rows,most", [([0, 30_000, 1, 0, 3] + [40] * 21, None), ([0, 30_000, 1, 0, 3] + [40] * 21, 64),
+                                       ([128, 3], 0), ([128, 3], 1 << 40)])
+def test_neither_the_bound_nor_the_workspace_changes_the_result(oracle, rows, most):
+    """A bound that is too small or too large, and a workspace of the least size that was ever asked for."""
+    D = 64
+    wl = W.Workload("quant", (100_000,) * len(rows), D=D, B=4, alpha=None)
+    rng = np.random.default_rng(len(rows))
+    uo = np.concatenate([[0], np.cumsum(rows)]).astype(np.int32)
+    gr = rng.standard_normal((int(uo[-1]), D)).astype(np.float32)
+    o_codes, o_gs = oracle.grad_quant_int8(gr, uo, D)
+    c = Case(wl, max_lookups=len(gr))
+    t = c.torch
+    d_gr, d_uo, codes, gs = c.dev(gr), c.dev(uo), c.empty((len(gr), D), t.int8), c.empty(wl.T, t.float32)
+    for room in (256, c.ctx.scratch_bytes):
+        codes.fill_(99)
+        assert c.ctx.lib.dqrm_grad_quant_int8_bounded(
+            c.ctx._h, d_gr.data_ptr(), d_uo.data_ptr(), codes.data_ptr(), gs.data_ptr(), gr.size if most is None else most,
+            c.ctx._scratch_ptr, room, t.cuda.current_stream().cuda_stream) == 0
+        assert bit_equal(gs.cpu().numpy(), o_gs) and bit_equal(codes.cpu().numpy(), o_codes)
     c.ctx.close()
