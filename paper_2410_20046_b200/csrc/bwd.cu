@@ -239,14 +239,21 @@ int launch_sum(dqrm_ctx *ctx, const segred::Args &a, bool small, cudaStream_t st
     using namespace segred;
     const size_t smem = smem_bytes(ctx->T);
     const int64_t ranges = (a.num_tiles + a.range_tiles - 1) / a.range_tiles;
-    const dim3 grid((unsigned)((ranges + WARPS - 1) / WARPS), (unsigned)column_blocks(ctx->D));
-    const bool exact = ctx->D == LPR * VEC;
-#define DQ_SUM(EXACT, SMALL) DQRM_CUDA_TRY(ctx, (dq_launch(seg_sum_kernel<LPR, VEC, EXACT, SMALL>, grid, dim3(THREADS), smem, st, a)))
-    if (LPR == 32 && small) {
-        if (exact) DQ_SUM(true, LPR == 32); else DQ_SUM(false, LPR == 32);
-    } else {
-        if (exact) DQ_SUM(true, false); else DQ_SUM(false, false);
-    }
+    const dim3 grid((unsigned)((ranges * a.columns + WARPS - 1) / WARPS));
+    const bool exact = ctx->D % (LPR * VEC) == 0;
+    constexpr bool wide = LPR == 32 && VEC == 4;             // (only those rows may have several blocks of features)
+#define DQ_SUM(EXACT, SMALL, COLS) \
+    DQRM_CUDA_TRY(ctx, (dq_launch(seg_sum_kernel<LPR, VEC, EXACT, SMALL, COLS>, grid, dim3(THREADS), smem, st, a)))
+#define DQ_SUM2(SMALL)                                                              \
+    do {                                                                            \
+        if (a.columns > 1 && exact) DQ_SUM(true, SMALL, wide);                      \
+        else if (a.columns > 1) DQ_SUM(false, SMALL, wide);                         \
+        else if (exact) DQ_SUM(true, SMALL, false);                                 \
+        else DQ_SUM(false, SMALL, false);                                           \
+    } while (0)
+    if (LPR == 32 && small) DQ_SUM2(LPR == 32);
+    else DQ_SUM2(false);
+#undef DQ_SUM2
 #undef DQ_SUM
     dq_mark(ctx, st, DQ_K_SEG_SUM);
     return DQRM_OK;
@@ -484,6 +491,7 @@ int dq_launch_bwd_sum(dqrm_ctx *ctx, const float *grad_out, int32_t *unique_rows
     if (L == 0) return DQRM_OK;
     char *ws = reinterpret_cast<char *>(ws_);
     segred::Args a = {};
+    const int D = ctx->D;
     // both sort paths leave the sorted pairs in the first key / payload buffers
     a.keys = reinterpret_cast<const u32 *>(ws + y.keys_a);
     a.vals = reinterpret_cast<const u32 *>(ws + y.vals_a);
@@ -502,8 +510,8 @@ int dq_launch_bwd_sum(dqrm_ctx *ctx, const float *grad_out, int32_t *unique_rows
     a.T = ctx->T; a.D = ctx->D;
     a.L = L; a.G = (int64_t)ctx->T * B; a.num_tiles = y.sum_tiles;
     a.range_tiles = y.range_tiles;
+    a.columns = segred::column_blocks(D);
     a.status = ctx->d_status;
-    const int D = ctx->D;
     if (D <= 4) return launch_sum<4, 1>(ctx, a, y.sum_small, st);
     if (D <= 8) return launch_sum<4, 2>(ctx, a, y.sum_small, st);
     if (D <= 16) return launch_sum<4, 4>(ctx, a, y.sum_small, st);

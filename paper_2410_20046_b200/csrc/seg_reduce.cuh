@@ -70,6 +70,7 @@ struct Args {
     int T, D;
     int64_t L, G, num_tiles;
     int range_tiles;            // tiles per warp
+    int columns;                // blocks of 128 features
     int *status;
 };
 
@@ -147,8 +148,10 @@ __device__ __noinline__ void note_max(u32 *absmax, const u32 *s_uoff, int t_firs
     if (lane_w % LPR == 0 && m) atomicMax(absmax + last_not_above(s_uoff, t_first, T, u), m);
 }
 
-// blockIdx.x * WARPS + warp: range of tiles; blockIdx.y: block of 128 features (one unless D > 128)
-template <int LPR, int VEC, bool EXACT, bool SMALL>
+// blockIdx.x * WARPS + warp: range of tiles and block of 128 features (COLS: D > 128, there are several).  EXACT: every lane
+// holds features.  Rows of 3 KB and more are not asked into L2 ahead: their blocks of features ask for whole rows already
+// (65 K rows of 4080 bytes 138 us, 154 with the request; of 2064 bytes 87 and 85)
+template <int LPR, int VEC, bool EXACT, bool SMALL, bool COLS>
 __global__ void __launch_bounds__(THREADS, blocks_per_sm(LPR))
 seg_sum_kernel(const Args a)
 {
@@ -165,12 +168,14 @@ seg_sum_kernel(const Args a)
     u32 *s_row = s_tb + (a.T + 1);                                                       // [T+1] (by table)
     __shared__ u32 s_broken;
 
-    const int T = a.T, D = EXACT ? LPR * VEC : a.D, dv = D / VEC;
+    const int T = a.T, D = EXACT && !COLS ? LPR * VEC : a.D, dv = D / VEC;
     const int wl = threadIdx.x & 31, lane = wl % LPR, grp = wl / LPR;
-    const int cv = (EXACT ? 0 : blockIdx.y * LPR) + lane;      // this lane's vector of the row
+    // the blocks of features of a range are neighbouring warps: a row's pieces are asked for at about the same time
+    const u32 cols = COLS ? (u32)a.columns : 1u, slot = blockIdx.x * WARPS + (threadIdx.x >> 5);
+    const u32 col = COLS ? slot % cols : 0u, range = COLS ? slot / cols : slot;
+    const int cv = (int)col * LPR + lane;      // this lane's vector of the row
     const bool on = EXACT || cv < dv;
-    const bool first_col = EXACT || blockIdx.y == 0;
-    const u32 range = blockIdx.x * WARPS + (threadIdx.x >> 5);
+    const bool first_col = col == 0u;
     const u32 tile0 = min((u32)a.num_tiles, range * (u32)a.range_tiles);
     const u32 tile1 = min((u32)a.num_tiles, tile0 + (u32)a.range_tiles);
 
@@ -227,7 +232,7 @@ seg_sum_kernel(const Args a)
         if (threadIdx.x == 0) s_broken = 0u;
     }
     __syncthreads();
-    if (a.by_table && blockIdx.x == 0 && first_col)
+    if (a.by_table && blockIdx.x == 0)
         for (int t = threadIdx.x; t <= T; t += THREADS) a.uniq_off[t] = s_broken ? 0 : (int32_t)s_uoff[t];
     if (s_broken || tile0 >= tile1) return;       // (warp-uniform; no block barrier below)
 
@@ -250,8 +255,8 @@ seg_sum_kernel(const Args a)
     };
     // asks L2 for the rows of the tile whose indices have just arrived: a row per lane and word
     auto prefetch = [&]() {
-        const int c0 = EXACT ? 0 : blockIdx.y * LPR * VEC;
-        const int bytes = (EXACT ? D : min(D - c0, LPR * VEC)) * (int)sizeof(float);
+        const int c0 = (int)col * LPR * VEC;
+        const int bytes = (EXACT ? LPR * VEC : min(D - c0, LPR * VEC)) * (int)sizeof(float);
 #pragma unroll
         for (int w = 0; w < W; ++w) {
             if (I % 32 != 0 && wl >= I) break;
@@ -319,7 +324,7 @@ seg_sum_kernel(const Args a)
                 before += __popc(hw[w]);
             }
         }
-        if (tile + 1 < tile1) prefetch();
+        if (tile + 1 < tile1 && (!COLS || D < 768)) prefetch();
         if constexpr (GP == 1) {
             u32 u = u_base;
             const u32 heads = hw[0];
@@ -449,7 +454,7 @@ seg_sum_kernel(const Args a)
             arrived = &a.range_done[2 * group + (group == g0 ? 1 : 0)].y;
         }
         __threadfence();
-        last = atomicAdd(arrived, 1u) == pieces * gridDim.y - 1u ? pieces : 0u;
+        last = atomicAdd(arrived, 1u) == pieces * cols - 1u ? pieces : 0u;
         __threadfence();
     }
     __syncwarp();
@@ -491,7 +496,7 @@ seg_sum_kernel(const Args a)
         const u32 u = q ? u_base : u_lead, f = __shfl_sync(0xffffffffu, first_range, q);
         const u32 ng = __shfl_sync(0xffffffffu, groups, q), g0 = f / FOLD_GROUP;
         const u32 p_first = ng ? max(f, group * FOLD_GROUP) : f;
-        for (int cc = lane; cc - lane < dv; cc += LPR) {
+        for (int cc = lane; cc - lane < (COLS ? dv : 1); cc += LPR) {
             double sum[VEC];
             fold(np, cc, sum, [&](int p) { return a.partials + ((size_t)(p_first + p) * 2 + (p_first + p == f ? 1 : 0)) * D; });
             if (ng == 0) {
@@ -510,7 +515,7 @@ seg_sum_kernel(const Args a)
                 __threadfence();
             }
             if (!__shfl_sync(0xffffffffu, final, 0)) continue;
-            for (int cc = lane; cc - lane < dv; cc += LPR) {
+            for (int cc = lane; cc - lane < (COLS ? dv : 1); cc += LPR) {
                 double sum[VEC];
                 fold((int)ng, cc, sum, [&](int p) { return a.group_partials + ((size_t)(g0 + p) * 2 + (p == 0 ? 1 : 0)) * D; });
                 store_total(u, cc, sum);

@@ -45,3 +45,46 @@ def test_runs_at_the_edges(oracle, split, D, sort_path):
     n = max(max(r) for r in runs)
     np.testing.assert_allclose(gr, o_gr, rtol=2.0 ** -23, atol=12.0 * n * n * 2.0 ** -53)
     c.ctx.close()
+
+
+# tables of 1,024 to 98,304 lookups on average, which the clusters sort and number themselves: a run over hundreds of
+# ranges in a table alone (sixteen blocks) and beside small ones (eight), a table beyond its blocks' shared memory, runs
+# on the edges of tiles
+CLUSTER_SPLITS = {
+    "one_run": [[3, 80_000, 5]],
+    "one_run_uneven": [[7, 1]] * 2 + [[3, 40_000, 5]] + [[1, 31, 32, 33] * 20, [1] * 2_500, [64] * 33, [2, 30] * 40],
+    "edges": [[31, 1, 1, 31, 32, 33, 63, 1, 64, 65, 31] * 9] * 7,
+}
+
+
+@pytest.mark.parametrize("D", [8, 16, 32, 64, 100, 128, 200, 256, 1020, 1024])
+@pytest.mark.parametrize("split", list(CLUSTER_SPLITS))
+def test_runs_of_the_cluster_sort(oracle, split, D):
+    if D > 128 and split == "one_run":
+        pytest.skip("the table alone takes the narrower rows")
+    runs = CLUSTER_SPLITS[split]
+    counts = [sum(r) for r in runs]
+    B = max(counts)                     # bags of one index; tables with fewer lookups end in empty bags
+    wl = W.Workload("runs", tuple(max(4, len(r)) for r in runs), D=D, B=B, alpha=None)
+    rng = np.random.default_rng(len(split) + D)
+    idx = np.concatenate([rng.permutation(np.repeat(np.arange(len(r)), r)) for r in runs]).astype(np.int32)
+    lens = np.zeros((wl.T, B), dtype=np.int64)
+    for t, n in enumerate(counts):
+        lens[t, :n] = 1
+    off = np.concatenate([[0], np.cumsum(lens.reshape(-1))]).astype(np.int32)
+    L = len(idx)
+    # of the bags behind the last lookup nothing is read: one row of zeros would do, so only the used ones are drawn
+    go = np.zeros((B, wl.T, D), dtype=np.float32)
+    for t, n in enumerate(counts):
+        go[:n, t] = rng.standard_normal((n, D), dtype=np.float32)
+    c = Case(wl, max_lookups=L)
+    c.ctx.profile_begin()
+    ur, uo, gr = c.gpu_bwd(idx, off, go)
+    names = set(c.ctx.profile_end())
+    assert names & {"small_sort_kernel", "cluster_sort_kernel", "rs_scatter_kernel"} == {"cluster_sort_kernel"}, names
+    o_ur, o_uo, o_gr = oracle.emb_bwd(go, wl.T, D, B, idx, off)
+    assert bit_equal(uo, o_uo) and bit_equal(ur, o_ur)
+    # as above
+    n = max(max(r) for r in runs)
+    np.testing.assert_allclose(gr, o_gr, rtol=2.0 ** -23, atol=12.0 * n * n * 2.0 ** -53)
+    c.ctx.close()
