@@ -300,24 +300,26 @@ int launch_radix_sort(dqrm_ctx *ctx, const rsort::Args &a, int passes, uint2 *co
     return DQRM_OK;
 }
 
-template <int CL>
-cudaError_t launch_cluster_sort(dqrm_ctx *ctx, csort::Args ca, int64_t per_table, cudaStream_t st)
+template <int CL, int EPT = 0>
+cudaError_t launch_cluster_sort(dqrm_ctx *ctx, csort::Args ca, int cap, cudaStream_t st)
 {
-    ca.cap = csort::choose_cap(per_table, CL);
-    bool &raised = ctx->smem_raised[DQ_SMEM_SLOT_CSORT + (CL == csort::CLUSTER ? 0 : 1)];
+    ca.cap = cap;
+    const size_t smem = std::max(csort::smem_bytes(cap), (size_t)csort::THREADS * EPT * 2 * sizeof(ssort::u64));
+    static_assert(CL == csort::CLUSTER || EPT == 0, "");
+    bool &raised = ctx->smem_raised[DQ_SMEM_SLOT_CSORT + (CL == csort::CLUSTER ? EPT : 3)];
     cudaError_t e = cudaSuccess;
     if (!raised) {
-        e = cudaFuncSetAttribute(csort::cluster_sort_kernel<CL>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        e = cudaFuncSetAttribute(csort::cluster_sort_kernel<CL, EPT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)csort::smem_bytes(12288));
         if (e == cudaSuccess && CL > 8)       // more than eight blocks in a cluster is an opt-in
-            e = cudaFuncSetAttribute(csort::cluster_sort_kernel<CL>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+            e = cudaFuncSetAttribute(csort::cluster_sort_kernel<CL, EPT>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
         raised = (e == cudaSuccess);
     }
     if (e == cudaSuccess) {
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3((unsigned)(ctx->T * CL));
         cfg.blockDim = dim3(csort::THREADS);
-        cfg.dynamicSmemBytes = csort::smem_bytes(ca.cap);
+        cfg.dynamicSmemBytes = smem;
         cfg.stream = st;
         cudaLaunchAttribute attr[2];
         attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -325,7 +327,7 @@ cudaError_t launch_cluster_sort(dqrm_ctx *ctx, csort::Args ca, int64_t per_table
         attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
         attr[1].val.programmaticStreamSerializationAllowed = 1;
         cfg.attrs = attr; cfg.numAttrs = 2;
-        e = cudaLaunchKernelEx(&cfg, csort::cluster_sort_kernel<CL>, ca);
+        e = cudaLaunchKernelEx(&cfg, csort::cluster_sort_kernel<CL, EPT>, ca);
     }
     if (e != cudaSuccess) (void)cudaGetLastError();
     return e;
@@ -334,7 +336,10 @@ cudaError_t launch_cluster_sort(dqrm_ctx *ctx, csort::Args ca, int64_t per_table
 // The block sort; false where the batch is too large for it.  `per_table` lookups a table on average, with room for a
 // quarter more where bags are uneven.  Measured on B200 against the cluster sort (graph replay, 26 tables of 900 K rows,
 // us per batch): 128 lookups a table 3.5 against 12.3, 500 5.4 / 12.5, 1000 8.0 / 12.6, 2048 14.9 / 13.4; with 100
-// tables, whose clusters take turns, 1000 lookups 8.5 / 33.
+// tables, whose clusters take turns, 1000 lookups 8.5 / 33.  Unless the batch has an index a bag, one table may hold most
+// of it: a cluster of blocks then stands by for every table (a table of
+// 12.8 K lookups beside 25 of 128: 22.8 us, 99 by one block in global memory, 34.8 in a cluster of whole batches; bags of
+// five everywhere 11.6, 9.2 without the clusters standing by).
 template <int THREADS, int EPT>
 cudaError_t launch_small_sort2(dqrm_ctx *ctx, const csort::Args &ca, cudaStream_t st)
 {
@@ -348,6 +353,13 @@ bool launch_small_sort(dqrm_ctx *ctx, const csort::Args &ca, int64_t per_table, 
     const int64_t want = even ? per_table : per_table + per_table / 4;
     const bool many = ctx->T * csort::CLUSTER > 2 * ctx->num_sms;
     if (want > (many ? 2048 : 1024)) return false;
+    if (!even) {
+        const int cap = csort::shared_cap(ca.L);
+        e = want <= 512    ? launch_cluster_sort<csort::CLUSTER, 1>(ctx, ca, cap, st)
+            : want <= 1024 ? launch_cluster_sort<csort::CLUSTER, 2>(ctx, ca, cap, st)
+                           : launch_cluster_sort<csort::CLUSTER, 4>(ctx, ca, cap, st);
+        return true;
+    }
     if (want <= 256) e = launch_small_sort2<256, 1>(ctx, ca, st);
     else if (want <= 512) e = launch_small_sort2<512, 1>(ctx, ca, st);
     else if (want <= 1024) e = launch_small_sort2<512, 2>(ctx, ca, st);
@@ -430,7 +442,7 @@ int dq_launch_bwd_sort(dqrm_ctx *ctx, const int32_t *indices, const int32_t *off
         cudaError_t e = cudaErrorUnknown;
         if (lists_by_table && launch_small_sort(ctx, ca, per_table, L == G, st, e)) {
             if (e == cudaSuccess) {
-                dq_mark(ctx, st, DQ_K_SMALL_SORT);
+                dq_mark(ctx, st, L == G ? DQ_K_SMALL_SORT : DQ_K_CLUSTER_SORT);
                 if (by_table) *by_table = true;
                 return DQRM_OK;
             }
@@ -438,9 +450,9 @@ int dq_launch_bwd_sort(dqrm_ctx *ctx, const int32_t *indices, const int32_t *off
             (void)cudaGetLastError();
         }
         const bool wide = ctx->T * csort::CLUSTER_WIDE * 2 <= ctx->num_sms && per_table >= csort::CLUSTER_WIDE * 1024;
-        if (wide) e = launch_cluster_sort<csort::CLUSTER_WIDE>(ctx, ca, per_table, st);
+        if (wide) e = launch_cluster_sort<csort::CLUSTER_WIDE>(ctx, ca, csort::choose_cap(per_table, csort::CLUSTER_WIDE), st);
         else e = cudaErrorUnknown;
-        if (e != cudaSuccess) e = launch_cluster_sort<csort::CLUSTER>(ctx, ca, per_table, st);
+        if (e != cudaSuccess) e = launch_cluster_sort<csort::CLUSTER>(ctx, ca, csort::choose_cap(per_table, csort::CLUSTER), st);
         if (e == cudaSuccess) {
             dq_mark(ctx, st, DQ_K_CLUSTER_SORT);
             skeys = keys[0];

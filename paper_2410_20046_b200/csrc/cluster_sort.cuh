@@ -58,6 +58,17 @@ struct Args {
     u32 cnt_broken;
 };
 
+}  // namespace csort
+
+namespace ssort {
+// one block's sort of table t (small_sort.cuh): its lookups [tb0, tb1), at most THREADS * EPT of them, and its lists; shared
+// memory for twice that many pairs
+template <int THREADS, int EPT>
+__device__ void sort_table(const csort::Args &a, int t, int64_t tb0, int64_t tb1, unsigned long long *s_net);
+}
+
+namespace csort {
+
 __device__ __forceinline__ u32 *remote(cg::cluster_group &cluster, u32 *p, unsigned rank)
 {
     return cluster.map_shared_rank(p, rank);
@@ -75,7 +86,10 @@ __device__ __forceinline__ u32 same_digit_lanes(u32 d, bool valid)
 // kernel takes 95 registers and 26 tables of 16 K lookups 40 us instead of 32, with three 37.  Clusters of sixteen are
 // launched for a few tables only and have their SMs to themselves: 36.6 us without the bound, 42.2 with it, for one table
 // of 64 K lookups)
-template <int CL>
+//
+// EPT > 0: for small batches whose bags may be uneven.  A table of up to THREADS * EPT lookups, which is nearly all of them,
+// is sorted by the cluster's first block alone, with the network of small_sort.cuh, and only a larger one by the cluster.
+template <int CL, int EPT>
 __global__ void __launch_bounds__(THREADS, CL > 8 ? 1 : 2)
 cluster_sort_kernel(const Args a)
 {
@@ -112,6 +126,12 @@ cluster_sort_kernel(const Args a)
         if (t == a.T - 1) a.tb[a.T] = (u32)tb1;
         a.absmax[t] = 0u;
         if (n == 0) a.table_cnt[t] = 0u;
+    }
+    if constexpr (EPT > 0) {
+        if (n <= THREADS * EPT) {
+            if (c == 0) ssort::sort_table<THREADS, EPT>(a, t, tb0, tb1, reinterpret_cast<unsigned long long *>(s_dyn));
+            return;
+        }
     }
     if (n == 0) return;
     const int64_t r0 = __ldg(a.row_off + t);
@@ -391,6 +411,10 @@ cluster_sort_kernel(const Args a)
 }
 
 inline size_t smem_bytes(int cap) { return (size_t)2 * cap * sizeof(uint2); }
+
+// the same for the clusters of which only the first block works in nearly every table: room for the batch in one of them, up
+// to what leaves two blocks resident
+inline int shared_cap(int64_t L) { return (int)((L < 8 * 5600 ? L / 8 : 5600) + 32) / 32 * 32; }
 
 // pairs per block to provision in shared memory for an expected n per table sorted by `cluster` blocks
 inline int choose_cap(int64_t expect_n, int cluster)

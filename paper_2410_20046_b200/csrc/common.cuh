@@ -132,7 +132,7 @@ __device__ __forceinline__ void dq_let_next()
 static inline size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
 // slots of dqrm_ctx::smem_raised
-constexpr int DQ_SMEM_SLOT_STEP = 4, DQ_SMEM_SLOT_CSORT = 24;
+constexpr int DQ_SMEM_SLOT_STEP = 4, DQ_SMEM_SLOT_CSORT = 8;
 constexpr int dq_log2c(int x) { return x <= 1 ? 0 : 1 + dq_log2c(x / 2); }
 
 // ---------------------------------------------------------------------------------

@@ -16,8 +16,6 @@ namespace ssort {
 
 typedef unsigned long long u64;
 
-constexpr int MAX_THREADS = 1024;
-
 inline size_t smem_bytes(int threads, int ept)
 {
     const size_t net = (size_t)threads * ept * 2 * sizeof(u64);
@@ -205,45 +203,16 @@ __device__ __forceinline__ void sort_in_block(const csort::Args &a, int t, int64
     __syncthreads();
 }
 
-template <int THREADS, int EPT>
-__global__ void __launch_bounds__(THREADS)
-small_sort_kernel(const csort::Args a)
+// The sorted keys and payloads of the block's table, and where its segments stand: THREADS consecutive entries at a time, out
+// of the network's places or of memory
+template <int THREADS>
+__device__ __forceinline__ void write_table(const csort::Args &a, int t, int64_t tb0, int64_t tb1, const u64 *s_net, const uint2 *mem)
 {
-    dq_wait_before();
-    constexpr int WARPS = THREADS / 32, N = THREADS * EPT;
-    extern __shared__ u64 s_net[];                 // [2][N]
+    constexpr int WARPS = THREADS / 32;
     __shared__ u32 s_warp[WARPS];
     __shared__ u32 s_total;
-    const int t = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int64_t tb0 = __ldg(a.offsets + (int64_t)t * a.B), tb1 = __ldg(a.offsets + (int64_t)(t + 1) * a.B);
-    if (tb0 < 0 || tb1 < tb0 || tb1 > a.L || (t == 0 && tb0 != 0) || (t == a.T - 1 && tb1 != a.L)) {
-        if (tid == 0) {
-            dq_report(a.status, DQRM_ERR_INDEX_RANGE);
-            a.table_cnt[t] = a.cnt_broken;         // nothing is summed; the quantiser behind finds an empty gradient
-            a.absmax[t] = 0u;
-        }
-        return;
-    }
-    const int64_t n = tb1 - tb0, r0 = __ldg(a.row_off + t), nrows = __ldg(a.row_off + t + 1) - r0;
-    if (tid == 0) {
-        a.tb[t] = (u32)tb0;
-        if (t == a.T - 1) a.tb[a.T] = (u32)tb1;
-        a.absmax[t] = 0u;
-        if (n == 0) a.table_cnt[t] = 0u;
-    }
-    bool bad = false;
-    if (n != a.B)                                  // (otherwise every lookup looks at its own bag's offsets)
-        for (int i = tid; i < a.B; i += THREADS) bad |= __ldg(a.offsets + (int64_t)t * a.B + i) > __ldg(a.offsets + (int64_t)t * a.B + i + 1);
-    if (bad) dq_report(a.status, DQRM_ERR_INDEX_RANGE);
-    if (n == 0) return;
-    const uint2 *mem = nullptr;                    // the sorted pairs of a table that does not fit the block
-    if (n > N) {
-        mem = sort_in_memory<THREADS>(a, t, tb0, n, nrows, reinterpret_cast<u32 *>(s_net));
-    } else {
-        sort_in_block<THREADS, EPT>(a, t, tb0, n, nrows, s_net, bad);
-        if (bad) dq_report(a.status, DQRM_ERR_INDEX_RANGE);
-    }
-    // ---- sorted keys and payloads, and where the segments stand: THREADS consecutive entries at a time
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int64_t n = tb1 - tb0, r0 = __ldg(a.row_off + t);
     u32 *segs = a.seg_start + tb0 + t;
     const u32 ck_mask = (1u << a.ck_shift) - 1u;
     u32 base = 0;                                  // segments that begin before these entries
@@ -294,6 +263,62 @@ small_sort_kernel(const csort::Args a)
     if (tid == 0) {
         a.table_cnt[t] = base;
         segs[base] = (u32)tb1;                     // the slot behind the last segment holds the table's end
+    }
+}
+
+// offsets must not decrease inside the table
+template <int THREADS>
+__device__ __forceinline__ bool offsets_fall(const csort::Args &a, int t)
+{
+    bool bad = false;
+    for (int i = threadIdx.x; i < a.B; i += THREADS) bad |= __ldg(a.offsets + (int64_t)t * a.B + i) > __ldg(a.offsets + (int64_t)t * a.B + i + 1);
+    return bad;
+}
+
+template <int THREADS, int EPT>
+__device__ void sort_table(const csort::Args &a, int t, int64_t tb0, int64_t tb1, u64 *s_net)
+{
+    const int64_t n = tb1 - tb0, nrows = __ldg(a.row_off + t + 1) - __ldg(a.row_off + t);
+    bool bad = n != a.B && offsets_fall<THREADS>(a, t);       // (otherwise every lookup looks at its own bag's offsets)
+    if (n == 0) {                                  // (its empty lists have been written)
+        if (bad) dq_report(a.status, DQRM_ERR_INDEX_RANGE);
+        return;
+    }
+    sort_in_block<THREADS, EPT>(a, t, tb0, n, nrows, s_net, bad);
+    if (bad) dq_report(a.status, DQRM_ERR_INDEX_RANGE);
+    write_table<THREADS>(a, t, tb0, tb1, s_net, nullptr);
+}
+
+template <int THREADS, int EPT>
+__global__ void __launch_bounds__(THREADS)
+small_sort_kernel(const csort::Args a)
+{
+    dq_wait_before();
+    extern __shared__ u64 s_net[];                 // [2][THREADS * EPT]
+    const int t = blockIdx.x, tid = threadIdx.x;
+    const int64_t tb0 = __ldg(a.offsets + (int64_t)t * a.B), tb1 = __ldg(a.offsets + (int64_t)(t + 1) * a.B);
+    if (tb0 < 0 || tb1 < tb0 || tb1 > a.L || (t == 0 && tb0 != 0) || (t == a.T - 1 && tb1 != a.L)) {
+        if (tid == 0) {
+            dq_report(a.status, DQRM_ERR_INDEX_RANGE);
+            a.table_cnt[t] = a.cnt_broken;         // nothing is summed; the quantiser behind finds an empty gradient
+            a.absmax[t] = 0u;
+        }
+        return;
+    }
+    const int64_t n = tb1 - tb0;
+    if (tid == 0) {
+        a.tb[t] = (u32)tb0;
+        if (t == a.T - 1) a.tb[a.T] = (u32)tb1;
+        a.absmax[t] = 0u;
+        if (n == 0) a.table_cnt[t] = 0u;
+    }
+    if (n <= THREADS * EPT) {
+        sort_table<THREADS, EPT>(a, t, tb0, tb1, s_net);
+    } else {                                       // (a one-index batch that is none)
+        if (offsets_fall<THREADS>(a, t)) dq_report(a.status, DQRM_ERR_INDEX_RANGE);
+        const int64_t nrows = __ldg(a.row_off + t + 1) - __ldg(a.row_off + t);
+        const uint2 *mem = sort_in_memory<THREADS>(a, t, tb0, n, nrows, reinterpret_cast<u32 *>(s_net));
+        write_table<THREADS>(a, t, tb0, tb1, nullptr, mem);
     }
 }
 

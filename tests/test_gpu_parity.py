@@ -415,3 +415,44 @@ def test_gradient_scales_of_a_batch_with_unusable_boundaries(oracle, B, calls):
     assert (gs.cpu().numpy() == oracle.scale_from_absmax(0.0, 8)).all()
     assert bit_equal(d_tables.cpu().numpy(), tables)
     c.ctx.close()
+
+
+# bags per table and mean indices per bag: tables that one block sorts, tables that their clusters sort, a radix sort
+@pytest.mark.parametrize("B,bag,sort_path,kernel", [(300, 1, 0, "small_sort_kernel"), (1500, 3, 0, "cluster_sort_kernel"),
+                                                    (1500, 3, 1, "rs_scatter_kernel")])
+@pytest.mark.parametrize("fault", ["decrease", "boundary"])
+def test_unusable_offsets_by_sort(oracle, B, bag, sort_path, kernel, fault):
+    """What the small batches above check, at the sizes of each sort: reported, nothing out of bounds, and the context stays
+    usable.  An unusable table boundary is not summed at all by the sorts that number their own tables."""
+    import paper_2410_20046_b200 as dq
+
+    wl = W.Workload("bad_bags", (50, 7, 300), D=16, B=B, alpha=1.1, bits=4, **({} if bag == 1 else dict(bag_mean=float(bag), bag_max=6)))
+    c = Case(wl)
+    idx, off, go = c.batch(0)
+    L, bad = len(idx), off.copy()
+    if fault == "decrease":
+        g = wl.B + 5                                  # a bag inside table 1
+        bad[g], bad[g + 1] = off[g + 1], off[g]
+        assert bad[g] > bad[g + 1]
+    else:
+        bad[wl.B] = L + 3                             # where table 1 begins
+    c.ctx.set_sort_path(sort_path)
+    ur = c.torch.full((L,), -1, dtype=c.torch.int32, device="cuda")
+    uo = c.torch.full((wl.T + 1,), -1, dtype=c.torch.int32, device="cuda")
+    gr = c.torch.full((L, wl.D), 7.0, dtype=c.torch.float32, device="cuda")
+    c.ctx.profile_begin()
+    c.ctx.emb_bwd(c.dev(go), c.dev(idx), c.dev(bad), ur, uo, gr, B=wl.B, L=L)
+    names = set(c.ctx.profile_end())
+    assert names & {"small_sort_kernel", "cluster_sort_kernel", "rs_scatter_kernel"} == {kernel}, names
+    with pytest.raises(dq.DqrmError) as e:
+        c.ctx.raise_on_device_error()
+    assert e.value.status == dq.ERR_INDEX_RANGE
+    if fault == "boundary" and sort_path == 0:
+        assert not uo.cpu().numpy().any()
+        assert (gr.cpu().numpy() == 7.0).all() and (ur.cpu().numpy() == -1).all()
+    assert c.ctx.check_status() == dq.OK
+    g_ur, g_uo, g_gr = c.gpu_bwd(idx, off, go)        # still usable and correct
+    o_ur, o_uo, o_gr = oracle.emb_bwd(go, wl.T, wl.D, wl.B, idx, off)
+    assert bit_equal(g_ur, o_ur) and bit_equal(g_uo, o_uo)
+    assert_close_fp32(g_gr, o_gr)
+    c.ctx.close()

@@ -35,3 +35,39 @@ def test_block_sort(oracle, name, rows):
     # at most 4000 terms of magnitude below 6 in FP64 in two orders, each sum rounded once
     np.testing.assert_allclose(gr, o_gr, rtol=2.0 ** -23, atol=12.0 * 4000 ** 2 * 2.0 ** -53)
     c.ctx.close()
+
+
+# (lookups per table, bags per table, kernel): small batches in which one table is beyond a block, whose cluster then sorts it
+UNEVEN = {
+    "shared_1": ([13, 0, 3_000] + [40] * 23, 150, "cluster_sort_kernel"), "shared_2": ([9_000, 500, 1] + [300] * 21, 600, "cluster_sort_kernel"),
+    "edges_1": ([511, 512, 513, 514] + [0, 1], 700, "cluster_sort_kernel"), "edges_2": ([1023, 1024, 1025, 90] + [0, 1], 1100, "cluster_sort_kernel"),
+    "beyond_the_clusters": ([700] * 98 + [60_000, 1], 800, "cluster_sort_kernel"),
+    "edges_4": ([2047, 2048, 2049, 2050] + [1_400] * 60, 2100, "cluster_sort_kernel"),
+    # as many lookups as bags, but not one in each
+    "in_memory": ([400, 0, 0, 0], 100, "small_sort_kernel"), "in_memory_wide": ([3_000, 1_000, 72, 24], 1_024, "small_sort_kernel"),
+}
+
+
+@pytest.mark.parametrize("rows", [1, 300, 70_000])
+@pytest.mark.parametrize("name", list(UNEVEN))
+def test_uneven_tables(oracle, name, rows):
+    counts, B, kernel = UNEVEN[name]
+    D = 8
+    wl = W.Workload("uneven", tuple(max(1, rows + t) for t in range(len(counts))), D=D, B=B, alpha=None)
+    rng = np.random.default_rng(rows + B)
+    idx = np.concatenate([rng.integers(0, wl.rows[t], n) for t, n in enumerate(counts)]).astype(np.int32)
+    lens = np.zeros((wl.T, B), dtype=np.int64)
+    for t, n in enumerate(counts):
+        np.add.at(lens[t], rng.integers(0, B, n), 1)
+    off = np.concatenate([[0], np.cumsum(lens.reshape(-1))]).astype(np.int32)
+    go = rng.standard_normal((B, wl.T, D)).astype(np.float32)
+    c = Case(wl, max_lookups=len(idx))
+    c.ctx.profile_begin()
+    ur, uo, gr = c.gpu_bwd(idx, off, go)
+    names = set(c.ctx.profile_end())
+    assert names & {"small_sort_kernel", "cluster_sort_kernel", "rs_scatter_kernel"} == {kernel}, names
+    o_ur, o_uo, o_gr = oracle.emb_bwd(go, wl.T, D, B, idx, off)
+    assert bit_equal(uo, o_uo) and bit_equal(ur, o_ur)
+    # at most 60,000 terms of magnitude below 6 in FP64 in two orders, each sum rounded once
+    np.testing.assert_allclose(gr, o_gr, rtol=2.0 ** -23, atol=12.0 * max(counts) ** 2 * 2.0 ** -53)
+    c.ctx.close()
