@@ -360,9 +360,10 @@ int dqrm_set_sort_path(dqrm_ctx *ctx, int path);
  * sort, gradient summation: neither needs the tables or the forward's output) on a second
  * stream owned by the context (created by dqrm_create), beside the forward on the caller's
  * stream, and join the two before the touched rows are updated; the caller's stream sees one
- * ordered step.  dqrm_train_step does so from 16 MB of gathered rows on; smaller batches, for
- * which fork and join cost more than the overlap gives, stay on the caller's stream (the
- * smallest as one launch behind the forward).  dqrm_train_step_sorted also moves its forward to
+ * ordered step.  dqrm_train_step does so from 16 MB of gathered rows on, and for batches
+ * of up to 16384 lookups that are not one a bag; other small batches, for which fork and join
+ * cost more than the overlap gives, stay on the caller's stream, and the smallest of all take
+ * one launch behind the forward.  dqrm_train_step_sorted also moves its forward to
  * a third, lowest-priority stream of the context (forked from and joined to the caller's
  * stream), so that the forward's many blocks do not keep a sort of the next batch, running
  * elsewhere, off the SMs.

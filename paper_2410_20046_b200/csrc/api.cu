@@ -60,6 +60,19 @@ int64_t host_lookups_for(const dqrm_ctx *ctx, size_t workspace_bytes, int64_t L,
     return lo;
 }
 
+// Whether dqrm_train_step runs the backward beside the forward.  From 16 MB of gathered rows on it does; below, fork and join
+// and the forward's blocks in the sort's way cost about what the overlap gives (measured on B200, graph replay, two streams /
+// one: 26 tables of 4096 lookups of 64 bytes 34.2 / 34.6 us, 6 of 16 K 45.3 / 39.7, 4 of 8192 of 256 bytes 39.6 / 36.4; few
+// tables are 2 to 4 us faster in two, 24.4 / 28.8 for three of 4096 of 256 bytes, but launched one by one the same or slower).
+// Batches of up to 16 K lookups that are not an index a bag fork too: a few long bags are a long chain for their lane groups
+// while the rest of the chip waits (26 tables of 64 bags, one table with 100 indices a bag, 64-byte rows: 30.8 / 53.8 us; even
+// bags of three, three tables of 600: 30.8 / 32.7 with 64-byte rows, 26.5 / 25.6 with 256-byte rows).
+bool step_forks(const dqrm_ctx *ctx, int B, int64_t L)
+{
+    if (L * ctx->D * (int64_t)sizeof(float) >= ((int64_t)16 << 20)) return true;
+    return L > 0 && L != (int64_t)ctx->T * B && L <= 16384;
+}
+
 }  // namespace
 
 extern "C" {
@@ -336,10 +349,7 @@ int dqrm_train_step(dqrm_ctx *ctx, float *tables, const int32_t *indices, const 
     // tables nor the forward's output, so it runs on the context's second stream while the forward runs on
     // the caller's (per-launch profiling keeps one stream, because its events time consecutive launches).
     // The quantise-and-update kernel writes the rows the forward reads, so it waits for both.
-    // Below 16 MB of gathered rows the fork and the join cost more than the overlap gives, and the step is one chain of
-    // launches on the caller's stream (measured on B200, two streams / one: 512 lookups of 64-byte rows 20.5 / 18.5 us,
-    // 53 K of 64 bytes 34.8 / 32.6, 213 K of 64 bytes 46.6 / 43.9, 64 K of 512 bytes 87.4 / 89.8).
-    const bool overlap = ctx->overlap && !ctx->prof_on && L * ctx->D * (int64_t)sizeof(float) >= ((int64_t)16 << 20);
+    const bool overlap = ctx->overlap && !ctx->prof_on && step_forks(ctx, B, L);
     cudaStream_t ss = overlap ? ctx->side : st;
     if (overlap) {
         DQRM_CUDA_TRY(ctx, cudaEventRecord(ctx->ev_fork, st));

@@ -15,6 +15,9 @@ SHAPES = {
     "block": (16, [512, 511, 513, 512]), "beyond_it": (16, [513, 513, 513, 513]), "all": (32, [512] * 8), "and_one": (4, [512] * 7 + [513]),
     "one_table_holds_all": (8, [0, 2, 3200, 0, 0, 0, 1, 0]), "wide": (128, [127, 128]), "narrow": (4, [300] * 13),
     "many_tables": (8, [1, 0, 40, 33] * 30),
+    # uneven batches up to the most that one block may have to take alone, and one lookup beyond
+    "one_block_takes_most": (16, [3, 0, 1500, 33]), "and_one_more": (16, [3, 0, 1501, 33]), "few_in_many_tables": (8, [1, 0, 10, 13] * 30),
+    "widest_uneven": (64, [500, 1, 11]), "too_wide_uneven": (64, [501, 1, 11]),
 }
 
 
