@@ -15,6 +15,7 @@ CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libdqrm_b200.so")
 NATIVE_SRC = os.path.join(CSRC, "binding.cpp")
 NATIVE = os.path.join(HERE, "_dqrm_native.so")
+NATIVE_FOR = NATIVE + ".for"          # what the module was built for
 
 NVCC_FLAGS = [
     "-gencode", "arch=compute_100a,code=sm_100a",
@@ -35,9 +36,22 @@ def _stale() -> bool:
     return any(os.path.getmtime(d) > os.path.getmtime(LIB) for d in deps)
 
 
+def _native_for() -> str:
+    """The Python and the torch that a module built now could be loaded by."""
+    from importlib import metadata
+
+    return f"python {sys.implementation.cache_tag} torch {metadata.version('torch')}\n"
+
+
 def _native_stale() -> bool:
     deps = [NATIVE_SRC, os.path.join(ROOT, "include", "dqrm.h")]
-    return not os.path.exists(NATIVE) or any(os.path.getmtime(d) > os.path.getmtime(NATIVE) for d in deps)
+    if not os.path.exists(NATIVE) or any(os.path.getmtime(d) > os.path.getmtime(NATIVE) for d in deps):
+        return True
+    try:
+        with open(NATIVE_FOR) as f:
+            return f.read() != _native_for()
+    except OSError:
+        return True
 
 
 def build_native() -> None:
@@ -57,6 +71,8 @@ def build_native() -> None:
            "-ltorch_python", "-ltorch_cpu", "-lc10", "-lc10_cuda"]
     subprocess.check_call(cmd)
     os.replace(tmp, NATIVE)
+    with open(NATIVE_FOR, "w") as f:
+        f.write(_native_for())
 
 
 def build(force: bool = False, verbose: bool = False) -> str:

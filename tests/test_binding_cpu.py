@@ -50,3 +50,13 @@ CASES = {
 def test_native_calls_raise_and_do_not_abort(case):
     r = subprocess.run([sys.executable, "-c", PRELUDE + CASES[case]], cwd=ROOT, capture_output=True, text=True, timeout=300)
     assert r.returncode == 0 and "raised" in r.stdout, (r.returncode, r.stdout, r.stderr[-2000:])
+
+
+def test_native_module_is_rebuilt_for_another_torch_or_python(monkeypatch):
+    """Dates alone say nothing of a module that another torch was installed under."""
+    from paper_2410_20046_b200 import build
+
+    build.build()
+    assert not build._native_stale()
+    monkeypatch.setattr(build, "_native_for", lambda: "python cpython-399 torch 9.9\n")
+    assert build._native_stale()
