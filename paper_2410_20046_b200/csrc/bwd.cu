@@ -3,9 +3,10 @@
 // touched; lookups that hit the same row are coalesced.  Sum pooling and the
 // straight-through quantiser hand every lookup its bag's upstream gradient unchanged.
 //
-// Pipeline (all on one stream, no inter-block waits anywhere):
-//   sort         one cluster of blocks per table (cluster_sort.cuh), or a radix sort of all
-//                tables at once (radix_sort.cuh); the cluster sort can also number the segments
+// Pipeline (all on one stream; no block waits for another outside its cluster):
+//   sort         one block per table (small_sort.cuh), one cluster of blocks per table
+//                (cluster_sort.cuh), or a radix sort of all tables at once (radix_sort.cuh); the
+//                first two can also number the segments
 //   seg_count / seg_emit  head flags of the sorted keys -> unique_rows, uniq_off,
 //                         segment starts, first segment of every tile of the sum
 //   seg_sum      every warp walks a range of the sorted order: gathers the upstream gradient rows,
@@ -32,11 +33,10 @@ constexpr int ST_WARPS = ST_THREADS / 32;
 struct Layout {
     int passes, digit_bits;                    // radix sort: digits of the row number within a table
     int64_t radix_tiles, num_tiles;
-    // the summing kernel: log2 of the entries between two of chunk_first, small tiles, tiles, at most sum_ranges ranges of
-    // range_tiles tiles
+    // the summing kernel: log2 of the entries between two of chunk_first, small tiles, tiles, tiles of a warp's range
     int sum_shift;
     bool sum_small;
-    int64_t sum_tiles, sum_ranges;
+    int64_t sum_tiles;
     int range_tiles;
     size_t absmax, tile_heads, tile0, tile_table, totals, tilehist;
     size_t keys_a, vals_a, pairs_a, pairs_b, seg_start, chunk_first, tile_done, partials, group_partials, table_cnt, tb;
@@ -60,7 +60,6 @@ Layout make_layout(const dqrm_ctx *ctx, int64_t L)
     const int I = segred::tile_entries(lpr, y.sum_small);
     y.sum_shift = segred::chunk_shift(lpr, y.sum_small);
     y.sum_tiles = (Lc + I - 1) / I;
-    y.sum_ranges = y.sum_tiles < warps ? y.sum_tiles : warps;
     y.range_tiles = (int)((y.sum_tiles + warps - 1) / warps);
     size_t o = 0;
     auto take = [&](size_t bytes) { size_t at = o; o = align_up(o + bytes, 256); return at; };
@@ -428,7 +427,7 @@ int dq_launch_bwd_sort(dqrm_ctx *ctx, const int32_t *indices, const int32_t *off
         ca.status = ctx->d_status;
         ca.payload_position = ctx->payload_position;
         ca.tile_heads = reinterpret_cast<u32 *>(ws + y.tile_heads);
-        // when dq_launch_bwd_reduce follows, the clusters number their own tables' segments and seg_emit is not run
+        // when dq_launch_bwd_sum follows, the clusters number their own tables' segments and seg_emit is not run
         ca.lists_by_table = lists_by_table ? 1 : 0;
         ca.seg_start = reinterpret_cast<u32 *>(ws + y.seg_start);
         ca.chunk_first = reinterpret_cast<u32 *>(ws + y.chunk_first);

@@ -133,7 +133,6 @@ static inline size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; 
 
 // slots of dqrm_ctx::smem_raised
 constexpr int DQ_SMEM_SLOT_STEP = 4, DQ_SMEM_SLOT_CSORT = 8;
-constexpr int dq_log2c(int x) { return x <= 1 ? 0 : 1 + dq_log2c(x / 2); }
 
 // ---------------------------------------------------------------------------------
 // quantiser arithmetic: each operation is one IEEE round-to-nearest FP32 operation

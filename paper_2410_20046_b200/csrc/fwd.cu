@@ -5,8 +5,8 @@
 //
 // HBM-bound random row gather.  Measured on B200, a bare gather of this access pattern
 // runs fastest with many resident warps and only two to four independent 128-bit loads
-// per lane, so the kernels are kept lean (about 40 registers) rather than deeply
-// unrolled.  blockIdx.y is the table, which makes scale, bit width and row base block
+// per lane, so the kernels are kept lean (46 to 64 registers, a few of the one-index
+// kernel's values spilled for its fifth block) rather than deeply unrolled.  blockIdx.y is the table, which makes scale, bit width and row base block
 // constants.  A group of LPR lanes owns one row: a feature-16 row is one 64-byte request
 // of four lanes, a feature-64 row one 256-byte request of sixteen.
 //   * fwd_onehot_kernel (launched when L == T*B and no codes are asked for, the Criteo-shaped
@@ -44,6 +44,15 @@ struct FwdArgs {
     int *status;
     int let_next;                // the kernel behind this one may begin (it waits itself where it has to)
 };
+
+// Waits for the kernels before this one and only then lets the next one begin.  The order is what the one-launch step
+// (small_step.cuh) stands on: it reads the batch and writes the workspace, unique_rows and grad_rows before its own wait, so
+// everything before this kernel must be over by then.  The other way round it would race with all of that.
+__device__ __forceinline__ void before_and_next(const FwdArgs &a)
+{
+    dq_wait_before();
+    if (a.let_next) dq_let_next();
+}
 
 __device__ __forceinline__ void store_codes(int8_t *codes_out, int64_t j, int D, int c4, const float4 &c)
 {
@@ -109,8 +118,7 @@ template <int LPR, int CH, bool EXACT>
 __global__ void __launch_bounds__(FW_THREADS, 5)
 fwd_onehot_kernel(const FwdArgs a)
 {
-    dq_wait_before();
-    if (a.let_next) dq_let_next();
+    before_and_next(a);
     constexpr int NB = NBOf<LPR, CH>::v;      // row steps in flight
     constexpr int RPW = 32 / LPR;             // rows one warp instruction covers
     constexpr int WPB = FW_THREADS / 32;
@@ -226,8 +234,7 @@ template <int LPR, int CH, bool EXACT, bool CODES>
 __global__ void __launch_bounds__(FW_THREADS, bags_blocks(CH))
 fwd_bags_kernel(const FwdArgs a)
 {
-    dq_wait_before();
-    if (a.let_next) dq_let_next();
+    before_and_next(a);
     constexpr int NB = NBOf<LPR, CH>::v;
     constexpr int GPB = FW_THREADS / LPR;
     const int D = EXACT ? 4 * LPR * CH : a.D;
@@ -290,8 +297,7 @@ template <bool EXACT>
 __global__ void __launch_bounds__(FW_THREADS, 4)
 fwd_long_bags_kernel(const FwdArgs a)
 {
-    dq_wait_before();
-    if (a.let_next) dq_let_next();
+    before_and_next(a);
     constexpr int WPB = FW_THREADS / 32;
     const int D = EXACT ? 64 : a.D;
     const int t = blockIdx.y, lane = threadIdx.x & 31;

@@ -7,7 +7,9 @@
 // Every thread holds EPT consecutive entries: steps across less than EPT entries are register moves, across less than
 // 32 * EPT shuffles, wider ones go through shared memory (two buffers in turn, one barrier a step).  Row and position
 // make every key distinct, so the order is that of a stable sort.  A table with more lookups than the block holds
-// (an uneven batch) is sorted by the block in global memory instead, with 8-bit digits: slow, but it need not be fast.
+// is sorted by its cluster where the batch may have one (cluster_sort_kernel with EPT > 0).  By the block in global memory,
+// with 8-bit digits, only where a batch with as many lookups as bags is uneven all the same, and in the one-launch step, which
+// takes no batch in which that is the longer way: 7 ns a lookup against 2 in a cluster (12.8 K lookups).
 // The lists that it leaves are those of the cluster sort's lists_by_table.
 #pragma once
 #include "cluster_sort.cuh"

@@ -8,13 +8,15 @@
 // most MAX_LOOKUPS of them): cheaper than a launch more, and no block waits for another.
 //
 // The kernel begins while the forward runs: up to the update it touches neither tables nor pooled output, and only
-// there waits for the forward to end.
+// there waits for the forward to end.  What it reads before that (offsets, indices, upstream gradient) and writes
+// (unique_rows, grad_rows, the workspace) may belong to kernels before the forward: it is launched behind a forward that
+// waits for them before it lets this kernel begin (before_and_next in fwd.cu), and must not be launched behind anything else.
 //
 // Sums are FP64, in order of the entries inside a lane group's share and then over the shares: results are
 // reproducible.
 //
-// Bound by its chain of latencies (two loads, the network, a gather, a row).  Measured on B200: a step of 4 tables of 128
-// lookups of 16 features 10.2 us (17.0 in four launches), 26 tables of 128 13.9 (16.1).
+// Bound by its chain of latencies (two loads, the network, a gather, a row).  Measured on B200 (graph replay): a step of 4
+// tables of 128 lookups of 16 features 9.3 us (15.7 in four launches), 26 tables of 128 13.9 (16.1).
 #pragma once
 #include "small_sort.cuh"
 
