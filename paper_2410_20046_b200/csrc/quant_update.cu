@@ -302,10 +302,20 @@ int launch_quant_table(dqrm_ctx *ctx, const float *grad_rows, const int32_t *uni
     return DQRM_OK;
 }
 
-// (with the rows' (min, max) stored the compiler would take registers that cost a resident block: 190 K rows of 64 features
-// 38.9 us with four blocks, 48.7 without the bound; 108 K rows of 16 features 15.7 with three)
+// Blocks resident (with the rows' (min, max) stored the compiler would take registers that cost a block: 190 K rows of 64
+// features 38.9 us with four, 48.7 without the bound; 108 K rows of 16 features 15.7 with three; quantise and update of
+// rows of up to 32 features would take 85 registers and a block fewer: 131 K rows of 16 features 15.9 us with three, 16.6
+// with two, eight pipelined steps around it 376 and 387.  The others are best with what a minimum of one gives: without any
+// the update alone of 426 K rows of 128 features takes 88 us instead of 85)
+constexpr int stream_blocks(int mode, int lpr, int ch, bool track)
+{
+    if (ch > 1) return 1;
+    if (track) return lpr >= 16 ? 4 : 3;
+    return mode == MODE_FUSED && lpr < 16 ? 3 : 1;
+}
+
 template <int MODE, int LPR, int CH, bool EXACT, bool TRACK = false>
-__global__ void __launch_bounds__(QU_THREADS, TRACK && CH == 1 ? (LPR >= 16 ? 4 : 3) : 1)
+__global__ void __launch_bounds__(QU_THREADS, stream_blocks(MODE, LPR, CH, TRACK))
 row_stream_kernel(float *__restrict__ tables, const int64_t *__restrict__ row_off,
                   const int32_t *__restrict__ unique_rows, const int32_t *__restrict__ uniq_off,
                   const float *__restrict__ grad_rows, const u32 *__restrict__ absmax,
