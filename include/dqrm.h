@@ -164,8 +164,8 @@ int dqrm_grad_quant_int8(dqrm_ctx *ctx, const float *grad_rows, const int32_t *u
                          void *workspace, size_t workspace_bytes, void *stream);
 
 /* The same for a caller that knows on the host how many values (U*D) there can be, for
- * instance the size of its buffers: few values are quantised in one launch instead of three.
- * max_values only chooses the kernel; the result does not depend on it. */
+ * instance the size of its buffers: few values are quantised in one or two launches instead of
+ * three.  max_values only chooses the kernels; the result does not depend on it. */
 int dqrm_grad_quant_int8_bounded(dqrm_ctx *ctx, const float *grad_rows, const int32_t *uniq_off,
                                  int8_t *codes, float *grad_scales, int64_t max_values,
                                  void *workspace, size_t workspace_bytes, void *stream);
