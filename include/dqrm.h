@@ -348,7 +348,7 @@ int dqrm_decode_payload(dqrm_ctx *ctx, const uint8_t *payload, const float *scal
 
 /* ---- choice of the backward's sort (no counterpart in the paper) --------------------
  * dqrm_emb_bwd and dqrm_train_step order the batch's lookups by row before they sum
- * duplicates.  path 0 (default): per table, one block with a sorting network (up to about a
+ * duplicates.  path 0 (default): per table, one block (up to about two
  * thousand lookups a table), or one thread-block cluster (eight blocks, sixteen when the batch
  * has very few tables) in distributed shared memory; a batch with more lookups per table than
  * such a cluster holds takes path 1 by itself.  path 1: a least-significant-digit radix sort in

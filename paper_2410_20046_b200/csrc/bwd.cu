@@ -303,7 +303,7 @@ template <int CL, int EPT = 0>
 cudaError_t launch_cluster_sort(dqrm_ctx *ctx, csort::Args ca, int cap, cudaStream_t st)
 {
     ca.cap = cap;
-    const size_t smem = std::max(csort::smem_bytes(cap), (size_t)csort::THREADS * EPT * 2 * sizeof(ssort::u64));
+    const size_t smem = std::max(csort::smem_bytes(cap), EPT ? sizeof(uint2) * csort::SORT_ROOM : (size_t)0);
     static_assert(CL == csort::CLUSTER || EPT == 0, "");
     bool &raised = ctx->smem_raised[DQ_SMEM_SLOT_CSORT + (CL == csort::CLUSTER ? EPT : 3)];
     cudaError_t e = cudaSuccess;
@@ -333,36 +333,28 @@ cudaError_t launch_cluster_sort(dqrm_ctx *ctx, csort::Args ca, int cap, cudaStre
 }
 
 // The block sort; false where the batch is too large for it.  `per_table` lookups a table on average, with room for a
-// quarter more where bags are uneven.  Measured on B200 against the cluster sort (graph replay, 26 tables of 900 K rows,
-// us per batch): 128 lookups a table 3.5 against 12.3, 500 5.4 / 12.5, 1000 8.0 / 12.6, 2048 14.9 / 13.4; with 100
-// tables, whose clusters take turns, 1000 lookups 8.5 / 33.  Unless the batch has an index a bag, one table may hold most
-// of it: a cluster of blocks then stands by for every table (a table of
+// quarter more where bags are uneven.  Up to 256 the network, beyond it the radix sort.  Measured on B200 (graph replay, 26
+// tables of up to 6 M rows, us per batch; radix sort / network / cluster): 64 lookups a table 4.9 / 3.2, 256 4.9 / 4.1, 500
+// 4.7 / 6.2, 1000 5.8 / 8.2 / 12.6, 2000 8.2 / - / 13.3, one table of 3000 11.5 / - / 11.1.  Unless the batch has an index a
+// bag, one table may hold most of it: a cluster of blocks then stands by for every table (a table of
 // 12.8 K lookups beside 25 of 128: 22.8 us, 99 by one block in global memory, 34.8 in a cluster of whole batches; bags of
-// five everywhere 11.6, 9.2 without the clusters standing by).
-template <int THREADS, int EPT>
-cudaError_t launch_small_sort2(dqrm_ctx *ctx, const csort::Args &ca, cudaStream_t st)
-{
-    const size_t smem = ssort::smem_bytes(THREADS, EPT);
-    static_assert(THREADS >= csort::BINS && (size_t)THREADS * EPT * 2 * sizeof(ssort::u64) <= 48 * 1024, "");
-    return dq_launch(ssort::small_sort_kernel<THREADS, EPT>, dim3((unsigned)ctx->T), dim3(THREADS), smem, st, ca);
-}
-
+// five everywhere 9.9, 9.2 by the network without the clusters standing by).
 bool launch_small_sort(dqrm_ctx *ctx, const csort::Args &ca, int64_t per_table, bool even, cudaStream_t st, cudaError_t &e)
 {
     const int64_t want = even ? per_table : per_table + per_table / 4;
-    const bool many = ctx->T * csort::CLUSTER > 2 * ctx->num_sms;
-    if (want > (many ? 2048 : 1024)) return false;
+    if (want > 2048) return false;
+    const dim3 grid((unsigned)ctx->T), block(csort::THREADS);
+    constexpr size_t room = sizeof(uint2) * csort::SORT_ROOM;
+    static_assert(csort::SORT_ROOM >= 4 * csort::THREADS, "");
     if (!even) {
         const int cap = csort::shared_cap(ca.L);
         e = want <= 512    ? launch_cluster_sort<csort::CLUSTER, 1>(ctx, ca, cap, st)
             : want <= 1024 ? launch_cluster_sort<csort::CLUSTER, 2>(ctx, ca, cap, st)
                            : launch_cluster_sort<csort::CLUSTER, 4>(ctx, ca, cap, st);
-        return true;
-    }
-    if (want <= 256) e = launch_small_sort2<256, 1>(ctx, ca, st);
-    else if (want <= 512) e = launch_small_sort2<512, 1>(ctx, ca, st);
-    else if (want <= 1024) e = launch_small_sort2<512, 2>(ctx, ca, st);
-    else e = launch_small_sort2<1024, 2>(ctx, ca, st);
+    } else if (want <= 256) e = dq_launch(ssort::small_sort_kernel<256, 1>, grid, dim3(256), ssort::smem_bytes(256, 1), st, ca);
+    else if (want <= 512) e = dq_launch(ssort::block_sort_kernel<1>, grid, block, room, st, ca);
+    else if (want <= 1024) e = dq_launch(ssort::block_sort_kernel<2>, grid, block, room, st, ca);
+    else e = dq_launch(ssort::block_sort_kernel<4>, grid, block, room, st, ca);
     return true;
 }
 

@@ -17,57 +17,12 @@
 // (the kernel that sums them adds the tables' bases), or it counts the segment starts per
 // 2048-entry tile for a kernel that numbers them over the whole batch.
 #pragma once
-#include <cooperative_groups.h>
-#include "common.cuh"
-
+#include "sort_parts.cuh"
 
 namespace csort {
 
-namespace cg = cooperative_groups;
-
-constexpr int THREADS = 512;
-constexpr int WARPS = THREADS / 32;
 constexpr int CLUSTER = 8;            // blocks per table
 constexpr int CLUSTER_WIDE = 16;      // ... when the batch has so few tables that eight blocks each would leave most SMs idle
-constexpr int BINS = 256;
-
-struct Args {
-    const int32_t *indices;
-    const int32_t *offsets;
-    const int64_t *row_off;
-    int T, B;
-    int64_t L;
-    u32 *keys_out, *vals_out;       // [L] sorted result
-    uint2 *gp[2];                   // [L] global staging of pairs (tables too large for shared memory)
-    int cap;                        // pairs per block that fit in shared memory
-    int payload_position;           // 0: payload = row of grad_out [B][T][D]; 1: payload = position of the lookup in indices
-    int *status;
-    u32 *tile_heads;                // [ceil(L / 2048)] zeroed by the caller: segment heads per tile of the sorted order
-    // lists_by_table: instead of the per-tile head counts (from which a later kernel numbers the segments over the
-    // whole batch), every cluster numbers its own table's segments from 0 and leaves
-    //   seg_start[tb0 + t + u] = sorted position where the table's segment u begins, [.. + count] = the table's end
-    //   chunk_first[c]         = the table's segment that holds sorted entry c << ck_shift (for c inside the table)
-    //   table_cnt[t], tb[t]    = segments and first sorted position of table t (tb[T] = L)
-    //                            (cnt_broken instead when boundary offsets are unusable)
-    // and zeroes what the kernel behind it counts in (tile_done[c], absmax[t]); that kernel, which sums the segments,
-    // adds the tables' bases
-    int lists_by_table;
-    u32 *seg_start, *chunk_first, *table_cnt, *tb, *absmax;
-    uint2 *tile_done;
-    int ck_shift;
-    u32 cnt_broken;
-};
-
-}  // namespace csort
-
-namespace ssort {
-// one block's sort of table t (small_sort.cuh): its lookups [tb0, tb1), at most THREADS * EPT of them, and its lists; shared
-// memory for twice that many pairs
-template <int THREADS, int EPT>
-__device__ void sort_table(const csort::Args &a, int t, int64_t tb0, int64_t tb1, unsigned long long *s_net);
-}
-
-namespace csort {
 
 __device__ __forceinline__ u32 *remote(cg::cluster_group &cluster, u32 *p, unsigned rank)
 {
@@ -75,7 +30,7 @@ __device__ __forceinline__ u32 *remote(cg::cluster_group &cluster, u32 *p, unsig
 }
 
 // lanes of the warp that hold the same 8-bit digit as this lane (one call by all lanes; a lane without an
-// entry matches nobody)
+// entry matches nobody).  Slow, but hidden behind the stores into the other blocks' shared memory
 __device__ __forceinline__ u32 same_digit_lanes(u32 d, bool valid)
 {
     const u32 peers = __match_any_sync(0xffffffffu, valid ? d : 256u + (threadIdx.x & 31));
@@ -88,14 +43,14 @@ __device__ __forceinline__ u32 same_digit_lanes(u32 d, bool valid)
 // of 64 K lookups)
 //
 // EPT > 0: for small batches whose bags may be uneven.  A table of up to THREADS * EPT lookups, which is nearly all of them,
-// is sorted by the cluster's first block alone, with the network of small_sort.cuh, and only a larger one by the cluster.
+// is sorted by the cluster's first block alone (sort_parts.cuh), and only a larger one by the cluster.
 template <int CL, int EPT>
 __global__ void __launch_bounds__(THREADS, CL > 8 ? 1 : 2)
-cluster_sort_kernel(const Args a)
+cluster_sort_kernel(const __grid_constant__ Args a)
 {
     dq_wait_before();
     extern __shared__ uint2 s_dyn[];               // pair buffers [2][cap]: (row within table, payload)
-    __shared__ u32 s_cnt[WARPS][BINS];
+    __shared__ __align__(16) u32 s_cnt[WARPS][BINS];
     __shared__ u32 s_hist[BINS];
     __shared__ u32 s_scan[BINS / 32];
     __shared__ u32 s_wheads[WARPS];                // write-out: segment starts in each warp's part of the slice
@@ -108,34 +63,18 @@ cluster_sort_kernel(const Args a)
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const u32 lt = (1u << lane) - 1u;
 
-    int64_t tb0 = __ldg(a.offsets + (int64_t)t * a.B), tb1 = __ldg(a.offsets + (int64_t)(t + 1) * a.B);
-    if (tb0 < 0 || tb1 < tb0 || tb1 > a.L ||
-        (a.lists_by_table && ((t == 0 && tb0 != 0) || (t == a.T - 1 && tb1 != a.L)))) {
-        if (threadIdx.x == 0 && c == 0) {
-            dq_report(a.status, DQRM_ERR_INDEX_RANGE);
-            if (a.lists_by_table) {                // nothing is summed; the quantiser behind finds an empty gradient
-                a.table_cnt[t] = a.cnt_broken;
-                a.absmax[t] = 0u;
-            }
-        }
-        return;                                    // uniform over the cluster
-    }
+    const int64_t tb0 = __ldg(a.offsets + (int64_t)t * a.B), tb1 = __ldg(a.offsets + (int64_t)(t + 1) * a.B);
+    const int64_t r0 = __ldg(a.row_off + t), nrows = __ldg(a.row_off + t + 1) - r0;
+    if (broken_table(a, t, tb0, tb1, c == 0 && threadIdx.x == 0)) return;         // uniform over the cluster
     const int64_t n = tb1 - tb0;
-    if (a.lists_by_table && c == 0 && threadIdx.x == 0) {
-        a.tb[t] = (u32)tb0;
-        if (t == a.T - 1) a.tb[a.T] = (u32)tb1;
-        a.absmax[t] = 0u;
-        if (n == 0) a.table_cnt[t] = 0u;
-    }
+    if (a.lists_by_table && c == 0 && threadIdx.x == 0) open_table(a, t, tb0, tb1);
     if constexpr (EPT > 0) {
         if (n <= THREADS * EPT) {
-            if (c == 0) ssort::sort_table<THREADS, EPT>(a, t, tb0, tb1, reinterpret_cast<unsigned long long *>(s_dyn));
+            if (c == 0) sort_alone<EPT>(a, t, (u32)tb0, (u32)tb1, &s_cnt[0][0], s_dyn);
             return;
         }
     }
     if (n == 0) return;
-    const int64_t r0 = __ldg(a.row_off + t);
-    const int64_t nrows = __ldg(a.row_off + t + 1) - r0;
     const int npc = (int)(((n + CL - 1) / CL + 31) / 32 * 32);      // pairs per block
     const bool in_smem = npc <= a.cap;
     const int my_n = (int)max((int64_t)0, min((int64_t)npc, n - (int64_t)c * npc));

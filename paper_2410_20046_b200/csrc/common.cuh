@@ -308,6 +308,20 @@ __device__ __forceinline__ void dq_report(int *status, int code)
     atomicCAS(status, 0, code);   // first error wins
 }
 
+// Lanes of the warp that hold the same digit as this lane; called by all lanes together, a lane without an entry matches nobody.
+// mask: a word for every digit, zero before and after.  (An OR into shared memory, a read and a clear take the SM 10 clocks a
+// call with sixteen warps at it; __match_any_sync 59, eight votes 28.)
+__device__ __forceinline__ u32 dq_same_digit_lanes(u32 *mask, u32 d, bool valid)
+{
+    const u32 lane = threadIdx.x & 31;
+    if (valid) atomicOr(mask + d, 1u << lane);
+    __syncwarp();
+    const u32 peers = valid ? *reinterpret_cast<volatile u32 *>(mask + d) : 0u;
+    __syncwarp();
+    if (valid && (peers & ((1u << lane) - 1u)) == 0u) *reinterpret_cast<volatile u32 *>(mask + d) = 0u;
+    return peers;
+}
+
 // table that owns arena row `key`: largest t with row_off[t] <= key
 __device__ __forceinline__ int dq_table_of(const int64_t *row_off, int T, int64_t key)
 {

@@ -1,16 +1,20 @@
-// Per-table stable sort of a small batch's lookups by row: one block per table, a bitonic network over
-// (row, position) held in registers.  At a few hundred to a few thousand lookups a table the radix sort of
-// cluster_sort.cuh is all fixed cost (digit tables, cluster barriers, three passes for large tables): 128 lookups a table take
-// 3.5 us here and 12.3 there.  The network needs log2(n) (log2(n) + 1) / 2 steps whatever the row count; most of them
-// stay inside a warp, and unrolled they cost about 0.15 us each (with the steps in a loop, 1.5 times that).
+// Per-table stable sort of a small batch's lookups by row: one block per table.  At up to two thousand lookups a table the
+// sort of cluster_sort.cuh is all fixed cost (cluster barriers, three passes through other blocks' memory for large tables).
 //
-// Every thread holds EPT consecutive entries: steps across less than EPT entries are register moves, across less than
+// Up to 256 lookups: a bitonic network over (row, position) held in registers: log2(n) (log2(n) + 1) / 2 steps whatever the row
+// count; most of them stay inside a warp, and unrolled they cost about 0.15 us each (with the steps in a loop, 1.5 times
+// that).  Every thread holds EPT consecutive entries: steps across less than EPT entries are register moves, across less than
 // 32 * EPT shuffles, wider ones go through shared memory (two buffers in turn, one barrier a step).  Row and position
-// make every key distinct, so the order is that of a stable sort.  A table with more lookups than the block holds
+// make every key distinct, so the order is that of a stable sort.  Beyond that: the radix sort of sort_parts.cuh.
+//
+// A table with more lookups than the block holds
 // is sorted by its cluster where the batch may have one (cluster_sort_kernel with EPT > 0).  By the block in global memory,
 // with 8-bit digits, only where a batch with as many lookups as bags is uneven all the same, and in the one-launch step, which
 // takes no batch in which that is the longer way: 7 ns a lookup against 2 in a cluster (12.8 K lookups).
 // The lists that it leaves are those of the cluster sort's lists_by_table.
+//
+// Kernels take their arguments as grid constants: the functions that stay out of line get a pointer to them, and without that
+// every thread would first copy them to its stack (128 lookups a table 4.0 -> 3.6 us).
 #pragma once
 #include "cluster_sort.cuh"
 
@@ -104,7 +108,7 @@ __device__ __noinline__ const uint2 *sort_in_memory(const csort::Args &a, int t,
             const bool valid = i0 + lane < w1;
             const uint2 pr = valid ? src[i0 + lane] : make_uint2(0u, 0u);
             const u32 d = (pr.x >> shift) & 255u;
-            const u32 peers = csort::same_digit_lanes(d, valid);
+            const u32 peers = __match_any_sync(0xffffffffu, valid ? d : 256u + lane);       // (slow, but without room of its own)
             const int leader = __ffs(peers) - 1;
             u32 base = 0;
             if (valid && lane == leader) { base = s_cnt[warp * BINS + d]; s_cnt[warp * BINS + d] = base + __popc(peers); }
@@ -278,22 +282,8 @@ __device__ __forceinline__ bool offsets_fall(const csort::Args &a, int t)
 }
 
 template <int THREADS, int EPT>
-__device__ void sort_table(const csort::Args &a, int t, int64_t tb0, int64_t tb1, u64 *s_net)
-{
-    const int64_t n = tb1 - tb0, nrows = __ldg(a.row_off + t + 1) - __ldg(a.row_off + t);
-    bool bad = n != a.B && offsets_fall<THREADS>(a, t);       // (otherwise every lookup looks at its own bag's offsets)
-    if (n == 0) {                                  // (its empty lists have been written)
-        if (bad) dq_report(a.status, DQRM_ERR_INDEX_RANGE);
-        return;
-    }
-    sort_in_block<THREADS, EPT>(a, t, tb0, n, nrows, s_net, bad);
-    if (bad) dq_report(a.status, DQRM_ERR_INDEX_RANGE);
-    write_table<THREADS>(a, t, tb0, tb1, s_net, nullptr);
-}
-
-template <int THREADS, int EPT>
 __global__ void __launch_bounds__(THREADS)
-small_sort_kernel(const csort::Args a)
+small_sort_kernel(const __grid_constant__ csort::Args a)
 {
     dq_wait_before();
     extern __shared__ u64 s_net[];                 // [2][THREADS * EPT]
@@ -315,12 +305,39 @@ small_sort_kernel(const csort::Args a)
         if (n == 0) a.table_cnt[t] = 0u;
     }
     if (n <= THREADS * EPT) {
-        sort_table<THREADS, EPT>(a, t, tb0, tb1, s_net);
+        const int64_t nrows = __ldg(a.row_off + t + 1) - __ldg(a.row_off + t);
+        bool bad = n != a.B && offsets_fall<THREADS>(a, t);       // (otherwise every lookup looks at its own bag's offsets)
+        if (n > 0) sort_in_block<THREADS, EPT>(a, t, tb0, n, nrows, s_net, bad);
+        if (bad) dq_report(a.status, DQRM_ERR_INDEX_RANGE);
+        if (n > 0) write_table<THREADS>(a, t, tb0, tb1, s_net, nullptr);
     } else {                                       // (a one-index batch that is none)
         if (offsets_fall<THREADS>(a, t)) dq_report(a.status, DQRM_ERR_INDEX_RANGE);
         const int64_t nrows = __ldg(a.row_off + t + 1) - __ldg(a.row_off + t);
         const uint2 *mem = sort_in_memory<THREADS>(a, t, tb0, n, nrows, reinterpret_cast<u32 *>(s_net));
         write_table<THREADS>(a, t, tb0, tb1, nullptr, mem);
+    }
+}
+
+// The same for larger tables: up to THREADS * E lookups by the radix sort of sort_parts.cuh
+template <int E>
+__global__ void __launch_bounds__(csort::THREADS)
+block_sort_kernel(const __grid_constant__ csort::Args a)
+{
+    dq_wait_before();
+    extern __shared__ __align__(16) uint2 s_pair[];              // [THREADS * E]
+    __shared__ __align__(16) u32 s_cnt[csort::WARPS * csort::BINS];
+    const int t = blockIdx.x;
+    const int64_t tb0 = __ldg(a.offsets + (int64_t)t * a.B), tb1 = __ldg(a.offsets + (int64_t)(t + 1) * a.B);
+    if (csort::broken_table(a, t, tb0, tb1, threadIdx.x == 0)) return;
+    if (threadIdx.x == 0) csort::open_table(a, t, tb0, tb1);
+    const int64_t n = tb1 - tb0;
+    if (n <= csort::THREADS * E) {
+        csort::sort_alone<E>(a, t, (u32)tb0, (u32)tb1, s_cnt, s_pair);
+    } else {                                       // (a one-index batch that is none)
+        if (offsets_fall<csort::THREADS>(a, t)) dq_report(a.status, DQRM_ERR_INDEX_RANGE);
+        const int64_t nrows = __ldg(a.row_off + t + 1) - __ldg(a.row_off + t);
+        const uint2 *mem = sort_in_memory<csort::THREADS>(a, t, tb0, n, nrows, s_cnt);
+        csort::write_part<1>(a, t, (u32)tb0, (u32)tb1, mem, (int)n, 0u, 0xffffffffu);
     }
 }
 

@@ -47,7 +47,7 @@ static_assert(MID_WORDS >= (size_t)WARPS * csort::BINS && MID_WORDS >= (size_t)T
 inline size_t smem_bytes(int T) { return (size_t)THREADS * 2 * sizeof(u64) + (MID_WORDS + T + 1) * sizeof(u32); }
 
 __global__ void __launch_bounds__(THREADS)
-small_step_kernel(const Args x)
+small_step_kernel(const __grid_constant__ Args x)
 {
     extern __shared__ u64 s_net[];                 // [2][THREADS]
     u32 *s_mid = reinterpret_cast<u32 *>(s_net + 2 * THREADS);

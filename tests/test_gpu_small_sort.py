@@ -71,3 +71,27 @@ def test_uneven_tables(oracle, name, rows):
     # at most 60,000 terms of magnitude below 6 in FP64 in two orders, each sum rounded once
     np.testing.assert_allclose(gr, o_gr, rtol=2.0 ** -23, atol=12.0 * max(counts) ** 2 * 2.0 ** -53)
     c.ctx.close()
+
+
+@pytest.mark.parametrize("rows", [1 << 16, (1 << 16) + 1, 1 << 24, 20_000_000])      # two, three and four digits
+@pytest.mark.parametrize("n", [257, 511, 512, 513, 1025, 2047, 2048])
+def test_block_radix_sort(oracle, rows, n):
+    """The block's radix sort at the edges of its groups and of its digits; rows at both ends of the table, and one that a
+    third of the lookups hit."""
+    D, T = 4, 2
+    wl = W.Workload("radix", (rows, rows), D=D, B=n, alpha=None)
+    rng = np.random.default_rng(rows + n)
+    idx = rng.integers(0, rows, T * n).astype(np.int32)
+    idx[rng.random(T * n) < 0.33] = rows // 3
+    idx[[0, 1, n - 1, n, T * n - 1]] = [rows - 1, 0, rows - 1, 0, rows - 1]
+    off = np.arange(T * n + 1, dtype=np.int32)
+    go = rng.standard_normal((n, T, D)).astype(np.float32)
+    c = Case(wl)
+    c.ctx.profile_begin()
+    ur, uo, gr = c.gpu_bwd(idx, off, go)
+    assert "small_sort_kernel" in c.ctx.profile_end()
+    o_ur, o_uo, o_gr = oracle.emb_bwd(go, T, D, n, idx, off)
+    assert bit_equal(uo, o_uo) and bit_equal(ur, o_ur)
+    # at most 800 terms of magnitude below 6 in FP64 in two orders, each sum rounded once
+    np.testing.assert_allclose(gr, o_gr, rtol=2.0 ** -23, atol=12.0 * 800 ** 2 * 2.0 ** -53)
+    c.ctx.close()
