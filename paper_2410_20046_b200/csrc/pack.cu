@@ -191,14 +191,14 @@ packed_fwd_kernel(const PfArgs a)
     dq_wait_before();
     constexpr int GPB = PK_THREADS / LPR;
     const int units = a.D / EPL;
-    const int t = blockIdx.y;
+    const int t = blockIdx.x;
     const int lane = threadIdx.x % LPR, grp = threadIdx.x / LPR;
     const float s = __ldg(a.scales + t);
     const int64_t r0 = __ldg(a.row_off + t);
     const int32_t nrows = (int32_t)(__ldg(a.row_off + t + 1) - r0);
     const int64_t g0 = (int64_t)t * a.B;
     bool bad = false;
-    for (int i = blockIdx.x * GPB + grp; i < a.B; i += gridDim.x * GPB)
+    for (int i = blockIdx.y * GPB + grp; i < a.B; i += gridDim.y * GPB)
         pool_bag<BITS, EPL, LPR, CH>(a, r0, nrows, s, units, __ldg(a.offsets + g0 + i), __ldg(a.offsets + g0 + i + 1),
                                      a.out + ((int64_t)i * a.T + t) * a.D, lane, bad);
     if (bad) dq_report(a.status, DQRM_ERR_INDEX_RANGE);
@@ -217,7 +217,7 @@ packed_fwd_onehot_kernel(const PfArgs a)
     constexpr int RPW = 32 / LPR;
     constexpr int WPB = PK_THREADS / 32;
     const int units = a.D / EPL;
-    const int t = blockIdx.y;
+    const int t = blockIdx.x;
     const int wlane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int lane = wlane % LPR, grp = wlane / LPR;
     const float s = __ldg(a.scales + t);
@@ -226,7 +226,7 @@ packed_fwd_onehot_kernel(const PfArgs a)
     const int64_t g0 = (int64_t)t * a.B;
     const int TD4 = a.T * (a.D >> 2);            // 128-bit vectors between the output rows of bags i and i+1
     bool bad = false;
-    for (int i0 = (blockIdx.x * WPB + warp) * 32; i0 < a.B; i0 += gridDim.x * (WPB * 32)) {
+    for (int i0 = (blockIdx.y * WPB + warp) * 32; i0 < a.B; i0 += gridDim.y * (WPB * 32)) {
         const int i = i0 + wlane;
         int32_t idx = 0;
         bool single = false;
@@ -329,7 +329,8 @@ int launch_pfwd(dqrm_ctx *ctx, const PfArgs &a, cudaStream_t st)
     const int cap = (ctx->num_sms * 32 + ctx->T - 1) / ctx->T;
     if (bx > cap) bx = cap;
     if (bx < 1) bx = 1;
-    dim3 grid((unsigned)bx, (unsigned)ctx->T);
+    // (all tables' blocks for the same bags side by side: see the forward; 852 K rows of 64 features 42.5 -> 40.6 us)
+    const dim3 grid((unsigned)ctx->T, (unsigned)bx);
     DQRM_CUDA_TRY(ctx, (onehot ? dq_launch(packed_fwd_onehot_kernel<BITS, EPL, LPR, CH>, grid, dim3(PK_THREADS), 0, st, a)
                                : dq_launch(packed_fwd_kernel<BITS, EPL, LPR, CH>, grid, dim3(PK_THREADS), 0, st, a)));
     dq_mark(ctx, st, DQ_K_PACKED_FWD);
