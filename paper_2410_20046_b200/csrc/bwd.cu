@@ -18,6 +18,7 @@
 #include <algorithm>
 #include "common.cuh"
 #include "seg_reduce.cuh"
+#include "seg_groups.cuh"
 #include "cluster_sort.cuh"
 #include "radix_sort.cuh"
 #include "small_sort.cuh"
@@ -33,11 +34,12 @@ constexpr int ST_WARPS = ST_THREADS / 32;
 struct Layout {
     int passes, digit_bits;                    // radix sort: digits of the row number within a table
     int64_t radix_tiles, num_tiles;
-    // the summing kernel: log2 of the entries between two of chunk_first, small tiles, tiles, tiles of a warp's range
+    // the summing kernel: log2 of the entries between two of chunk_first; rows of more than 32 features: small tiles, tiles, tiles of
+    // a warp's range; narrower ones: entries of a lane group's range, ranges of warps
     int sum_shift;
     bool sum_small;
-    int64_t sum_tiles;
-    int range_tiles;
+    int64_t sum_tiles, sum_ranges;
+    int range_tiles, sum_span;
     size_t absmax, tile_heads, tile0, tile_table, totals, tilehist;
     size_t keys_a, vals_a, pairs_a, pairs_b, seg_start, chunk_first, tile_done, partials, group_partials, table_cnt, tb;
     size_t total;
@@ -51,16 +53,19 @@ Layout make_layout(const dqrm_ctx *ctx, int64_t L)
     int64_t Lc = L < 1 ? 1 : L;
     y.num_tiles = (Lc + ST_TILE - 1) / ST_TILE;
     y.radix_tiles = rsort::max_tiles(ctx->T, Lc);
-    // the sum: every warp that the GPU holds at once walks one range of tiles
-    const int lpr = segred::lanes_per_row(ctx->D);
-    int64_t warps = (int64_t)ctx->num_sms * segred::blocks_per_sm(lpr) / segred::column_blocks(ctx->D) * segred::WARPS;
+    // the sum: every warp that the GPU holds at once walks one range
+    int64_t warps = segred::takes_groups(ctx->D) ? (int64_t)ctx->num_sms * segred::GROUPS_BLOCKS * segred::GROUPS_THREADS / 32
+                                                 : (int64_t)ctx->num_sms * segred::BLOCKS_PER_SM / segred::column_blocks(ctx->D) * segred::WARPS;
     if (warps < 1) warps = 1;
     y.sum_small = Lc < 96 * warps;         // (three tiles of 32 a warp: 160 K rows of 192 bytes 38.9 -> 28.7 us, 208 K of
                                               // 256 bytes 30.7 -> 28.7; at 852 K rows tiles of 32 are 2 us the faster)
-    const int I = segred::tile_entries(lpr, y.sum_small);
-    y.sum_shift = segred::chunk_shift(lpr, y.sum_small);
+    const int I = segred::tile_entries(y.sum_small);
+    y.sum_shift = segred::takes_groups(ctx->D) ? segred::CHUNK_SHIFT : segred::chunk_shift(y.sum_small);
     y.sum_tiles = (Lc + I - 1) / I;
     y.range_tiles = (int)((y.sum_tiles + warps - 1) / warps);
+    const int64_t groups = 32 / segred::lanes_per_row(ctx->D), chunk = (int64_t)1 << segred::CHUNK_SHIFT;
+    y.sum_span = (int)(((Lc + warps * groups - 1) / (warps * groups) + chunk - 1) / chunk * chunk);
+    y.sum_ranges = (Lc + y.sum_span * groups - 1) / (y.sum_span * groups);
     size_t o = 0;
     auto take = [&](size_t bytes) { size_t at = o; o = align_up(o + bytes, 256); return at; };
     y.absmax = take(sizeof(u32) * ctx->T);
@@ -232,17 +237,17 @@ seg_emit_kernel(const u32 *__restrict__ keys, int64_t L, const u32 *__restrict__
 }
 
 // ---------------------------------------------------------------------------------
-template <int LPR, int VEC>
+template <int VEC>
 int launch_sum(dqrm_ctx *ctx, const segred::Args &a, bool small, cudaStream_t st)
 {
     using namespace segred;
     const size_t smem = smem_bytes(ctx->T);
     const int64_t ranges = (a.num_tiles + a.range_tiles - 1) / a.range_tiles;
     const dim3 grid((unsigned)((ranges * a.columns + WARPS - 1) / WARPS));
-    const bool exact = ctx->D % (LPR * VEC) == 0;
-    constexpr bool wide = LPR == 32 && VEC == 4;             // (only those rows may have several blocks of features)
+    const bool exact = ctx->D % (32 * VEC) == 0;
+    constexpr bool wide = VEC == 4;                          // (only those rows may have several blocks of features)
 #define DQ_SUM(EXACT, SMALL, COLS) \
-    DQRM_CUDA_TRY(ctx, (dq_launch(seg_sum_kernel<LPR, VEC, EXACT, SMALL, COLS>, grid, dim3(THREADS), smem, st, a)))
+    DQRM_CUDA_TRY(ctx, (dq_launch(seg_sum_kernel<VEC, EXACT, SMALL, COLS>, grid, dim3(THREADS), smem, st, a)))
 #define DQ_SUM2(SMALL)                                                              \
     do {                                                                            \
         if (a.columns > 1 && exact) DQ_SUM(true, SMALL, wide);                      \
@@ -250,10 +255,24 @@ int launch_sum(dqrm_ctx *ctx, const segred::Args &a, bool small, cudaStream_t st
         else if (exact) DQ_SUM(true, SMALL, false);                                 \
         else DQ_SUM(false, SMALL, false);                                           \
     } while (0)
-    if (LPR == 32 && small) DQ_SUM2(LPR == 32);
+    if (small) DQ_SUM2(true);
     else DQ_SUM2(false);
 #undef DQ_SUM2
 #undef DQ_SUM
+    dq_mark(ctx, st, DQ_K_SEG_SUM);
+    return DQRM_OK;
+}
+
+template <int LPR>
+int launch_sum_groups(dqrm_ctx *ctx, const segred::Args &a, cudaStream_t st)
+{
+    using namespace segred;
+    // (small batches: smaller blocks, on more SMs)
+    unsigned warps = GROUPS_THREADS / 32;
+    while (warps > 2 && a.ranges < warps * (unsigned)ctx->num_sms) warps /= 2;
+    const dim3 grid((a.ranges + warps - 1) / warps), block(warps * 32);
+    if (ctx->D == LPR * 4) DQRM_CUDA_TRY(ctx, (dq_launch(seg_groups_kernel<LPR, true>, grid, block, smem_bytes(ctx->T), st, a)));
+    else DQRM_CUDA_TRY(ctx, (dq_launch(seg_groups_kernel<LPR, false>, grid, block, smem_bytes(ctx->T), st, a)));
     dq_mark(ctx, st, DQ_K_SEG_SUM);
     return DQRM_OK;
 }
@@ -511,16 +530,20 @@ int dq_launch_bwd_sum(dqrm_ctx *ctx, const float *grad_out, int32_t *unique_rows
     a.group_partials = reinterpret_cast<double *>(ws + y.group_partials);
     a.absmax = reinterpret_cast<u32 *>(ws + y.absmax);
     a.T = ctx->T; a.D = ctx->D;
-    a.L = L; a.G = (int64_t)ctx->T * B; a.num_tiles = y.sum_tiles;
+    a.L = L; a.G = (int64_t)ctx->T * B;
+    a.num_tiles = y.sum_tiles;
     a.range_tiles = y.range_tiles;
     a.columns = segred::column_blocks(D);
+    a.span = (u32)y.sum_span;
+    a.ranges = (u32)y.sum_ranges;
     a.status = ctx->d_status;
-    if (D <= 4) return launch_sum<4, 1>(ctx, a, y.sum_small, st);
-    if (D <= 8) return launch_sum<4, 2>(ctx, a, y.sum_small, st);
-    if (D <= 16) return launch_sum<4, 4>(ctx, a, y.sum_small, st);
-    if (D <= 32) return launch_sum<8, 4>(ctx, a, y.sum_small, st);
-    if (D <= 64) return launch_sum<32, 2>(ctx, a, y.sum_small, st);
-    return launch_sum<32, 4>(ctx, a, y.sum_small, st);
+    if (!segred::takes_groups(D)) return D <= 64 ? launch_sum<2>(ctx, a, y.sum_small, st) : launch_sum<4>(ctx, a, y.sum_small, st);
+    switch (segred::lanes_per_row(D)) {
+    case 1: return launch_sum_groups<1>(ctx, a, st);
+    case 2: return launch_sum_groups<2>(ctx, a, st);
+    case 4: return launch_sum_groups<4>(ctx, a, st);
+    default: return launch_sum_groups<8>(ctx, a, st);
+    }
 }
 
 // The one-launch step takes tables of up to 512 lookups and 16 K gathered values, up to 4096 lookups in all (what a block

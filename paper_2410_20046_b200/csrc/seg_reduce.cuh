@@ -10,18 +10,17 @@
 // entries at a time.  The sum is bound by the latency of the chain index -> payload -> row: indices are fetched a
 // tile ahead, the rows of the next tile are asked into L2 as soon as its payloads are there (without that the kernel
 // took 89 instead of 71 us on 852 K rows of 256 bytes, 541 instead of 318 us on 8.5 M), and the next batch of rows is
-// requested before the present one is summed.  A row takes LPR lanes with VEC features each.  Rows of 36 features and
-// more take the whole warp: every branch on a run's end is then uniform and a run that goes on is simply carried in
-// registers.  Narrower rows are taken by 32/LPR lane groups at once, C consecutive entries each; a segmented scan over
-// the groups (shuffles) joins the runs that cross them.  Only a run cut by the edge of a warp's range leaves a partial
+// requested before the present one is summed.  A row takes the whole warp, VEC features a lane (rows of up to 32 features go
+// to seg_groups.cuh): every branch on a run's end is then uniform and a run that goes on is simply carried in
+// registers.  Only a run cut by the edge of a warp's range leaves a partial
 // in global memory; the warp that brings a run's last partial adds all of them, in order (nobody waits; the pieces of a
 // long run are first added by groups of 32 ranges, or one warp's chain over hundreds of them is what the kernel waits
 // for).  All sums are
 // FP64 and have a shape fixed by the entry positions and the launch, so results are reproducible.  The per-table
 // abs-max of the rounded sums is collected on the way.
 //
-// Measured on B200 (cold L2, alone) against the kernel before it, which walked 32-entry chunks per lane group and left
-// a partial per chunk for a second launch: 426 K rows of 64 bytes 26.7 + 10.6 -> 25.4 us, 852 K rows of 256 bytes
+// Measured on B200 (cold L2, alone) against a kernel that walked 32-entry chunks per lane group and left
+// a partial per chunk for a second launch: 852 K rows of 256 bytes
 // 69.9 + 12.9 -> 70.9 us, 8.5 M lookups of 256-byte rows 330 + 63 -> 318 us.
 #pragma once
 #include "common.cuh"
@@ -33,19 +32,17 @@ constexpr int WARPS = THREADS / 32;
 constexpr u32 FOLD_GROUP = 32;               // ranges whose pieces of one run are added before the groups' sums are
 constexpr u32 CNT_BROKEN = 0xFFFFFFFFu;      // table_cnt[t]: the table's boundary offsets were unusable (reported)
 
-// lanes per row and features per lane for feature size D (D > 128: 128 features per block of the grid's y)
-__host__ __device__ constexpr int lanes_per_row(int D) { return D <= 16 ? 4 : D <= 32 ? 8 : 32; }
-__host__ __device__ constexpr int floats_per_lane(int D) { return D <= 4 ? 1 : D <= 8 ? 2 : D <= 32 ? 4 : D <= 64 ? 2 : 4; }
+// features per lane for feature size D (D > 128: 128 features per warp)
+__host__ __device__ constexpr int floats_per_lane(int D) { return D <= 64 ? 2 : 4; }
 __host__ __device__ constexpr int column_blocks(int D) { return (D + 127) / 128; }
-// rows of a lane group in flight, entries of a tile, resident blocks.  Lane groups: eight rows and two blocks (with
-// three the kernel spills and takes 31 us instead of 25 at 426 K rows of 64 bytes); whole warps: 4 KB in flight (two
+// rows in flight, entries of a tile, resident blocks: 4 KB in flight (two
 // batches in turn) and three blocks (four blocks: 78 instead of 71 us at 852 K rows of 256 bytes)
-__host__ __device__ constexpr int batch_entries(int lpr, int vec, bool small) { return lpr == 32 ? (small ? 4 : 16 / vec) : 8; }
+__host__ __device__ constexpr int batch_entries(int vec, bool small) { return small ? 4 : 16 / vec; }
 // A warp that has one tile takes its batches of rows one after the other, 4 to 8 us for 32 rows, so a batch of wide
 // rows that would give every resident warp less than three tiles of 32 entries is cut into tiles of 8
-__host__ __device__ constexpr int tile_entries(int lpr, bool small) { return lpr == 4 ? 64 : lpr == 32 && small ? 8 : 32; }
-__host__ __device__ constexpr int chunk_shift(int lpr, bool small) { return lpr == 32 && small ? 3 : 5; }    // of chunk_first
-__host__ __device__ constexpr int blocks_per_sm(int lpr) { return lpr == 32 ? 3 : 2; }
+__host__ __device__ constexpr int tile_entries(bool small) { return small ? 8 : 32; }
+__host__ __device__ constexpr int chunk_shift(bool small) { return small ? 3 : 5; }    // of chunk_first
+constexpr int BLOCKS_PER_SM = 3;
 
 struct Args {
     const u32 *keys, *vals, *seg_start, *chunk_first;
@@ -68,9 +65,10 @@ struct Args {
     double *group_partials;     // [ranges / 32 + 1][2][D]: the same for groups of 32 ranges
     u32 *absmax;                // [T] zero
     int T, D;
-    int64_t L, G, num_tiles;
-    int range_tiles;            // tiles per warp
-    int columns;                // blocks of 128 features
+    int64_t L, G;
+    int64_t num_tiles;          // rows that take a warp: tiles, tiles of a warp's range, blocks of 128 features
+    int range_tiles, columns;
+    u32 span, ranges;           // rows that take a lane group: entries of a group's range, a multiple of eight, and ranges of warps
     int *status;
 };
 
@@ -87,18 +85,11 @@ __device__ __forceinline__ int last_not_above(const u32 *list, int lo, int T, u3
     return lo;
 }
 
-// VEC consecutive floats (1, 2 or 4)
+// VEC consecutive floats (2 or 4)
 template <int VEC> struct Vec;
-template <> struct Vec<1> { typedef float type; };
 template <> struct Vec<2> { typedef float2 type; };
 template <> struct Vec<4> { typedef float4 type; };
 
-__device__ __forceinline__ float ld_row(const float *p, uint64_t pol)
-{
-    float v;
-    asm volatile("ld.global.nc.L2::cache_hint.f32 %0, [%1], %2;\n" : "=f"(v) : "l"(p), "l"(pol));
-    return v;
-}
 __device__ __forceinline__ float2 ld_row(const float2 *p, uint64_t pol)
 {
     float2 v;
@@ -106,24 +97,18 @@ __device__ __forceinline__ float2 ld_row(const float2 *p, uint64_t pol)
     return v;
 }
 __device__ __forceinline__ float4 ld_row(const float4 *p, uint64_t pol) { return dq_ld_nc(p, pol); }
-__device__ __forceinline__ void st_row(float *p, float v, uint64_t pol)
-{
-    asm volatile("st.global.L2::cache_hint.f32 [%0], %1, %2;\n" ::"l"(p), "f"(v), "l"(pol) : "memory");
-}
 __device__ __forceinline__ void st_row(float2 *p, const float2 &v, uint64_t pol)
 {
     asm volatile("st.global.L2::cache_hint.v2.f32 [%0], {%1, %2}, %3;\n" ::"l"(p), "f"(v.x), "f"(v.y), "l"(pol) : "memory");
 }
 __device__ __forceinline__ void st_row(float4 *p, const float4 &v, uint64_t pol) { dq_st_keep(p, v, pol); }
 
-__device__ __forceinline__ void add(double (&acc)[1], float v) { acc[0] += (double)v; }
 __device__ __forceinline__ void add(double (&acc)[2], const float2 &v) { acc[0] += (double)v.x; acc[1] += (double)v.y; }
 __device__ __forceinline__ void add(double (&acc)[4], const float4 &v)
 {
     acc[0] += (double)v.x; acc[1] += (double)v.y; acc[2] += (double)v.z; acc[3] += (double)v.w;
 }
 // rounds a finished sum
-__device__ __forceinline__ float rounded(const double (&a)[1], float &mx) { const float r = (float)a[0]; mx = fabsf(r); return r; }
 __device__ __forceinline__ float2 rounded(const double (&a)[2], float &mx)
 {
     const float2 r = make_float2((float)a[0], (float)a[1]);
@@ -138,74 +123,63 @@ __device__ __forceinline__ float4 rounded(const double (&a)[4], float &mx)
 }
 
 // abs-max of a row where the tile holds rows of several tables (rare in large batches: kept out of the unrolled code).
-// Called by all lanes of a group together.
-template <int LPR>
+// Called by the warp together.
 __device__ __noinline__ void note_max(u32 *absmax, const u32 *s_uoff, int t_first, int T, u32 u, float x)
 {
-    const unsigned lane_w = threadIdx.x & 31;
-    const unsigned mask = LPR == 32 ? 0xffffffffu : (((1u << (LPR & 31)) - 1u) << (lane_w / LPR * LPR));
-    const u32 m = __reduce_max_sync(mask, __float_as_uint(x));
-    if (lane_w % LPR == 0 && m) atomicMax(absmax + last_not_above(s_uoff, t_first, T, u), m);
+    const u32 m = __reduce_max_sync(0xffffffffu, __float_as_uint(x));
+    if ((threadIdx.x & 31) == 0 && m) atomicMax(absmax + last_not_above(s_uoff, t_first, T, u), m);
 }
 
 // blockIdx.x * WARPS + warp: range of tiles and block of 128 features (COLS: D > 128, there are several).  EXACT: every lane
 // holds features.  Rows of 3 KB and more are not asked into L2 ahead: their blocks of features ask for whole rows already
 // (65 K rows of 4080 bytes 138 us, 154 with the request; of 2064 bytes 87 and 85)
-template <int LPR, int VEC, bool EXACT, bool SMALL, bool COLS>
-__global__ void __launch_bounds__(THREADS, blocks_per_sm(LPR))
+template <int VEC, bool EXACT, bool SMALL, bool COLS>
+__global__ void __launch_bounds__(THREADS, BLOCKS_PER_SM)
 seg_sum_kernel(const Args a)
 {
     dq_wait_before();
-    constexpr int C = batch_entries(LPR, VEC, SMALL);    // rows of a lane group in flight
-    constexpr int GP = 32 / LPR;                  // lane groups of the warp
-    constexpr int I = tile_entries(LPR, SMALL);
-    constexpr int W = (I + 31) / 32;              // index words per lane, words of head bits
-    constexpr int NB = I / (GP * C);              // batches per tile (one when the warp has several groups)
-    static_assert(GP == 1 ? NB % 2 == 0 : NB == 1, "");
+    constexpr int C = batch_entries(VEC, SMALL);         // rows in flight
+    constexpr int I = tile_entries(SMALL);
+    constexpr int NB = I / C;                     // batches per tile
+    static_assert(NB % 2 == 0 && I <= 32, "");
     typedef typename Vec<VEC>::type vec_t;
     extern __shared__ u32 s_uoff[];                                                      // [T+1]
     u32 *s_tb = s_uoff + (a.T + 1);                                                      // [T+1] (by table)
     u32 *s_row = s_tb + (a.T + 1);                                                       // [T+1] (by table)
     __shared__ u32 s_broken;
 
-    const int T = a.T, D = EXACT && !COLS ? LPR * VEC : a.D, dv = D / VEC;
-    const int wl = threadIdx.x & 31, lane = wl % LPR, grp = wl / LPR;
+    const int T = a.T, D = EXACT && !COLS ? 32 * VEC : a.D, dv = D / VEC;
+    const int wl = threadIdx.x & 31;
     // the blocks of features of a range are neighbouring warps: a row's pieces are asked for at about the same time
     const u32 cols = COLS ? (u32)a.columns : 1u, slot = blockIdx.x * WARPS + (threadIdx.x >> 5);
     const u32 col = COLS ? slot % cols : 0u, range = COLS ? slot / cols : slot;
-    const int cv = (int)col * LPR + lane;      // this lane's vector of the row
+    const int cv = (int)col * 32 + wl;         // this lane's vector of the row
     const bool on = EXACT || cv < dv;
     const bool first_col = col == 0u;
     const u32 tile0 = min((u32)a.num_tiles, range * (u32)a.range_tiles);
     const u32 tile1 = min((u32)a.num_tiles, tile0 + (u32)a.range_tiles);
 
-    // ---- indices of a tile, one entry per lane and word.  An entry starts a segment when its key differs from the key
+    // ---- indices of a tile, one entry per lane.  An entry starts a segment when its key differs from the key
     // before it
-    u32 kn[W], vn[W], kp[W];
+    u32 kn, vn, kp;
     auto fetch = [&](u32 tile) {
-#pragma unroll
-        for (int w = 0; w < W; ++w) {
-            const int64_t i = (int64_t)tile * I + w * 32 + wl;
-            kn[w] = vn[w] = kp[w] = 0u;
-            if (i < a.L && (I % 32 == 0 || wl < I)) {
-                kn[w] = __ldg(a.keys + i);
-                vn[w] = __ldg(a.vals + i);
-                kp[w] = i > 0 ? __ldg(a.keys + i - 1) : ~kn[w];
-            }
+        const int64_t i = (int64_t)tile * I + wl;
+        kn = vn = kp = 0u;
+        if (i < a.L && (I == 32 || wl < I)) {
+            kn = __ldg(a.keys + i);
+            vn = __ldg(a.vals + i);
+            kp = i > 0 ? __ldg(a.keys + i - 1) : ~kn;
         }
     };
-    u32 kc[W], vc[W], hw[W];                      // the present tile's keys, payloads and head bits
+    u32 kc, vc, heads;                            // the present tile's keys, payloads and head bits
     auto take = [&]() {
-#pragma unroll
-        for (int w = 0; w < W; ++w) {
-            hw[w] = __ballot_sync(0xffffffffu, kn[w] != kp[w]);       // (equal past the end)
-            kc[w] = kn[w];
-            vc[w] = vn[w];
-            if ((int64_t)vc[w] >= a.G) { dq_report(a.status, DQRM_ERR_INDEX_RANGE); vc[w] = 0u; }
-        }
+        heads = __ballot_sync(0xffffffffu, kn != kp);         // (equal past the end)
+        kc = kn;
+        vc = vn;
+        if ((int64_t)vc >= a.G) { dq_report(a.status, DQRM_ERR_INDEX_RANGE); vc = 0u; }
     };
     fetch(tile0);
-    u32 u_base = tile0 < tile1 ? a.chunk_first[(int64_t)tile0 * I >> chunk_shift(LPR, SMALL)] : 0u;
+    u32 u_base = tile0 < tile1 ? a.chunk_first[(int64_t)tile0 * I >> chunk_shift(SMALL)] : 0u;
     if (a.by_table) {
         if (threadIdx.x < 32) {                   // the tables' first segments: a running sum over their counts
             u32 run = 0;
@@ -225,8 +199,9 @@ seg_sum_kernel(const Args a)
             }
             broken = __any_sync(0xffffffffu, broken);
             if (wl == 0) { s_uoff[T] = run; s_broken = broken; }
+        } else {
+            for (int t = threadIdx.x - 32; t <= T; t += THREADS - 32) { s_tb[t] = a.tb[t]; s_row[t] = (u32)a.row_off[t]; }
         }
-        for (int t = threadIdx.x; t <= T; t += THREADS) { s_tb[t] = a.tb[t]; s_row[t] = (u32)a.row_off[t]; }
     } else {
         for (int t = threadIdx.x; t <= T; t += THREADS) s_uoff[t] = (u32)a.uniq_off[t];
         if (threadIdx.x == 0) s_broken = 0u;
@@ -244,34 +219,26 @@ seg_sum_kernel(const Args a)
     // the rows of batch b of the present tile, all at once (row 0 for entries past the end, and a vector of the row for
     // lanes past its end: nothing is done with either)
     auto request = [&](int b, vec_t (&r)[C]) {
-        const int e0 = b * (GP * C) + grp * C;
 #pragma unroll
-        for (int k = 0; k < C; ++k) {
-            const int e = e0 + k;
-            u32 row = __shfl_sync(0xffffffffu, vc[0], e & 31);
-            if (W == 2) { const u32 r1 = __shfl_sync(0xffffffffu, vc[W - 1], e & 31); if (e >= 32) row = r1; }
-            r[k] = ld_row(go + (int64_t)row * dv, pol);       // (no condition: a branch per row would expose every shuffle)
-        }
+        for (int k = 0; k < C; ++k)
+            r[k] = ld_row(go + (int64_t)__shfl_sync(0xffffffffu, vc, b * C + k) * dv, pol);       // (no condition: a branch per row would expose every shuffle)
     };
-    // asks L2 for the rows of the tile whose indices have just arrived: a row per lane and word
+    // asks L2 for the rows of the tile whose indices have just arrived: a row per lane
     auto prefetch = [&]() {
-        const int c0 = (int)col * LPR * VEC;
-        const int bytes = (EXACT ? LPR * VEC : min(D - c0, LPR * VEC)) * (int)sizeof(float);
+        const int c0 = (int)col * 32 * VEC;
+        const int bytes = (EXACT ? 32 * VEC : min(D - c0, 32 * VEC)) * (int)sizeof(float);
+        if (I < 32 && wl >= I) return;
+        const char *row = reinterpret_cast<const char *>(a.grad_out + (int64_t)((int64_t)vn < a.G ? vn : 0u) * D + c0);
 #pragma unroll
-        for (int w = 0; w < W; ++w) {
-            if (I % 32 != 0 && wl >= I) break;
-            const char *row = reinterpret_cast<const char *>(a.grad_out + (int64_t)((int64_t)vn[w] < a.G ? vn[w] : 0u) * D + c0);
-#pragma unroll
-            for (int b = 0; b < LPR * VEC * 4; b += 128)
-                if (EXACT || b < bytes) dq_prefetch_l2(row + b);
-            if (!EXACT) dq_prefetch_l2(row + bytes - 4);      // (rows that do not begin on a line's start)
-        }
+        for (int b = 0; b < 32 * VEC * 4; b += 128)
+            if (EXACT || b < bytes) dq_prefetch_l2(row + b);
+        if (!EXACT) dq_prefetch_l2(row + bytes - 4);          // (rows that do not begin on a line's start)
     };
     take();
     request(0, v[0]);
     fetch(tile0 + 1);
 
-    const bool head0 = hw[0] & 1u;
+    const bool head0 = heads & 1u;
     int t_first = a.by_table ? last_not_above(s_tb, 0, T, tile0 * I) : last_not_above(s_uoff, 0, T, u_base);
     if (a.by_table) u_base += s_uoff[t_first];
     const u32 u_lead = u_base;                    // the run that enters the range, if one does
@@ -290,7 +257,7 @@ seg_sum_kernel(const Args a)
         float x = 0.f;
         if (on) st_row(reinterpret_cast<vec_t *>(a.grad_rows + (int64_t)u * D) + cv, rounded(acc, x), keep);  // quantise+update reads it next
         if (one_table) m = fmaxf(m, x);
-        else note_max<LPR>(a.absmax, s_uoff, t_first, T, u, x);
+        else note_max(a.absmax, s_uoff, t_first, T, u, x);
     };
     auto store_piece = [&](int slot, const double (&acc)[VEC]) {
         if (on) {
@@ -299,138 +266,61 @@ seg_sum_kernel(const Args a)
             for (int q = 0; q < VEC; ++q) p[q] = acc[q];
         }
     };
-    double acc[VEC];                              // GP == 1: the open run; else: what the tiles before left of it
+    double acc[VEC];                              // the open run
 #pragma unroll
     for (int q = 0; q < VEC; ++q) acc[q] = 0.0;
 
     for (u32 tile = tile0; tile < tile1; ++tile) {
         const int n = (int)min((int64_t)I, a.L - (int64_t)tile * I);
-        u32 n_heads = __popc(hw[0]);
-        if (W == 2) n_heads += __popc(hw[W - 1]);
+        const u32 n_heads = __popc(heads);
         // the table of the run that is open when the tile begins (of the first entry's when none is)
         const bool fresh = tile == tile0 && head0;
         while (t_first < T - 1 && u_base + fresh >= s_uoff[t_first + 1]) ++t_first;
         one_table = u_base + n_heads < s_uoff[t_first + 1];
         if (one_table && t_first != t_max) { push_max(); t_max = t_first; }
-        if (a.by_table && first_col) {
-            u32 before = 0;
-#pragma unroll
-            for (int w = 0; w < W; ++w) {         // every entry that starts a segment names the segment's row
-                if (w * 32 + wl < n && ((hw[w] >> wl) & 1u)) {
-                    const u32 u = u_base + before + __popc(hw[w] & (0xffffffffu >> (31 - wl)));
-                    const int t = one_table ? t_first : last_not_above(s_uoff, t_first, T, u);
-                    a.unique_rows[u] = (int32_t)(kc[w] - s_row[t]);
-                }
-                before += __popc(hw[w]);
-            }
+        if (a.by_table && first_col && wl < n && ((heads >> wl) & 1u)) {      // every entry that starts a segment names the segment's row
+            const u32 u = u_base + __popc(heads & (0xffffffffu >> (31 - wl)));
+            const int t = one_table ? t_first : last_not_above(s_uoff, t_first, T, u);
+            a.unique_rows[u] = (int32_t)(kc - s_row[t]);
         }
         if (tile + 1 < tile1 && (!COLS || D < 768)) prefetch();
-        if constexpr (GP == 1) {
-            u32 u = u_base;
-            const u32 heads = hw[0];
+        u32 u = u_base;
+        const u32 now = heads;
 #pragma unroll
-            for (int b = 0; b < NB; ++b) {
-                if (b + 1 < NB) {
-                    request(b + 1, v[(b + 1) & 1]);
-                } else if (tile + 1 < tile1) {
-                    take();
-                    request(0, v[0]);
-                    fetch(tile + 2);
-                }
-                const u32 bits = (heads >> (b * C)) & ((1u << C) - 1u);
-                if (bits == 0u && n >= (b + 1) * C) {         // inside a run
-#pragma unroll
-                    for (int k = 0; k < C; ++k) add(acc, v[b & 1][k]);
-                } else {
-#pragma unroll
-                    for (int k = 0; k < C; ++k) {
-                        if ((bits >> k) & 1u) {               // (warp-uniform)
-                            if (open_lead) { store_piece(0, acc); open_lead = false; }
-                            else if (!(fresh && b * C + k == 0)) store_row(u, acc);
-                            ++u;
-#pragma unroll
-                            for (int q = 0; q < VEC; ++q) acc[q] = 0.0;
-                        }
-                        if (b * C + k < n) add(acc, v[b & 1][k]);
-                    }
-                }
-            }
-            u_base = u;
-        } else {
-            const u32 word = W == 2 && grp * C >= 32 ? hw[W - 1] : hw[0];
-            const int es = grp * C, sh = es & 31;
-            const u32 hb = (word >> sh) & ((1u << C) - 1u);
-            const int nv = min(max(n - es, 0), C);
-            const u32 before = __popc(word & ((1u << sh) - 1u)) + (W == 2 && es >= 32 ? __popc(hw[0]) : 0);
-            u32 u = u_base + before;              // the run that is open when the group begins
-            const u32 u_in = u;
-            bool seen = false;
-            double in[VEC], sum[VEC];             // what the group adds to that run; the present run
-#pragma unroll
-            for (int q = 0; q < VEC; ++q) in[q] = sum[q] = 0.0;
-#pragma unroll
-            for (int k = 0; k < C; ++k) {
-                if (k < nv) {
-                    if ((hb >> k) & 1u) {
-                        if (seen) store_row(u, sum);
-                        else {
-#pragma unroll
-                            for (int q = 0; q < VEC; ++q) in[q] = sum[q];
-                        }
-                        seen = true;
-                        ++u;
-#pragma unroll
-                        for (int q = 0; q < VEC; ++q) sum[q] = 0.0;
-                    }
-                    add(sum, v[0][k]);
-                }
-            }
-            __syncwarp();
-            u_base += n_heads;
-            const bool enters_lead = open_lead;
-            open_lead = open_lead && n_heads == 0u;
-            if (tile + 1 < tile1) {
+        for (int b = 0; b < NB; ++b) {
+            if (b + 1 < NB) {
+                request(b + 1, v[(b + 1) & 1]);
+            } else if (tile + 1 < tile1) {
                 take();
                 request(0, v[0]);
                 fetch(tile + 2);
             }
-            // segmented scan over the groups: sum becomes the open run behind the group, counted from the last head
-            bool any = seen;
+            const u32 bits = (now >> (b * C)) & ((1u << C) - 1u);
+            if (bits == 0u && n >= (b + 1) * C) {             // inside a run
 #pragma unroll
-            for (int o = 1; o < GP; o <<= 1) {
-                const bool any_o = __shfl_up_sync(0xffffffffu, any, o * LPR);
+                for (int k = 0; k < C; ++k) add(acc, v[b & 1][k]);
+            } else {
 #pragma unroll
-                for (int q = 0; q < VEC; ++q) {
-                    const double x = __shfl_up_sync(0xffffffffu, sum[q], o * LPR);
-                    if (grp >= o && !any) sum[q] = x + sum[q];
+                for (int k = 0; k < C; ++k) {
+                    if ((bits >> k) & 1u) {                   // (warp-uniform)
+                        if (open_lead) { store_piece(0, acc); open_lead = false; }
+                        else if (!(fresh && b * C + k == 0)) store_row(u, acc);
+                        ++u;
+#pragma unroll
+                        for (int q = 0; q < VEC; ++q) acc[q] = 0.0;
+                    }
+                    if (b * C + k < n) add(acc, v[b & 1][k]);
                 }
-                if (grp >= o) any |= any_o;
             }
-            const bool any_in = __shfl_up_sync(0xffffffffu, any, LPR) && grp > 0;
-            const bool any_all = __shfl_sync(0xffffffffu, any, 31);
-#pragma unroll
-            for (int q = 0; q < VEC; ++q) {
-                const double x = __shfl_up_sync(0xffffffffu, sum[q], LPR);
-                if (grp > 0) in[q] = (any_in ? x : acc[q] + x) + in[q];
-                else in[q] = acc[q] + in[q];
-                const double last = __shfl_sync(0xffffffffu, sum[q], (GP - 1) * LPR + lane);
-                acc[q] = any_all ? last : acc[q] + last;
-            }
-            if (seen) {
-                if (enters_lead && before == 0u) store_piece(0, in);
-                else if (!(fresh && before == 0u)) store_row(u_in, in);
-            }
-            __syncwarp();
         }
+        u_base = u;
     }
     // ---- the run that is open at the end of the range
     const int64_t i1 = min((int64_t)tile1 * I, a.L);
     const bool ends = i1 == a.L || __ldg(a.keys + i1) != __ldg(a.keys + i1 - 1);
     const bool cut_lead = !head0, cut_trail = !open_lead && !ends;
-    if (grp == 0) {
-        if (open_lead || cut_trail) store_piece(open_lead ? 0 : 1, acc);
-        else store_row(u_base, acc);
-    }
+    if (open_lead || cut_trail) store_piece(open_lead ? 0 : 1, acc);
+    else store_row(u_base, acc);
     __syncwarp();
     push_max();
 
@@ -462,11 +352,11 @@ seg_sum_kernel(const Args a)
     auto fold = [&](int np, int cc, double (&sum)[VEC], auto at) {
 #pragma unroll
         for (int x = 0; x < VEC; ++x) sum[x] = 0.0;
-        for (int p0 = grp; (EXACT || cc < dv) && p0 < np; p0 += 8 * GP) {
+        for (int p0 = 0; (EXACT || cc < dv) && p0 < np; p0 += 8) {
             double x[8][VEC];
 #pragma unroll
             for (int j = 0; j < 8; ++j) {
-                const int p = p0 + j * GP;
+                const int p = p0 + j;
                 const double *src = at(min(p, np - 1)) + cc * VEC;
 #pragma unroll
                 for (int q = 0; q < VEC; ++q) x[j][q] = p < np ? __ldcg(src + q) : 0.0;
@@ -476,18 +366,11 @@ seg_sum_kernel(const Args a)
 #pragma unroll
                 for (int q = 0; q < VEC; ++q) sum[q] += x[j][q];
         }
-#pragma unroll
-        for (int o = LPR; o < 32; o <<= 1)
-#pragma unroll
-            for (int x = 0; x < VEC; ++x) sum[x] += __shfl_xor_sync(0xffffffffu, sum[x], o);
     };
     auto store_total = [&](u32 u, int cc, const double (&sum)[VEC]) {
-        if (grp == 0) {
-            float x = 0.f;
-            if (EXACT || cc < dv) st_row(reinterpret_cast<vec_t *>(a.grad_rows + (int64_t)u * D) + cc, rounded(sum, x), keep);
-            note_max<LPR>(a.absmax, s_uoff, 0, T, u, x);
-        }
-        __syncwarp();
+        float x = 0.f;
+        if (EXACT || cc < dv) st_row(reinterpret_cast<vec_t *>(a.grad_rows + (int64_t)u * D) + cc, rounded(sum, x), keep);
+        note_max(a.absmax, s_uoff, 0, T, u, x);
     };
 #pragma unroll 1
     for (int q = 0; q < 2; ++q) {                 // (columns: all of them, the blocks of the others are done too)
@@ -496,12 +379,12 @@ seg_sum_kernel(const Args a)
         const u32 u = q ? u_base : u_lead, f = __shfl_sync(0xffffffffu, first_range, q);
         const u32 ng = __shfl_sync(0xffffffffu, groups, q), g0 = f / FOLD_GROUP;
         const u32 p_first = ng ? max(f, group * FOLD_GROUP) : f;
-        for (int cc = lane; cc - lane < (COLS ? dv : 1); cc += LPR) {
+        for (int cc = wl; cc - wl < (COLS ? dv : 1); cc += 32) {
             double sum[VEC];
             fold(np, cc, sum, [&](int p) { return a.partials + ((size_t)(p_first + p) * 2 + (p_first + p == f ? 1 : 0)) * D; });
             if (ng == 0) {
                 store_total(u, cc, sum);
-            } else if (grp == 0 && (EXACT || cc < dv)) {
+            } else if (EXACT || cc < dv) {
 #pragma unroll
                 for (int x = 0; x < VEC; ++x) a.group_partials[((size_t)group * 2 + (group == g0 ? 1 : 0)) * D + cc * VEC + x] = sum[x];
             }
@@ -515,7 +398,7 @@ seg_sum_kernel(const Args a)
                 __threadfence();
             }
             if (!__shfl_sync(0xffffffffu, final, 0)) continue;
-            for (int cc = lane; cc - lane < (COLS ? dv : 1); cc += LPR) {
+            for (int cc = wl; cc - wl < (COLS ? dv : 1); cc += 32) {
                 double sum[VEC];
                 fold((int)ng, cc, sum, [&](int p) { return a.group_partials + ((size_t)(g0 + p) * 2 + (p == 0 ? 1 : 0)) * D; });
                 store_total(u, cc, sum);

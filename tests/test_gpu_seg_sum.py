@@ -88,3 +88,29 @@ def test_runs_of_the_cluster_sort(oracle, split, D):
     n = max(max(r) for r in runs)
     np.testing.assert_allclose(gr, o_gr, rtol=2.0 ** -23, atol=12.0 * n * n * 2.0 ** -53)
     c.ctx.close()
+
+
+@pytest.mark.parametrize("D", [4, 8, 16, 20, 32])
+@pytest.mark.parametrize("n", [1, 7, 8, 9, 255, 257, 4_099])
+def test_runs_of_lane_groups(oracle, n, D):
+    """Rows that take a lane group, where the groups' ranges, the tables and the runs all end at different entries: tables
+    of one lookup beside larger ones, runs of one to nine entries, signed zeros among the gradients."""
+    rng = np.random.default_rng(n + D)
+    counts = [n, 1, 0, max(1, n // 3), 5]
+    B = max(counts)
+    runs = [np.repeat(np.arange(c), rng.integers(1, 10, c))[:c] for c in counts]
+    wl = W.Workload("groups", tuple(max(4, c) for c in counts), D=D, B=B, alpha=None)
+    idx = np.concatenate([rng.permutation(r) for r in runs]).astype(np.int32)
+    lens = np.zeros((wl.T, B), dtype=np.int64)
+    for t, c in enumerate(counts):
+        lens[t, :c] = 1
+    off = np.concatenate([[0], np.cumsum(lens.reshape(-1))]).astype(np.int32)
+    go = rng.standard_normal((B, wl.T, D)).astype(np.float32)
+    go[rng.random(go.shape) < 0.1] = -0.0
+    c = Case(wl, max_lookups=len(idx))
+    ur, uo, gr = c.gpu_bwd(idx, off, go)
+    o_ur, o_uo, o_gr = oracle.emb_bwd(go, wl.T, D, B, idx, off)
+    assert bit_equal(uo, o_uo) and bit_equal(ur, o_ur)
+    # nine terms of magnitude below 6 in FP64 in two orders, each sum rounded once
+    np.testing.assert_allclose(gr, o_gr, rtol=2.0 ** -23, atol=12.0 * 9 * 9 * 2.0 ** -53)
+    c.ctx.close()
