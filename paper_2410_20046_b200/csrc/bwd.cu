@@ -50,6 +50,7 @@ Layout make_layout(const dqrm_ctx *ctx, int64_t L)
     Layout y;
     y.passes = (ctx->row_bits + rsort::MAX_DIGIT_BITS - 1) / rsort::MAX_DIGIT_BITS;
     y.digit_bits = (ctx->row_bits + y.passes - 1) / y.passes;
+    if (y.digit_bits < 2) y.digit_bits = 2;        // (the scatter takes four digits a thread)
     int64_t Lc = L < 1 ? 1 : L;
     y.num_tiles = (Lc + ST_TILE - 1) / ST_TILE;
     y.radix_tiles = rsort::max_tiles(ctx->T, Lc);

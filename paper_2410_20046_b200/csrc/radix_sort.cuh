@@ -1,8 +1,9 @@
 // Stable radix sort of a batch's lookups by (table, row) for batches whose tables are too large for the cluster sort
 // (or on request): the lookups arrive table-major, so every table is sorted by itself, by the row number within the
 // table, and all tables move through the same launches.  Digits are at most ten bits wide and as few as the largest
-// table needs: a million rows take two passes.  Measured on B200, 8.5 M lookups of 26 tables of a million rows: 240 us,
-// and 290 with the kernels that number the segments behind it; one sort over the arena rows of all tables, with a
+// table needs: a million rows take two passes.  Measured on B200, 8.5 M lookups of 26 tables of a million rows: 160 us,
+// and 204 with the kernels that number the segments behind it (232 before the first pass ranked by masks); one sort over the
+// arena rows of all tables, with a
 // kernel of its own that expanded the bags and three passes of nine bits, took 435 and 490.
 //
 //   rs_setup     one block: where each table begins, which table each tile of TILE lookups belongs to
@@ -228,7 +229,6 @@ rs_scatter_kernel(const Args a, const uint2 *__restrict__ pairs_in, uint2 *__res
     const int w0 = warp * (TILE / WARPS) + lane;       // a warp holds 512 consecutive entries, 32 at a time
     const int64_t r0 = __ldg(a.row_off + x.t);
     u32 key[ITEMS], val[ITEMS], rank[ITEMS / 2];       // ranks: two 16-bit halves per word
-
     for (int i = threadIdx.x; i < WARPS * nb / 2; i += THREADS) reinterpret_cast<u32 *>(s_cnt)[i] = 0u;
     if (FIRST) {
         const int32_t nrows = (int32_t)(__ldg(a.row_off + x.t + 1) - r0);
@@ -296,13 +296,22 @@ rs_scatter_kernel(const Args a, const uint2 *__restrict__ pairs_in, uint2 *__res
         }
     }
     __syncthreads();
-    // ---- rank within (warp, digit), counting on the way
+    // ---- rank within (warp, digit), counting on the way.  The first pass finds the lanes with the same digit by an OR into shared
+    // memory, where the pairs will stand (by match.any, which takes the longer the more digits differ, 16 K of a tile's 38 K clocks);
+    // in the later ones equal rows already stand together, and a match of few digits is the faster.  With what the digits' places
+    // below save: two passes over 8.5 M lookups 160 -> 131 us
+    u32 *my_mask = reinterpret_cast<u32 *>(s_pair) + warp * nb;
+    static_assert(sizeof(uint2) * TILE >= (sizeof(u32) * WARPS << MAX_DIGIT_BITS), "");
+    if (FIRST) {
+        for (int i = lane; i < nb; i += 32) my_mask[i] = 0u;
+        __syncwarp();
+    }
     unsigned short *my_cnt = s_cnt + warp * nb;
 #pragma unroll
     for (int k = 0; k < ITEMS; ++k) {
         const bool valid = w0 + k * 32 < x.len;
         const u32 d = (key[k] >> shift) & mask;
-        const u32 peers = __match_any_sync(0xffffffffu, valid ? d : (u32)nb);     // (ten votes instead take as long)
+        const u32 peers = FIRST ? dq_same_digit_lanes(my_mask, d, valid) : __match_any_sync(0xffffffffu, valid ? d : (u32)nb);
         u32 r = 0;
         if (valid) r = my_cnt[d] + __popc(peers & lt);
         __syncwarp();
@@ -310,38 +319,39 @@ rs_scatter_kernel(const Args a, const uint2 *__restrict__ pairs_in, uint2 *__res
         __syncwarp();
         if (k & 1) rank[k / 2] |= r << 16; else rank[k / 2] = r;
     }
+    // the digits of this thread (four consecutive ones): how many entries the table has, and the tiles before this one
+    const int d0 = (int)threadIdx.x * 4;
+    uint4 all = make_uint4(0u, 0u, 0u, 0u), earlier = all;
+    if (d0 < nb) {
+        all = __ldg(reinterpret_cast<const uint4 *>(a.totals + (size_t)x.t * nb + d0));
+        earlier = __ldg(reinterpret_cast<const uint4 *>(a.tilehist + (size_t)blockIdx.x * nb + d0));
+    }
     __syncthreads();
-    // ---- per digit: the warps' counts become places in the tile's order, and what leads from there to the output
+    // ---- per digit: the warps' counts become places in the tile's order, and what leads from there to the output.  Two
+    // digits a word: a tile's counts fit 16 bits
     {
-        const int per = max(1, nb / THREADS), d0 = (int)threadIdx.x * per;               // 1, 2 or 4 digits per thread
-        u32 tot[4], all[4], tsum = 0, asum = 0;
+        uint2 before[WARPS], tot = make_uint2(0u, 0u);
+        uint2 *c4 = reinterpret_cast<uint2 *>(s_cnt) + threadIdx.x;
+        if (d0 < nb) {
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            tot[j] = all[j] = 0u;
-            if (j < per && d0 + j < nb) {
+            for (int w = 0; w < WARPS; ++w) before[w] = c4[w * (nb / 4)];
 #pragma unroll
-                for (int w = 0; w < WARPS; ++w) tot[j] += s_cnt[w * nb + d0 + j];
-                all[j] = __ldg(a.totals + (size_t)x.t * nb + d0 + j);
+            for (int w = 0; w < WARPS; ++w) {
+                const uint2 c = before[w];
+                before[w] = tot;
+                tot.x += c.x;
+                tot.y += c.y;
             }
-            tsum += tot[j];
-            asum += all[j];
         }
-        u32 place = block_exclusive(tsum, s_warp);
-        u32 base = block_exclusive(asum, s_warp) + __ldg(a.tb + x.t);
+        const u32 n0 = tot.x & 0xffffu, n1 = tot.x >> 16, n2 = tot.y & 0xffffu, n3 = tot.y >> 16;
+        const u32 place = block_exclusive(n0 + n1 + n2 + n3, s_warp);
+        const u32 base = block_exclusive(all.x + all.y + all.z + all.w, s_warp) + __ldg(a.tb + x.t);
+        if (d0 < nb) {
+            const u32 p1 = place + n0, p2 = p1 + n1, p3 = p2 + n2, b1 = base + all.x, b2 = b1 + all.y, b3 = b2 + all.z;
+            *reinterpret_cast<uint4 *>(s_delta + d0) = make_uint4(base + earlier.x - place, b1 + earlier.y - p1, b2 + earlier.z - p2, b3 + earlier.w - p3);
+            const uint2 p = make_uint2(place | p1 << 16, p2 | p3 << 16);
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            if (j < per && d0 + j < nb) {
-                s_delta[d0 + j] = base + __ldg(a.tilehist + (size_t)blockIdx.x * nb + d0 + j) - place;
-                u32 run = place;
-#pragma unroll
-                for (int w = 0; w < WARPS; ++w) {
-                    const u32 c = s_cnt[w * nb + d0 + j];
-                    s_cnt[w * nb + d0 + j] = (unsigned short)run;
-                    run += c;
-                }
-            }
-            place += tot[j];
-            base += all[j];
+            for (int w = 0; w < WARPS; ++w) c4[w * (nb / 4)] = make_uint2(p.x + before[w].x, p.y + before[w].y);
         }
     }
     __syncthreads();

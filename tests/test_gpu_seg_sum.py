@@ -114,3 +114,27 @@ def test_runs_of_lane_groups(oracle, n, D):
     # nine terms of magnitude below 6 in FP64 in two orders, each sum rounded once
     np.testing.assert_allclose(gr, o_gr, rtol=2.0 ** -23, atol=12.0 * 9 * 9 * 2.0 ** -53)
     c.ctx.close()
+
+
+@pytest.mark.parametrize("rows", [1, 2, 3, 5, 1 << 10, (1 << 10) + 1, 1 << 20, (1 << 20) + 1])      # one to three digits of one bit and up
+def test_radix_sort_digits(oracle, rows):
+    """The radix sort's ranks and places at the edges of its digits and of its tiles of 4096: bags of zero to five, a
+    row that a third of the lookups hit, rows at both ends of the table."""
+    rng = np.random.default_rng(rows)
+    T, B, D = 3, 4_100, 4
+    wl = W.Workload("digits", (rows, rows, max(1, rows // 2)), D=D, B=B, alpha=None)
+    lens = rng.integers(0, 6, T * B)
+    off = np.concatenate([[0], np.cumsum(lens)]).astype(np.int32)
+    table = np.repeat(np.arange(T), lens.reshape(T, B).sum(1))
+    idx = (rng.random(off[-1]) * np.array(wl.rows)[table]).astype(np.int32)
+    idx[rng.random(len(idx)) < 0.33] = wl.rows[2] // 3
+    idx[0], idx[-1] = rows - 1, wl.rows[2] - 1
+    go = rng.standard_normal((B, T, D)).astype(np.float32)
+    c = Case(wl, max_lookups=len(idx))
+    c.ctx.set_sort_path(1)
+    ur, uo, gr = c.gpu_bwd(idx, off, go)
+    o_ur, o_uo, o_gr = oracle.emb_bwd(go, T, D, B, idx, off)
+    assert bit_equal(uo, o_uo) and bit_equal(ur, o_ur)
+    # at most 25,000 terms of magnitude below 6 in FP64 in two orders, each sum rounded once
+    np.testing.assert_allclose(gr, o_gr, rtol=2.0 ** -23, atol=12.0 * 25_000 ** 2 * 2.0 ** -53)
+    c.ctx.close()
