@@ -34,7 +34,7 @@ constexpr int ST_WARPS = ST_THREADS / 32;
 struct Layout {
     int passes, digit_bits;                    // radix sort: digits of the row number within a table
     int64_t radix_tiles, num_tiles;
-    // the summing kernel: log2 of the entries between two of chunk_first; rows of more than 32 features: small tiles, tiles, tiles of
+    // the summing kernel: log2 of the entries between two of chunk_first; rows of more than 48 features: small tiles, tiles, tiles of
     // a warp's range; narrower ones: entries of a lane group's range, ranges of warps
     int sum_shift;
     bool sum_small;
@@ -543,7 +543,8 @@ int dq_launch_bwd_sum(dqrm_ctx *ctx, const float *grad_out, int32_t *unique_rows
     case 1: return launch_sum_groups<1>(ctx, a, st);
     case 2: return launch_sum_groups<2>(ctx, a, st);
     case 4: return launch_sum_groups<4>(ctx, a, st);
-    default: return launch_sum_groups<8>(ctx, a, st);
+    case 8: return launch_sum_groups<8>(ctx, a, st);
+    default: return launch_sum_groups<16>(ctx, a, st);
     }
 }
 

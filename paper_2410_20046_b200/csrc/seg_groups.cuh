@@ -1,4 +1,4 @@
-// Segmented sum of the upstream gradient over the sorted lookups for rows of up to 32 features (wider ones: seg_reduce.cuh, whose
+// Segmented sum of the upstream gradient over the sorted lookups for rows of up to 48 features (wider ones: seg_reduce.cuh, whose
 // inputs, arguments and results these are).
 //
 // A row takes LPR lanes with four features each; a warp has 32 / LPR such lane groups, and every group walks a contiguous
@@ -17,9 +17,11 @@
 // (graph replay, us) against seg_reduce.cuh's way with several groups a warp, which scanned over the groups for every tile of
 // 64 entries and looked up the table of every row where a tile held several: 13 K rows of 64 bytes in 26 tables 17.5 -> 8.3, 52 K
 // 16.6 -> 9.0, 426 K 18.9 -> 16.3, 5.4 M in bags of 18 99.9 -> 81.9; 426 K rows of 32 bytes 15.7 -> 13.6, of 80 27.4 -> 24, of 128
-// 25.0 -> 24.0.  Rows of 36 features and more are better off with a warp each, whose branches are uniform: this way 53 K
-// of 256 bytes took 17.9 instead of 11.5, 8.5 M 380 instead of 318.  Integer conversions into a scaled range instead of those
-// by the conversion unit: 16.7 -> 18.2.
+// 25.0 -> 24.0; with two groups a warp, 64 K rows of 144 bytes 15.0 -> 13.8, 20 K of 192 13.1 -> 10.5, 426 K of 192 40.6 -> 37.2.
+// Rows of 52 features and more are better off with a warp each, whose branches are uniform: this way 100 K of 240 bytes took 18.8
+// instead of 17.1 us, 53 K of 256 14.7 instead of 11.5, 8.5 M in bags of 20 387 instead of 319, 82 K of 384 25.9 instead of 19.0
+// (but 852 K of 256 56.6 instead of 60.3, 13 K of 512 10.8 instead of 12.7; none of it shows beside a forward and a sort).  Integer
+// conversions into a scaled range instead of those by the conversion unit: 16.7 -> 18.2.
 #pragma once
 #include <type_traits>
 #include "seg_reduce.cuh"
@@ -32,10 +34,11 @@ constexpr int AHEAD = 4;                     // batches between a row's request 
 // their rows (5.4 M rows of 64 bytes 90.2, 81.9)
 constexpr int GROUPS_THREADS = 128, GROUPS_BLOCKS = 5;
 constexpr int CHUNK_SHIFT = 3;               // a group's range begins at a multiple of eight entries
+static_assert((1 << CHUNK_SHIFT) % (2 * BATCH) == 0, "the walk takes two batches a round and has no rest of one");
 
 // the rows that come here, and lanes for one of them
-__host__ __device__ constexpr bool takes_groups(int D) { return D <= 32; }
-__host__ __device__ constexpr int lanes_per_row(int D) { return D <= 4 ? 1 : D <= 8 ? 2 : D <= 16 ? 4 : 8; }
+__host__ __device__ constexpr bool takes_groups(int D) { return D <= 48; }
+__host__ __device__ constexpr int lanes_per_row(int D) { return D <= 4 ? 1 : D <= 8 ? 2 : D <= 16 ? 4 : D <= 32 ? 8 : 16; }
 
 // One range a warp; blocks of two warps at least.  EXACT: every lane holds features
 template <int LPR, bool EXACT>

@@ -10,7 +10,7 @@
 // entries at a time.  The sum is bound by the latency of the chain index -> payload -> row: indices are fetched a
 // tile ahead, the rows of the next tile are asked into L2 as soon as its payloads are there (without that the kernel
 // took 89 instead of 71 us on 852 K rows of 256 bytes, 541 instead of 318 us on 8.5 M), and the next batch of rows is
-// requested before the present one is summed.  A row takes the whole warp, VEC features a lane (rows of up to 32 features go
+// requested before the present one is summed.  A row takes the whole warp, VEC features a lane (rows of up to 48 features go
 // to seg_groups.cuh): every branch on a run's end is then uniform and a run that goes on is simply carried in
 // registers.  Only a run cut by the edge of a warp's range leaves a partial
 // in global memory; the warp that brings a run's last partial adds all of them, in order (nobody waits; the pieces of a

@@ -90,7 +90,7 @@ def test_runs_of_the_cluster_sort(oracle, split, D):
     c.ctx.close()
 
 
-@pytest.mark.parametrize("D", [4, 8, 16, 20, 32])
+@pytest.mark.parametrize("D", [4, 8, 16, 20, 32, 36, 48])
 @pytest.mark.parametrize("n", [1, 7, 8, 9, 255, 257, 4_099])
 def test_runs_of_lane_groups(oracle, n, D):
     """Rows that take a lane group, where the groups' ranges, the tables and the runs all end at different entries: tables
