@@ -357,15 +357,15 @@ int dqrm_decode_payload(dqrm_ctx *ctx, const uint8_t *payload, const float *scal
 int dqrm_set_sort_path(dqrm_ctx *ctx, int path);
 
 /* dqrm_train_step and dqrm_train_step_sorted run the backward up to the summed gradient (index
- * sort, gradient summation: neither needs the tables or the forward's output) on a second
- * stream owned by the context (created by dqrm_create), beside the forward on the caller's
- * stream, and join the two before the touched rows are updated; the caller's stream sees one
- * ordered step.  dqrm_train_step does so from 16 MB of gathered rows on, and for batches
- * of up to 16384 lookups that are not one a bag; other small batches, for which fork and join
- * cost more than the overlap gives, stay on the caller's stream, and the smallest of all take
- * one launch behind the forward.  dqrm_train_step_sorted also moves its forward to
- * a third, lowest-priority stream of the context (forked from and joined to the caller's
- * stream), so that the forward's many blocks do not keep a sort of the next batch, running
+ * sort, gradient summation: neither needs the tables or the forward's output) beside the
+ * forward and join the two before the touched rows are updated; the caller's stream sees one
+ * ordered step.  dqrm_train_step does so from 1 MB of gathered rows on, and for batches
+ * of up to 16384 lookups that are not one a bag; the smallest of all take
+ * one launch behind the forward.  Its forward runs on a lowest-priority stream of the context and its
+ * backward, from 64 MB on, on a highest-priority one (both created by dqrm_create, forked from
+ * and joined to the caller's); from 1 GB on the forward stays on the caller's stream.
+ * dqrm_train_step_sorted has its summation on the highest-priority stream and
+ * its forward on the lowest-priority one, so that the forward's many blocks do not keep a sort of the next batch, running
  * elsewhere, off the SMs.
  * on = 0 keeps every launch on the caller's stream.  Default: 1. */
 int dqrm_set_overlap(dqrm_ctx *ctx, int on);

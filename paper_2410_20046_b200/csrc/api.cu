@@ -60,16 +60,26 @@ int64_t host_lookups_for(const dqrm_ctx *ctx, size_t workspace_bytes, int64_t L,
     return lo;
 }
 
-// Whether dqrm_train_step runs the backward beside the forward.  From 16 MB of gathered rows on it does; below, fork and join
-// and the forward's blocks in the sort's way cost about what the overlap gives (measured on B200, graph replay, two streams /
-// one: 26 tables of 4096 lookups of 64 bytes 34.2 / 34.6 us, 6 of 16 K 45.3 / 39.7, 4 of 8192 of 256 bytes 39.6 / 36.4; few
-// tables are 2 to 4 us faster in two, 24.4 / 28.8 for three of 4096 of 256 bytes, but launched one by one the same or slower).
+// Whether dqrm_train_step runs the backward beside the forward.  From 1 MB of gathered rows on it does: the sort leaves most of
+// the chip idle, and with the forward on the other stream the fork is not in the backward's way (measured on B200, us a step, two
+// streams / one, graph replay and launched one by one: 26 tables of 2048 lookups of 256 bytes 26.0 / 31.6, 28.5 / 30.7; of 2000 of 64
+// bytes 22.6 / 26.0, 25.6 / 25.9; 40 tables of 500 of 192 bytes 20.5 / 26.6, 22.9 / 25.7; 26 of 500 of 144 bytes 18.5 / 24.7,
+// 21.3 / 23.9; below, 26 of 500 of 64 bytes, 22.2 / 22.1, 22.2 / 21.4).
 // Batches of up to 16 K lookups that are not an index a bag fork too: a few long bags are a long chain for their lane groups
 // while the rest of the chip waits (26 tables of 64 bags, one table with 100 indices a bag, 64-byte rows: 30.8 / 53.8 us; even
 // bags of three, three tables of 600: 30.8 / 32.7 with 64-byte rows, 26.5 / 25.6 with 256-byte rows).
+//
+// Which half moves.  A forward of a few blocks an SM that starts first keeps the sort's clusters, which want eight or sixteen
+// SMs of a GPC with half or all of their registers free, waiting until it is over: so the backward stays on the caller's stream,
+// where it begins at once, and the forward goes to the context's lowest-priority one (65 K rows of 512 bytes 82.0 -> 64.3 us,
+// 426 K of 64 57.6 -> 50.8).  From BWD_ASIDE bytes on the forward outlasts the sort and would then take half of the memory
+// from the sum: the backward goes to the highest-priority stream (240 K rows of 384 bytes 110.2, 111.9 on the caller's; 852 K of
+// 256 153.0 and 160.8; but 65 K of 512 66.5).  From FWD_STAYS on the forward is the longer half and begins at once itself (8.5 M
+// rows of 256 bytes 936 us, 944 on the other stream; 5.4 M of 64 303 both ways).
+constexpr int64_t STEP_FORKS = (int64_t)1 << 20, BWD_ASIDE = (int64_t)64 << 20, FWD_STAYS = (int64_t)1 << 30;
 bool step_forks(const dqrm_ctx *ctx, int B, int64_t L)
 {
-    if (L * ctx->D * (int64_t)sizeof(float) >= ((int64_t)16 << 20)) return true;
+    if (L * ctx->D * (int64_t)sizeof(float) >= STEP_FORKS) return true;
     return L > 0 && L != (int64_t)ctx->T * B && L <= 16384;
 }
 
@@ -346,19 +356,26 @@ int dqrm_train_step(dqrm_ctx *ctx, float *tables, const int32_t *indices, const 
                                     grad_scales, lr, B, L, workspace, workspace_bytes, st);
     }
     // The backward up to the summed gradient needs the indices and the upstream gradient but neither the
-    // tables nor the forward's output, so it runs on the context's second stream while the forward runs on
+    // tables nor the forward's output, so the two run side by side, each on a stream of the context or on
     // the caller's (per-launch profiling keeps one stream, because its events time consecutive launches).
     // The quantise-and-update kernel writes the rows the forward reads, so it waits for both.
     const bool overlap = ctx->overlap && !ctx->prof_on && step_forks(ctx, B, L);
-    cudaStream_t ss = overlap ? ctx->side : st;
+    const int64_t gathered = L * ctx->D * (int64_t)sizeof(float);
+    const cudaStream_t bs = overlap && gathered >= BWD_ASIDE ? ctx->side : st, fs = overlap && gathered < FWD_STAYS ? ctx->low : st;
     if (overlap) {
         DQRM_CUDA_TRY(ctx, cudaEventRecord(ctx->ev_fork, st));
-        DQRM_CUDA_TRY(ctx, cudaStreamWaitEvent(ctx->side, ctx->ev_fork, 0));
+        if (bs != st) DQRM_CUDA_TRY(ctx, cudaStreamWaitEvent(bs, ctx->ev_fork, 0));
+        if (fs != st) DQRM_CUDA_TRY(ctx, cudaStreamWaitEvent(fs, ctx->ev_fork, 0));
     }
-    int rc = dq_launch_bwd(ctx, grad_out, indices, offsets, unique_rows, uniq_off, grad_rows, B, L, workspace, workspace_bytes, ss);
-    int rc2 = dq_launch_fwd(ctx, tables, indices, offsets, scales, bits, out, nullptr, B, L, st);
-    if (overlap) {   // join even after an error so that the caller's stream stays ordered behind the side stream
-        cudaEventRecord(ctx->ev_join, ctx->side);
+    int rc = dq_launch_bwd(ctx, grad_out, indices, offsets, unique_rows, uniq_off, grad_rows, B, L, workspace, workspace_bytes, bs);
+    int rc2 = dq_launch_fwd(ctx, tables, indices, offsets, scales, bits, out, nullptr, B, L, fs);
+    // join even after an error so that the caller's stream stays ordered behind the others
+    if (fs != st) {
+        cudaEventRecord(ctx->ev_low_join, fs);
+        cudaStreamWaitEvent(st, ctx->ev_low_join, 0);
+    }
+    if (bs != st) {
+        cudaEventRecord(ctx->ev_join, bs);
         cudaStreamWaitEvent(st, ctx->ev_join, 0);
     }
     if (rc != DQRM_OK) return rc;
