@@ -220,19 +220,28 @@ packed_fwd_onehot_kernel(const PfArgs a)
     const int t = blockIdx.x;
     const int wlane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int lane = wlane % LPR, grp = wlane / LPR;
+    const int64_t g0 = (int64_t)t * a.B;
+    // (as in the forward: on their way before the table's constants are waited for)
+    int32_t lo = 0, hi = 0, idx = 0;
+    auto load = [&](int i) {
+        if (i < a.B) {
+            lo = __ldg(a.offsets + g0 + i);
+            hi = __ldg(a.offsets + g0 + i + 1);
+            idx = __ldg(a.indices + g0 + i);            // right when the offsets are the identity (L == T*B)
+        }
+    };
+    const int stride = gridDim.y * (WPB * 32);
+    int i0 = (blockIdx.y * WPB + warp) * 32;
+    load(i0 + wlane);
     const float s = __ldg(a.scales + t);
     const int64_t r0 = __ldg(a.row_off + t);
     const int32_t nrows = (int32_t)(__ldg(a.row_off + t + 1) - r0);
-    const int64_t g0 = (int64_t)t * a.B;
     const int TD4 = a.T * (a.D >> 2);            // 128-bit vectors between the output rows of bags i and i+1
     bool bad = false;
-    for (int i0 = (blockIdx.y * WPB + warp) * 32; i0 < a.B; i0 += gridDim.y * (WPB * 32)) {
+    for (; i0 < a.B; i0 += stride, load(i0 + wlane)) {
         const int i = i0 + wlane;
-        int32_t idx = 0;
         bool single = false;
         if (i < a.B) {
-            const int32_t lo = __ldg(a.offsets + g0 + i), hi = __ldg(a.offsets + g0 + i + 1);
-            idx = __ldg(a.indices + g0 + i);            // right when the offsets are the identity (L == T*B)
             single = (hi - lo == 1) & (lo >= 0) & ((int64_t)hi <= a.L);
             if (single) {
                 if ((int64_t)lo != g0 + i) idx = __ldg(a.indices + lo);
