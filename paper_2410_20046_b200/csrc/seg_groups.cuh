@@ -294,9 +294,7 @@ seg_groups_kernel(const __grid_constant__ Args a)
             pieces = min(last_range, group * FOLD_GROUP + FOLD_GROUP - 1) - max(first_range, group * FOLD_GROUP) + 1;
             arrived = &a.range_done[2 * group + (group == g0 ? 1 : 0)].y;
         }
-        __threadfence();
-        last = atomicAdd(arrived, 1u) == pieces - 1u ? pieces : 0u;
-        __threadfence();
+        last = arrive(arrived) == pieces - 1u ? pieces : 0u;
     }
     __syncwarp();
     // adds np partials of D features each (`at(p)` = where piece p lies), this lane's features
@@ -340,11 +338,7 @@ seg_groups_kernel(const __grid_constant__ Args a)
             }
             __syncwarp();
             bool final = false;
-            if (wl == 0) {
-                __threadfence();
-                final = atomicAdd(&a.range_done[f].x, 1u) == ng - 1u;
-                __threadfence();
-            }
+            if (wl == 0) final = arrive(&a.range_done[f].x) == ng - 1u;
             if (!__shfl_sync(0xffffffffu, final, 0)) continue;
             fold((int)ng, sum, [&](int p) { return a.group_partials + ((size_t)(g0 + p) * 2 + (p == 0 ? 1 : 0)) * D; });
         }
