@@ -16,7 +16,8 @@
 // reproducible.
 //
 // Bound by its chain of latencies (two loads, the network, a gather, a row).  Measured on B200 (graph replay): a step of 4
-// tables of 128 lookups of 16 features 9.3 us (15.7 in four launches), 26 tables of 128 13.9 (16.1).
+// tables of 128 lookups of 16 features 9.3 us (15.7 in four launches), 26 tables of 128 12.0 (13.9 before the counted lookups
+// were all asked for at once; 16.1 in four).
 #pragma once
 #include "small_sort.cuh"
 
@@ -44,7 +45,7 @@ struct Args {
 // network | hash table, digit counts or shares' sums, whichever is in use | tables' boundaries
 constexpr size_t MID_WORDS = (size_t)1 << HASH_BITS;
 static_assert(MID_WORDS >= (size_t)WARPS * csort::BINS && MID_WORDS >= (size_t)THREADS * 8, "");
-inline size_t smem_bytes(int T) { return (size_t)THREADS * 2 * sizeof(u64) + (MID_WORDS + T + 1) * sizeof(u32); }
+inline size_t smem_bytes(int T) { return (size_t)THREADS * 2 * sizeof(u64) + (MID_WORDS + 3 * T + 1) * sizeof(u32); }
 
 __global__ void __launch_bounds__(THREADS)
 small_step_kernel(const __grid_constant__ Args x)
@@ -52,13 +53,20 @@ small_step_kernel(const __grid_constant__ Args x)
     extern __shared__ u64 s_net[];                 // [2][THREADS]
     u32 *s_mid = reinterpret_cast<u32 *>(s_net + 2 * THREADS);
     u32 *s_tb = s_mid + MID_WORDS;                 // [T+1]
+    u32 *s_first = s_tb + x.s.T + 1, *s_rows = s_first + x.s.T;        // [T] arena row where a table begins, and its rows
     __shared__ u32 s_head[WORDS], s_pre[WORDS + 1], s_base, s_max;
     const csort::Args &a = x.s;
     const int t = blockIdx.x, T = a.T, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
 
     // ---- the tables' boundaries
-    for (int i = tid; i <= T; i += THREADS) s_tb[i] = (u32)__ldg(a.offsets + (int64_t)i * a.B);
-    for (int i = tid; i < (1 << HASH_BITS); i += THREADS) s_mid[i] = 0xffffffffu;
+    static_assert(THREADS > 148, "a thread has one table's boundary");
+    u32 bound = 0, first = 0, rows = 0;
+    if (tid <= T) bound = (u32)__ldg(a.offsets + (int64_t)tid * a.B);
+    if (tid < T) { first = (u32)__ldg(a.row_off + tid); rows = (u32)__ldg(a.row_off + tid + 1) - first; }
+    for (int i = tid; i < (1 << HASH_BITS) / 4; i += THREADS)
+        reinterpret_cast<uint4 *>(s_mid)[i] = make_uint4(0xffffffffu, 0xffffffffu, 0xffffffffu, 0xffffffffu);
+    if (tid <= T) s_tb[tid] = bound;
+    if (tid < T) { s_first[tid] = first; s_rows[tid] = rows; }
     if (tid == 0) s_base = s_max = 0u;
     __syncthreads();
     bool broken = false;
@@ -75,21 +83,29 @@ small_step_kernel(const __grid_constant__ Args x)
         return;
     }
     const int tb0 = (int)s_tb[t], n = (int)s_tb[t + 1] - tb0;
-    const int64_t r0 = __ldg(a.row_off + t), nrows = __ldg(a.row_off + t + 1) - r0;
+    const int64_t r0 = s_first[t], nrows = s_rows[t];
     bool bad = false;
 
     // ---- distinct rows of the tables before this one
     {
         u32 fresh = 0;
-        for (int p = tid; p < tb0; p += THREADS) {
-            const int64_t idx = __ldg(a.indices + p);
+        constexpr int EACH = MAX_LOOKUPS / THREADS;
+        int32_t idx[EACH];                         // (all of a thread's at once: in turn they were 8.4 K clocks for 3.2 K lookups)
+#pragma unroll
+        for (int k = 0; k < EACH; ++k) idx[k] = k * THREADS + tid < tb0 ? __ldg(a.indices + k * THREADS + tid) : 0;
+#pragma unroll 1
+        for (int k = 0; k * THREADS < tb0; ++k) {
+            const int p = k * THREADS + tid;
+            if (p >= tb0) break;
+            int32_t row = idx[0];
+#pragma unroll
+            for (int j = 1; j < EACH; ++j) if (k == j) row = idx[j];
             int lo = 0, hi = t;
             while (hi - lo > 1) {
                 const int mid = (lo + hi) >> 1;
                 if ((int)s_tb[mid] <= p) lo = mid; else hi = mid;
             }
-            const int64_t first = __ldg(a.row_off + lo), rows = __ldg(a.row_off + lo + 1) - first;
-            const u32 key = (u32)(first + min(max(idx, (int64_t)0), rows - 1));
+            const u32 key = s_first[lo] + min((u32)max(row, 0), s_rows[lo] - 1u);
             u32 h = (key * 2654435761u) >> (32 - HASH_BITS);
             for (int tries = 0; tries < (1 << HASH_BITS); ++tries) {
                 const u32 seen = reinterpret_cast<volatile u32 *>(s_mid)[h];
