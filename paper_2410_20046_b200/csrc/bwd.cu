@@ -141,7 +141,7 @@ seg_emit_kernel(const u32 *__restrict__ keys, int64_t L, const u32 *__restrict__
                 u32 *__restrict__ absmax, int ck_shift)
 {
     dq_wait_before();
-    extern __shared__ unsigned char smem_raw[];
+    extern __shared__ __align__(16) unsigned char smem_raw[];
     int64_t *s_off = reinterpret_cast<int64_t *>(smem_raw);   // [T+1]
     __shared__ u32 wsum[ST_WARPS];
     __shared__ u32 s_prefix;

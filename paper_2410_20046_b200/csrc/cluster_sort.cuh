@@ -49,7 +49,7 @@ __global__ void __launch_bounds__(THREADS, CL > 8 ? 1 : 2)
 cluster_sort_kernel(const __grid_constant__ Args a)
 {
     dq_wait_before();
-    extern __shared__ uint2 s_dyn[];               // pair buffers [2][cap]: (row within table, payload)
+    extern __shared__ __align__(16) uint2 s_dyn[];               // pair buffers [2][cap]: (row within table, payload)
     __shared__ __align__(16) u32 s_cnt[WARPS][BINS];
     __shared__ u32 s_hist[BINS];
     __shared__ u32 s_scan[BINS / 32];

@@ -95,7 +95,7 @@ dp_sum_update_kernel(float *__restrict__ tables, const int64_t *__restrict__ row
                      const int8_t *__restrict__ codes_cat, const float *__restrict__ grad_scales, float lr,
                      int32_t *__restrict__ sums_out, int T, int D, int64_t n_src, float2 *__restrict__ row_summary)
 {
-    extern __shared__ unsigned char smem_raw[];
+    extern __shared__ __align__(16) unsigned char smem_raw[];
     int32_t *s_uoff = reinterpret_cast<int32_t *>(smem_raw);
     for (int t = threadIdx.x; t <= T; t += blockDim.x) s_uoff[t] = union_off[t];
     __syncthreads();

@@ -40,7 +40,7 @@ pack_kernel(const float4 *__restrict__ arena4, const int64_t *__restrict__ row_o
             const float *__restrict__ scales, uint8_t *__restrict__ packed)
 {
     dq_wait_before();
-    extern __shared__ unsigned char smem_raw[];
+    extern __shared__ __align__(16) unsigned char smem_raw[];
     int64_t *v4_off = reinterpret_cast<int64_t *>(smem_raw);       // table starts in 128-bit vectors
     const int d4 = D >> 2;
     for (int t = threadIdx.x; t <= T; t += PK_THREADS) v4_off[t] = row_off[t] * d4;

@@ -23,7 +23,7 @@ absmax_kernel(const float *__restrict__ grad_rows, const int32_t *__restrict__ u
               u32 *__restrict__ absmax)
 {
     dq_wait_before();
-    extern __shared__ unsigned char smem_raw[];
+    extern __shared__ __align__(16) unsigned char smem_raw[];
     int32_t *s_uoff = reinterpret_cast<int32_t *>(smem_raw);      // [T+1]
     u32 *s_max = reinterpret_cast<u32 *>(s_uoff + (T + 1));       // [T]
     for (int t = threadIdx.x; t <= T; t += QU_THREADS) s_uoff[t] = uniq_off[t];
@@ -323,7 +323,7 @@ row_stream_kernel(float *__restrict__ tables, const int64_t *__restrict__ row_of
                   int *__restrict__ status, float2 *__restrict__ row_summary)
 {
     dq_wait_before();
-    extern __shared__ unsigned char smem_raw[];
+    extern __shared__ __align__(16) unsigned char smem_raw[];
     row_stream_body<MODE, LPR, CH, EXACT, TRACK>(smem_raw, tables, row_off, unique_rows, uniq_off, grad_rows, absmax,
                                                  codes, grad_scales, lr, T, D_any, status, row_summary);
 }

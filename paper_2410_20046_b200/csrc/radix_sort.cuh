@@ -46,7 +46,7 @@ __global__ void __launch_bounds__(1024)
 rs_setup_kernel(const Args a)
 {
     dq_wait_before();
-    extern __shared__ u32 s_tb[];                      // [T+1]
+    extern __shared__ __align__(16) u32 s_tb[];                      // [T+1]
     u32 *s_t0 = s_tb + (a.T + 1);                      // [T+1]
     const int lane = threadIdx.x & 31;
     if (threadIdx.x < 32) {
@@ -217,7 +217,7 @@ rs_scatter_kernel(const Args a, const uint2 *__restrict__ pairs_in, uint2 *__res
                   u32 *__restrict__ keys_out, u32 *__restrict__ vals_out, int shift)
 {
     dq_wait_before();
-    extern __shared__ uint2 s_pair[];                  // [TILE]
+    extern __shared__ __align__(16) uint2 s_pair[];                  // [TILE]
     const int nb = 1 << a.dbits;
     u32 *s_delta = reinterpret_cast<u32 *>(s_pair + TILE);                               // [nb]
     unsigned short *s_cnt = reinterpret_cast<unsigned short *>(s_delta + nb);            // [WARPS][nb]

@@ -45,7 +45,7 @@ refresh_kernel(const V *__restrict__ arena4, const int64_t *__restrict__ row_off
                u32 *__restrict__ done)
 {
     dq_wait_before();
-    extern __shared__ unsigned char smem_raw[];
+    extern __shared__ __align__(16) unsigned char smem_raw[];
     int64_t *v4_off = reinterpret_cast<int64_t *>(smem_raw);             // [T+1] table starts in float4 units
     u32 *s_min = reinterpret_cast<u32 *>(v4_off + (T + 1));              // [T]
     u32 *s_max = s_min + T;                                              // [T]

@@ -47,7 +47,7 @@ seg_groups_kernel(const __grid_constant__ Args a)
 {
     dq_wait_before();
     constexpr int GP = 32 / LPR;                  // lane groups of the warp
-    extern __shared__ u32 s_uoff[];                                                      // [T+1]
+    extern __shared__ __align__(16) u32 s_uoff[];                                                      // [T+1]
     u32 *s_tb = s_uoff + (a.T + 1);                                                      // [T+1] (by table)
     u32 *s_row = s_tb + (a.T + 1);                                                       // [T+1] (by table)
     __shared__ u32 s_broken;

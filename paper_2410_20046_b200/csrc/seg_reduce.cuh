@@ -154,7 +154,7 @@ seg_sum_kernel(const Args a)
     constexpr int NB = I / C;                     // batches per tile
     static_assert(NB % 2 == 0 && I <= 32, "");
     typedef typename Vec<VEC>::type vec_t;
-    extern __shared__ u32 s_uoff[];                                                      // [T+1]
+    extern __shared__ __align__(16) u32 s_uoff[];                                                      // [T+1]
     u32 *s_tb = s_uoff + (a.T + 1);                                                      // [T+1] (by table)
     u32 *s_row = s_tb + (a.T + 1);                                                       // [T+1] (by table)
     __shared__ u32 s_broken;

@@ -286,7 +286,7 @@ __global__ void __launch_bounds__(THREADS)
 small_sort_kernel(const __grid_constant__ csort::Args a)
 {
     dq_wait_before();
-    extern __shared__ u64 s_net[];                 // [2][THREADS * EPT]
+    extern __shared__ __align__(16) u64 s_net[];                 // [2][THREADS * EPT]
     const int t = blockIdx.x, tid = threadIdx.x;
     const int64_t tb0 = __ldg(a.offsets + (int64_t)t * a.B), tb1 = __ldg(a.offsets + (int64_t)(t + 1) * a.B);
     if (tb0 < 0 || tb1 < tb0 || tb1 > a.L || (t == 0 && tb0 != 0) || (t == a.T - 1 && tb1 != a.L)) {

@@ -50,7 +50,7 @@ inline size_t smem_bytes(int T) { return (size_t)THREADS * 2 * sizeof(u64) + (MI
 __global__ void __launch_bounds__(THREADS)
 small_step_kernel(const __grid_constant__ Args x)
 {
-    extern __shared__ u64 s_net[];                 // [2][THREADS]
+    extern __shared__ __align__(16) u64 s_net[];                 // [2][THREADS]
     u32 *s_mid = reinterpret_cast<u32 *>(s_net + 2 * THREADS);
     u32 *s_tb = s_mid + MID_WORDS;                 // [T+1]
     u32 *s_first = s_tb + x.s.T + 1, *s_rows = s_first + x.s.T;        // [T] arena row where a table begins, and its rows
