@@ -339,6 +339,7 @@ seg_groups_kernel(const __grid_constant__ Args a)
             __syncwarp();
             bool final = false;
             if (wl == 0) final = arrive(&a.range_done[f].x) == ng - 1u;
+            __syncwarp();                         // (what lane 0 has acquired, the warp loads)
             if (!__shfl_sync(0xffffffffu, final, 0)) continue;
             fold((int)ng, sum, [&](int p) { return a.group_partials + ((size_t)(g0 + p) * 2 + (p == 0 ? 1 : 0)) * D; });
         }

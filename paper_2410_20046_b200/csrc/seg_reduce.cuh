@@ -402,6 +402,7 @@ seg_sum_kernel(const Args a)
             __syncwarp();
             bool final = false;
             if (wl == 0) final = arrive(&a.range_done[f].x) == ng - 1u;
+            __syncwarp();                         // (what lane 0 has acquired, the warp loads)
             if (!__shfl_sync(0xffffffffu, final, 0)) continue;
             for (int cc = wl; cc - wl < (COLS ? dv : 1); cc += 32) {
                 double sum[VEC];
