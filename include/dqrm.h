@@ -43,6 +43,10 @@
  *   - offsets[T*B + 1] int32, non-decreasing, offsets[0] = 0, offsets[T*B] = L:
  *     bag g = t*B + i owns indices[offsets[g] .. offsets[g+1]).  Empty bags are allowed.
  *   - out and grad_out are [B, T, D] float32 (sample-major).  T*B < 2^31.
+ *   - Alignment: tables, out, grad_out, grad_rows and sums_out 16 bytes, codes 4, packed rows and payloads
+ *     `bits` bytes.  (dqrm_emb_bwd and the training steps also take a grad_out, dqrm_emb_bwd a grad_rows, that
+ *     is aligned to 4 bytes where D is 4, and to 8 where D is 8 to 64.)  A pointer that the call's kernels
+ *     cannot use is refused with DQRM_ERR_INVALID_ARG.
  *   - bits[T] int32, each in 2..16.  scales[T] float32.
  *   - Return value: DQRM_OK or a negative error.  Invalid arguments are detected on the
  *     host before anything is launched.  Conditions only the device can see (an index
@@ -61,7 +65,7 @@ extern "C" {
 #endif
 
 #define DQRM_OK                 0
-#define DQRM_ERR_INVALID_ARG   (-1)  /* null pointer, bad T/D/B/L, bits outside 2..16 */
+#define DQRM_ERR_INVALID_ARG   (-1)  /* null or misaligned pointer, bad T/D/B/L, bits outside 2..16 */
 #define DQRM_ERR_WORKSPACE     (-2)  /* workspace null, misaligned (256 B) or too small */
 #define DQRM_ERR_CUDA          (-3)  /* a CUDA runtime call failed; see dqrm_last_cuda_error */
 #define DQRM_ERR_INDEX_RANGE   (-4)  /* device saw an index outside [0, R_t) or a bad offset */

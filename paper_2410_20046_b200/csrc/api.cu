@@ -19,6 +19,24 @@ inline bool batch_ok(const dqrm_ctx *ctx, int B, int64_t L)
     return ctx && B > 0 && L >= 0 && L < (int64_t)1 << 31 && (int64_t)ctx->T * B < ((int64_t)1 << 31) - 1;
 }
 
+// Rows are read and written 128 bits at a time, codes 32; a pointer that lies otherwise is refused before anything is launched (it
+// would be a misaligned access on the device).  The pooled forward of long bags and the sum take less where they need less.
+constexpr size_t ROW = sizeof(float4), CODES = sizeof(char4);
+
+bool fwd_aligned(const dqrm_ctx *ctx, const float *tables, const float *out, const int8_t *codes_out, int B, int64_t L)
+{
+    const size_t to = dq_fwd_align(ctx, codes_out, B, L);
+    return dq_aligned(out, to) && (L == 0 || (dq_aligned(tables, to) && dq_aligned(codes_out, CODES)));
+}
+
+bool step_aligned(const dqrm_ctx *ctx, const float *tables, const float *grad_out, const float *out, const float *grad_rows,
+                  const int8_t *codes, int B, int64_t L)
+{
+    return fwd_aligned(ctx, tables, out, nullptr, B, L) &&
+           (L == 0 || (dq_aligned(tables, ROW) && dq_aligned(grad_rows, ROW) && dq_aligned(codes, CODES) &&
+                       dq_aligned(grad_out, dq_sum_align(ctx))));
+}
+
 struct HostStepLayout {
     size_t indices[2], offsets[2], grad_out[2], out[2];      // two sets of staging buffers, used by alternate calls
     size_t unique_rows, uniq_off, grad_rows, codes, grad_scales, step_ws, total;
@@ -289,7 +307,7 @@ const char *dqrm_status_string(int status)
 int dqrm_scale_refresh(dqrm_ctx *ctx, const float *tables, const int32_t *bits, float *scales, float *minmax,
                        void *workspace, size_t workspace_bytes, void *stream)
 {
-    if (!ctx || !tables || !bits || !scales) return DQRM_ERR_INVALID_ARG;
+    if (!ctx || !tables || !bits || !scales || (!ctx->row_summary && !dq_aligned(tables, ROW))) return DQRM_ERR_INVALID_ARG;
     if (!ws_ok(workspace, workspace_bytes, dq_refresh_ws_bytes(ctx))) return DQRM_ERR_WORKSPACE;
     return dq_launch_refresh(ctx, tables, bits, scales, minmax, workspace, workspace_bytes, as_stream(stream));
 }
@@ -299,7 +317,7 @@ int dqrm_emb_fwd(dqrm_ctx *ctx, const float *tables, const int32_t *indices, con
                  void *stream)
 {
     if (!batch_ok(ctx, B, L) || !tables || !offsets || !scales || !bits || !out) return DQRM_ERR_INVALID_ARG;
-    if (L > 0 && !indices) return DQRM_ERR_INVALID_ARG;
+    if ((L > 0 && !indices) || !fwd_aligned(ctx, tables, out, codes_out, B, L)) return DQRM_ERR_INVALID_ARG;
     return dq_launch_fwd(ctx, tables, indices, offsets, scales, bits, out, codes_out, B, L, as_stream(stream));
 }
 
@@ -308,7 +326,9 @@ int dqrm_emb_bwd(dqrm_ctx *ctx, const float *grad_out, const int32_t *indices, c
                  void *workspace, size_t workspace_bytes, void *stream)
 {
     if (!batch_ok(ctx, B, L) || !grad_out || !offsets || !uniq_off) return DQRM_ERR_INVALID_ARG;
-    if (L > 0 && (!indices || !unique_rows || !grad_rows)) return DQRM_ERR_INVALID_ARG;
+    if (L > 0 && (!indices || !unique_rows || !grad_rows || !dq_aligned(grad_out, dq_sum_align(ctx)) ||
+                  !dq_aligned(grad_rows, dq_sum_align(ctx))))
+        return DQRM_ERR_INVALID_ARG;
     if (!ws_ok(workspace, workspace_bytes, dq_bwd_ws_bytes(ctx, L, (int64_t)ctx->T * B))) return DQRM_ERR_WORKSPACE;
     return dq_launch_bwd(ctx, grad_out, indices, offsets, unique_rows, uniq_off, grad_rows, B, L, workspace,
                          workspace_bytes, as_stream(stream));
@@ -317,7 +337,9 @@ int dqrm_emb_bwd(dqrm_ctx *ctx, const float *grad_out, const int32_t *indices, c
 int dqrm_grad_quant_int8_bounded(dqrm_ctx *ctx, const float *grad_rows, const int32_t *uniq_off, int8_t *codes,
                          float *grad_scales, int64_t max_values, void *workspace, size_t workspace_bytes, void *stream)
 {
-    if (!ctx || !grad_rows || !uniq_off || !codes || !grad_scales || max_values < 0) return DQRM_ERR_INVALID_ARG;
+    if (!ctx || !grad_rows || !uniq_off || !codes || !grad_scales || max_values < 0 || !dq_aligned(grad_rows, ROW) ||
+        !dq_aligned(codes, CODES))
+        return DQRM_ERR_INVALID_ARG;
     if (!ws_ok(workspace, workspace_bytes, dq_quant_ws_bytes(ctx))) return DQRM_ERR_WORKSPACE;
     return dq_launch_grad_quant(ctx, grad_rows, uniq_off, codes, grad_scales, max_values, workspace, workspace_bytes,
                                 as_stream(stream));
@@ -333,7 +355,8 @@ int dqrm_grad_quant_int8(dqrm_ctx *ctx, const float *grad_rows, const int32_t *u
 int dqrm_row_update(dqrm_ctx *ctx, float *tables, const int32_t *unique_rows, const int32_t *uniq_off,
                     const int8_t *codes, const float *grad_scales, float lr, void *stream)
 {
-    if (!ctx || !tables || !unique_rows || !uniq_off || !codes || !grad_scales) return DQRM_ERR_INVALID_ARG;
+    if (!ctx || !tables || !unique_rows || !uniq_off || !codes || !grad_scales || !dq_aligned(tables, ROW) || !dq_aligned(codes, CODES))
+        return DQRM_ERR_INVALID_ARG;
     return dq_launch_row_update(ctx, tables, unique_rows, uniq_off, codes, grad_scales, lr, as_stream(stream));
 }
 
@@ -346,10 +369,11 @@ int dqrm_train_step(dqrm_ctx *ctx, float *tables, const int32_t *indices, const 
         !grad_scales)
         return DQRM_ERR_INVALID_ARG;
     if (L > 0 && (!indices || !unique_rows || !grad_rows || !codes)) return DQRM_ERR_INVALID_ARG;
+    if (!step_aligned(ctx, tables, grad_out, out, grad_rows, codes, B, L)) return DQRM_ERR_INVALID_ARG;
     if (!ws_ok(workspace, workspace_bytes, dq_bwd_ws_bytes(ctx, L, (int64_t)ctx->T * B))) return DQRM_ERR_WORKSPACE;
     cudaStream_t st = as_stream(stream);
     if (ctx->prof_on) dq_mark(ctx, st, DQ_K_BEGIN);
-    if (dq_small_step_takes(ctx, B, L)) {
+    if (dq_small_step_takes(ctx, B, L) && dq_aligned(grad_out, ROW)) {
         const int rc = dq_launch_fwd(ctx, tables, indices, offsets, scales, bits, out, nullptr, B, L, st, true);
         if (rc != DQRM_OK) return rc;
         return dq_launch_small_step(ctx, tables, indices, offsets, grad_out, unique_rows, uniq_off, grad_rows, codes,
@@ -386,14 +410,16 @@ int dqrm_train_step(dqrm_ctx *ctx, float *tables, const int32_t *indices, const 
 
 int dqrm_grad_absmax(dqrm_ctx *ctx, const float *grad_rows, const int32_t *uniq_off, float *absmax, void *stream)
 {
-    if (!ctx || !grad_rows || !uniq_off || !absmax) return DQRM_ERR_INVALID_ARG;
+    if (!ctx || !grad_rows || !uniq_off || !absmax || !dq_aligned(grad_rows, ROW)) return DQRM_ERR_INVALID_ARG;
     return dq_launch_grad_absmax(ctx, grad_rows, uniq_off, absmax, as_stream(stream));
 }
 
 int dqrm_grad_quant_int8_unified(dqrm_ctx *ctx, const float *grad_rows, const int32_t *uniq_off,
                                  const float *unified_absmax, int8_t *codes, float *grad_scales, void *stream)
 {
-    if (!ctx || !grad_rows || !uniq_off || !unified_absmax || !codes || !grad_scales) return DQRM_ERR_INVALID_ARG;
+    if (!ctx || !grad_rows || !uniq_off || !unified_absmax || !codes || !grad_scales || !dq_aligned(grad_rows, ROW) ||
+        !dq_aligned(codes, CODES))
+        return DQRM_ERR_INVALID_ARG;
     return dq_launch_grad_quant_unified(ctx, grad_rows, uniq_off, unified_absmax, codes, grad_scales, as_stream(stream));
 }
 
@@ -412,7 +438,9 @@ int dqrm_dp_merge_update(dqrm_ctx *ctx, float *tables, int W, int64_t rank_strid
         n_entries > (int64_t)W * rank_stride || max_table_entries < 0 || max_table_entries > n_entries ||
         n_entries >= ((int64_t)1 << 31))
         return DQRM_ERR_INVALID_ARG;
-    if (n_entries > 0 && (!rows_cat || !codes_cat || !union_rows)) return DQRM_ERR_INVALID_ARG;
+    if (n_entries > 0 && (!rows_cat || !codes_cat || !union_rows || !dq_aligned(tables, ROW) || !dq_aligned(codes_cat, CODES) ||
+                          !dq_aligned(sums_out, sizeof(int4))))
+        return DQRM_ERR_INVALID_ARG;
     if (!ws_ok(workspace, workspace_bytes, 1)) return DQRM_ERR_WORKSPACE;
     return dq_launch_dp_merge_update(ctx, tables, W, rank_stride, rows_cat, uoff_cat, codes_cat, grad_scales, lr,
                                      n_entries, max_table_entries, union_rows, union_off, sums_out, workspace,
@@ -459,6 +487,7 @@ int dqrm_train_step_sorted(dqrm_ctx *ctx, float *tables, const int32_t *indices,
         !grad_scales)
         return DQRM_ERR_INVALID_ARG;
     if (L > 0 && (!indices || !unique_rows || !grad_rows || !codes)) return DQRM_ERR_INVALID_ARG;
+    if (!step_aligned(ctx, tables, grad_out, out, grad_rows, codes, B, L)) return DQRM_ERR_INVALID_ARG;
     if (!ws_ok(workspace, workspace_bytes, dq_bwd_ws_bytes(ctx, L, (int64_t)ctx->T * B))) return DQRM_ERR_WORKSPACE;
     cudaEvent_t sort_done = nullptr;
     bool sort_captured = false, by_table = false;
@@ -528,7 +557,7 @@ size_t dqrm_row_summary_bytes(const dqrm_ctx *ctx)
 
 int dqrm_row_summary_attach(dqrm_ctx *ctx, const float *tables, void *summary, size_t summary_bytes, void *stream)
 {
-    if (!ctx || !tables || !summary || ((uintptr_t)summary & 7u)) return DQRM_ERR_INVALID_ARG;
+    if (!ctx || !tables || !summary || !dq_aligned(summary, sizeof(float2)) || !dq_aligned(tables, ROW)) return DQRM_ERR_INVALID_ARG;
     if (summary_bytes < dqrm_row_summary_bytes(ctx)) return DQRM_ERR_WORKSPACE;
     const int rc = dq_launch_row_summary(ctx, tables, reinterpret_cast<float2 *>(summary), as_stream(stream));
     if (rc == DQRM_OK) ctx->row_summary = reinterpret_cast<float2 *>(summary);
@@ -555,6 +584,7 @@ int dqrm_emb_fwd_codes(dqrm_ctx *ctx, const float *tables, const int32_t *indice
     if (!batch_ok(ctx, B, L) || !tables || !offsets || !scales || !payload || (bits != 2 && bits != 4 && bits != 8))
         return DQRM_ERR_INVALID_ARG;
     if (L != (int64_t)ctx->T * B || (L > 0 && !indices)) return DQRM_ERR_INVALID_ARG;     // one index per bag
+    if (!dq_aligned(tables, ROW) || !dq_aligned(payload, dq_pack_align(bits))) return DQRM_ERR_INVALID_ARG;
     return dq_launch_fwd_codes(ctx, tables, indices, offsets, scales, bits, payload, B, L, as_stream(stream));
 }
 
@@ -564,6 +594,7 @@ int dqrm_decode_payload(dqrm_ctx *ctx, const uint8_t *payload, const float *scal
     if (!ctx || !payload || !scales || !out || B < 0 || T_blk < 0 || t0 < 0 || t0 + T_blk > T_total ||
         (bits != 2 && bits != 4 && bits != 8))
         return DQRM_ERR_INVALID_ARG;
+    if (B > 0 && T_blk > 0 && (!dq_aligned(payload, dq_pack_align(bits)) || !dq_aligned(out, ROW))) return DQRM_ERR_INVALID_ARG;
     return dq_launch_decode_payload(ctx, payload, scales, bits, out, B, T_blk, T_total, t0, as_stream(stream));
 }
 
@@ -576,6 +607,7 @@ size_t dqrm_packed_bytes(const dqrm_ctx *ctx, int bits)
 int dqrm_pack_tables(dqrm_ctx *ctx, const float *tables, const float *scales, int bits, uint8_t *packed, void *stream)
 {
     if (!ctx || !tables || !scales || !packed || (bits != 2 && bits != 4 && bits != 8)) return DQRM_ERR_INVALID_ARG;
+    if (!dq_aligned(tables, ROW) || !dq_aligned(packed, dq_pack_align(bits))) return DQRM_ERR_INVALID_ARG;
     return dq_launch_pack(ctx, tables, scales, bits, packed, as_stream(stream));
 }
 
@@ -584,7 +616,8 @@ int dqrm_packed_fwd(dqrm_ctx *ctx, const uint8_t *packed, const int32_t *indices
 {
     if (!batch_ok(ctx, B, L) || !packed || !offsets || !scales || !out || (bits != 2 && bits != 4 && bits != 8))
         return DQRM_ERR_INVALID_ARG;
-    if (L > 0 && !indices) return DQRM_ERR_INVALID_ARG;
+    if (L > 0 && (!indices || !dq_aligned(packed, dq_packed_align(ctx, bits, B, L)))) return DQRM_ERR_INVALID_ARG;
+    if (!dq_aligned(out, ROW)) return DQRM_ERR_INVALID_ARG;
     return dq_launch_packed_fwd(ctx, packed, indices, offsets, scales, bits, out, B, L, as_stream(stream));
 }
 
@@ -600,7 +633,7 @@ int dqrm_train_step_host(dqrm_ctx *ctx, float *tables, const int32_t *h_indices,
 {
     if (!batch_ok(ctx, B, L) || !tables || !h_offsets || !h_grad_out || !scales || !bits || !h_out)
         return DQRM_ERR_INVALID_ARG;
-    if (L > 0 && !h_indices) return DQRM_ERR_INVALID_ARG;
+    if (L > 0 && (!h_indices || !dq_aligned(tables, ROW))) return DQRM_ERR_INVALID_ARG;
     const int64_t G = (int64_t)ctx->T * B;
     if (!ws_ok(workspace, workspace_bytes, host_layout(ctx, L, G).total)) return DQRM_ERR_WORKSPACE;
     // the places follow from (workspace, its size, bags): worked out again only when one of them is another

@@ -272,7 +272,9 @@ int launch_sum_groups(dqrm_ctx *ctx, const segred::Args &a, cudaStream_t st)
     unsigned warps = GROUPS_THREADS / 32;
     while (warps > 2 && a.ranges < warps * (unsigned)ctx->num_sms) warps /= 2;
     const dim3 grid((a.ranges + warps - 1) / warps), block(warps * 32);
-    if (ctx->D == LPR * 4) DQRM_CUDA_TRY(ctx, (dq_launch(seg_groups_kernel<LPR, true>, grid, block, smem_bytes(ctx->T), st, a)));
+    if (!dq_aligned(a.grad_out, sizeof(float4)) || !dq_aligned(a.grad_rows, sizeof(float4)))
+        DQRM_CUDA_TRY(ctx, (dq_launch(seg_groups_kernel<LPR, false, unaligned_vec(LPR)>, grid, block, smem_bytes(ctx->T), st, a)));
+    else if (ctx->D == LPR * 4) DQRM_CUDA_TRY(ctx, (dq_launch(seg_groups_kernel<LPR, true>, grid, block, smem_bytes(ctx->T), st, a)));
     else DQRM_CUDA_TRY(ctx, (dq_launch(seg_groups_kernel<LPR, false>, grid, block, smem_bytes(ctx->T), st, a)));
     dq_mark(ctx, st, DQ_K_SEG_SUM);
     return DQRM_OK;
@@ -396,6 +398,12 @@ size_t dq_bwd_ws_bytes(const dqrm_ctx *ctx, int64_t L, int64_t G)
 {
     (void)G;
     return make_layout(ctx, L).total;
+}
+
+size_t dq_sum_align(const dqrm_ctx *ctx)
+{
+    if (segred::takes_groups(ctx->D)) return sizeof(float) * segred::unaligned_vec(segred::lanes_per_row(ctx->D));
+    return sizeof(float) * segred::floats_per_lane(ctx->D);
 }
 
 // first half of the backward: everything that depends only on the indices (sort, unique rows,

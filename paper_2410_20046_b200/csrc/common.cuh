@@ -130,6 +130,7 @@ __device__ __forceinline__ void dq_let_next()
 }
 
 static inline size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
+static inline bool dq_aligned(const void *p, size_t to) { return (reinterpret_cast<uintptr_t>(p) & (to - 1)) == 0; }
 
 // slots of dqrm_ctx::smem_raised
 constexpr int DQ_SMEM_SLOT_STEP = 4, DQ_SMEM_SLOT_CSORT = 8;
@@ -364,6 +365,8 @@ size_t dq_refresh_ws_bytes(const dqrm_ctx *ctx);
 int dq_launch_refresh(dqrm_ctx *ctx, const float *tables, const int32_t *bits, float *scales,
                       float *minmax, void *ws, size_t ws_bytes, cudaStream_t st);
 
+// bytes that tables and out have to be aligned to
+size_t dq_fwd_align(const dqrm_ctx *ctx, const int8_t *codes_out, int B, int64_t L);
 int dq_launch_fwd(dqrm_ctx *ctx, const float *tables, const int32_t *indices, const int32_t *offsets,
                   const float *scales, const int32_t *bits, float *out, int8_t *codes_out,
                   int B, int64_t L, cudaStream_t st, bool let_next = false);
@@ -375,6 +378,8 @@ int dq_launch_small_step(dqrm_ctx *ctx, float *tables, const int32_t *indices, c
                          int B, int64_t L, void *ws, size_t ws_bytes, cudaStream_t st);
 
 size_t dq_bwd_ws_bytes(const dqrm_ctx *ctx, int64_t L, int64_t G);
+// bytes that the summed gradient and what it is summed from have to be aligned to
+size_t dq_sum_align(const dqrm_ctx *ctx);
 // per-table |grad| maxima (float bit patterns) inside a workspace that dq_launch_bwd_sort and
 // dq_launch_bwd_sum have filled
 const u32 *dq_bwd_absmax_bits(const dqrm_ctx *ctx, int64_t L, const void *ws);
@@ -397,6 +402,9 @@ int dq_launch_grad_absmax(dqrm_ctx *ctx, const float *grad_rows, const int32_t *
 int dq_launch_grad_quant_unified(dqrm_ctx *ctx, const float *grad_rows, const int32_t *uniq_off,
                                  const float *unified_absmax, int8_t *codes, float *grad_scales, cudaStream_t st);
 int dq_launch_pack(dqrm_ctx *ctx, const float *tables, const float *scales, int bits, uint8_t *packed, cudaStream_t st);
+// bytes that packed rows have to be aligned to, written and read
+inline size_t dq_pack_align(int bits) { return bits / 2; }
+size_t dq_packed_align(const dqrm_ctx *ctx, int bits, int B, int64_t L);
 int dq_launch_packed_fwd(dqrm_ctx *ctx, const uint8_t *packed, const int32_t *indices, const int32_t *offsets,
                          const float *scales, int bits, float *out, int B, int64_t L, cudaStream_t st);
 int dq_launch_fwd_codes(dqrm_ctx *ctx, const float *tables, const int32_t *indices, const int32_t *offsets,

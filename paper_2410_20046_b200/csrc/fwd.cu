@@ -360,7 +360,8 @@ fwd_long_bags_kernel(const FwdArgs a)
 // batches (26 x 8192 bags of 256-byte rows 159 us both) and lane groups ahead in small ones (4 x 2048 bags 9.2 against 10.3
 // us); at 24 it is 212 against 223 us, and with bags of uneven length the warps are ahead from 12 on
 constexpr int LONG_BAG = 18;
-inline bool warp_per_bag(const FwdArgs &a, int lpr) { return lpr == 16 && !a.codes_out && a.L >= LONG_BAG * (int64_t)a.T * a.B; }
+inline bool long_bags(const int8_t *codes_out, int T, int B, int64_t L) { return !codes_out && L >= LONG_BAG * (int64_t)T * B; }
+inline bool warp_per_bag(const FwdArgs &a, int lpr) { return lpr == 16 && long_bags(a.codes_out, a.T, a.B, a.L); }
 
 template <int LPR, int CH, bool EXACT>
 cudaError_t launch_bags(const FwdArgs &a, dim3 grid, cudaStream_t st)
@@ -400,6 +401,11 @@ int launch(dqrm_ctx *ctx, const FwdArgs &a, cudaStream_t st)
 }
 
 }  // namespace
+
+size_t dq_fwd_align(const dqrm_ctx *ctx, const int8_t *codes_out, int B, int64_t L)
+{
+    return ctx->D > 32 && ctx->D <= 64 && long_bags(codes_out, ctx->T, B, L) ? sizeof(float2) : sizeof(float4);
+}
 
 int dq_launch_fwd(dqrm_ctx *ctx, const float *tables, const int32_t *indices, const int32_t *offsets,
                   const float *scales, const int32_t *bits, float *out, int8_t *codes_out,

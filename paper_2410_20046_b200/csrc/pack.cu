@@ -363,11 +363,12 @@ int dispatch_pfwd2(dqrm_ctx *ctx, const PfArgs &a, cudaStream_t st)
 #undef DQ_PF
 }
 
+inline bool eight_a_lane(int T, int D, int B, int64_t L) { return D % 8 == 0 && (D > 128 || L != (int64_t)T * B); }
+
 template <int BITS>
 int dispatch_pfwd(dqrm_ctx *ctx, const PfArgs &a, cudaStream_t st)
 {
-    const bool onehot = a.L == (int64_t)a.T * a.B;
-    if (a.D % 8 == 0 && (a.D > 128 || !onehot)) return dispatch_pfwd2<BITS, 8>(ctx, a, st);
+    if (eight_a_lane(a.T, a.D, a.B, a.L)) return dispatch_pfwd2<BITS, 8>(ctx, a, st);
     return dispatch_pfwd2<BITS, 4>(ctx, a, st);
 }
 
@@ -378,6 +379,11 @@ int dq_launch_pack(dqrm_ctx *ctx, const float *tables, const float *scales, int 
     if (bits == 2) return launch_pack<2>(ctx, tables, scales, packed, st);
     if (bits == 4) return launch_pack<4>(ctx, tables, scales, packed, st);
     return launch_pack<8>(ctx, tables, scales, packed, st);
+}
+
+size_t dq_packed_align(const dqrm_ctx *ctx, int bits, int B, int64_t L)
+{
+    return dq_pack_align(bits) * (eight_a_lane(ctx->T, ctx->D, B, L) ? 2 : 1);
 }
 
 int dq_launch_packed_fwd(dqrm_ctx *ctx, const uint8_t *packed, const int32_t *indices, const int32_t *offsets,

@@ -465,7 +465,8 @@ std::mutex g_static_mutex;        // host threads may make a device's first call
 extern "C" int dqrm_grad_quant_int8_static(int T, int D, const float *grad_rows, const int32_t *uniq_off,
                                            int8_t *codes, float *grad_scales, void *stream)
 {
-    if (T <= 0 || D < 4 || D > 1024 || (D % 4) != 0 || !grad_rows || !uniq_off || !codes || !grad_scales)
+    if (T <= 0 || D < 4 || D > 1024 || (D % 4) != 0 || !grad_rows || !uniq_off || !codes || !grad_scales ||
+        !dq_aligned(grad_rows, sizeof(float4)) || !dq_aligned(codes, sizeof(char4)))
         return DQRM_ERR_INVALID_ARG;
     if (T > DQRM_STATIC_MAX_TABLES) return DQRM_ERR_STATIC_LIMIT;
     int dev = -1;

@@ -40,8 +40,11 @@ static_assert((1 << CHUNK_SHIFT) % (2 * BATCH) == 0, "the walk takes two batches
 __host__ __device__ constexpr bool takes_groups(int D) { return D <= 48; }
 __host__ __device__ constexpr int lanes_per_row(int D) { return D <= 4 ? 1 : D <= 8 ? 2 : D <= 16 ? 4 : D <= 32 ? 8 : 16; }
 
-// One range a warp; blocks of two warps at least.  EXACT: every lane holds features
-template <int LPR, bool EXACT>
+// One range a warp; blocks of two warps at least.  EXACT: every lane holds features.  VEC: features of one access to the rows,
+// fewer than four where a caller's rows do not begin on 16 bytes
+__host__ __device__ constexpr int unaligned_vec(int LPR) { return LPR == 1 ? 1 : 2; }
+
+template <int LPR, bool EXACT, int VEC = 4>
 __global__ void __launch_bounds__(GROUPS_THREADS, GROUPS_BLOCKS)
 seg_groups_kernel(const __grid_constant__ Args a)
 {
@@ -127,6 +130,18 @@ seg_groups_kernel(const __grid_constant__ Args a)
     const uint64_t keep = dq_policy_evict_last();
     const uint64_t pol = L <= G ? dq_policy_evict_first() : dq_policy_evict_normal();
     const float4 *go = reinterpret_cast<const float4 *>(a.grad_out) + (on ? lane : 0);
+    auto load_row = [&](u32 row) {
+        const float4 *p = go + (int64_t)row * dv;
+        if constexpr (VEC == 4) {
+            return dq_ld_nc(p, pol);
+        } else if constexpr (VEC == 2) {
+            const float2 *q = reinterpret_cast<const float2 *>(p), x = ld_row(q, pol), y = ld_row(q + 1, pol);
+            return make_float4(x.x, x.y, y.x, y.y);
+        } else {
+            const float *q = reinterpret_cast<const float *>(p);
+            return make_float4(__ldg(q), __ldg(q + 1), __ldg(q + 2), __ldg(q + 3));
+        }
+    };
     auto checked = [&](u32 row) {
         if (row >= G) { dq_report(a.status, DQRM_ERR_INDEX_RANGE); row = 0u; }
         return row;
@@ -134,10 +149,10 @@ seg_groups_kernel(const __grid_constant__ Args a)
     // the rows of a batch, all at once (any row for entries past the end, and a vector of the row for lanes past its end:
     // nothing is done with either)
     auto request = [&](const uint4 &v, float4 (&r)[BATCH]) {
-        r[0] = dq_ld_nc(go + (int64_t)checked(v.x) * dv, pol);
-        r[1] = dq_ld_nc(go + (int64_t)checked(v.y) * dv, pol);
-        r[2] = dq_ld_nc(go + (int64_t)checked(v.z) * dv, pol);
-        r[3] = dq_ld_nc(go + (int64_t)checked(v.w) * dv, pol);
+        r[0] = load_row(checked(v.x));
+        r[1] = load_row(checked(v.y));
+        r[2] = load_row(checked(v.z));
+        r[3] = load_row(checked(v.w));
     };
     float4 v[2][BATCH];
     request(val, v[0]);
@@ -164,7 +179,18 @@ seg_groups_kernel(const __grid_constant__ Args a)
     auto note = [&](int tt, float x) { if (x > 0.f) atomicMax(a.absmax + tt, __float_as_uint(x)); };
     auto store_row = [&](u32 uu, const double (&acc)[4]) {
         float x = 0.f;
-        if (on) dq_st_keep(reinterpret_cast<float4 *>(a.grad_rows + (int64_t)uu * D) + lane, rounded(acc, x), keep);  // quantise+update reads it next
+        if (on) {
+            const float4 r = rounded(acc, x);
+            float *p = reinterpret_cast<float *>(reinterpret_cast<float4 *>(a.grad_rows + (int64_t)uu * D) + lane);
+            if constexpr (VEC == 4) {
+                dq_st_keep(reinterpret_cast<float4 *>(p), r, keep);      // quantise+update reads it next
+            } else if constexpr (VEC == 2) {
+                st_row(reinterpret_cast<float2 *>(p), make_float2(r.x, r.y), keep);
+                st_row(reinterpret_cast<float2 *>(p) + 1, make_float2(r.z, r.w), keep);
+            } else {
+                p[0] = r.x; p[1] = r.y; p[2] = r.z; p[3] = r.w;
+            }
+        }
         return x;
     };
     double acc[4] = {0.0, 0.0, 0.0, 0.0};         // the open run

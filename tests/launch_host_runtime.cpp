@@ -50,6 +50,13 @@ void **__cudaRegisterFatBinary(void *)
 void __cudaRegisterFatBinaryEnd(void **) {}
 void __cudaUnregisterFatBinary(void **) {}
 void __cudaRegisterFunction(void **, const char *, char *, const char *, int, uint3 *, uint3 *, dim3 *, dim3 *, int *) {}
-unsigned __cudaPushCallConfiguration(dim3, dim3, size_t, struct CUstream_st *) { return 0; }
-cudaError_t __cudaPopCallConfiguration(dim3 *, dim3 *, size_t *, void *) { return cudaSuccess; }
+static size_t pushed_smem;
+unsigned __cudaPushCallConfiguration(dim3, dim3, size_t smem, struct CUstream_st *) { return pushed_smem = smem, 0; }
+cudaError_t __cudaPopCallConfiguration(dim3 *grid, dim3 *block, size_t *smem, void *stream)
+{
+    *grid = *block = dim3(1);
+    *smem = pushed_smem;
+    *static_cast<cudaStream_t *>(stream) = nullptr;
+    return cudaSuccess;
+}
 }
