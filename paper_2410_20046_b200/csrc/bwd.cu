@@ -321,19 +321,16 @@ int launch_radix_sort(dqrm_ctx *ctx, const rsort::Args &a, int passes, uint2 *co
     return DQRM_OK;
 }
 
-template <int CL, int EPT = 0>
-cudaError_t launch_cluster_sort(dqrm_ctx *ctx, csort::Args ca, int cap, cudaStream_t st)
+// (slot: of smem_raised, one for each kernel)
+template <int CL>
+cudaError_t launch_clusters(dqrm_ctx *ctx, void (*kernel)(csort::Args), int slot, const csort::Args &ca, size_t smem, cudaStream_t st)
 {
-    ca.cap = cap;
-    const size_t smem = std::max(csort::smem_bytes(cap), EPT ? sizeof(uint2) * csort::SORT_ROOM : (size_t)0);
-    static_assert(CL == csort::CLUSTER || EPT == 0, "");
-    bool &raised = ctx->smem_raised[DQ_SMEM_SLOT_CSORT + (CL == csort::CLUSTER ? EPT : 3)];
+    bool &raised = ctx->smem_raised[DQ_SMEM_SLOT_CSORT + slot];
     cudaError_t e = cudaSuccess;
     if (!raised) {
-        e = cudaFuncSetAttribute(csort::cluster_sort_kernel<CL, EPT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)csort::smem_bytes(12288));
+        e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)csort::smem_bytes(12288));
         if (e == cudaSuccess && CL > 8)       // more than eight blocks in a cluster is an opt-in
-            e = cudaFuncSetAttribute(csort::cluster_sort_kernel<CL, EPT>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+            e = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
         raised = (e == cudaSuccess);
     }
     if (e == cudaSuccess) {
@@ -348,10 +345,29 @@ cudaError_t launch_cluster_sort(dqrm_ctx *ctx, csort::Args ca, int cap, cudaStre
         attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
         attr[1].val.programmaticStreamSerializationAllowed = 1;
         cfg.attrs = attr; cfg.numAttrs = 2;
-        e = cudaLaunchKernelEx(&cfg, csort::cluster_sort_kernel<CL, EPT>, ca);
+        e = cudaLaunchKernelEx(&cfg, kernel, ca);
     }
     if (e != cudaSuccess) (void)cudaGetLastError();
     return e;
+}
+
+template <int CL>
+cudaError_t launch_cluster_sort(dqrm_ctx *ctx, csort::Args ca, int cap, cudaStream_t st)
+{
+    ca.cap = cap;
+    return launch_clusters<CL>(ctx, csort::cluster_sort_kernel<CL, 0>, CL == csort::CLUSTER ? 0 : 3, ca, csort::smem_bytes(cap), st);
+}
+
+// clusters that stand by for tables beyond what their first block takes
+template <int EPT>
+cudaError_t launch_standby_sort(dqrm_ctx *ctx, csort::Args ca, bool even, cudaStream_t st)
+{
+    constexpr int CL = csort::CLUSTER;
+    ca.cap = even ? csort::SORT_ROOM / 2 : csort::shared_cap(ca.L);
+    const size_t smem = std::max(csort::smem_bytes(ca.cap), sizeof(uint2) * csort::SORT_ROOM);
+    if constexpr (EPT == 4)
+        if (even) return launch_clusters<CL>(ctx, ssort::block_sort_kernel<EPT, CL>, 5, ca, smem, st);
+    return launch_clusters<CL>(ctx, csort::cluster_sort_kernel<CL, EPT>, EPT, ca, smem, st);
 }
 
 // The block sort; false where the batch is too large for it.  `per_table` lookups a table on average, with room for a
@@ -360,7 +376,10 @@ cudaError_t launch_cluster_sort(dqrm_ctx *ctx, csort::Args ca, int cap, cudaStre
 // 4.7 / 6.2, 1000 5.8 / 8.2 / 12.6, 2000 8.2 / - / 13.3, one table of 3000 11.5 / - / 11.1.  Unless the batch has an index a
 // bag, one table may hold most of it: a cluster of blocks then stands by for every table (a table of
 // 12.8 K lookups beside 25 of 128: 22.8 us, 99 by one block in global memory, 34.8 in a cluster of whole batches; bags of
-// five everywhere 9.9, 9.2 by the network without the clusters standing by).
+// five everywhere 9.9, 9.2 by the network without the clusters standing by).  Even batches (as many lookups as bags, which
+// need not be one in each) have them from 1024 lookups a table on, where there is room for the clusters: 26 tables of 2048 with 90 %
+// of the lookups in one 66 us, 390 without, and none the slower where they are not needed; pairs beyond 8192 in a table go through
+// global memory, since more shared memory would be held by every block.
 bool launch_small_sort(dqrm_ctx *ctx, const csort::Args &ca, int64_t per_table, bool even, cudaStream_t st, cudaError_t &e)
 {
     const int64_t want = even ? per_table : per_table + per_table / 4;
@@ -368,11 +387,10 @@ bool launch_small_sort(dqrm_ctx *ctx, const csort::Args &ca, int64_t per_table, 
     const dim3 grid((unsigned)ctx->T), block(csort::THREADS);
     constexpr size_t room = sizeof(uint2) * csort::SORT_ROOM;
     static_assert(csort::SORT_ROOM >= 4 * csort::THREADS, "");
-    if (!even) {
-        const int cap = csort::shared_cap(ca.L);
-        e = want <= 512    ? launch_cluster_sort<csort::CLUSTER, 1>(ctx, ca, cap, st)
-            : want <= 1024 ? launch_cluster_sort<csort::CLUSTER, 2>(ctx, ca, cap, st)
-                           : launch_cluster_sort<csort::CLUSTER, 4>(ctx, ca, cap, st);
+    if (!even || (want > 1024 && ctx->T * csort::CLUSTER <= 2 * ctx->num_sms)) {
+        e = want <= 512    ? launch_standby_sort<1>(ctx, ca, even, st)
+            : want <= 1024 ? launch_standby_sort<2>(ctx, ca, even, st)
+                           : launch_standby_sort<4>(ctx, ca, even, st);
     } else if (want <= 256) e = dq_launch(ssort::small_sort_kernel<256, 1>, grid, dim3(256), ssort::smem_bytes(256, 1), st, ca);
     else if (want <= 512) e = dq_launch(ssort::block_sort_kernel<1>, grid, block, room, st, ca);
     else if (want <= 1024) e = dq_launch(ssort::block_sort_kernel<2>, grid, block, room, st, ca);

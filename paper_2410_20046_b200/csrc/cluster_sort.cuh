@@ -37,18 +37,14 @@ __device__ __forceinline__ u32 same_digit_lanes(u32 d, bool valid)
     return valid ? peers : 0u;
 }
 
-// (two blocks resident for clusters of eight, so that the clusters of all tables run at once: without the bound the
-// kernel takes 95 registers and 26 tables of 16 K lookups 40 us instead of 32, with three 37.  Clusters of sixteen are
-// launched for a few tables only and have their SMs to themselves: 36.6 us without the bound, 42.2 with it, for one table
-// of 64 K lookups)
-//
-// EPT > 0: for small batches whose bags may be uneven.  A table of up to THREADS * EPT lookups, which is nearly all of them,
-// is sorted by the cluster's first block alone (sort_parts.cuh), and only a larger one by the cluster.
+// What every block of the cluster does.  EPT > 0: for small batches whose tables may be uneven.  A table of up to THREADS * EPT
+// lookups, which is nearly all of them, is sorted by one of the cluster's blocks alone (sort_parts.cuh), and only a larger one by
+// the cluster.  Which block that is goes round the tables: from the sixteenth on clusters share their SMs with earlier ones, and two
+// working blocks on one SM take half as long again (26 tables of 2000 lookups: 11.5 us with the first block working in every
+// cluster, 8.2 this way, 8.5 without clusters; from 33 tables on 11.5, a third cluster waiting for its SMs).
 template <int CL, int EPT>
-__global__ void __launch_bounds__(THREADS, CL > 8 ? 1 : 2)
-cluster_sort_kernel(const __grid_constant__ Args a)
+__device__ __forceinline__ void sort_by_cluster(const Args &a)
 {
-    dq_wait_before();
     extern __shared__ __align__(16) uint2 s_dyn[];               // pair buffers [2][cap]: (row within table, payload)
     __shared__ __align__(16) u32 s_cnt[WARPS][BINS];
     __shared__ u32 s_hist[BINS];
@@ -70,7 +66,7 @@ cluster_sort_kernel(const __grid_constant__ Args a)
     if (a.lists_by_table && c == 0 && threadIdx.x == 0) open_table(a, t, tb0, tb1);
     if constexpr (EPT > 0) {
         if (n <= THREADS * EPT) {
-            if (c == 0) sort_alone<EPT>(a, t, (u32)tb0, (u32)tb1, &s_cnt[0][0], s_dyn);
+            if (c == (unsigned)(t / 3) % CL) sort_alone<EPT>(a, t, (u32)tb0, (u32)tb1, &s_cnt[0][0], s_dyn);
             return;
         }
     }
@@ -347,6 +343,20 @@ cluster_sort_kernel(const __grid_constant__ Args a)
     // nobody leaves while its shared memory may still be read or written (with the lists, the last remote access came before
     // the barrier behind the totals)
     if (!a.lists_by_table) cluster.sync();
+}
+
+// Two blocks resident for clusters of eight, so that the clusters of all tables run at once: without the bound the
+// kernel takes 95 registers and 26 tables of 16 K lookups 40 us instead of 32, with three 37.  Clusters of sixteen are
+// launched for a few tables only and have their SMs to themselves: 36.6 us without the bound, 42.2 with it, for one table
+// of 64 K lookups
+__host__ __device__ constexpr int resident(int CL) { return CL == CLUSTER ? 2 : 1; }
+
+template <int CL, int EPT>
+__global__ void __launch_bounds__(THREADS, resident(CL))
+cluster_sort_kernel(const __grid_constant__ Args a)
+{
+    dq_wait_before();
+    sort_by_cluster<CL, EPT>(a);
 }
 
 inline size_t smem_bytes(int cap) { return (size_t)2 * cap * sizeof(uint2); }

@@ -7,10 +7,10 @@
 // 32 * EPT shuffles, wider ones go through shared memory (two buffers in turn, one barrier a step).  Row and position
 // make every key distinct, so the order is that of a stable sort.  Beyond that: the radix sort of sort_parts.cuh.
 //
-// A table with more lookups than the block holds
-// is sorted by its cluster where the batch may have one (cluster_sort_kernel with EPT > 0).  By the block in global memory,
-// with 8-bit digits, only where a batch with as many lookups as bags is uneven all the same, and in the one-launch step, which
-// takes no batch in which that is the longer way: 7 ns a lookup against 2 in a cluster (12.8 K lookups).
+// A table with more lookups than the block holds is sorted by its cluster where the batch has clusters standing by
+// (csort::sort_by_cluster with EPT > 0).  By the block in global memory, with 8-bit digits, at 7 ns a lookup against 2 in a cluster
+// (12.8 K lookups), only in the one-launch step, which takes no batch in which that is the longer way, and in batches with as many
+// lookups as bags that are uneven all the same, of up to 1024 lookups a table or of more tables than have room for clusters.
 // The lists that it leaves are those of the cluster sort's lists_by_table.
 //
 // Kernels take their arguments as grid constants: the functions that stay out of line get a pointer to them, and without that
@@ -320,10 +320,8 @@ small_sort_kernel(const __grid_constant__ csort::Args a)
 
 // The same for larger tables: up to THREADS * E lookups by the radix sort of sort_parts.cuh
 template <int E>
-__global__ void __launch_bounds__(csort::THREADS)
-block_sort_kernel(const __grid_constant__ csort::Args a)
+__device__ __forceinline__ void sort_by_block(const csort::Args &a)
 {
-    dq_wait_before();
     extern __shared__ __align__(16) uint2 s_pair[];              // [THREADS * E]
     __shared__ __align__(16) u32 s_cnt[csort::WARPS * csort::BINS];
     const int t = blockIdx.x;
@@ -339,6 +337,16 @@ block_sort_kernel(const __grid_constant__ csort::Args a)
         const uint2 *mem = sort_in_memory<csort::THREADS>(a, t, tb0, n, nrows, s_cnt);
         csort::write_part<1>(a, t, (u32)tb0, (u32)tb1, mem, (int)n, 0u, 0xffffffffu);
     }
+}
+
+// CL > 1: a cluster of blocks stands by for every table and sorts one that is larger
+template <int E, int CL = 1>
+__global__ void __launch_bounds__(csort::THREADS, csort::resident(CL))
+block_sort_kernel(const __grid_constant__ csort::Args a)
+{
+    dq_wait_before();
+    if constexpr (CL > 1) csort::sort_by_cluster<CL, E>(a);
+    else sort_by_block<E>(a);
 }
 
 }  // namespace ssort

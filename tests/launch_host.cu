@@ -69,6 +69,20 @@ int refused_sorts()
     return 0;
 }
 
+// a batch with as many lookups as bags may hold most of them in one table: beyond a thousand a table a cluster stands by for it,
+// while the clusters of all tables have room
+int clusters_stand_by()
+{
+    bool by_table = false;
+    for (const int T : {1, 2, 26, 37, 38, 100})
+        for (const int B : {300, 1024, 1025, 1500, 2048, 2049}) {
+            Ctx x(T, 16);
+            WANT(x.sort(B, (int64_t)T * B, &by_table) == DQRM_OK && by_table);
+            WANT((fake::cluster > 1) == (B > 2048 || (B > 1024 && T <= 37)));
+        }
+    return 0;
+}
+
 }  // namespace
 
 int main(int argc, char **argv)
@@ -76,6 +90,7 @@ int main(int argc, char **argv)
     const char *name = argc > 1 ? argv[1] : "";
     if (!strcmp(name, "contexts_in_turn")) return contexts_in_turn();
     if (!strcmp(name, "refused_sorts")) return refused_sorts();
+    if (!strcmp(name, "clusters_stand_by")) return clusters_stand_by();
     std::printf("no scenario %s\n", name);
     return 2;
 }

@@ -8,6 +8,7 @@ namespace fake {
 
 std::set<int> refuse;
 int launches = 0;
+unsigned cluster = 1;
 static cudaError_t pending = cudaSuccess;
 static std::map<const void *, size_t> smem_limit;
 
@@ -23,7 +24,13 @@ static cudaError_t launch(const void *f, size_t smem)
 
 extern "C" {
 
-cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t *c, const void *f, void **) { return fake::launch(f, c->dynamicSmemBytes); }
+cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t *c, const void *f, void **)
+{
+    fake::cluster = 1;
+    for (unsigned k = 0; k < c->numAttrs; ++k)
+        if (c->attrs[k].id == cudaLaunchAttributeClusterDimension) fake::cluster = c->attrs[k].val.clusterDim.x;
+    return fake::launch(f, c->dynamicSmemBytes);
+}
 cudaError_t cudaLaunchKernel(const void *f, dim3, dim3, void **, size_t smem, cudaStream_t) { return fake::launch(f, smem); }
 cudaError_t cudaFuncSetAttribute(const void *f, cudaFuncAttribute a, int v)
 {

@@ -95,3 +95,30 @@ def test_block_radix_sort(oracle, rows, n):
     # at most 800 terms of magnitude below 6 in FP64 in two orders, each sum rounded once
     np.testing.assert_allclose(gr, o_gr, rtol=2.0 ** -23, atol=12.0 * 800 ** 2 * 2.0 ** -53)
     c.ctx.close()
+
+
+@pytest.mark.parametrize("counts,B", [
+    ([6_000, 0, 0], 2_000), ([15_000, 17] + [400] * 7 + [2_183], 2_000), ([1] * 25 + [53_223], 2_048), ([2_049] + [1_050] * 35 + [1_901], 1_100),
+    ([80, 2_046], 1_063), ([70_000] + [100] * 35 + [2_276], 2_048),
+])
+@pytest.mark.parametrize("rows", [1, 70_000])
+def test_even_batches_that_are_uneven(oracle, rows, counts, B):
+    """As many lookups as bags, on average more than a thousand a table, but some or most of them in one."""
+    T, D = len(counts), 8
+    counts = counts[:-1] + [counts[-1] + T * B - sum(counts)]
+    wl = W.Workload("even", tuple(max(1, rows + t) for t in range(T)), D=D, B=B, alpha=None)
+    rng = np.random.default_rng(rows + B)
+    idx = np.concatenate([rng.integers(0, wl.rows[t], n) for t, n in enumerate(counts)]).astype(np.int32)
+    lens = np.zeros((T, B), dtype=np.int64)
+    for t, n in enumerate(counts):
+        np.add.at(lens[t], rng.integers(0, B, n), 1)
+    off = np.concatenate([[0], np.cumsum(lens.reshape(-1))]).astype(np.int32)
+    assert len(idx) == T * B
+    go = rng.standard_normal((B, T, D)).astype(np.float32)
+    c = Case(wl)
+    ur, uo, gr = c.gpu_bwd(idx, off, go)
+    o_ur, o_uo, o_gr = oracle.emb_bwd(go, T, D, B, idx, off)
+    assert bit_equal(uo, o_uo) and bit_equal(ur, o_ur)
+    # at most T * B terms of magnitude below 6 in FP64 in two orders, each sum rounded once
+    np.testing.assert_allclose(gr, o_gr, rtol=2.0 ** -23, atol=12.0 * max(counts) ** 2 * 2.0 ** -53)
+    c.ctx.close()
