@@ -243,7 +243,8 @@ __host__ __device__ constexpr int bags_blocks(int CH) { return CH == 2 ? 5 : CH 
 // in length wait for one another on the way (measured on
 // B200, random rows of 26 tables: 640 K rows of 64 bytes in bags of three on average 29 us this way, 42 by shuffle; of 256
 // bytes 67 and 88).
-template <int LPR, int CH, bool EXACT, bool CODES>
+// MIXED: the grid is (tables, blocks of a table), else (blocks of a table, tables)
+template <int LPR, int CH, bool EXACT, bool CODES, bool MIXED>
 __global__ void __launch_bounds__(FW_THREADS, bags_blocks(CH))
 fwd_bags_kernel(const FwdArgs a)
 {
@@ -252,13 +253,13 @@ fwd_bags_kernel(const FwdArgs a)
     constexpr int GPB = FW_THREADS / LPR;
     const int D = EXACT ? 4 * LPR * CH : a.D;
     const int d4 = D >> 2;
-    const int t = blockIdx.x;
+    const int t = MIXED ? blockIdx.x : blockIdx.y;
     const int lane = threadIdx.x % LPR;
     const int grp = threadIdx.x / LPR;
     const TableCtx tc = table_ctx(a, t, D);
     bool bad = false;
 
-    for (int i = blockIdx.y * GPB + grp; i < a.B; i += gridDim.y * GPB) {
+    for (int i = (MIXED ? blockIdx.y : blockIdx.x) * GPB + grp; i < a.B; i += (MIXED ? gridDim.y : gridDim.x) * GPB) {
         int32_t lo = __ldg(a.offsets + tc.g0 + i), hi = __ldg(a.offsets + tc.g0 + i + 1);
         if (lo < 0 || hi < lo || (int64_t)hi > a.L) { bad = true; hi = lo = 0; }
         double acc[CH][4];
@@ -363,12 +364,31 @@ constexpr int LONG_BAG = 18;
 inline bool long_bags(const int8_t *codes_out, int T, int B, int64_t L) { return !codes_out && L >= LONG_BAG * (int64_t)T * B; }
 inline bool warp_per_bag(const FwdArgs &a, int lpr) { return lpr == 16 && long_bags(a.codes_out, a.T, a.B, a.L); }
 
+constexpr int MIXED_TABLES = 8;
+// Order of the blocks.  All tables' blocks for the same bags side by side: the pooled rows of a bag lie next to one another in the
+// output, and DRAM takes them better together (one index a bag, 852 K rows of 256 bytes 49.0 -> 46.9 us, 426 K of 64 bytes 9.1 -> 8.9).
+// Table by table: the rows that a bag shares with others are found again in L2, or a warp's in L1.  Which of the two counts for
+// more goes by the width of the rows and the length of the bags.  Measured on B200 for pooled bags, 26 tables of 8192 bags, side by
+// side / table by table (uniform indices over 30 K to 1.5 M rows a table, and Zipf 1.2): 4 to 16 features 0.97 to 1.02 for bags of
+// two, 1.0 to 1.14 for twelve, 1.0 to 1.51 for thirty; 32 features 0.96 to 0.98 up to eight indices a bag, 0.96 to 1.00 for twelve, 1.03
+// for 17 where every row comes several times; 64 features 0.94 to 0.98 for two to four, 0.97 to 1.02 for six, 1.08 for twelve; 128
+// features 0.94 to 0.97 for two, 0.98 to 1.03 for four, up to 1.08 for six; 256 features 0.99 and 1.07 for two, 1.18 for twelve.  Five
+// tables: 0.99 to 1.02.  Long bags, a warp each: 8.5 M rows of 256 bytes 324 us side by side, 314 table by table
+__host__ __device__ constexpr int mixed_upto(int LPR, int CH) { return CH > 1 ? 0 : LPR == 8 ? 16 : LPR == 16 ? 5 : LPR == 32 ? 3 : 0; }
+template <int LPR, int CH>
+inline bool bags_mixed(const FwdArgs &a) { return a.T >= MIXED_TABLES && a.L < mixed_upto(LPR, CH) * (int64_t)a.T * a.B; }
+
 template <int LPR, int CH, bool EXACT>
 cudaError_t launch_bags(const FwdArgs &a, dim3 grid, cudaStream_t st)
 {
     if (LPR == 16 && warp_per_bag(a, LPR)) return dq_launch(fwd_long_bags_kernel<EXACT>, grid, dim3(FW_THREADS), 0, st, a);
-    if (a.codes_out) return dq_launch(fwd_bags_kernel<LPR, CH, EXACT, true>, grid, dim3(FW_THREADS), 0, st, a);
-    return dq_launch(fwd_bags_kernel<LPR, CH, EXACT, false>, grid, dim3(FW_THREADS), 0, st, a);
+    constexpr bool MAY = mixed_upto(LPR, CH) > 0;
+    if (MAY && bags_mixed<LPR, CH>(a)) {
+        if (a.codes_out) return dq_launch(fwd_bags_kernel<LPR, CH, EXACT, true, MAY>, grid, dim3(FW_THREADS), 0, st, a);
+        return dq_launch(fwd_bags_kernel<LPR, CH, EXACT, false, MAY>, grid, dim3(FW_THREADS), 0, st, a);
+    }
+    if (a.codes_out) return dq_launch(fwd_bags_kernel<LPR, CH, EXACT, true, false>, grid, dim3(FW_THREADS), 0, st, a);
+    return dq_launch(fwd_bags_kernel<LPR, CH, EXACT, false, false>, grid, dim3(FW_THREADS), 0, st, a);
 }
 
 template <int LPR, int CH, bool EXACT>
@@ -382,11 +402,8 @@ int launch2(dqrm_ctx *ctx, const FwdArgs &a, cudaStream_t st)
     const int cap = (ctx->num_sms * 32 + ctx->T - 1) / ctx->T;     // a few waves over all tables
     if (bx > cap) bx = cap;
     if (bx < 1) bx = 1;
-    // Blocks of all tables for the same bags side by side: the pooled rows of a bag lie next to one another in the output, and
-    // DRAM takes them better together (852 K rows of 256 bytes 49.0 -> 46.9 us, 426 K of 64 bytes 9.1 -> 8.9).  Not where a warp
-    // takes a long bag: there a table's hot rows are found again in L1 (8.5 M rows 314 us table by table, 324 mixed)
-    const bool by_table = !onehot && LPR == 16 && warp_per_bag(a, LPR);
-    const dim3 grid((unsigned)(by_table ? bx : ctx->T), (unsigned)(by_table ? ctx->T : bx));
+    const bool mixed = onehot || bags_mixed<LPR, CH>(a);
+    const dim3 grid((unsigned)(mixed ? ctx->T : bx), (unsigned)(mixed ? bx : ctx->T));
     DQRM_CUDA_TRY(ctx, (onehot ? dq_launch(fwd_onehot_kernel<LPR, CH, EXACT>, grid, dim3(FW_THREADS), 0, st, a)
                                : launch_bags<LPR, CH, EXACT>(a, grid, st)));
     dq_mark(ctx, st, DQ_K_FWD);

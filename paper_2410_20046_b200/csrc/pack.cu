@@ -124,6 +124,7 @@ struct PfArgs {
     int T, D, B;
     int64_t L;
     int *status;
+    int mixed;                   // grid (tables, blocks of a table), else (blocks of a table, tables)
 };
 
 // pools one bag in bag order in FP64 and rounds once (any bag length, zero included)
@@ -191,14 +192,14 @@ packed_fwd_kernel(const PfArgs a)
     dq_wait_before();
     constexpr int GPB = PK_THREADS / LPR;
     const int units = a.D / EPL;
-    const int t = blockIdx.x;
+    const int t = a.mixed ? blockIdx.x : blockIdx.y, block = a.mixed ? blockIdx.y : blockIdx.x, blocks = a.mixed ? gridDim.y : gridDim.x;
     const int lane = threadIdx.x % LPR, grp = threadIdx.x / LPR;
     const float s = __ldg(a.scales + t);
     const int64_t r0 = __ldg(a.row_off + t);
     const int32_t nrows = (int32_t)(__ldg(a.row_off + t + 1) - r0);
     const int64_t g0 = (int64_t)t * a.B;
     bool bad = false;
-    for (int i = blockIdx.y * GPB + grp; i < a.B; i += gridDim.y * GPB)
+    for (int i = block * GPB + grp; i < a.B; i += blocks * GPB)
         pool_bag<BITS, EPL, LPR, CH>(a, r0, nrows, s, units, __ldg(a.offsets + g0 + i), __ldg(a.offsets + g0 + i + 1),
                                      a.out + ((int64_t)i * a.T + t) * a.D, lane, bad);
     if (bad) dq_report(a.status, DQRM_ERR_INDEX_RANGE);
@@ -329,7 +330,7 @@ int launch_pack(dqrm_ctx *ctx, const float *tables, const float *scales, uint8_t
 }
 
 template <int BITS, int EPL, int LPR, int CH>
-int launch_pfwd(dqrm_ctx *ctx, const PfArgs &a, cudaStream_t st)
+int launch_pfwd(dqrm_ctx *ctx, PfArgs a, cudaStream_t st)
 {
     constexpr int GPB = PK_THREADS / LPR;
     const bool onehot = a.L == (int64_t)a.T * a.B;
@@ -338,8 +339,11 @@ int launch_pfwd(dqrm_ctx *ctx, const PfArgs &a, cudaStream_t st)
     const int cap = (ctx->num_sms * 32 + ctx->T - 1) / ctx->T;
     if (bx > cap) bx = cap;
     if (bx < 1) bx = 1;
-    // (all tables' blocks for the same bags side by side: see the forward; 852 K rows of 64 features 42.5 -> 40.6 us)
-    const dim3 grid((unsigned)ctx->T, (unsigned)bx);
+    // Order of the blocks (see the forward).  One index a bag: side by side (852 K rows of 64 features 42.5 -> 40.6 us).  Bags, 26 tables of
+    // 8192, side by side / table by table, bags of two to thirty: 4 to 32 features 0.97 to 1.25 (uniform indices over 1.5 M rows of
+    // 16 features, thirty a bag), 48 and 64 features 0.94 to 0.99, 128 0.95 to 0.99, 256 0.96 and 0.98; five tables 0.99 to 1.03
+    a.mixed = onehot || (a.D > 32 && a.T >= 8);
+    const dim3 grid((unsigned)(a.mixed ? ctx->T : bx), (unsigned)(a.mixed ? bx : ctx->T));
     DQRM_CUDA_TRY(ctx, (onehot ? dq_launch(packed_fwd_onehot_kernel<BITS, EPL, LPR, CH>, grid, dim3(PK_THREADS), 0, st, a)
                                : dq_launch(packed_fwd_kernel<BITS, EPL, LPR, CH>, grid, dim3(PK_THREADS), 0, st, a)));
     dq_mark(ctx, st, DQ_K_PACKED_FWD);
@@ -389,7 +393,7 @@ size_t dq_packed_align(const dqrm_ctx *ctx, int bits, int B, int64_t L)
 int dq_launch_packed_fwd(dqrm_ctx *ctx, const uint8_t *packed, const int32_t *indices, const int32_t *offsets,
                          const float *scales, int bits, float *out, int B, int64_t L, cudaStream_t st)
 {
-    const PfArgs a{packed, ctx->d_row_off, indices, offsets, scales, out, ctx->T, ctx->D, B, L, ctx->d_status};
+    const PfArgs a{packed, ctx->d_row_off, indices, offsets, scales, out, ctx->T, ctx->D, B, L, ctx->d_status, 1};
     if (bits == 2) return dispatch_pfwd<2>(ctx, a, st);
     if (bits == 4) return dispatch_pfwd<4>(ctx, a, st);
     return dispatch_pfwd<8>(ctx, a, st);

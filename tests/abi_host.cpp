@@ -1,5 +1,5 @@
-// The C ABI over a stand-in for the CUDA runtime that counts launches: which pointers a call takes, by their alignment.  Nothing
-// runs on a device and no pointer is followed.  One scenario per run, named by argv[1]; 0 when what it asserts holds.
+// The C ABI over a stand-in for the CUDA runtime that counts launches: which pointers a call takes, by their alignment, and what its
+// grids are.  Nothing runs on a device and no pointer is followed.  One scenario per run, named by argv[1]; 0 when what it asserts holds.
 #include <cstdint>
 #include <cstdio>
 #include <cstring>
@@ -19,10 +19,11 @@ uint8_t *u8(int by) { return at<uint8_t *>(by); }
 
 struct Ctx {
     dqrm_ctx *h = nullptr;
-    explicit Ctx(int D)
+    explicit Ctx(int D, int tables = T)
     {
-        const int64_t off[T + 1] = {0, 100, 200, 300, 400};
-        if (dqrm_create(&h, T, D, off) != DQRM_OK) h = nullptr;
+        int64_t off[16];
+        for (int t = 0; t <= tables; ++t) off[t] = 100 * t;
+        if (dqrm_create(&h, tables, D, off) != DQRM_OK) h = nullptr;
     }
     ~Ctx() { dqrm_destroy(h); }
 };
@@ -155,6 +156,27 @@ int empty()
     return failed;
 }
 
+// the blocks of short bags of wide rows stand side by side for all tables, those of long bags and narrow rows table by table
+int order()
+{
+    const int B = 3000;
+    for (const int T : {7, 8}) {
+        for (const int D : {4, 8, 16, 20, 32, 36, 48, 64, 68, 128, 132, 256, 1024}) {
+            Ctx x(D, T);
+            const int upto = T < 8 || D <= 16 ? 0 : D <= 32 ? 16 : D <= 64 ? 5 : D <= 128 ? 3 : 0;
+            for (const int bag : {1, 2, 3, 4, 5, 12, 16, 30}) {
+                const int64_t L = (int64_t)T * B * bag;
+                auto mixed = [=] { return fake::grid_x == (unsigned)T && fake::grid_y > (unsigned)T; };
+                if (dqrm_emb_fwd(x.h, f(0), i32(), i32(), f(0), i32(), f(0), nullptr, B, L, nullptr) != DQRM_OK || mixed() != (bag == 1 || bag < upto))
+                    failed = 1, std::printf("forward, D = %d, bags of %d: grid %u, %u\n", D, bag, fake::grid_x, fake::grid_y);
+                if (dqrm_packed_fwd(x.h, u8(0), i32(), i32(), f(0), 4, f(0), B, L, nullptr) != DQRM_OK || mixed() != (bag == 1 || (D > 32 && T >= 8)))
+                    failed = 1, std::printf("packed lookup, D = %d, bags of %d: grid %u, %u\n", D, bag, fake::grid_x, fake::grid_y);
+            }
+        }
+    }
+    return failed;
+}
+
 }  // namespace
 
 int main(int argc, char **argv)
@@ -164,6 +186,7 @@ int main(int argc, char **argv)
     if (!strcmp(name, "forward")) return forward();
     if (!strcmp(name, "rows")) return rows();
     if (!strcmp(name, "empty")) return empty();
+    if (!strcmp(name, "order")) return order();
     std::printf("no scenario %s\n", name);
     return 2;
 }

@@ -8,7 +8,7 @@ namespace fake {
 
 std::set<int> refuse;
 int launches = 0;
-unsigned cluster = 1;
+unsigned cluster = 1, grid_x = 0, grid_y = 0;
 static cudaError_t pending = cudaSuccess;
 static std::map<const void *, size_t> smem_limit;
 
@@ -27,6 +27,8 @@ extern "C" {
 cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t *c, const void *f, void **)
 {
     fake::cluster = 1;
+    fake::grid_x = c->gridDim.x;
+    fake::grid_y = c->gridDim.y;
     for (unsigned k = 0; k < c->numAttrs; ++k)
         if (c->attrs[k].id == cudaLaunchAttributeClusterDimension) fake::cluster = c->attrs[k].val.clusterDim.x;
     return fake::launch(f, c->dynamicSmemBytes);

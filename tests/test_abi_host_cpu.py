@@ -1,5 +1,6 @@
-"""Pointers that a call's kernels cannot use are refused on the host, before anything is launched, and all others are taken:
-abi_host.cpp calls the library over a stand-in for the CUDA runtime."""
+"""abi_host.cpp calls the library over a stand-in for the CUDA runtime: pointers that a call's kernels cannot use are refused on
+the host, before anything is launched, and all others are taken; pooled lookups have their blocks in the order that suits their
+bags."""
 import glob
 import os
 import shutil
@@ -23,7 +24,7 @@ def program(tmp_path_factory):
     return out
 
 
-@pytest.mark.parametrize("scenario", ["sum", "forward", "rows", "empty"])
-def test_alignment(program, scenario):
+@pytest.mark.parametrize("scenario", ["sum", "forward", "rows", "empty", "order"])
+def test_calls(program, scenario):
     r = subprocess.run([program, scenario], capture_output=True, text=True, timeout=60)
     assert r.returncode == 0, r.stdout + r.stderr
