@@ -136,7 +136,7 @@ def base_config(wl):
 # profiles/ (set an entry to None when its kernel has changed since the capture)
 NCU_TRAFFIC = {
     ("kaggle_b16384", "fwd_kernel"): None,
-    ("kaggle_b16384", "seg_sum_kernel"): None,
+    ("kaggle_b16384", "seg_groups_kernel"): None,
     ("kaggle_b16384", "row_stream_kernel<fused>"): 25.21e6,
     # the Terabyte-shaped step captured over 2 GB of tables (the full tables are too large for a counter capture)
     ("terabyte_2gb_b32768", "fwd_kernel"): None,
@@ -147,6 +147,7 @@ NCU_TRAFFIC = {
 KERNEL_BYTES = {
     "fwd_kernel": lambda ab, wl, L, G, U: ab["fwd"],
     "seg_sum_kernel": lambda ab, wl, L, G, U: 4 * wl.D * G + 4 * wl.D * U,
+    "seg_groups_kernel": lambda ab, wl, L, G, U: 4 * wl.D * G + 4 * wl.D * U,
     "row_stream_kernel<fused>": lambda ab, wl, L, G, U: ab["quant_update"],
     "refresh_kernel": lambda ab, wl, L, G, U: ab["refresh"],
 }

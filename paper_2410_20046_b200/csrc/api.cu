@@ -283,7 +283,7 @@ const char *dqrm_kernel_name(int kernel_id)
         "rs_scatter_kernel", "seg_count_kernel", "seg_emit_kernel", "seg_sum_kernel",
         "zero_kernel", "absmax_kernel", "row_stream_kernel<quant>", "row_stream_kernel<update>", "row_stream_kernel<fused>",
         "copy", "small_sort_kernel", "small_step_kernel", "cluster_sort_kernel", "dp_pack_kernel", "dp_sum_update_kernel", "pack_kernel", "packed_fwd_kernel", "fwd_codes_kernel", "decode_payload_kernel",
-        "quant_table_kernel", "quant_heavy_kernel"};
+        "quant_table_kernel", "quant_heavy_kernel", "seg_groups_kernel"};
     return (kernel_id >= 0 && kernel_id < DQ_K_COUNT) ? names[kernel_id] : "?";
 }
 

@@ -276,7 +276,7 @@ int launch_sum_groups(dqrm_ctx *ctx, const segred::Args &a, cudaStream_t st)
         DQRM_CUDA_TRY(ctx, (dq_launch(seg_groups_kernel<LPR, false, unaligned_vec(LPR)>, grid, block, smem_bytes(ctx->T), st, a)));
     else if (ctx->D == LPR * 4) DQRM_CUDA_TRY(ctx, (dq_launch(seg_groups_kernel<LPR, true>, grid, block, smem_bytes(ctx->T), st, a)));
     else DQRM_CUDA_TRY(ctx, (dq_launch(seg_groups_kernel<LPR, false>, grid, block, smem_bytes(ctx->T), st, a)));
-    dq_mark(ctx, st, DQ_K_SEG_SUM);
+    dq_mark(ctx, st, DQ_K_SEG_GROUPS);
     return DQRM_OK;
 }
 
@@ -366,7 +366,7 @@ cudaError_t launch_standby_sort(dqrm_ctx *ctx, csort::Args ca, bool even, cudaSt
     ca.cap = even ? csort::SORT_ROOM / 2 : csort::shared_cap(ca.L);
     const size_t smem = std::max(csort::smem_bytes(ca.cap), sizeof(uint2) * csort::SORT_ROOM);
     if constexpr (EPT == 4)
-        if (even) return launch_clusters<CL>(ctx, ssort::block_sort_kernel<EPT, CL>, 5, ca, smem, st);
+        if (even) return launch_clusters<CL>(ctx, ssort::small_sort_kernel<csort::THREADS, EPT, CL>, 5, ca, smem, st);
     return launch_clusters<CL>(ctx, csort::cluster_sort_kernel<CL, EPT>, EPT, ca, smem, st);
 }
 
@@ -391,10 +391,10 @@ bool launch_small_sort(dqrm_ctx *ctx, const csort::Args &ca, int64_t per_table, 
         e = want <= 512    ? launch_standby_sort<1>(ctx, ca, even, st)
             : want <= 1024 ? launch_standby_sort<2>(ctx, ca, even, st)
                            : launch_standby_sort<4>(ctx, ca, even, st);
-    } else if (want <= 256) e = dq_launch(ssort::small_sort_kernel<256, 1>, grid, dim3(256), ssort::smem_bytes(256, 1), st, ca);
-    else if (want <= 512) e = dq_launch(ssort::block_sort_kernel<1>, grid, block, room, st, ca);
-    else if (want <= 1024) e = dq_launch(ssort::block_sort_kernel<2>, grid, block, room, st, ca);
-    else e = dq_launch(ssort::block_sort_kernel<4>, grid, block, room, st, ca);
+    } else if (want <= 256) e = dq_launch(ssort::small_sort_kernel<256, 1, 1>, grid, dim3(256), ssort::smem_bytes(256, 1), st, ca);
+    else if (want <= 512) e = dq_launch(ssort::small_sort_kernel<csort::THREADS, 1, 1>, grid, block, room, st, ca);
+    else if (want <= 1024) e = dq_launch(ssort::small_sort_kernel<csort::THREADS, 2, 1>, grid, block, room, st, ca);
+    else e = dq_launch(ssort::small_sort_kernel<csort::THREADS, 4, 1>, grid, block, room, st, ca);
     return true;
 }
 

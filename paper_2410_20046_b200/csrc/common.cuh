@@ -73,7 +73,7 @@ enum {
     DQ_K_BEGIN = 0, DQ_K_REFRESH, DQ_K_FWD, DQ_K_MEMSET, DQ_K_SORT_SETUP, DQ_K_SORT_HIST, DQ_K_SORT_SCAN, DQ_K_SORT_SCATTER,
     DQ_K_SEG_COUNT, DQ_K_SEG_EMIT, DQ_K_SEG_SUM, DQ_K_ZERO, DQ_K_ABSMAX, DQ_K_QUANT, DQ_K_UPDATE,
     DQ_K_QUANT_UPDATE, DQ_K_COPY, DQ_K_SMALL_SORT, DQ_K_SMALL_STEP, DQ_K_CLUSTER_SORT, DQ_K_DP_PACK, DQ_K_DP_SUM_UPDATE, DQ_K_PACK, DQ_K_PACKED_FWD, DQ_K_FWD_CODES, DQ_K_DECODE_PAYLOAD,
-    DQ_K_QUANT_TABLE, DQ_K_QUANT_HEAVY, DQ_K_COUNT
+    DQ_K_QUANT_TABLE, DQ_K_QUANT_HEAVY, DQ_K_SEG_GROUPS, DQ_K_COUNT
 };
 constexpr int DQ_PROF_MAX = 4096;
 

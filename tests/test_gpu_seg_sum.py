@@ -138,3 +138,15 @@ def test_radix_sort_digits(oracle, rows):
     # at most 25,000 terms of magnitude below 6 in FP64 in two orders, each sum rounded once
     np.testing.assert_allclose(gr, o_gr, rtol=2.0 ** -23, atol=12.0 * 25_000 ** 2 * 2.0 ** -53)
     c.ctx.close()
+
+
+@pytest.mark.parametrize("D,kernel", [(4, "seg_groups_kernel"), (16, "seg_groups_kernel"), (48, "seg_groups_kernel"), (52, "seg_sum_kernel"), (128, "seg_sum_kernel")])
+def test_profile_names_the_kernel(D, kernel):
+    """The profile says which of the two summing kernels ran."""
+    B = 60
+    wl = W.Workload("names", (50,), D=D, B=B, alpha=None)
+    c = Case(wl)
+    c.ctx.profile_begin()
+    c.gpu_bwd(np.arange(B, dtype=np.int32) % 50, np.arange(B + 1, dtype=np.int32), np.ones((B, 1, D), dtype=np.float32))
+    assert set(c.ctx.profile_end()) & {"seg_groups_kernel", "seg_sum_kernel"} == {kernel}
+    c.ctx.close()
