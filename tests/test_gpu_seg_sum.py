@@ -140,6 +140,34 @@ def test_radix_sort_digits(oracle, rows):
     c.ctx.close()
 
 
+# On 148 SMs a lane group's range is one round of eight entries up to 47 K lookups of 36 to 48 features, 95 K of 20 to 32, 189 K of
+# 12 and 16, 379 K of 8 and 758 K of 4: these take more rounds
+@pytest.mark.parametrize("D,B", [(36, 7_001), (48, 12_003), (44, 40_001), (20, 14_002), (32, 27_001), (24, 60_005), (12, 30_003), (16, 50_001), (8, 60_001), (4, 120_003)])
+@pytest.mark.parametrize("sort_path", [0, 1])
+def test_lane_groups_of_many_rounds(oracle, D, B, sort_path):
+    rng = np.random.default_rng(D)
+    rows = (40_000, 3, 900_000, 1)
+    T = len(rows)
+    wl = W.Workload("rounds", rows, D=D, B=B, alpha=None)
+    lens = rng.integers(0, 6, T * B)
+    lens[:B // 3] = 0                               # a table of fewer lookups
+    off = np.concatenate([[0], np.cumsum(lens)]).astype(np.int32)
+    L = int(off[-1])
+    table = np.repeat(np.arange(T), lens.reshape(T, B).sum(1))
+    idx = (rng.random(L) ** rng.choice([1, 8], L) * np.array(rows)[table]).astype(np.int32)      # runs of one to thousands
+    assert L > 8 * 2960 * (32 // (1 if D <= 4 else 2 if D <= 8 else 4 if D <= 16 else 8 if D <= 32 else 16))
+    go = rng.standard_normal((B, T, D), dtype=np.float32)
+    c = Case(wl, max_lookups=L)
+    c.ctx.set_sort_path(sort_path)
+    ur, uo, gr = c.gpu_bwd(idx, off, go)
+    o_ur, o_uo, o_gr = oracle.emb_bwd(go, T, D, B, idx, off)
+    assert bit_equal(uo, o_uo) and bit_equal(ur, o_ur)
+    # n terms of magnitude below 6 in FP64 in two orders, each sum rounded once
+    n = int(np.bincount(idx + 1_000_000 * table).max())
+    np.testing.assert_allclose(gr, o_gr, rtol=2.0 ** -23, atol=12.0 * n * n * 2.0 ** -53)
+    c.ctx.close()
+
+
 @pytest.mark.parametrize("D,kernel", [(4, "seg_groups_kernel"), (16, "seg_groups_kernel"), (48, "seg_groups_kernel"), (52, "seg_sum_kernel"), (128, "seg_sum_kernel")])
 def test_profile_names_the_kernel(D, kernel):
     """The profile says which of the two summing kernels ran."""

@@ -50,3 +50,11 @@ def test_streams_do_not_matter(T, B, bag, D):
     for a, b in zip(*seen):
         assert bit_equal(a, b)
     c.ctx.close()
+
+
+@pytest.mark.parametrize("T,B,D", [
+    (2, 8_191, 16), (2, 8_192, 16), (2, 3_640, 36), (2, 3_641, 36),                  # 1 MB
+    (4, 262_143, 16), (4, 262_144, 16), (2, 233_016, 36), (2, 233_017, 36),          # 64 MB
+])
+def test_streams_do_not_matter_to_lane_groups(T, B, D):
+    test_streams_do_not_matter(T, B, 1, D)
