@@ -274,7 +274,8 @@ int launch_sum_groups(dqrm_ctx *ctx, const segred::Args &a, cudaStream_t st)
     const dim3 grid((a.ranges + warps - 1) / warps), block(warps * 32);
     if (!dq_aligned(a.grad_out, sizeof(float4)) || !dq_aligned(a.grad_rows, sizeof(float4)))
         DQRM_CUDA_TRY(ctx, (dq_launch(seg_groups_kernel<LPR, false, unaligned_vec(LPR)>, grid, block, smem_bytes(ctx->T), st, a)));
-    else if (ctx->D == LPR * 4) DQRM_CUDA_TRY(ctx, (dq_launch(seg_groups_kernel<LPR, true>, grid, block, smem_bytes(ctx->T), st, a)));
+    else if (takes_groups(LPR * 4) && ctx->D == LPR * 4)
+        DQRM_CUDA_TRY(ctx, (dq_launch(seg_groups_kernel<LPR, takes_groups(LPR * 4)>, grid, block, smem_bytes(ctx->T), st, a)));
     else DQRM_CUDA_TRY(ctx, (dq_launch(seg_groups_kernel<LPR, false>, grid, block, smem_bytes(ctx->T), st, a)));
     dq_mark(ctx, st, DQ_K_SEG_GROUPS);
     return DQRM_OK;
@@ -391,7 +392,7 @@ bool launch_small_sort(dqrm_ctx *ctx, const csort::Args &ca, int64_t per_table, 
         e = want <= 512    ? launch_standby_sort<1>(ctx, ca, even, st)
             : want <= 1024 ? launch_standby_sort<2>(ctx, ca, even, st)
                            : launch_standby_sort<4>(ctx, ca, even, st);
-    } else if (want <= 256) e = dq_launch(ssort::small_sort_kernel<256, 1, 1>, grid, dim3(256), ssort::smem_bytes(256, 1), st, ca);
+    } else if (want <= 256) e = dq_launch(ssort::small_sort_kernel<256, 1, 1>, grid, dim3(256), ssort::smem_bytes(256), st, ca);
     else if (want <= 512) e = dq_launch(ssort::small_sort_kernel<csort::THREADS, 1, 1>, grid, block, room, st, ca);
     else if (want <= 1024) e = dq_launch(ssort::small_sort_kernel<csort::THREADS, 2, 1>, grid, block, room, st, ca);
     else e = dq_launch(ssort::small_sort_kernel<csort::THREADS, 4, 1>, grid, block, room, st, ca);

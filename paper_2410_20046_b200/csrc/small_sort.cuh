@@ -3,8 +3,8 @@
 //
 // Up to 256 lookups: a bitonic network over (row, position) held in registers: log2(n) (log2(n) + 1) / 2 steps whatever the row
 // count; most of them stay inside a warp, and unrolled they cost about 0.15 us each (with the steps in a loop, 1.5 times
-// that).  Every thread holds EPT consecutive entries: steps across less than EPT entries are register moves, across less than
-// 32 * EPT shuffles, wider ones go through shared memory (two buffers in turn, one barrier a step).  Row and position
+// that).  Every thread holds one entry: steps across less than 32 entries are shuffles, wider ones go through shared memory (two
+// buffers in turn, one barrier a step).  Row and position
 // make every key distinct, so the order is that of a stable sort.  Beyond that: the radix sort of sort_parts.cuh.
 //
 // A table with more lookups than the block holds is sorted by its cluster where the batch has clusters standing by
@@ -22,9 +22,9 @@ namespace ssort {
 
 typedef unsigned long long u64;
 
-inline size_t smem_bytes(int threads, int ept)
+inline size_t smem_bytes(int threads)
 {
-    const size_t net = (size_t)threads * ept * 2 * sizeof(u64);
+    const size_t net = (size_t)threads * 2 * sizeof(u64);
     const size_t digits = (size_t)(threads / 32) * csort::BINS * sizeof(u32);
     return net > digits ? net : digits;
 }
@@ -122,90 +122,50 @@ __device__ __noinline__ const uint2 *sort_in_memory(const csort::Args &a, int t,
     return a.gp[s] + tb0;
 }
 
-// The block's table (n <= THREADS * EPT lookups) into s_net[0 .. n): row << 32 | payload; s_net has 2 * THREADS * EPT places
-template <int THREADS, int EPT>
+// The block's table (n <= THREADS lookups) into s_net[0 .. n): row << 32 | payload; s_net has 2 * THREADS places
+template <int THREADS>
 __device__ __forceinline__ void sort_in_block(const csort::Args &a, int t, int64_t tb0, int64_t n, int64_t nrows, u64 *s_net, bool &bad)
 {
-    constexpr int N = THREADS * EPT;
     const int tid = threadIdx.x;
-    u64 e[EPT];                                    // row << 32 | position, later row << 32 | payload
-    u32 pay[EPT];
-#pragma unroll
-    for (int k = 0; k < EPT; ++k) {            // (loads coalesced: thread tid takes entries tid, tid + THREADS, ...)
-        const int p = k * THREADS + tid;
-        e[k] = ~0ull;
-        pay[k] = 0u;
-        if (p < n) {
-            const uint2 pr = lookup(a, t, tb0, n, nrows, p, bad);
-            e[k] = (u64)pr.x << 32 | (u32)p;
-            pay[k] = pr.y;
-        }
+    u64 e = ~0ull;                                 // row << 32 | position, later row << 32 | payload
+    u32 pay = 0u;
+    if (tid < n) {
+        const uint2 pr = lookup(a, t, tb0, n, nrows, tid, bad);
+        e = (u64)pr.x << 32 | (u32)tid;
+        pay = pr.y;
     }
-    int top = 1;                               // entries that the network covers: a power of two from 32 * EPT on
+    int top = 1;                               // entries that the network covers: a power of two from 32 on
     while ((1 << top) < n) ++top;
-    const bool live = (tid & ~31) * EPT < (1 << top);       // (warps of places beyond only keep the barriers)
+    const bool live = (tid & ~31) < (1 << top);       // (warps of places beyond only keep the barriers)
     u64 *buf = s_net;
-    if (EPT > 1) {                             // to EPT consecutive entries per thread
-#pragma unroll
-        for (int k = 0; k < EPT; ++k) buf[k * THREADS + tid] = e[k];
-        __syncthreads();
-#pragma unroll
-        for (int k = 0; k < EPT; ++k) e[k] = buf[tid * EPT + k];
-        buf = s_net + N;
-    }
-    const int i0 = tid * EPT;                  // first entry of this thread
-    constexpr int TOP = log2c(N);
+    constexpr int TOP = log2c(THREADS);
 #pragma unroll
     for (int p = 1; p <= TOP; ++p) {
         if (p > top) break;                    // (block-uniform)
 #pragma unroll
         for (int s = p - 1; s >= 0; --s) {
             const int stride = 1 << s;
-            if (stride >= 32 * EPT) {
-#pragma unroll
-                for (int k = 0; k < EPT; ++k) buf[i0 + k] = e[k];
+            const bool up = ((tid >> p) & 1) == 0, low = (tid & stride) == 0;
+            if (stride >= 32) {
+                buf[tid] = e;
                 __syncthreads();
-                const bool up = ((i0 >> p) & 1) == 0, low = (i0 & stride) == 0;
-#pragma unroll
-                for (int k = 0; k < EPT; ++k) {
-                    const u64 o = buf[(i0 + k) ^ stride];
-                    e[k] = (up == low) == (e[k] < o) ? e[k] : o;
-                }
-                buf = buf == s_net ? s_net + N : s_net;
-            } else if (stride >= EPT) {
-                const bool up = ((i0 >> p) & 1) == 0, low = (i0 & stride) == 0;
-#pragma unroll
-                for (int k = 0; live && k < EPT; ++k) {
-                    const u64 o = shfl_xor64(e[k], stride / EPT);
-                    e[k] = (up == low) == (e[k] < o) ? e[k] : o;
-                }
-            } else {
-#pragma unroll
-                for (int k = 0; k < EPT; ++k) {
-                    if ((k & stride) == 0) {
-                        const bool up = (((i0 + k) >> p) & 1) == 0;
-                        const u64 x = e[k], y = e[(k + stride) % EPT];
-                        const bool swap = up ? y < x : x < y;
-                        e[k] = swap ? y : x;
-                        e[(k + stride) % EPT] = swap ? x : y;
-                    }
-                }
+                const u64 o = buf[tid ^ stride];
+                e = (up == low) == (e < o) ? e : o;
+                buf = buf == s_net ? s_net + THREADS : s_net;
+            } else if (live) {
+                const u64 o = shfl_xor64(e, stride);
+                e = (up == low) == (e < o) ? e : o;
             }
         }
     }
     // the payloads come back by position
     __syncthreads();
     u32 *s_pay = reinterpret_cast<u32 *>(s_net);
-#pragma unroll
-    for (int k = 0; k < EPT; ++k) s_pay[k * THREADS + tid] = pay[k];
+    s_pay[tid] = pay;
     __syncthreads();
-#pragma unroll
-    for (int k = 0; k < EPT; ++k)
-        if (i0 + k < n) e[k] = (e[k] & 0xffffffff00000000ull) | s_pay[(u32)e[k]];
+    if (tid < n) e = (e & 0xffffffff00000000ull) | s_pay[(u32)e];
     __syncthreads();
-    u64 *s_out = s_net;
-#pragma unroll
-    for (int k = 0; k < EPT; ++k) s_out[i0 + k] = e[k];
+    s_net[tid] = e;
     __syncthreads();
 }
 
@@ -282,10 +242,10 @@ __device__ __forceinline__ bool offsets_fall(const csort::Args &a, int t)
 }
 
 // A block's table by the network
-template <int THREADS, int EPT>
+template <int THREADS>
 __device__ __forceinline__ void sort_by_network(const csort::Args &a)
 {
-    extern __shared__ __align__(16) u64 s_net[];                 // [2][THREADS * EPT]
+    extern __shared__ __align__(16) u64 s_net[];                 // [2][THREADS]
     const int t = blockIdx.x, tid = threadIdx.x;
     const int64_t tb0 = __ldg(a.offsets + (int64_t)t * a.B), tb1 = __ldg(a.offsets + (int64_t)(t + 1) * a.B);
     if (tb0 < 0 || tb1 < tb0 || tb1 > a.L || (t == 0 && tb0 != 0) || (t == a.T - 1 && tb1 != a.L)) {
@@ -303,10 +263,10 @@ __device__ __forceinline__ void sort_by_network(const csort::Args &a)
         a.absmax[t] = 0u;
         if (n == 0) a.table_cnt[t] = 0u;
     }
-    if (n <= THREADS * EPT) {
+    if (n <= THREADS) {
         const int64_t nrows = __ldg(a.row_off + t + 1) - __ldg(a.row_off + t);
         bool bad = n != a.B && offsets_fall<THREADS>(a, t);       // (otherwise every lookup looks at its own bag's offsets)
-        if (n > 0) sort_in_block<THREADS, EPT>(a, t, tb0, n, nrows, s_net, bad);
+        if (n > 0) sort_in_block<THREADS>(a, t, tb0, n, nrows, s_net, bad);
         if (bad) dq_report(a.status, DQRM_ERR_INDEX_RANGE);
         if (n > 0) write_table<THREADS>(a, t, tb0, tb1, s_net, nullptr);
     } else {                                       // (a one-index batch that is none)
@@ -334,7 +294,7 @@ __device__ __forceinline__ void sort_by_block(const csort::Args &a)
         if (offsets_fall<csort::THREADS>(a, t)) dq_report(a.status, DQRM_ERR_INDEX_RANGE);
         const int64_t nrows = __ldg(a.row_off + t + 1) - __ldg(a.row_off + t);
         const uint2 *mem = sort_in_memory<csort::THREADS>(a, t, tb0, n, nrows, s_cnt);
-        csort::write_part<1>(a, t, (u32)tb0, (u32)tb1, mem, (int)n, 0u, 0xffffffffu);
+        csort::write_sorted(a, t, (u32)tb0, (u32)tb1, mem);
     }
 }
 
@@ -348,7 +308,7 @@ small_sort_kernel(const __grid_constant__ csort::Args a)
     dq_wait_before();
     if constexpr (CL > 1) csort::sort_by_cluster<CL, E>(a);
     else if constexpr (THREADS == csort::THREADS) sort_by_block<E>(a);
-    else sort_by_network<THREADS, E>(a);
+    else sort_by_network<THREADS>(a);
 }
 
 }  // namespace ssort

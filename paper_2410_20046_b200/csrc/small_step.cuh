@@ -129,7 +129,7 @@ small_step_kernel(const __grid_constant__ Args x)
     // ---- sorted (row, row of grad_out); where the segments begin
     const uint2 *mem = nullptr;                    // (an uneven batch: a table that does not fit the block)
     if (n > THREADS) mem = ssort::sort_in_memory<THREADS>(a, t, tb0, n, nrows, s_mid);
-    else if (n > 0) ssort::sort_in_block<THREADS, 1>(a, t, tb0, n, nrows, s_net, bad);
+    else if (n > 0) ssort::sort_in_block<THREADS>(a, t, tb0, n, nrows, s_net, bad);
     if (bad) dq_report(a.status, DQRM_ERR_INDEX_RANGE);
     auto row_at = [&](int i) { return mem ? mem[i].x : (u32)(s_net[i] >> 32); };
     const int words = (n + 31) / 32;

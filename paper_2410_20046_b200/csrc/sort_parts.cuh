@@ -1,5 +1,6 @@
-// What the two sorts that a table's own blocks do (small_sort.cuh: one block, cluster_sort.cuh: a cluster of blocks) share:
-// arguments, loading of lookups, a block's stable radix sort in registers, the write-out with the segment lists.
+// Arguments of the two sorts that a table's own blocks do (small_sort.cuh: one block, cluster_sort.cuh: a cluster of blocks), and
+// how one block sorts a table alone, which both use: loading of lookups, a stable radix sort in registers, the write-out with the
+// segment lists.
 //
 // Entries are (row within the table, payload).  A block holds them warp-striped: warp w has `rounds` consecutive groups of 32
 // entries, the group's entry l in lane l.  Places beyond the last entry hold the row ~0, which sorts behind every other.
@@ -67,40 +68,37 @@ __device__ __forceinline__ void open_table(const Args &a, int t, int64_t tb0, in
     if (tb1 == tb0) a.table_cnt[t] = 0u;
 }
 
-// The rows of grad_out of lookups [first, first + count) of table t, into s_pay; whether an offset was found to fall.  Apart from
+// The rows of grad_out of table t's n lookups, into s_pay; whether an offset was found to fall.  Apart from
 // load_lookups: batches with an index a bag do not come here
-__device__ __noinline__ bool find_bags(const Args &a, int t, u32 at, u32 n, u32 first, int count, u32 *s_pay)
+__device__ __noinline__ bool find_bags(const Args &a, int t, u32 tb0, int n, u32 *s_pay)
 {
     __shared__ u32 s_last[WARPS];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int32_t *off_t = a.offsets + (int64_t)t * a.B;
     bool bad = false;
-    {   // offsets must not decrease inside the table: this block's share of its bags
-        const int64_t b0 = n == (u32)a.B ? first : (int64_t)first * a.B / n, b1 = n == (u32)a.B ? first + count : (int64_t)(first + count) * a.B / n;
-        for (int64_t i = b0 + tid; i < b1; i += THREADS) bad |= __ldg(off_t + i) > __ldg(off_t + i + 1);
-    }
+    for (int i = tid; i < a.B; i += THREADS) bad |= __ldg(off_t + i) > __ldg(off_t + i + 1);      // (they must not decrease)
     if (a.payload_position) {
-        for (int i = tid; i < count; i += THREADS) s_pay[i] = at + i;
+        for (int i = tid; i < n; i += THREADS) s_pay[i] = tb0 + i;
         __syncthreads();
         return bad;
     }
     int lo = 0, size = a.B;                        // the first lookup's bag is in [lo, lo + size)
     while (size > 1) {
         const int step = (size + THREADS - 1) / THREADS;
-        const int c = __syncthreads_count(tid * step < size && __ldg(off_t + lo + tid * step) <= (int32_t)at);
+        const int c = __syncthreads_count(tid * step < size && __ldg(off_t + lo + tid * step) <= (int32_t)tb0);
         const int skip = max(c - 1, 0) * step;
         lo += skip;
         size = min(step, size - skip);
     }
-    for (int i = tid; i < count; i += THREADS) s_pay[i] = 0u;
+    for (int i = tid; i < n; i += THREADS) s_pay[i] = 0u;
     __syncthreads();
     for (int g = lo + tid; g < a.B; g += THREADS) {
-        const int64_t o = (int64_t)__ldg(off_t + g) - at;
-        if (o >= count) break;
+        const int64_t o = (int64_t)__ldg(off_t + g) - tb0;
+        if (o >= n) break;
         if (o >= 0) atomicMax(&s_pay[o], (u32)(g - lo) + 1u);
     }
     __syncthreads();
-    const int share = ((count + WARPS - 1) / WARPS + 31) / 32 * 32, w0 = min(count, warp * share), w1 = min(count, w0 + share);
+    const int share = ((n + WARPS - 1) / WARPS + 31) / 32 * 32, w0 = min(n, warp * share), w1 = min(n, w0 + share);
     u32 last = 0;                                  // of the warp's lookups the last mark
     for (int i0 = w0; i0 < w1; i0 += 32) {
         const u32 v = i0 + lane < w1 ? s_pay[i0 + lane] : 0u, marked = __ballot_sync(0xffffffffu, v != 0u);
@@ -123,8 +121,7 @@ __device__ __noinline__ bool find_bags(const Args &a, int t, u32 at, u32 n, u32 
     return bad;
 }
 
-// Lookups [first, first + count) of table t, `n` in all, into registers; every thread of the block calls this.  s_mark: a word
-// for each of them.
+// Table t's n lookups into registers; every thread of the block calls this.  s_mark: a word for each of them.
 //
 // In a table of one-index bags in order (n == B, offsets = identity: the Criteo-shaped case) the bag of lookup p is bag p, which
 // every lookup checks from the two offsets around it, loaded beside the index.  Otherwise the first lookup's bag is found by a
@@ -132,24 +129,23 @@ __device__ __noinline__ bool find_bags(const Args &a, int t, u32 at, u32 n, u32 
 // begin at the same lookup the last counts: the others are empty).  A search for every lookup by itself is a chain of a
 // dozen loads.
 template <int E>
-__device__ __forceinline__ void load_lookups(const Args &a, int t, u32 tb0, u32 n, u32 nrows, u32 first, int count, int rounds,
-                                             u32 (&row)[E], u32 (&pay)[E], u32 *s_mark, bool &bad)
+__device__ __forceinline__ void load_lookups(const Args &a, int t, u32 tb0, int n, u32 nrows, int rounds, u32 (&row)[E], u32 (&pay)[E],
+                                             u32 *s_mark, bool &bad)
 {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int w0 = warp * rounds * 32 + lane;
     const int32_t *off_t = a.offsets + (int64_t)t * a.B;
-    const u32 at = tb0 + first;                    // of the first lookup in the batch
-    bool single = n == (u32)a.B && !a.payload_position;
+    bool single = n == a.B && !a.payload_position;
     {
         int32_t idx[E];
 #pragma unroll
         for (int e = 0; e < E; ++e)
-            if (e < rounds) idx[e] = __ldg(a.indices + at + min(w0 + e * 32, count - 1));
-        if (n == (u32)a.B) {
+            if (e < rounds) idx[e] = __ldg(a.indices + tb0 + min(w0 + e * 32, n - 1));
+        if (n == a.B) {
 #pragma unroll
             for (int e = 0; e < E; ++e) {
                 if (e < rounds) {
-                    const u32 p = first + min(w0 + e * 32, count - 1);
+                    const u32 p = min(w0 + e * 32, n - 1);
                     single &= ((u32)__ldg(off_t + p) == tb0 + p) & ((u32)__ldg(off_t + p + 1) == tb0 + p + 1);
                 }
             }
@@ -159,19 +155,19 @@ __device__ __forceinline__ void load_lookups(const Args &a, int t, u32 tb0, u32 
             row[e] = 0xffffffffu;
             pay[e] = 0u;
             const int i = w0 + e * 32;
-            if (e < rounds && i < count) {
+            if (e < rounds && i < n) {
                 bad |= (u32)idx[e] >= nrows;
                 row[e] = min((u32)max(idx[e], 0), nrows - 1u);
-                pay[e] = (first + i) * a.T + t;
+                pay[e] = i * a.T + t;
             }
         }
     }
     if (__syncthreads_and(single)) return;
-    bad |= find_bags(a, t, at, n, first, count, s_mark);
+    bad |= find_bags(a, t, tb0, n, s_mark);
 #pragma unroll
     for (int e = 0; e < E; ++e) {
         const int i = w0 + e * 32;
-        if (e < rounds && i < count) pay[e] = s_mark[i];
+        if (e < rounds && i < n) pay[e] = s_mark[i];
     }
     __syncthreads();                               // (s_mark may be written again)
 }
@@ -290,20 +286,17 @@ __device__ __forceinline__ void sort_block(u32 (&key)[E], u32 (&pay)[E], int rou
     }
 }
 
-// Writes a block's part of sorted table t, entries fin[0, m) from place `pos` of the table on, `before` the row of the entry before
-// them (none: ~0): arena row keys, payloads, and what `lists_by_table` asks for.  CL = 1: the block has the whole table
-template <int CL>
-__device__ __forceinline__ void write_part(const Args &a, int t, u32 tb0, u32 tb1, const uint2 *fin, int m, u32 pos, u32 before)
+// Writes sorted table t, entries fin[0, n): arena row keys, payloads, and the lists (lists_by_table)
+__device__ __forceinline__ void write_sorted(const Args &a, int t, u32 tb0, u32 tb1, const uint2 *fin)
 {
-    __shared__ u32 s_wheads[WARPS];                // segment starts in each warp's share
-    __shared__ u32 s_totals[16];                   // ... and in every block's part (each block sends its own)
-    __shared__ u32 s_cbase, s_ctotal;              // ... in the blocks before this one, and in the whole table
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const u32 c = CL > 1 ? blockIdx.x % CL : 0u, first_key = (u32)__ldg(a.row_off + t), j0 = tb0 + pos;
-    // every warp takes a contiguous share [w0, w1), so that the segment starts before an entry are those of the blocks before,
-    // of the warps before, and a count the warp carries along (of up to 32 rounds lane k keeps the k-th one's head bits, so that
-    // the second walk need not read the entries again)
-    const int share = ((m + WARPS - 1) / WARPS + 31) / 32 * 32, w0 = min(m, warp * share), w1 = min(m, w0 + share);
+    __shared__ u32 s_wheads[WARPS];                // segment starts in each warp's share, then before it
+    __shared__ u32 s_total;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, n = (int)(tb1 - tb0);
+    const u32 first_key = (u32)__ldg(a.row_off + t);
+    // every warp takes a contiguous share [w0, w1), so that the segment starts before an entry are those of the warps before and a
+    // count the warp carries along (of up to 32 rounds lane k keeps the k-th one's head bits, so that the second walk need not
+    // read the entries again)
+    const int share = ((n + WARPS - 1) / WARPS + 31) / 32 * 32, w0 = min(n, warp * share), w1 = min(n, w0 + share);
     u32 mine = 0, kept = 0;
 #pragma unroll 2
     for (int i0 = w0, it = 0; i0 < w1; i0 += 32, ++it) {
@@ -311,26 +304,17 @@ __device__ __forceinline__ void write_part(const Args &a, int t, u32 tb0, u32 tb
         bool head = false;
         if (i < w1) {
             const uint2 pr = fin[i];
-            a.keys_out[j0 + i] = first_key + pr.x;
-            a.vals_out[j0 + i] = pr.y;
-            head = pr.x != (i > 0 ? fin[i - 1].x : before);
+            a.keys_out[tb0 + i] = first_key + pr.x;
+            a.vals_out[tb0 + i] = pr.y;
+            head = pr.x != (i > 0 ? fin[i - 1].x : 0xffffffffu);
         }
         const u32 bits = __ballot_sync(0xffffffffu, head);
         if (lane == it) kept = bits;
         mine += __popc(bits);
-        if (!a.lists_by_table) {
-            const u32 tile0 = (j0 + i0) >> 11;
-            const u32 here = __popc(__ballot_sync(0xffffffffu, head && ((j0 + i) >> 11) == tile0));
-            if (lane == 0) {
-                if (here) atomicAdd(&a.tile_heads[tile0], here);
-                if (__popc(bits) > here) atomicAdd(&a.tile_heads[tile0 + 1], __popc(bits) - here);
-            }
-        }
     }
-    if (!a.lists_by_table) return;
     if (lane == 0) s_wheads[warp] = mine;
     __syncthreads();
-    if (warp == 0) {                               // the warps' bases within the block, and the block's total
+    if (warp == 0) {
         const u32 v = lane < WARPS ? s_wheads[lane] : 0u;
         u32 incl = v;
 #pragma unroll
@@ -339,36 +323,22 @@ __device__ __forceinline__ void write_part(const Args &a, int t, u32 tb0, u32 tb
             if (lane >= o) incl += x;
         }
         if (lane < WARPS) s_wheads[lane] = incl - v;
-        const u32 all = __shfl_sync(0xffffffffu, incl, WARPS - 1);
-        if constexpr (CL > 1) {                    // into every block's shared memory, under cover of the barrier below
-            if (lane < CL) *cg::this_cluster().map_shared_rank(&s_totals[c], (unsigned)lane) = all;
-        } else if (lane == 0) {
-            s_cbase = 0u;
-            s_ctotal = all;
-        }
-    }
-    if constexpr (CL > 1) {
-        cg::this_cluster().sync();
-        if (warp == 0) {
-            const u32 v = lane < CL ? s_totals[lane] : 0u;
-            const u32 first = __reduce_add_sync(0xffffffffu, lane < (int)c ? v : 0u), all = __reduce_add_sync(0xffffffffu, v);
-            if (lane == 0) { s_cbase = first; s_ctotal = all; }
-        }
+        if (lane == WARPS - 1) s_total = incl;
     }
     __syncthreads();
     u32 *segs = a.seg_start + tb0 + t;
-    if (c == 0 && tid == 0) {
-        a.table_cnt[t] = s_ctotal;
-        segs[s_ctotal] = tb1;                      // the slot behind the last segment holds the table's end
+    if (tid == 0) {
+        a.table_cnt[t] = s_total;
+        segs[s_total] = tb1;                       // the slot behind the last segment holds the table's end
     }
     const u32 ck_mask = (1u << a.ck_shift) - 1u, upto_me = 0xffffffffu >> (31 - lane);
-    u32 seg = s_cbase + s_wheads[warp] - 1u;
+    u32 seg = s_wheads[warp] - 1u;
 #pragma unroll 2
     for (int i0 = w0, it = 0; i0 < w1; i0 += 32, ++it) {
         const int i = i0 + lane;
-        const u32 j = j0 + i;
+        const u32 j = tb0 + i;
         const u32 bits = share <= 1024 ? __shfl_sync(0xffffffffu, kept, it & 31)
-                                       : __ballot_sync(0xffffffffu, i < w1 && fin[i].x != (i > 0 ? fin[i - 1].x : before));
+                                       : __ballot_sync(0xffffffffu, i < w1 && fin[i].x != (i > 0 ? fin[i - 1].x : 0xffffffffu));
         if (i < w1) {
             const u32 u = seg + __popc(bits & upto_me);            // the entry's segment
             if ((bits >> lane) & 1u) segs[u] = j;
@@ -398,10 +368,10 @@ __device__ __forceinline__ void sort_alone(const Args &a, int t, u32 tb0, u32 tb
         return;
     }
     u32 row[E], pay[E];
-    load_lookups<E>(a, t, tb0, n, nrows, 0, n, rounds, row, pay, reinterpret_cast<u32 *>(s_pair), bad);
+    load_lookups<E>(a, t, tb0, n, nrows, rounds, row, pay, reinterpret_cast<u32 *>(s_pair), bad);
     if (bad) dq_report(a.status, DQRM_ERR_INDEX_RANGE);
     sort_block<E>(row, pay, rounds, n, row_bits(nrows), cnt, s_pair);
-    write_part<1>(a, t, tb0, tb1, s_pair, n, 0u, 0xffffffffu);
+    write_sorted(a, t, tb0, tb1, s_pair);
 }
 
 }  // namespace csort
