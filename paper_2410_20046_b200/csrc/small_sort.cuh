@@ -145,16 +145,19 @@ __device__ __forceinline__ void sort_in_block(const csort::Args &a, int t, int64
 #pragma unroll
         for (int s = p - 1; s >= 0; --s) {
             const int stride = 1 << s;
-            const bool up = ((tid >> p) & 1) == 0, low = (tid & stride) == 0;
             if (stride >= 32) {
                 buf[tid] = e;
                 __syncthreads();
+                const bool up = ((tid >> p) & 1) == 0, low = (tid & stride) == 0;      // (before the barrier they cost it 0.07 us)
                 const u64 o = buf[tid ^ stride];
                 e = (up == low) == (e < o) ? e : o;
                 buf = buf == s_net ? s_net + THREADS : s_net;
-            } else if (live) {
-                const u64 o = shfl_xor64(e, stride);
-                e = (up == low) == (e < o) ? e : o;
+            } else {
+                const bool up = ((tid >> p) & 1) == 0, low = (tid & stride) == 0;
+                if (live) {
+                    const u64 o = shfl_xor64(e, stride);
+                    e = (up == low) == (e < o) ? e : o;
+                }
             }
         }
     }
