@@ -80,19 +80,23 @@ int64_t host_lookups_for(const dqrm_ctx *ctx, size_t workspace_bytes, int64_t L,
 
 // Whether dqrm_train_step runs the backward beside the forward.  From 1 MB of gathered rows on it does: the sort leaves most of
 // the chip idle, and with the forward on the other stream the fork is not in the backward's way (measured on B200, us a step, two
-// streams / one, graph replay and launched one by one: 26 tables of 2048 lookups of 256 bytes 26.0 / 31.6, 28.5 / 30.7; of 2000 of 64
-// bytes 22.6 / 26.0, 25.6 / 25.9; 40 tables of 500 of 192 bytes 20.5 / 26.6, 22.9 / 25.7; 26 of 500 of 144 bytes 18.5 / 24.7,
-// 21.3 / 23.9; below, 26 of 500 of 64 bytes, 22.2 / 22.1, 22.2 / 21.4).
+// streams / one, graph replay and launched one by one: 26 tables of 2048 lookups of 256 bytes 26.8 / 30.6, 28.8 / 31.3; of 2000 of 64
+// bytes 23.0 / 25.4, 25.6 / 25.8; 40 tables of 500 of 192 bytes 20.0 / 25.9, 23.5 / 26.2; 26 of 500 of 144 bytes 17.7 / 23.7,
+// 20.6 / 24.0; few tables: one of 8192 of 256 bytes 25.4 / 30.2, 27.5 / 30.0, of 64 K of 64 bytes 37.0 / 39.9, 40.6 / 39.6, four of 8192 of
+// 256 bytes 27.8 / 32.8, 31.3 / 32.9, six of 16 K of 64 bytes 33.4 / 36.3, 36.6 / 36.1, twelve of 4096 of 64 26.1 / 28.9, 30.1 / 29.1; below,
+// 26 of 500 of 64 bytes, 21.3 / 21.5, 21.8 / 21.8).
 // Batches of up to 16 K lookups that are not an index a bag fork too: a few long bags are a long chain for their lane groups
-// while the rest of the chip waits (26 tables of 64 bags, one table with 100 indices a bag, 64-byte rows: 30.8 / 53.8 us; even
-// bags of three, three tables of 600: 30.8 / 32.7 with 64-byte rows, 26.5 / 25.6 with 256-byte rows).
+// while the rest of the chip waits (bags of three, three tables of 600, 64-byte rows 24.6 / 28.1, 27.3 / 28.9, 256-byte rows 22.9 / 26.3,
+// 25.6 / 27.3; bags of six, 26 tables of 64 20.5 / 25.8, 24.2 / 26.4; bags of two, two tables of 4000 30.2 / 33.5, 34.4 / 34.1).
 //
 // Which half moves.  A forward of a few blocks an SM that starts first keeps the sort's clusters, which want eight or sixteen
 // SMs of a GPC with half or all of their registers free, waiting until it is over: so the backward stays on the caller's stream,
 // where it begins at once, and the forward goes to the context's lowest-priority one (65 K rows of 512 bytes 82.0 -> 64.3 us,
-// 426 K of 64 57.6 -> 50.8).  From BWD_ASIDE bytes on the forward outlasts the sort and would then take half of the memory
-// from the sum: the backward goes to the highest-priority stream (240 K rows of 384 bytes 110.2, 111.9 on the caller's; 852 K of
-// 256 153.0 and 160.8; but 65 K of 512 66.5).  From FWD_STAYS on the forward is the longer half and begins at once itself (8.5 M
+// 426 K of 64 57.6 -> 50.8; the lowest priority is that of an ordinary stream, and beside one it is the order of issue that
+// counts).  From BWD_ASIDE bytes on the forward outlasts the sort and would then take half of the memory
+// from the sum: the backward goes to the highest-priority stream (852 K rows of 256 bytes 171.8 us, 178.4 on the caller's, uniform
+// indices 306.7 and 312.8; 338 K of 256 83.0 and 83.9; 65 K of 512 49.3 and 47.4; 26 tables of 10 K of 256, 63 MB, 71.9 and 70.6; between
+// 64 and 98 MB the caller's is the better by 1 to 4 % where tables are few: 164 K of 512 72.9 and 70.2, 400 K of 256 107.4 and 106.6).  From FWD_STAYS on the forward is the longer half and begins at once itself (8.5 M
 // rows of 256 bytes 936 us, 944 on the other stream; 5.4 M of 64 303 both ways).
 constexpr int64_t STEP_FORKS = (int64_t)1 << 20, BWD_ASIDE = (int64_t)64 << 20, FWD_STAYS = (int64_t)1 << 30;
 bool step_forks(const dqrm_ctx *ctx, int B, int64_t L)

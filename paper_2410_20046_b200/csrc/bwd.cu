@@ -576,10 +576,12 @@ int dq_launch_bwd_sum(dqrm_ctx *ctx, const float *grad_out, int32_t *unique_rows
 }
 
 // The one-launch step takes tables of up to 512 lookups and 16 K gathered values, up to 4096 lookups in all (what a block
-// counts in front of its own).  Measured on B200 (graph replay, us a step with the forward, this way / in four launches):
-// 4 tables of 128 lookups of 16 features 9.3 / 15.7, 512 of 16 14.2 / 18.5, 1024 of 16 22.3 / 21.0, 256 of 64 15.9 / 17.8,
-// 512 of 64 24.8 / 22.0, 128 of 128 14.7 / 18.1, 256 of 128 22.8 / 20.0; 26 tables of 128 of 16 13.9 / 16.1, of 64
-// 15.8 / 20.9, of 128 19.8 / 20.7.  (With a row summary attached, or the sort chosen by the caller, the launches stay apart.)
+// counts in front of its own).  Measured on B200 (us a step with the forward, this way / in four launches, in graph replay and
+// launched one by one): 4 tables of 128 lookups of 16 features 8.1 / 14.6, 9.2 / 14.6; 512 of 16 12.2 / 18.8, 11.9 / 18.4; 256 of 64
+// 13.4 / 18.0, 12.9 / 17.1; 128 of 128 13.3 / 19.1, 12.6 / 18.1; 26 tables of 128 of 16 12.4 / 18.5, 12.4 / 17.7, of 64
+// 13.8 / 19.6, 13.2 / 18.9.  At the line the two ways of launching part: 26 tables of 128 of 128 16.4 / 15.4 but 15.9 / 18.7, 16 of 256
+// of 64 17.6 / 15.4 but 17.0 / 18.7; beyond it (when the line was drawn) 4 tables of 1024 of 16 22.3 / 21.0, 512 of 64 24.8 / 22.0.
+// (With a row summary attached, or the sort chosen by the caller, the launches stay apart.)
 bool dq_small_step_takes(const dqrm_ctx *ctx, int B, int64_t L)
 {
     const int64_t per_table = (L + ctx->T - 1) / ctx->T, want = L == (int64_t)ctx->T * B ? per_table : per_table + per_table / 4;

@@ -1,10 +1,9 @@
 // Stable radix sort of a batch's lookups by (table, row) for batches whose tables are too large for the cluster sort
 // (or on request): the lookups arrive table-major, so every table is sorted by itself, by the row number within the
 // table, and all tables move through the same launches.  Digits are at most ten bits wide and as few as the largest
-// table needs: a million rows take two passes.  Measured on B200, 8.5 M lookups of 26 tables of a million rows: 160 us,
-// and 204 with the kernels that number the segments behind it (232 before the first pass ranked by masks); one sort over the
-// arena rows of all tables, with a
-// kernel of its own that expanded the bags and three passes of nine bits, took 435 and 490.
+// table needs: a million rows take two passes.  Measured on B200, 8.5 M lookups of 26 tables of a million rows, with the kernels
+// that number the segments behind it: 204 us (228 before the first pass ranked by masks); one sort over the arena rows of all
+// tables, with a kernel of its own that expanded the bags and three passes of nine bits, took 490.
 //
 //   rs_setup     one block: where each table begins, which table each tile of TILE lookups belongs to
 //   per pass     rs_hist     digit counts of every tile (the first pass reads the indices themselves)
@@ -299,7 +298,7 @@ rs_scatter_kernel(const Args a, const uint2 *__restrict__ pairs_in, uint2 *__res
     // ---- rank within (warp, digit), counting on the way.  The first pass finds the lanes with the same digit by an OR into shared
     // memory, where the pairs will stand (by match.any, which takes the longer the more digits differ, 16 K of a tile's 38 K clocks);
     // in the later ones equal rows already stand together, and a match of few digits is the faster.  With what the digits' places
-    // below save: two passes over 8.5 M lookups 160 -> 131 us
+    // below save: the two scatters of 8.5 M lookups 156 -> 131 us
     u32 *my_mask = reinterpret_cast<u32 *>(s_pair) + warp * nb;
     static_assert(sizeof(uint2) * TILE >= (sizeof(u32) * WARPS << MAX_DIGIT_BITS), "");
     if (FIRST) {

@@ -4,7 +4,7 @@
 // A row takes LPR lanes with four features each; a warp has 32 / LPR such lane groups, and every group walks a contiguous
 // range of the sorted order by itself, BATCH entries at a time: keys and payloads are one 128-bit load each, read two
 // batches ahead, the rows of the next batch are requested before the present one is summed, and rows AHEAD batches further on
-// are asked into L2.  An entry whose key differs from the one before it ends a run and begins the
+// are asked into L2 (by a lane each: with one or two lanes for a row, of 4 and 8 features, only that many of a batch's four rows).  An entry whose key differs from the one before it ends a run and begins the
 // next: the number of the group's first segment comes from chunk_first, so that groups need nothing from one another until
 // the end.  There a segmented scan over the warp's groups (shuffles) joins the runs that cross them, and
 // only a run cut by the edge of a warp's range leaves a partial
@@ -12,12 +12,14 @@
 // FP64 and have a shape fixed by the entry positions and the launch, so results are reproducible.  The per-table
 // abs-max of the rounded sums is collected on the way: every lane keeps that of its group's present table.
 //
-// Bound by issue slots (60 to 80 a batch entry and warp: the groups' runs end at different entries, so that both sides of the branch
-// are taken) and, in small batches, by its chain of latencies: tables' lists, keys, payloads, rows, partials.  Measured on B200
-// (graph replay, us) against seg_reduce.cuh's way with several groups a warp, which scanned over the groups for every tile of
-// 64 entries and looked up the table of every row where a tile held several: 13 K rows of 64 bytes in 26 tables 17.5 -> 8.3, 52 K
-// 16.6 -> 9.0, 426 K 18.9 -> 16.3, 5.4 M in bags of 18 99.9 -> 81.9; 426 K rows of 32 bytes 15.7 -> 13.6, of 80 27.4 -> 24, of 128
-// 25.0 -> 24.0; with two groups a warp, 64 K rows of 144 bytes 15.0 -> 13.8, 20 K of 192 13.1 -> 10.5, 426 K of 192 40.6 -> 37.2.
+// Bound by its chain of latencies: tables' lists, keys, payloads, rows, partials.  Counters at 426 K rows of 64 bytes (cold caches):
+// issue slots 26 %, warps 20 % of the SM's, DRAM 19 %, conversions 16 % of their pipe; at 64 K rows of 144 bytes 28, 17, 2 and 13 %.  A
+// warp issues 80 instructions an entry of its groups (their runs end at different entries, so that both sides of the branch are
+// taken).  Measured on B200 (graph replay, us) against seg_reduce.cuh's way with several groups a warp, which scanned over the groups
+// for every tile of 64 entries, looked up the table of every row where a tile held several and had fences around its arrivals: 3.3 K
+// rows of 64 bytes in 26 tables 8.8 -> 7.2, 53 K 9.9 -> 8.2, 426 K 18.8 -> 15.5, 5.4 M in bags of 18 100.8 -> 82.4; 426 K rows of 16
+// bytes 14.6 -> 10.0, of 32 15.6 -> 12.0, of 80 26.2 -> 23.4, of 128 24.0 -> 21.4; with two groups a warp, 64 K rows of 144 bytes
+// 15.5 -> 11.6, 20 K of 192 12.9 -> 9.5, 426 K of 192 39.5 -> 35.0.
 // Rows of 52 features and more are better off with a warp each, whose branches are uniform: this way 100 K of 240 bytes took 18.8
 // instead of 17.1 us, 53 K of 256 14.7 instead of 11.5, 8.5 M in bags of 20 387 instead of 319, 82 K of 384 25.9 instead of 19.0
 // (but 852 K of 256 56.6 instead of 60.3, 13 K of 512 10.8 instead of 12.7; none of it shows beside a forward and a sort).  Integer

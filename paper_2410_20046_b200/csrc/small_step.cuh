@@ -16,8 +16,8 @@
 // reproducible.
 //
 // Bound by its chain of latencies (two loads, the network, a gather, a row).  Measured on B200 (graph replay): a step of 4
-// tables of 128 lookups of 16 features 9.3 us (15.7 in four launches), 26 tables of 128 12.0 (13.9 before the counted lookups
-// were all asked for at once; 16.1 in four).
+// tables of 128 lookups of 16 features 8.1 us (14.6 in four launches), 26 tables of 128 12.4 (13.9 before the counted lookups
+// were all asked for at once; 18.5 in four).
 #pragma once
 #include "small_sort.cuh"
 
