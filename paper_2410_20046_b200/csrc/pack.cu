@@ -5,7 +5,7 @@
 // lowest bits first, as a b-bit two's-complement code, b in {2, 4, 8}; a row takes D*b/8 bytes.
 //
 // pack_kernel      streams the arena once (4 bytes read, b/8 bytes written per element); one
-//                  thread turns one 128-bit vector of weights into b/2 bytes
+//                  thread turns 32 bytes of weights into b bytes
 // packed_fwd_kernel gathers packed rows, decodes, multiplies by the table's scale and sum-pools
 //                  in bag order in FP64 - bit-identical to the training forward on the same
 //                  master weights and scales
@@ -15,8 +15,9 @@ namespace {
 
 constexpr int PK_THREADS = 256;
 constexpr int PK_CHUNK4 = 4096;          // 128-bit vectors per chunk
-constexpr int PK_UNROLL = 8;             // vectors of a thread in flight (one at a time: 427 us for 2.16 GB at 4 bits, eight: 405,
-                                         // sixteen: 437; block and chunk sizes make no difference)
+// Loads of 32 bytes of a thread in flight.  Bound by DRAM: 2.16 GB at 4 bits 376 us, of which reading and writing at the rate of a copy are 371
+// (with loads of 16 bytes, eight in flight, stores of two bytes and a conversion instruction for every code 411)
+constexpr int PK_UNROLL = 4;
 
 template <int BITS>
 __device__ __forceinline__ u32 pack4(const float4 &codes)
@@ -24,6 +25,29 @@ __device__ __forceinline__ u32 pack4(const float4 &codes)
     const u32 m = (1u << BITS) - 1u;
     return ((u32)(int)codes.x & m) | (((u32)(int)codes.y & m) << BITS) | (((u32)(int)codes.z & m) << (2 * BITS)) |
            (((u32)(int)codes.w & m) << (3 * BITS));
+}
+
+// The packed codes of four elements.  Away from ties the four m = lo - code, integers of at most 2^BITS held as floats, are put
+// side by side by multiply-adds, all exact (below 2^16; eight bits: two halves), and one addition of 1.5*2^23 leaves the
+// integer in the low bits: no conversion instruction.  Code and lo - m agree modulo 2^BITS
+template <int BITS>
+__device__ __forceinline__ u32 quantise_packed4(const float4 &v, const QuantScale &q)
+{
+    float dist = q.fast ? 0.f : 1.f;
+    const float2 ma = dq_codes2(make_float2(v.x, v.y), q, dist), mb = dq_codes2(make_float2(v.z, v.w), q, dist);
+    if (!(dist < q.tie_lim)) {
+        return pack4<BITS>(make_float4(dq_codef_ieee(v.x, q), dq_codef_ieee(v.y, q), dq_codef_ieee(v.z, q), dq_codef_ieee(v.w, q)));
+    }
+    const float MAGIC = 12582912.0f, step = (float)(1 << BITS);
+    // (-m is code - lo, in [0, 2^BITS))
+    if constexpr (BITS == 8) {
+        const float x = __fmaf_rn(ma.y, -step, __fsub_rn(MAGIC, ma.x)), y = __fmaf_rn(mb.y, -step, __fsub_rn(MAGIC, mb.x));
+        return __byte_perm(__float_as_uint(x), __float_as_uint(y), 0x5410) ^ 0x80808080u;
+    } else {
+        const float2 pair = __ffma2_rn(mb, make_float2(-step * step, -step * step), make_float2(-ma.x, -ma.y));
+        const float x = __fmaf_rn(pair.y, step, __fadd_rn(pair.x, MAGIC));
+        return (__float_as_uint(x) & ((1u << (4 * BITS)) - 1u)) ^ (BITS == 4 ? 0x8888u : 0xaau);
+    }
 }
 
 template <int BITS>
@@ -34,10 +58,26 @@ __device__ __forceinline__ void store_packed(uint8_t *dst, int64_t v4, u32 bits4
     else reinterpret_cast<u32 *>(dst)[v4] = bits4;
 }
 
+// ... of two vectors that lie side by side, the first at an even place
+template <int BITS>
+__device__ __forceinline__ void store_packed2(uint8_t *dst, int64_t v8, u32 first, u32 second)
+{
+    if constexpr (BITS == 2) __stcs(reinterpret_cast<unsigned short *>(dst) + v8, (unsigned short)(first | second << 8));
+    else if constexpr (BITS == 4) __stcs(reinterpret_cast<u32 *>(dst) + v8, first | second << 16);
+    else __stcs(reinterpret_cast<uint2 *>(dst) + v8, make_uint2(first, second));
+}
+
+// 32 bytes that are read once
+__device__ __forceinline__ void load8(const float4 *p, float4 &a, float4 &b)
+{
+    asm volatile("ld.global.nc.L1::no_allocate.L2::evict_first.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];\n"
+                 : "=f"(a.x), "=f"(a.y), "=f"(a.z), "=f"(a.w), "=f"(b.x), "=f"(b.y), "=f"(b.z), "=f"(b.w) : "l"(p));
+}
+
 template <int BITS>
 __global__ void __launch_bounds__(PK_THREADS)
 pack_kernel(const float4 *__restrict__ arena4, const int64_t *__restrict__ row_off, int T, int D, int64_t n4,
-            const float *__restrict__ scales, uint8_t *__restrict__ packed)
+            const float *__restrict__ scales, uint8_t *__restrict__ packed, int pairs)
 {
     dq_wait_before();
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -51,27 +91,31 @@ pack_kernel(const float4 *__restrict__ arena4, const int64_t *__restrict__ row_o
         const int t0 = dq_table_of(v4_off, T, c0);
         const bool one_table = c1 <= v4_off[t0 + 1];
         QuantScale qs = dq_make_scale(__ldg(scales + t0), BITS);
-        if (one_table && c1 - c0 == PK_CHUNK4) {
-            // a thread's vectors of PK_UNROLL rounds are all in flight before the first is quantised
+        if (pairs && one_table && c1 - c0 == PK_CHUNK4) {
+            // a thread's loads of PK_UNROLL rounds are all in flight before the first is quantised
 #pragma unroll 1
-            for (int r = 0; r < PK_CHUNK4; r += PK_THREADS * PK_UNROLL) {
-                float4 v[PK_UNROLL];
-#pragma unroll
-                for (int k = 0; k < PK_UNROLL; ++k) v[k] = __ldcs(arena4 + c0 + r + k * PK_THREADS + threadIdx.x);
+            for (int r = 0; r < PK_CHUNK4 / 2; r += PK_THREADS * PK_UNROLL) {
+                float4 v[PK_UNROLL][2];
 #pragma unroll
                 for (int k = 0; k < PK_UNROLL; ++k) {
-                    float4 cd, dq;
-                    dq_fq4(v[k], qs, cd, dq);
-                    store_packed<BITS>(packed, c0 + r + k * PK_THREADS + threadIdx.x, pack4<BITS>(cd));
+                    const float4 *p = arena4 + c0 + 2 * (r + k * PK_THREADS + threadIdx.x);
+                    if (pairs == 2) {
+                        load8(p, v[k][0], v[k][1]);
+                    } else {
+                        v[k][0] = __ldcs(p);
+                        v[k][1] = __ldcs(p + 1);
+                    }
                 }
+#pragma unroll
+                for (int k = 0; k < PK_UNROLL; ++k)
+                    store_packed2<BITS>(packed, c0 / 2 + r + k * PK_THREADS + threadIdx.x, quantise_packed4<BITS>(v[k][0], qs),
+                                        quantise_packed4<BITS>(v[k][1], qs));
             }
             continue;
         }
         for (int64_t i = c0 + threadIdx.x; i < c1; i += PK_THREADS) {
             if (!one_table) qs = dq_make_scale(__ldg(scales + dq_table_of(v4_off, T, i)), BITS);
-            float4 cd, dq;
-            dq_fq4(__ldcs(arena4 + i), qs, cd, dq);
-            store_packed<BITS>(packed, i, pack4<BITS>(cd));
+            store_packed<BITS>(packed, i, quantise_packed4<BITS>(__ldcs(arena4 + i), qs));
         }
     }
 }
@@ -323,8 +367,10 @@ int launch_pack(dqrm_ctx *ctx, const float *tables, const float *scales, uint8_t
 {
     const int64_t n4 = ctx->total_rows * (ctx->D / 4);
     const size_t smem = (size_t)(ctx->T + 1) * sizeof(int64_t);
+    // vectors in pairs where their packed bytes may be stored at once; read at once, too, where the arena begins on 32 bytes
+    const int pairs = !dq_aligned(packed, (size_t)BITS) ? 0 : dq_aligned(tables, 2 * sizeof(float4)) ? 2 : 1;
     DQRM_CUDA_TRY(ctx, dq_launch(pack_kernel<BITS>, dim3(ctx->num_sms * 8), dim3(PK_THREADS), smem, st,
-                                 reinterpret_cast<const float4 *>(tables), ctx->d_row_off, ctx->T, ctx->D, n4, scales, packed));
+                                 reinterpret_cast<const float4 *>(tables), ctx->d_row_off, ctx->T, ctx->D, n4, scales, packed, pairs));
     dq_mark(ctx, st, DQ_K_PACK);
     return DQRM_OK;
 }

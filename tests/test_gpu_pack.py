@@ -130,3 +130,29 @@ def test_packed_lookup_uneven_bags_with_one_index_per_bag_on_average(oracle):
     c.ctx.raise_on_device_error()
     assert bit_equal(out.cpu().numpy(), want)
     c.ctx.close()
+
+
+# whole chunks of 4096 vectors and what is left of them, tables that begin inside a chunk; arenas and packed rows that begin where
+# 32 bytes of weights or a pair's packed bytes cannot be taken at once
+@pytest.mark.parametrize("bits", [2, 4, 8])
+@pytest.mark.parametrize("shift,packed_shift", [(0, 0), (4, 0), (0, 1), (4, 1)])
+def test_pack_of_whole_chunks(oracle, bits, shift, packed_shift):
+    wl = W.Workload("chunks", (9_000, 7, 12_001), D=16, B=1, alpha=None)
+    c = Case(wl)
+    t = c.torch
+    tables = W.tables_np(wl)
+    b = np.full(wl.T, bits, dtype=np.int32)
+    scales, _ = oracle.scale_refresh(tables, c.row_off, wl.D, b)
+    scales = (scales * np.float32(0.7)).astype(np.float32)          # some values beyond the range
+    want = oracle.pack_tables(tables, c.row_off, wl.D, scales, bits)
+    arena = t.empty(tables.size + 8, dtype=t.float32, device="cuda")
+    d_tables = arena[shift:shift + tables.size].view(tables.shape)
+    d_tables.copy_(c.dev(tables))
+    step = packed_shift * max(1, bits // 2)                         # the least that the call takes
+    buf = t.full((want.size + 64,), 0xA5, dtype=t.uint8, device="cuda")
+    c.ctx.pack_tables(d_tables, c.dev(scales), bits, buf[step:])
+    c.ctx.raise_on_device_error()
+    got = buf.cpu().numpy()
+    assert (got[:step] == 0xA5).all() and (got[step + want.size:] == 0xA5).all()
+    assert bit_equal(got[step:step + want.size].reshape(want.shape), want)
+    c.ctx.close()
