@@ -42,6 +42,7 @@ struct FwdArgs {
     int T, D, B;
     int64_t L;
     int *status;
+    int per_warp;                // one-index batches: bags of a warp, up to 32
     int let_next;                // the kernel behind this one may begin (it waits itself where it has to)
 };
 
@@ -128,19 +129,21 @@ fwd_onehot_kernel(const FwdArgs a)
     const int wlane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int lane = wlane % LPR, grp = wlane / LPR;
     const int64_t g0 = (int64_t)t * a.B;
+    const int per = RPW * NB >= 32 ? 32 : a.per_warp;
+    const unsigned all = 0xffffffffu >> (32 - per);
     // a bag's offsets and its index, the right one when the offsets are the identity (L == T*B): on their way before the
     // table's constants are waited for (426 K rows of 64 bytes 8.9 -> 8.4 us, 852 K packed ones of 32 40.6 -> 39.5; not where the
     // rows take the whole warp, which would spill more: 65 K of 512 bytes 12.8, 13.0)
     int32_t lo = 0, hi = 0, idx = 0;
     auto load = [&](int i) {
-        if (i < a.B) {
+        if (i < a.B && wlane < per) {
             lo = __ldg(a.offsets + g0 + i);
             hi = __ldg(a.offsets + g0 + i + 1);
             idx = __ldg(a.indices + g0 + i);
         }
     };
-    const int stride = gridDim.y * (WPB * 32);
-    const int start = (blockIdx.y * WPB + warp) * 32;
+    const int stride = gridDim.y * (WPB * per);
+    const int start = (blockIdx.y * WPB + warp) * per;
     if (LPR < 32) load(start + wlane);
     const TableCtx tc = table_ctx(a, t, D);
     const float4 *tbl_lane = reinterpret_cast<const float4 *>(tc.tbl) + lane;
@@ -152,8 +155,9 @@ fwd_onehot_kernel(const FwdArgs a)
         if (LPR == 32 || i0 != start) load(i0 + wlane);
         // ---- lane-per-bag bookkeeping
         const int i = i0 + wlane;
+        const bool mine = i < a.B && wlane < per;
         bool single = false;
-        if (i < a.B) {
+        if (mine) {
             single = (hi - lo == 1) & (lo >= 0) & ((int64_t)hi <= a.L);
             if (single) {
                 if ((int64_t)lo != tc.g0 + i) idx = __ldg(a.indices + lo);
@@ -161,15 +165,15 @@ fwd_onehot_kernel(const FwdArgs a)
             }
         }
         const unsigned one = __ballot_sync(0xffffffffu, single);
-        unsigned rare = __ballot_sync(0xffffffffu, (i < a.B) && !single);
+        unsigned rare = __ballot_sync(0xffffffffu, mine && !single);
         float4 *out_lane = reinterpret_cast<float4 *>(a.out) + ((int64_t)i0 * a.T + t) * d4 + lane;
 
         // ---- rows, RPW per step, NB steps in flight
         // (nearly always: no checks; but rows of more than 1 KB whose last lanes stand idle are better without their loads: 65 K
         // of 2064 bytes 112 us, 120 with)
-        if ((EXACT || CH <= 2) && one == 0xffffffffu) {
+        if ((EXACT || CH <= 2) && one == all) {
 #pragma unroll 1
-            for (int k0 = 0; k0 < 32; k0 += RPW * NB) {
+            for (int k0 = 0; k0 < per; k0 += RPW * NB) {
                 int32_t ib[NB];
 #pragma unroll
                 for (int b = 0; b < NB; ++b) ib[b] = __shfl_sync(0xffffffffu, idx, (k0 + b * RPW + grp) & 31);
@@ -193,7 +197,7 @@ fwd_onehot_kernel(const FwdArgs a)
             continue;
         }
 #pragma unroll 1
-        for (int k0 = 0; k0 < 32; k0 += RPW * NB) {
+        for (int k0 = 0; k0 < per; k0 += RPW * NB) {
             if ((one >> k0) == 0u) break;
             int32_t ib[NB];
 #pragma unroll
@@ -364,6 +368,12 @@ constexpr int LONG_BAG = 18;
 inline bool long_bags(const int8_t *codes_out, int T, int B, int64_t L) { return !codes_out && L >= LONG_BAG * (int64_t)T * B; }
 inline bool warp_per_bag(const FwdArgs &a, int lpr) { return lpr == 16 && long_bags(a.codes_out, a.T, a.B, a.L); }
 
+// Warps an SM below which a one-index batch's warps take fewer bags, down to one step of their rows: a warp's steps are a chain, and a
+// small batch has too few warps to hide it.  Measured on B200 (us; 32 bags a warp / so many that there are twelve warps an SM
+// at least): 26 tables of 2048 bags of 64 features (11 warps an SM) 5.25 / 4.45, one of 5000 of 128 6.51 / 2.82, four of 9000 of 32 3.35 / 2.94.  With more than twelve the
+// forward alone would gain on, but not the step in which it runs beside the sort: one table of 65,536 bags of 128 features (14 warps an
+// SM) 12.6 / 10.6, the step around it 67.7 / 68.3
+constexpr int FEW_WARPS = 12;
 constexpr int MIXED_TABLES = 8;
 // Order of the blocks.  All tables' blocks for the same bags side by side: the pooled rows of a bag lie next to one another in the
 // output, and DRAM takes them better together (one index a bag, 852 K rows of 256 bytes 49.0 -> 46.9 us, 426 K of 64 bytes 9.1 -> 8.9).
@@ -392,12 +402,17 @@ cudaError_t launch_bags(const FwdArgs &a, dim3 grid, cudaStream_t st)
 }
 
 template <int LPR, int CH, bool EXACT>
-int launch2(dqrm_ctx *ctx, const FwdArgs &a, cudaStream_t st)
+int launch2(dqrm_ctx *ctx, FwdArgs a, cudaStream_t st)
 {
     constexpr int GPB = FW_THREADS / LPR;
     // the one-index kernel does not emit codes; a caller that asks for them gets the general kernel
     const bool onehot = a.L == (int64_t)a.T * a.B && a.codes_out == nullptr;
-    const int per_block = onehot ? FW_THREADS : warp_per_bag(a, LPR) ? GPB / 2 : GPB;
+    a.per_warp = 32;
+    if (onehot) {
+        constexpr int STEP = 32 / LPR * NBOf<LPR, CH>::v;
+        while (a.per_warp / 2 >= STEP && (int64_t)a.T * ((a.B + a.per_warp - 1) / a.per_warp) < (int64_t)ctx->num_sms * FEW_WARPS) a.per_warp /= 2;
+    }
+    const int per_block = onehot ? FW_THREADS / 32 * a.per_warp : warp_per_bag(a, LPR) ? GPB / 2 : GPB;
     int bx = (a.B + per_block - 1) / per_block;
     const int cap = (ctx->num_sms * 32 + ctx->T - 1) / ctx->T;     // a few waves over all tables
     if (bx > cap) bx = cap;
@@ -429,7 +444,7 @@ int dq_launch_fwd(dqrm_ctx *ctx, const float *tables, const int32_t *indices, co
                   int B, int64_t L, cudaStream_t st, bool let_next)
 {
     FwdArgs a{tables, ctx->d_row_off, indices, offsets, scales, bits, out, codes_out, ctx->T, ctx->D, B, L,
-              ctx->d_status, let_next ? 1 : 0};
+              ctx->d_status, 32, let_next ? 1 : 0};
     const int d4 = ctx->D / 4;
     if (d4 <= 1) return launch<1, 1>(ctx, a, st);
     if (d4 <= 2) return launch<2, 1>(ctx, a, st);

@@ -44,3 +44,29 @@ def test_order_of_the_blocks(oracle, D, B, bag):
     c.ctx.raise_on_device_error()
     assert bit_equal(d_out.cpu().numpy(), want)
     c.ctx.close()
+
+
+# one-index batches of few warps, which take 32 bags each down to one step of rows: whole and cut warps, and bags of none and of two
+@pytest.mark.parametrize("D", [16, 20, 32, 36, 64, 100, 128, 200, 256, 1020])
+@pytest.mark.parametrize("T,B", [(1, 1), (3, 5), (2, 33), (5, 100), (26, 517), (7, 2049), (26, 2048)])
+def test_few_warps(oracle, D, T, B):
+    if T * B > 20_000 and D not in (32, 64, 100, 256):
+        pytest.skip("the larger batches take one width of each kind")
+    wl = W.Workload("few", tuple(3 + 50 * t for t in range(T)), D=D, B=B, alpha=None)
+    rng = np.random.default_rng(D + B)
+    lens = np.ones(T * B, dtype=np.int64)
+    for odd in (False, True):
+        if odd:                          # (as many lookups as bags all the same)
+            if T * B < 5:
+                break
+            at = rng.permutation(T * B)[:T * B // 50 * 2 + 2]
+            lens[at[::2]], lens[at[1::2]] = 0, 2
+        off = np.concatenate([[0], np.cumsum(lens)]).astype(np.int32)
+        table = np.repeat(np.arange(T), lens.reshape(T, B).sum(1))
+        idx = (rng.random(off[-1]) * np.array(wl.rows)[table]).astype(np.int32)
+        c = Case(wl, max_lookups=len(idx))
+        tables = W.tables_np(wl)
+        scales, _ = oracle.scale_refresh(tables, c.row_off, D, c.bits_np)
+        out, _ = c.gpu_fwd(c.dev(tables), idx, off, c.dev(scales), want_codes=False)
+        assert bit_equal(out, oracle.emb_fwd(tables, c.row_off, D, B, idx, off, scales, c.bits_np))
+        c.ctx.close()
