@@ -54,16 +54,17 @@ Layout make_layout(const dqrm_ctx *ctx, int64_t L)
     int64_t Lc = L < 1 ? 1 : L;
     y.num_tiles = (Lc + ST_TILE - 1) / ST_TILE;
     y.radix_tiles = rsort::max_tiles(ctx->T, Lc);
-    // the sum: every warp that the GPU holds at once walks one range
+    // the sum: every warp that the GPU holds at once walks one range (long batches: segred::range_tiles)
     int64_t warps = segred::takes_groups(ctx->D) ? (int64_t)ctx->num_sms * segred::GROUPS_BLOCKS * segred::GROUPS_THREADS / 32
-                                                 : (int64_t)ctx->num_sms * segred::BLOCKS_PER_SM / segred::column_blocks(ctx->D) * segred::WARPS;
+                                                 : (int64_t)ctx->num_sms * segred::sum_blocks(segred::floats_per_lane(ctx->D)) /
+                                                       segred::column_blocks(ctx->D) * segred::WARPS;
     if (warps < 1) warps = 1;
     y.sum_small = Lc < 96 * warps;         // (three tiles of 32 a warp: 160 K rows of 192 bytes 38.9 -> 28.7 us, 208 K of
                                               // 256 bytes 30.7 -> 28.7; at 852 K rows tiles of 32 are 2 us the faster)
     const int I = segred::tile_entries(y.sum_small);
     y.sum_shift = segred::takes_groups(ctx->D) ? segred::CHUNK_SHIFT : segred::chunk_shift(y.sum_small);
     y.sum_tiles = (Lc + I - 1) / I;
-    y.range_tiles = (int)((y.sum_tiles + warps - 1) / warps);
+    y.range_tiles = segred::range_tiles(ctx->D, y.sum_tiles, warps);
     const int64_t groups = 32 / segred::lanes_per_row(ctx->D), chunk = (int64_t)1 << segred::CHUNK_SHIFT;
     y.sum_span = (int)(((Lc + warps * groups - 1) / (warps * groups) + chunk - 1) / chunk * chunk);
     y.sum_ranges = (Lc + y.sum_span * groups - 1) / (y.sum_span * groups);
@@ -84,8 +85,10 @@ Layout make_layout(const dqrm_ctx *ctx, int64_t L)
     y.tb = take(sizeof(u32) * (ctx->T + 1));
     y.chunk_first = take(sizeof(u32) * (Lc / 8 + 1));      // (the most that any L up to this one may need)
     y.tile_done = take(sizeof(uint2) * (Lc / 8 + 1));
-    y.partials = take(sizeof(double) * std::min(Lc / 8 + 1, warps) * 2 * ctx->D);
-    y.group_partials = take(sizeof(double) * (std::min(Lc / 8 + 1, warps) / segred::FOLD_GROUP + 1) * 2 * ctx->D);
+    // (ranges: the most that any L up to this one may need)
+    const int64_t ranges = std::max(std::min(Lc / 8 + 1, warps), segred::takes_groups(ctx->D) ? (int64_t)0 : Lc / (32 * segred::RANGE_TILES) + 1);
+    y.partials = take(sizeof(double) * ranges * 2 * ctx->D);
+    y.group_partials = take(sizeof(double) * (ranges / segred::FOLD_GROUP + 1) * 2 * ctx->D);
     y.total = o;
     return y;
 }

@@ -35,14 +35,26 @@ constexpr u32 CNT_BROKEN = 0xFFFFFFFFu;      // table_cnt[t]: the table's bounda
 // features per lane for feature size D (D > 128: 128 features per warp)
 __host__ __device__ constexpr int floats_per_lane(int D) { return D <= 64 ? 2 : 4; }
 __host__ __device__ constexpr int column_blocks(int D) { return (D + 127) / 128; }
-// rows in flight, entries of a tile, resident blocks: 4 KB in flight (two
-// batches in turn) and three blocks (four blocks: 78 instead of 71 us at 852 K rows of 256 bytes)
-__host__ __device__ constexpr int batch_entries(int vec, bool small) { return small ? 4 : 16 / vec; }
+// rows of a batch, of which one is in flight while the other is summed.  With two features a lane four of them leave room for a fourth
+// resident block: 852 K rows of 256 bytes 58.4 -> 56.5 us, 1.3 M in bags of twenty 97.9 -> 89.7 (eight rows and three blocks
+// before; five blocks 65 and more: values are spilled).  With four features a lane a fourth block spills, 984 K rows of 512 bytes 82 -> 119
+constexpr int BATCH_ROWS = 4;
 // A warp that has one tile takes its batches of rows one after the other, 4 to 8 us for 32 rows, so a batch of wide
 // rows that would give every resident warp less than three tiles of 32 entries is cut into tiles of 8
 __host__ __device__ constexpr int tile_entries(bool small) { return small ? 8 : 32; }
 __host__ __device__ constexpr int chunk_shift(bool small) { return small ? 3 : 5; }    // of chunk_first
-constexpr int BLOCKS_PER_SM = 3;
+__host__ __device__ constexpr int sum_blocks(int vec) { return vec == 2 ? 4 : 3; }
+// A warp that would get more than a dozen tiles gets eight, and there are more blocks than the GPU holds at once: they pass over the
+// tables one after the other, each table's share of grad_out stays in L2 while it is read from all sides, and warps with many short runs
+// hold up fewer others.  8.5 M rows of 256 bytes (multi-hot) 306 us with one range for every resident warp, 285 with ranges of sixteen
+// tiles, 276 with eight; a loop over the ranges in each warp, instead of more blocks, costs registers (356).  With four
+// features a lane it does not help: 1.6 M rows of 512 bytes 116 -> 122
+constexpr int RANGE_TILES = 8;
+inline int range_tiles(int D, int64_t tiles, int64_t warps)
+{
+    const int64_t even = (tiles + warps - 1) / warps;
+    return (int)(floats_per_lane(D) == 2 && even > RANGE_TILES + RANGE_TILES / 2 ? RANGE_TILES : even);
+}
 
 struct Args {
     const u32 *keys, *vals, *seg_start, *chunk_first;
@@ -145,11 +157,11 @@ __device__ __noinline__ void note_max(u32 *absmax, const u32 *s_uoff, int t_firs
 // holds features.  Rows of 3 KB and more are not asked into L2 ahead: their blocks of features ask for whole rows already
 // (65 K rows of 4080 bytes 138 us, 154 with the request; of 2064 bytes 87 and 85)
 template <int VEC, bool EXACT, bool SMALL, bool COLS>
-__global__ void __launch_bounds__(THREADS, BLOCKS_PER_SM)
+__global__ void __launch_bounds__(THREADS, sum_blocks(VEC))
 seg_sum_kernel(const Args a)
 {
     dq_wait_before();
-    constexpr int C = batch_entries(VEC, SMALL);         // rows in flight
+    constexpr int C = BATCH_ROWS;
     constexpr int I = tile_entries(SMALL);
     constexpr int NB = I / C;                     // batches per tile
     static_assert(NB % 2 == 0 && I <= 32, "");

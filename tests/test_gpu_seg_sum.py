@@ -168,6 +168,32 @@ def test_lane_groups_of_many_rounds(oracle, D, B, sort_path):
     c.ctx.close()
 
 
+# more than a dozen tiles of 32 for each of the 4736 warps that 148 SMs hold: ranges of eight tiles, several of them for a warp's place
+@pytest.mark.parametrize("D", [52, 64])
+@pytest.mark.parametrize("sort_path", [0, 1])
+def test_ranges_beyond_the_resident_warps(oracle, D, sort_path):
+    rng = np.random.default_rng(D)
+    rows, B = (40_000, 3, 900_000), 40_003
+    T = len(rows)
+    wl = W.Workload("ranges", rows, D=D, B=B, alpha=None)
+    lens = rng.integers(0, 36, T * B)
+    off = np.concatenate([[0], np.cumsum(lens)]).astype(np.int32)
+    L = int(off[-1])
+    assert L > 32 * 13 * 4736
+    table = np.repeat(np.arange(T), lens.reshape(T, B).sum(1))
+    idx = (rng.random(L) ** rng.choice([1, 8], L) * np.array(rows)[table]).astype(np.int32)      # runs of one to hundreds of thousands
+    go = rng.standard_normal((B, T, D), dtype=np.float32)
+    c = Case(wl, max_lookups=L)
+    c.ctx.set_sort_path(sort_path)
+    ur, uo, gr = c.gpu_bwd(idx, off, go)
+    o_ur, o_uo, o_gr = oracle.emb_bwd(go, T, D, B, idx, off)
+    assert bit_equal(uo, o_uo) and bit_equal(ur, o_ur)
+    # n terms of magnitude below 6 in FP64 in two orders, each sum rounded once
+    n = int(np.bincount(idx + 1_000_000 * table).max())
+    np.testing.assert_allclose(gr, o_gr, rtol=2.0 ** -23, atol=12.0 * n * n * 2.0 ** -53)
+    c.ctx.close()
+
+
 @pytest.mark.parametrize("D,kernel", [(4, "seg_groups_kernel"), (16, "seg_groups_kernel"), (48, "seg_groups_kernel"), (52, "seg_sum_kernel"), (128, "seg_sum_kernel")])
 def test_profile_names_the_kernel(D, kernel):
     """The profile says which of the two summing kernels ran."""
