@@ -80,9 +80,10 @@ Layout make_layout(const dqrm_ctx *ctx, int64_t L)
     y.vals_a = take(sizeof(u32) * Lc);
     y.pairs_a = take(sizeof(uint2) * Lc);
     y.pairs_b = take(sizeof(uint2) * Lc);
-    y.seg_start = take(sizeof(u32) * (Lc + ctx->T + 1));     // (lists by table: one slot more per table)
-    y.table_cnt = take(sizeof(u32) * ctx->T);
-    y.tb = take(sizeof(u32) * (ctx->T + 1));
+    const int64_t lists = (int64_t)ctx->T * csort::MAX_PARTS;
+    y.seg_start = take(sizeof(u32) * (Lc + lists + 1));      // (lists by table: one slot more per list)
+    y.table_cnt = take(sizeof(u32) * lists);
+    y.tb = take(sizeof(u32) * (lists + 1));
     y.chunk_first = take(sizeof(u32) * (Lc / 8 + 1));      // (the most that any L up to this one may need)
     y.tile_done = take(sizeof(uint2) * (Lc / 8 + 1));
     // (ranges: the most that any L up to this one may need)
@@ -245,7 +246,7 @@ template <int VEC>
 int launch_sum(dqrm_ctx *ctx, const segred::Args &a, bool small, cudaStream_t st)
 {
     using namespace segred;
-    const size_t smem = smem_bytes(ctx->T);
+    const size_t smem = smem_bytes(a.T);
     const int64_t ranges = (a.num_tiles + a.range_tiles - 1) / a.range_tiles;
     const dim3 grid((unsigned)((ranges * a.columns + WARPS - 1) / WARPS));
     const bool exact = ctx->D % (32 * VEC) == 0;
@@ -276,10 +277,10 @@ int launch_sum_groups(dqrm_ctx *ctx, const segred::Args &a, cudaStream_t st)
     while (warps > 2 && a.ranges < warps * (unsigned)ctx->num_sms) warps /= 2;
     const dim3 grid((a.ranges + warps - 1) / warps), block(warps * 32);
     if (!dq_aligned(a.grad_out, sizeof(float4)) || !dq_aligned(a.grad_rows, sizeof(float4)))
-        DQRM_CUDA_TRY(ctx, (dq_launch(seg_groups_kernel<LPR, false, unaligned_vec(LPR)>, grid, block, smem_bytes(ctx->T), st, a)));
+        DQRM_CUDA_TRY(ctx, (dq_launch(seg_groups_kernel<LPR, false, unaligned_vec(LPR)>, grid, block, smem_bytes(a.T), st, a)));
     else if (takes_groups(LPR * 4) && ctx->D == LPR * 4)
-        DQRM_CUDA_TRY(ctx, (dq_launch(seg_groups_kernel<LPR, takes_groups(LPR * 4)>, grid, block, smem_bytes(ctx->T), st, a)));
-    else DQRM_CUDA_TRY(ctx, (dq_launch(seg_groups_kernel<LPR, false>, grid, block, smem_bytes(ctx->T), st, a)));
+        DQRM_CUDA_TRY(ctx, (dq_launch(seg_groups_kernel<LPR, takes_groups(LPR * 4)>, grid, block, smem_bytes(a.T), st, a)));
+    else DQRM_CUDA_TRY(ctx, (dq_launch(seg_groups_kernel<LPR, false>, grid, block, smem_bytes(a.T), st, a)));
     dq_mark(ctx, st, DQ_K_SEG_GROUPS);
     return DQRM_OK;
 }
@@ -339,7 +340,7 @@ cudaError_t launch_clusters(dqrm_ctx *ctx, void (*kernel)(csort::Args), int slot
     }
     if (e == cudaSuccess) {
         cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3((unsigned)(ctx->T * CL));
+        cfg.gridDim = dim3((unsigned)(ca.T * ca.parts * CL));
         cfg.blockDim = dim3(csort::THREADS);
         cfg.dynamicSmemBytes = smem;
         cfg.stream = st;
@@ -355,11 +356,20 @@ cudaError_t launch_clusters(dqrm_ctx *ctx, void (*kernel)(csort::Args), int slot
     return e;
 }
 
-template <int CL>
+template <int CL, bool PARTS = false>
 cudaError_t launch_cluster_sort(dqrm_ctx *ctx, csort::Args ca, int cap, cudaStream_t st)
 {
     ca.cap = cap;
-    return launch_clusters<CL>(ctx, csort::cluster_sort_kernel<CL, 0>, CL == csort::CLUSTER ? 0 : 3, ca, csort::smem_bytes(cap), st);
+    return launch_clusters<CL>(ctx, csort::cluster_sort_kernel<CL, 0, PARTS>, PARTS ? 6 : CL == csort::CLUSTER ? 0 : 3, ca, csort::smem_bytes(cap), st);
+}
+
+// A table alone is shared by four clusters of sixteen blocks where as many as eight would fit (eight do not find room at the same
+// moment: 34 us).  Measured on B200 (us; four clusters / one): 65,536 lookups of 10 M rows 19.9 / 29.5, Zipf 1.2 19.9 / 24.2, of 3000
+// rows 15.3 / 19.9, 40,000 of 50 K 14.4 / 15.6, 17,000 of 1 M 14.9 / 15.5.  Two tables by two clusters each: 65,536 of 2 M rows 18.1 / 18.6,
+// 30,000 of 1500 13.9 / 13.2, so they have one each.  Clusters of eight as parts: 28.9 (four), 40.3 (sixteen)
+int table_parts(const dqrm_ctx *ctx)
+{
+    return 2 * ctx->T * csort::CLUSTER_WIDE * csort::MAX_PARTS <= ctx->num_sms ? csort::MAX_PARTS : 1;
 }
 
 // clusters that stand by for tables beyond what their first block takes
@@ -432,13 +442,13 @@ size_t dq_sum_align(const dqrm_ctx *ctx)
 // segment starts).  It needs no upstream gradient, so a training step runs it beside the forward.
 int dq_launch_bwd_sort(dqrm_ctx *ctx, const int32_t *indices, const int32_t *offsets,
                        int32_t *unique_rows, int32_t *uniq_off, int B, int64_t L,
-                       void *ws_, size_t ws_bytes, cudaStream_t st, bool lists_by_table, bool *by_table)
+                       void *ws_, size_t ws_bytes, cudaStream_t st, bool lists_by_table, int *by_table)
 {
     const Layout y = make_layout(ctx, L);
     if (ws_bytes < y.total) return DQRM_ERR_WORKSPACE;
     char *ws = reinterpret_cast<char *>(ws_);
     const int64_t G = (int64_t)ctx->T * B;
-    if (by_table) *by_table = false;
+    if (by_table) *by_table = 0;
     const bool fits_cluster = (L + ctx->T - 1) / ctx->T <= (int64_t)csort::CLUSTER * 12288;   // (a table beyond its
     // blocks' shared memory still sorts, through global staging, but slowly)
     const bool try_cluster = ctx->sort_path != 1 && fits_cluster;
@@ -452,6 +462,7 @@ int dq_launch_bwd_sort(dqrm_ctx *ctx, const int32_t *indices, const int32_t *off
     uint2 *pairs[2] = {reinterpret_cast<uint2 *>(ws + y.pairs_a), reinterpret_cast<uint2 *>(ws + y.pairs_b)};
     const u32 *skeys = nullptr;      // sorted keys; the sorted payloads sit beside them in vals[0]
     bool sorted = false;
+    int parts = 1;                   // clusters, and so lists, of a table
     // (tables far beyond the shared-memory slices sort faster with the global radix sort)
     if (try_cluster) {
         if (!lists_by_table) {
@@ -479,25 +490,32 @@ int dq_launch_bwd_sort(dqrm_ctx *ctx, const int32_t *indices, const int32_t *off
         ca.absmax = reinterpret_cast<u32 *>(ws + y.absmax);
         ca.ck_shift = y.sum_shift;
         ca.cnt_broken = segred::CNT_BROKEN;
+        ca.parts = 1;
         const int64_t per_table = (L + ctx->T - 1) / ctx->T;
         cudaError_t e = cudaErrorUnknown;
         if (lists_by_table && launch_small_sort(ctx, ca, per_table, L == G, st, e)) {
             if (e == cudaSuccess) {
                 dq_mark(ctx, st, L == G ? DQ_K_SMALL_SORT : DQ_K_CLUSTER_SORT);
-                if (by_table) *by_table = true;
+                if (by_table) *by_table = 1;
                 return DQRM_OK;
             }
             ctx->last_cuda_error = (int)e;         // (taken off the runtime, so that nobody finds it behind the sort that follows)
             (void)cudaGetLastError();
         }
         const bool wide = ctx->T * csort::CLUSTER_WIDE * 2 <= ctx->num_sms && per_table >= csort::CLUSTER_WIDE * 1024;
-        if (wide) e = launch_cluster_sort<csort::CLUSTER_WIDE>(ctx, ca, csort::choose_cap(per_table, csort::CLUSTER_WIDE), st);
-        else e = cudaErrorUnknown;
+        e = cudaErrorUnknown;
+        if (wide && lists_by_table) {
+            ca.parts = table_parts(ctx);
+            if (ca.parts > 1) e = launch_cluster_sort<csort::CLUSTER_WIDE, true>(ctx, ca, csort::choose_cap(per_table, csort::CLUSTER_WIDE), st);
+            if (e != cudaSuccess) ca.parts = 1;
+        }
+        if (wide && e != cudaSuccess) e = launch_cluster_sort<csort::CLUSTER_WIDE>(ctx, ca, csort::choose_cap(per_table, csort::CLUSTER_WIDE), st);
         if (e != cudaSuccess) e = launch_cluster_sort<csort::CLUSTER>(ctx, ca, csort::choose_cap(per_table, csort::CLUSTER), st);
         if (e == cudaSuccess) {
             dq_mark(ctx, st, DQ_K_CLUSTER_SORT);
             skeys = keys[0];
             sorted = true;
+            parts = ca.parts;
         } else {
             ctx->last_cuda_error = (int)e;
         }
@@ -519,7 +537,7 @@ int dq_launch_bwd_sort(dqrm_ctx *ctx, const int32_t *indices, const int32_t *off
         skeys = keys[0];
     }
     if (sorted && lists_by_table) {                    // the lists are there; unique_rows and uniq_off come with the sums
-        if (by_table) *by_table = true;
+        if (by_table) *by_table = parts;
         return DQRM_OK;
     }
     if (!sorted) {        // (a cluster sort that did not number the segments itself has counted the segment heads of every tile)
@@ -537,7 +555,7 @@ int dq_launch_bwd_sort(dqrm_ctx *ctx, const int32_t *indices, const int32_t *off
 
 // second half: segmented sum of the upstream gradient over the sorted lookups
 int dq_launch_bwd_sum(dqrm_ctx *ctx, const float *grad_out, int32_t *unique_rows, int32_t *uniq_off, float *grad_rows,
-                      int B, int64_t L, bool by_table, void *ws_, size_t ws_bytes, cudaStream_t st)
+                      int B, int64_t L, int by_table, void *ws_, size_t ws_bytes, cudaStream_t st)
 {
     const Layout y = make_layout(ctx, L);
     if (ws_bytes < y.total) return DQRM_ERR_WORKSPACE;
@@ -552,6 +570,7 @@ int dq_launch_bwd_sum(dqrm_ctx *ctx, const float *grad_out, int32_t *unique_rows
     a.chunk_first = reinterpret_cast<const u32 *>(ws + y.chunk_first);
     a.range_done = reinterpret_cast<uint2 *>(ws + y.tile_done);
     a.by_table = by_table ? 1 : 0;
+    while ((1 << a.parts_log) < by_table) ++a.parts_log;
     a.table_cnt = reinterpret_cast<const u32 *>(ws + y.table_cnt);
     a.tb = reinterpret_cast<const u32 *>(ws + y.tb);
     a.row_off = ctx->d_row_off;
@@ -560,7 +579,7 @@ int dq_launch_bwd_sum(dqrm_ctx *ctx, const float *grad_out, int32_t *unique_rows
     a.partials = reinterpret_cast<double *>(ws + y.partials);
     a.group_partials = reinterpret_cast<double *>(ws + y.group_partials);
     a.absmax = reinterpret_cast<u32 *>(ws + y.absmax);
-    a.T = ctx->T; a.D = ctx->D;
+    a.T = ctx->T << a.parts_log; a.D = ctx->D;
     a.L = L; a.G = (int64_t)ctx->T * B;
     a.num_tiles = y.sum_tiles;
     a.range_tiles = y.range_tiles;
@@ -628,7 +647,7 @@ int dq_launch_bwd(dqrm_ctx *ctx, const float *grad_out, const int32_t *indices, 
                   int32_t *unique_rows, int32_t *uniq_off, float *grad_rows, int B, int64_t L,
                   void *ws, size_t ws_bytes, cudaStream_t st)
 {
-    bool by_table = false;
+    int by_table = 0;
     int rc = dq_launch_bwd_sort(ctx, indices, offsets, unique_rows, uniq_off, B, L, ws, ws_bytes, st, true, &by_table);
     if (rc != DQRM_OK) return rc;
     return dq_launch_bwd_sum(ctx, grad_out, unique_rows, uniq_off, grad_rows, B, L, by_table, ws, ws_bytes, st);

@@ -23,6 +23,7 @@ namespace csort {
 
 constexpr int CLUSTER = 8;            // blocks per table
 constexpr int CLUSTER_WIDE = 16;      // ... when the batch has so few tables that eight blocks each would leave most SMs idle
+constexpr int MAX_PARTS = 4;           // ... of such clusters for a table alone, which would leave more of them idle still
 
 __device__ __forceinline__ u32 *remote(cg::cluster_group &cluster, u32 *p, unsigned rank)
 {
@@ -42,7 +43,12 @@ __device__ __forceinline__ u32 same_digit_lanes(u32 d, bool valid)
 // the cluster.  Which block that is goes round the tables: from the sixteenth on clusters share their SMs with earlier ones, and two
 // working blocks on one SM take half as long again (26 tables of 2000 lookups: 11.5 us with the first block working in every
 // cluster, 8.2 this way, 8.5 without clusters; from 33 tables on 11.5, a third cluster waiting for its SMs).
-template <int CL, int EPT>
+//
+// PARTS: few tables, of which one cluster each would leave most SMs idle.  a.parts clusters take a table, each a share of its rows: every one
+// reads all the table's lookups and keeps those of its rows, so nothing passes between the clusters; where its lookups stand behind those
+// of the rows before it counts itself, and its segments have lists of their own.  Rows are shared out evenly, lookups need not fall so: in the worst case
+// one cluster sorts them all, as it would alone.  A table beyond the blocks' shared memory is its first cluster's.
+template <int CL, int EPT, bool PARTS>
 __device__ __forceinline__ void sort_by_cluster(const Args &a)
 {
     extern __shared__ __align__(16) uint2 s_dyn[];               // pair buffers [2][cap]: (row within table, payload)
@@ -52,18 +58,26 @@ __device__ __forceinline__ void sort_by_cluster(const Args &a)
     __shared__ u32 s_wheads[WARPS];                // write-out: segment starts in each warp's part of the slice
     __shared__ u32 s_totals[16];                   // ... and in every block's slice (each block sends its own)
     __shared__ u32 s_cbase, s_ctotal;              // ... in the blocks before this one, and in the whole table
+    __shared__ u32 s_kept[2], s_below[PARTS ? WARPS : 1];      // PARTS: the block's lookups in the cluster's rows and in rows before them
+    __shared__ u32 s_sum[2];                       // ... the cluster's
 
     cg::cluster_group cluster = cg::this_cluster();
     const unsigned c = cluster.block_rank();
-    const int t = blockIdx.x / CL;
+    const int list = blockIdx.x / CL, t = PARTS ? list / a.parts : list, part = PARTS ? list % a.parts : 0;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const u32 lt = (1u << lane) - 1u;
 
     const int64_t tb0 = __ldg(a.offsets + (int64_t)t * a.B), tb1 = __ldg(a.offsets + (int64_t)(t + 1) * a.B);
     const int64_t r0 = __ldg(a.row_off + t), nrows = __ldg(a.row_off + t + 1) - r0;
-    if (broken_table(a, t, tb0, tb1, c == 0 && threadIdx.x == 0)) return;         // uniform over the cluster
+    if (broken_table(a, t, list, tb0, tb1, c == 0 && threadIdx.x == 0)) return;   // uniform over the cluster
     const int64_t n = tb1 - tb0;
-    if (a.lists_by_table && c == 0 && threadIdx.x == 0) open_table(a, t, tb0, tb1);
+    if (PARTS) {
+        if (c == 0 && threadIdx.x == 0) {
+            if (part == 0) a.absmax[t] = 0u;
+            if (list + 1 == a.T * a.parts) a.tb[list + 1] = (u32)tb1;
+            if (n == 0) { a.tb[list] = (u32)tb0; a.table_cnt[list] = 0u; }
+        }
+    } else if (a.lists_by_table && c == 0 && threadIdx.x == 0) open_table(a, t, tb0, tb1);
     if constexpr (EPT > 0) {
         if (n <= THREADS * EPT) {
             if (c == (unsigned)(t / 3) % CL) sort_alone<EPT>(a, t, (u32)tb0, (u32)tb1, &s_cnt[0][0], s_dyn);
@@ -71,12 +85,16 @@ __device__ __forceinline__ void sort_by_cluster(const Args &a)
         }
     }
     if (n == 0) return;
-    const int npc = (int)(((n + CL - 1) / CL + 31) / 32 * 32);      // pairs per block
+    int npc = (int)(((n + CL - 1) / CL + 31) / 32 * 32);            // pairs per block
     const bool in_smem = npc <= a.cap;
-    const int my_n = (int)max((int64_t)0, min((int64_t)npc, n - (int64_t)c * npc));
+    int my_n = (int)max((int64_t)0, min((int64_t)npc, n - (int64_t)c * npc));
     // the scatter divides every destination by npc: a float reciprocal gives the quotient (a block number,
     // since pos < n <= CL * npc) to within one, and one correction step settles it
-    const float npc_inv = 1.0f / (float)npc;
+    float npc_inv = 1.0f / (float)npc;
+    // the cluster's rows, its lookups and their place among the sorted ones (PARTS: known behind the first barrier)
+    const int64_t row0 = PARTS && in_smem ? nrows * part / a.parts : 0;
+    const int64_t row1 = PARTS ? (in_smem ? nrows * (part + 1) / a.parts : part == 0 ? nrows : 0) : nrows;
+    int64_t m = n, first = tb0;
 
     // buffers of this block for stage s (shared memory slices, or this block's part of the global staging)
     // a pair travels as one 8-byte store: distributed-shared-memory traffic is bound by the number of stores
@@ -103,42 +121,103 @@ __device__ __forceinline__ void sort_by_cluster(const Args &a)
         (__ldg(a.offsets) != 0 || (int64_t)__ldg(a.offsets + (int64_t)a.T * a.B) != a.L))
         dq_report(a.status, DQRM_ERR_INDEX_RANGE);
     bool bad = false;
-    for (int i0 = threadIdx.x; i0 < my_n; i0 += 4 * THREADS) {
-        int32_t idx[4], o0[4], o1[4];              // (four lookups in flight: one at a time, 34 us instead of 32 for 26 tables of 16 K)
+    if constexpr (PARTS) {
+        // each warp has a contiguous part of the slice: it counts its lookups that are kept, then puts them behind those of the warps before
+        const int wsz = ((my_n + WARPS - 1) / WARPS + 31) / 32 * 32, w0 = min(my_n, warp * wsz), w1 = min(my_n, w0 + wsz);
+        const int32_t *idx_c = a.indices + tb0 + (int64_t)c * npc;
+        u32 kept = 0, below = 0;
+        for (int i0 = w0; i0 < w1; i0 += 8 * 32) {
+            int32_t idx[8];
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            const int64_t p = (int64_t)c * npc + min(i0 + k * THREADS, my_n - 1);      // position within the table's lookups
-            idx[k] = __ldg(a.indices + tb0 + p);
-            o0[k] = n == a.B ? __ldg(off_t + p) : 1;
-            o1[k] = n == a.B ? __ldg(off_t + p + 1) : 1;
-        }
+            for (int k = 0; k < 8; ++k) idx[k] = __ldg(idx_c + min(i0 + k * 32 + lane, my_n - 1));
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            const int i = i0 + k * THREADS;
-            if (i >= my_n) break;
-            const int64_t p = (int64_t)c * npc + i;
-            const bool single = o0[k] == tb0 + p && o1[k] == tb0 + p + 1;
-            bad |= (o0[k] > o1[k]) | (idx[k] < 0) | (idx[k] >= nrows);
-            int64_t bag = p;
-            if (!single || n != a.B) {             // largest bag b with offsets[t*B + b] <= tb0 + p
-                int lo = 0, hi = a.B;
-                while (hi - lo > 1) {
-                    const int mid = (lo + hi) >> 1;
-                    if ((int64_t)__ldg(off_t + mid) <= tb0 + p) lo = mid; else hi = mid;
-                }
-                bag = lo;
+            for (int k = 0; k < 8; ++k) {
+                const bool valid = i0 + k * 32 + lane < w1;
+                const int64_t row = min((int64_t)max(idx[k], 0), nrows - 1);
+                kept += __popc(__ballot_sync(0xffffffffu, valid && row >= row0 && row < row1));
+                below += __popc(__ballot_sync(0xffffffffu, valid && row < row0));
             }
-            pb0[i] = make_uint2((u32)min((int64_t)max(idx[k], 0), nrows - 1), a.payload_position ? (u32)(tb0 + p) : (u32)(bag * a.T + t));
+        }
+        if (lane == 0) { s_wheads[warp] = kept; s_below[warp] = below; }
+        __syncthreads();
+        u32 at = 0, all = 0, all_below = 0;
+#pragma unroll
+        for (int w = 0; w < WARPS; ++w) {
+            if (w < warp) at += s_wheads[w];
+            all += s_wheads[w];
+            all_below += s_below[w];
+        }
+        if (threadIdx.x == 0) { s_kept[0] = all; s_kept[1] = all_below; }
+        for (int i0 = w0; i0 < w1; i0 += 4 * 32) {
+            int32_t idx[4], o0[4], o1[4];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const int i = min(i0 + k * 32 + lane, my_n - 1);
+                idx[k] = __ldg(idx_c + i);
+                o0[k] = n == a.B ? __ldg(off_t + (int64_t)c * npc + i) : 1;
+                o1[k] = n == a.B ? __ldg(off_t + (int64_t)c * npc + i + 1) : 1;
+            }
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const bool valid = i0 + k * 32 + lane < w1;
+                const int64_t p = (int64_t)c * npc + i0 + k * 32 + lane, row = min((int64_t)max(idx[k], 0), nrows - 1);
+                const bool single = o0[k] == tb0 + p && o1[k] == tb0 + p + 1, in = valid && row >= row0 && row < row1;
+                bad |= valid && ((o0[k] > o1[k]) | (idx[k] < 0) | (idx[k] >= nrows));
+                const u32 in_mask = __ballot_sync(0xffffffffu, in), to = at + __popc(in_mask & lt);
+                at += __popc(in_mask);
+                if (in) {
+                    int64_t bag = p;
+                    if (!single || n != a.B) {     // (as below)
+                        int lo = 0, hi = a.B;
+                        while (hi - lo > 1) {
+                            const int mid = (lo + hi) >> 1;
+                            if ((int64_t)__ldg(off_t + mid) <= tb0 + p) lo = mid; else hi = mid;
+                        }
+                        bag = lo;
+                    }
+                    pb0[to] = make_uint2((u32)(row - row0), a.payload_position ? (u32)(tb0 + p) : (u32)(bag * a.T + t));
+                }
+            }
+        }
+        my_n = (int)all;
+    } else {
+        for (int i0 = threadIdx.x; i0 < my_n; i0 += 4 * THREADS) {
+            int32_t idx[4], o0[4], o1[4];              // (four lookups in flight: one at a time, 34 us instead of 32 for 26 tables of 16 K)
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const int64_t p = (int64_t)c * npc + min(i0 + k * THREADS, my_n - 1);      // position within the table's lookups
+                idx[k] = __ldg(a.indices + tb0 + p);
+                o0[k] = n == a.B ? __ldg(off_t + p) : 1;
+                o1[k] = n == a.B ? __ldg(off_t + p + 1) : 1;
+            }
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const int i = i0 + k * THREADS;
+                if (i >= my_n) break;
+                const int64_t p = (int64_t)c * npc + i;
+                const bool single = o0[k] == tb0 + p && o1[k] == tb0 + p + 1;
+                bad |= (o0[k] > o1[k]) | (idx[k] < 0) | (idx[k] >= nrows);
+                int64_t bag = p;
+                if (!single || n != a.B) {             // largest bag b with offsets[t*B + b] <= tb0 + p
+                    int lo = 0, hi = a.B;
+                    while (hi - lo > 1) {
+                        const int mid = (lo + hi) >> 1;
+                        if ((int64_t)__ldg(off_t + mid) <= tb0 + p) lo = mid; else hi = mid;
+                    }
+                    bag = lo;
+                }
+                pb0[i] = make_uint2((u32)min((int64_t)max(idx[k], 0), nrows - 1), a.payload_position ? (u32)(tb0 + p) : (u32)(bag * a.T + t));
+            }
         }
     }
     if (bad) dq_report(a.status, DQRM_ERR_INDEX_RANGE);
 
     int bits = 0;
-    while (((int64_t)1 << bits) < nrows) ++bits;
-    const int passes = (bits + 7) / 8;
+    while (((int64_t)1 << bits) < row1 - row0) ++bits;
+    const int passes = PARTS ? max(1, (bits + 7) / 8) : (bits + 7) / 8;      // (PARTS: the first pass also shares the lookups out over the blocks)
     // the slice of this block is cut into WARPS contiguous parts, walked 32 entries at a time
-    const int wsz = ((my_n + WARPS - 1) / WARPS + 31) / 32 * 32;
-    const int w0 = min(my_n, warp * wsz), w1 = min(my_n, w0 + wsz);
+    int wsz = ((my_n + WARPS - 1) / WARPS + 31) / 32 * 32;
+    int w0 = min(my_n, warp * wsz), w1 = min(my_n, w0 + wsz);
 
     int s = 0;
     __syncthreads();
@@ -162,6 +241,25 @@ __device__ __forceinline__ void sort_by_cluster(const Args &a)
             s_hist[threadIdx.x] = h;
         }
         cluster.sync();
+        if (PARTS && pass == 0) {
+            if (warp == WARPS - 1) {
+                u32 kept = lane < CL ? *remote(cluster, &s_kept[0], lane % CL) : 0u, below = lane < CL ? *remote(cluster, &s_kept[1], lane % CL) : 0u;
+                kept = __reduce_add_sync(0xffffffffu, kept);
+                below = __reduce_add_sync(0xffffffffu, below);
+                if (lane == 0) { s_sum[0] = kept; s_sum[1] = below; }
+            }
+            __syncthreads();
+            m = s_sum[0];
+            first = tb0 + (in_smem ? s_sum[1] : part == 0 ? 0u : (u32)n);
+            npc = (int)(((m + CL - 1) / CL + 31) / 32 * 32);
+            npc_inv = 1.0f / (float)npc;
+            if (c == 0 && threadIdx.x == 0) a.tb[list] = (u32)first;
+            if (m == 0) {                          // (uniform over the cluster)
+                if (c == 0 && threadIdx.x == 0) a.table_cnt[list] = 0u;
+                cluster.sync();                    // nobody leaves while its shared memory is read
+                return;
+            }
+        }
         // offsets: digits first, then blocks of the cluster, then warps of this block
         u32 tot = 0, pre = 0, incl = 0;
         if (threadIdx.x < BINS) {                  // one thread per digit (the first BINS / 32 warps)
@@ -206,7 +304,7 @@ __device__ __forceinline__ void sort_by_cluster(const Args &a)
             __syncwarp();
             if (valid) {
                 const u32 pos = base + __popc(peers & lt);      // position within the table, < n
-                if ((int64_t)pos < n) {
+                if ((int64_t)pos < m) {
                     if (in_smem) {
                         unsigned owner = (unsigned)((float)pos * npc_inv);       // within one of pos / npc
                         if (owner * (u32)npc > pos) --owner;
@@ -221,6 +319,12 @@ __device__ __forceinline__ void sort_by_cluster(const Args &a)
         }
         cluster.sync();
         s ^= 1;
+        if (PARTS && pass == 0) {
+            my_n = (int)max((int64_t)0, min((int64_t)npc, m - (int64_t)c * npc));
+            wsz = ((my_n + WARPS - 1) / WARPS + 31) / 32 * 32;
+            w0 = min(my_n, warp * wsz);
+            w1 = min(my_n, w0 + wsz);
+        }
     }
     // ---- write the sorted slice: arena row keys ----
     // and either count, per 2048-entry tile of the sorted order, the entries that start a new row, or number the
@@ -266,9 +370,9 @@ __device__ __forceinline__ void sort_by_cluster(const Args &a)
                 const int i = i0 + lane;
                 bool head = false;
                 if (i < w1) {
-                    const int64_t j = tb0 + (int64_t)c * npc + i;
+                    const int64_t j = first + (int64_t)c * npc + i;
                     const uint2 pr = fin[i];
-                    a.keys_out[j] = (u32)(r0 + pr.x);
+                    a.keys_out[j] = (u32)(r0 + row0 + pr.x);
                     a.vals_out[j] = pr.y;
                     const u32 before = i > 0 ? fin[i - 1].x : prev_last;
                     head = (c == 0 && i == 0) || before != pr.x;
@@ -306,16 +410,16 @@ __device__ __forceinline__ void sort_by_cluster(const Args &a)
             }
             __syncthreads();
             const u32 base = s_cbase, total = s_ctotal;
-            u32 *segs = a.seg_start + tb0 + t;
+            u32 *segs = a.seg_start + first + list;
             if (c == 0 && threadIdx.x == 0) {
-                a.table_cnt[t] = total;
-                segs[total] = (u32)tb1;            // the slot behind the last segment holds the table's end
+                a.table_cnt[list] = total;
+                segs[total] = (u32)(first + m);    // the slot behind the last segment holds the table's end
             }
             const u32 ck_mask = (1u << a.ck_shift) - 1u;
             u32 before_me = base + s_wheads[warp];
             for (int i0 = w0, it = 0; i0 < w1; i0 += 32, ++it) {
                 const int i = i0 + lane;
-                const int64_t j = tb0 + (int64_t)c * npc + i;
+                const int64_t j = first + (int64_t)c * npc + i;
                 u32 m;
                 if (few) {
                     m = __shfl_sync(0xffffffffu, kept, it);
@@ -351,12 +455,12 @@ __device__ __forceinline__ void sort_by_cluster(const Args &a)
 // of 64 K lookups
 __host__ __device__ constexpr int resident(int CL) { return CL == CLUSTER ? 2 : 1; }
 
-template <int CL, int EPT>
+template <int CL, int EPT, bool PARTS = false>
 __global__ void __launch_bounds__(THREADS, resident(CL))
 cluster_sort_kernel(const __grid_constant__ Args a)
 {
     dq_wait_before();
-    sort_by_cluster<CL, EPT>(a);
+    sort_by_cluster<CL, EPT, PARTS>(a);
 }
 
 inline size_t smem_bytes(int cap) { return (size_t)2 * cap * sizeof(uint2); }

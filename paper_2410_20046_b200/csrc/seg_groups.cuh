@@ -117,7 +117,7 @@ seg_groups_kernel(const __grid_constant__ Args a)
             broken = __any_sync(0xffffffffu, broken);
             if (wl == 0) { s_uoff[T] = run; s_broken = broken; }
         } else {
-            for (int t = threadIdx.x - 32; t <= T; t += threads - 32) { s_tb[t] = __ldg(a.tb + t); s_row[t] = (u32)__ldg(a.row_off + t); }
+            for (int t = threadIdx.x - 32; t <= T; t += threads - 32) { s_tb[t] = __ldg(a.tb + t); s_row[t] = (u32)__ldg(a.row_off + (t >> a.parts_log)); }
         }
     } else {
         for (int t = threadIdx.x; t <= T; t += threads) s_uoff[t] = (u32)__ldg(a.uniq_off + t);
@@ -125,7 +125,7 @@ seg_groups_kernel(const __grid_constant__ Args a)
     }
     __syncthreads();
     if (a.by_table && blockIdx.x == 0)
-        for (int t = threadIdx.x; t <= T; t += threads) a.uniq_off[t] = s_broken ? 0 : (int32_t)s_uoff[t];
+        for (int t = threadIdx.x; t <= T >> a.parts_log; t += threads) a.uniq_off[t] = s_broken ? 0 : (int32_t)s_uoff[t << a.parts_log];
     if (s_broken || w0 >= w1) return;             // (warp-uniform; no block barrier below)
 
     // a one-index batch reads every upstream-gradient row once, a pooled one as often as the bag has indices
@@ -178,7 +178,7 @@ seg_groups_kernel(const __grid_constant__ Args a)
     const u32 u_in = u;
     u32 t_end = s_uoff[t + 1], t_row = a.by_table ? s_row[t] : 0u;
     float m = 0.f;                                // abs-max of the rows of table t that this lane has rounded
-    auto note = [&](int tt, float x) { if (x > 0.f) atomicMax(a.absmax + tt, __float_as_uint(x)); };
+    auto note = [&](int tt, float x) { if (x > 0.f) atomicMax(a.absmax + (tt >> a.parts_log), __float_as_uint(x)); };
     auto store_row = [&](u32 uu, const double (&acc)[4]) {
         float x = 0.f;
         if (on) {
@@ -302,7 +302,7 @@ seg_groups_kernel(const __grid_constant__ Args a)
         const int t_first = __shfl_sync(0xffffffffu, t, 0);
         if (__all_sync(0xffffffffu, t == t_first)) {
             const u32 mb = __reduce_max_sync(0xffffffffu, __float_as_uint(m));
-            if (wl == 0 && mb) atomicMax(a.absmax + t_first, mb);
+            if (wl == 0 && mb) atomicMax(a.absmax + (t_first >> a.parts_log), mb);
         } else {
             note(t, m);
         }

@@ -76,7 +76,8 @@ struct Args {
     double *partials;           // [ranges][2][D]: run that enters the range, run that leaves it
     double *group_partials;     // [ranges / 32 + 1][2][D]: the same for groups of 32 ranges
     u32 *absmax;                // [T] zero
-    int T, D;
+    int T, D;                   // T: lists, 2^parts_log for every table (by_table; one otherwise)
+    int parts_log;
     int64_t L, G;
     int64_t num_tiles;          // rows that take a warp: tiles, tiles of a warp's range, blocks of 128 features
     int range_tiles, columns;
@@ -147,10 +148,10 @@ __device__ __forceinline__ float4 rounded(const double (&a)[4], float &mx)
 
 // abs-max of a row where the tile holds rows of several tables (rare in large batches: kept out of the unrolled code).
 // Called by the warp together.
-__device__ __noinline__ void note_max(u32 *absmax, const u32 *s_uoff, int t_first, int T, u32 u, float x)
+__device__ __noinline__ void note_max(u32 *absmax, const u32 *s_uoff, int t_first, int T, int parts_log, u32 u, float x)
 {
     const u32 m = __reduce_max_sync(0xffffffffu, __float_as_uint(x));
-    if ((threadIdx.x & 31) == 0 && m) atomicMax(absmax + last_not_above(s_uoff, t_first, T, u), m);
+    if ((threadIdx.x & 31) == 0 && m) atomicMax(absmax + (last_not_above(s_uoff, t_first, T, u) >> parts_log), m);
 }
 
 // blockIdx.x * WARPS + warp: range of tiles and block of 128 features (COLS: D > 128, there are several).  EXACT: every lane
@@ -223,7 +224,7 @@ seg_sum_kernel(const Args a)
             broken = __any_sync(0xffffffffu, broken);
             if (wl == 0) { s_uoff[T] = run; s_broken = broken; }
         } else {
-            for (int t = threadIdx.x - 32; t <= T; t += THREADS - 32) { s_tb[t] = a.tb[t]; s_row[t] = (u32)a.row_off[t]; }
+            for (int t = threadIdx.x - 32; t <= T; t += THREADS - 32) { s_tb[t] = a.tb[t]; s_row[t] = (u32)a.row_off[t >> a.parts_log]; }
         }
     } else {
         for (int t = threadIdx.x; t <= T; t += THREADS) s_uoff[t] = (u32)a.uniq_off[t];
@@ -231,7 +232,7 @@ seg_sum_kernel(const Args a)
     }
     __syncthreads();
     if (a.by_table && blockIdx.x == 0)
-        for (int t = threadIdx.x; t <= T; t += THREADS) a.uniq_off[t] = s_broken ? 0 : (int32_t)s_uoff[t];
+        for (int t = threadIdx.x; t <= T >> a.parts_log; t += THREADS) a.uniq_off[t] = s_broken ? 0 : (int32_t)s_uoff[t << a.parts_log];
     if (s_broken || tile0 >= tile1) return;       // (warp-uniform; no block barrier below)
 
     // a one-index batch reads every upstream-gradient row once, a pooled one as often as the bag has indices
@@ -272,7 +273,7 @@ seg_sum_kernel(const Args a)
     float m = 0.f;                                // abs-max of the rows of table t_max that this thread has rounded
     auto push_max = [&]() {
         const u32 mb = __reduce_max_sync(0xffffffffu, __float_as_uint(m));
-        if (wl == 0 && mb) atomicMax(a.absmax + t_max, mb);
+        if (wl == 0 && mb) atomicMax(a.absmax + (t_max >> a.parts_log), mb);
         m = 0.f;
     };
     // rounds a finished sum and writes it; leaves a piece of a cut run (called by all lanes of a group)
@@ -280,7 +281,7 @@ seg_sum_kernel(const Args a)
         float x = 0.f;
         if (on) st_row(reinterpret_cast<vec_t *>(a.grad_rows + (int64_t)u * D) + cv, rounded(acc, x), keep);  // quantise+update reads it next
         if (one_table) m = fmaxf(m, x);
-        else note_max(a.absmax, s_uoff, t_first, T, u, x);
+        else note_max(a.absmax, s_uoff, t_first, T, a.parts_log, u, x);
     };
     auto store_piece = [&](int slot, const double (&acc)[VEC]) {
         if (on) {
@@ -391,7 +392,7 @@ seg_sum_kernel(const Args a)
     auto store_total = [&](u32 u, int cc, const double (&sum)[VEC]) {
         float x = 0.f;
         if (EXACT || cc < dv) st_row(reinterpret_cast<vec_t *>(a.grad_rows + (int64_t)u * D) + cc, rounded(sum, x), keep);
-        note_max(a.absmax, s_uoff, 0, T, u, x);
+        note_max(a.absmax, s_uoff, 0, T, a.parts_log, u, x);
     };
 #pragma unroll 1
     for (int q = 0; q < 2; ++q) {                 // (columns: all of them, the blocks of the others are done too)

@@ -288,7 +288,7 @@ __device__ __forceinline__ void sort_by_block(const csort::Args &a)
     __shared__ __align__(16) u32 s_cnt[csort::WARPS * csort::BINS];
     const int t = blockIdx.x;
     const int64_t tb0 = __ldg(a.offsets + (int64_t)t * a.B), tb1 = __ldg(a.offsets + (int64_t)(t + 1) * a.B);
-    if (csort::broken_table(a, t, tb0, tb1, threadIdx.x == 0)) return;
+    if (csort::broken_table(a, t, t, tb0, tb1, threadIdx.x == 0)) return;
     if (threadIdx.x == 0) csort::open_table(a, t, tb0, tb1);
     const int64_t n = tb1 - tb0;
     if (n <= csort::THREADS * E) {
@@ -309,7 +309,7 @@ __global__ void __launch_bounds__(THREADS, CL > 1 ? csort::resident(CL) : 0)
 small_sort_kernel(const __grid_constant__ csort::Args a)
 {
     dq_wait_before();
-    if constexpr (CL > 1) csort::sort_by_cluster<CL, E>(a);
+    if constexpr (CL > 1) csort::sort_by_cluster<CL, E, false>(a);
     else if constexpr (THREADS == csort::THREADS) sort_by_block<E>(a);
     else sort_by_network<THREADS>(a);
 }

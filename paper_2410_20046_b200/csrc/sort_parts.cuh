@@ -42,17 +42,19 @@ struct Args {
     uint2 *tile_done;
     int ck_shift;
     u32 cnt_broken;
+    int parts;                      // (cluster sort with the lists only) clusters of a table, each with its own share of the rows and its own
+                                    // lists, numbered table by table; a power of two
 };
 
 // a table whose boundary offsets cannot be used is reported and left out (the same answer in every thread)
-__device__ __forceinline__ bool broken_table(const Args &a, int t, int64_t tb0, int64_t tb1, bool reports)
+__device__ __forceinline__ bool broken_table(const Args &a, int t, int list, int64_t tb0, int64_t tb1, bool reports)
 {
     if (tb0 >= 0 && tb1 >= tb0 && tb1 <= a.L && !(a.lists_by_table && ((t == 0 && tb0 != 0) || (t == a.T - 1 && tb1 != a.L))))
         return false;
     if (reports) {
         dq_report(a.status, DQRM_ERR_INDEX_RANGE);
         if (a.lists_by_table) {                    // nothing is summed; the quantiser behind finds an empty gradient
-            a.table_cnt[t] = a.cnt_broken;
+            a.table_cnt[list] = a.cnt_broken;
             a.absmax[t] = 0u;
         }
     }

@@ -168,6 +168,34 @@ def test_lane_groups_of_many_rounds(oracle, D, B, sort_path):
     c.ctx.close()
 
 
+@pytest.mark.parametrize("D", [8, 64])
+@pytest.mark.parametrize("rows", [1, 3, 257, 70_001, 3_000_000])
+@pytest.mark.parametrize("where", ["all", "first", "last", "ends", "one"])
+def test_table_alone_by_its_parts(oracle, where, rows, D):
+    """A large table alone, whose rows four clusters share: lookups over all of them, in the first or the last share only (the
+    other lists stay empty), on the shares' edges, in one row; an index a bag and uneven bags."""
+    rng = np.random.default_rng(rows + D)
+    edges = sorted({min(max(rows * q // 4 + d, 0), rows - 1) for q in range(5) for d in (-1, 0, 1)})
+    for bags in (False, True):
+        B = 17_001 if not bags else 9_000
+        lens = rng.integers(0, 5, B) if bags else np.ones(B, dtype=np.int64)
+        L = int(lens.sum())
+        assert 16 * 1024 <= L
+        u = rng.random(L)
+        idx = {"all": u * rows, "first": u * max(1, rows // 4), "last": rows - 1 - u * max(1, rows // 4),
+               "ends": np.array(edges)[(u * len(edges)).astype(int)], "one": np.full(L, rows // 2)}[where].astype(np.int32).clip(0, rows - 1)
+        off = np.concatenate([[0], np.cumsum(lens)]).astype(np.int32)
+        go = rng.standard_normal((B, 1, D)).astype(np.float32)
+        c = Case(W.Workload("alone", (rows,), D=D, B=B, alpha=None), max_lookups=L)
+        ur, uo, gr = c.gpu_bwd(idx, off, go)
+        o_ur, o_uo, o_gr = oracle.emb_bwd(go, 1, D, B, idx, off)
+        assert bit_equal(uo, o_uo) and bit_equal(ur, o_ur)
+        # n terms of magnitude below 6 in FP64 in two orders, each sum rounded once
+        n = int(np.unique(idx, return_counts=True)[1].max())
+        np.testing.assert_allclose(gr, o_gr, rtol=2.0 ** -23, atol=12.0 * n * n * 2.0 ** -53)
+        c.ctx.close()
+
+
 # more than a dozen tiles of 32 for each of the 4736 warps that 148 SMs hold: ranges of eight tiles, several of them for a warp's place
 @pytest.mark.parametrize("D", [52, 64])
 @pytest.mark.parametrize("sort_path", [0, 1])
