@@ -459,8 +459,8 @@ int dqrm_sort_batch(dqrm_ctx *ctx, const int32_t *indices, const int32_t *offset
     if (!ws_ok(workspace, workspace_bytes, dq_bwd_ws_bytes(ctx, L, (int64_t)ctx->T * B))) return DQRM_ERR_WORKSPACE;
     cudaStream_t st = as_stream(stream);
     if (ctx->prof_on) dq_mark(ctx, st, DQ_K_BEGIN);
-    int by_table = 0;
-    const int rc = dq_launch_bwd_sort(ctx, indices, offsets, unique_rows, uniq_off, B, L, workspace, workspace_bytes, st, true, &by_table);
+    int lists = 0;
+    const int rc = dq_launch_bwd_sort(ctx, indices, offsets, unique_rows, uniq_off, B, L, workspace, workspace_bytes, st, true, nullptr, &lists);
     {
         std::lock_guard<std::mutex> lock(ctx->sorted_mu);
         dqrm_ctx::SortedBatch &sb = ctx->sorted[workspace];
@@ -475,7 +475,7 @@ int dqrm_sort_batch(dqrm_ctx *ctx, const int32_t *indices, const int32_t *offset
         sb.capture_id = id;
         sb.L = L;
         sb.B = B;
-        sb.by_table = by_table;
+        sb.lists = lists;
         sb.fresh = true;
     }
     return rc;
@@ -495,7 +495,7 @@ int dqrm_train_step_sorted(dqrm_ctx *ctx, float *tables, const int32_t *indices,
     if (!ws_ok(workspace, workspace_bytes, dq_bwd_ws_bytes(ctx, L, (int64_t)ctx->T * B))) return DQRM_ERR_WORKSPACE;
     cudaEvent_t sort_done = nullptr;
     bool sort_captured = false;
-    int by_table = 0;
+    int lists = 0;
     unsigned long long sort_capture_id = 0;
     {   // the workspace must hold this batch, sorted by dqrm_sort_batch and not consumed yet: the summation
         // trusts the segment lists in it and zeroes nothing itself
@@ -506,7 +506,7 @@ int dqrm_train_step_sorted(dqrm_ctx *ctx, float *tables, const int32_t *indices,
         it->second.fresh = false;
         sort_done = it->second.done;
         sort_captured = it->second.captured;
-        by_table = it->second.by_table;
+        lists = it->second.lists;
         sort_capture_id = it->second.capture_id;
     }
     cudaStream_t st = as_stream(stream);
@@ -528,7 +528,7 @@ int dqrm_train_step_sorted(dqrm_ctx *ctx, float *tables, const int32_t *indices,
         if (captured == sort_captured && (!captured || id == sort_capture_id))
             DQRM_CUDA_TRY(ctx, cudaStreamWaitEvent(ss, sort_done, 0));
     }
-    int rc = dq_launch_bwd_sum(ctx, grad_out, unique_rows, uniq_off, grad_rows, B, L, by_table, workspace,
+    int rc = dq_launch_bwd_sum(ctx, grad_out, unique_rows, uniq_off, grad_rows, B, L, lists, workspace,
                                workspace_bytes, ss);
     // The forward goes to the context's lowest-priority stream: its many blocks then do not keep the next batch's
     // sort, which a pipelined loop runs on a stream of its own, from getting SMs (with the forward on the caller's
@@ -695,8 +695,8 @@ int dqrm_train_step_host(dqrm_ctx *ctx, float *tables, const int32_t *h_indices,
     DQRM_CUDA_TRY(ctx, cudaStreamWaitEvent(ctx->side, ctx->ev_fork, 0));
     char *step_ws = ws + y.step_ws;
     const size_t step_ws_bytes = workspace_bytes - y.step_ws;
-    int by_table = 0;
-    int rc = dq_launch_bwd_sort(ctx, d_idx, d_off, d_ur, d_uo, B, L, step_ws, step_ws_bytes, ctx->side, true, &by_table);
+    int lists = 0;
+    int rc = dq_launch_bwd_sort(ctx, d_idx, d_off, d_ur, d_uo, B, L, step_ws, step_ws_bytes, ctx->side, true, nullptr, &lists);
     if (rc == DQRM_OK) rc = dq_launch_fwd(ctx, tables, d_idx, d_off, scales, bits, d_out, nullptr, B, L, st);
     // join every stream even after an error, so that the caller's stream stays ordered behind them
     cudaEventRecord(ctx->ev_h_fwd, st);
@@ -705,7 +705,7 @@ int dqrm_train_step_host(dqrm_ctx *ctx, float *tables, const int32_t *h_indices,
     cudaEventRecord(ctx->ev_h_out, ctx->copy_out);
     // the gradient summation follows the sort on the second stream as soon as the upstream gradient has arrived
     cudaStreamWaitEvent(ctx->side, ctx->ev_h_go, 0);
-    if (rc == DQRM_OK) rc = dq_launch_bwd_sum(ctx, d_go, d_ur, d_uo, d_gr, B, L, by_table, step_ws, step_ws_bytes, ctx->side);
+    if (rc == DQRM_OK) rc = dq_launch_bwd_sum(ctx, d_go, d_ur, d_uo, d_gr, B, L, lists, step_ws, step_ws_bytes, ctx->side);
     cudaEventRecord(ctx->ev_join, ctx->side);
     cudaStreamWaitEvent(st, ctx->ev_join, 0);
     if (rc == DQRM_OK)

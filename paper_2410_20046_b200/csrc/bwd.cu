@@ -442,13 +442,14 @@ size_t dq_sum_align(const dqrm_ctx *ctx)
 // segment starts).  It needs no upstream gradient, so a training step runs it beside the forward.
 int dq_launch_bwd_sort(dqrm_ctx *ctx, const int32_t *indices, const int32_t *offsets,
                        int32_t *unique_rows, int32_t *uniq_off, int B, int64_t L,
-                       void *ws_, size_t ws_bytes, cudaStream_t st, bool lists_by_table, int *by_table)
+                       void *ws_, size_t ws_bytes, cudaStream_t st, bool lists_by_table, bool *by_table, int *lists)
 {
     const Layout y = make_layout(ctx, L);
     if (ws_bytes < y.total) return DQRM_ERR_WORKSPACE;
     char *ws = reinterpret_cast<char *>(ws_);
     const int64_t G = (int64_t)ctx->T * B;
-    if (by_table) *by_table = 0;
+    if (by_table) *by_table = false;
+    if (lists) *lists = 0;
     const bool fits_cluster = (L + ctx->T - 1) / ctx->T <= (int64_t)csort::CLUSTER * 12288;   // (a table beyond its
     // blocks' shared memory still sorts, through global staging, but slowly)
     const bool try_cluster = ctx->sort_path != 1 && fits_cluster;
@@ -496,7 +497,8 @@ int dq_launch_bwd_sort(dqrm_ctx *ctx, const int32_t *indices, const int32_t *off
         if (lists_by_table && launch_small_sort(ctx, ca, per_table, L == G, st, e)) {
             if (e == cudaSuccess) {
                 dq_mark(ctx, st, L == G ? DQ_K_SMALL_SORT : DQ_K_CLUSTER_SORT);
-                if (by_table) *by_table = 1;
+                if (by_table) *by_table = true;
+                if (lists) *lists = 1;
                 return DQRM_OK;
             }
             ctx->last_cuda_error = (int)e;         // (taken off the runtime, so that nobody finds it behind the sort that follows)
@@ -504,7 +506,7 @@ int dq_launch_bwd_sort(dqrm_ctx *ctx, const int32_t *indices, const int32_t *off
         }
         const bool wide = ctx->T * csort::CLUSTER_WIDE * 2 <= ctx->num_sms && per_table >= csort::CLUSTER_WIDE * 1024;
         e = cudaErrorUnknown;
-        if (wide && lists_by_table) {
+        if (wide && lists_by_table && lists) {
             ca.parts = table_parts(ctx);
             if (ca.parts > 1) e = launch_cluster_sort<csort::CLUSTER_WIDE, true>(ctx, ca, csort::choose_cap(per_table, csort::CLUSTER_WIDE), st);
             if (e != cudaSuccess) ca.parts = 1;
@@ -537,7 +539,8 @@ int dq_launch_bwd_sort(dqrm_ctx *ctx, const int32_t *indices, const int32_t *off
         skeys = keys[0];
     }
     if (sorted && lists_by_table) {                    // the lists are there; unique_rows and uniq_off come with the sums
-        if (by_table) *by_table = parts;
+        if (by_table) *by_table = true;
+        if (lists) *lists = parts;
         return DQRM_OK;
     }
     if (!sorted) {        // (a cluster sort that did not number the segments itself has counted the segment heads of every tile)
@@ -555,7 +558,7 @@ int dq_launch_bwd_sort(dqrm_ctx *ctx, const int32_t *indices, const int32_t *off
 
 // second half: segmented sum of the upstream gradient over the sorted lookups
 int dq_launch_bwd_sum(dqrm_ctx *ctx, const float *grad_out, int32_t *unique_rows, int32_t *uniq_off, float *grad_rows,
-                      int B, int64_t L, int by_table, void *ws_, size_t ws_bytes, cudaStream_t st)
+                      int B, int64_t L, int lists, void *ws_, size_t ws_bytes, cudaStream_t st)
 {
     const Layout y = make_layout(ctx, L);
     if (ws_bytes < y.total) return DQRM_ERR_WORKSPACE;
@@ -569,8 +572,8 @@ int dq_launch_bwd_sum(dqrm_ctx *ctx, const float *grad_out, int32_t *unique_rows
     a.seg_start = reinterpret_cast<const u32 *>(ws + y.seg_start);
     a.chunk_first = reinterpret_cast<const u32 *>(ws + y.chunk_first);
     a.range_done = reinterpret_cast<uint2 *>(ws + y.tile_done);
-    a.by_table = by_table ? 1 : 0;
-    while ((1 << a.parts_log) < by_table) ++a.parts_log;
+    a.by_table = lists > 0;
+    while ((1 << a.parts_log) < lists) ++a.parts_log;
     a.table_cnt = reinterpret_cast<const u32 *>(ws + y.table_cnt);
     a.tb = reinterpret_cast<const u32 *>(ws + y.tb);
     a.row_off = ctx->d_row_off;
@@ -647,8 +650,8 @@ int dq_launch_bwd(dqrm_ctx *ctx, const float *grad_out, const int32_t *indices, 
                   int32_t *unique_rows, int32_t *uniq_off, float *grad_rows, int B, int64_t L,
                   void *ws, size_t ws_bytes, cudaStream_t st)
 {
-    int by_table = 0;
-    int rc = dq_launch_bwd_sort(ctx, indices, offsets, unique_rows, uniq_off, B, L, ws, ws_bytes, st, true, &by_table);
+    int lists = 0;
+    int rc = dq_launch_bwd_sort(ctx, indices, offsets, unique_rows, uniq_off, B, L, ws, ws_bytes, st, true, nullptr, &lists);
     if (rc != DQRM_OK) return rc;
-    return dq_launch_bwd_sum(ctx, grad_out, unique_rows, uniq_off, grad_rows, B, L, by_table, ws, ws_bytes, st);
+    return dq_launch_bwd_sum(ctx, grad_out, unique_rows, uniq_off, grad_rows, B, L, lists, ws, ws_bytes, st);
 }

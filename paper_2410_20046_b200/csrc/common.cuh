@@ -51,7 +51,7 @@ struct dqrm_ctx {
         int64_t L = 0;
         int B = 0;
         cudaEvent_t done = nullptr;
-        int by_table = 0;               // how the sort left its lists (dq_launch_bwd_sort)
+        int lists = 0;                  // how the sort left its lists: so many for each table, 0: over the batch (dq_launch_bwd_sort)
         bool captured = false;
         unsigned long long capture_id = 0;
     };
@@ -388,13 +388,13 @@ int dq_launch_bwd(dqrm_ctx *ctx, const float *grad_out, const int32_t *indices, 
                   void *ws, size_t ws_bytes, cudaStream_t st);
 
 // lists_by_table: dq_launch_bwd_sum follows on the same workspace; the cluster sort then numbers each table's
-// segments itself (*by_table says how many lists each table then has, 0 if it did not), no separate kernel numbers them over the batch, and unique_rows /
+// segments itself (*by_table says whether it did; *lists, without which it is one, how many lists each table then has), no separate kernel numbers them over the batch, and unique_rows /
 // uniq_off are written by dq_launch_bwd_sum.  Without it they are complete when the sort is.
 int dq_launch_bwd_sort(dqrm_ctx *ctx, const int32_t *indices, const int32_t *offsets, int32_t *unique_rows,
                        int32_t *uniq_off, int B, int64_t L, void *ws, size_t ws_bytes, cudaStream_t st,
-                       bool lists_by_table, int *by_table);
+                       bool lists_by_table, bool *by_table, int *lists = nullptr);
 int dq_launch_bwd_sum(dqrm_ctx *ctx, const float *grad_out, int32_t *unique_rows, int32_t *uniq_off, float *grad_rows,
-                      int B, int64_t L, int by_table, void *ws, size_t ws_bytes, cudaStream_t st);
+                      int B, int64_t L, int lists, void *ws, size_t ws_bytes, cudaStream_t st);
 
 size_t dq_quant_ws_bytes(const dqrm_ctx *ctx);
 int dq_launch_grad_absmax(dqrm_ctx *ctx, const float *grad_rows, const int32_t *uniq_off, float *absmax,
