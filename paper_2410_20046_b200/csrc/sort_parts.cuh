@@ -38,12 +38,12 @@ struct Args {
     // and zeroes what the kernel behind it counts in (tile_done[c], absmax[t]); that kernel, which sums the segments,
     // adds the tables' bases
     int lists_by_table;
+    int parts;                      // (cluster sort with the lists only) clusters of a table, each with its own share of the rows and its own
+                                    // lists, numbered table by table; a power of two
     u32 *seg_start, *chunk_first, *table_cnt, *tb, *absmax;
     uint2 *tile_done;
     int ck_shift;
     u32 cnt_broken;
-    int parts;                      // (cluster sort with the lists only) clusters of a table, each with its own share of the rows and its own
-                                    // lists, numbered table by table; a power of two
 };
 
 // a table whose boundary offsets cannot be used is reported and left out (the same answer in every thread)
