@@ -204,6 +204,17 @@ seg_sum_kernel(const Args a)
     };
     fetch(tile0);
     u32 u_base = tile0 < tile1 ? a.chunk_first[(int64_t)tile0 * I >> chunk_shift(SMALL)] : 0u;
+    // the runs that may be cut: lane 0 has the one that enters the range, lane 1 the one that leaves it.  Where rows take several
+    // warps what is to be known of them is asked for now (243 K rows of 1200 bytes 111 -> 109 us; narrower rows, whose loop wants the
+    // registers, 78.6 -> 79.5 at 520 K of 512 bytes, and small batches are better without)
+    constexpr bool EARLY = COLS && !SMALL;
+    u32 cut_u = 0u;                               // segment of the entry at the edge
+    bool cut = false;
+    const u32 edge = (wl == 0 ? tile0 : tile1) * I;
+    if (EARLY && wl < 2 && tile0 < tile1 && edge > 0u && edge < (u32)a.L) {
+        cut_u = __ldg(a.chunk_first + (edge >> chunk_shift(SMALL)));
+        cut = __ldg(a.keys + edge) == __ldg(a.keys + edge - 1u);
+    }
     if (a.by_table) {
         if (threadIdx.x < 32) {                   // the tables' first segments: a running sum over their counts
             u32 run = 0;
@@ -262,6 +273,15 @@ seg_sum_kernel(const Args a)
     request(0, v[0]);
     fetch(tile0 + 1);
 
+    u32 first_range = 0, last_range = 0;          // of a run that is cut: in which ranges its pieces are
+    auto find_pieces = [&](int t, int64_t at) {
+        const u32 R = (u32)a.range_tiles * I;
+        const u32 *start = a.seg_start + (a.by_table ? (int64_t)s_tb[t] + t + at : at);
+        first_range = __ldg(start) / R;
+        last_range = (__ldg(start + 1) - 1u) / R;
+    };
+    if (EARLY && cut) find_pieces(last_not_above(a.by_table ? s_tb : s_uoff, 0, T, a.by_table ? edge : cut_u), cut_u);
+    const u32 cuts = EARLY ? __ballot_sync(0xffffffffu, cut) : 0u;
     const bool head0 = heads & 1u;
     int t_first = a.by_table ? last_not_above(s_tb, 0, T, tile0 * I) : last_not_above(s_uoff, 0, T, u_base);
     if (a.by_table) u_base += s_uoff[t_first];
@@ -341,7 +361,7 @@ seg_sum_kernel(const Args a)
     }
     // ---- the run that is open at the end of the range
     const int64_t i1 = min((int64_t)tile1 * I, a.L);
-    const bool ends = i1 == a.L || __ldg(a.keys + i1) != __ldg(a.keys + i1 - 1);
+    const bool ends = EARLY ? !(cuts & 2u) : i1 == a.L || __ldg(a.keys + i1) != __ldg(a.keys + i1 - 1);
     const bool cut_lead = !head0, cut_trail = !open_lead && !ends;
     if (open_lead || cut_trail) store_piece(open_lead ? 0 : 1, acc);
     else store_row(u_base, acc);
@@ -351,15 +371,14 @@ seg_sum_kernel(const Args a)
     // ---- the warp that brings a cut run's last piece adds the pieces
     if (!(cut_lead || cut_trail)) return;
     const u32 group = range / FOLD_GROUP;
-    u32 last = 0, first_range = 0, groups = 0;    // pieces to add here; the run's first range; its groups, when it has many pieces
+    u32 last = 0, groups = 0;                     // pieces to add here; the run's groups, when it has many pieces
     if (wl == 0 ? cut_lead : (wl == 1 && cut_trail)) {
-        const u32 u = wl == 0 ? u_lead : u_base;
-        const int t = last_not_above(s_uoff, 0, T, u);
-        const int64_t at = a.by_table ? (int64_t)s_tb[t] + t + (u - s_uoff[t]) : (int64_t)u;
-        const u32 R = (u32)a.range_tiles * I;
-        const u32 sa = __ldg(a.seg_start + at), sb = __ldg(a.seg_start + at + 1);
-        first_range = sa / R;
-        const u32 last_range = (sb - 1) / R, g0 = first_range / FOLD_GROUP;
+        if (!EARLY) {
+            const u32 u = wl == 0 ? u_lead : u_base;
+            const int t = last_not_above(s_uoff, 0, T, u);
+            find_pieces(t, a.by_table ? u - s_uoff[t] : u);
+        }
+        const u32 g0 = first_range / FOLD_GROUP;
         u32 pieces = last_range - first_range + 1;
         u32 *arrived = &a.range_done[first_range].x;
         if (pieces > FOLD_GROUP) {
