@@ -335,7 +335,7 @@ int dqrm_emb_bwd(dqrm_ctx *ctx, const float *grad_out, const int32_t *indices, c
         return DQRM_ERR_INVALID_ARG;
     if (!ws_ok(workspace, workspace_bytes, dq_bwd_ws_bytes(ctx, L, (int64_t)ctx->T * B))) return DQRM_ERR_WORKSPACE;
     return dq_launch_bwd(ctx, grad_out, indices, offsets, unique_rows, uniq_off, grad_rows, B, L, workspace,
-                         workspace_bytes, as_stream(stream));
+                         workspace_bytes, as_stream(stream), true);
 }
 
 int dqrm_grad_quant_int8_bounded(dqrm_ctx *ctx, const float *grad_rows, const int32_t *uniq_off, int8_t *codes,

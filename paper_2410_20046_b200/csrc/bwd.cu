@@ -607,17 +607,20 @@ int dq_launch_bwd_sum(dqrm_ctx *ctx, const float *grad_out, int32_t *unique_rows
 // 13.8 / 19.6, 13.2 / 18.9.  At the line the two ways of launching part: 26 tables of 128 of 128 16.4 / 15.4 but 15.9 / 18.7, 16 of 256
 // of 64 17.6 / 15.4 but 17.0 / 18.7; beyond it (when the line was drawn) 4 tables of 1024 of 16 22.3 / 21.0, 512 of 64 24.8 / 22.0.
 // (With a row summary attached, or the sort chosen by the caller, the launches stay apart.)
-bool dq_small_step_takes(const dqrm_ctx *ctx, int B, int64_t L)
+static bool small_bwd_takes(const dqrm_ctx *ctx, int B, int64_t L)
 {
     const int64_t per_table = (L + ctx->T - 1) / ctx->T, want = L == (int64_t)ctx->T * B ? per_table : per_table + per_table / 4;
     // unless the batch has an index a bag, all of it may lie in one table, whose block then does everything: 1536 lookups of 16
     // features 29.8 us, 32.2 in separate launches; 2048 38 / 29, 1024 of 32 features 29 / 27, of 64 42 / 27
     if (L != (int64_t)ctx->T * B && (L > 1536 || L * ctx->D > 32768)) return false;
     return L > 0 && L <= sstep::MAX_LOOKUPS && want <= sstep::THREADS && want * ctx->D <= 16384 && ctx->D <= 128 &&
-           ctx->T <= ctx->num_sms && ctx->sort_path != 1 && !ctx->row_summary && !ctx->payload_position;
+           ctx->T <= ctx->num_sms && ctx->sort_path != 1 && !ctx->payload_position;
 }
 
-int dq_launch_small_step(dqrm_ctx *ctx, float *tables, const int32_t *indices, const int32_t *offsets, const float *grad_out,
+bool dq_small_step_takes(const dqrm_ctx *ctx, int B, int64_t L) { return !ctx->row_summary && small_bwd_takes(ctx, B, L); }
+
+template <bool STEP>
+static int launch_small(dqrm_ctx *ctx, float *tables, const int32_t *indices, const int32_t *offsets, const float *grad_out,
                          int32_t *unique_rows, int32_t *uniq_off, float *grad_rows, int8_t *codes, float *grad_scales, float lr,
                          int B, int64_t L, void *ws_, size_t ws_bytes, cudaStream_t st)
 {
@@ -634,22 +637,39 @@ int dq_launch_small_step(dqrm_ctx *ctx, float *tables, const int32_t *indices, c
     x.lr = lr; x.D = ctx->D;
     while ((4 << x.lpr_log) < ctx->D) ++x.lpr_log;
     const size_t smem = sstep::smem_bytes(ctx->T);
-    bool &raised = ctx->smem_raised[DQ_SMEM_SLOT_STEP];
+    bool &raised = ctx->smem_raised[DQ_SMEM_SLOT_STEP + (STEP ? 0 : 1)];
     // (the limit belongs to the function on the device, not to this context: every context sets the same, that of the most
     // tables that dq_small_step_takes lets through, or one with few tables would lower it for one with many)
     if (!raised)
-        DQRM_CUDA_TRY(ctx, cudaFuncSetAttribute(sstep::small_step_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        DQRM_CUDA_TRY(ctx, cudaFuncSetAttribute(sstep::small_step_kernel<STEP>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                 (int)sstep::smem_bytes(ctx->num_sms)));
     raised = true;
-    DQRM_CUDA_TRY(ctx, dq_launch(sstep::small_step_kernel, dim3((unsigned)ctx->T), dim3(sstep::THREADS), smem, st, x));
+    DQRM_CUDA_TRY(ctx, dq_launch(sstep::small_step_kernel<STEP>, dim3((unsigned)ctx->T), dim3(sstep::THREADS), smem, st, x));
     dq_mark(ctx, st, DQ_K_SMALL_STEP);
     return DQRM_OK;
 }
 
+int dq_launch_small_step(dqrm_ctx *ctx, float *tables, const int32_t *indices, const int32_t *offsets, const float *grad_out,
+                         int32_t *unique_rows, int32_t *uniq_off, float *grad_rows, int8_t *codes, float *grad_scales, float lr,
+                         int B, int64_t L, void *ws, size_t ws_bytes, cudaStream_t st)
+{
+    return launch_small<true>(ctx, tables, indices, offsets, grad_out, unique_rows, uniq_off, grad_rows, codes, grad_scales, lr, B, L, ws,
+                              ws_bytes, st);
+}
+
 int dq_launch_bwd(dqrm_ctx *ctx, const float *grad_out, const int32_t *indices, const int32_t *offsets,
                   int32_t *unique_rows, int32_t *uniq_off, float *grad_rows, int B, int64_t L,
-                  void *ws, size_t ws_bytes, cudaStream_t st)
+                  void *ws, size_t ws_bytes, cudaStream_t st, bool alone)
 {
+    // Up to 64 K gathered values a backward that stands alone (behind it a step would read the workspace's maxima) is one launch instead of
+    // two; while launches are timed one by one they stay two.  Measured on B200 (us, graph replay; two launches / one): 4 tables of 128
+    // lookups of 16 features 9.5 / 7.2, of 512 11.3 / 9.8, one of 400 10.8 / 8.2, 4 of 90 bags of four 13.4 / 9.7, 2 of 100 of 128
+    // features 10.0 / 8.1, 40 of 80 of 16 11.6 / 10.9, 26 of 128 10.1 / 10.1 (the four calls around it 20.2 / 19.7); 26 of 128 of 64
+    // 10.1 / 11.0, 16 of 256 of 64 10.6 / 13.3
+    if (alone && L * ctx->D <= 65536 && !ctx->prof_on && small_bwd_takes(ctx, B, L) && dq_aligned(grad_out, sizeof(float4)) &&
+        dq_aligned(grad_rows, sizeof(float4)))
+        return launch_small<false>(ctx, nullptr, indices, offsets, grad_out, unique_rows, uniq_off, grad_rows, nullptr, nullptr, 0.f, B, L, ws,
+                                   ws_bytes, st);
     int lists = 0;
     int rc = dq_launch_bwd_sort(ctx, indices, offsets, unique_rows, uniq_off, B, L, ws, ws_bytes, st, true, nullptr, &lists);
     if (rc != DQRM_OK) return rc;

@@ -385,7 +385,7 @@ size_t dq_sum_align(const dqrm_ctx *ctx);
 const u32 *dq_bwd_absmax_bits(const dqrm_ctx *ctx, int64_t L, const void *ws);
 int dq_launch_bwd(dqrm_ctx *ctx, const float *grad_out, const int32_t *indices, const int32_t *offsets,
                   int32_t *unique_rows, int32_t *uniq_off, float *grad_rows, int B, int64_t L,
-                  void *ws, size_t ws_bytes, cudaStream_t st);
+                  void *ws, size_t ws_bytes, cudaStream_t st, bool alone = false);
 
 // lists_by_table: dq_launch_bwd_sum follows on the same workspace; the cluster sort then numbers each table's
 // segments itself (*by_table says whether it did; *lists, without which it is one, how many lists each table then has), no separate kernel numbers them over the batch, and unique_rows /

@@ -47,9 +47,13 @@ constexpr size_t MID_WORDS = (size_t)1 << HASH_BITS;
 static_assert(MID_WORDS >= (size_t)WARPS * csort::BINS && MID_WORDS >= (size_t)THREADS * 8, "");
 inline size_t smem_bytes(int T) { return (size_t)THREADS * 2 * sizeof(u64) + (MID_WORDS + 3 * T + 1) * sizeof(u32); }
 
+// STEP: the whole step behind the forward; otherwise the backward alone (unique_rows, uniq_off, grad_rows), an ordinary kernel that
+// may be launched behind anything
+template <bool STEP>
 __global__ void __launch_bounds__(THREADS)
 small_step_kernel(const __grid_constant__ Args x)
 {
+    if (!STEP) dq_wait_before();
     extern __shared__ __align__(16) u64 s_net[];                 // [2][THREADS]
     u32 *s_mid = reinterpret_cast<u32 *>(s_net + 2 * THREADS);
     u32 *s_tb = s_mid + MID_WORDS;                 // [T+1]
@@ -73,10 +77,10 @@ small_step_kernel(const __grid_constant__ Args x)
     for (int i = tid; i <= T; i += THREADS)
         broken |= (int64_t)s_tb[i] > a.L || (i == 0 ? s_tb[0] != 0u : s_tb[i] < s_tb[i - 1]) || (i == T && (int64_t)s_tb[i] != a.L);
     if (__syncthreads_or(broken)) {                // nothing is summed, no row is updated
-        dq_wait_before();
+        if (STEP) dq_wait_before();
         if (tid == 0) {
             dq_report(a.status, DQRM_ERR_INDEX_RANGE);
-            x.grad_scales[t] = dq_scale_from_absmax(0.f, 8);
+            if (STEP) x.grad_scales[t] = dq_scale_from_absmax(0.f, 8);
             x.uniq_off[t] = 0;
             if (t == T - 1) x.uniq_off[T] = 0;
         }
@@ -137,7 +141,7 @@ small_step_kernel(const __grid_constant__ Args x)
         const int i = c0 + tid;
         const u32 row = i < n ? row_at(i) : 0u;
         const bool head = i < n && (i == 0 || row_at(i - 1) != row);
-        if (head)                                  // the update needs the row soon
+        if (STEP && head)                          // the update needs the row soon
             for (int o = 0; o < x.D; o += 32) dq_prefetch_l2(x.tables + (r0 + row) * x.D + o);
         const u32 m = __ballot_sync(0xffffffffu, head);
         if (lane == 0 && c0 + warp * 32 < n) s_head[(c0 >> 5) + warp] = m;
@@ -229,6 +233,13 @@ small_step_kernel(const __grid_constant__ Args x)
 #pragma unroll
             for (int j = 0; j < 4; ++j) acc[j] += s_sum[4 * ((g << x.lpr_log) + col) + j];
         put(seg);
+    }
+    if (!STEP) {
+        if (tid == 0) {
+            x.uniq_off[t] = (int32_t)base;
+            if (t == T - 1) x.uniq_off[T] = (int32_t)base + U;
+        }
+        return;
     }
     const u32 wm = __reduce_max_sync(0xffffffffu, __float_as_uint(mx));
     if (lane == 0 && wm) atomicMax(&s_max, wm);

@@ -109,3 +109,27 @@ def test_contexts_of_many_and_of_few_tables_take_turns(oracle):
             assert bit_equal(d_tables.cpu().numpy(), o_tables)
     for c, *_ in cases:
         c.ctx.close()
+
+
+BACKWARDS = dict(SHAPES, most_values=(64, [512, 512]), a_value_more=(64, [512, 511, 2]), most_lookups=(16, [256] * 16), most_of_a_table=(32, [512, 1, 0, 300]))
+
+
+@pytest.mark.parametrize("rows", [1, 9, 50_000])
+@pytest.mark.parametrize("name", list(BACKWARDS))
+def test_small_backward(oracle, name, rows):
+    """The backward alone in one launch, on both sides of what it takes."""
+    D, counts = BACKWARDS[name]
+    T, B = len(counts), max(1, max(counts))
+    wl = W.Workload("bwd", tuple(rows + t for t in range(T)), D=D, B=B, alpha=None)
+    rng = np.random.default_rng(rows + B + D)
+    idx = np.concatenate([rng.integers(0, wl.rows[t], n) for t, n in enumerate(counts)]).astype(np.int32)
+    lens = np.zeros((T, B), dtype=np.int64)
+    for t, n in enumerate(counts):
+        np.add.at(lens[t], rng.integers(0, B, n) if t % 2 else np.arange(n), 1)
+    off = np.concatenate([[0], np.cumsum(lens.reshape(-1))]).astype(np.int32)
+    go = (rng.integers(-1024, 1025, (B, T, D)) / 256).astype(np.float32)      # (exact sums, as above)
+    c = Case(wl, max_lookups=len(idx))
+    got, want = c.gpu_bwd(idx, off, go), oracle.emb_bwd(go, T, D, B, idx, off)
+    for g, w in zip(got, (want[0], want[1], want[2])):
+        assert bit_equal(g, w)
+    c.ctx.close()
