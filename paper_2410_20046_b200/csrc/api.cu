@@ -396,7 +396,7 @@ int dqrm_train_step(dqrm_ctx *ctx, float *tables, const int32_t *indices, const 
         if (fs != st) DQRM_CUDA_TRY(ctx, cudaStreamWaitEvent(fs, ctx->ev_fork, 0));
     }
     int rc = dq_launch_bwd(ctx, grad_out, indices, offsets, unique_rows, uniq_off, grad_rows, B, L, workspace, workspace_bytes, bs);
-    int rc2 = dq_launch_fwd(ctx, tables, indices, offsets, scales, bits, out, nullptr, B, L, fs);
+    int rc2 = dq_launch_fwd(ctx, tables, indices, offsets, scales, bits, out, nullptr, B, L, fs, false, overlap);
     // join even after an error so that the caller's stream stays ordered behind the others
     if (fs != st) {
         cudaEventRecord(ctx->ev_low_join, fs);

@@ -365,11 +365,12 @@ size_t dq_refresh_ws_bytes(const dqrm_ctx *ctx);
 int dq_launch_refresh(dqrm_ctx *ctx, const float *tables, const int32_t *bits, float *scales,
                       float *minmax, void *ws, size_t ws_bytes, cudaStream_t st);
 
+// let_next: see before_and_next; beside: a sort runs at the same time, to which the forward leaves room
 // bytes that tables and out have to be aligned to
 size_t dq_fwd_align(const dqrm_ctx *ctx, const int8_t *codes_out, int B, int64_t L);
 int dq_launch_fwd(dqrm_ctx *ctx, const float *tables, const int32_t *indices, const int32_t *offsets,
                   const float *scales, const int32_t *bits, float *out, int8_t *codes_out,
-                  int B, int64_t L, cudaStream_t st, bool let_next = false);
+                  int B, int64_t L, cudaStream_t st, bool let_next = false, bool beside = false);
 
 // the step's backward, quantiser and update in one launch, for small batches
 bool dq_small_step_takes(const dqrm_ctx *ctx, int B, int64_t L);

@@ -18,6 +18,7 @@
 //     rows per batch, and sums them in bag order in FP64, rounded once, so the result
 //     does not depend on the launch shape.
 //   * fwd_long_bags_kernel: the same for long bags of rows of 36 to 64 features, a warp a bag.
+#include <algorithm>
 #include <type_traits>
 #include "common.cuh"
 
@@ -42,7 +43,7 @@ struct FwdArgs {
     int T, D, B;
     int64_t L;
     int *status;
-    int per_warp;                // one-index batches: bags of a warp, up to 32
+    int per_warp;                // one-index batches: bags of a warp, up to 32 (before the launch: the fewest that it may take)
     int let_next;                // the kernel behind this one may begin (it waits itself where it has to)
 };
 
@@ -370,9 +371,9 @@ inline bool warp_per_bag(const FwdArgs &a, int lpr) { return lpr == 16 && long_b
 
 // Warps an SM below which a one-index batch's warps take fewer bags, down to one step of their rows: a warp's steps are a chain, and a
 // small batch has too few warps to hide it.  Measured on B200 (us; 32 bags a warp / so many that there are twelve warps an SM
-// at least): 26 tables of 2048 bags of 64 features (11 warps an SM) 5.25 / 4.45, one of 5000 of 128 6.51 / 2.82, four of 9000 of 32 3.35 / 2.94.  With more than twelve the
-// forward alone would gain on, but not the step in which it runs beside the sort: one table of 65,536 bags of 128 features (14 warps an
-// SM) 12.6 / 10.6, the step around it 67.7 / 68.3
+// at least): 26 tables of 2048 bags of 64 features (11 warps an SM) 5.25 / 4.45, one of 5000 of 128 6.51 / 2.82, four of 9000 of 32
+// 3.35 / 2.94.  Not in the one-call step, where it runs beside the sort, which needs the room: five tables of 10,000 bags of 128 features
+// 40.8, 42.6 with fewer bags a warp; nor with more warps: one table of 65,536 of 128 (14 warps an SM) 12.6 / 10.6 alone
 constexpr int FEW_WARPS = 12;
 constexpr int MIXED_TABLES = 8;
 // Order of the blocks.  All tables' blocks for the same bags side by side: the pooled rows of a bag lie next to one another in the
@@ -407,10 +408,10 @@ int launch2(dqrm_ctx *ctx, FwdArgs a, cudaStream_t st)
     constexpr int GPB = FW_THREADS / LPR;
     // the one-index kernel does not emit codes; a caller that asks for them gets the general kernel
     const bool onehot = a.L == (int64_t)a.T * a.B && a.codes_out == nullptr;
+    const int fewest = std::max(a.per_warp, 32 / LPR * NBOf<LPR, CH>::v);
     a.per_warp = 32;
     if (onehot) {
-        constexpr int STEP = 32 / LPR * NBOf<LPR, CH>::v;
-        while (a.per_warp / 2 >= STEP && (int64_t)a.T * ((a.B + a.per_warp - 1) / a.per_warp) < (int64_t)ctx->num_sms * FEW_WARPS) a.per_warp /= 2;
+        while (a.per_warp / 2 >= fewest && (int64_t)a.T * ((a.B + a.per_warp - 1) / a.per_warp) < (int64_t)ctx->num_sms * FEW_WARPS) a.per_warp /= 2;
     }
     const int per_block = onehot ? FW_THREADS / 32 * a.per_warp : warp_per_bag(a, LPR) ? GPB / 2 : GPB;
     int bx = (a.B + per_block - 1) / per_block;
@@ -441,10 +442,10 @@ size_t dq_fwd_align(const dqrm_ctx *ctx, const int8_t *codes_out, int B, int64_t
 
 int dq_launch_fwd(dqrm_ctx *ctx, const float *tables, const int32_t *indices, const int32_t *offsets,
                   const float *scales, const int32_t *bits, float *out, int8_t *codes_out,
-                  int B, int64_t L, cudaStream_t st, bool let_next)
+                  int B, int64_t L, cudaStream_t st, bool let_next, bool beside)
 {
     FwdArgs a{tables, ctx->d_row_off, indices, offsets, scales, bits, out, codes_out, ctx->T, ctx->D, B, L,
-              ctx->d_status, 32, let_next ? 1 : 0};
+              ctx->d_status, beside ? 32 : 1, let_next ? 1 : 0};
     const int d4 = ctx->D / 4;
     if (d4 <= 1) return launch<1, 1>(ctx, a, st);
     if (d4 <= 2) return launch<2, 1>(ctx, a, st);
