@@ -460,7 +460,7 @@ int dqrm_sort_batch(dqrm_ctx *ctx, const int32_t *indices, const int32_t *offset
     cudaStream_t st = as_stream(stream);
     if (ctx->prof_on) dq_mark(ctx, st, DQ_K_BEGIN);
     int lists = 0;
-    const int rc = dq_launch_bwd_sort(ctx, indices, offsets, unique_rows, uniq_off, B, L, workspace, workspace_bytes, st, true, nullptr, &lists);
+    const int rc = dq_launch_bwd_sort(ctx, indices, offsets, unique_rows, uniq_off, B, L, workspace, workspace_bytes, st, true, nullptr, &lists, true);
     {
         std::lock_guard<std::mutex> lock(ctx->sorted_mu);
         dqrm_ctx::SortedBatch &sb = ctx->sorted[workspace];

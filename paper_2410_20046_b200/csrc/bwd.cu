@@ -360,7 +360,7 @@ template <int CL, bool PARTS = false>
 cudaError_t launch_cluster_sort(dqrm_ctx *ctx, csort::Args ca, int cap, cudaStream_t st)
 {
     ca.cap = cap;
-    return launch_clusters<CL>(ctx, csort::cluster_sort_kernel<CL, 0, PARTS>, PARTS ? 6 : CL == csort::CLUSTER ? 0 : 3, ca, csort::smem_bytes(cap), st);
+    return launch_clusters<CL>(ctx, csort::cluster_sort_kernel<CL, 0, PARTS>, PARTS ? 6 : CL == csort::CLUSTER_NARROW ? 7 : CL == csort::CLUSTER ? 0 : 3, ca, csort::smem_bytes(cap), st);
 }
 
 // A table alone is shared by four clusters of sixteen blocks where as many as eight would fit (eight do not find room at the same
@@ -370,6 +370,19 @@ cudaError_t launch_cluster_sort(dqrm_ctx *ctx, csort::Args ca, int cap, cudaStre
 int table_parts(const dqrm_ctx *ctx)
 {
     return 2 * ctx->T * csort::CLUSTER_WIDE * csort::MAX_PARTS <= ctx->num_sms ? csort::MAX_PARTS : 1;
+}
+
+// Clusters of four blocks instead of eight.  Where clusters of eight for all tables do not fit at once (two blocks an SM: from 38 tables on)
+// the last of them wait for the first: 40 tables of 4000 lookups 20.5 -> 16.3 us, of 10,000 26.8 -> 24.1, eight pipelined steps around them
+// (3000 of 16 features, 16,000 of 8) 328 -> 224 and 510 -> 410; of 20,000 36.1 -> 40.5, four blocks have too much to do.  Where they fit,
+// but share SMs (from 19 tables on): 26 tables of 2500 lookups 32.7 -> 31.5 us a step, of 6000 17.7 -> 15.4, of 8000 41.6 -> 40.5 a step,
+// of 9000 18.1 -> 18.4.  Beside a training step (dqrm_sort_batch) four blocks leave it more room and take longer themselves, so
+// that count the step's rows: 26 tables of 8000 lookups of 48 features 497 -> 468 us for eight steps, of 16 282 -> 287, of 8 250 -> 266, of
+// 2500 of 16 192 -> 162; they are taken there for rows of 32 features and more, and for small tables
+bool narrow_clusters(const dqrm_ctx *ctx, int64_t per_table, bool beside)
+{
+    if (ctx->T * csort::CLUSTER > 2 * ctx->num_sms) return per_table <= 16384;
+    return ctx->T * csort::CLUSTER > ctx->num_sms && per_table <= (!beside || ctx->D >= 32 ? 8192 : 2560);
 }
 
 // clusters that stand by for tables beyond what their first block takes
@@ -442,7 +455,8 @@ size_t dq_sum_align(const dqrm_ctx *ctx)
 // segment starts).  It needs no upstream gradient, so a training step runs it beside the forward.
 int dq_launch_bwd_sort(dqrm_ctx *ctx, const int32_t *indices, const int32_t *offsets,
                        int32_t *unique_rows, int32_t *uniq_off, int B, int64_t L,
-                       void *ws_, size_t ws_bytes, cudaStream_t st, bool lists_by_table, bool *by_table, int *lists)
+                       void *ws_, size_t ws_bytes, cudaStream_t st, bool lists_by_table, bool *by_table, int *lists,
+                       bool beside)
 {
     const Layout y = make_layout(ctx, L);
     if (ws_bytes < y.total) return DQRM_ERR_WORKSPACE;
@@ -512,6 +526,8 @@ int dq_launch_bwd_sort(dqrm_ctx *ctx, const int32_t *indices, const int32_t *off
             if (e != cudaSuccess) ca.parts = 1;
         }
         if (wide && e != cudaSuccess) e = launch_cluster_sort<csort::CLUSTER_WIDE>(ctx, ca, csort::choose_cap(per_table, csort::CLUSTER_WIDE), st);
+        if (e != cudaSuccess && narrow_clusters(ctx, per_table, beside))
+            e = launch_cluster_sort<csort::CLUSTER_NARROW>(ctx, ca, csort::choose_cap(per_table, csort::CLUSTER_NARROW), st);
         if (e != cudaSuccess) e = launch_cluster_sort<csort::CLUSTER>(ctx, ca, csort::choose_cap(per_table, csort::CLUSTER), st);
         if (e == cudaSuccess) {
             dq_mark(ctx, st, DQ_K_CLUSTER_SORT);

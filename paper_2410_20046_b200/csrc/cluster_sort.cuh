@@ -22,6 +22,7 @@
 namespace csort {
 
 constexpr int CLUSTER = 8;            // blocks per table
+constexpr int CLUSTER_NARROW = 4;     // ... of many tables of few lookups
 constexpr int CLUSTER_WIDE = 16;      // ... when the batch has so few tables that eight blocks each would leave most SMs idle
 constexpr int MAX_PARTS = 4;           // ... of such clusters for a table alone, which would leave more of them idle still
 
@@ -453,7 +454,7 @@ __device__ __forceinline__ void sort_by_cluster(const Args &a)
 // kernel takes 95 registers and 26 tables of 16 K lookups 40 us instead of 32, with three 37.  Clusters of sixteen are
 // launched for a few tables only and have their SMs to themselves: 36.6 us without the bound, 42.2 with it, for one table
 // of 64 K lookups
-__host__ __device__ constexpr int resident(int CL) { return CL == CLUSTER ? 2 : 1; }
+__host__ __device__ constexpr int resident(int CL) { return CL <= CLUSTER ? 2 : 1; }
 
 template <int CL, int EPT, bool PARTS = false>
 __global__ void __launch_bounds__(THREADS, resident(CL))

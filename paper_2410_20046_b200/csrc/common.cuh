@@ -390,10 +390,10 @@ int dq_launch_bwd(dqrm_ctx *ctx, const float *grad_out, const int32_t *indices, 
 
 // lists_by_table: dq_launch_bwd_sum follows on the same workspace; the cluster sort then numbers each table's
 // segments itself (*by_table says whether it did; *lists, without which it is one, how many lists each table then has), no separate kernel numbers them over the batch, and unique_rows /
-// uniq_off are written by dq_launch_bwd_sum.  Without it they are complete when the sort is.
+// uniq_off are written by dq_launch_bwd_sum.  beside: a training step runs at the same time.  Without it they are complete when the sort is.
 int dq_launch_bwd_sort(dqrm_ctx *ctx, const int32_t *indices, const int32_t *offsets, int32_t *unique_rows,
                        int32_t *uniq_off, int B, int64_t L, void *ws, size_t ws_bytes, cudaStream_t st,
-                       bool lists_by_table, bool *by_table, int *lists = nullptr);
+                       bool lists_by_table, bool *by_table, int *lists = nullptr, bool beside = false);
 int dq_launch_bwd_sum(dqrm_ctx *ctx, const float *grad_out, int32_t *unique_rows, int32_t *uniq_off, float *grad_rows,
                       int B, int64_t L, int lists, void *ws, size_t ws_bytes, cudaStream_t st);
 

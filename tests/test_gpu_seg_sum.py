@@ -196,6 +196,36 @@ def test_table_alone_by_its_parts(oracle, where, rows, D):
         c.ctx.close()
 
 
+# many tables, which clusters of four blocks sort: on both sides of the numbers of tables and lookups at which they do
+@pytest.mark.parametrize("D", [8, 36])
+@pytest.mark.parametrize("T,per_table", [(18, 2_100), (19, 2_100), (19, 8_192), (19, 8_200), (37, 2_561), (38, 2_600), (38, 9_000), (40, 16_384)])
+def test_narrow_clusters(oracle, T, per_table, D):
+    if per_table > 9_000 and D > 8:
+        pytest.skip("the largest batch takes the narrow rows")
+    rng = np.random.default_rng(T + per_table)
+    rows = tuple(int(r) for r in rng.choice([1, 3, 300, 70_000], T))
+    B = per_table
+    for bags in (False, True):
+        lens = np.ones((T, B), dtype=np.int64)
+        if bags:                         # uneven tables and bags, of the same mean
+            half = rng.permutation(T * B)[:T * B // 2 * 2]
+            lens.reshape(-1)[half[::2]] -= 1
+            lens.reshape(-1)[half[1::2]] += 1
+            lens[0, 0] += 1              # (not as many lookups as bags)
+        off = np.concatenate([[0], np.cumsum(lens.reshape(-1))]).astype(np.int32)
+        table = np.repeat(np.arange(T), lens.sum(1))
+        idx = (rng.random(off[-1]) ** rng.choice([1, 6], off[-1]) * np.array(rows)[table]).astype(np.int32)
+        go = rng.standard_normal((B, T, D), dtype=np.float32)
+        c = Case(W.Workload("narrow", rows, D=D, B=B, alpha=None), max_lookups=len(idx))
+        ur, uo, gr = c.gpu_bwd(idx, off, go)
+        o_ur, o_uo, o_gr = oracle.emb_bwd(go, T, D, B, idx, off)
+        assert bit_equal(uo, o_uo) and bit_equal(ur, o_ur)
+        # n terms of magnitude below 6 in FP64 in two orders, each sum rounded once
+        n = int(np.bincount(idx + 100_000 * table).max())
+        np.testing.assert_allclose(gr, o_gr, rtol=2.0 ** -23, atol=12.0 * n * n * 2.0 ** -53)
+        c.ctx.close()
+
+
 # more than a dozen tiles of 32 for each of the 4736 warps that 148 SMs hold: ranges of eight tiles, several of them for a warp's place
 @pytest.mark.parametrize("D", [52, 64])
 @pytest.mark.parametrize("sort_path", [0, 1])
