@@ -363,6 +363,17 @@ cudaError_t launch_cluster_sort(dqrm_ctx *ctx, csort::Args ca, int cap, cudaStre
     return launch_clusters<CL>(ctx, csort::cluster_sort_kernel<CL, 0, PARTS>, PARTS ? 6 : CL == csort::CLUSTER_NARROW ? 7 : CL == csort::CLUSTER ? 0 : 3, ca, csort::smem_bytes(cap), st);
 }
 
+// Clusters of sixteen blocks for few tables of 16 K lookups and more, and of 5 K (a table alone: 8 K) where the rows take three passes and no
+// training step runs beside, from which they would take twice the room.  Measured on B200 (us; sixteen blocks / eight): sort of 2 tables of
+// 12,000 lookups of 1.5 M rows 15.2 / 16.8, 3 of 8000 13.4 / 14.3, 4 of 5000 13.0 / 13.3, of one (in its parts, see below) of 15,000 15.5 / 19.7,
+// of 10,000 14.6 / 15.2, of 8000 of 30 K rows 12.0 / 11.3; steps of 4 tables of 4100 29.2 / 28.9, of one of 4500 28.8 / 28.1; eight
+// pipelined steps of one table of 10,000 182 / 142, of 4 of 5000 172 / 142
+bool wide_clusters(const dqrm_ctx *ctx, int64_t per_table, bool beside)
+{
+    const int64_t least = ctx->row_bits <= 16 || beside ? 1024 : ctx->T > 1 ? 320 : 512;       // lookups for a block
+    return ctx->T * csort::CLUSTER_WIDE * 2 <= ctx->num_sms && per_table >= csort::CLUSTER_WIDE * least;
+}
+
 // A table alone is shared by four clusters of sixteen blocks where as many as eight would fit (eight do not find room at the same
 // moment: 34 us).  Measured on B200 (us; four clusters / one): 65,536 lookups of 10 M rows 19.9 / 29.5, Zipf 1.2 19.9 / 24.2, of 3000
 // rows 15.3 / 19.9, 40,000 of 50 K 14.4 / 15.6, 17,000 of 1 M 14.9 / 15.5.  Two tables by two clusters each: 65,536 of 2 M rows 18.1 / 18.6,
@@ -518,7 +529,7 @@ int dq_launch_bwd_sort(dqrm_ctx *ctx, const int32_t *indices, const int32_t *off
             ctx->last_cuda_error = (int)e;         // (taken off the runtime, so that nobody finds it behind the sort that follows)
             (void)cudaGetLastError();
         }
-        const bool wide = ctx->T * csort::CLUSTER_WIDE * 2 <= ctx->num_sms && per_table >= csort::CLUSTER_WIDE * 1024;
+        const bool wide = wide_clusters(ctx, per_table, beside);
         e = cudaErrorUnknown;
         if (wide && lists_by_table && lists) {
             ca.parts = table_parts(ctx);

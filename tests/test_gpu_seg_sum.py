@@ -196,6 +196,27 @@ def test_table_alone_by_its_parts(oracle, where, rows, D):
         c.ctx.close()
 
 
+# few tables of 5 K lookups and more, of rows of two and of three digits, which clusters of sixteen and of eight blocks sort
+@pytest.mark.parametrize("T,per_table", [(1, 8_191), (1, 8_192), (1, 12_001), (2, 5_119), (2, 5_120), (4, 7_003)])
+@pytest.mark.parametrize("rows", [60_000, 70_000])
+def test_wide_clusters(oracle, T, per_table, rows):
+    rng = np.random.default_rng(T + per_table)
+    D, B = 12, per_table
+    for bags in (False, True):
+        lens = rng.integers(0, 3, T * B) if bags else np.ones(T * B, dtype=np.int64)
+        off = np.concatenate([[0], np.cumsum(lens)]).astype(np.int32)
+        idx = (rng.random(off[-1]) ** rng.choice([1, 6], off[-1]) * rows).astype(np.int32)
+        go = rng.standard_normal((B, T, D), dtype=np.float32)
+        c = Case(W.Workload("wide", (rows,) * T, D=D, B=B, alpha=None), max_lookups=len(idx))
+        ur, uo, gr = c.gpu_bwd(idx, off, go)
+        o_ur, o_uo, o_gr = oracle.emb_bwd(go, T, D, B, idx, off)
+        assert bit_equal(uo, o_uo) and bit_equal(ur, o_ur)
+        # n terms of magnitude below 6 in FP64 in two orders, each sum rounded once
+        n = int(np.bincount(idx + rows * np.repeat(np.arange(T), lens.reshape(T, B).sum(1))).max())
+        np.testing.assert_allclose(gr, o_gr, rtol=2.0 ** -23, atol=12.0 * n * n * 2.0 ** -53)
+        c.ctx.close()
+
+
 # many tables, which clusters of four blocks sort: on both sides of the numbers of tables and lookups at which they do
 @pytest.mark.parametrize("D", [8, 36])
 @pytest.mark.parametrize("T,per_table", [(18, 2_100), (19, 2_100), (19, 8_192), (19, 8_200), (37, 2_561), (38, 2_600), (38, 9_000), (40, 16_384)])
