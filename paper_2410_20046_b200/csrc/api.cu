@@ -538,7 +538,7 @@ int dqrm_train_step_sorted(dqrm_ctx *ctx, float *tables, const int32_t *indices,
     if (overlap) {
         DQRM_CUDA_TRY(ctx, cudaEventRecord(ctx->ev_low_fork, st));
         DQRM_CUDA_TRY(ctx, cudaStreamWaitEvent(ctx->low, ctx->ev_low_fork, 0));
-        rc2 = dq_launch_fwd(ctx, tables, indices, offsets, scales, bits, out, nullptr, B, L, ctx->low);
+        rc2 = dq_launch_fwd(ctx, tables, indices, offsets, scales, bits, out, nullptr, B, L, ctx->low, false, true);
         cudaEventRecord(ctx->ev_low_join, ctx->low);
         cudaStreamWaitEvent(st, ctx->ev_low_join, 0);
     } else {

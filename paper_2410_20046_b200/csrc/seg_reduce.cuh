@@ -68,6 +68,7 @@ struct Args {
     // how many segments the table has (CNT_BROKEN: nothing is summed, no row is updated); unique_rows and uniq_off
     // are then written here, with the tables' bases added
     int by_table;
+    int parts_log;
     const u32 *table_cnt, *tb;
     const int64_t *row_off;
     int32_t *unique_rows, *uniq_off;
@@ -77,7 +78,6 @@ struct Args {
     double *group_partials;     // [ranges / 32 + 1][2][D]: the same for groups of 32 ranges
     u32 *absmax;                // [T] zero
     int T, D;                   // T: lists, 2^parts_log for every table (by_table; one otherwise)
-    int parts_log;
     int64_t L, G;
     int64_t num_tiles;          // rows that take a warp: tiles, tiles of a warp's range, blocks of 128 features
     int range_tiles, columns;
