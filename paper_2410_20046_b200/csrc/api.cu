@@ -696,7 +696,8 @@ int dqrm_train_step_host(dqrm_ctx *ctx, float *tables, const int32_t *h_indices,
     char *step_ws = ws + y.step_ws;
     const size_t step_ws_bytes = workspace_bytes - y.step_ws;
     int lists = 0;
-    int rc = dq_launch_bwd_sort(ctx, d_idx, d_off, d_ur, d_uo, B, L, step_ws, step_ws_bytes, ctx->side, true, nullptr, &lists);
+    // (beside: the forward, whose output has to leave soon, and the call before)
+    int rc = dq_launch_bwd_sort(ctx, d_idx, d_off, d_ur, d_uo, B, L, step_ws, step_ws_bytes, ctx->side, true, nullptr, &lists, true);
     if (rc == DQRM_OK) rc = dq_launch_fwd(ctx, tables, d_idx, d_off, scales, bits, d_out, nullptr, B, L, st);
     // join every stream even after an error, so that the caller's stream stays ordered behind them
     cudaEventRecord(ctx->ev_h_fwd, st);
