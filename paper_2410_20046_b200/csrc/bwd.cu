@@ -86,8 +86,7 @@ Layout make_layout(const dqrm_ctx *ctx, int64_t L)
     y.tb = take(sizeof(u32) * (lists + 1));
     y.chunk_first = take(sizeof(u32) * (Lc / 8 + 1));      // (the most that any L up to this one may need)
     y.tile_done = take(sizeof(uint2) * (Lc / 8 + 1));
-    // (ranges: the most that any L up to this one may need)
-    const int64_t ranges = std::max(std::min(Lc / 8 + 1, warps), segred::takes_groups(ctx->D) ? (int64_t)0 : Lc / (32 * segred::RANGE_TILES) + 1);
+    const int64_t ranges = std::max(std::min(Lc / 8 + 1, warps), segred::max_ranges(ctx->D, Lc));      // (the most that any L up to this one may need)
     y.partials = take(sizeof(double) * ranges * 2 * ctx->D);
     y.group_partials = take(sizeof(double) * (ranges / segred::FOLD_GROUP + 1) * 2 * ctx->D);
     y.total = o;

@@ -55,6 +55,8 @@ inline int range_tiles(int D, int64_t tiles, int64_t warps)
     const int64_t even = (tiles + warps - 1) / warps;
     return (int)(floats_per_lane(D) == 2 && even > RANGE_TILES + RANGE_TILES / 2 ? RANGE_TILES : even);
 }
+// of such ranges, for L lookups (rows of 48 features and fewer have ranges of their own, seg_groups.cuh)
+inline int64_t max_ranges(int D, int64_t L) { return D > 48 && floats_per_lane(D) == 2 ? L / (32 * RANGE_TILES) + 1 : 0; }
 
 struct Args {
     const u32 *keys, *vals, *seg_start, *chunk_first;
