@@ -116,7 +116,10 @@ __device__ __forceinline__ void pool_bag_plain(const FwdArgs &a, const TableCtx 
 // 32/LPR at a time by all lanes, each step reading its bag's index from the owner lane by shuffle.
 // Measured on B200 the kernel is bound by instruction issue, not by HBM, at 256-byte rows, which
 // is why the per-bag work is kept off the per-row path.
-template <int LPR, int CH, bool EXACT>
+//
+// FEW: a warp takes a.per_warp bags instead of 32 (launch2).  An instance of its own: as a value at run time the number of bags cost the
+// others registers, and values were spilled (200 K rows of 800 bytes 65.2 -> 69.4 us, 65 K 17.6 -> 19.7, 426 K of 80 15.1 -> 15.4).
+template <int LPR, int CH, bool EXACT, bool FEW>
 __global__ void __launch_bounds__(FW_THREADS, 5)
 fwd_onehot_kernel(const FwdArgs a)
 {
@@ -130,7 +133,7 @@ fwd_onehot_kernel(const FwdArgs a)
     const int wlane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int lane = wlane % LPR, grp = wlane / LPR;
     const int64_t g0 = (int64_t)t * a.B;
-    const int per = RPW * NB >= 32 ? 32 : a.per_warp;
+    const int per = FEW ? a.per_warp : 32;
     const unsigned all = 0xffffffffu >> (32 - per);
     // a bag's offsets and its index, the right one when the offsets are the identity (L == T*B): on their way before the
     // table's constants are waited for (426 K rows of 64 bytes 8.9 -> 8.4 us, 852 K packed ones of 32 40.6 -> 39.5; not where the
@@ -421,8 +424,10 @@ int launch2(dqrm_ctx *ctx, FwdArgs a, cudaStream_t st)
     if (bx < 1) bx = 1;
     const bool mixed = onehot || bags_mixed<LPR, CH>(a);
     const dim3 grid((unsigned)(mixed ? ctx->T : bx), (unsigned)(mixed ? bx : ctx->T));
-    DQRM_CUDA_TRY(ctx, (onehot ? dq_launch(fwd_onehot_kernel<LPR, CH, EXACT>, grid, dim3(FW_THREADS), 0, st, a)
-                               : launch_bags<LPR, CH, EXACT>(a, grid, st)));
+    constexpr bool MAY = 32 / LPR * NBOf<LPR, CH>::v < 32;
+    DQRM_CUDA_TRY(ctx, (!onehot                 ? launch_bags<LPR, CH, EXACT>(a, grid, st)
+                        : MAY && a.per_warp < 32 ? dq_launch(fwd_onehot_kernel<LPR, CH, EXACT, MAY>, grid, dim3(FW_THREADS), 0, st, a)
+                                                 : dq_launch(fwd_onehot_kernel<LPR, CH, EXACT, false>, grid, dim3(FW_THREADS), 0, st, a)));
     dq_mark(ctx, st, DQ_K_FWD);
     return DQRM_OK;
 }

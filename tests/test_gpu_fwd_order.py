@@ -46,9 +46,10 @@ def test_order_of_the_blocks(oracle, D, B, bag):
     c.ctx.close()
 
 
-# one-index batches of few warps, which take 32 bags each down to one step of rows: whole and cut warps, and bags of none and of two
+# one-index batches of few warps, which take 32 bags each (from twelve warps an SM of 148 on: 26 tables of 2177) down to one step of
+# rows: whole and cut warps, and bags of none and of two
 @pytest.mark.parametrize("D", [16, 20, 32, 36, 64, 100, 128, 200, 256, 1020])
-@pytest.mark.parametrize("T,B", [(1, 1), (3, 5), (2, 33), (5, 100), (26, 517), (7, 2049), (26, 2048)])
+@pytest.mark.parametrize("T,B", [(1, 1), (3, 5), (2, 33), (5, 100), (26, 517), (7, 2049), (26, 2048), (26, 2176), (26, 2177)])
 def test_few_warps(oracle, D, T, B):
     if T * B > 20_000 and D not in (32, 64, 100, 256):
         pytest.skip("the larger batches take one width of each kind")
