@@ -77,7 +77,7 @@ __device__ __forceinline__ void load8(const float4 *p, float4 &a, float4 &b)
 template <int BITS>
 __global__ void __launch_bounds__(PK_THREADS)
 pack_kernel(const float4 *__restrict__ arena4, const int64_t *__restrict__ row_off, int T, int D, int64_t n4,
-            const float *__restrict__ scales, uint8_t *__restrict__ packed, int pairs)
+            const float *__restrict__ scales, uint8_t *__restrict__ packed, bool read8, bool store8)
 {
     dq_wait_before();
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -91,7 +91,7 @@ pack_kernel(const float4 *__restrict__ arena4, const int64_t *__restrict__ row_o
         const int t0 = dq_table_of(v4_off, T, c0);
         const bool one_table = c1 <= v4_off[t0 + 1];
         QuantScale qs = dq_make_scale(__ldg(scales + t0), BITS);
-        if (pairs && one_table && c1 - c0 == PK_CHUNK4) {
+        if (one_table && c1 - c0 == PK_CHUNK4) {
             // a thread's loads of PK_UNROLL rounds are all in flight before the first is quantised
 #pragma unroll 1
             for (int r = 0; r < PK_CHUNK4 / 2; r += PK_THREADS * PK_UNROLL) {
@@ -99,7 +99,7 @@ pack_kernel(const float4 *__restrict__ arena4, const int64_t *__restrict__ row_o
 #pragma unroll
                 for (int k = 0; k < PK_UNROLL; ++k) {
                     const float4 *p = arena4 + c0 + 2 * (r + k * PK_THREADS + threadIdx.x);
-                    if (pairs == 2) {
+                    if (read8) {
                         load8(p, v[k][0], v[k][1]);
                     } else {
                         v[k][0] = __ldcs(p);
@@ -107,9 +107,16 @@ pack_kernel(const float4 *__restrict__ arena4, const int64_t *__restrict__ row_o
                     }
                 }
 #pragma unroll
-                for (int k = 0; k < PK_UNROLL; ++k)
-                    store_packed2<BITS>(packed, c0 / 2 + r + k * PK_THREADS + threadIdx.x, quantise_packed4<BITS>(v[k][0], qs),
-                                        quantise_packed4<BITS>(v[k][1], qs));
+                for (int k = 0; k < PK_UNROLL; ++k) {
+                    const int64_t v8 = c0 / 2 + r + k * PK_THREADS + threadIdx.x;
+                    const u32 first = quantise_packed4<BITS>(v[k][0], qs), second = quantise_packed4<BITS>(v[k][1], qs);
+                    if (store8) {
+                        store_packed2<BITS>(packed, v8, first, second);
+                    } else {
+                        store_packed<BITS>(packed, 2 * v8, first);
+                        store_packed<BITS>(packed, 2 * v8 + 1, second);
+                    }
+                }
             }
             continue;
         }
@@ -367,10 +374,10 @@ int launch_pack(dqrm_ctx *ctx, const float *tables, const float *scales, uint8_t
 {
     const int64_t n4 = ctx->total_rows * (ctx->D / 4);
     const size_t smem = (size_t)(ctx->T + 1) * sizeof(int64_t);
-    // vectors in pairs where their packed bytes may be stored at once; read at once, too, where the arena begins on 32 bytes
-    const int pairs = !dq_aligned(packed, (size_t)BITS) ? 0 : dq_aligned(tables, 2 * sizeof(float4)) ? 2 : 1;
+    // two vectors are read at once where the arena begins on 32 bytes, and their packed bytes stored at once where those may be
+    const bool read8 = dq_aligned(tables, 2 * sizeof(float4)), store8 = dq_aligned(packed, (size_t)BITS);
     DQRM_CUDA_TRY(ctx, dq_launch(pack_kernel<BITS>, dim3(ctx->num_sms * 8), dim3(PK_THREADS), smem, st,
-                                 reinterpret_cast<const float4 *>(tables), ctx->d_row_off, ctx->T, ctx->D, n4, scales, packed, pairs));
+                                 reinterpret_cast<const float4 *>(tables), ctx->d_row_off, ctx->T, ctx->D, n4, scales, packed, read8, store8));
     dq_mark(ctx, st, DQ_K_PACK);
     return DQRM_OK;
 }
