@@ -22,7 +22,7 @@
 namespace csort {
 
 constexpr int CLUSTER = 8;            // blocks per table
-constexpr int CLUSTER_NARROW = 4;     // ... of many tables of few lookups
+constexpr int CLUSTER_HALF = 4;       // ... of which so many work where there are many tables of few lookups
 constexpr int CLUSTER_WIDE = 16;      // ... when the batch has so few tables that eight blocks each would leave most SMs idle
 constexpr int MAX_PARTS = 4;           // ... of such clusters for a table alone, which would leave more of them idle still
 
@@ -49,8 +49,10 @@ __device__ __forceinline__ u32 same_digit_lanes(u32 d, bool valid)
 // reads all the table's lookups and keeps those of its rows, so nothing passes between the clusters; where its lookups stand behind those
 // of the rows before it counts itself, and its segments have lists of their own.  Rows are shared out evenly, lookups need not fall so: in the worst case
 // one cluster sorts them all, as it would alone.  A table beyond the blocks' shared memory is its first cluster's.
-template <int CL, int EPT, bool PARTS>
-__device__ __forceinline__ void sort_by_cluster(const Args &a)
+//
+// OF: blocks launched for every cluster, of which CL call this, from block `from` on; the others have left.
+template <int CL, int EPT, bool PARTS, int OF = CL>
+__device__ __forceinline__ void sort_by_cluster(const Args &a, unsigned from = 0)
 {
     extern __shared__ __align__(16) uint2 s_dyn[];               // pair buffers [2][cap]: (row within table, payload)
     __shared__ __align__(16) u32 s_cnt[WARPS][BINS];
@@ -63,8 +65,8 @@ __device__ __forceinline__ void sort_by_cluster(const Args &a)
     __shared__ u32 s_sum[2];                       // ... the cluster's
 
     cg::cluster_group cluster = cg::this_cluster();
-    const unsigned c = cluster.block_rank();
-    const int list = blockIdx.x / CL, t = PARTS ? list / a.parts : list, part = PARTS ? list % a.parts : 0;
+    const unsigned rank0 = OF > CL ? from : 0u, c = cluster.block_rank() - rank0;
+    const int list = blockIdx.x / OF, t = PARTS ? list / a.parts : list, part = PARTS ? list % a.parts : 0;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const u32 lt = (1u << lane) - 1u;
 
@@ -266,7 +268,7 @@ __device__ __forceinline__ void sort_by_cluster(const Args &a)
         if (threadIdx.x < BINS) {                  // one thread per digit (the first BINS / 32 warps)
             u32 h[CL];
 #pragma unroll
-            for (unsigned cc = 0; cc < CL; ++cc) h[cc] = *remote(cluster, &s_hist[threadIdx.x], cc);
+            for (unsigned cc = 0; cc < CL; ++cc) h[cc] = *remote(cluster, &s_hist[threadIdx.x], rank0 + cc);
 #pragma unroll
             for (unsigned cc = 0; cc < CL; ++cc) { if (cc < c) pre += h[cc]; tot += h[cc]; }
             incl = tot;
@@ -311,7 +313,7 @@ __device__ __forceinline__ void sort_by_cluster(const Args &a)
                         if (owner * (u32)npc > pos) --owner;
                         else if ((owner + 1u) * (u32)npc <= pos) ++owner;
                         const u32 j = pos - owner * npc;
-                        cluster.map_shared_rank(dst, owner)[j] = pr;
+                        cluster.map_shared_rank(dst, rank0 + owner)[j] = pr;
                     } else {
                         gdst[tb0 + pos] = pr;
                     }
@@ -334,7 +336,7 @@ __device__ __forceinline__ void sort_by_cluster(const Args &a)
         const uint2 *fin = s ? pb1 : pb0;
         u32 prev_last = 0xFFFFFFFFu;               // last row of the previous block's slice (full by construction)
         if (c > 0) {
-            const uint2 *pf = in_smem ? cluster.map_shared_rank(s ? pb1 : pb0, c - 1)
+            const uint2 *pf = in_smem ? cluster.map_shared_rank(s ? pb1 : pb0, rank0 + c - 1)
                                       : (s ? a.gp[1] : a.gp[0]) + tb0 + (int64_t)(c - 1) * npc;
             prev_last = pf[npc - 1].x;
         }
@@ -396,7 +398,7 @@ __device__ __forceinline__ void sort_by_cluster(const Args &a)
                 // the block's total goes into every block's shared memory, under cover of the barrier below
                 // (sending or fetching made no measurable difference, here or for the passes' digit counts)
                 const u32 mine_all = __shfl_sync(0xffffffffu, incl, WARPS - 1);
-                if (lane < CL) *cluster.map_shared_rank(&s_totals[c], (unsigned)lane) = mine_all;
+                if (lane < CL) *cluster.map_shared_rank(&s_totals[c], rank0 + lane) = mine_all;
             }
             cluster.sync();                        // every block's total has arrived (and the warps' bases are here)
             if (warp == 0) {
@@ -462,6 +464,19 @@ cluster_sort_kernel(const __grid_constant__ Args a)
 {
     dq_wait_before();
     sort_by_cluster<CL, EPT, PARTS>(a);
+}
+
+// Clusters of eight of which four blocks sort the table where it fits into their shared memory, and all eight where it does not: how
+// large a table is shows on the device alone.  The four that leave make room for the clusters that wait; which four they are alternates
+// from table to table, so that clusters that share SMs work on different ones (64 tables of 4000 lookups 46.3 -> 43.2 us a backward).
+__global__ void __launch_bounds__(THREADS, resident(CLUSTER))
+cluster_sort_half_kernel(const __grid_constant__ Args a)
+{
+    dq_wait_before();
+    const unsigned t = blockIdx.x / CLUSTER, from = t % 2 * CLUSTER_HALF;
+    const int64_t n = (int64_t)__ldg(a.offsets + (int64_t)(t + 1) * a.B) - __ldg(a.offsets + (int64_t)t * a.B);
+    if (n > (int64_t)CLUSTER_HALF * a.cap) sort_by_cluster<CLUSTER, 0, false>(a);
+    else if (blockIdx.x % CLUSTER / CLUSTER_HALF == t % 2) sort_by_cluster<CLUSTER_HALF, 0, false, CLUSTER>(a, from);
 }
 
 inline size_t smem_bytes(int cap) { return (size_t)2 * cap * sizeof(uint2); }

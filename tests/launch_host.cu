@@ -83,6 +83,22 @@ int clusters_stand_by()
     return 0;
 }
 
+// a batch's mean does not say how large its largest table is: whatever the mean, clusters of eight stand ready for a table
+int eight_blocks_a_table()
+{
+    bool by_table = false;
+    for (const int T : {10, 19, 26, 33, 34, 38, 64, 100})
+        for (const int B : {2100, 2600, 8000, 12000}) {
+            if ((int64_t)T * B > 260000) continue;
+            Ctx x(T, 16);
+            WANT(x.sort(B, (int64_t)T * B, &by_table) == DQRM_OK && by_table);
+            WANT(fake::cluster == 8 && fake::grid_x == 8u * T);
+            WANT(x.sort(B, (int64_t)T * B + 1, &by_table) == DQRM_OK && by_table);
+            WANT(fake::cluster == 8 && fake::grid_x == 8u * T);
+        }
+    return 0;
+}
+
 }  // namespace
 
 int main(int argc, char **argv)
@@ -91,6 +107,7 @@ int main(int argc, char **argv)
     if (!strcmp(name, "contexts_in_turn")) return contexts_in_turn();
     if (!strcmp(name, "refused_sorts")) return refused_sorts();
     if (!strcmp(name, "clusters_stand_by")) return clusters_stand_by();
+    if (!strcmp(name, "eight_blocks_a_table")) return eight_blocks_a_table();
     std::printf("no scenario %s\n", name);
     return 2;
 }

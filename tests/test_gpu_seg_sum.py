@@ -217,9 +217,10 @@ def test_wide_clusters(oracle, T, per_table, rows):
         c.ctx.close()
 
 
-# many tables, which clusters of four blocks sort: on both sides of the numbers of tables and lookups at which they do
+# many tables, which half of a cluster's blocks sort: on both sides of the numbers of tables and lookups at which they do
 @pytest.mark.parametrize("D", [8, 36])
-@pytest.mark.parametrize("T,per_table", [(18, 2_100), (19, 2_100), (19, 8_192), (19, 8_200), (37, 2_561), (38, 2_600), (38, 9_000), (40, 16_384)])
+@pytest.mark.parametrize("T,per_table", [(18, 2_100), (19, 2_100), (19, 8_192), (19, 8_200), (37, 2_561), (38, 2_600), (38, 9_000), (40, 16_384),
+                                         (33, 2_100), (34, 2_100), (34, 8_193), (59, 4_096), (59, 4_097), (66, 4_096), (67, 4_097)])
 def test_narrow_clusters(oracle, T, per_table, D):
     if per_table > 9_000 and D > 8:
         pytest.skip("the largest batch takes the narrow rows")
@@ -245,6 +246,34 @@ def test_narrow_clusters(oracle, T, per_table, D):
         n = int(np.bincount(idx + 100_000 * table).max())
         np.testing.assert_allclose(gr, o_gr, rtol=2.0 ** -23, atol=12.0 * n * n * 2.0 ** -53)
         c.ctx.close()
+
+
+# clusters of which half works: a table that fits their shared memory to the last pair (3200 at a mean of 2500 lookups a table), one pair
+# more, the last pair that all eight blocks hold, and beyond; in tables of both halves
+@pytest.mark.parametrize("T", [34, 40, 66])
+@pytest.mark.parametrize("large", [3_199, 3_200, 3_201, 6_400, 6_401, 40_000])
+def test_tables_beyond_half_a_cluster(oracle, T, large):
+    rng = np.random.default_rng(T + large)
+    D, B = 8, 2_500
+    counts = np.full(T, (T * B - 2 * large) // (T - 2))
+    counts[[2, T - 1]] = large
+    counts[0] += T * B - counts.sum()
+    rows = tuple(int(r) for r in rng.choice([1, 300, 70_000], T))
+    lens = np.zeros((T, B), dtype=np.int64)
+    for t, n in enumerate(counts):
+        np.add.at(lens[t], rng.integers(0, B, n), 1)
+    off = np.concatenate([[0], np.cumsum(lens.reshape(-1))]).astype(np.int32)
+    table = np.repeat(np.arange(T), counts)
+    idx = (rng.random(off[-1]) * np.array(rows)[table]).astype(np.int32)
+    go = rng.standard_normal((B, T, D), dtype=np.float32)
+    c = Case(W.Workload("half", rows, D=D, B=B, alpha=None), max_lookups=len(idx))
+    ur, uo, gr = c.gpu_bwd(idx, off, go)
+    o_ur, o_uo, o_gr = oracle.emb_bwd(go, T, D, B, idx, off)
+    assert bit_equal(uo, o_uo) and bit_equal(ur, o_ur)
+    # n terms of magnitude below 6 in FP64 in two orders, each sum rounded once
+    n = int(np.bincount(idx + 100_000 * table).max())
+    np.testing.assert_allclose(gr, o_gr, rtol=2.0 ** -23, atol=12.0 * n * n * 2.0 ** -53)
+    c.ctx.close()
 
 
 # more than a dozen tiles of 32 for each of the 4736 warps that 148 SMs hold: ranges of eight tiles, several of them for a warp's place
