@@ -380,12 +380,17 @@ bool wide_clusters(const dqrm_ctx *ctx, int64_t per_table, bool beside)
 }
 
 // A table alone is shared by four clusters of sixteen blocks where as many as eight would fit (eight do not find room at the same
-// moment: 34 us).  Measured on B200 (us; four clusters / one): 65,536 lookups of 10 M rows 19.9 / 29.5, Zipf 1.2 19.9 / 24.2, of 3000
-// rows 15.3 / 19.9, 40,000 of 50 K 14.4 / 15.6, 17,000 of 1 M 14.9 / 15.5.  Two tables by two clusters each: 65,536 of 2 M rows 18.1 / 18.6,
-// 30,000 of 1500 13.9 / 13.2, so they have one each.  Clusters of eight as parts: 28.9 (four), 40.3 (sixteen)
-int table_parts(const dqrm_ctx *ctx)
+// moment: 34 us), from 16 K lookups on; of tables whose rows take two passes from 48 K, of those whose quarters take a pass less than
+// they do from 8 K.  Measured on B200 (us a backward; four clusters / one): 65,536 lookups of 4 M rows 26.5 / 35.3, Zipf 1.2 28.1 / 32.0, all in
+// the first quarter 27.7 / 34.2, nine tenths in one row 26.7 / 33.2, all in one 21.8 / 27.8; 25,000 21.1 / 23.2, 23.4 / 24.1, 23.4 /
+// 24.4, 23.8 / 24.5, 18.6 / 22.5; 17,000 20.4 / 21.5, but rows numbered by how often they come 23.4 / 22.8 (eight pipelined steps
+// around them 160 / 180); of 260 K rows 10,000 18.4 / 20.7; of 3000 rows 50,000 22.1 / 24.9, nine tenths in one row 22.5 / 23.2, 32,000 20.0 /
+// 21.1 but 21.1 / 20.0.  Two tables by two clusters each: 65,536 of 2 M rows 18.1 / 18.6 the sort, 30,000 of 1500 13.9 / 13.2, so they
+// have one each.  Clusters of eight as parts: 28.9 (four), 40.3 (sixteen)
+int table_parts(const dqrm_ctx *ctx, int64_t per_table)
 {
-    return 2 * ctx->T * csort::CLUSTER_WIDE * csort::MAX_PARTS <= ctx->num_sms ? csort::MAX_PARTS : 1;
+    if (ctx->T > 1 || per_table < csort::CLUSTER_WIDE * (ctx->row_bits <= 16 ? 3072 : ctx->row_bits <= 18 ? 512 : 1024)) return 1;
+    return 2 * csort::CLUSTER_WIDE * csort::MAX_PARTS <= ctx->num_sms ? csort::MAX_PARTS : 1;
 }
 
 // Clusters of eight of which only half works unless a table is large (cluster_sort_half_kernel).  33 clusters of eight run at
@@ -542,7 +547,7 @@ int dq_launch_bwd_sort(dqrm_ctx *ctx, const int32_t *indices, const int32_t *off
         const bool wide = wide_clusters(ctx, per_table, beside);
         e = cudaErrorUnknown;
         if (wide && lists_by_table && lists) {
-            ca.parts = table_parts(ctx);
+            ca.parts = table_parts(ctx, per_table);
             if (ca.parts > 1) e = launch_cluster_sort<csort::CLUSTER_WIDE, true>(ctx, ca, csort::choose_cap(per_table, csort::CLUSTER_WIDE), st);
             if (e != cudaSuccess) ca.parts = 1;
         }

@@ -39,16 +39,83 @@ __device__ __forceinline__ u32 same_digit_lanes(u32 d, bool valid)
     return valid ? peers : 0u;
 }
 
+// Rows [row0, row1) of a table alone that list `list` of MAX_PARTS takes; the same shares in every block, whose s_room takes
+// SAMPLE * (1 + THREADS / SAMPLE) words and a few.  Called by the block together.
+constexpr int SAMPLE = 128;
+__device__ __forceinline__ void share_rows(const Args &a, int64_t n, int64_t nrows, u32 *s_room, u32 list, int64_t &row0, int64_t &row1)
+{
+    constexpr int RANKERS = THREADS / SAMPLE;      // threads that rank a lookup of the sample, each against a part of it
+    static_assert(MAX_PARTS == 4 && SAMPLE % (4 * RANKERS) == 0, "");
+    u32 *s_rank = s_room + SAMPLE, *s_share = s_rank + THREADS, *s_cut = s_share + SAMPLE / 32 * 4;
+    const u32 tid = threadIdx.x, i = tid % SAMPLE, rows = (u32)nrows;
+    auto even = [&](u32 q) { return (u32)((uint64_t)rows * q >> 2); };
+    auto passes = [](u32 x) { return x <= 1 ? 0 : (39 - __clz(x - 1u)) / 8; };
+    row0 = even(list);
+    row1 = even(list + 1);
+    // (a quarter that takes a pass less than the table makes up for lookups that fall unevenly: 10,000 of 120 K rows that are numbered by
+    // how often they come 20.2 us a backward, at the quantiles 22.3, by one cluster 21.3; 65,536 29.4, 27.7, 32.4)
+    if (n < 32768 && passes((rows + 3) / 4) < passes(rows)) return;
+    u32 mine = 0;
+    if (tid < SAMPLE) {
+        mine = min((u32)max(__ldg(a.indices + tid * n / SAMPLE), 0), rows - 1u);
+        s_room[tid] = mine;
+        const u32 q = (mine >= even(1)) + (mine >= even(2)) + (mine >= even(3));
+        u32 share = 0;
+#pragma unroll
+        for (u32 k = 0; k < 4; ++k) {
+            const u32 in = __ballot_sync(0xffffffffu, q == k);
+            if ((tid & 31) == k) share = __popc(in);
+        }
+        if ((tid & 31) < 4) s_share[tid / 32 * 4 + (tid & 31)] = share;
+    }
+    __syncthreads();
+    u32 most = 0;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        u32 share = 0;
+#pragma unroll
+        for (int w = 0; w < SAMPLE / 32; ++w) share += s_share[w * 4 + q];
+        most = max(most, share);
+    }
+    // (a share of two fifths is sorted no later than the whole table by one cluster, and even shares often take a pass less)
+    if (most * 5 <= SAMPLE * 2) return;
+    const u32 me = s_room[i], j0 = tid / SAMPLE * (SAMPLE / RANKERS);
+    u32 rank = 0;
+#pragma unroll
+    for (u32 j = j0; j < j0 + SAMPLE / RANKERS; j += 4) {
+        const uint4 x = *reinterpret_cast<const uint4 *>(s_room + j);
+        rank += (x.x < me + (j < i)) + (x.y < me + (j + 1 < i)) + (x.z < me + (j + 2 < i)) + (x.w < me + (j + 3 < i));
+    }
+    s_rank[tid] = rank;
+    __syncthreads();
+    if (tid < SAMPLE) {
+#pragma unroll
+        for (int k = 1; k < RANKERS; ++k) rank += s_rank[k * SAMPLE + tid];
+        if (rank % (SAMPLE / 4) == 0) s_cut[rank / (SAMPLE / 4)] = mine;
+    }
+    __syncthreads();
+    u32 cut = 0;                                   // where share q begins: behind the one before, which has a row at least
+#pragma unroll
+    for (u32 q = 0; q < 4; ++q) {
+        if (q == list) row0 = cut;
+        cut = q < 3 ? min(rows, max(s_cut[q + 1], cut + 1u)) : rows;
+        if (q == list) row1 = cut;
+    }
+    __syncthreads();                               // (s_room is used again)
+}
+
 // What every block of the cluster does.  EPT > 0: for small batches whose tables may be uneven.  A table of up to THREADS * EPT
 // lookups, which is nearly all of them, is sorted by one of the cluster's blocks alone (sort_parts.cuh), and only a larger one by
 // the cluster.  Which block that is goes round the tables: from the sixteenth on clusters share their SMs with earlier ones, and two
 // working blocks on one SM take half as long again (26 tables of 2000 lookups: 11.5 us with the first block working in every
 // cluster, 8.2 this way, 8.5 without clusters; from 33 tables on 11.5, a third cluster waiting for its SMs).
 //
-// PARTS: few tables, of which one cluster each would leave most SMs idle.  a.parts clusters take a table, each a share of its rows: every one
-// reads all the table's lookups and keeps those of its rows, so nothing passes between the clusters; where its lookups stand behind those
-// of the rows before it counts itself, and its segments have lists of their own.  Rows are shared out evenly, lookups need not fall so: in the worst case
-// one cluster sorts them all, as it would alone.  A table beyond the blocks' shared memory is its first cluster's.
+// PARTS: a table alone, for which one cluster would leave most SMs idle.  a.parts clusters take it, each a share of its rows: every one
+// reads all lookups and keeps those of its rows, so nothing passes between the clusters; where its lookups stand behind those
+// of the rows before it counts itself, and its segments have lists of their own.  Rows are shared out evenly where a sample of the
+// lookups falls evenly, and otherwise at the sample's quantiles: rows may be numbered by how often they come (65,536 lookups all in
+// the first quarter of 4 M rows 36.4 us a backward with even shares, 27.7), and padding that is most of a batch becomes a share of one row.
+// All pairs fit the blocks' shared memory (the launch sees to that).
 //
 // OF: blocks launched for every cluster, of which CL call this, from block `from` on; the others have left.
 template <int CL, int EPT, bool PARTS, int OF = CL>
@@ -66,7 +133,7 @@ __device__ __forceinline__ void sort_by_cluster(const Args &a, unsigned from = 0
 
     cg::cluster_group cluster = cg::this_cluster();
     const unsigned rank0 = OF > CL ? from : 0u, c = cluster.block_rank() - rank0;
-    const int list = blockIdx.x / OF, t = PARTS ? list / a.parts : list, part = PARTS ? list % a.parts : 0;
+    const int list = blockIdx.x / OF, t = PARTS ? 0 : list;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const u32 lt = (1u << lane) - 1u;
 
@@ -76,9 +143,8 @@ __device__ __forceinline__ void sort_by_cluster(const Args &a, unsigned from = 0
     const int64_t n = tb1 - tb0;
     if (PARTS) {
         if (c == 0 && threadIdx.x == 0) {
-            if (part == 0) a.absmax[t] = 0u;
-            if (list + 1 == a.T * a.parts) a.tb[list + 1] = (u32)tb1;
-            if (n == 0) { a.tb[list] = (u32)tb0; a.table_cnt[list] = 0u; }
+            if (list == 0) a.absmax[0] = 0u;
+            if (list + 1 == MAX_PARTS) a.tb[MAX_PARTS] = (u32)tb1;
         }
     } else if (a.lists_by_table && c == 0 && threadIdx.x == 0) open_table(a, t, tb0, tb1);
     if constexpr (EPT > 0) {
@@ -89,15 +155,13 @@ __device__ __forceinline__ void sort_by_cluster(const Args &a, unsigned from = 0
     }
     if (n == 0) return;
     int npc = (int)(((n + CL - 1) / CL + 31) / 32 * 32);            // pairs per block
-    const bool in_smem = npc <= a.cap;
+    const bool in_smem = PARTS || npc <= a.cap;
     int my_n = (int)max((int64_t)0, min((int64_t)npc, n - (int64_t)c * npc));
     // the scatter divides every destination by npc: a float reciprocal gives the quotient (a block number,
     // since pos < n <= CL * npc) to within one, and one correction step settles it
     float npc_inv = 1.0f / (float)npc;
-    // the cluster's rows, its lookups and their place among the sorted ones (PARTS: known behind the first barrier)
-    const int64_t row0 = PARTS && in_smem ? nrows * part / a.parts : 0;
-    const int64_t row1 = PARTS ? (in_smem ? nrows * (part + 1) / a.parts : part == 0 ? nrows : 0) : nrows;
-    int64_t m = n, first = tb0;
+    // the cluster's rows, its lookups and their place among the sorted ones (PARTS: known further on)
+    int64_t row0 = 0, row1 = nrows, m = n, first = tb0;
 
     // buffers of this block for stage s (shared memory slices, or this block's part of the global staging)
     // a pair travels as one 8-byte store: distributed-shared-memory traffic is bound by the number of stores
@@ -128,11 +192,16 @@ __device__ __forceinline__ void sort_by_cluster(const Args &a, unsigned from = 0
         // each warp has a contiguous part of the slice: it counts its lookups that are kept, then puts them behind those of the warps before
         const int wsz = ((my_n + WARPS - 1) / WARPS + 31) / 32 * 32, w0 = min(my_n, warp * wsz), w1 = min(my_n, w0 + wsz);
         const int32_t *idx_c = a.indices + tb0 + (int64_t)c * npc;
-        u32 kept = 0, below = 0;
-        for (int i0 = w0; i0 < w1; i0 += 8 * 32) {
-            int32_t idx[8];
+        int32_t idx[8];
+        auto fetch = [&](int i0) {
 #pragma unroll
             for (int k = 0; k < 8; ++k) idx[k] = __ldg(idx_c + min(i0 + k * 32 + lane, my_n - 1));
+        };
+        if (w0 < w1) fetch(w0);                    // (on their way while the sample is looked at)
+        share_rows(a, n, nrows, &s_cnt[0][0], (u32)list, row0, row1);
+        u32 kept = 0, below = 0;
+        for (int i0 = w0; i0 < w1; i0 += 8 * 32) {
+            if (i0 != w0) fetch(i0);
 #pragma unroll
             for (int k = 0; k < 8; ++k) {
                 const bool valid = i0 + k * 32 + lane < w1;
@@ -178,7 +247,7 @@ __device__ __forceinline__ void sort_by_cluster(const Args &a, unsigned from = 0
                         }
                         bag = lo;
                     }
-                    pb0[to] = make_uint2((u32)(row - row0), a.payload_position ? (u32)(tb0 + p) : (u32)(bag * a.T + t));
+                    pb0[to] = make_uint2((u32)(row - row0), (u32)bag);
                 }
             }
         }
@@ -253,7 +322,7 @@ __device__ __forceinline__ void sort_by_cluster(const Args &a, unsigned from = 0
             }
             __syncthreads();
             m = s_sum[0];
-            first = tb0 + (in_smem ? s_sum[1] : part == 0 ? 0u : (u32)n);
+            first = tb0 + s_sum[1];
             npc = (int)(((m + CL - 1) / CL + 31) / 32 * 32);
             npc_inv = 1.0f / (float)npc;
             if (c == 0 && threadIdx.x == 0) a.tb[list] = (u32)first;
