@@ -359,7 +359,7 @@ template <int CL, bool PARTS = false>
 cudaError_t launch_cluster_sort(dqrm_ctx *ctx, csort::Args ca, int cap, cudaStream_t st)
 {
     ca.cap = cap;
-    return launch_clusters<CL>(ctx, csort::cluster_sort_kernel<CL, 0, PARTS>, PARTS ? 6 : CL == csort::CLUSTER ? 0 : 3, ca, csort::smem_bytes(cap), st);
+    return launch_clusters<CL>(ctx, csort::cluster_sort_kernel<CL, 0, PARTS>, PARTS ? 6 : CL == csort::CLUSTER_HALF ? 8 : CL == csort::CLUSTER ? 0 : 3, ca, csort::smem_bytes(cap), st);
 }
 
 cudaError_t launch_half_clusters(dqrm_ctx *ctx, csort::Args ca, int cap, cudaStream_t st)
@@ -393,14 +393,29 @@ int table_parts(const dqrm_ctx *ctx, int64_t per_table)
     return 2 * csort::CLUSTER_WIDE * csort::MAX_PARTS <= ctx->num_sms ? csort::MAX_PARTS : 1;
 }
 
-// Clusters of eight of which only half works unless a table is large (cluster_sort_half_kernel).  33 clusters of eight run at
-// once (two blocks an SM); beyond that the last of them wait for the first, and blocks that leave at once let them in.  Measured on B200
-// (us a backward, eight blocks / half of them): 34 tables of 2100 lookups 30.5 / 22.7, 40 of 4000 37.5 / 27.9, of 10,000 55.9 / 45.7, 46 of
+// Batches of an index a bag, whose tables are all alike: clusters of four blocks.  Where clusters of eight for all tables do not fit at
+// once (two blocks an SM: from 34 tables on) the last of them wait for the first: 40 tables of 4000 lookups 37.5 -> 26.7 us a backward, of
+// 10,000 55.9 -> 43.7, 64 of 4000 42.7 -> 30.3, eight pipelined steps around them (40 of 3000 of 16 features, of 16,000 of 8) 313 -> 213 and
+// 530 -> 426; the sort of 20,000 36.1 -> 40.5, four blocks have too much to do.  Where they fit, but share SMs (from 19 tables on): 26 tables of
+// 2500 lookups 21.2 -> 19.5 a backward, of 8000 29.7 -> 28.0, the sort of 9000 18.1 -> 18.4.  Beside a training step (dqrm_sort_batch) four
+// blocks leave it more room and take longer themselves, so that count the step's rows: 26 tables of 8000 lookups of 48 features 487 -> 452 us
+// for eight steps, of 16 282 -> 287, of 8 250 -> 266, of 2500 of 16 189 -> 160; they are taken there for rows of 32 features and
+// more, and for small tables.  (A batch that has as many lookups as bags without one in each, and most of them in one table, pays for it:
+// 26 tables of 8000 with nine tenths in one 240 -> 430.  All that is known at the launch are the two numbers.)
+bool narrow_clusters(const dqrm_ctx *ctx, int64_t per_table, bool beside)
+{
+    if (ctx->T * csort::CLUSTER > 2 * ctx->num_sms) return per_table <= 16384;
+    return ctx->T * csort::CLUSTER > ctx->num_sms && per_table <= (!beside || ctx->D >= 32 ? 8192 : 2560);
+}
+
+// Other batches, of which one table may hold most, and the merge of ranks' gradients: clusters of eight of which half works unless a table
+// is large (cluster_sort_half_kernel).  33 clusters of eight run at once; blocks that leave at once let those beyond in.  Measured on B200
+// (us a backward; eight blocks / half of them): 34 tables of 2100 lookups 30.5 / 22.7, 40 of 4000 37.5 / 27.9, of 10,000 55.9 / 45.7, 46 of
 // 16,000 70.3 / 59.9, 58 of 12,000 63.5 / 54.0, 64 of 2100 35.3 / 34.6, of 8000 54.7 / 56.2, of 12,000 66.5 / 74.1 (two full rounds of clusters
-// of eight), 70 of 16,000 100.2 / 98.3, 148 of 6000 109.1 / 84.5; 33 of 6000 27.3 / 30.0; 36 of 12,000 52.8 / 53.3.  With nine tenths of the lookups in one table
-// as before: 40 of 4000 194 / 194, 64 of 4000 287 / 288 (clusters of four in every table 344 and 524).
-// Beside a training step (dqrm_sort_batch) of rows of 32 features and more the room counts from 19 tables on, where clusters begin to
-// share SMs: eight pipelined steps of 26 tables of 2500 lookups of 32 features 225 / 205, of 8000 of 48 487 / 455; of 2500 of 16 189 / 195
+// of eight), 70 of 16,000 100.2 / 98.3, 148 of 6000 109.1 / 84.5; 33 of 6000 27.3 / 30.0; 36 of 12,000 52.8 / 53.3.  With nine tenths
+// of the lookups in one table as before: 40 of 4000 194 / 194, 64 of 4000 287 / 288 (clusters of four in every table 344 and 524).
+// Beside a training step of rows of 32 features and more the room counts from 19 tables on: eight pipelined steps of 26 tables of 2500
+// lookups of 32 features 225 / 205, of 8000 of 48 487 / 455; of 2500 of 16 189 / 195
 bool half_clusters(const dqrm_ctx *ctx, int64_t per_table, bool beside)
 {
     constexpr int AT_ONCE = 33;
@@ -552,7 +567,9 @@ int dq_launch_bwd_sort(dqrm_ctx *ctx, const int32_t *indices, const int32_t *off
             if (e != cudaSuccess) ca.parts = 1;
         }
         if (wide && e != cudaSuccess) e = launch_cluster_sort<csort::CLUSTER_WIDE>(ctx, ca, csort::choose_cap(per_table, csort::CLUSTER_WIDE), st);
-        if (e != cudaSuccess && half_clusters(ctx, per_table, beside))
+        if (e != cudaSuccess && L == G && lists_by_table && narrow_clusters(ctx, per_table, beside))
+            e = launch_cluster_sort<csort::CLUSTER_HALF>(ctx, ca, csort::choose_cap(per_table, csort::CLUSTER_HALF), st);
+        else if (e != cudaSuccess && half_clusters(ctx, per_table, beside))
             e = launch_half_clusters(ctx, ca, csort::choose_cap(per_table, csort::CLUSTER_HALF), st);
         if (e != cudaSuccess) e = launch_cluster_sort<csort::CLUSTER>(ctx, ca, csort::choose_cap(per_table, csort::CLUSTER), st);
         if (e == cudaSuccess) {

@@ -275,7 +275,7 @@ def test_wide_clusters(oracle, T, per_table, rows):
         c.ctx.close()
 
 
-# many tables, which half of a cluster's blocks sort: on both sides of the numbers of tables and lookups at which they do
+# many tables, which four blocks or half of a cluster's sort: on both sides of the numbers of tables and lookups at which they do
 @pytest.mark.parametrize("D", [8, 36])
 @pytest.mark.parametrize("T,per_table", [(18, 2_100), (19, 2_100), (19, 8_192), (19, 8_200), (37, 2_561), (38, 2_600), (38, 9_000), (40, 16_384),
                                          (33, 2_100), (34, 2_100), (34, 8_193), (59, 4_096), (59, 4_097), (66, 4_096), (67, 4_097)])
@@ -306,16 +306,18 @@ def test_narrow_clusters(oracle, T, per_table, D):
         c.ctx.close()
 
 
-# clusters of which half works: a table that fits their shared memory to the last pair (3200 at a mean of 2500 lookups a table), one pair
-# more, the last pair that all eight blocks hold, and beyond; in tables of both halves
+# clusters of four blocks (as many lookups as bags) and clusters of eight of which half works: a table that fits four blocks' shared memory
+# to the last pair (3200 at a mean of 2500 lookups a table), one pair more, the last pair that eight blocks hold, and beyond; in
+# tables of both halves
+@pytest.mark.parametrize("even", [True, False])
 @pytest.mark.parametrize("T", [34, 40, 66])
 @pytest.mark.parametrize("large", [3_199, 3_200, 3_201, 6_400, 6_401, 40_000])
-def test_tables_beyond_half_a_cluster(oracle, T, large):
+def test_tables_beyond_half_a_cluster(oracle, T, large, even):
     rng = np.random.default_rng(T + large)
     D, B = 8, 2_500
     counts = np.full(T, (T * B - 2 * large) // (T - 2))
     counts[[2, T - 1]] = large
-    counts[0] += T * B - counts.sum()
+    counts[0] += T * B - counts.sum() - (not even)
     rows = tuple(int(r) for r in rng.choice([1, 300, 70_000], T))
     lens = np.zeros((T, B), dtype=np.int64)
     for t, n in enumerate(counts):
