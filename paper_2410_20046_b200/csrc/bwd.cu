@@ -716,17 +716,31 @@ int dq_launch_small_step(dqrm_ctx *ctx, float *tables, const int32_t *indices, c
                               ws_bytes, st);
 }
 
+// A backward that stands alone (behind it a step would read the workspace's maxima) in one launch instead of two: up to 3072 lookups of
+// an index a bag, fewer of rows of less than 16 features, 64 K gathered values, unless they are many tables of up to 64.  Measured on
+// B200 (us a backward in graph replay; two launches / one): 4 tables of 128 lookups of 16 features 9.5 / 7.2, of 512 11.6 / 10.4, 16 of
+// 200 10.9 / 10.2, of 128 of 32 features 10.4 / 9.1, 2 of 100 of 128 10.0 / 8.1; around it the four calls of 16 tables of 200 22.0 / 20.0, of
+// 26 of 64 19.0 / 18.2, of 26 of 90 22.0 / 20.0, but of 26 of 128 20.0 / 20.2 to 20.8, of 48 of 64 19.8 / 21.2, of 8 of 512 21.1 / 21.5
+// to 22.1, of 10 of 400 19.7 / 21.0 where tables have three rows, and of 26 of 128 of 8 features 19.2 / 20.6.  (The block counts the
+// lookups in front of its own by their rows; all in one row they wait for one another: 8 tables of 256 of one row each 20.5 / 22.9.)
+// Other batches may lie in one table, whose block then does everything: up to 1100 lookups and 32 K values.  13 tables of 40 bags of two
+// 13.4 / 7.5, with nine tenths of the lookups in one 16.1 / 14.5; 4 of 90 bags of four 11.3 / 8.8, but 15.5 / 20.2; 4 of 64 bags of four of
+// 16 features 13.4 / 8.2 and 15.7 / 15.6; 10 of 25 of 32 features 13.6 / 7.5 and 15.5 / 17.5.
+static bool small_bwd_takes_alone(const dqrm_ctx *ctx, int B, int64_t L)
+{
+    if (L == (int64_t)ctx->T * B) {
+        if (L > std::min(3072, 192 * ctx->D) || L * ctx->D > 65536 || (L > 2048 && B <= 64)) return false;
+    } else if (L > 1100 || L * 4 * segred::lanes_per_row(ctx->D) > 32768) {        // (with the features that idle lanes stand for)
+        return false;
+    }
+    return small_bwd_takes(ctx, B, L);
+}
+
 int dq_launch_bwd(dqrm_ctx *ctx, const float *grad_out, const int32_t *indices, const int32_t *offsets,
                   int32_t *unique_rows, int32_t *uniq_off, float *grad_rows, int B, int64_t L,
                   void *ws, size_t ws_bytes, cudaStream_t st, bool alone)
 {
-    // Up to 64 K gathered values a backward that stands alone (behind it a step would read the workspace's maxima) is one launch instead of
-    // two; while launches are timed one by one they stay two.  Measured on B200 (us, graph replay; two launches / one): 4 tables of 128
-    // lookups of 16 features 9.5 / 7.2, of 512 11.3 / 9.8, one of 400 10.8 / 8.2, 4 of 90 bags of four 13.4 / 9.7, 2 of 100 of 128
-    // features 10.0 / 8.1, 40 of 80 of 16 11.6 / 10.9, 26 of 128 10.1 / 10.1 (the four calls around it 20.2 / 19.7); 26 of 128 of 64
-    // 10.1 / 11.0, 16 of 256 of 64 10.6 / 13.3
-    if (alone && L * ctx->D <= 65536 && !ctx->prof_on && small_bwd_takes(ctx, B, L) && dq_aligned(grad_out, sizeof(float4)) &&
-        dq_aligned(grad_rows, sizeof(float4)))
+    if (alone && !ctx->prof_on && small_bwd_takes_alone(ctx, B, L) && dq_aligned(grad_out, sizeof(float4)) && dq_aligned(grad_rows, sizeof(float4)))
         return launch_small<false>(ctx, nullptr, indices, offsets, grad_out, unique_rows, uniq_off, grad_rows, nullptr, nullptr, 0.f, B, L, ws,
                                    ws_bytes, st);
     int lists = 0;

@@ -111,25 +111,43 @@ def test_contexts_of_many_and_of_few_tables_take_turns(oracle):
         c.ctx.close()
 
 
-BACKWARDS = dict(SHAPES, most_values=(64, [512, 512]), a_value_more=(64, [512, 511, 2]), most_lookups=(16, [256] * 16), most_of_a_table=(32, [512, 1, 0, 300]))
+# the backward alone: feature size, lookups per table, launches: one up to the line, two (sort and sum) beyond it.  An index a bag:
+ALONE_EVEN = {
+    "single": (16, [1], 1), "tiny": (16, [128] * 4, 1), "most_lookups": (16, [256] * 12, 1), "a_table_more": (16, [256] * 13, 2),
+    "most_values": (32, [256] * 8, 1), "a_table_of_values_more": (32, [256] * 9, 2), "most_of_a_table": (32, [512] * 2, 1),
+    "a_table_too_long": (16, [513] * 2, 2), "a_table_too_wide": (64, [257] * 2, 2), "narrow": (4, [384] * 2, 1), "too_narrow": (4, [385] * 2, 2),
+    "many_tables": (16, [64] * 32, 1), "one_too_many": (16, [64] * 33, 2), "idle_lanes": (20, [90] * 7, 1), "wide": (128, [128] * 4, 1),
+}
+# and others:
+ALONE_UNEVEN = {
+    "empty_tables": (4, [0, 3, 0, 0, 40, 0], 1), "one_holds_most": (16, [3, 0, 1064, 33], 1), "and_one_more": (16, [3, 0, 1065, 33], 2),
+    "widest": (64, [500, 1, 11], 1), "too_wide": (64, [501, 1, 11], 2), "idle_lanes": (20, [33, 934, 57], 1), "idle_lanes_more": (20, [33, 935, 57], 2),
+    "many_tables": (8, [1, 0, 7, 13] * 30, 1), "in_memory": (8, [0, 2, 900, 1], 1),
+}
 
 
 @pytest.mark.parametrize("rows", [1, 9, 50_000])
-@pytest.mark.parametrize("name", list(BACKWARDS))
+@pytest.mark.parametrize("name", list(ALONE_EVEN) + ["uneven " + k for k in ALONE_UNEVEN])
 def test_small_backward(oracle, name, rows):
     """The backward alone in one launch, on both sides of what it takes."""
-    D, counts = BACKWARDS[name]
-    T, B = len(counts), max(1, max(counts))
+    even = not name.startswith("uneven ")
+    D, counts, launches = ALONE_EVEN[name] if even else ALONE_UNEVEN[name[7:]]
+    T, B = len(counts), counts[0] if even else max(counts)
     wl = W.Workload("bwd", tuple(rows + t for t in range(T)), D=D, B=B, alpha=None)
     rng = np.random.default_rng(rows + B + D)
     idx = np.concatenate([rng.integers(0, wl.rows[t], n) for t, n in enumerate(counts)]).astype(np.int32)
-    lens = np.zeros((T, B), dtype=np.int64)
-    for t, n in enumerate(counts):
-        np.add.at(lens[t], rng.integers(0, B, n) if t % 2 else np.arange(n), 1)
+    lens = np.ones((T, B), dtype=np.int64)
+    if not even:
+        lens[:] = 0
+        for t, n in enumerate(counts):
+            np.add.at(lens[t], rng.integers(0, B, n) if t % 2 else np.arange(n), 1)
     off = np.concatenate([[0], np.cumsum(lens.reshape(-1))]).astype(np.int32)
+    assert len(idx) == off[-1] and (len(idx) == T * B) == even
     go = (rng.integers(-1024, 1025, (B, T, D)) / 256).astype(np.float32)      # (exact sums, as above)
     c = Case(wl, max_lookups=len(idx))
+    before = c.ctx.launch_count()
     got, want = c.gpu_bwd(idx, off, go), oracle.emb_bwd(go, T, D, B, idx, off)
-    for g, w in zip(got, (want[0], want[1], want[2])):
+    assert c.ctx.launch_count() - before == launches
+    for g, w in zip(got, want[:3]):
         assert bit_equal(g, w)
     c.ctx.close()
