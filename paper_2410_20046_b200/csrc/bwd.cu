@@ -740,7 +740,7 @@ int dq_launch_bwd(dqrm_ctx *ctx, const float *grad_out, const int32_t *indices, 
                   int32_t *unique_rows, int32_t *uniq_off, float *grad_rows, int B, int64_t L,
                   void *ws, size_t ws_bytes, cudaStream_t st, bool alone)
 {
-    if (alone && !ctx->prof_on && small_bwd_takes_alone(ctx, B, L) && dq_aligned(grad_out, sizeof(float4)) && dq_aligned(grad_rows, sizeof(float4)))
+    if (alone && small_bwd_takes_alone(ctx, B, L) && dq_aligned(grad_out, sizeof(float4)) && dq_aligned(grad_rows, sizeof(float4)))
         return launch_small<false>(ctx, nullptr, indices, offsets, grad_out, unique_rows, uniq_off, grad_rows, nullptr, nullptr, 0.f, B, L, ws,
                                    ws_bytes, st);
     int lists = 0;

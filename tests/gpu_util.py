@@ -71,6 +71,28 @@ class Case:
         assert (ur_h[U:] == -7).all() and np.isnan(gr_h[U:]).all()
         return ur_h[:U].copy(), uo_h, gr_h[:U].copy()
 
+    def gpu_bwd_two_calls(self, idx, off, grad_out, ws=0):
+        """The same in the two-call form of a step that changes no row: the sort and the sum are kernels of their own however
+        small the batch is."""
+        t = self.torch
+        L, T, B, D = len(idx), self.wl.T, self.wl.B, self.wl.D
+        ur = t.full((L,), -7, dtype=t.int32, device="cuda")
+        uo = self.empty(T + 1, t.int32)
+        gr = t.full((L, D), float("nan"), dtype=t.float32, device="cuda")
+        d_idx, d_off = self.dev(idx), self.dev(off)
+        tables = t.zeros((int(self.row_off[-1]), D), dtype=t.float32, device="cuda")
+        out, codes, gs = self.empty((B, T, D), t.float32), self.empty((L, D), t.int8), self.empty(T, t.float32)
+        scales = t.ones(T, dtype=t.float32, device="cuda")
+        self.ctx.sort_batch(d_idx, d_off, ur, uo, B=B, L=L, ws=ws)
+        self.ctx.train_step_sorted(tables, d_idx, d_off, self.dev(grad_out), scales, self.bits, out, ur, uo, gr, codes, gs, 0.0, B=B,
+                                   L=L, ws=ws)
+        self.ctx.raise_on_device_error()
+        uo_h = uo.cpu().numpy()
+        U = int(uo_h[-1])
+        ur_h, gr_h = ur.cpu().numpy(), gr.cpu().numpy()
+        assert (ur_h[U:] == -7).all() and np.isnan(gr_h[U:]).all()
+        return ur_h[:U].copy(), uo_h, gr_h[:U].copy()
+
     def gpu_quant(self, grad_rows, uniq_off):
         t = self.torch
         U = grad_rows.shape[0]

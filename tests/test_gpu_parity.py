@@ -418,7 +418,7 @@ def test_gradient_scales_of_a_batch_with_unusable_boundaries(oracle, B, calls):
 
 
 # bags per table and mean indices per bag: tables that one block sorts, tables that their clusters sort, a radix sort
-@pytest.mark.parametrize("B,bag,sort_path,kernel", [(300, 1, 0, "small_sort_kernel"), (1500, 3, 0, "cluster_sort_kernel"),
+@pytest.mark.parametrize("B,bag,sort_path,kernel", [(600, 1, 0, "small_sort_kernel"), (1500, 3, 0, "cluster_sort_kernel"),
                                                     (1500, 3, 1, "rs_scatter_kernel")])
 @pytest.mark.parametrize("fault", ["decrease", "boundary"])
 def test_unusable_offsets_by_sort(oracle, B, bag, sort_path, kernel, fault):

@@ -108,7 +108,7 @@ def test_runs_of_lane_groups(oracle, n, D):
     go = rng.standard_normal((B, wl.T, D)).astype(np.float32)
     go[rng.random(go.shape) < 0.1] = -0.0
     c = Case(wl, max_lookups=len(idx))
-    ur, uo, gr = c.gpu_bwd(idx, off, go)
+    ur, uo, gr = c.gpu_bwd_two_calls(idx, off, go)
     o_ur, o_uo, o_gr = oracle.emb_bwd(go, wl.T, D, B, idx, off)
     assert bit_equal(uo, o_uo) and bit_equal(ur, o_ur)
     # nine terms of magnitude below 6 in FP64 in two orders, each sum rounded once
@@ -369,6 +369,6 @@ def test_profile_names_the_kernel(D, kernel):
     wl = W.Workload("names", (50,), D=D, B=B, alpha=None)
     c = Case(wl)
     c.ctx.profile_begin()
-    c.gpu_bwd(np.arange(B, dtype=np.int32) % 50, np.arange(B + 1, dtype=np.int32), np.ones((B, 1, D), dtype=np.float32))
+    c.gpu_bwd_two_calls(np.arange(B, dtype=np.int32) % 50, np.arange(B + 1, dtype=np.int32), np.ones((B, 1, D), dtype=np.float32))
     assert set(c.ctx.profile_end()) & {"seg_groups_kernel", "seg_sum_kernel"} == {kernel}
     c.ctx.close()

@@ -29,7 +29,7 @@ def test_block_sort(oracle, name, rows):
     off = np.concatenate([[0], np.cumsum(lens.reshape(-1))]).astype(np.int32)
     go = rng.standard_normal((B, wl.T, D)).astype(np.float32)
     c = Case(wl, max_lookups=len(idx))
-    ur, uo, gr = c.gpu_bwd(idx, off, go)
+    ur, uo, gr = c.gpu_bwd_two_calls(idx, off, go)
     o_ur, o_uo, o_gr = oracle.emb_bwd(go, wl.T, D, B, idx, off)
     assert bit_equal(uo, o_uo) and bit_equal(ur, o_ur)
     # at most 4000 terms of magnitude below 6 in FP64 in two orders, each sum rounded once
@@ -63,7 +63,7 @@ def test_uneven_tables(oracle, name, rows):
     go = rng.standard_normal((B, wl.T, D)).astype(np.float32)
     c = Case(wl, max_lookups=len(idx))
     c.ctx.profile_begin()
-    ur, uo, gr = c.gpu_bwd(idx, off, go)
+    ur, uo, gr = c.gpu_bwd_two_calls(idx, off, go)
     names = set(c.ctx.profile_end())
     assert names & {"small_sort_kernel", "cluster_sort_kernel", "rs_scatter_kernel"} == {kernel}, names
     o_ur, o_uo, o_gr = oracle.emb_bwd(go, wl.T, D, B, idx, off)
@@ -88,7 +88,7 @@ def test_block_radix_sort(oracle, rows, n):
     go = rng.standard_normal((n, T, D)).astype(np.float32)
     c = Case(wl)
     c.ctx.profile_begin()
-    ur, uo, gr = c.gpu_bwd(idx, off, go)
+    ur, uo, gr = c.gpu_bwd_two_calls(idx, off, go)
     assert "small_sort_kernel" in c.ctx.profile_end()
     o_ur, o_uo, o_gr = oracle.emb_bwd(go, T, D, n, idx, off)
     assert bit_equal(uo, o_uo) and bit_equal(ur, o_ur)

@@ -129,7 +129,7 @@ ALONE_UNEVEN = {
 @pytest.mark.parametrize("rows", [1, 9, 50_000])
 @pytest.mark.parametrize("name", list(ALONE_EVEN) + ["uneven " + k for k in ALONE_UNEVEN])
 def test_small_backward(oracle, name, rows):
-    """The backward alone in one launch, on both sides of what it takes."""
+    """The backward alone in one launch, on both sides of what it takes; what the profile names is what runs."""
     even = not name.startswith("uneven ")
     D, counts, launches = ALONE_EVEN[name] if even else ALONE_UNEVEN[name[7:]]
     T, B = len(counts), counts[0] if even else max(counts)
@@ -148,6 +148,10 @@ def test_small_backward(oracle, name, rows):
     before = c.ctx.launch_count()
     got, want = c.gpu_bwd(idx, off, go), oracle.emb_bwd(go, T, D, B, idx, off)
     assert c.ctx.launch_count() - before == launches
-    for g, w in zip(got, want[:3]):
-        assert bit_equal(g, w)
+    c.ctx.profile_begin()
+    again = c.gpu_bwd(idx, off, go)
+    named = c.ctx.profile_end()
+    assert sum(n for _, n in named.values()) == launches and ("small_step_kernel" in named) == (launches == 1), named
+    for g, a, w in zip(got, again, want[:3]):
+        assert bit_equal(g, w) and bit_equal(a, w)
     c.ctx.close()
