@@ -45,7 +45,8 @@ struct Layout {
     size_t total;
 };
 
-Layout make_layout(const dqrm_ctx *ctx, int64_t L)
+// one_index: the batch has at most an index a bag on average; where the parts lie does not depend on it
+Layout make_layout(const dqrm_ctx *ctx, int64_t L, bool one_index = false)
 {
     Layout y;
     y.passes = (ctx->row_bits + rsort::MAX_DIGIT_BITS - 1) / rsort::MAX_DIGIT_BITS;
@@ -59,12 +60,11 @@ Layout make_layout(const dqrm_ctx *ctx, int64_t L)
                                                  : (int64_t)ctx->num_sms * segred::sum_blocks(segred::floats_per_lane(ctx->D)) /
                                                        segred::column_blocks(ctx->D) * segred::WARPS;
     if (warps < 1) warps = 1;
-    y.sum_small = Lc < 96 * warps;         // (three tiles of 32 a warp: 160 K rows of 192 bytes 38.9 -> 28.7 us, 208 K of
-                                              // 256 bytes 30.7 -> 28.7; at 852 K rows tiles of 32 are 2 us the faster)
+    y.sum_small = segred::small_tiles(ctx->D, Lc, warps, one_index);
     const int I = segred::tile_entries(y.sum_small);
     y.sum_shift = segred::takes_groups(ctx->D) ? segred::CHUNK_SHIFT : segred::chunk_shift(y.sum_small);
     y.sum_tiles = (Lc + I - 1) / I;
-    y.range_tiles = segred::range_tiles(ctx->D, y.sum_tiles, warps);
+    y.range_tiles = segred::range_tiles(ctx->D, y.sum_tiles, warps, y.sum_small);
     const int64_t groups = 32 / segred::lanes_per_row(ctx->D), chunk = (int64_t)1 << segred::CHUNK_SHIFT;
     y.sum_span = (int)(((Lc + warps * groups - 1) / (warps * groups) + chunk - 1) / chunk * chunk);
     y.sum_ranges = (Lc + y.sum_span * groups - 1) / (y.sum_span * groups);
@@ -499,10 +499,10 @@ int dq_launch_bwd_sort(dqrm_ctx *ctx, const int32_t *indices, const int32_t *off
                        void *ws_, size_t ws_bytes, cudaStream_t st, bool lists_by_table, bool *by_table, int *lists,
                        bool beside)
 {
-    const Layout y = make_layout(ctx, L);
+    const int64_t G = (int64_t)ctx->T * B;
+    const Layout y = make_layout(ctx, L, L <= G);
     if (ws_bytes < y.total) return DQRM_ERR_WORKSPACE;
     char *ws = reinterpret_cast<char *>(ws_);
-    const int64_t G = (int64_t)ctx->T * B;
     if (by_table) *by_table = false;
     if (lists) *lists = 0;
     const bool fits_cluster = (L + ctx->T - 1) / ctx->T <= (int64_t)csort::CLUSTER * 12288;   // (a table beyond its
@@ -619,7 +619,7 @@ int dq_launch_bwd_sort(dqrm_ctx *ctx, const int32_t *indices, const int32_t *off
 int dq_launch_bwd_sum(dqrm_ctx *ctx, const float *grad_out, int32_t *unique_rows, int32_t *uniq_off, float *grad_rows,
                       int B, int64_t L, int lists, void *ws_, size_t ws_bytes, cudaStream_t st)
 {
-    const Layout y = make_layout(ctx, L);
+    const Layout y = make_layout(ctx, L, L <= (int64_t)ctx->T * B);
     if (ws_bytes < y.total) return DQRM_ERR_WORKSPACE;
     if (L == 0) return DQRM_OK;
     char *ws = reinterpret_cast<char *>(ws_);

@@ -39,21 +39,34 @@ __host__ __device__ constexpr int column_blocks(int D) { return (D + 127) / 128;
 // resident block: 852 K rows of 256 bytes 58.4 -> 56.5 us, 1.3 M in bags of twenty 97.9 -> 89.7 (eight rows and three blocks
 // before; five blocks 65 and more: values are spilled).  With four features a lane a fourth block spills, 984 K rows of 512 bytes 82 -> 119
 constexpr int BATCH_ROWS = 4;
-// A warp that has one tile takes its batches of rows one after the other, 4 to 8 us for 32 rows, so a batch of wide
-// rows that would give every resident warp less than three tiles of 32 entries is cut into tiles of 8
 __host__ __device__ constexpr int tile_entries(bool small) { return small ? 8 : 32; }
 __host__ __device__ constexpr int chunk_shift(bool small) { return small ? 3 : 5; }    // of chunk_first
 __host__ __device__ constexpr int sum_blocks(int vec) { return vec == 2 ? 4 : 3; }
-// A warp that would get more than a dozen tiles gets eight, and there are more blocks than the GPU holds at once: they pass over the
-// tables one after the other, each table's share of grad_out stays in L2 while it is read from all sides, and warps with many short runs
-// hold up fewer others.  8.5 M rows of 256 bytes (multi-hot) 306 us with one range for every resident warp, 285 with ranges of sixteen
-// tiles, 276 with eight; a loop over the ranges in each warp, instead of more blocks, costs registers (356).  With four
-// features a lane it does not help: 1.6 M rows of 512 bytes 116 -> 122
+// Tiles of 8 entries instead of 32.  A warp that has one tile takes its batches of rows one after the other, 4 to 8 us for 32 rows, so a
+// batch that would give every resident warp less than three tiles of 32 is cut into tiles of 8 (160 K rows of 192 bytes 38.9 ->
+// 28.7 us, 208 K of 256 bytes 30.7 -> 28.7).  Rows of two features a lane, for which four blocks are resident: with an index a bag tiles
+// of 8 are never the slower (us a backward of 64 features, tiles of 32 / of 8, uniform indices and Zipf 1.1: 343 K rows 71.3 / 59.8 and
+// 56.2 / 52.9, 468 K 90.3 / 74.0 and 67.1 / 63.8, 852 K 147 / 124 and 99.2 / 97.6, 1.6 M 286 / 240 and 187 / 183, 2.4 M 421 / 362 and 284 / 274); in
+// bags tiles of 32 are ahead from where three blocks would have three of them (400 K rows in bags of twenty 79.2 / 80.5 and 60.1 /
+// 63.1, 900 K in bags of nine 154 / 160 and 126 / 138)
+inline bool small_tiles(int D, int64_t L, int64_t warps, bool one_index)
+{
+    return floats_per_lane(D) == 2 ? one_index || L < 72 * warps : L < 96 * warps;
+}
+// A warp that would get more than sixteen tiles of 32 gets eight, and there are more blocks than the GPU holds at once: they pass over
+// the tables one after the other, each table's share of grad_out stays in L2 while it is read from all sides, and warps with many short
+// runs hold up fewer others.  Measured on B200 (us a backward of 64 features, one range for every resident warp / of eight tiles, Zipf 1.1):
+// 8.5 M rows in bags of twenty 546 / 512, 5.1 M in bags of twelve 363 / 346, 3.6 M 261 / 253, 3.3 M in bags of two 337 / 312, 2 M in bags of
+// twelve 167 / 172.  Where lanes stand idle the line is eighteen, and from 24 tiles on a range has twelve: 52 features, one range / eight
+// tiles / twelve: 8.5 M 643 / 678 / 656, 5.1 M 424 / 442 / 433, 3.6 M 304 / 317 / 311 (uniform 384 / 373 / 372), 3.3 M in bags of two 390 / 358 /
+// 363, 2.6 M 248 / 268 / 277.  A loop over the ranges in each warp, instead of more blocks, costs registers (356 against 276 us a sum).
+// With four features a lane it does not help: 1.6 M rows of 512 bytes 116 -> 122
 constexpr int RANGE_TILES = 8;
-inline int range_tiles(int D, int64_t tiles, int64_t warps)
+inline int range_tiles(int D, int64_t tiles, int64_t warps, bool small)
 {
     const int64_t even = (tiles + warps - 1) / warps;
-    return (int)(floats_per_lane(D) == 2 && even > RANGE_TILES + RANGE_TILES / 2 ? RANGE_TILES : even);
+    if (small || floats_per_lane(D) != 2 || even <= (D == 64 ? 16 : 18)) return (int)even;
+    return D == 64 || even < 24 ? RANGE_TILES : RANGE_TILES + RANGE_TILES / 2;
 }
 // of such ranges, for L lookups (rows of 48 features and fewer have ranges of their own, seg_groups.cuh)
 inline int64_t max_ranges(int D, int64_t L) { return D > 48 && floats_per_lane(D) == 2 ? L / (32 * RANGE_TILES) + 1 : 0; }

@@ -100,6 +100,27 @@ int eight_blocks_a_table()
     return 0;
 }
 
+// rows of two features a lane: an index a bag is summed by tiles of 8 whatever the batch's size, bags by tiles of 32 from 341 K lookups
+// on; long bags by ranges of a few tiles, of which there are no more than the workspace has room for
+int tiles_of_the_sum()
+{
+    const int64_t warps = 148 * 4 * 8;
+    auto cut = [](int64_t n, int64_t by) { return (n + by - 1) / by; };
+    for (const int D : {52, 64})
+        for (const int64_t L : {300000LL, 350000LL, 468000LL, 852000LL, 2000000LL, 2600000LL, 3000000LL, 3700000LL, 8500000LL})
+            for (const bool bags : {false, true}) {
+                Ctx x(4, D);
+                const int B = (int)(bags ? L / 8 : L / 4);
+                const bool small = !bags || L < 72 * warps;
+                const int64_t tiles = cut(L, small ? 8 : 32), even = cut(tiles, warps);
+                const int64_t range = small || even <= (D == 64 ? 16 : 18) ? even : D == 64 || even < 24 ? 8 : 12;
+                WANT(dq_launch_bwd_sum(&x.c, nullptr, dummy, dummy, nullptr, B, L, 1, workspace, (size_t)1 << 40, nullptr) == DQRM_OK);
+                WANT((int64_t)fake::grid_x == cut(cut(tiles, range), 8));
+                WANT(cut(tiles, range) <= std::max(warps, L / 256 + 1));
+            }
+    return 0;
+}
+
 }  // namespace
 
 int main(int argc, char **argv)
@@ -109,6 +130,7 @@ int main(int argc, char **argv)
     if (!strcmp(name, "refused_sorts")) return refused_sorts();
     if (!strcmp(name, "clusters_stand_by")) return clusters_stand_by();
     if (!strcmp(name, "eight_blocks_a_table")) return eight_blocks_a_table();
+    if (!strcmp(name, "tiles_of_the_sum")) return tiles_of_the_sum();
     std::printf("no scenario %s\n", name);
     return 2;
 }

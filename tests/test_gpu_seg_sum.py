@@ -336,18 +336,20 @@ def test_tables_beyond_half_a_cluster(oracle, T, large, even):
     c.ctx.close()
 
 
-# more than a dozen tiles of 32 for each of the 4736 warps that 148 SMs hold: ranges of eight tiles, several of them for a warp's place
-@pytest.mark.parametrize("D", [52, 64])
+# more than a dozen tiles of 32 for each of the 4736 warps that 148 SMs hold: one range for each of them, and from sixteen tiles on (64
+# features; eighteen) ranges of eight (of twelve), several of them for a warp's place
+@pytest.mark.parametrize("D,most", [(52, 36), (64, 36), (64, 46), (52, 51), (52, 64)])
 @pytest.mark.parametrize("sort_path", [0, 1])
-def test_ranges_beyond_the_resident_warps(oracle, D, sort_path):
+def test_ranges_beyond_the_resident_warps(oracle, D, most, sort_path):
     rng = np.random.default_rng(D)
     rows, B = (40_000, 3, 900_000), 40_003
     T = len(rows)
     wl = W.Workload("ranges", rows, D=D, B=B, alpha=None)
-    lens = rng.integers(0, 36, T * B)
+    lens = rng.integers(0, most, T * B)
     off = np.concatenate([[0], np.cumsum(lens)]).astype(np.int32)
     L = int(off[-1])
-    assert L > 32 * 13 * 4736
+    tiles = {36: 13, 46: 17, 51: 19, 64: 24}[most]
+    assert -(-L // (32 * 4736)) >= tiles
     table = np.repeat(np.arange(T), lens.reshape(T, B).sum(1))
     idx = (rng.random(L) ** rng.choice([1, 8], L) * np.array(rows)[table]).astype(np.int32)      # runs of one to hundreds of thousands
     go = rng.standard_normal((B, T, D), dtype=np.float32)
@@ -358,6 +360,26 @@ def test_ranges_beyond_the_resident_warps(oracle, D, sort_path):
     assert bit_equal(uo, o_uo) and bit_equal(ur, o_ur)
     # n terms of magnitude below 6 in FP64 in two orders, each sum rounded once
     n = int(np.bincount(idx + 1_000_000 * table).max())
+    np.testing.assert_allclose(gr, o_gr, rtol=2.0 ** -23, atol=12.0 * n * n * 2.0 ** -53)
+    c.ctx.close()
+
+
+# an index a bag: tiles of 8, up to sixteen of them for a warp
+@pytest.mark.parametrize("D", [52, 60, 64])
+@pytest.mark.parametrize("B", [113_700, 200_003])
+def test_small_tiles_of_large_batches(oracle, D, B):
+    rng = np.random.default_rng(D)
+    rows = (40_000, 3, 900_000)
+    T = len(rows)
+    off = np.arange(T * B + 1, dtype=np.int32)
+    idx = (rng.random(T * B) ** rng.choice([1, 8], T * B) * np.repeat(rows, B)).astype(np.int32)
+    go = rng.standard_normal((B, T, D), dtype=np.float32)
+    c = Case(W.Workload("tiles", rows, D=D, B=B, alpha=None))
+    ur, uo, gr = c.gpu_bwd(idx, off, go)
+    o_ur, o_uo, o_gr = oracle.emb_bwd(go, T, D, B, idx, off)
+    assert bit_equal(uo, o_uo) and bit_equal(ur, o_ur)
+    # as above
+    n = int(np.bincount(idx + 1_000_000 * np.repeat(np.arange(T), B)).max())
     np.testing.assert_allclose(gr, o_gr, rtol=2.0 ** -23, atol=12.0 * n * n * 2.0 ** -53)
     c.ctx.close()
 

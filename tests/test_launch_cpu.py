@@ -7,7 +7,7 @@ import subprocess
 import pytest
 
 HERE = os.path.dirname(os.path.abspath(__file__))
-SCENARIOS = ["contexts_in_turn", "refused_sorts", "clusters_stand_by", "eight_blocks_a_table"]
+SCENARIOS = ["contexts_in_turn", "refused_sorts", "clusters_stand_by", "eight_blocks_a_table", "tiles_of_the_sum"]
 
 
 @pytest.fixture(scope="module")
