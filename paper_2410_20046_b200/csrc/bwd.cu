@@ -496,14 +496,13 @@ size_t dq_sum_align(const dqrm_ctx *ctx)
 // segment starts).  It needs no upstream gradient, so a training step runs it beside the forward.
 int dq_launch_bwd_sort(dqrm_ctx *ctx, const int32_t *indices, const int32_t *offsets,
                        int32_t *unique_rows, int32_t *uniq_off, int B, int64_t L,
-                       void *ws_, size_t ws_bytes, cudaStream_t st, bool lists_by_table, bool *by_table, int *lists,
-                       bool beside)
+                       void *ws_, size_t ws_bytes, cudaStream_t st, int *lists, bool beside)
 {
+    const bool lists_by_table = lists != nullptr;
     const int64_t G = (int64_t)ctx->T * B;
     const Layout y = make_layout(ctx, L, L <= G);
     if (ws_bytes < y.total) return DQRM_ERR_WORKSPACE;
     char *ws = reinterpret_cast<char *>(ws_);
-    if (by_table) *by_table = false;
     if (lists) *lists = 0;
     const bool fits_cluster = (L + ctx->T - 1) / ctx->T <= (int64_t)csort::CLUSTER * 12288;   // (a table beyond its
     // blocks' shared memory still sorts, through global staging, but slowly)
@@ -552,8 +551,7 @@ int dq_launch_bwd_sort(dqrm_ctx *ctx, const int32_t *indices, const int32_t *off
         if (lists_by_table && launch_small_sort(ctx, ca, per_table, L == G, st, e)) {
             if (e == cudaSuccess) {
                 dq_mark(ctx, st, L == G ? DQ_K_SMALL_SORT : DQ_K_CLUSTER_SORT);
-                if (by_table) *by_table = true;
-                if (lists) *lists = 1;
+                *lists = 1;
                 return DQRM_OK;
             }
             ctx->last_cuda_error = (int)e;         // (taken off the runtime, so that nobody finds it behind the sort that follows)
@@ -561,7 +559,7 @@ int dq_launch_bwd_sort(dqrm_ctx *ctx, const int32_t *indices, const int32_t *off
         }
         const bool wide = wide_clusters(ctx, per_table, beside);
         e = cudaErrorUnknown;
-        if (wide && lists_by_table && lists) {
+        if (wide && lists_by_table) {
             ca.parts = table_parts(ctx, per_table);
             if (ca.parts > 1) e = launch_cluster_sort<csort::CLUSTER_WIDE, true>(ctx, ca, csort::choose_cap(per_table, csort::CLUSTER_WIDE), st);
             if (e != cudaSuccess) ca.parts = 1;
@@ -598,8 +596,7 @@ int dq_launch_bwd_sort(dqrm_ctx *ctx, const int32_t *indices, const int32_t *off
         skeys = keys[0];
     }
     if (sorted && lists_by_table) {                    // the lists are there; unique_rows and uniq_off come with the sums
-        if (by_table) *by_table = true;
-        if (lists) *lists = parts;
+        *lists = parts;
         return DQRM_OK;
     }
     if (!sorted) {        // (a cluster sort that did not number the segments itself has counted the segment heads of every tile)
@@ -744,7 +741,7 @@ int dq_launch_bwd(dqrm_ctx *ctx, const float *grad_out, const int32_t *indices, 
         return launch_small<false>(ctx, nullptr, indices, offsets, grad_out, unique_rows, uniq_off, grad_rows, nullptr, nullptr, 0.f, B, L, ws,
                                    ws_bytes, st);
     int lists = 0;
-    int rc = dq_launch_bwd_sort(ctx, indices, offsets, unique_rows, uniq_off, B, L, ws, ws_bytes, st, true, nullptr, &lists);
+    int rc = dq_launch_bwd_sort(ctx, indices, offsets, unique_rows, uniq_off, B, L, ws, ws_bytes, st, &lists);
     if (rc != DQRM_OK) return rc;
     return dq_launch_bwd_sum(ctx, grad_out, unique_rows, uniq_off, grad_rows, B, L, lists, ws, ws_bytes, st);
 }

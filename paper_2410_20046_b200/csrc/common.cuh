@@ -365,9 +365,9 @@ size_t dq_refresh_ws_bytes(const dqrm_ctx *ctx);
 int dq_launch_refresh(dqrm_ctx *ctx, const float *tables, const int32_t *bits, float *scales,
                       float *minmax, void *ws, size_t ws_bytes, cudaStream_t st);
 
-// let_next: see before_and_next; beside: a sort runs at the same time, to which the forward leaves room
 // bytes that tables and out have to be aligned to
 size_t dq_fwd_align(const dqrm_ctx *ctx, const int8_t *codes_out, int B, int64_t L);
+// let_next: see before_and_next; beside: a sort runs at the same time, to which the forward leaves room
 int dq_launch_fwd(dqrm_ctx *ctx, const float *tables, const int32_t *indices, const int32_t *offsets,
                   const float *scales, const int32_t *bits, float *out, int8_t *codes_out,
                   int B, int64_t L, cudaStream_t st, bool let_next = false, bool beside = false);
@@ -388,12 +388,13 @@ int dq_launch_bwd(dqrm_ctx *ctx, const float *grad_out, const int32_t *indices, 
                   int32_t *unique_rows, int32_t *uniq_off, float *grad_rows, int B, int64_t L,
                   void *ws, size_t ws_bytes, cudaStream_t st, bool alone = false);
 
-// lists_by_table: dq_launch_bwd_sum follows on the same workspace; the cluster sort then numbers each table's
-// segments itself (*by_table says whether it did; *lists, without which it is one, how many lists each table then has), no separate kernel numbers them over the batch, and unique_rows /
-// uniq_off are written by dq_launch_bwd_sum.  beside: a training step runs at the same time.  Without it they are complete when the sort is.
+// With `lists` dq_launch_bwd_sum follows on the same workspace: a sort by the tables' own blocks then numbers each table's segments itself
+// (*lists says how many lists each table has; 0: the radix sort ran, and they are numbered over the batch), no separate kernel does, and
+// unique_rows / uniq_off are written by dq_launch_bwd_sum.  Without it they are complete when the sort is.  beside: a training step
+// runs at the same time
 int dq_launch_bwd_sort(dqrm_ctx *ctx, const int32_t *indices, const int32_t *offsets, int32_t *unique_rows,
                        int32_t *uniq_off, int B, int64_t L, void *ws, size_t ws_bytes, cudaStream_t st,
-                       bool lists_by_table, bool *by_table, int *lists = nullptr, bool beside = false);
+                       int *lists, bool beside = false);
 int dq_launch_bwd_sum(dqrm_ctx *ctx, const float *grad_out, int32_t *unique_rows, int32_t *uniq_off, float *grad_rows,
                       int B, int64_t L, int lists, void *ws, size_t ws_bytes, cudaStream_t st);
 

@@ -195,7 +195,7 @@ int dq_launch_dp_merge_update(dqrm_ctx *ctx, float *tables, int W, int64_t rank_
     dq_mark(ctx, st, DQ_K_DP_PACK);
     ctx->payload_position = 1;
     int rc = dq_launch_bwd_sort(ctx, indices, offsets, union_rows, union_off, (int)y.Bp, n_entries, ws + y.sort_ws,
-                                ws_bytes - y.sort_ws, st, false, nullptr);
+                                ws_bytes - y.sort_ws, st, nullptr);
     ctx->payload_position = 0;
     if (rc != DQRM_OK) return rc;
     if (n_entries == 0) return DQRM_OK;

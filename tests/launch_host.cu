@@ -28,7 +28,10 @@ struct Ctx {
     }
     int sort(int B, int64_t L, bool *by_table)
     {
-        return dq_launch_bwd_sort(&c, dummy, dummy, dummy, dummy, B, L, workspace, sizeof(workspace), nullptr, true, by_table);
+        int lists = -1;
+        const int rc = dq_launch_bwd_sort(&c, dummy, dummy, dummy, dummy, B, L, workspace, sizeof(workspace), nullptr, &lists);
+        *by_table = lists > 0;
+        return rc;
     }
     int small_step(int B, int64_t L)
     {
