@@ -375,9 +375,10 @@ inline bool warp_per_bag(const FwdArgs &a, int lpr) { return lpr == 16 && long_b
 // Warps an SM below which a one-index batch's warps take fewer bags, down to one step of their rows: a warp's steps are a chain, and a
 // small batch has too few warps to hide it.  Measured on B200 (us; 32 bags a warp / so many that there are twelve warps an SM
 // at least): 26 tables of 2048 bags of 64 features (11 warps an SM) 5.25 / 4.45, one of 5000 of 128 6.51 / 2.82, four of 9000 of 32
-// 3.35 / 2.94.  Not in a step, where it runs beside a sort, which needs the room: five tables of 10,000 bags of 128 features in one call
-// 40.8, 42.6 with fewer bags a warp, eight pipelined steps of three of 8000 of 64 206 and 210; nor with more warps: one table of
-// 65,536 of 128 (14 warps an SM) 12.6 / 10.6 alone
+// 3.35 / 2.94.  Not in a step that runs it beside a sort, which needs the room: five tables of 10,000 bags of 128 features in one call
+// 40.8, 42.6 with fewer bags a warp, eight pipelined steps of three of 8000 of 64 206 and 210; but in a step that keeps to one stream
+// (eight steps of five of 10,000 of 128 274 / 262) and in the host-fed one (train_step_host).  The line was drawn while steps were
+// under the rule, too; a forward alone gains beyond it (one table of 65,536 of 128, 14 warps an SM, 12.6 / 10.6)
 constexpr int FEW_WARPS = 12;
 constexpr int MIXED_TABLES = 8;
 // Order of the blocks.  All tables' blocks for the same bags side by side: the pooled rows of a bag lie next to one another in the

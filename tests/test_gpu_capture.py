@@ -9,8 +9,9 @@ pytestmark = pytest.mark.gpu
 
 
 # tables, bags, indices a bag, features: one launch behind the forward, a chain, forked (an index a bag and not), backward aside,
-# forward on the caller's stream
-@pytest.mark.parametrize("T,B,bag,D", [(4, 100, 1, 16), (4, 700, 1, 16), (3, 900, 3, 16), (6, 1_100, 1, 64), (26, 2_000, 1, 16), (3, 50_000, 1, 128), (1, 70_000, 64, 64)])
+# forward on the caller's stream, a radix sort, a table alone by its parts
+@pytest.mark.parametrize("T,B,bag,D", [(4, 100, 1, 16), (4, 700, 1, 16), (3, 900, 3, 16), (6, 1_100, 1, 64), (26, 2_000, 1, 16), (3, 50_000, 1, 128), (1, 70_000, 64, 64),
+                                         (1, 50_001, 1, 16), (1, 60_000, 1, 64)])
 @pytest.mark.parametrize("two_calls", [False, True])
 def test_captured_steps(T, B, bag, D, two_calls):
     import torch
