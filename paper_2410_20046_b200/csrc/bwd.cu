@@ -34,10 +34,9 @@ constexpr int ST_WARPS = ST_THREADS / 32;
 struct Layout {
     int passes, digit_bits;                    // radix sort: digits of the row number within a table
     int64_t radix_tiles, num_tiles;
-    // the summing kernel: log2 of the entries between two of chunk_first; rows of more than 48 features: small tiles, tiles, tiles of
+    // the summing kernel: log2 of the entries between two of chunk_first; rows of more than 48 features: entries of a tile, tiles, tiles of
     // a warp's range; narrower ones: entries of a lane group's range, ranges of warps
-    int sum_shift;
-    bool sum_small;
+    int sum_shift, sum_tile;
     int64_t sum_tiles, sum_ranges;
     int range_tiles, sum_span;
     size_t absmax, tile_heads, tile0, tile_table, totals, tilehist;
@@ -45,8 +44,8 @@ struct Layout {
     size_t total;
 };
 
-// one_index: the batch has at most an index a bag on average; where the parts lie does not depend on it
-Layout make_layout(const dqrm_ctx *ctx, int64_t L, bool one_index = false)
+// bags: of the batch, which how it is summed depends on, but not where the parts lie
+Layout make_layout(const dqrm_ctx *ctx, int64_t L, int64_t bags = 0)
 {
     Layout y;
     y.passes = (ctx->row_bits + rsort::MAX_DIGIT_BITS - 1) / rsort::MAX_DIGIT_BITS;
@@ -60,11 +59,10 @@ Layout make_layout(const dqrm_ctx *ctx, int64_t L, bool one_index = false)
                                                  : (int64_t)ctx->num_sms * segred::sum_blocks(segred::floats_per_lane(ctx->D)) /
                                                        segred::column_blocks(ctx->D) * segred::WARPS;
     if (warps < 1) warps = 1;
-    y.sum_small = segred::small_tiles(ctx->D, Lc, warps, one_index);
-    const int I = segred::tile_entries(y.sum_small);
-    y.sum_shift = segred::takes_groups(ctx->D) ? segred::CHUNK_SHIFT : segred::chunk_shift(y.sum_small);
-    y.sum_tiles = (Lc + I - 1) / I;
-    y.range_tiles = segred::range_tiles(ctx->D, y.sum_tiles, warps, y.sum_small);
+    y.sum_tile = segred::tile_entries(ctx->D, Lc, warps, bags);
+    y.sum_shift = segred::takes_groups(ctx->D) ? segred::CHUNK_SHIFT : segred::log2_of(y.sum_tile);
+    y.sum_tiles = (Lc + y.sum_tile - 1) / y.sum_tile;
+    y.range_tiles = segred::range_tiles(ctx->D, y.sum_tiles, warps, y.sum_tile);
     const int64_t groups = 32 / segred::lanes_per_row(ctx->D), chunk = (int64_t)1 << segred::CHUNK_SHIFT;
     y.sum_span = (int)(((Lc + warps * groups - 1) / (warps * groups) + chunk - 1) / chunk * chunk);
     y.sum_ranges = (Lc + y.sum_span * groups - 1) / (y.sum_span * groups);
@@ -242,7 +240,7 @@ seg_emit_kernel(const u32 *__restrict__ keys, int64_t L, const u32 *__restrict__
 
 // ---------------------------------------------------------------------------------
 template <int VEC>
-int launch_sum(dqrm_ctx *ctx, const segred::Args &a, bool small, cudaStream_t st)
+int launch_sum(dqrm_ctx *ctx, const segred::Args &a, int tile, cudaStream_t st)
 {
     using namespace segred;
     const size_t smem = smem_bytes(a.T);
@@ -250,17 +248,18 @@ int launch_sum(dqrm_ctx *ctx, const segred::Args &a, bool small, cudaStream_t st
     const dim3 grid((unsigned)((ranges * a.columns + WARPS - 1) / WARPS));
     const bool exact = ctx->D % (32 * VEC) == 0;
     constexpr bool wide = VEC == 4;                          // (only those rows may have several blocks of features)
-#define DQ_SUM(EXACT, SMALL, COLS) \
-    DQRM_CUDA_TRY(ctx, (dq_launch(seg_sum_kernel<VEC, EXACT, SMALL, COLS>, grid, dim3(THREADS), smem, st, a)))
-#define DQ_SUM2(SMALL)                                                              \
+#define DQ_SUM(EXACT, I, COLS) \
+    DQRM_CUDA_TRY(ctx, (dq_launch(seg_sum_kernel<VEC, EXACT, I, COLS>, grid, dim3(THREADS), smem, st, a)))
+#define DQ_SUM2(I)                                                                  \
     do {                                                                            \
-        if (a.columns > 1 && exact) DQ_SUM(true, SMALL, wide);                      \
-        else if (a.columns > 1) DQ_SUM(false, SMALL, wide);                         \
-        else if (exact) DQ_SUM(true, SMALL, false);                                 \
-        else DQ_SUM(false, SMALL, false);                                           \
+        if (a.columns > 1 && exact) DQ_SUM(true, I, wide);                          \
+        else if (a.columns > 1) DQ_SUM(false, I, wide);                             \
+        else if (exact) DQ_SUM(true, I, false);                                     \
+        else DQ_SUM(false, I, false);                                               \
     } while (0)
-    if (small) DQ_SUM2(true);
-    else DQ_SUM2(false);
+    if (tile == 8) DQ_SUM2(8);
+    else if (tile == 16) DQ_SUM2(16);
+    else if constexpr (VEC == 2) DQ_SUM(true, 32, false);    // (64 features)
 #undef DQ_SUM2
 #undef DQ_SUM
     dq_mark(ctx, st, DQ_K_SEG_SUM);
@@ -500,7 +499,7 @@ int dq_launch_bwd_sort(dqrm_ctx *ctx, const int32_t *indices, const int32_t *off
 {
     const bool lists_by_table = lists != nullptr;
     const int64_t G = (int64_t)ctx->T * B;
-    const Layout y = make_layout(ctx, L, L <= G);
+    const Layout y = make_layout(ctx, L, G);
     if (ws_bytes < y.total) return DQRM_ERR_WORKSPACE;
     char *ws = reinterpret_cast<char *>(ws_);
     if (lists) *lists = 0;
@@ -616,7 +615,7 @@ int dq_launch_bwd_sort(dqrm_ctx *ctx, const int32_t *indices, const int32_t *off
 int dq_launch_bwd_sum(dqrm_ctx *ctx, const float *grad_out, int32_t *unique_rows, int32_t *uniq_off, float *grad_rows,
                       int B, int64_t L, int lists, void *ws_, size_t ws_bytes, cudaStream_t st)
 {
-    const Layout y = make_layout(ctx, L, L <= (int64_t)ctx->T * B);
+    const Layout y = make_layout(ctx, L, (int64_t)ctx->T * B);
     if (ws_bytes < y.total) return DQRM_ERR_WORKSPACE;
     if (L == 0) return DQRM_OK;
     char *ws = reinterpret_cast<char *>(ws_);
@@ -646,7 +645,7 @@ int dq_launch_bwd_sum(dqrm_ctx *ctx, const float *grad_out, int32_t *unique_rows
     a.span = (u32)y.sum_span;
     a.ranges = (u32)y.sum_ranges;
     a.status = ctx->d_status;
-    if (!segred::takes_groups(D)) return D <= 64 ? launch_sum<2>(ctx, a, y.sum_small, st) : launch_sum<4>(ctx, a, y.sum_small, st);
+    if (!segred::takes_groups(D)) return D <= 64 ? launch_sum<2>(ctx, a, y.sum_tile, st) : launch_sum<4>(ctx, a, y.sum_tile, st);
     switch (segred::lanes_per_row(D)) {
     case 1: return launch_sum_groups<1>(ctx, a, st);
     case 2: return launch_sum_groups<2>(ctx, a, st);
@@ -713,12 +712,12 @@ int dq_launch_small_step(dqrm_ctx *ctx, float *tables, const int32_t *indices, c
                               ws_bytes, st);
 }
 
-// A backward that stands alone (behind it a step would read the workspace's maxima) in one launch instead of two: up to 3072 lookups of
+// A backward that stands alone (behind it a step would read the workspace's maxima) in one launch instead of two: up to 3600 lookups of
 // an index a bag, fewer of rows of less than 16 features, 64 K gathered values, unless they are many tables of up to 64.  Measured on
 // B200 (us a backward in graph replay; two launches / one): 4 tables of 128 lookups of 16 features 9.5 / 7.2, of 512 11.6 / 10.4, 16 of
 // 200 10.9 / 10.2, of 128 of 32 features 10.4 / 9.1, 2 of 100 of 128 10.0 / 8.1; around it the four calls of 16 tables of 200 22.0 / 20.0, of
-// 26 of 64 19.0 / 18.2, of 26 of 90 22.0 / 20.0, but of 26 of 128 20.0 / 20.2 to 20.8, of 48 of 64 19.8 / 21.2, of 8 of 512 21.1 / 21.5
-// to 22.1, of 10 of 400 19.7 / 21.0 where tables have three rows, and of 26 of 128 of 8 features 19.2 / 20.6.  (The block counts the
+// 26 of 64 19.0 / 18.2, of 26 of 90 22.0 / 20.0, of 26 of 128 20.2 / 19.8 (all of 100 K rows 20.1 / 20.9), of 13 of 256 21.7 / 20.3, of 40 of
+// 90 22.5 / 22.1, but of 48 of 64 19.8 / 21.2, of 8 of 512 21.1 / 21.5 to 22.1, of 10 of 400 19.7 / 21.0 where tables have three rows, and of 26 of 128 of 8 features 19.2 / 20.6.  (The block counts the
 // lookups in front of its own by their rows; all in one row they wait for one another: 8 tables of 256 of one row each 20.5 / 22.9.)
 // Other batches may lie in one table, whose block then does everything: up to 1100 lookups and 32 K values.  13 tables of 40 bags of two
 // 13.4 / 7.5, with nine tenths of the lookups in one 16.1 / 14.5; 4 of 90 bags of four 11.3 / 8.8, but 15.5 / 20.2; 4 of 64 bags of four of
@@ -726,7 +725,7 @@ int dq_launch_small_step(dqrm_ctx *ctx, float *tables, const int32_t *indices, c
 static bool small_bwd_takes_alone(const dqrm_ctx *ctx, int B, int64_t L)
 {
     if (L == (int64_t)ctx->T * B) {
-        if (L > std::min(3072, 192 * ctx->D) || L * ctx->D > 65536 || (L > 2048 && B <= 64)) return false;
+        if (L > (ctx->D < 16 ? 192 * ctx->D : 3600) || L * ctx->D > 65536 || (L > 2048 && B <= 64)) return false;
     } else if (L > 1100 || L * 4 * segred::lanes_per_row(ctx->D) > 32768) {        // (with the features that idle lanes stand for)
         return false;
     }

@@ -2,7 +2,7 @@
 // Section 4.3 / Appendix B.1: duplicates of a row are coalesced).
 //
 // Input: keys[L] (arena rows, ascending), vals[L] (row of grad_out for each lookup, in stable order),
-// chunk_first[c] = index of the segment that holds sorted entry c << chunk_shift, seg_start[] = sorted position where
+// chunk_first[c] = index of the segment that holds sorted entry c << log2_of(I), seg_start[] = sorted position where
 // every segment begins; the segments are numbered over the whole batch, or per table (Args::by_table), and
 // in the second case this kernel also writes unique_rows and uniq_off.
 //
@@ -39,37 +39,38 @@ __host__ __device__ constexpr int column_blocks(int D) { return (D + 127) / 128;
 // resident block: 852 K rows of 256 bytes 58.4 -> 56.5 us, 1.3 M in bags of twenty 97.9 -> 89.7 (eight rows and three blocks
 // before; five blocks 65 and more: values are spilled).  With four features a lane a fourth block spills, 984 K rows of 512 bytes 82 -> 119
 constexpr int BATCH_ROWS = 4;
-__host__ __device__ constexpr int tile_entries(bool small) { return small ? 8 : 32; }
-__host__ __device__ constexpr int chunk_shift(bool small) { return small ? 3 : 5; }    // of chunk_first
+__host__ __device__ constexpr int log2_of(int tile) { return tile == 8 ? 3 : tile == 16 ? 4 : 5; }
 __host__ __device__ constexpr int sum_blocks(int vec) { return vec == 2 ? 4 : 3; }
-// Tiles of 8 entries instead of 32.  A warp that has one tile takes its batches of rows one after the other, 4 to 8 us for 32 rows, so a
-// batch that would give every resident warp less than three tiles of 32 is cut into tiles of 8 (160 K rows of 192 bytes 38.9 ->
-// 28.7 us, 208 K of 256 bytes 30.7 -> 28.7).  Rows of two features a lane, for which four blocks are resident: with an index a bag tiles
-// of 8 are never the slower (us a backward of 64 features, tiles of 32 / of 8, uniform indices and Zipf 1.1: 343 K rows 71.3 / 59.8 and
-// 56.2 / 52.9, 468 K 90.3 / 74.0 and 67.1 / 63.8, 852 K 147 / 124 and 99.2 / 97.6, 1.6 M 286 / 240 and 187 / 183, 2.4 M 421 / 362 and 284 / 274); in
-// bags tiles of 32 are ahead from where three blocks would have three of them (400 K rows in bags of twenty 79.2 / 80.5 and 60.1 /
-// 63.1, 900 K in bags of nine 154 / 160 and 126 / 138)
-inline bool small_tiles(int D, int64_t L, int64_t warps, bool one_index)
+// Entries of a tile: 8, 16 or (64 features alone) 32.  A warp that has one tile takes its batches of rows one after the other, 4 to 8 us
+// for 32 rows, so a batch that would give every resident warp few tiles is cut finely; a tile's heads and keys cost the same whatever it
+// holds.  Measured on B200 (us a backward; 128 features, tiles of 8 / of 16, uniform indices and Zipf 1.1: 26 K rows 13.4 / 17.1 and 15.7 / 17.3,
+// 213 K 56.2 / 60.5 and 47.0 / 49.3; 16 / 32: 416 K 118 / 124 and 80.1 / 88.6, 855 K in bags of two 263 / 276 and 166 / 183; 96 features, 16 /
+// 32: 416 K 93.9 / 104 and 73.5 / 91.5, 901 K in bags of nine 189 / 202 and 149 / 175).  Rows whose lanes stand idle part from tiles of 8
+// sooner (52 features, 8 / 16: 53 K 17.5 / 16.8 and 18.9 / 18.1, 156 K 38.7 / 35.9 and 36.1 / 33.5, but in bags of six 94 K 31.1 / 33.0).
+// 64 features, an index a bag: 8 / 16 213 K 42.0 / 43.9 and 38.3 / 37.0, 416 K 66.7 / 70.4 and 57.6 / 56.2, 16 / 32 624 K 101 / 107 and
+// 75.2 / 78.9, 900 K 157 / 170 and 114 / 117; in bags 8 / 16 416 K 69.8 / 69.9 and 56.9 / 56.4, 400 K in bags of twenty 80.5 / 77.6 and 63.1 /
+// 61.0, but with bags of more than four 16 / 32 901 K 150 / 152 and 122 / 119, 2 M 226 / 227 and 162 / 158, 8.5 M 710 / 692 and 497 / 475
+inline int tile_entries(int D, int64_t L, int64_t warps, int64_t bags)
 {
-    return floats_per_lane(D) == 2 ? one_index || L < 72 * warps : L < 96 * warps;
+    if (L < (D < 64 ? 24 : D == 64 && L > bags ? 72 : 96) * warps) return 8;
+    return D == 64 && L > 4 * bags ? 32 : 16;
 }
-// A warp that would get more than sixteen tiles of 32 gets eight, and there are more blocks than the GPU holds at once: they pass over
+// Where a warp would get far more than 512 entries its range has fewer, and there are more blocks than the GPU holds at once: they pass over
 // the tables one after the other, each table's share of grad_out stays in L2 while it is read from all sides, and warps with many short
-// runs hold up fewer others.  Measured on B200 (us a backward of 64 features, one range for every resident warp / of eight tiles, Zipf 1.1):
-// 8.5 M rows in bags of twenty 546 / 512, 5.1 M in bags of twelve 363 / 346, 3.6 M 261 / 253, 3.3 M in bags of two 337 / 312, 2 M in bags of
-// twelve 167 / 172.  Where lanes stand idle the line is eighteen, and from 24 tiles on a range has twelve: 52 features, one range / eight
-// tiles / twelve: 8.5 M 643 / 678 / 656, 5.1 M 424 / 442 / 433, 3.6 M 304 / 317 / 311 (uniform 384 / 373 / 372), 3.3 M in bags of two 390 / 358 /
-// 363, 2.6 M 248 / 268 / 277.  A loop over the ranges in each warp, instead of more blocks, costs registers (356 against 276 us a sum).
+// runs hold up fewer others.  Measured on B200 (us a backward, one range for every resident warp / of 256 entries, Zipf 1.1): 64 features,
+// 8.5 M rows in bags of twenty 546 / 512, 5.1 M in bags of twelve 363 / 346, 3.6 M 261 / 253, 2 M 167 / 172; of 52 features, one range / 256
+// entries / 384: 8.5 M 643 / 678 / 656, 3.6 M 304 / 317 / 311 (uniform 384 / 373 / 372), 3.3 M in bags of two 390 / 358 / 363, 2.6 M in
+// bags of twelve 248 / 268 / 277.  A loop over the ranges in each warp, instead of more blocks, costs registers (356 against 276 us a sum).
 // With four features a lane it does not help: 1.6 M rows of 512 bytes 116 -> 122
-constexpr int RANGE_TILES = 8;
-inline int range_tiles(int D, int64_t tiles, int64_t warps, bool small)
+constexpr int RANGE_ENTRIES = 256;
+inline int range_tiles(int D, int64_t tiles, int64_t warps, int tile)
 {
     const int64_t even = (tiles + warps - 1) / warps;
-    if (small || floats_per_lane(D) != 2 || even <= (D == 64 ? 16 : 18)) return (int)even;
-    return D == 64 || even < 24 ? RANGE_TILES : RANGE_TILES + RANGE_TILES / 2;
+    if (tile == 8 || floats_per_lane(D) != 2 || even <= (tile == 32 ? 16 : 36)) return (int)even;
+    return (D == 64 || even < 48 ? RANGE_ENTRIES : RANGE_ENTRIES + RANGE_ENTRIES / 2) / tile;
 }
 // of such ranges, for L lookups (rows of 48 features and fewer have ranges of their own, seg_groups.cuh)
-inline int64_t max_ranges(int D, int64_t L) { return D > 48 && floats_per_lane(D) == 2 ? L / (32 * RANGE_TILES) + 1 : 0; }
+inline int64_t max_ranges(int D, int64_t L) { return D > 48 && floats_per_lane(D) == 2 ? L / RANGE_ENTRIES + 1 : 0; }
 
 struct Args {
     const u32 *keys, *vals, *seg_start, *chunk_first;
@@ -79,7 +80,7 @@ struct Args {
     uint2 *range_done;
     // by_table: the cluster sort numbered each table's segments from 0: table t's starts sit at
     // seg_start[tb[t] + t + .] (tb[t] = first sorted position of the table, one slot more than it has segments: the
-    // last holds the table's end), chunk_first[c] counts within the table that holds entry c << chunk_shift, table_cnt[t] says
+    // last holds the table's end), chunk_first[c] counts within the table that holds entry c << log2_of(I), table_cnt[t] says
     // how many segments the table has (CNT_BROKEN: nothing is summed, no row is updated); unique_rows and uniq_off
     // are then written here, with the tables' bases added
     int by_table;
@@ -169,16 +170,15 @@ __device__ __noinline__ void note_max(u32 *absmax, const u32 *s_uoff, int t_firs
     if ((threadIdx.x & 31) == 0 && m) atomicMax(absmax + (last_not_above(s_uoff, t_first, T, u) >> parts_log), m);
 }
 
-// blockIdx.x * WARPS + warp: range of tiles and block of 128 features (COLS: D > 128, there are several).  EXACT: every lane
+// I: entries of a tile.  blockIdx.x * WARPS + warp: range of tiles and block of 128 features (COLS: D > 128, there are several).  EXACT: every lane
 // holds features.  Rows of 3 KB and more are not asked into L2 ahead: their blocks of features ask for whole rows already
 // (65 K rows of 4080 bytes 138 us, 154 with the request; of 2064 bytes 87 and 85)
-template <int VEC, bool EXACT, bool SMALL, bool COLS>
+template <int VEC, bool EXACT, int I, bool COLS>
 __global__ void __launch_bounds__(THREADS, sum_blocks(VEC))
 seg_sum_kernel(const Args a)
 {
     dq_wait_before();
     constexpr int C = BATCH_ROWS;
-    constexpr int I = tile_entries(SMALL);
     constexpr int NB = I / C;                     // batches per tile
     static_assert(NB % 2 == 0 && I <= 32, "");
     typedef typename Vec<VEC>::type vec_t;
@@ -218,16 +218,16 @@ seg_sum_kernel(const Args a)
         if ((int64_t)vc >= a.G) { dq_report(a.status, DQRM_ERR_INDEX_RANGE); vc = 0u; }
     };
     fetch(tile0);
-    u32 u_base = tile0 < tile1 ? a.chunk_first[(int64_t)tile0 * I >> chunk_shift(SMALL)] : 0u;
+    u32 u_base = tile0 < tile1 ? a.chunk_first[(int64_t)tile0 * I >> log2_of(I)] : 0u;
     // the runs that may be cut: lane 0 has the one that enters the range, lane 1 the one that leaves it.  Where rows take several
     // warps what is to be known of them is asked for now (243 K rows of 1200 bytes 111 -> 109 us; narrower rows, whose loop wants the
     // registers, 78.6 -> 79.5 at 520 K of 512 bytes, and small batches are better without)
-    constexpr bool EARLY = COLS && !SMALL;
+    constexpr bool EARLY = COLS && I > 8;
     u32 cut_u = 0u;                               // segment of the entry at the edge
     bool cut = false;
     const u32 edge = (wl == 0 ? tile0 : tile1) * I;
     if (EARLY && wl < 2 && tile0 < tile1 && edge > 0u && edge < (u32)a.L) {
-        cut_u = __ldg(a.chunk_first + (edge >> chunk_shift(SMALL)));
+        cut_u = __ldg(a.chunk_first + (edge >> log2_of(I)));
         cut = __ldg(a.keys + edge) == __ldg(a.keys + edge - 1u);
     }
     if (a.by_table) {

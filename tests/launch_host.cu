@@ -103,22 +103,22 @@ int eight_blocks_a_table()
     return 0;
 }
 
-// rows of two features a lane: an index a bag is summed by tiles of 8 whatever the batch's size, bags by tiles of 32 from 341 K lookups
-// on; long bags by ranges of a few tiles, of which there are no more than the workspace has room for
+// tiles of 8, 16 and 32 entries on both sides of the lines, and ranges of a few of them, of which there are no more than the workspace
+// has room for
 int tiles_of_the_sum()
 {
-    const int64_t warps = 148 * 4 * 8;
     auto cut = [](int64_t n, int64_t by) { return (n + by - 1) / by; };
-    for (const int D : {52, 64})
-        for (const int64_t L : {300000LL, 350000LL, 468000LL, 852000LL, 2000000LL, 2600000LL, 3000000LL, 3700000LL, 8500000LL})
-            for (const bool bags : {false, true}) {
+    for (const int D : {52, 64, 96, 128})
+        for (const int64_t L : {60000LL, 113600LL, 113700LL, 340000LL, 342000LL, 454600LL, 454700LL, 852000LL, 2000000LL, 2800000LL, 3700000LL, 8500000LL})
+            for (const int bag : {1, 4, 5}) {
                 Ctx x(4, D);
-                const int B = (int)(bags ? L / 8 : L / 4);
-                const bool small = !bags || L < 72 * warps;
-                const int64_t tiles = cut(L, small ? 8 : 32), even = cut(tiles, warps);
-                const int64_t range = small || even <= (D == 64 ? 16 : 18) ? even : D == 64 || even < 24 ? 8 : 12;
-                WANT(dq_launch_bwd_sum(&x.c, nullptr, dummy, dummy, nullptr, B, L, 1, workspace, (size_t)1 << 40, nullptr) == DQRM_OK);
-                WANT((int64_t)fake::grid_x == cut(cut(tiles, range), 8));
+                const int64_t warps = 148 * (D <= 64 ? 4 : 3) * 8, B = L / 4 / bag;
+                const int64_t tile = L < (D < 64 ? 24 : D == 64 && bag > 1 ? 72 : 96) * warps ? 8 : D == 64 && bag > 4 ? 32 : 16;
+                const int64_t tiles = cut(L, tile), even = cut(tiles, warps);
+                int64_t range = even;
+                if (D <= 64 && tile > 8 && even > (tile == 32 ? 16 : 36)) range = (D == 64 || even < 48 ? 256 : 384) / tile;
+                WANT(dq_launch_bwd_sum(&x.c, nullptr, dummy, dummy, nullptr, (int)B, L / bag / 4 * 4 * bag, 1, workspace, (size_t)1 << 40, nullptr) == DQRM_OK);
+                WANT((int64_t)fake::grid_x == cut(cut(cut(L / bag / 4 * 4 * bag, tile), range), 8));
                 WANT(cut(tiles, range) <= std::max(warps, L / 256 + 1));
             }
     return 0;

@@ -336,8 +336,8 @@ def test_tables_beyond_half_a_cluster(oracle, T, large, even):
     c.ctx.close()
 
 
-# more than a dozen tiles of 32 for each of the 4736 warps that 148 SMs hold: one range for each of them, and from sixteen tiles on (64
-# features; eighteen) ranges of eight (of twelve), several of them for a warp's place
+# hundreds of entries for each of the 4736 warps that 148 SMs hold: one range for each of them, and from 512 on (64 features in long bags;
+# 576) ranges of 256 (of 384), several of them for a warp's place
 @pytest.mark.parametrize("D,most", [(52, 36), (64, 36), (64, 46), (52, 51), (52, 64)])
 @pytest.mark.parametrize("sort_path", [0, 1])
 def test_ranges_beyond_the_resident_warps(oracle, D, most, sort_path):
@@ -364,22 +364,23 @@ def test_ranges_beyond_the_resident_warps(oracle, D, most, sort_path):
     c.ctx.close()
 
 
-# an index a bag: tiles of 8, up to sixteen of them for a warp
+# an index a bag and short bags: tiles of 8 and of 16, up to sixteen of them for a warp, and more ranges than warps
 @pytest.mark.parametrize("D", [52, 60, 64])
-@pytest.mark.parametrize("B", [113_700, 200_003])
-def test_small_tiles_of_large_batches(oracle, D, B):
+@pytest.mark.parametrize("B,bag", [(37_700, 1), (113_700, 1), (200_003, 1), (260_000, 4)])
+def test_tiles_of_large_batches(oracle, D, B, bag):
     rng = np.random.default_rng(D)
     rows = (40_000, 3, 900_000)
     T = len(rows)
-    off = np.arange(T * B + 1, dtype=np.int32)
-    idx = (rng.random(T * B) ** rng.choice([1, 8], T * B) * np.repeat(rows, B)).astype(np.int32)
+    L = T * B * bag
+    off = np.arange(0, L + 1, bag, dtype=np.int32)
+    idx = (rng.random(L) ** rng.choice([1, 8], L) * np.repeat(rows, B * bag)).astype(np.int32)
     go = rng.standard_normal((B, T, D), dtype=np.float32)
-    c = Case(W.Workload("tiles", rows, D=D, B=B, alpha=None))
+    c = Case(W.Workload("tiles", rows, D=D, B=B, alpha=None), max_lookups=L)
     ur, uo, gr = c.gpu_bwd(idx, off, go)
     o_ur, o_uo, o_gr = oracle.emb_bwd(go, T, D, B, idx, off)
     assert bit_equal(uo, o_uo) and bit_equal(ur, o_ur)
     # as above
-    n = int(np.bincount(idx + 1_000_000 * np.repeat(np.arange(T), B)).max())
+    n = int(np.bincount(idx + 1_000_000 * np.repeat(np.arange(T), B * bag)).max())
     np.testing.assert_allclose(gr, o_gr, rtol=2.0 ** -23, atol=12.0 * n * n * 2.0 ** -53)
     c.ctx.close()
 

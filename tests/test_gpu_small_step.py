@@ -113,7 +113,7 @@ def test_contexts_of_many_and_of_few_tables_take_turns(oracle):
 
 # the backward alone: feature size, lookups per table, launches: one up to the line, two (sort and sum) beyond it.  An index a bag:
 ALONE_EVEN = {
-    "single": (16, [1], 1), "tiny": (16, [128] * 4, 1), "most_lookups": (16, [256] * 12, 1), "a_table_more": (16, [256] * 13, 2),
+    "single": (16, [1], 1), "tiny": (16, [128] * 4, 1), "most_lookups": (16, [225] * 16, 1), "a_table_more": (16, [225] * 17, 2),
     "most_values": (32, [256] * 8, 1), "a_table_of_values_more": (32, [256] * 9, 2), "most_of_a_table": (32, [512] * 2, 1),
     "a_table_too_long": (16, [513] * 2, 2), "a_table_too_wide": (64, [257] * 2, 2), "narrow": (4, [384] * 2, 1), "too_narrow": (4, [385] * 2, 2),
     "many_tables": (16, [64] * 32, 1), "one_too_many": (16, [64] * 33, 2), "idle_lanes": (20, [90] * 7, 1), "wide": (128, [128] * 4, 1),
