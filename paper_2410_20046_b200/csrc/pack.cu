@@ -15,7 +15,7 @@ namespace {
 
 constexpr int PK_THREADS = 256;
 constexpr int PK_CHUNK4 = 4096;          // 128-bit vectors per chunk
-// Loads of 32 bytes of a thread in flight.  Bound by DRAM: 2.16 GB at 4 bits 376 us, of which reading and writing at the rate of a copy are 371
+// Loads of 32 bytes of a thread in flight.  Bound by DRAM: 2.16 GB at 4 bits 369 us, of which reading and writing at the rate of a copy are 371
 // (with loads of 16 bytes, eight in flight, stores of two bytes and a conversion instruction for every code 411)
 constexpr int PK_UNROLL = 4;
 
@@ -74,10 +74,36 @@ __device__ __forceinline__ void load8(const float4 *p, float4 &a, float4 &b)
                  : "=f"(a.x), "=f"(a.y), "=f"(a.z), "=f"(a.w), "=f"(b.x), "=f"(b.y), "=f"(b.z), "=f"(b.w) : "l"(p));
 }
 
-template <int BITS>
+// A chunk [c0, c1) one vector of a thread at a time, EACH of them in flight: chunks that tables share, what is left of the last, and all into
+// packed rows that do not begin on b bytes.  The former are few, but in a small arena the whole call waits for them: 29 MB of 14 tables at 2
+// bits 12.0 us with one load in flight, 10.0 with four, 51 MB of four tables 12.2 and 9.4.  Apart from the kernel, whose registers it would double
+template <int BITS, int EACH>
+__device__ __noinline__ void pack_singly(const float4 *__restrict__ arena4, const int64_t *v4_off, int T, const float *__restrict__ scales,
+                                         uint8_t *__restrict__ packed, int64_t c0, int64_t c1, bool one_table)
+{
+    QuantScale qs = dq_make_scale(__ldg(scales + dq_table_of(v4_off, T, c0)), BITS);
+    const int n = (int)(c1 - c0);
+    arena4 += c0;
+#pragma unroll 1
+    for (int i0 = threadIdx.x; i0 < n; i0 += PK_THREADS * EACH) {
+        float4 v[EACH];
+#pragma unroll
+        for (int k = 0; k < EACH; ++k) v[k] = __ldcs(arena4 + min(i0 + k * PK_THREADS, n - 1));
+#pragma unroll
+        for (int k = 0; k < EACH; ++k) {
+            const int i = i0 + k * PK_THREADS;
+            if (i >= n) break;
+            if (!one_table) qs = dq_make_scale(__ldg(scales + dq_table_of(v4_off, T, c0 + i)), BITS);
+            store_packed<BITS>(packed, c0 + i, quantise_packed4<BITS>(v[k], qs));
+        }
+    }
+}
+
+// PAIRS: whole chunks inside a table go by pairs of vectors, whose packed bytes are stored at once; READ8: and which are read at once
+template <int BITS, bool PAIRS, bool READ8>
 __global__ void __launch_bounds__(PK_THREADS)
 pack_kernel(const float4 *__restrict__ arena4, const int64_t *__restrict__ row_off, int T, int D, int64_t n4,
-            const float *__restrict__ scales, uint8_t *__restrict__ packed, bool read8, bool store8)
+            const float *__restrict__ scales, uint8_t *__restrict__ packed)
 {
     dq_wait_before();
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -90,8 +116,8 @@ pack_kernel(const float4 *__restrict__ arena4, const int64_t *__restrict__ row_o
         const int64_t c0 = c * PK_CHUNK4, c1 = min(c0 + (int64_t)PK_CHUNK4, n4);
         const int t0 = dq_table_of(v4_off, T, c0);
         const bool one_table = c1 <= v4_off[t0 + 1];
-        QuantScale qs = dq_make_scale(__ldg(scales + t0), BITS);
-        if (one_table && c1 - c0 == PK_CHUNK4) {
+        if (PAIRS && one_table && c1 - c0 == PK_CHUNK4) {
+            const QuantScale qs = dq_make_scale(__ldg(scales + t0), BITS);
             // a thread's loads of PK_UNROLL rounds are all in flight before the first is quantised
 #pragma unroll 1
             for (int r = 0; r < PK_CHUNK4 / 2; r += PK_THREADS * PK_UNROLL) {
@@ -99,7 +125,7 @@ pack_kernel(const float4 *__restrict__ arena4, const int64_t *__restrict__ row_o
 #pragma unroll
                 for (int k = 0; k < PK_UNROLL; ++k) {
                     const float4 *p = arena4 + c0 + 2 * (r + k * PK_THREADS + threadIdx.x);
-                    if (read8) {
+                    if (READ8) {
                         load8(p, v[k][0], v[k][1]);
                     } else {
                         v[k][0] = __ldcs(p);
@@ -107,23 +133,13 @@ pack_kernel(const float4 *__restrict__ arena4, const int64_t *__restrict__ row_o
                     }
                 }
 #pragma unroll
-                for (int k = 0; k < PK_UNROLL; ++k) {
-                    const int64_t v8 = c0 / 2 + r + k * PK_THREADS + threadIdx.x;
-                    const u32 first = quantise_packed4<BITS>(v[k][0], qs), second = quantise_packed4<BITS>(v[k][1], qs);
-                    if (store8) {
-                        store_packed2<BITS>(packed, v8, first, second);
-                    } else {
-                        store_packed<BITS>(packed, 2 * v8, first);
-                        store_packed<BITS>(packed, 2 * v8 + 1, second);
-                    }
-                }
+                for (int k = 0; k < PK_UNROLL; ++k)
+                    store_packed2<BITS>(packed, c0 / 2 + r + k * PK_THREADS + threadIdx.x, quantise_packed4<BITS>(v[k][0], qs),
+                                        quantise_packed4<BITS>(v[k][1], qs));
             }
             continue;
         }
-        for (int64_t i = c0 + threadIdx.x; i < c1; i += PK_THREADS) {
-            if (!one_table) qs = dq_make_scale(__ldg(scales + dq_table_of(v4_off, T, i)), BITS);
-            store_packed<BITS>(packed, i, quantise_packed4<BITS>(__ldcs(arena4 + i), qs));
-        }
+        pack_singly<BITS, PAIRS ? PK_UNROLL : 2 * PK_UNROLL>(arena4, v4_off, T, scales, packed, c0, c1, one_table);
     }
 }
 
@@ -374,10 +390,14 @@ int launch_pack(dqrm_ctx *ctx, const float *tables, const float *scales, uint8_t
 {
     const int64_t n4 = ctx->total_rows * (ctx->D / 4);
     const size_t smem = (size_t)(ctx->T + 1) * sizeof(int64_t);
-    // two vectors are read at once where the arena begins on 32 bytes, and their packed bytes stored at once where those may be
-    const bool read8 = dq_aligned(tables, 2 * sizeof(float4)), store8 = dq_aligned(packed, (size_t)BITS);
-    DQRM_CUDA_TRY(ctx, dq_launch(pack_kernel<BITS>, dim3(ctx->num_sms * 8), dim3(PK_THREADS), smem, st,
-                                 reinterpret_cast<const float4 *>(tables), ctx->d_row_off, ctx->T, ctx->D, n4, scales, packed, read8, store8));
+    auto launch = [&](auto kernel) {
+        return dq_launch(kernel, dim3(ctx->num_sms * 8), dim3(PK_THREADS), smem, st, reinterpret_cast<const float4 *>(tables), ctx->d_row_off, ctx->T,
+                         ctx->D, n4, scales, packed);
+    };
+    // vectors in pairs where their packed bytes may be stored at once; read at once, too, where the arena begins on 32 bytes
+    DQRM_CUDA_TRY(ctx, (!dq_aligned(packed, (size_t)BITS)        ? launch(pack_kernel<BITS, false, false>)
+                        : dq_aligned(tables, 2 * sizeof(float4)) ? launch(pack_kernel<BITS, true, true>)
+                                                                 : launch(pack_kernel<BITS, true, false>)));
     dq_mark(ctx, st, DQ_K_PACK);
     return DQRM_OK;
 }
