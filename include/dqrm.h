@@ -86,7 +86,8 @@ int dqrm_destroy(dqrm_ctx *ctx);
 
 /* Bytes of scratch the calls below need for at most max_lookups lookups and max_bags
  * bags per call.  The workspace must be 256-byte aligned.  Contents need not be
- * preserved between calls and need no initialisation. */
+ * preserved between calls and need no initialisation.  The size may differ between
+ * builds of this library: ask for it, do not keep it. */
 size_t dqrm_workspace_bytes(const dqrm_ctx *ctx, int64_t max_lookups, int64_t max_bags);
 
 /* Synchronises `stream`, returns DQRM_OK or the first device-detected error since the
