@@ -56,10 +56,10 @@ Layout make_layout(const dqrm_ctx *ctx, int64_t L, int64_t bags = 0)
     y.radix_tiles = rsort::max_tiles(ctx->T, Lc);
     // the sum: every warp that the GPU holds at once walks one range (long batches: segred::range_tiles)
     int64_t warps = segred::takes_groups(ctx->D) ? (int64_t)ctx->num_sms * segred::GROUPS_BLOCKS * segred::GROUPS_THREADS / 32
-                                                 : (int64_t)ctx->num_sms * segred::sum_blocks(segred::floats_per_lane(ctx->D)) /
+                                                 : (int64_t)ctx->num_sms * segred::sum_blocks(ctx->D, Lc, ctx->num_sms) /
                                                        segred::column_blocks(ctx->D) * segred::WARPS;
     if (warps < 1) warps = 1;
-    y.sum_tile = segred::tile_entries(ctx->D, Lc, warps, bags);
+    y.sum_tile = segred::tile_entries(ctx->D, Lc, ctx->num_sms, bags);
     y.sum_shift = segred::takes_groups(ctx->D) ? segred::CHUNK_SHIFT : segred::log2_of(y.sum_tile);
     y.sum_tiles = (Lc + y.sum_tile - 1) / y.sum_tile;
     y.range_tiles = segred::range_tiles(ctx->D, y.sum_tiles, warps, y.sum_tile);
@@ -248,18 +248,20 @@ int launch_sum(dqrm_ctx *ctx, const segred::Args &a, int tile, cudaStream_t st)
     const dim3 grid((unsigned)((ranges * a.columns + WARPS - 1) / WARPS));
     const bool exact = ctx->D % (32 * VEC) == 0;
     constexpr bool wide = VEC == 4;                          // (only those rows may have several blocks of features)
-#define DQ_SUM(EXACT, I, COLS) \
-    DQRM_CUDA_TRY(ctx, (dq_launch(seg_sum_kernel<VEC, EXACT, I, COLS>, grid, dim3(THREADS), smem, st, a)))
-#define DQ_SUM2(I)                                                                  \
+    constexpr int MOST = VEC == 2 ? 4 : 3;                   // blocks an SM
+#define DQ_SUM(EXACT, I, COLS, BLOCKS) \
+    DQRM_CUDA_TRY(ctx, (dq_launch(seg_sum_kernel<VEC, EXACT, I, COLS, BLOCKS>, grid, dim3(THREADS), smem, st, a)))
+#define DQ_SUM2(I, BLOCKS)                                                          \
     do {                                                                            \
-        if (a.columns > 1 && exact) DQ_SUM(true, I, wide);                          \
-        else if (a.columns > 1) DQ_SUM(false, I, wide);                             \
-        else if (exact) DQ_SUM(true, I, false);                                     \
-        else DQ_SUM(false, I, false);                                               \
+        if (a.columns > 1 && exact) DQ_SUM(true, I, wide, BLOCKS);                  \
+        else if (a.columns > 1) DQ_SUM(false, I, wide, BLOCKS);                     \
+        else if (exact) DQ_SUM(true, I, false, BLOCKS);                             \
+        else DQ_SUM(false, I, false, BLOCKS);                                       \
     } while (0)
-    if (tile == 8) DQ_SUM2(8);
-    else if (tile == 16) DQ_SUM2(16);
-    else if constexpr (VEC == 2) DQ_SUM(true, 32, false);    // (64 features)
+    if (tile == 8 && sum_blocks(ctx->D, a.L, ctx->num_sms) == 3) DQ_SUM2(8, 3);
+    else if (tile == 8) DQ_SUM2(8, MOST);
+    else if (tile == 16) DQ_SUM2(16, MOST);
+    else if constexpr (VEC == 2) DQ_SUM(true, 32, false, MOST);        // (64 features)
 #undef DQ_SUM2
 #undef DQ_SUM
     dq_mark(ctx, st, DQ_K_SEG_SUM);

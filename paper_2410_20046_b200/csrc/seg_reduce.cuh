@@ -40,7 +40,9 @@ __host__ __device__ constexpr int column_blocks(int D) { return (D + 127) / 128;
 // before; five blocks 65 and more: values are spilled).  With four features a lane a fourth block spills, 984 K rows of 512 bytes 82 -> 119
 constexpr int BATCH_ROWS = 4;
 __host__ __device__ constexpr int log2_of(int tile) { return tile == 8 ? 3 : tile == 16 ? 4 : 5; }
-__host__ __device__ constexpr int sum_blocks(int vec) { return vec == 2 ? 4 : 3; }
+// ... but where that gives a warp less than 18 entries, registers count for more than warps: 53 K rows of 208 bytes 17.6 us a backward with
+// four blocks, 17.2 with three (Zipf 1.1 19.1 and 18.6), 80 K 28.8 and 28.1 (28.9 and 28.2); 112 K 30.1 and 31.3
+inline int sum_blocks(int D, int64_t L, int num_sms) { return floats_per_lane(D) == 2 && L >= 18LL * num_sms * 4 * WARPS ? 4 : 3; }
 // Entries of a tile: 8, 16 or (64 features alone) 32.  A warp that has one tile takes its batches of rows one after the other, 4 to 8 us
 // for 32 rows, so a batch that would give every resident warp few tiles is cut finely; a tile's heads and keys cost the same whatever it
 // holds.  Measured on B200 (us a backward; 128 features, tiles of 8 / of 16, uniform indices and Zipf 1.1: 26 K rows 13.4 / 17.1 and 15.7 / 17.3,
@@ -50,8 +52,9 @@ __host__ __device__ constexpr int sum_blocks(int vec) { return vec == 2 ? 4 : 3;
 // 64 features, an index a bag: 8 / 16 213 K 42.0 / 43.9 and 38.3 / 37.0, 416 K 66.7 / 70.4 and 57.6 / 56.2, 16 / 32 624 K 101 / 107 and
 // 75.2 / 78.9, 900 K 157 / 170 and 114 / 117; in bags 8 / 16 416 K 69.8 / 69.9 and 56.9 / 56.4, 400 K in bags of twenty 80.5 / 77.6 and 63.1 /
 // 61.0, but with bags of more than four 16 / 32 901 K 150 / 152 and 122 / 119, 2 M 226 / 227 and 162 / 158, 8.5 M 710 / 692 and 497 / 475
-inline int tile_entries(int D, int64_t L, int64_t warps, int64_t bags)
+inline int tile_entries(int D, int64_t L, int num_sms, int64_t bags)
 {
+    const int64_t warps = (int64_t)num_sms * (floats_per_lane(D) == 2 ? 4 : 3) / column_blocks(D) * WARPS;
     if (L < (D < 64 ? 24 : D == 64 && L > bags ? 72 : 96) * warps) return 8;
     return D == 64 && L > 4 * bags ? 32 : 16;
 }
@@ -173,8 +176,8 @@ __device__ __noinline__ void note_max(u32 *absmax, const u32 *s_uoff, int t_firs
 // I: entries of a tile.  blockIdx.x * WARPS + warp: range of tiles and block of 128 features (COLS: D > 128, there are several).  EXACT: every lane
 // holds features.  Rows of 3 KB and more are not asked into L2 ahead: their blocks of features ask for whole rows already
 // (65 K rows of 4080 bytes 138 us, 154 with the request; of 2064 bytes 87 and 85)
-template <int VEC, bool EXACT, int I, bool COLS>
-__global__ void __launch_bounds__(THREADS, sum_blocks(VEC))
+template <int VEC, bool EXACT, int I, bool COLS, int BLOCKS>
+__global__ void __launch_bounds__(THREADS, BLOCKS)
 seg_sum_kernel(const Args a)
 {
     dq_wait_before();

@@ -109,11 +109,11 @@ int tiles_of_the_sum()
 {
     auto cut = [](int64_t n, int64_t by) { return (n + by - 1) / by; };
     for (const int D : {52, 64, 96, 128})
-        for (const int64_t L : {60000LL, 113600LL, 113700LL, 340000LL, 342000LL, 454600LL, 454700LL, 852000LL, 2000000LL, 2800000LL, 3700000LL, 8500000LL})
+        for (const int64_t L : {60000LL, 85200LL, 85300LL, 113600LL, 113700LL, 340000LL, 342000LL, 454600LL, 454700LL, 852000LL, 2000000LL, 2800000LL, 3700000LL, 8500000LL})
             for (const int bag : {1, 4, 5}) {
                 Ctx x(4, D);
-                const int64_t warps = 148 * (D <= 64 ? 4 : 3) * 8, B = L / 4 / bag;
-                const int64_t tile = L < (D < 64 ? 24 : D == 64 && bag > 1 ? 72 : 96) * warps ? 8 : D == 64 && bag > 4 ? 32 : 16;
+                const int64_t full = 148 * (D <= 64 ? 4 : 3) * 8, warps = D <= 64 && L < 18 * full ? full / 4 * 3 : full, B = L / 4 / bag;
+                const int64_t tile = L < (D < 64 ? 24 : D == 64 && bag > 1 ? 72 : 96) * full ? 8 : D == 64 && bag > 4 ? 32 : 16;
                 const int64_t tiles = cut(L, tile), even = cut(tiles, warps);
                 int64_t range = even;
                 if (D <= 64 && tile > 8 && even > (tile == 32 ? 16 : 36)) range = (D == 64 || even < 48 ? 256 : 384) / tile;
