@@ -124,7 +124,7 @@ def test_unusable_boundaries(oracle, T, B, bag, where, calls):
     rng = np.random.default_rng(T)
     off = np.arange(0, L + 1, bag, dtype=np.int32)
     bad = off.copy()
-    at, value = {"first": (0, 5), "inside": (7 * B, L + 3), "last": (T * B, L - 1)}[where]
+    at, value = {"first": (0, 5), "inside": ((7 if T > 7 else 1) * B, L + 3), "last": (T * B, L - 1)}[where]
     bad[at] = value
     idx = rng.integers(0, 50, L).astype(np.int32)
     go = rng.standard_normal((B, T, D)).astype(np.float32)
